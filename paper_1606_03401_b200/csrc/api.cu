@@ -13,6 +13,7 @@
 #include "mebptt.h"
 #include "plan.hpp"
 #include "tc.hpp"
+#include "team_run.hpp"
 
 using namespace mebptt;
 
@@ -105,6 +106,7 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
   if (y.tensor_path) {
     return (int)tc::run_step(y, p, io, desc->want_dx != 0, s, false, side_stream && !env::no_overlap());
   }
+  if (y.team) return (int)team::run_step(y, p, io, desc->want_dx != 0, s, false);
   const size_t bh = (size_t)y.B * y.H;
   const size_t plane_elems = y.plane / y.esz;
   char* ws = io.ws;
@@ -489,6 +491,7 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
   Layout y;
   workspace_layout(desc, p, y);
   if (y.tensor_path) return tc::run_step(y, p, StepIO{}, desc->want_dx != 0, nullptr, true, false);
+  if (y.team) return team::run_step(y, p, StepIO{}, desc->want_dx != 0, nullptr, true);
   // forward operation: one kernel per layer; backward operation: 5 for the readout and
   // 4 per layer; one to finalise
   const int64_t L = desc->layers;
@@ -545,6 +548,13 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
 }  // extern "C"
 
 namespace mebptt {
+size_t least_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
+  if (check_common(desc, plan) != MEBPTT_OK) return 0;
+  Layout y;
+  workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y, true);
+  if (y.tensor_path && y.total >= ((size_t)1 << 36)) return 0;
+  return y.total;
+}
 int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, const void* W, const void* b,
                     const void* W_out, const void* b_out, const void* x, const void* targets, const void* h0,
                     const void* c0, void* workspace, size_t workspace_bytes, void* stream, float* loss, float* dW,
@@ -557,6 +567,8 @@ int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, con
   const Plan* p = reinterpret_cast<const Plan*>(plan);
   Layout y;
   workspace_layout(desc, p, y);
+  // a fixed workspace that is too small for the team path's stages can still serve the kernels without
+  if (!side_stream && y.team && y.total > workspace_bytes) workspace_layout(desc, p, y, true);
   if (y.tensor_path && y.total >= ((size_t)1 << 36)) return MEBPTT_ERR_UNSUPPORTED;   // 16-byte offsets in 32 bits
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < y.total)
     return MEBPTT_ERR_WORKSPACE;

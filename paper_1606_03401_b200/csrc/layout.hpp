@@ -23,6 +23,11 @@ namespace mebptt {
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline size_t gcd_sz(size_t a, size_t b) { while (b) { size_t r = a % b; a = b; b = r; } return a; }
 
+namespace team {
+bool supported(const mebptt_lstm_desc* d);
+constexpr size_t kMaxLaunchTasks = 32768;   // 1 MB of tasks per launch at most: what the workspace holds at a time
+}
+
 struct Layout {
   int L = 0, I = 0, H = 0, O = 0, B = 0;
   int dtype = 0;
@@ -31,6 +36,7 @@ struct Layout {
   bool stepwise_tc = false;   // step-by-step operations with their contractions on the tensor cores
   bool stepwise_x3 = false;   // likewise for float32 storage, operands split into bfloat16 halves
   bool gru = false;           // the core is a GRU (CUDA-core kernels)
+  bool team = false;          // CUDA-core shapes walked by the persistent kernel of team.cu
   int NG = 4;                 // row blocks of H rows in a layer's weight matrix and bias: 4 (LSTM) or 3 (GRU)
   size_t esz = 0;        // bytes of one operand element
   size_t granule = 0;
@@ -45,7 +51,7 @@ struct Layout {
   size_t rec_gates = 0;  // gates of layer 0
   size_t rec_in = 0;     // input hidden state
   // workspace offsets: states
-  size_t off_arena = 0, off_core = 0, off_ping = 0, off_pong = 0, off_init = 0;
+  size_t off_arena = 0, off_core = 0, off_core2 = 0, off_ping = 0, off_pong = 0, off_init = 0;
   // carried gradients and per-step scratch of the CUDA-core path
   size_t off_dh = 0, off_dc = 0, off_dha = 0, off_dz = 0, off_dy = 0;
   size_t off_loss_part = 0, off_loss_t = 0;
@@ -58,6 +64,8 @@ struct Layout {
   size_t off_sync = 0, off_tape = 0, off_status = 0, off_split_dh = 0;
   size_t off_a3_run = 0, off_zrun = 0, off_hrun = 0, off_dha_run = 0, off_dy_run = 0, split_floats = 0;
   size_t n_sync = 0, tape_bytes = 0;
+  // team path: packed weights per layer, readout weights, dz of the step after a chunk, end of what a step clears
+  size_t off_wf[16] = {}, off_wb[16] = {}, off_wr = 0, off_carry = 0, off_zero_end = 0;
   size_t total = 0;
   int64_t arena_units = 0;
   int n_loss_part = 0;
@@ -207,8 +215,11 @@ inline std::vector<WorkItem> work_items(const Plan* p, int S) {
   return items;
 }
 
-inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y) {
+// compact: the least working memory, for callers that bring a fixed amount (the team path's stages and
+// packed weights are then done without)
+inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y, bool compact = false) {
   state_layout(d, y);
+  y.team = !compact && team::supported(d);
   y.arena_units = p->arena_units;
   y.loc_bytes = y.unit / (size_t)(p->sigma > 0 ? p->sigma : 1);
   size_t o = 0;
@@ -221,7 +232,34 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
   y.off_dh = take((size_t)y.L * bh4);
   y.off_dc = take((size_t)y.L * bh4);
   y.off_loss_t = take((size_t)y.t * 4);
-  if (!y.tensor_path) {
+  if (y.team) {
+    const size_t G = 4 * (size_t)y.H, hp = align_up(y.H, 8), gp = align_up(G, 8), h4 = align_up(y.H, 4) + 4;
+    y.S = 2048 / y.B > 0 ? 2048 / y.B : 1;
+    if (y.S > 64) y.S = 64;
+    if (y.S > y.t) y.S = (int)y.t;
+    const size_t rows = (size_t)y.S * y.B;
+    y.off_core2 = take(y.rec);   // the working core alternates, so that one leaf's forward operation can pass the last one's backward
+    for (int l = 0; l < y.L; ++l) {
+      y.off_wf[l] = take(G * (align_up(l ? y.H : y.I, 8) + hp) * y.esz);
+      y.off_wb[l] = take(h4 * (gp + (l + 1 < y.L ? gp : align_up(y.O, 8))) * y.esz);
+    }
+    y.off_wr = take(align_up(y.O, 4) * hp * y.esz);
+    y.off_st_dz = y.off_dz = take((size_t)y.L * rows * G * 4);
+    y.off_st_h = take((size_t)y.L * rows * y.H * y.esz);
+    y.off_st_hp = take((size_t)y.L * rows * y.H * y.esz);
+    y.off_dy = take(rows * y.O * 4);
+    // what a step clears: carried gradients, the teams' counters, status
+    y.off_dc = take((size_t)y.L * bh4);
+    y.off_carry = take((size_t)2 * y.L * y.B * G * 4);
+    y.n_sync = 32 * 16;
+    y.off_sync = take(y.n_sync * 4);
+    y.off_status = take(256);
+    y.off_zero_end = o;
+    size_t tasks = 4 * ((size_t)p->cost * y.L + (size_t)y.t * (y.L + 1));   // with the load tasks of the pod kernel
+    tasks += tasks / 4 + 256;   // windows are filled up where a phase would straddle two
+    y.tape_bytes = (tasks < team::kMaxLaunchTasks ? align_up(tasks, 64) : team::kMaxLaunchTasks) * 32;
+    y.off_tape = take(y.tape_bytes);
+  } else if (!y.tensor_path) {
     y.off_dha = take(bh4);
     y.off_dz = take((size_t)y.B * 4 * y.H * 4);
     y.off_dy = take((size_t)y.B * y.O * 4);

@@ -18,6 +18,7 @@
 
 namespace mebptt {
 namespace tc { void forget_plan(uint64_t plan_id); }
+namespace team { void forget_plan(uint64_t plan_id); }
 namespace {
 Plan* new_plan() {
   static std::atomic<uint64_t> next_id{1};
@@ -734,6 +735,7 @@ int mebptt_plan_ex(int64_t t, int64_t m, int mode, int alpha, int beta, mebptt_p
 void mebptt_plan_free(mebptt_plan_t* plan) {
   if (!plan) return;
   mebptt::tc::forget_plan(reinterpret_cast<Plan*>(plan)->id);   // what the executor prepared for this plan goes with it
+  mebptt::team::forget_plan(reinterpret_cast<Plan*>(plan)->id);
   delete reinterpret_cast<Plan*>(plan);
 }
 

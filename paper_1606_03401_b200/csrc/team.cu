@@ -1,0 +1,947 @@
+// Kernels and launches of the team path (team.hpp has the scheme).
+//
+// One persistent kernel walks the phases of a chunk: float32 FMA arithmetic whatever the storage type
+// (operands are widened, all sums are float32 in a fixed order), weights of the CTA's hidden units in
+// shared memory.  What bounds it is the chain of phases: at the sizes it serves the arithmetic of a
+// phase is a fraction of a microsecond, and the rest is the trip of the new states through the L2 and
+// the meeting of the team.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdlib>
+#include <cstring>
+#include <memory>
+#include <mutex>
+#include <vector>
+
+#include "env.hpp"
+#include "kernels.hpp"
+#include "layout.hpp"
+#include "plan.hpp"
+#include "sm100.cuh"
+#include "pod.hpp"
+#include "pod_run.hpp"
+#include "team.hpp"
+#include "team_dev.cuh"
+#include "team_run.hpp"
+
+namespace mebptt {
+namespace team {
+
+namespace {
+
+struct Args {
+  int L, I, H, O, B, S;
+  int T, rows, cluster;
+  Dims d;
+  int ns_f[kMaxLayers], ns_b[kMaxLayers], ns_r;
+  uint64_t resident;
+  int pool_floats;
+  size_t hc, csz_off, plane, gsz;      // bytes: layer stride of a hidden state, its c part, gate plane, a layer's planes
+  size_t rec_gates;                    // bytes into a record
+  char* ws;
+  size_t off_wf[kMaxLayers], off_wb[kMaxLayers], off_wr;
+  size_t off_dz, off_hk, off_hp, off_dy, off_carry, off_dc;
+  const void *x, *h0;
+  const float *c0, *bias, *b_out, *targets;
+  const Task* tasks;
+  int n_tasks;
+  unsigned* sync;                      // one 128-byte line per team
+  unsigned sync_base;                  // arrivals before this launch, per team
+  int* status;
+  int64_t* counters;
+};
+
+// Four weight rows (ld apart) against NB operand rows (lda apart) over the 128-wide slices [i0, i1) of
+// the contraction index (nv float4 in all).  Each lane takes four consecutive elements of a slice.
+template <class T, int NB>
+__device__ __forceinline__ void four_rows(const float* a, int lda, const T* w, int ldw, int i0, int i1, int nv, int lane,
+                                          float (&acc)[NB * 4]) {
+  for (int i = i0; i < i1; ++i) {
+    const int v = i * 32 + lane;
+    if (v < nv) {
+      float4 wr[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) wr[r] = load4(w + (size_t)r * ldw + 4 * v);
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const float4 x = *reinterpret_cast<const float4*>(a + (size_t)b * lda + 4 * v);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          float s = acc[b * 4 + r];
+          s = fmaf(x.x, wr[r].x, s);
+          s = fmaf(x.y, wr[r].y, s);
+          s = fmaf(x.z, wr[r].z, s);
+          acc[b * 4 + r] = fmaf(x.w, wr[r].w, s);
+        }
+      }
+    }
+  }
+}
+
+// Copies rows [0, nb) of a staged operand segment: src row stride `ld` elements, `len` elements, zeros
+// up to `padded` and for rows past `valid`.
+template <class T>
+__device__ __forceinline__ void stage(float* dst, int lda, const T* src, size_t ld, int len, int padded, int nb, int valid,
+                                      int tid) {
+  const int total = nb * padded;
+  for (int e = tid; e < total; e += kThreads) {
+    const int b = e / padded, k = e - b * padded;
+    float v = 0.f;
+    if (k < len && b < valid) v = to_f(ld_l2(src + (size_t)b * ld + k));
+    dst[(size_t)b * lda + k] = v;
+  }
+}
+// The same for float32 rows that allow 16-byte accesses.
+__device__ __forceinline__ void stage4(float* dst, int lda, const float* src, size_t ld, int len, int padded, int nb,
+                                       int valid, int tid) {
+  const int q = padded >> 2, total = nb * q;
+  for (int e = tid; e < total; e += kThreads) {
+    const int b = e / q, k = (e - b * q) * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (k < len && b < valid) v = __ldcg(reinterpret_cast<const float4*>(src + (size_t)b * ld + k));
+    *reinterpret_cast<float4*>(dst + (size_t)b * lda + k) = v;
+  }
+}
+// ... and for bfloat16 rows that allow 8-byte accesses.
+__device__ __forceinline__ void stage4(float* dst, int lda, const __nv_bfloat16* src, size_t ld, int len, int padded, int nb,
+                                       int valid, int tid) {
+  const int q = padded >> 2, total = nb * q;
+  for (int e = tid; e < total; e += kThreads) {
+    const int b = e / q, k = (e - b * q) * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (k < len && b < valid) {
+      const uint2 u = __ldcg(reinterpret_cast<const uint2*>(src + (size_t)b * ld + k));
+      v = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                      __uint_as_float(u.y & 0xffff0000u));
+    }
+    *reinterpret_cast<float4*>(dst + (size_t)b * lda + k) = v;
+  }
+}
+template <class T>
+__device__ __forceinline__ void stage_any(float* dst, int lda, const T* src, size_t ld, int len, int padded, int nb, int valid,
+                                          int tid) {
+  if (((ld | (size_t)len) & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & (4 * sizeof(T) - 1)) == 0)
+    stage4(dst, lda, src, ld, len, padded, nb, valid, tid);
+  else
+    stage(dst, lda, src, ld, len, padded, nb, valid, tid);
+}
+
+// The state of layer l in a block of whole-stack states (or the caller's initial state).
+template <class T>
+__device__ __forceinline__ const T* h_at(const Args& A, uint32_t loc, int l) {
+  if (loc == kInit) return reinterpret_cast<const T*>(A.h0) + (size_t)l * A.B * A.H;
+  return reinterpret_cast<const T*>(A.ws + ((size_t)loc << 8) + (size_t)l * A.hc);
+}
+__device__ __forceinline__ const float* c_at(const Args& A, uint32_t loc, int l) {
+  if (loc == kInit) return A.c0 + (size_t)l * A.B * A.H;
+  return reinterpret_cast<const float*>(A.ws + ((size_t)loc << 8) + (size_t)l * A.hc + A.csz_off);
+}
+template <class T>
+__device__ __forceinline__ T* gates_at(const Args& A, uint32_t rec, int l) {
+  return reinterpret_cast<T*>(A.ws + ((size_t)rec << 8) + A.rec_gates + (size_t)l * A.gsz);
+}
+
+// What a task's element needs from memory beside its sums; fetched while the operands are staged.
+struct Operands { float v[9]; };
+
+template <class T, bool GRU>
+__device__ __forceinline__ void fetch(const Args& A, const Task& t, size_t row, int j, Operands& o) {
+  const int H = A.H, l = t.layer;
+  const size_t e = row * H + j;
+  if (t.kind == FWD) {
+    const float* bias = A.bias + (size_t)l * (GRU ? 3 : 4) * H + j;
+#pragma unroll
+    for (int q = 0; q < (GRU ? 3 : 4); ++q) o.v[q] = __ldg(bias + (size_t)q * H);
+    if (GRU) {
+      o.v[4] = to_f(ld_l2(h_at<T>(A, t.src, l) + e));
+    } else {
+      o.v[4] = ld_l2(c_at(A, t.src, l) + e);
+      if (t.flags & COPY_IN) o.v[5] = to_f(ld_l2(h_at<T>(A, t.src, l) + e));
+    }
+  } else if (t.kind == READ) {
+    o.v[0] = __ldg(A.b_out + j);
+    o.v[1] = __ldg(A.targets + ((size_t)(t.k - 1) * A.B + row) * A.O + j);
+  } else {
+    const T* g = gates_at<T>(A, t.src, l) + e;
+    const size_t pl = A.plane / sizeof(T);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) o.v[q] = to_f(ld_l2(g + q * pl));
+    o.v[4] = ld_l2(reinterpret_cast<const float*>(A.ws + A.off_dc) + (size_t)l * A.B * H + e);
+    o.v[5] = to_f(ld_l2(h_at<T>(A, t.dst, l) + e));   // h_{k-1}
+    o.v[6] = to_f(ld_l2(h_at<T>(A, t.src, l) + e));   // h_k
+    if (!GRU) {
+      o.v[7] = ld_l2(c_at(A, t.src, l) + e);
+      o.v[8] = ld_l2(c_at(A, t.dst, l) + e);
+    }
+  }
+}
+
+// z: the element's sums (four gates; one value for R and B).
+template <class T, bool GRU>
+__device__ __forceinline__ void apply(const Args& A, const Task& t, size_t row, int j, const Operands& o, const float (&z)[4]) {
+  const int H = A.H, l = t.layer;
+  const size_t e = row * H + j;
+  if (t.kind == FWD) {
+    char* dst = A.ws + ((size_t)t.dst << 8);
+    T* h_out = reinterpret_cast<T*>(dst + (size_t)l * A.hc) + e;
+    T* g = gates_at<T>(A, t.dst, l) + e;
+    const size_t pl = A.plane / sizeof(T);
+    char* in = A.ws + ((size_t)t.dst << 8) + A.rec_gates + (size_t)A.L * A.gsz;   // copy of the input state
+    const float bias[4] = {o.v[0], o.v[1], o.v[2], o.v[3]}, cp = o.v[4];
+    float gv[4], h, cv;
+    cell_forward<GRU>(z, bias, cp, gv, h, cv);
+    store(h_out, h);
+    if (!GRU) reinterpret_cast<float*>(dst + (size_t)l * A.hc + A.csz_off)[e] = cv;
+    if (t.flags & GATES) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) store(g + q * pl, gv[q]);
+    }
+    if (t.flags & COPY_IN) {
+      store(reinterpret_cast<T*>(in + (size_t)l * A.hc) + e, GRU ? cp : o.v[5]);
+      if (!GRU) reinterpret_cast<float*>(in + (size_t)l * A.hc + A.csz_off)[e] = cp;
+    }
+  } else if (t.kind == READ) {
+    const float d = z[0] + o.v[0] - o.v[1];
+    reinterpret_cast<float*>(A.ws + A.off_dy)[((size_t)t.sidx * A.B + row) * A.O + j] = 2.f * d * (1.f / ((float)A.B * (float)A.O));
+  } else {
+    const size_t G = (size_t)4 * H, srow = ((size_t)l * A.S + t.sidx) * A.B + row;
+    float* dc_p = reinterpret_cast<float*>(A.ws + A.off_dc) + (size_t)l * A.B * H + e;
+    const float gv[4] = {o.v[0], o.v[1], o.v[2], o.v[3]};
+    float d4[4], carry = o.v[4];
+    cell_backward<GRU>(z[0], gv, o.v[5], o.v[7], o.v[8], carry, d4);
+    *dc_p = carry;
+    const float4 quad = make_float4(d4[0], d4[1], d4[2], d4[3]);   // the four gates of a unit side by side
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(A.ws + A.off_dz) + srow * G + 4 * j) = quad;
+    if (t.flags & CARRY_OUT)
+      *reinterpret_cast<float4*>(reinterpret_cast<float*>(A.ws + A.off_carry) + (((size_t)(t.k & 1) * A.L + l) * A.B + row) * G + 4 * j) = quad;
+    store(reinterpret_cast<T*>(A.ws + A.off_hp) + srow * H + j, o.v[5]);
+    store(reinterpret_cast<T*>(A.ws + A.off_hk) + srow * H + j, o.v[6]);
+  }
+}
+
+// Meeting of the team's CTAs: everything written before it is visible after it.
+__device__ __forceinline__ bool meet(const Args& A, unsigned* line, unsigned target, volatile int* flag) {
+  if (A.T == 1) { __syncthreads(); return true; }
+  if (A.cluster) {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(line) : "memory");
+    bool ok = false;
+    for (uint32_t i = 0; i < sm100::kSpinLimit; ++i) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(line) : "memory");
+      if ((int)(v - target) >= 0) { ok = true; break; }
+      if (i > 256) __nanosleep(32);
+    }
+    if (!ok) { *A.status = MEBPTT_ERR_TIMEOUT; *flag = 1; }
+  }
+  __syncthreads();
+  return *flag == 0;
+}
+
+template <class T, bool GRU, int NB>
+__global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args A) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  Task* window = reinterpret_cast<Task*>(smem);                       // two windows of tasks
+  volatile int& s_flag = *reinterpret_cast<volatile int*>(smem + 2 * kTaskWindow * sizeof(Task));
+  float* pool = reinterpret_cast<float*>(smem + 2 * kTaskWindow * sizeof(Task) + 256);
+  T* held = reinterpret_cast<T*>(pool + A.pool_floats);               // resident weights
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int team = blockIdx.x / A.T, rank = blockIdx.x - team * A.T;
+  const int H = A.H, L = A.L;
+  const int row0 = team * A.rows, rows = min(A.rows, A.B - row0);
+  if (tid == 0) s_flag = *A.status;   // an earlier launch gave up: do nothing
+  int u0, u1, gh0, gh1, go0, go1;
+  part(H, A.T, rank, u0, u1);
+  part(A.d.groups_h, A.T, rank, gh0, gh1);
+  part(A.d.groups_o, A.T, rank, go0, go1);
+
+  // resident weights, in the order of their bits; offsets in elements
+  const int nf = (u1 - u0) * 4, nbk = (gh1 - gh0) * 4, nr = (go1 - go0) * 4;
+  auto f_at = [&](int l) { int o = 0; for (int i = 0; i < l; ++i) if (A.resident >> (2 * i) & 1) o += nf * A.d.kf[i]; return o; };
+  auto b_at = [&](int l) {
+    int o = f_at(L);
+    for (int i = 0; i < l; ++i) if (A.resident >> (2 * i + 1) & 1) o += nbk * A.d.kb[i];
+    return o;
+  };
+  auto copy_in = [&](T* dst, const T* src, size_t n) {   // n is a multiple of 8, both sides are 16-byte aligned
+    const uint4* s4 = reinterpret_cast<const uint4*>(src);
+    uint4* d4 = reinterpret_cast<uint4*>(dst);
+    const int q = (int)(n * sizeof(T) / 16);
+    for (int i = tid; i < q; i += kThreads) d4[i] = __ldcg(s4 + i);
+  };
+  for (int l = 0; l < L; ++l) {
+    const T* wf = reinterpret_cast<const T*>(A.ws + A.off_wf[l]) + (size_t)u0 * 4 * A.d.kf[l];
+    const T* wb = reinterpret_cast<const T*>(A.ws + A.off_wb[l]) + (size_t)gh0 * 4 * A.d.kb[l];
+    if (A.resident >> (2 * l) & 1) copy_in(held + f_at(l), wf, (size_t)nf * A.d.kf[l]);
+    if (A.resident >> (2 * l + 1) & 1) copy_in(held + b_at(l), wb, (size_t)nbk * A.d.kb[l]);
+  }
+  if (A.resident >> 63) copy_in(held + b_at(L), reinterpret_cast<const T*>(A.ws + A.off_wr) + (size_t)go0 * 4 * A.d.hp, (size_t)nr * A.d.hp);
+
+  auto load_window = [&](int w) {
+    if (tid < kTaskWindow * 2)
+      reinterpret_cast<uint4*>(window + (w & 1) * kTaskWindow)[tid] =
+          __ldg(reinterpret_cast<const uint4*>(A.tasks + (size_t)w * kTaskWindow) + tid);
+  };
+  const int windows = A.n_tasks / kTaskWindow;
+  load_window(0);
+  __syncthreads();
+  if (s_flag != 0) return;
+
+  int64_t fwd_ops = 0, bwd_ops = 0;
+  unsigned target = A.sync_base;
+  int w = 0, i0 = 0;
+  if (windows > 1) load_window(1);
+  while (w < windows) {
+    const Task* t = window + (w & 1) * kTaskWindow + i0;
+    if (i0 >= kTaskWindow || t[0].kind == NOP) {   // next window; the one after it is fetched meanwhile
+      ++w; i0 = 0;
+      __syncthreads();
+      if (w + 1 < windows) load_window(w + 1);
+      continue;
+    }
+    int n = 1;
+    while (!(t[n - 1].flags & LAST)) ++n;
+    i0 += n;
+    for (int sub = 0; sub * NB < rows; ++sub) {
+      const int r0 = row0 + sub * NB, valid = min(NB, rows - sub * NB);
+      int works = 0, elems = 0;
+      // operands of every task of the phase
+      for (int i = 0; i < n; ++i) {
+        const Task& k = t[i];
+        const int l = k.layer;
+        float* a = pool + k.a_off;
+        if (k.kind == FWD) {
+          const int lda = A.d.kf[l], I = l ? H : A.I;
+          const T* in = l ? h_at<T>(A, k.dst, l - 1) : reinterpret_cast<const T*>(A.x) + (size_t)(k.k - 1) * A.B * A.I;
+          stage_any(a, lda, in + (size_t)r0 * I, I, I, A.d.ip[l], NB, valid, tid);
+          stage_any(a + A.d.ip[l], lda, h_at<T>(A, k.src, l) + (size_t)r0 * H, H, H, A.d.hp, NB, valid, tid);
+          works += (u1 - u0) * A.ns_f[l];
+          elems += (u1 - u0) * NB;
+        } else if (k.kind == READ) {
+          stage_any(a, A.d.hp, h_at<T>(A, k.src, l) + (size_t)r0 * H, H, H, A.d.hp, NB, valid, tid);
+          works += (go1 - go0) * A.ns_r;
+          elems += (min(go1 * 4, A.O) - go0 * 4) * NB;
+        } else {
+          const int lda = A.d.kb[l], G = 4 * H;
+          const float* dzn = (k.flags & CARRY_IN)
+                                 ? reinterpret_cast<const float*>(A.ws + A.off_carry) + ((size_t)((k.k + 1) & 1) * L + l) * A.B * G
+                                 : reinterpret_cast<const float*>(A.ws + A.off_dz) + ((size_t)l * A.S + k.sidx + 1) * A.B * G;
+          stage_any(a, lda, dzn + (size_t)r0 * G, G, G, A.d.gp, NB, valid, tid);
+          if (l + 1 < L)
+            stage_any(a + A.d.gp, lda,
+                      reinterpret_cast<const float*>(A.ws + A.off_dz) + (((size_t)(l + 1) * A.S + k.sidx) * A.B + r0) * G, G, G,
+                      A.d.gp, NB, valid, tid);
+          else
+            stage_any(a + A.d.gp, lda, reinterpret_cast<const float*>(A.ws + A.off_dy) + ((size_t)k.sidx * A.B + r0) * A.O, A.O,
+                      A.O, lda - A.d.gp, NB, valid, tid);
+          works += (gh1 - gh0) * A.ns_b[l];
+          elems += (min(gh1 * 4, H) - gh0 * 4) * NB;
+        }
+      }
+      // element f of the phase: its task, batch row and column
+      auto locate = [&](int f, const Task*& k, int& b, int& j, int& j0) {
+        for (int i = 0; i < n; ++i) {
+          k = t + i;
+          const int lo = k->kind == FWD ? u0 : k->kind == READ ? go0 * 4 : gh0 * 4;
+          const int hi = k->kind == FWD ? u1 : k->kind == READ ? min(go1 * 4, A.O) : min(gh1 * 4, H);
+          const int m = (hi - lo) * NB;
+          if (f < m) { b = f / (hi - lo); j = lo + f - b * (hi - lo); j0 = lo; return; }
+          f -= m;
+        }
+      };
+      Operands o;
+      const Task* ek = nullptr;
+      int eb = 0, ej = 0, ej0 = 0;
+      if (tid < elems) {
+        locate(tid, ek, eb, ej, ej0);
+        if (eb < valid) fetch<T, GRU>(A, *ek, (size_t)(r0 + eb), ej, o);
+      }
+      __syncthreads();
+      // partial sums
+      for (int wk = warp; wk < works; wk += kWarps) {
+        int rem = wk, i = 0, ns = 1, groups = 0;
+        for (;; ++i) {
+          const Task& k = t[i];
+          ns = k.kind == FWD ? A.ns_f[k.layer] : k.kind == READ ? A.ns_r : A.ns_b[k.layer];
+          groups = k.kind == FWD ? u1 - u0 : k.kind == READ ? go1 - go0 : gh1 - gh0;
+          if (rem < groups * ns) break;
+          rem -= groups * ns;
+        }
+        const Task& k = t[i];
+        const int l = k.layer, g = rem / ns, s = rem - g * ns;
+        const int ld = k.kind == FWD ? A.d.kf[l] : k.kind == READ ? A.d.hp : A.d.kb[l];
+        const int nv = ld >> 2, its = (nv + 31) >> 5;
+        const int b0 = its * s / ns, b1 = its * (s + 1) / ns;
+        float acc[NB * 4];
+#pragma unroll
+        for (int q = 0; q < NB * 4; ++q) acc[q] = 0.f;
+        const int bit = k.kind == FWD ? 2 * l : k.kind == READ ? 63 : 2 * l + 1;
+        if (A.resident >> bit & 1) {
+          const int off = k.kind == FWD ? f_at(l) : k.kind == READ ? b_at(L) : b_at(l);
+          four_rows<T, NB>(pool + k.a_off, ld, held + off + (size_t)g * 4 * ld, ld, b0, b1, nv, lane, acc);
+        } else {
+          const size_t off = k.kind == FWD ? A.off_wf[l] : k.kind == READ ? A.off_wr : A.off_wb[l];
+          const int first = k.kind == FWD ? u0 : k.kind == READ ? go0 : gh0;
+          four_rows<T, NB>(pool + k.a_off, ld, reinterpret_cast<const T*>(A.ws + off) + (size_t)(first + g) * 4 * ld, ld, b0, b1,
+                           nv, lane, acc);
+        }
+        const float v = lane_sums<NB * 4>(acc, lane);
+        constexpr int per = 32 / (NB * 4);
+        if (lane % per == 0) pool[k.red_off + (size_t)(g * ns + s) * NB * 4 + lane / per] = v;
+      }
+      __syncthreads();
+      for (int f = tid; f < elems; f += kThreads) {
+        if (f != tid) {
+          locate(f, ek, eb, ej, ej0);
+          if (eb < valid) fetch<T, GRU>(A, *ek, (size_t)(r0 + eb), ej, o);
+        }
+        if (eb >= valid) continue;
+        const Task& k = *ek;
+        const int ns = k.kind == FWD ? A.ns_f[k.layer] : k.kind == READ ? A.ns_r : A.ns_b[k.layer];
+        float z[4] = {0.f, 0.f, 0.f, 0.f};
+        if (k.kind == FWD) {
+          const float* p = pool + k.red_off + (size_t)(ej - ej0) * ns * NB * 4 + eb * 4;
+          for (int s = 0; s < ns; ++s, p += NB * 4) {
+            const float4 v = *reinterpret_cast<const float4*>(p);
+            z[0] += v.x; z[1] += v.y; z[2] += v.z; z[3] += v.w;
+          }
+        } else {
+          const int jj = ej - ej0;
+          const float* p = pool + k.red_off + (size_t)(jj >> 2) * ns * NB * 4 + eb * 4 + (jj & 3);
+          for (int s = 0; s < ns; ++s, p += NB * 4) z[0] += *p;
+        }
+        apply<T, GRU>(A, k, (size_t)(r0 + eb), ej, o, z);
+      }
+      if ((sub + 1) * NB < rows) __syncthreads();
+    }
+    if (tid == 0 && blockIdx.x == 0)
+      for (int i = 0; i < n; ++i)
+        if (t[i].flags & COUNT) { if (t[i].kind == FWD) ++fwd_ops; else ++bwd_ops; }
+    target += (unsigned)A.T;
+    if (!meet(A, A.sync + (size_t)team * 32, target, &s_flag)) return;
+  }
+  if (tid == 0 && blockIdx.x == 0) {
+    A.counters[0] += fwd_ops;
+    A.counters[1] += bwd_ops;
+  }
+}
+
+// ---- what surrounds the walk ---------------------------------------------------------------
+
+// Packed weights, zeroed carries and counters.  Blocks of 32 x 32 elements; the transposed matrices
+// go through shared memory so that both sides are read and written along rows.
+template <class T>
+struct PackArgs {
+  int L, I, H, O;
+  Dims d;
+  const T *W, *W_out;
+  size_t w_off[kMaxLayers];
+  T *wf[kMaxLayers], *wb[kMaxLayers], *wr;
+  float* zero; size_t n_zero;     // carried gradients, sync lines, status
+  int64_t* counters;
+};
+
+template <class T, bool GRU>
+__global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
+  __shared__ float tile[32][33];
+  const int x = threadIdx.x & 31, y0 = threadIdx.x >> 5, H = P.H;
+  for (size_t i = blockIdx.x * 256 + threadIdx.x; i < P.n_zero; i += (size_t)gridDim.x * 256) P.zero[i] = 0.f;
+  if (blockIdx.x == 0 && threadIdx.x < 8) P.counters[threadIdx.x] = 0;
+  auto tiles = [](int rows, int cols) { return ((rows + 31) / 32) * ((cols + 31) / 32); };
+  int total = tiles(P.d.groups_o * 4, P.d.hp);
+  for (int l = 0; l < P.L; ++l) total += tiles(4 * H, P.d.kf[l]) + tiles(P.d.groups_h * 4, P.d.kb[l]);
+  for (int b = blockIdx.x; b < total; b += gridDim.x) {
+    int t = b, l = 0, what = 0;   // 0: forward rows, 1: transposed, 2: readout
+    for (; l < P.L; ++l) {
+      int n = tiles(4 * H, P.d.kf[l]);
+      if (t < n) { what = 0; break; }
+      t -= n;
+      n = tiles(P.d.groups_h * 4, P.d.kb[l]);
+      if (t < n) { what = 1; break; }
+      t -= n;
+    }
+    if (l == P.L) what = 2;
+    if (what == 0) {
+      const int kf = P.d.kf[l], nx = (kf + 31) / 32, r0 = (t / nx) * 32, c = (t % nx) * 32 + x;
+      const int I = l ? H : P.I, K = I + H, ip = P.d.ip[l];
+      const T* W = P.W + P.w_off[l];
+      for (int r = r0 + y0; r < r0 + 32 && r < 4 * H; r += 8) {
+        if (c >= kf) continue;
+        const int j = r >> 2, q = r & 3;
+        const bool rec = c >= ip;
+        const int col = rec ? c - ip + I : c;
+        bool on = rec ? c - ip < H : c < I;
+        int row = q * H + j;
+        if (GRU && q >= 2) { on = on && (rec == (q == 3)); row = 2 * H + j; }
+        P.wf[l][(size_t)r * kf + c] = on ? W[(size_t)row * K + col] : T(0.f);
+      }
+    } else if (what == 2) {
+      const int hp = P.d.hp, nx = (hp + 31) / 32, r0 = (t / nx) * 32, c = (t % nx) * 32 + x;
+      for (int r = r0 + y0; r < r0 + 32 && r < P.d.groups_o * 4; r += 8)
+        if (c < hp) P.wr[(size_t)r * hp + c] = (r < P.O && c < H) ? P.W_out[(size_t)r * H + c] : T(0.f);
+    } else {
+      // out[j][g]: tile rows j0.., columns g0..; read with j fastest
+      const int kb = P.d.kb[l], nx = (kb + 31) / 32, j0 = (t / nx) * 32, g0 = (t % nx) * 32;
+      const bool top = l + 1 == P.L;
+      for (int yy = y0; yy < 32; yy += 8) {
+        const int g = g0 + yy, j = j0 + x;
+        float v = 0.f;
+        if (j < H && g < kb) {
+          if (g < P.d.gp) {
+            if (g < 4 * H) {
+              const int c = g & 3, u = g >> 2, row = (GRU && c == 3 ? 2 : c) * H + u, I = l ? H : P.I;
+              if (!(GRU && c == 2)) v = to_f(P.W[P.w_off[l] + (size_t)row * (I + H) + I + j]);
+            }
+          } else if (top) {
+            const int o = g - P.d.gp;
+            if (o < P.O) v = to_f(P.W_out[(size_t)o * H + j]);
+          } else {
+            const int gu = g - P.d.gp, c = gu & 3, u = gu >> 2;
+            if (u < H && !(GRU && c == 3)) v = to_f(P.W[P.w_off[l + 1] + (size_t)(c * H + u) * (2 * H) + j]);
+          }
+        }
+        tile[yy][x] = v;
+      }
+      __syncthreads();
+      for (int yy = y0; yy < 32; yy += 8) {
+        const int j = j0 + yy, g = g0 + x;
+        if (j < P.d.groups_h * 4 && g < kb) store(P.wb[l] + (size_t)j * kb + g, tile[x][yy]);
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// The contractions of a finished chunk: weight gradients and dx, all in one launch, 64 x 64 tiles.
+// C[m][n] (+)= sum_k A(m, k) B[k][n]; A is stored [k][m] (a_mn) or [m][k].
+struct Product {
+  const float* A; const void* B; float* C;
+  int lda, ldb, ldc, M, N, K, a_mn, accumulate, tile0;
+  int H, skip, last;   // H > 0: gate rows 4 u + q of A (a_mn) or of the contraction belong to rows q H + u of the weights;
+                       // rows with q == skip to none, and those with q == 3 to block `last`
+};
+constexpr int kMaxProducts = 2 * kMaxLayers + 2;
+struct Products { int n, tiles; Product p[kMaxProducts]; };
+
+template <class T>
+__global__ void __launch_bounds__(256) chunk_products(const __grid_constant__ Products P) {
+  constexpr int TK = 16;
+  __shared__ __align__(16) float As[2][TK][68], Bs[2][TK][68];
+  int i = P.n - 1;
+  while ((int)blockIdx.x < P.p[i].tile0) --i;
+  const Product& p = P.p[i];
+  const int t = blockIdx.x - p.tile0, nx = (p.N + 63) / 64, m0 = (t / nx) * 64, n0 = (t % nx) * 64;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const T* B = reinterpret_cast<const T*>(p.B);
+  float ra[4], rb[4], acc[4][4] = {};
+  auto fetch_tile = [&](int k0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int idx = tid + e * 256;
+      const int km = idx >> 6, mm = idx & 63;      // [k][m] order
+      const int mk = idx >> 4, kk = idx & 15;      // [m][k] order
+      const int m = p.a_mn ? mm : mk, k = k0 + (p.a_mn ? km : kk);
+      const bool on = m0 + m < p.M && k < p.K;
+      ra[e] = on ? p.A[p.a_mn ? (size_t)k * p.lda + m0 + m : (size_t)(m0 + m) * p.lda + k] : 0.f;
+      const int kb = k0 + km, row = (p.a_mn || !p.H) ? kb : ((kb & 3) == 3 ? p.last : kb & 3) * p.H + (kb >> 2);
+      rb[e] = (n0 + mm < p.N && kb < p.K && (p.a_mn || (kb & 3) != p.skip)) ? to_f(B[(size_t)row * p.ldb + n0 + mm]) : 0.f;
+    }
+  };
+  auto put_tile = [&](int s) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int idx = tid + e * 256;
+      if (p.a_mn) As[s][idx >> 6][idx & 63] = ra[e]; else As[s][idx & 15][idx >> 4] = ra[e];
+      Bs[s][idx >> 6][idx & 63] = rb[e];
+    }
+  };
+  fetch_tile(0);
+  put_tile(0);
+  __syncthreads();
+  const int its = (p.K + TK - 1) / TK;
+  for (int it = 0; it < its; ++it) {
+    const int s = it & 1;
+    if (it + 1 < its) fetch_tile((it + 1) * TK);
+#pragma unroll
+    for (int k = 0; k < TK; ++k) {
+      const float4 a = *reinterpret_cast<const float4*>(&As[s][k][ty * 4]), b = *reinterpret_cast<const float4*>(&Bs[s][k][tx * 4]);
+      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(av[r], bv[c], acc[r][c]);
+    }
+    if (it + 1 < its) put_tile(s ^ 1);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int m = m0 + ty * 4 + r, n = n0 + tx * 4 + c;
+      if (m < p.M && n < p.N) {
+        int row = m;
+        if (p.a_mn && p.H) {
+          if ((m & 3) == p.skip) continue;
+          row = ((m & 3) == 3 ? p.last : m & 3) * p.H + (m >> 2);
+        }
+        float* q = p.C + (size_t)row * p.ldc + n;
+        *q = p.accumulate ? *q + acc[r][c] : acc[r][c];
+      }
+    }
+}
+
+// Bias gradients (column sums of a chunk's dz and dy) and the loss terms of its steps.  dy = 2 d / (B O),
+// so the mean of d * d over a step is the sum of dy * dy times B O / 4.
+struct Sums {
+  const float *dz, *dy; float *db, *db_out, *loss_t;
+  int L, NG, H, O, B, S, steps, accumulate;
+};
+__global__ void __launch_bounds__(1024) chunk_sums(const Sums q) {
+  __shared__ float part_s[32][33];
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5, G = 4 * q.H, nh = (G + 31) / 32, no = (q.O + 31) / 32;
+  const int rows = q.steps * q.B;
+  int b = blockIdx.x;
+  if (b < q.L * nh + no) {
+    const bool out = b >= q.L * nh;
+    const int l = b / nh, n = (out ? b - q.L * nh : b - l * nh) * 32 + x, N = out ? q.O : G, ld = out ? q.O : G;
+    const float* v = out ? q.dy : q.dz + (size_t)l * q.S * q.B * G;
+    float a0 = 0.f, a1 = 0.f;
+    if (n < N) {
+      int r = y;
+      for (; r + 32 < rows; r += 64) { a0 += v[(size_t)r * ld + n]; a1 += v[(size_t)(r + 32) * ld + n]; }
+      if (r < rows) a0 += v[(size_t)r * ld + n];
+    }
+    part_s[y][x] = a0 + a1;
+    __syncthreads();
+    if (y == 0 && n < N) {
+      float s = 0.f;
+#pragma unroll
+      for (int i = 0; i < 32; ++i) s += part_s[i][x];
+      if (!out && (n & 3) >= q.NG) return;   // (a GRU's d q belongs to no bias)
+      float* o = out ? q.db_out + n : q.db + (size_t)l * q.NG * q.H + (size_t)(n & 3) * q.H + (n >> 2);
+      *o = q.accumulate ? *o + s : s;
+    }
+  } else {
+    const int k = b - q.L * nh - no;
+    const float* v = q.dy + (size_t)k * q.B * q.O;
+    float a = 0.f;
+    for (int e = threadIdx.x; e < q.B * q.O; e += 1024) a = fmaf(v[e], v[e], a);
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if (x == 0) part_s[0][y] = a;
+    __syncthreads();
+    if (y == 0) {
+      a = part_s[0][x];
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+      if (x == 0) q.loss_t[k] = a * ((float)q.B * (float)q.O * 0.25f);
+    }
+  }
+}
+
+using WalkFn = void (*)(const Args);
+template <class T, bool GRU>
+WalkFn walk_nb(int nb) {
+  return nb == 1 ? walk<T, GRU, 1> : nb == 2 ? walk<T, GRU, 2> : nb == 4 ? walk<T, GRU, 4> : walk<T, GRU, 8>;
+}
+WalkFn walk_fn(const Layout& y, int nb) {
+  if (y.dtype == MEBPTT_BF16) return y.gru ? walk_nb<__nv_bfloat16, true>(nb) : walk_nb<__nv_bfloat16, false>(nb);
+  return y.gru ? walk_nb<float, true>(nb) : walk_nb<float, false>(nb);
+}
+
+}  // namespace
+
+// ------------------------------------------------------------------------------------------
+// host
+// ------------------------------------------------------------------------------------------
+namespace {
+
+// What a shape's configuration needs to know of a device: SMs, and clusters of 1, 2, .. 16 CTAs of the
+// walking kernel (a whole SM each) that fit at once.  Without a device: the figures of a B200.
+struct DeviceFacts { bool known = false; int sms = 148; int clusters[5] = {148, 74, 36, 16, 7}; };
+
+// The kernels take nearly a whole SM's shared memory and clusters of up to 16 CTAs.
+cudaError_t allow(const void* fn) {
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  return e;
+}
+
+DeviceFacts facts() {
+  static std::mutex mu;
+  static DeviceFacts table[64];
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return DeviceFacts{}; }
+  std::lock_guard<std::mutex> lock(mu);
+  DeviceFacts& f = table[dev];
+  if (!f.known) {
+    int sms = 0;
+    pod::Fn fn = pod::kernel(MEBPTT_FP32, false, 1);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || allow(reinterpret_cast<const void*>(fn)) != cudaSuccess) {
+      cudaGetLastError();
+      return DeviceFacts{};
+    }
+    f.sms = sms;
+    for (int i = 0; i <= 4; ++i) {
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = 1u << i; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)(sms >> i) << i); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemMax - 1024;
+      cfg.attrs = at; cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      f.clusters[i] = n;
+    }
+    f.known = true;
+  }
+  return f;
+}
+
+// The schedule of a plan for one problem on one device, kept from step to step (eight of them, most
+// recently used first); its tasks lie in page-locked memory where that can be had.
+struct Kept {
+  uint64_t plan_id = 0;
+  Layout y;
+  bool pageable = false;
+  bool pod = false;            // the pod kernel serves it (pc), else the walking kernel (c)
+  Config c;
+  pod::Config pc;
+  std::vector<Launch> launches;
+  char* tasks = nullptr;       // 32 bytes each
+  bool pinned = false;
+  Kept() = default;
+  Kept(const Kept&) = delete;
+  Kept& operator=(const Kept&) = delete;
+  ~Kept() {
+    if (tasks && pinned) cudaFreeHost(tasks);
+    else free(tasks);
+  }
+};
+std::mutex g_mu;
+std::vector<std::shared_ptr<Kept>> g_kept;
+constexpr size_t kKeep = 8, kMaxPinned = (size_t)64 << 20;
+
+bool same_problem(const Layout& a, const Layout& b) {
+  return a.L == b.L && a.I == b.I && a.H == b.H && a.O == b.O && a.B == b.B && a.dtype == b.dtype && a.t == b.t && a.gru == b.gru;
+}
+
+std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable) {
+  const DeviceFacts f = facts();
+  const Config c = choose_config(y, f.sms, f.clusters);
+  const pod::Config pc = pod::choose_config(y, f.sms, f.clusters);
+  if (!c.ok && !pc.ok) return nullptr;
+  const bool use_pod = pc.ok && (!c.ok || pc.cycles <= c.cycles);
+  {
+    std::lock_guard<std::mutex> lock(g_mu);
+    for (size_t i = 0; i < g_kept.size(); ++i) {
+      Kept& k = *g_kept[i];
+      if (k.plan_id == p->id && same_problem(k.y, y) && (k.pageable || !pageable) && k.pod == use_pod && k.c.T == c.T && k.c.teams == c.teams &&
+          k.c.cluster == c.cluster && k.pc.T == pc.T && k.pc.nb == pc.nb) {
+        std::shared_ptr<Kept> hit = g_kept[i];
+        g_kept.erase(g_kept.begin() + (long)i);
+        g_kept.insert(g_kept.begin(), hit);
+        return hit;
+      }
+    }
+  }
+  std::shared_ptr<Kept> k = std::make_shared<Kept>();
+  k->plan_id = p->id; k->y = y; k->c = c; k->pc = pc; k->pod = use_pod; k->pageable = pageable;
+  Schedule ws;
+  pod::Schedule ps;
+  if (use_pod) pod::build_schedule(y, p, pc, ps);
+  else build_schedule(y, p, c, ws);
+  k->launches = use_pod ? ps.launches : ws.launches;
+  const void* from = use_pod ? (const void*)ps.tasks.data() : (const void*)ws.tasks.data();
+  const size_t bytes = (use_pod ? ps.tasks.size() : ws.tasks.size()) * sizeof(Task);
+  void* mem = nullptr;
+  if (!pageable && bytes <= kMaxPinned && cudaHostAlloc(&mem, bytes, cudaHostAllocDefault) == cudaSuccess) {
+    k->pinned = true;
+  } else {
+    cudaGetLastError();
+    mem = malloc(bytes);
+    if (!mem) return nullptr;
+  }
+  k->tasks = static_cast<char*>(mem);
+  memcpy(mem, from, bytes);
+  std::lock_guard<std::mutex> lock(g_mu);
+  g_kept.insert(g_kept.begin(), k);
+  if (g_kept.size() > kKeep) g_kept.pop_back();
+  return k;
+}
+
+// cluster: CTAs per cluster, or 0 for a cooperative grid
+int launch(const void* fn, int grid, int cluster, int smem, void** args, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  if (cluster) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  } else {
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+  }
+  cfg.attrs = at; cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, args) == cudaSuccess ? MEBPTT_OK : MEBPTT_ERR_CUDA;
+}
+
+template <class T>
+void launch_pack(const Layout& y, const Dims& d, const tc::StepPtrs& io, cudaStream_t s) {
+  PackArgs<T> P{};
+  P.L = y.L; P.I = y.I; P.H = y.H; P.O = y.O; P.d = d;
+  P.W = reinterpret_cast<const T*>(io.W); P.W_out = reinterpret_cast<const T*>(io.W_out);
+  for (int l = 0; l < y.L; ++l) {
+    P.w_off[l] = y.w_layer_offset(l);
+    P.wf[l] = reinterpret_cast<T*>(io.ws + y.off_wf[l]);
+    P.wb[l] = reinterpret_cast<T*>(io.ws + y.off_wb[l]);
+  }
+  P.wr = reinterpret_cast<T*>(io.ws + y.off_wr);
+  P.zero = reinterpret_cast<float*>(io.ws + y.off_dc);
+  P.n_zero = (y.off_zero_end - y.off_dc) / 4;
+  P.counters = io.counters;
+  if (y.gru) pack<T, true><<<592, 256, 0, s>>>(P);
+  else pack<T, false><<<592, 256, 0, s>>>(P);
+}
+
+// The products of chunk `chunk` (steps [k0, k0 + steps), 0-based).
+void fill_products(Products& P, const Layout& y, const tc::StepPtrs& io, bool want_dx, int64_t k0, int steps, bool accumulate) {
+  const int H = y.H, G = 4 * H, rows = steps * y.B;
+  const size_t SB = (size_t)y.S * y.B;
+  const float* dz = reinterpret_cast<const float*>(io.ws + y.off_dz);
+  const char *hk = io.ws + y.off_st_h, *hp = io.ws + y.off_st_hp;
+  P.n = 0; P.tiles = 0;
+  auto add = [&](const float* A, int lda, bool a_mn, const void* B, int ldb, float* C, int ldc, int M, int N, int K, bool acc,
+                 int hidden, int skip, int last) {
+    P.p[P.n++] = Product{A, B, C, lda, ldb, ldc, M, N, K, a_mn ? 1 : 0, acc ? 1 : 0, P.tiles, hidden, skip, last};
+    P.tiles += ((M + 63) / 64) * ((N + 63) / 64);
+  };
+  for (int l = 0; l < y.L; ++l) {
+    const int I = l ? H : y.I, K = I + H;
+    const float* z = dz + (size_t)l * SB * G;
+    const void* in = l ? (const void*)(hk + (size_t)(l - 1) * SB * H * y.esz) : (const void*)(io.x + (size_t)k0 * y.B * I * y.esz);
+    float* dW = io.dW + y.w_layer_offset(l);
+    // (GRU: the rows of n meet the input through d n_pre and the state through d q)
+    add(z, G, true, in, I, dW, K, G, I, rows, accumulate, H, y.gru ? 3 : -1, 3);
+    add(z, G, true, hp + (size_t)l * SB * H * y.esz, H, dW + I, K, G, H, rows, accumulate, H, y.gru ? 2 : -1, y.gru ? 2 : 3);
+  }
+  add(reinterpret_cast<const float*>(io.ws + y.off_dy), y.O, true, hk + (size_t)(y.L - 1) * SB * H * y.esz, H, io.dW_out, H, y.O, H,
+      rows, accumulate, 0, -1, 3);
+  if (want_dx) add(dz, G, false, io.W, y.I + H, io.dx + (size_t)k0 * y.B * y.I, y.I, rows, y.I, G, false, H, y.gru ? 3 : -1, 3);
+}
+
+}  // namespace
+
+void forget_plan(uint64_t plan_id) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  for (size_t i = g_kept.size(); i-- > 0;)
+    if (g_kept[i]->plan_id == plan_id) g_kept.erase(g_kept.begin() + (long)i);
+}
+
+int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool want_dx, cudaStream_t s, bool dry) {
+  const std::shared_ptr<Kept> kept = schedule_for(y, p, io.pageable_tape);
+  if (!kept) return dry ? -1 : MEBPTT_ERR_OOM;
+  const Config& c = kept->c;
+  if (dry) {
+    int64_t n = 2;   // packing, finalisation
+    for (const Launch& g : kept->launches) n += g.chunk >= 0 ? 3 : 1;
+    return n;
+  }
+  const Dims d = dims(y);
+  if (y.dtype == MEBPTT_BF16) launch_pack<__nv_bfloat16>(y, d, io, s);
+  else launch_pack<float>(y, d, io, s);
+
+  Args a{};
+  pod::Args pa{};
+  WalkFn fn = nullptr;
+  pod::Fn pf = nullptr;
+  auto common = [&](auto& q) {
+    q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.S = y.S;
+    q.d = d;
+    for (int l = 0; l < y.L; ++l) { q.off_wf[l] = y.off_wf[l]; q.off_wb[l] = y.off_wb[l]; }
+    q.off_wr = y.off_wr;
+    q.hc = y.hsz + y.csz; q.csz_off = y.hsz; q.plane = y.plane; q.gsz = y.gsz; q.rec_gates = y.rec_gates;
+    q.ws = io.ws;
+    q.off_dz = y.off_dz; q.off_hk = y.off_st_h; q.off_hp = y.off_st_hp; q.off_dy = y.off_dy; q.off_carry = y.off_carry; q.off_dc = y.off_dc;
+    q.x = io.x; q.h0 = io.h0; q.c0 = io.c0; q.bias = io.b; q.b_out = io.b_out; q.targets = io.targets;
+    q.status = reinterpret_cast<int*>(io.ws + y.off_status);
+    q.counters = io.counters;
+  };
+  auto splits = [&](auto& q, const auto& cfg) {
+    for (int l = 0; l < y.L; ++l) { q.ns_f[l] = cfg.ns_f[l]; q.ns_b[l] = cfg.ns_b[l]; }
+    q.ns_r = cfg.ns_r; q.resident = cfg.resident; q.T = cfg.T;
+  };
+  if (kept->pod) {
+    const pod::Config& pc = kept->pc;
+    common(pa);
+    splits(pa, pc);
+    pa.slot_floats = pc.slot_floats; pa.red_floats = pc.red_floats;
+    pf = pod::kernel(y.dtype, y.gru, pc.nb);
+    if (allow(reinterpret_cast<const void*>(pf)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
+  } else {
+    common(a);
+    splits(a, c);
+    a.rows = c.rows; a.cluster = c.cluster ? 1 : 0; a.pool_floats = c.pool_floats;
+    a.sync = reinterpret_cast<unsigned*>(io.ws + y.off_sync);
+    fn = walk_fn(y, c.nb);
+    if (allow(reinterpret_cast<const void*>(fn)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
+  }
+
+  float* loss_t = reinterpret_cast<float*>(io.ws + y.off_loss_t);
+  Task* region = reinterpret_cast<Task*>(io.ws + y.off_tape);
+  const std::vector<Launch>& ls = kept->launches;
+  const size_t room = y.tape_bytes / sizeof(Task);
+  size_t up_lo = 0, up_hi = 0;   // tasks that lie in the region
+  bool first = true;
+  unsigned met = 0;
+  Products P;
+  for (size_t i = 0; i < ls.size(); ++i) {
+    const Launch& g = ls[i];
+    if (g.task0 + g.ntasks > up_hi) {   // the tasks of this launch and of as many after it as fit
+      up_lo = g.task0;
+      up_hi = up_lo;
+      for (size_t j = i; j < ls.size() && ls[j].task0 + ls[j].ntasks - up_lo <= room; ++j) up_hi = ls[j].task0 + ls[j].ntasks;
+      cudaMemcpyAsync(region, kept->tasks + up_lo * sizeof(Task), (up_hi - up_lo) * sizeof(Task), cudaMemcpyHostToDevice, s);
+    }
+    if (g.ntasks) {
+      int rc;
+      if (kept->pod) {
+        pa.tasks = reinterpret_cast<const pod::Task*>(region + (g.task0 - up_lo));
+        pa.n_tasks = (int)g.ntasks; pa.phases = g.phases;
+        void* args[1] = {&pa};
+        rc = launch(reinterpret_cast<const void*>(pf), kept->pc.pods * kept->pc.T, kept->pc.T, kept->pc.smem, args, s);
+      } else {
+        a.tasks = region + (g.task0 - up_lo);
+        a.n_tasks = (int)g.ntasks;
+        a.sync_base = met * (unsigned)c.T;
+        met += (unsigned)g.phases;
+        void* args[1] = {&a};
+        rc = launch(reinterpret_cast<const void*>(fn), c.teams * c.T, c.cluster ? c.T : 0, c.smem, args, s);
+      }
+      if (rc != MEBPTT_OK) return rc;
+    }
+    if (g.chunk >= 0) {
+      const int64_t k0 = (int64_t)g.chunk * y.S;
+      const int steps = (int)std::min<int64_t>(y.S, y.t - k0);
+      fill_products(P, y, io, want_dx, k0, steps, !first);
+      if (y.dtype == MEBPTT_BF16) chunk_products<__nv_bfloat16><<<P.tiles, 256, 0, s>>>(P);
+      else chunk_products<float><<<P.tiles, 256, 0, s>>>(P);
+      const Sums q{reinterpret_cast<const float*>(io.ws + y.off_dz), reinterpret_cast<const float*>(io.ws + y.off_dy), io.db, io.db_out,
+                   loss_t + k0, y.L, y.NG, y.H, y.O, y.B, y.S, steps, first ? 0 : 1};
+      chunk_sums<<<y.L * ((4 * y.H + 31) / 32) + (y.O + 31) / 32 + steps, 1024, 0, s>>>(q);
+      first = false;
+    }
+  }
+  generic::finalize_step(loss_t, y.t, io.loss, io.counters, p->peak_units, reinterpret_cast<int*>(io.ws + y.off_status), s);
+  return cudaGetLastError() == cudaSuccess ? MEBPTT_OK : MEBPTT_ERR_CUDA;
+}
+
+}  // namespace team
+}  // namespace mebptt

@@ -1,0 +1,327 @@
+// Host side of the team path: how a problem is laid over the device, and the schedule of phases a
+// plan's tape is turned into.  Plain C++, no CUDA.
+#include <algorithm>
+#include <cstring>
+
+#include "pod.hpp"
+#include "team.hpp"
+
+namespace mebptt {
+namespace team {
+
+namespace {
+inline int pad8(int v) { return (v + 7) & ~7; }
+inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
+inline int iters(int k) { return ceil_div(k, 128); }   // a warp takes 128 elements of the contraction index at a time
+}  // namespace
+
+Dims dims(const Layout& y) {
+  Dims d{};
+  d.gp = pad8(4 * y.H);
+  d.hp = pad8(y.H);
+  for (int l = 0; l < y.L; ++l) {
+    d.ip[l] = pad8(l == 0 ? y.I : y.H);
+    d.kf[l] = d.ip[l] + d.hp;
+    d.kb[l] = d.gp + (l + 1 < y.L ? d.gp : pad8(y.O));
+  }
+  d.groups_o = ceil_div(y.O, 4);
+  d.groups_h = ceil_div(y.H, 4);
+  return d;
+}
+
+Need need_f(const Layout& y, const Dims& d, const Config& c, int l) {
+  return Need{c.nb * d.kf[l], ceil_div(y.H, c.T) * c.ns_f[l] * c.nb * 4};
+}
+Need need_r(const Layout& y, const Dims& d, const Config& c) {
+  (void)y;
+  return Need{c.nb * d.hp, ceil_div(d.groups_o, c.T) * c.ns_r * c.nb * 4};
+}
+Need need_b(const Layout& y, const Dims& d, const Config& c, int l) {
+  (void)y;
+  return Need{c.nb * d.kb[l], ceil_div(d.groups_h, c.T) * c.ns_b[l] * c.nb * 4};
+}
+
+namespace {
+
+// One task's share of a phase in clock cycles, by what a CTA's shared memory delivers: per group and
+// 128 elements of the contraction, nb operand vectors and 4 weight vectors of 16 bytes a lane.
+double task_cycles(const Config& c, int groups_cta, int k, int ns, int esz, bool resident) {
+  const int nsub = ceil_div(c.rows, c.nb), w = groups_cta * ns;
+  const double through = (double)groups_cta * iters(k) * (4.0 * c.nb + 4.0 * esz);
+  const double chain = (double)ceil_div(w, kWarps) * (ceil_div(iters(k), ns) * 70.0 + 120.0);
+  double t = std::max(through, chain);
+  const double ctas = (double)c.teams * c.T;
+  if (!resident) {   // weights from the L2, as fast as an SM takes them in or all SMs together get them
+    const double bytes = (double)groups_cta * 4 * k * esz;
+    t = std::max(t, std::max(bytes / 45.0, bytes * ctas / 3000.0));
+  }
+  const double stage = (double)c.nb * k * 4;
+  return nsub * (t + std::max(stage / 40.0, stage * ctas / 3000.0));
+}
+
+// Fills in everything that follows from T, teams and rows; returns the estimated cycles of two
+// forward operations and one backward operation, or a negative value if the shape does not fit.
+double finish(const Layout& y, const Dims& d, Config& c) {
+  const int uf = ceil_div(y.H, c.T), ub = ceil_div(d.groups_h, c.T), ur = ceil_div(d.groups_o, c.T);
+  c.nb = 1;
+  while (c.nb < 8 && c.nb < c.rows) c.nb *= 2;
+  auto parts = [](int groups, int k) { return std::max(1, std::min(iters(k), kWarps / groups)); };
+  c.ns_r = parts(ur, d.hp);
+  int most = 0, sum_f = 0, sum_b = 0;
+  const Need nr = need_r(y, d, c);
+  for (int l = 0; l < y.L; ++l) {
+    c.ns_f[l] = parts(uf, d.kf[l]);
+    c.ns_b[l] = parts(ub, d.kb[l]);
+    const Need f = need_f(y, d, c, l), b = need_b(y, d, c, l);
+    most = std::max(most, std::max(f.a + f.red, b.a + b.red));
+    sum_f += f.a + f.red;
+    sum_b += b.a + b.red;
+  }
+  most = std::max(most, nr.a + nr.red);
+  const int want = std::max(sum_f, sum_b) + nr.a + nr.red;
+  const int fixed = 2 * kTaskWindow * (int)sizeof(Task) + 256;
+  const int budget = kSmemMax - fixed;
+  if ((int64_t)most * 4 > budget) return -1.0;
+  auto bytes_f = [&](int l) { return (int64_t)uf * 4 * d.kf[l] * (int64_t)y.esz; };
+  auto bytes_b = [&](int l) { return (int64_t)ub * 4 * d.kb[l] * (int64_t)y.esz; };
+  const int64_t bytes_r = (int64_t)ur * 4 * d.hp * (int64_t)y.esz;
+  int64_t all = bytes_r;
+  for (int l = 0; l < y.L; ++l) all += bytes_f(l) + bytes_b(l);
+  // room for a phase of the wavefront over the layers where the weights leave it, at least for one task
+  int64_t pool = std::min<int64_t>((int64_t)want * 4, std::max<int64_t>((int64_t)most * 4, budget - all));
+  int64_t left = budget - pool;
+  c.resident = 0;
+  int64_t held = 0;
+  auto keep = [&](int bit, int64_t bytes) {
+    if (bytes <= left) { c.resident |= 1ull << bit; left -= bytes; held += bytes; }
+  };
+  for (int l = 0; l < y.L; ++l) keep(2 * l, bytes_f(l));
+  for (int l = 0; l < y.L; ++l) keep(2 * l + 1, bytes_b(l));
+  keep(63, bytes_r);
+  c.pool_floats = (int)(pool / 4) & ~3;
+  c.w_floats4 = (int)(held / 16);
+  c.smem = fixed + c.pool_floats * 4 + (int)held;
+  const double sync = c.T == 1 ? 100.0 : (c.cluster ? 700.0 : 2600.0);
+  double cyc = 3 * (7000.0 + sync) + task_cycles(c, ur, d.hp, c.ns_r, (int)y.esz, (c.resident >> 63) & 1);
+  for (int l = 0; l < y.L; ++l)
+    cyc += 2 * task_cycles(c, uf, d.kf[l], c.ns_f[l], (int)y.esz, (c.resident >> (2 * l)) & 1) +
+           task_cycles(c, ub, d.kb[l], c.ns_b[l], (int)y.esz, (c.resident >> (2 * l + 1)) & 1);
+  c.ok = true;
+  return cyc;
+}
+
+}  // namespace
+
+// The team size with the least estimated time: small problems are bound by the meetings of a team's
+// CTAs (a CTA of its own meets nobody, a cluster meets in hardware, a slice of the grid through a
+// counter in the L2), large ones by the work, the weights an SM can hold and what the L2 delivers.
+Config choose_config(const Layout& y, int sms, const int* max_clusters) {
+  const Dims d = dims(y);
+  Config best;
+  double best_cyc = 0;
+  auto consider = [&](int T, int teams, bool cluster) {
+    if (teams < 1) return;
+    Config c;
+    c.T = T; c.cluster = cluster;
+    c.rows = ceil_div(y.B, std::min(teams, y.B));
+    c.teams = ceil_div(y.B, c.rows);
+    const double cyc = finish(y, d, c);
+    if (cyc >= 0 && (!best.ok || cyc < best_cyc)) { best = c; best_cyc = cyc; best.cycles = cyc; }
+  };
+  for (int i = 0; i <= 4; ++i) consider(1 << i, std::min(max_clusters[i], sms >> i), true);
+  for (int teams = 1; teams <= sms / 17; ++teams) consider(sms / teams, teams, false);
+  return best;
+}
+
+bool supported(const mebptt_lstm_desc* d) {
+  Layout y;
+  state_layout(d, y);
+  if (y.tensor_path || y.stepwise_tc || y.stepwise_x3 || y.L > kMaxLayers || y.t >= (1 << 30)) return false;
+  const int clusters[5] = {148, 74, 36, 16, 7};
+  return pod::choose_config(y, 148, clusters).ok || choose_config(y, 148, clusters).ok;
+}
+
+namespace {
+
+// Places each task in the earliest phase after everything it depends on.  Tasks come in the order of
+// the tape, so whatever an operation must wait for has its phase already.
+struct Scheduler {
+  const Layout& y;
+  const Config& c;
+  const Dims d;
+  Schedule& s;
+  std::vector<std::vector<Task>> open;     // tasks by phase, from phase `base` on
+  std::vector<int> used;                   // floats of the pool taken, likewise
+  int64_t base = 0;                        // phases before this one belong to earlier launches
+  int64_t top = -1;                        // last phase used
+  // when the cells (units) of the arena were last touched; the same for ping, pong and the two cores,
+  // per layer there (what lies in them always has the same format, so layers never share bytes)
+  std::vector<int64_t> cell, named;
+  // when the state at a location was written, per layer
+  std::vector<int64_t> state;              // [location slot][L]
+  std::vector<int64_t> bwd_prev;           // per layer: phase of the latest B
+  int core = 0;                            // the working core alternates between two buffers
+  uint32_t base_pingpong[2], base_core[2], base_arena, loc_step;
+
+  Scheduler(const Layout& y_, const Config& c_, Schedule& s_, int64_t arena_units)
+      : y(y_), c(c_), d(dims(y_)), s(s_), cell((size_t)arena_units, -1), named((size_t)4 * y_.L, -1), state((size_t)(arena_units + 5) * y_.L, -1),
+        bwd_prev((size_t)y_.L, -1) {
+    base_pingpong[0] = (uint32_t)(y.off_ping >> 8); base_pingpong[1] = (uint32_t)(y.off_pong >> 8);
+    base_core[0] = (uint32_t)(y.off_core >> 8); base_core[1] = (uint32_t)(y.off_core2 >> 8);
+    base_arena = (uint32_t)(y.off_arena >> 8);
+    loc_step = (uint32_t)(y.loc_bytes >> 8);
+  }
+  uint32_t address(int32_t loc) const {
+    switch (loc) {
+      case MEBPTT_LOC_INIT: return kInit;
+      case MEBPTT_LOC_PING: return base_pingpong[0];
+      case MEBPTT_LOC_PONG: return base_pingpong[1];
+      case MEBPTT_LOC_CORE: return base_core[core];
+      default: return base_arena + (uint32_t)loc * loc_step;
+    }
+  }
+  int64_t* state_of(int32_t loc) {
+    const size_t slot = loc >= 0 ? (size_t)loc + 5
+                        : loc == MEBPTT_LOC_INIT ? 0 : loc == MEBPTT_LOC_PING ? 1 : loc == MEBPTT_LOC_PONG ? 2 : 3 + (size_t)core;
+    return state.data() + slot * (size_t)y.L;
+  }
+  int units(int32_t loc, int fmt) const {   // cells a record takes
+    if (loc < 0) return 1;
+    const size_t bytes = fmt == MEBPTT_FMT_HIDDEN ? y.unit : fmt == MEBPTT_FMT_INTERNAL ? y.rec : y.rec_in;
+    return (int)((bytes + y.loc_bytes - 1) / y.loc_bytes);
+  }
+  template <class F> void cells(int32_t loc, int n, int l, F f) {
+    if (loc >= 0) { for (int i = 0; i < n && (size_t)(loc + i) < cell.size(); ++i) f(cell[(size_t)(loc + i)]); }
+    else if (loc != MEBPTT_LOC_INIT)
+      f(named[(size_t)(loc == MEBPTT_LOC_PING ? 0 : loc == MEBPTT_LOC_PONG ? 1 : 2 + core) * y.L + (size_t)l]);
+  }
+  int64_t last_touch(int32_t loc, int n, int l) {
+    int64_t p = -1;
+    cells(loc, n, l, [&](int64_t& v) { p = std::max(p, v); });
+    return p;
+  }
+  void touch(int32_t loc, int n, int l, int64_t phase) {
+    cells(loc, n, l, [&](int64_t& v) { v = std::max(v, phase); });
+  }
+  int64_t place(Task t, int64_t after, Need n) {
+    int64_t p = std::max(after + 1, base);
+    const int need = (n.a + n.red + 3) & ~3;
+    for (;; ++p) {
+      const size_t i = (size_t)(p - base);
+      if (i >= open.size()) { open.resize(i + 1); used.resize(i + 1, 0); }
+      if ((int)open[i].size() < kMaxPhaseTasks && used[i] + need <= c.pool_floats) {
+        t.a_off = (uint32_t)used[i];
+        t.red_off = (uint32_t)(used[i] + n.a);
+        used[i] += need;
+        open[i].push_back(t);
+        break;
+      }
+    }
+    top = std::max(top, p);
+    return p;
+  }
+  // Ends a launch: everything placed so far is emitted, later tasks start in new phases.
+  void close(int chunk) {
+    Launch cur;
+    cur.task0 = s.tasks.size();
+    auto pad = [&] { while (s.tasks.size() % kTaskWindow) s.tasks.push_back(Task{}); };
+    auto end = [&](int ch) {
+      pad();
+      cur.ntasks = s.tasks.size() - cur.task0;
+      cur.chunk = ch;
+      s.launches.push_back(cur);
+      cur = Launch{};
+      cur.task0 = s.tasks.size();
+    };
+    for (auto& ph : open) {
+      if (ph.empty()) continue;
+      if (s.tasks.size() % kTaskWindow + ph.size() > (size_t)kTaskWindow) pad();
+      if (s.tasks.size() - cur.task0 + kTaskWindow > kMaxLaunchTasks) end(-1);
+      ph.back().flags |= LAST;
+      s.tasks.insert(s.tasks.end(), ph.begin(), ph.end());
+      ++cur.phases;
+    }
+    end(chunk);
+    s.phases += s.launches.back().phases;
+    open.clear();
+    used.clear();
+    base = top + 1;
+  }
+  void forward(const mebptt_op& op) {
+    const uint32_t src = address(op.src);
+    const std::vector<int64_t> in(state_of(op.src), state_of(op.src) + y.L);
+    if (op.dst == MEBPTT_LOC_CORE) core ^= 1;   // (never the source as well: a valid tape does not read what it writes)
+    const int n = units(op.dst, op.dst_fmt), n_src = units(op.src, MEBPTT_FMT_HIDDEN);
+    const int64_t arena_free = op.dst >= 0 ? last_touch(op.dst, n, 0) : -1;   // before any layer of this operation
+    int64_t below = -1, last = -1;
+    int64_t* out = state_of(op.dst);
+    for (int l = 0; l < y.L; ++l) {
+      Task t{};
+      t.kind = FWD; t.layer = (uint8_t)l; t.k = (int32_t)op.k;
+      t.src = src; t.dst = address(op.dst);
+      if (op.dst_fmt != MEBPTT_FMT_HIDDEN) t.flags |= GATES;
+      if (op.dst_fmt == MEBPTT_FMT_INTERNAL) t.flags |= COPY_IN;
+      if (l == 0) t.flags |= COUNT;
+      const int64_t free_at = op.dst >= 0 ? arena_free : last_touch(op.dst, n, l);
+      const int64_t p = place(t, std::max(std::max(in[(size_t)l], below), free_at), need_f(y, d, c, l));
+      out[l] = p;
+      below = p;
+      last = std::max(last, p);
+      if (op.dst < 0) touch(op.dst, n, l, p);
+      if (op.dst < 0 && l > 0) touch(op.dst, n, l - 1, p);
+      if (op.src < 0) touch(op.src, n_src, l, p);
+    }
+    if (op.dst >= 0) touch(op.dst, n, 0, last);
+    if (op.src >= 0) touch(op.src, n_src, 0, last);
+  }
+  void backward(const mebptt_op& op) {
+    const int sidx = (int)((op.k - 1) % y.S);
+    const int64_t* in = state_of(op.src);
+    Task t{};
+    t.kind = READ; t.layer = (uint8_t)(y.L - 1); t.k = (int32_t)op.k; t.sidx = (uint32_t)sidx;
+    t.src = address(op.src);
+    int64_t above = place(t, in[y.L - 1], need_r(y, d, c)), last = above;
+    for (int l = y.L - 1; l >= 0; --l) {
+      Task b{};
+      b.kind = BWD; b.layer = (uint8_t)l; b.k = (int32_t)op.k; b.sidx = (uint32_t)sidx;
+      b.src = address(op.src);
+      int64_t after = std::max(std::max(in[l], above), bwd_prev[(size_t)l]);
+      if (op.dst_fmt == MEBPTT_FMT_INTERNAL) {
+        b.dst = b.src + (uint32_t)(y.rec_in >> 8);
+      } else {
+        b.dst = address(op.aux);
+        after = std::max(after, state_of(op.aux)[l]);
+      }
+      if (op.k == y.t || sidx == y.S - 1) b.flags |= CARRY_IN;
+      if (sidx == 0) b.flags |= CARRY_OUT;
+      if (l == y.L - 1) b.flags |= COUNT;
+      const int64_t p = place(b, after, need_b(y, d, c, l));
+      bwd_prev[(size_t)l] = p;
+      above = p;
+      last = std::max(last, p);
+    }
+    // (every layer at once: the working core is rewritten no sooner than two forward operations later)
+    for (int l = 0; l < (op.src < 0 ? y.L : 1); ++l) touch(op.src, units(op.src, op.dst_fmt), l, last);
+    if (op.dst_fmt != MEBPTT_FMT_INTERNAL)
+      for (int l = 0; l < (op.aux < 0 ? y.L : 1); ++l) touch(op.aux, units(op.aux, MEBPTT_FMT_HIDDEN), l, last);
+  }
+};
+
+}  // namespace
+
+void build_schedule(const Layout& y, const Plan* p, const Config& c, Schedule& s) {
+  Scheduler w(y, c, s, y.arena_units);
+  for (const mebptt_op& op : p->tape) {
+    if (op.kind == MEBPTT_OP_FWD) {
+      w.forward(op);
+    } else {
+      w.backward(op);
+      if ((op.k - 1) % y.S == 0) w.close((int)((op.k - 1) / y.S));
+    }
+    // a tape with very many recomputations between two backward operations: do not hold it all open
+    if (w.open.size() > 4 * kMaxLaunchTasks) w.close(-1);
+  }
+}
+
+}  // namespace team
+}  // namespace mebptt

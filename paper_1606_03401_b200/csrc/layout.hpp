@@ -35,6 +35,7 @@ struct Layout {
   bool tensor_path = false;
   bool stepwise_tc = false;   // step-by-step operations with their contractions on the tensor cores
   bool stepwise_x3 = false;   // likewise for float32 storage, operands split into bfloat16 halves
+  bool tensor_cores = true;   // not forbidden by the caller
   bool gru = false;           // the core is a GRU (CUDA-core kernels)
   bool team = false;          // CUDA-core shapes walked by the persistent kernel of team.cu
   int NG = 4;                 // row blocks of H rows in a layer's weight matrix and bias: 4 (LSTM) or 3 (GRU)
@@ -130,6 +131,7 @@ inline void state_layout(const mebptt_lstm_desc* d, Layout& y) {
   y.dtype = d->dtype; y.t = d->t;
   y.gru = (d->flags & MEBPTT_FLAG_GRU) != 0;
   y.NG = y.gru ? 3 : 4;
+  y.tensor_cores = (d->flags & MEBPTT_FLAG_NO_TENSOR_CORES) == 0;
   y.tensor_path = tensor_path_supported(d);
   y.stepwise_tc = stepwise_tc_supported(d);
   y.stepwise_x3 = stepwise_x3_supported(d);
@@ -239,14 +241,19 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     if (y.S > y.t) y.S = (int)y.t;
     const size_t rows = (size_t)y.S * y.B;
     y.off_core2 = take(y.rec);   // the working core alternates, so that one leaf's forward operation can pass the last one's backward
+    // packed weights, in whichever of the two kernels' orders is used (the pod kernel pads rows, and
+    // units to its CTAs: at most 16 and 96 more)
+    auto larger = [](size_t u, size_t v) { return u > v ? u : v; };
     for (int l = 0; l < y.L; ++l) {
-      y.off_wf[l] = take(G * (align_up(l ? y.H : y.I, 8) + hp) * y.esz);
+      const size_t in = l ? y.H + 96 : align_up(y.I, 16);
+      y.off_wf[l] = take(larger(G * (align_up(l ? y.H : y.I, 8) + hp), 4 * ((size_t)y.H + 16) * (in + y.H + 104)) * y.esz);
       y.off_wb[l] = take(h4 * (gp + (l + 1 < y.L ? gp : align_up(y.O, 8))) * y.esz);
     }
-    y.off_wr = take(align_up(y.O, 4) * hp * y.esz);
+    y.off_wr = take(larger(align_up(y.O, 4) * hp, ((size_t)y.O + 64) * (y.H + 104)) * y.esz);
+    y.off_init = take(y.unit);   // the caller's initial state, laid out like a hidden state
     y.off_st_dz = y.off_dz = take((size_t)y.L * rows * G * 4);
-    y.off_st_h = take((size_t)y.L * rows * y.H * y.esz);
-    y.off_st_hp = take((size_t)y.L * rows * y.H * y.esz);
+    // h of the chunk's steps and of the one before: row block i holds h_{k-1} of the step in block i of dz
+    y.off_st_h = take((size_t)y.L * (rows + y.B) * y.H * y.esz);
     y.off_dy = take(rows * y.O * 4);
     // what a step clears: carried gradients, the teams' counters, status
     y.off_dc = take((size_t)y.L * bh4);
@@ -255,7 +262,7 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     y.off_sync = take(y.n_sync * 4);
     y.off_status = take(256);
     y.off_zero_end = o;
-    size_t tasks = 4 * ((size_t)p->cost * y.L + (size_t)y.t * (y.L + 1));   // with the load tasks of the pod kernel
+    size_t tasks = 5 * ((size_t)p->cost * y.L + (size_t)y.t * (y.L + 2));   // with the headers and load tasks of the pod kernel
     tasks += tasks / 4 + 256;   // windows are filled up where a phase would straddle two
     y.tape_bytes = (tasks < team::kMaxLaunchTasks ? align_up(tasks, 64) : team::kMaxLaunchTasks) * 32;
     y.off_tape = take(y.tape_bytes);

@@ -1,16 +1,24 @@
 // The pod kernel: the team path's small and middle sizes, where a phase is a fraction of a microsecond
-// of arithmetic and everything else is the distance between the CTAs.
+// of arithmetic and everything else is the distance between the CTAs and the instructions in front of
+// and behind it.
 //
-// A pod is a thread-block cluster that walks the tape for NB batch rows.  What a phase produces for
-// the others -- h of a layer, dz, dy -- is pushed straight into the operand slots in every CTA's shared
-// memory (asynchronous stores that count their bytes on the receiver's barrier), so that the next
-// phase starts from shared memory; nothing crosses CTAs through global memory.  Everything else a
-// task reads there (cell states, gates, carried gradients, a stored state that comes back) was
-// written by the same thread, and is fetched one phase ahead.
+// A pod is a thread-block cluster of T CTAs that walks the tape for NB batch rows.  CTA r owns U hidden
+// units of every layer: their four gate rows of [W_ih | W_hh], U rows of carried state, a share of the
+// readout rows.  One copy of a CTA's weights, in shared memory, serves both directions:
 //
-// Which vector lies in which slot at which phase is decided on the host, like registers by a
-// compiler: a state that is not in a slot any more when it is needed is brought back by a load task
-// in the phase before.
+//   F(op, l)  z of the own units from all of the input and of h_{k-1}, which every CTA holds: h_k of the
+//             own units is pushed to all CTAs
+//   B(op, l)  dz_k of the own units, whose products with the own weight rows are shares of dh_{k-1} (and
+//             of the gradient of the layer below) for all units: each is pushed to the unit's owner, who
+//             adds the T shares in rank order
+//   R(op)     readout rows of the CTA, dy;  D(op)  their shares of the gradient entering the top layer
+//   Z(l)      B without the cell part, from the carried dz of the chunk after: at the start of a launch
+//
+// Pushes are asynchronous stores into the other CTAs' shared memory that count their bytes on the
+// receiver's barrier.  Nothing crosses CTAs through global memory; what a task reads there was written
+// by the same thread, and is fetched one phase ahead.  Which state lies in which slot of shared memory
+// at which phase is decided on the host, like registers by a compiler: a state that is no longer there
+// when it is needed comes back by a load task in the phase before.
 #pragma once
 
 #include <cstdint>
@@ -20,52 +28,82 @@
 #include "plan.hpp"
 #include "team.hpp"
 
+#ifdef __CUDACC__
+#define MEBPTT_BOTH __host__ __device__
+#else
+#define MEBPTT_BOTH
+#endif
+
 namespace mebptt {
 namespace pod {
 
 using team::kThreads;
 using team::kWarps;
-constexpr int kWindow = 64, kWindows = 4;     // tasks fetched at a time, windows held
-constexpr int kPhaseTasks = 12;
-constexpr int kHSlots = 4, kXSlots = 4, kDzSlots = 2, kDySlots = 4;   // operand slots (h, dz: per layer)
-constexpr uint16_t kNone = 0xffff;
+constexpr int kMaxLayers = 8;
+constexpr int kWindow = 64, kWindows = 4;     // records fetched at a time, windows held
+constexpr int kHSlots = 4, kXSlots = 4;       // h of a layer; x
 
-enum Kind : uint8_t { NOP = 0, FWD = 1, READ = 2, BWD = 3, LOAD_H = 4, LOAD_X = 5, LOAD_DZ = 6 };
+enum Kind : uint8_t { NOP = 0, FWD = 1, READ = 2, BWD = 3, LOAD_H = 4, LOAD_X = 5, DHA = 6, CARRY = 7 };
 enum Flag : uint8_t {
   GATES = 1, COPY_IN = 2,   // F: what the destination keeps
-  CARRY = 4,                // LOAD_DZ: from the carry buffer (else from the stage)
-  CARRY_OUT = 8,            // B: leave dz in the carry buffer too
-  COUNT = 16
+  FIRST = 4,                // B: nothing comes from step k + 1
+  OPEN = 8,                 // B: the chunk's last step: h_k goes to the stage as well
+  CLOSE = 16,               // B: the chunk's first step: dz_k goes to the carry buffer, no share for step k - 1
+  COUNT = 32
+};
+// A phase: a header, then its tasks.  At most one F or B, one load and one Z per layer, one R, one D
+// and one LOAD_X in a phase.
+struct Header {
+  uint8_t n;                // tasks; 0: nothing but padding up to the next window
+  uint8_t cells;            // has B or Z: dz is formed before the products
+  uint8_t sums;             // has F or R: partial sums are read after the products
+  uint8_t n_h, n_p, n_x;    // pushes every CTA receives of: h, shares, x
+  uint8_t r, d, x, pad[3];  // 1 + index of the READ, DHA, LOAD_X task; 0: none
+  uint32_t main, load, carry;   // 4 bits per layer: 1 + index of its F or B, of its load, of its Z
+  uint32_t pad2[2];
 };
 struct Task {
-  uint8_t kind, layer, flags, n;   // n: tasks of the phase, in its first task
+  uint8_t kind, layer, flags, pad0;
   int32_t k;
-  uint32_t src, dst;               // as team::Task; LOAD_H: src is the state
-  uint16_t sidx, sa, sb, so;       // row block in the stages; slots of the two operand segments and of the result (16-float units)
-  uint16_t red, pad[3];            // partial sums, 4-float units
+  uint32_t src, dst;        // F: input state, record written; B: record of step k, state k-1; LOAD_H: the state.  256-byte units
+  uint16_t sidx, sa, sb, so;   // row block of step k in the stages; slots of the operands (input, h) and of the result, 16-byte units
+  uint32_t pad[2];
 };
-static_assert(sizeof(Task) == 32, "Task layout");
+static_assert(sizeof(Header) == 32 && sizeof(Task) == 32, "records");
+constexpr uint16_t kNone = 0xffff;
+constexpr int kPhaseTasks = 14;
 
 struct Config {
   bool ok = false;
-  double cycles = 0;               // estimate for two forward operations and one backward operation
+  double cycles = 0;        // estimate for two forward operations and one backward operation
   int T = 1, nb = 1, pods = 1;
-  int ns_f[team::kMaxLayers] = {}, ns_b[team::kMaxLayers] = {}, ns_r = 1;
-  uint64_t resident = 0;           // as team::Config
-  int slot_floats = 0, red_floats = 0;   // all slots; partial sums of one phase (there are two such areas)
-  int x_slot = 0, h_slot = 0, dz_slot = 0, dy_slot = 0;   // floats of one slot
+  int U = 0, up = 0;        // units per CTA, the same padded to 4
+  int kx = 0, kh = 0;       // padded widths of x and of h (units in the order of their owners, `up` each)
+  int rows_o = 0, op = 0;   // readout rows per CTA, the same padded to 4
+  int extra = 0;            // elements added to a row of weights against bank conflicts
+  int ns_f[kMaxLayers] = {}, ns_r = 1, ns_b = 1;   // parts the contraction index is cut into; shares a CTA sends per unit
+  bool mma = false;         // bfloat16 weights on the tensor cores (else FMA on widened values)
+  bool resident = false;    // the weights fit in shared memory
+  int planes = 1;           // mma: bfloat16 planes a float32 gradient is split into
+  // byte offsets from the start of the operand area, and sizes
+  int x_slot = 0, h_slot = 0, pitch_x = 0, pitch_h = 0;   // pitches: bytes of one batch row
+  int at_h = 0, at_p = 0, p_slot = 0, at_dz = 0, dz_buf = 0, dz_pitch = 0, at_dy = 0, dy_buf = 0, dy_pitch = 0;
+  int at_red = 0, red_bytes = 0, at_dummy = 0, at_map = 0, at_w = 0;
   int smem = 0;
+  MEBPTT_BOTH int pitch_w(int l) const { return (l ? kh : kx) + kh + extra; }   // elements of a row of layer l's weights
+  MEBPTT_BOTH int pitch_r() const { return kh + extra; }
+  MEBPTT_BOTH int slot_x(int i) const { return i * x_slot; }
+  MEBPTT_BOTH int slot_h(int l, int i) const { return at_h + (l * kHSlots + i) * h_slot; }
 };
-// first float of a slot
-int slot_x(const Config& c, int i);
-int slot_h(const Layout& y, const Config& c, int l, int i);
-int slot_dz(const Layout& y, const Config& c, int l, int i);
-int slot_dy(const Layout& y, const Config& c, int i);
+inline int kin(const Config& c, int l) { return l ? c.kh : c.kx; }
 
-Config choose_config(const Layout& y, int sms, const int* max_clusters);
+Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max_clusters);
+// elements of the packed weights: layer l, readout
+size_t packed_elems(const Config& c, int l);
+size_t packed_readout_elems(const Config& c);
 
 struct Schedule {
-  std::vector<Task> tasks;
+  std::vector<Task> tasks;   // records
   std::vector<team::Launch> launches;
 };
 void build_schedule(const Layout& y, const Plan* p, const Config& c, Schedule& s);

@@ -1,5 +1,6 @@
 // Host side of the pod kernel: sizes, and the schedule of phases with the operand slots worked out.
 #include <algorithm>
+#include <cstring>
 #include <unordered_map>
 
 #include "pod.hpp"
@@ -9,80 +10,100 @@ namespace pod {
 
 namespace {
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
-inline int pad16(int v) { return (v + 15) & ~15; }
-inline int slices(int k) { return ceil_div(k, 128); }
+inline int up_to(int v, int m) { return (v + m - 1) / m * m; }
+inline int slices(int k) { return ceil_div(k, 128); }   // FMA: a warp takes 128 elements of the contraction index at a time
 }  // namespace
 
-int slot_x(const Config& c, int i) { return i * c.x_slot; }
-int slot_h(const Layout& y, const Config& c, int l, int i) { (void)y; return kXSlots * c.x_slot + (l * kHSlots + i) * c.h_slot; }
-int slot_dz(const Layout& y, const Config& c, int l, int i) {
-  return kXSlots * c.x_slot + y.L * kHSlots * c.h_slot + (l * kDzSlots + i) * c.dz_slot;
-}
-int slot_dy(const Layout& y, const Config& c, int i) {
-  return kXSlots * c.x_slot + y.L * (kHSlots * c.h_slot + kDzSlots * c.dz_slot) + i * c.dy_slot;
-}
+size_t packed_elems(const Config& c, int l) { return (size_t)c.T * 4 * c.U * c.pitch_w(l); }
+size_t packed_readout_elems(const Config& c) { return (size_t)c.T * c.op * c.pitch_r(); }
 
 // The pod size and the batch rows per pod with the least estimated time.  Rows are cheap until the
 // arithmetic of a phase shows beside its fixed part, CTAs until the pushes to all of them do; pods
-// that do not fit the device at once take turns.
-Config choose_config(const Layout& y, int sms, const int* max_clusters) {
-  const team::Dims d = team::dims(y);
+// that do not fit the device at once take turns.  The tensor cores want their weights in shared memory;
+// the FMA path can read them from the L2, which then bounds it.
+Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max_clusters) {
   Config best;
+  const int esz = (int)y.esz;
+  if (y.L > kMaxLayers || (y.dtype == MEBPTT_BF16 && !tensor_cores)) return best;
   for (int lt = 0; lt <= 4; ++lt)
     for (int nb = 1; nb <= 8; nb *= 2) {
       Config c;
       c.T = 1 << lt; c.nb = nb; c.pods = ceil_div(y.B, nb);
       const int fit = std::min(max_clusters[lt], sms >> lt);
-      if (fit < 1 || c.T > y.H) continue;
-      const int u = ceil_div(y.H, c.T), gb = ceil_div(u, 4), gr = ceil_div(d.groups_o, c.T), esz = (int)y.esz;
-      auto parts = [](int groups, int its) { return std::max(1, std::min(its, kWarps / std::max(1, groups))); };
-      c.x_slot = pad16(nb * d.ip[0]); c.h_slot = pad16(nb * d.hp); c.dz_slot = pad16(nb * d.gp); c.dy_slot = pad16(nb * ((y.O + 7) & ~7));
-      c.slot_floats = kXSlots * c.x_slot + y.L * (kHSlots * c.h_slot + kDzSlots * c.dz_slot) + kDySlots * c.dy_slot;
-      if (c.slot_floats / 16 >= kNone) continue;
-      c.ns_r = parts(gr, slices(d.hp));
-      int sum_f = 0, sum_b = 0, most = gr * c.ns_r;
-      double cyc_f = 0, cyc_b = 0;
-      int64_t bytes_f[team::kMaxLayers], bytes_b[team::kMaxLayers], bytes_r = (int64_t)gr * 4 * d.hp * esz, all = bytes_r;
-      for (int l = 0; l < y.L; ++l) {
-        const int its_f = slices(d.ip[l]) + slices(d.hp), its_b = slices(d.gp) + slices(d.kb[l] - d.gp);
-        c.ns_f[l] = parts(u, its_f); c.ns_b[l] = parts(gb, its_b);
-        sum_f += u * c.ns_f[l]; sum_b += gb * c.ns_b[l];
-        most = std::max(most, std::max(u * c.ns_f[l], gb * c.ns_b[l]));
-        bytes_f[l] = (int64_t)u * 4 * d.kf[l] * esz; bytes_b[l] = (int64_t)gb * 4 * d.kb[l] * esz;
-        all += bytes_f[l] + bytes_b[l];
-      }
-      // room for a phase of the wavefront over all layers in both directions, with the readout
-      c.red_floats = std::max(most, sum_f + sum_b + gr * c.ns_r) * nb * 4;
-      const int fixed = kWindows * kWindow * (int)sizeof(Task) + 2048;
-      int64_t left = team::kSmemMax - fixed - ((int64_t)c.slot_floats + 2 * c.red_floats) * 4;
-      if (left < 0) continue;
-      int64_t held = 0;
-      auto keep = [&](int bit, int64_t bytes) {
-        if (bytes <= left) { c.resident |= 1ull << bit; left -= bytes; held += bytes; }
+      if (fit < 1 || c.T > y.H || (nb > 1 && nb >= 2 * y.B)) continue;
+      c.mma = y.dtype == MEBPTT_BF16;
+      c.planes = 3;
+      c.U = ceil_div(y.H, c.T); c.up = up_to(c.U, 4);
+      c.kx = up_to(y.I, c.mma ? 16 : 4); c.kh = up_to(c.T * c.up, c.mma ? 32 : 4);
+      c.rows_o = ceil_div(y.O, c.T); c.op = up_to(c.rows_o, 4);
+      c.extra = c.mma ? 8 : 0;
+      if (y.L * c.up * nb > kThreads || c.op * nb > kThreads || ceil_div(ceil_div(y.I, 4), c.T) * nb > kThreads) continue;
+      int64_t weights = (int64_t)c.op * c.pitch_r() * esz;
+      for (int l = 0; l < y.L; ++l) weights += (int64_t)4 * c.U * c.pitch_w(l) * esz;
+      // parts of the contractions
+      const int ng = ceil_div(c.U, 8);
+      // a power of two; a piece of work has a fixed part, so none is cut below 8 steps of the tensor cores
+      auto parts = [&](int groups, int steps) {
+        int n = 1;
+        while (2 * n <= (c.mma ? steps / 8 : steps) && 2 * n * groups <= kWarps) n *= 2;
+        return n;
       };
-      for (int l = 0; l < y.L; ++l) keep(2 * l, bytes_f[l]);
-      for (int l = 0; l < y.L; ++l) keep(2 * l + 1, bytes_b[l]);
-      keep(63, bytes_r);
-      c.smem = fixed + (c.slot_floats + 2 * c.red_floats) * 4 + (int)held;
+      for (int l = 0; l < y.L; ++l)
+        c.ns_f[l] = c.mma ? parts(ng, (kin(c, l) + c.kh) / 16) : parts(c.U, slices(kin(c, l)) + slices(c.kh));
+      c.ns_r = c.mma ? parts(ceil_div(c.op, 16), c.kh / 16) : parts(c.op / 4, slices(c.kh));
+      c.ns_b = c.mma ? 1 : c.kh <= kThreads / 4 ? 4 : c.kh <= kThreads / 2 ? 2 : 1;
+      // the operand area
+      c.pitch_x = c.mma ? (c.kx + 8) * 2 : c.kx * 4;
+      c.pitch_h = c.mma ? (c.kh + 8) * 2 : c.kh * 4;
+      c.x_slot = up_to(nb * c.pitch_x, 16); c.h_slot = up_to(nb * c.pitch_h, 16);
+      int at = 0;
+      auto take = [&](int64_t bytes) { const int r = at; at += (int)std::min<int64_t>((bytes + 15) & ~15ll, 1 << 26); return r; };
+      take((int64_t)kXSlots * c.x_slot);
+      c.at_h = take((int64_t)y.L * kHSlots * c.h_slot);
+      c.p_slot = up_to(c.T * c.ns_b * c.U * nb * 4, 16);
+      c.at_p = take((int64_t)4 * y.L * c.p_slot);
+      c.dz_pitch = (up_to(4 * c.U, 16) + 8) * 2; c.dy_pitch = (up_to(c.op, 16) + 8) * 2;
+      c.dz_buf = c.mma ? c.planes * nb * c.dz_pitch : 4 * c.U * nb * 4;
+      c.dy_buf = c.mma ? c.planes * nb * c.dy_pitch : c.op * nb * 4;
+      c.dz_buf = up_to(c.dz_buf, 16); c.dy_buf = up_to(c.dy_buf, 16);
+      c.at_dz = take((int64_t)2 * y.L * c.dz_buf);
+      c.at_dy = take((int64_t)2 * c.dy_buf);
+      int64_t red = c.mma ? (int64_t)ceil_div(c.op, 16) * 16 * c.ns_r * nb * 4 : (int64_t)c.op * c.ns_r * nb * 4;
+      for (int l = 0; l < y.L; ++l) red += (int64_t)(c.mma ? ng * 8 : c.U) * c.ns_f[l] * nb * 16;
+      c.red_bytes = (int)std::min<int64_t>((red + 15) & ~15ll, 1 << 26);
+      c.at_red = take((int64_t)2 * c.red_bytes);
+      c.at_dummy = take(64);
+      c.at_map = take((int64_t)c.kh * 8);
+      if (at / 16 >= kNone) continue;
+      c.at_w = at;
+      const int fixed = kWindows * kWindow * (int)sizeof(Task) + 1024;
+      const int64_t left = team::kSmemMax - fixed - at;
+      if (left < 0) continue;
+      c.resident = weights <= left;
+      if (c.mma && !c.resident) continue;
+      c.smem = fixed + at + (c.resident ? (int)weights : 0);
       const int waves = ceil_div(c.pods, fit);
       const double active = (double)std::min(c.pods, fit) * c.T;
-      auto cycles = [&](int groups, int its, int k, int ns, bool res) {
-        const double through = (double)groups * its * (4.0 * nb + 4.0 * esz);
-        const double chain = (double)ceil_div(groups * ns, kWarps) * (ceil_div(its, ns) * 70.0 + 100.0);
-        double t = std::max(through, chain);
-        if (!res) {
-          const double bytes = (double)groups * 4 * k * esz;
-          t = std::max(t, std::max(bytes / 40.0, bytes * active / 2500.0));
-        }
-        return t;
-      };
+      // (fitted to a scan of T and nb over four problems: a phase's fixed part is some 5000 cycles, whatever it does)
+      double cyc_f = 0, cyc_b = 0;
       for (int l = 0; l < y.L; ++l) {
-        cyc_f += cycles(u, slices(d.ip[l]) + slices(d.hp), d.kf[l], c.ns_f[l], c.resident >> (2 * l) & 1);
-        cyc_b += cycles(gb, slices(d.gp) + slices(d.kb[l] - d.gp), d.kb[l], c.ns_b[l], c.resident >> (2 * l + 1) & 1);
+        const int kk = kin(c, l) + c.kh, nc = l ? kk : c.kh;
+        if (c.mma) {
+          cyc_f += ceil_div(ng * c.ns_f[l], kWarps) * (ceil_div(kk / 16, c.ns_f[l]) * 45.0 + 400.0);
+          cyc_b += ceil_div(nc / 32, kWarps) * (ceil_div(4 * c.U, 16) * c.planes * 45.0 + 600.0);
+        } else {
+          const int its = slices(kin(c, l)) + slices(c.kh);
+          double f = std::max(1.2 * c.U * its * (4.0 * nb + 16.0), ceil_div(c.U * c.ns_f[l], kWarps) * (ceil_div(its, c.ns_f[l]) * 120.0 + 300.0));
+          double b = ceil_div(nc * c.ns_b, kThreads) * (double)ceil_div(4 * c.U, c.ns_b) * std::max(16.0, (3.0 + nb) * kWarps / 4) + 400.0;
+          if (!c.resident) {
+            const double bf = 4.0 * c.U * kk * esz, bb = 4.0 * c.U * nc * esz;
+            f = std::max(f, std::max(bf / 40.0, bf * active / 5000.0));
+            b = std::max(b, std::max(bb / 40.0, bb * active / 5000.0));
+          }
+          cyc_f += f; cyc_b += b;
+        }
       }
-      const double push = 25.0 * c.T;   // what a thread spends on sending a value to every CTA
-      c.cycles = waves * (3 * (1100.0 + (c.T > 1 ? 300.0 : 0.0) + push) + 2 * cyc_f + cyc_b +
-                          cycles(gr, slices(d.hp), d.hp, c.ns_r, c.resident >> 63 & 1));
+      c.cycles = waves * (3 * (4500.0 + 20.0 * c.T) + 2 * cyc_f + cyc_b);
       c.ok = true;
       if (!best.ok || c.cycles < best.cycles) best = c;
     }
@@ -104,20 +125,21 @@ struct Slot { Key key = -1; int read = -9, pushed = -9; };
 struct Builder {
   const Layout& y;
   const Config& c;
-  const team::Dims d;
   Schedule& s;
 
   // ---- phases: each task in the earliest one after everything it depends on ----
   std::vector<std::vector<Item>> open;
-  std::vector<int> red;
+  std::vector<uint32_t> taken;             // classes in a phase: bit l its F or B, 16 R, 17 D
   int64_t base = 0, top = -1, n_open = 0;
-  std::vector<int64_t> cell, named, state, version, b_phase;   // b_phase: [L][4], phase of B(l, k) at k & 3
+  std::vector<int64_t> cell, named, state, version, b_phase, d_phase;   // phases of B(l, k) at [l][k & 3], of D(k) at [k & 3]
   int core = 0;
-  uint32_t at_ping, at_pong, at_core[2], at_arena, loc_step;
+  uint32_t at_init, at_ping, at_pong, at_core[2], at_arena, loc_step;
 
   Builder(const Layout& y_, const Config& c_, Schedule& s_)
-      : y(y_), c(c_), d(team::dims(y_)), s(s_), cell((size_t)y_.arena_units, -1), named((size_t)4 * y_.L, -1),
-        state((size_t)(y_.arena_units + 5) * y_.L, -1), version((size_t)y_.arena_units + 5, 0), b_phase((size_t)4 * y_.L, -1) {
+      : y(y_), c(c_), s(s_), cell((size_t)y_.arena_units, -1), named((size_t)4 * y_.L, -1),
+        state((size_t)(y_.arena_units + 5) * y_.L, -1), version((size_t)y_.arena_units + 5, 0), b_phase((size_t)4 * y_.L, -1),
+        d_phase(4, -1) {
+    at_init = (uint32_t)(y.off_init >> 8);
     at_ping = (uint32_t)(y.off_ping >> 8); at_pong = (uint32_t)(y.off_pong >> 8);
     at_core[0] = (uint32_t)(y.off_core >> 8); at_core[1] = (uint32_t)(y.off_core2 >> 8);
     at_arena = (uint32_t)(y.off_arena >> 8); loc_step = (uint32_t)(y.loc_bytes >> 8);
@@ -128,7 +150,7 @@ struct Builder {
   }
   uint32_t address(int32_t loc) const {
     switch (loc) {
-      case MEBPTT_LOC_INIT: return team::kInit;
+      case MEBPTT_LOC_INIT: return at_init;
       case MEBPTT_LOC_PING: return at_ping;
       case MEBPTT_LOC_PONG: return at_pong;
       case MEBPTT_LOC_CORE: return at_core[core];
@@ -152,22 +174,16 @@ struct Builder {
   void touch(int32_t loc, int n, int l, int64_t phase) {
     cells(loc, n, l, [&](int64_t& v) { v = std::max(v, phase); });
   }
-  int red_of(const Task& t) const {
-    const int u = ceil_div(y.H, c.T);
-    const int w = t.kind == FWD ? u * c.ns_f[t.layer] : t.kind == READ ? ceil_div(d.groups_o, c.T) * c.ns_r : ceil_div(u, 4) * c.ns_b[t.layer];
-    return w * c.nb * 4;
-  }
   int64_t place(const Item& it, int64_t after) {
+    const uint32_t bit = 1u << (it.t.kind == READ ? 16 : it.t.kind == DHA ? 17 : it.t.layer);
     int64_t p = std::max(after + 1, base);
     for (;; ++p) {
       const size_t i = (size_t)(p - base);
-      if (i >= open.size()) { open.resize(i + 1); red.resize(i + 1, 0); }
-      const int need = red_of(it.t);
-      if (open[i].size() < team::kMaxPhaseTasks && red[i] + need <= c.red_floats) {
-        red[i] += need;
-        open[i].push_back(it);
-        break;
-      }
+      if (i >= open.size()) { open.resize(i + 1); taken.resize(i + 1, 0); }
+      if (taken[i] & bit) continue;
+      taken[i] |= bit;
+      open[i].push_back(it);
+      break;
     }
     top = std::max(top, p);
     ++n_open;
@@ -209,14 +225,19 @@ struct Builder {
     r.t = Task{};
     r.t.kind = READ; r.t.layer = (uint8_t)(L - 1); r.t.k = (int32_t)op.k; r.t.sidx = (uint16_t)sidx; r.t.src = address(op.src);
     r.in = version[si];
-    // dy takes the place of dy_{k+4}
-    int64_t above = place(r, std::max(state[si * L + L - 1], b_phase[(size_t)(L - 1) * 4 + q])), last = above;
+    // dy takes the place of dy_{k+2}; its shares that of the ones the top layer used at step k + 2
+    const int64_t pr = place(r, std::max(state[si * L + L - 1], d_phase[(size_t)((q + 2) & 3)]));
+    Item dh;
+    dh.t = r.t;
+    dh.t.kind = DHA;
+    int64_t above = place(dh, std::max(pr, b_phase[(size_t)(L - 1) * 4 + ((q + 2) & 3)])), last = above;
+    d_phase[(size_t)q] = above;
     for (int l = L - 1; l >= 0; --l) {
       Item b;
       b.t = Task{};
       b.t.kind = BWD; b.t.layer = (uint8_t)l; b.t.k = (int32_t)op.k; b.t.sidx = (uint16_t)sidx; b.t.src = address(op.src);
       int64_t after = std::max(std::max(state[si * L + l], above), b_phase[(size_t)l * 4 + ((q + 1) & 3)]);
-      // dz_k takes the place of dz_{k+2}, which the layer below has to have read
+      // its shares for the layer below take the place of those of step k + 2
       if (l > 0) after = std::max(after, b_phase[(size_t)(l - 1) * 4 + ((q + 2) & 3)]);
       if (op.dst_fmt == MEBPTT_FMT_INTERNAL) {
         b.t.dst = b.t.src + (uint32_t)(y.rec_in >> 8);
@@ -224,7 +245,9 @@ struct Builder {
         b.t.dst = address(op.aux);
         after = std::max(after, state[slot_of(op.aux) * L + l]);
       }
-      if (sidx == 0) b.t.flags |= CARRY_OUT;
+      if (op.k == y.t) b.t.flags |= FIRST;
+      if (op.k == y.t || sidx == y.S - 1) b.t.flags |= OPEN;
+      if (sidx == 0) b.t.flags |= CLOSE;
       if (l == L - 1) b.t.flags |= COUNT;
       const int64_t p = place(b, after);
       b_phase[(size_t)l * 4 + q] = p;
@@ -261,7 +284,7 @@ struct Builder {
     for (int i = 0; i < n; ++i) if (pool[i].key == k) return i;
     return -1;
   }
-  static uint16_t u16(int floats) { return (uint16_t)(floats / 16); }
+  static uint16_t u16(int bytes) { return (uint16_t)(bytes / 16); }
 
   void close(int chunk) {
     uses.clear();
@@ -276,74 +299,88 @@ struct Builder {
         }
       }
     std::vector<std::vector<Task>> out;
+    // the launch's first backward operations lack the shares of the step after: from its carried dz
+    {
+      std::vector<Task> z;
+      uint32_t seen = 0;
+      for (const std::vector<Item>& ph : open)
+        for (const Item& it : ph)
+          if (it.t.kind == BWD && !(seen >> it.t.layer & 1)) {
+            seen |= 1u << it.t.layer;
+            if (it.t.flags & FIRST) continue;
+            Task t = it.t;
+            t.kind = CARRY; t.flags = 0;
+            t.sidx = (it.t.flags & OPEN) ? kNone : (uint16_t)(it.t.sidx + 1);   // the stage still holds a step of the same chunk
+            z.push_back(t);
+          }
+      if (!z.empty()) out.push_back(z);
+    }
     Pools pools;
     pools.x.resize(kXSlots);
     pools.h.resize((size_t)y.L * kHSlots);
-    std::vector<int64_t> dz((size_t)y.L * kDzSlots, -1);       // step whose dz lies in a slot
     for (size_t p = 0; p < open.size(); ++p) {
       std::vector<Item> rest(open[p]);
       while (!rest.empty()) {
         const int e = (int)out.size();                          // the phase being put together
         Pools q = pools;
-        std::vector<int64_t> qdz = dz;
         std::vector<Task> now, loads;
         std::vector<Item> later;
         bool gap = false;                                       // a phase of loads has to come first
-        auto operand = [&](Slot* pool, int n, Key key, const Task& load, int slot0, int floats, int& at) {
+        auto loaded = [&](const Task& l) {                      // its class is taken in the phase before
+          auto same = [&](const Task& o) { return o.kind == l.kind && (l.kind == LOAD_X || o.layer == l.layer); };
+          for (const Task& o : out.back()) if (same(o)) return true;
+          for (const Task& o : loads) if (same(o)) return true;
+          return out.back().size() + loads.size() >= (size_t)kPhaseTasks;
+        };
+        auto operand = [&](Slot* pool, int n, Key key, const Task& load, int slot0, int bytes, int& at) {
           int i = find(pool, n, key);
           if (i < 0) {
-            i = e > 0 ? victim(pool, n, e - 1, e, (int)p - 1) : -1;
-            if (i < 0 || (e > 0 && out.back().size() + loads.size() >= (size_t)kPhaseTasks)) { gap = true; return; }
+            i = e > 0 && !loaded(load) ? victim(pool, n, e - 1, e, (int)p - 1) : -1;
+            if (i < 0) { gap = true; return; }
             Task l = load;
-            l.so = u16(slot0 + i * floats);
+            l.so = u16(slot0 + i * bytes);
             loads.push_back(l);
             pool[i].key = key;
             pool[i].pushed = e - 1;
           }
           pool[i].read = e;
-          at = slot0 + i * floats;
+          at = slot0 + i * bytes;
         };
         for (size_t j = 0; j < rest.size() && !gap; ++j) {
           const Item& it = rest[j];
           Task t = it.t;
           const int l = t.layer;
           Slot* hl = q.h.data() + (size_t)l * kHSlots;
-          int a = 0, b = 0;
+          int a = -1, b = -1;
           Task load{};
           load.layer = (uint8_t)l;
-          if (t.kind == FWD || t.kind == READ) {
-            if (t.kind == FWD && l == 0) {
-              load.kind = LOAD_X; load.k = t.k;
-              operand(q.x.data(), kXSlots, key_x(t.k), load, slot_x(c, 0), c.x_slot, a);
-            } else if (t.kind == FWD) {
-              load.kind = LOAD_H; load.layer = (uint8_t)(l - 1); load.src = t.dst;
-              operand(hl - kHSlots, kHSlots, key_h(l - 1, it.out), load, slot_h(y, c, l - 1, 0), c.h_slot, a);
-              load.layer = (uint8_t)l;
-            }
-            if (gap) break;
-            load.kind = LOAD_H; load.src = t.src;
-            operand(hl, kHSlots, key_h(l, it.in), load, slot_h(y, c, l, 0), c.h_slot, b);
-            if (gap) break;
-            if (t.kind == READ) { a = b; b = -1; }
-          } else {
-            const int par = (t.k + 1) & 1;
-            if (qdz[(size_t)l * kDzSlots + par] != t.k + 1) {
-              if (e == 0 || out.back().size() + loads.size() >= (size_t)kPhaseTasks) { gap = true; break; }
-              load.kind = LOAD_DZ; load.k = t.k + 1; load.sidx = (uint16_t)(t.sidx + 1);
-              if (t.k == y.t || t.sidx == y.S - 1) load.flags |= CARRY;
-              load.so = u16(slot_dz(y, c, l, par));
-              loads.push_back(load);
-              qdz[(size_t)l * kDzSlots + par] = t.k + 1;
-            }
-            a = slot_dz(y, c, l, par);
-            b = l + 1 < y.L ? slot_dz(y, c, l + 1, t.k & 1) : slot_dy(y, c, t.k & 3);
+          if (t.kind == FWD && l == 0) {
+            load.kind = LOAD_X; load.k = t.k;
+            operand(q.x.data(), kXSlots, key_x(t.k), load, c.slot_x(0), c.x_slot, a);
+          } else if (t.kind == FWD) {
+            load.kind = LOAD_H; load.layer = (uint8_t)(l - 1); load.src = t.dst;
+            operand(hl - kHSlots, kHSlots, key_h(l - 1, it.out), load, c.slot_h(l - 1, 0), c.h_slot, a);
+            load.layer = (uint8_t)l;
           }
-          t.sa = u16(a);
+          if (gap) break;
+          if (t.kind == FWD || t.kind == READ) {
+            load.kind = LOAD_H; load.src = t.src;
+            operand(hl, kHSlots, key_h(l, it.in), load, c.slot_h(l, 0), c.h_slot, b);
+            if (gap) break;
+          }
+          t.sa = a < 0 ? kNone : u16(a);
           t.sb = b < 0 ? kNone : u16(b);
           now.push_back(t);
           later.push_back(it);
         }
-        if (gap) { out.emplace_back(); continue; }
+        if (gap) {                                              // what was found room for stays
+          if (!loads.empty()) {
+            out.back().insert(out.back().end(), loads.begin(), loads.end());
+            pools = q;
+          }
+          out.emplace_back();
+          continue;
+        }
         // results, once it is known what the phase reads; a task whose result finds no room waits for another phase
         std::vector<Item> wait;
         std::vector<Task> done;
@@ -359,13 +396,8 @@ struct Builder {
               if (i < 0) { wait.push_back(it); continue; }
               Slot& sl = q.h[(size_t)l * kHSlots + (size_t)i];
               sl.key = key; sl.pushed = e;
-              t.so = u16(slot_h(y, c, l, i));
+              t.so = u16(c.slot_h(l, i));
             }
-          } else if (t.kind == READ) {
-            t.so = u16(slot_dy(y, c, t.k & 3));
-          } else {
-            t.so = u16(slot_dz(y, c, l, t.k & 1));
-            qdz[(size_t)l * kDzSlots + (t.k & 1)] = t.k;
           }
           done.push_back(t);
         }
@@ -373,7 +405,6 @@ struct Builder {
         if (!loads.empty()) out.back().insert(out.back().end(), loads.begin(), loads.end());
         out.push_back(done);
         pools = q;
-        dz = qdz;
         rest = wait;
       }
     }
@@ -381,12 +412,28 @@ struct Builder {
     g.task0 = s.tasks.size();
     auto pad = [&] { while (s.tasks.size() % kWindow) s.tasks.push_back(Task{}); };
     for (std::vector<Task>& ph : out) {
-      if (ph.empty()) ph.push_back(Task{});                     // loads for nobody: keeps its place as an empty phase
-      int r = 0;
-      for (Task& t : ph)
-        if (t.kind == FWD || t.kind == READ || t.kind == BWD) { t.red = (uint16_t)(r / 4); r += red_of(t); }
-      if (s.tasks.size() % kWindow + ph.size() > (size_t)kWindow) pad();
-      ph[0].n = (uint8_t)ph.size();
+      if (ph.empty()) ph.push_back(Task{});                     // keeps its place as an empty phase
+      Header h{};
+      h.n = (uint8_t)ph.size();
+      for (size_t i = 0; i < ph.size(); ++i) {
+        const Task& t = ph[i];
+        if (t.flags & COUNT) ++(t.kind == FWD ? g.fwd_ops : g.bwd_ops);
+        const uint32_t at = (uint32_t)(i + 1), nib = at << (4 * t.layer);
+        switch (t.kind) {
+          case FWD: h.main |= nib; h.sums = 1; h.n_h += t.so != kNone; break;
+          case BWD: h.main |= nib; h.cells = 1; h.n_p += (t.flags & CLOSE ? 0 : 1) + (t.layer > 0); break;
+          case READ: h.r = (uint8_t)at; h.sums = 1; break;
+          case DHA: h.d = (uint8_t)at; h.cells = 1; ++h.n_p; break;   // (dy was left by other threads: the barrier before the products)
+          case CARRY: h.carry |= nib; h.cells = 1; ++h.n_p; break;
+          case LOAD_H: h.load |= nib; ++h.n_h; break;
+          case LOAD_X: h.x = (uint8_t)at; ++h.n_x; break;
+          default: break;
+        }
+      }
+      if (s.tasks.size() % kWindow + ph.size() + 1 > (size_t)kWindow) pad();
+      Task rec;
+      memcpy(&rec, &h, sizeof rec);
+      s.tasks.push_back(rec);
       s.tasks.insert(s.tasks.end(), ph.begin(), ph.end());
       ++g.phases;
     }
@@ -395,7 +442,7 @@ struct Builder {
     g.chunk = chunk;
     s.launches.push_back(g);
     open.clear();
-    red.clear();
+    taken.clear();
     n_open = 0;
     base = top + 1;
   }
@@ -414,7 +461,7 @@ void build_schedule(const Layout& y, const Plan* p, const Config& c, Schedule& s
       if ((op.k - 1) % y.S == 0) w.close((int)((op.k - 1) / y.S));
     }
     ++index;
-    if (w.n_open > (int64_t)team::kMaxLaunchTasks / 6) w.close(-1);
+    if (w.n_open > (int64_t)team::kMaxLaunchTasks / 7) w.close(-1);
   }
 }
 

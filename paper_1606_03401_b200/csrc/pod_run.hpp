@@ -13,25 +13,36 @@ namespace pod {
 
 struct Args {
   int L, I, H, O, B, S;
-  int T;
-  team::Dims d;
-  int ns_f[team::kMaxLayers], ns_b[team::kMaxLayers], ns_r;
-  uint64_t resident;
-  int slot_floats, red_floats;
-  size_t hc, csz_off, plane, gsz, rec_gates;   // bytes: layer stride of a hidden state, its c part, gate plane, a layer's planes, planes in a record
+  Config c;
+  size_t hc, csz_off, plane, gsz, rec_gates, rec_in;   // bytes: layer stride of a hidden state, its c part, gate plane, a layer's planes; planes and input state in a record
   char* ws;
-  size_t off_wf[team::kMaxLayers], off_wb[team::kMaxLayers], off_wr;
-  size_t off_dz, off_hk, off_hp, off_dy, off_carry, off_dc;
-  const void *x, *h0;
-  const float *c0, *bias, *b_out, *targets;
+  size_t off_wf[team::kMaxLayers], off_wr;
+  size_t off_dz, off_hk, off_dy, off_carry, off_dc;
+  const void* x;
+  const float *bias, *b_out, *targets;
   const Task* tasks;
-  int n_tasks, phases;
+  int n_tasks, phases, fwd_ops, bwd_ops;
   int* status;
   int64_t* counters;
 };
 
 using Fn = void (*)(const Args);
 Fn kernel(int dtype, bool gru, int nb);
+
+// Packs the weights in the order the kernel keeps them, lays the initial state out, clears what a step
+// starts from at zero.
+struct PackArgs {
+  int L, I, H, O, B;
+  Config c;
+  const void *W, *W_out, *h0;
+  const float* c0;
+  char *wf[kMaxLayers], *wr, *init;
+  size_t w_off[kMaxLayers], hc, csz_off;
+  float* zero;
+  size_t n_zero;
+  int64_t* counters;
+};
+void launch_pack(int dtype, bool gru, const PackArgs& p, cudaStream_t s);
 
 }  // namespace pod
 }  // namespace mebptt

@@ -42,9 +42,9 @@ struct Args {
   size_t rec_gates;                    // bytes into a record
   char* ws;
   size_t off_wf[kMaxLayers], off_wb[kMaxLayers], off_wr;
-  size_t off_dz, off_hk, off_hp, off_dy, off_carry, off_dc;
-  const void *x, *h0;
-  const float *c0, *bias, *b_out, *targets;
+  size_t off_dz, off_hk, off_dy, off_carry, off_dc;
+  const void* x;
+  const float *bias, *b_out, *targets;
   const Task* tasks;
   int n_tasks;
   unsigned* sync;                      // one 128-byte line per team
@@ -128,14 +128,12 @@ __device__ __forceinline__ void stage_any(float* dst, int lda, const T* src, siz
     stage(dst, lda, src, ld, len, padded, nb, valid, tid);
 }
 
-// The state of layer l in a block of whole-stack states (or the caller's initial state).
+// The state of layer l in a block of whole-stack states.
 template <class T>
 __device__ __forceinline__ const T* h_at(const Args& A, uint32_t loc, int l) {
-  if (loc == kInit) return reinterpret_cast<const T*>(A.h0) + (size_t)l * A.B * A.H;
   return reinterpret_cast<const T*>(A.ws + ((size_t)loc << 8) + (size_t)l * A.hc);
 }
 __device__ __forceinline__ const float* c_at(const Args& A, uint32_t loc, int l) {
-  if (loc == kInit) return A.c0 + (size_t)l * A.B * A.H;
   return reinterpret_cast<const float*>(A.ws + ((size_t)loc << 8) + (size_t)l * A.hc + A.csz_off);
 }
 template <class T>
@@ -170,7 +168,7 @@ __device__ __forceinline__ void fetch(const Args& A, const Task& t, size_t row, 
     for (int q = 0; q < 4; ++q) o.v[q] = to_f(ld_l2(g + q * pl));
     o.v[4] = ld_l2(reinterpret_cast<const float*>(A.ws + A.off_dc) + (size_t)l * A.B * H + e);
     o.v[5] = to_f(ld_l2(h_at<T>(A, t.dst, l) + e));   // h_{k-1}
-    o.v[6] = to_f(ld_l2(h_at<T>(A, t.src, l) + e));   // h_k
+    if (t.flags & CARRY_IN) o.v[6] = to_f(ld_l2(h_at<T>(A, t.src, l) + e));   // h_k
     if (!GRU) {
       o.v[7] = ld_l2(c_at(A, t.src, l) + e);
       o.v[8] = ld_l2(c_at(A, t.dst, l) + e);
@@ -216,8 +214,9 @@ __device__ __forceinline__ void apply(const Args& A, const Task& t, size_t row, 
     *reinterpret_cast<float4*>(reinterpret_cast<float*>(A.ws + A.off_dz) + srow * G + 4 * j) = quad;
     if (t.flags & CARRY_OUT)
       *reinterpret_cast<float4*>(reinterpret_cast<float*>(A.ws + A.off_carry) + (((size_t)(t.k & 1) * A.L + l) * A.B + row) * G + 4 * j) = quad;
-    store(reinterpret_cast<T*>(A.ws + A.off_hp) + srow * H + j, o.v[5]);
-    store(reinterpret_cast<T*>(A.ws + A.off_hk) + srow * H + j, o.v[6]);
+    T* hs = reinterpret_cast<T*>(A.ws + A.off_hk) + (((size_t)l * (A.S + 1) + t.sidx) * A.B + row) * H + j;
+    store(hs, o.v[5]);                                                    // h_{k-1}
+    if (t.flags & CARRY_IN) store(hs + (size_t)A.B * H, o.v[6]);          // the chunk's last step: h_k too
   }
 }
 
@@ -445,6 +444,9 @@ struct PackArgs {
   const T *W, *W_out;
   size_t w_off[kMaxLayers];
   T *wf[kMaxLayers], *wb[kMaxLayers], *wr;
+  char* init; size_t hc, csz_off;   // the caller's initial state goes to this block of states
+  const void* h0; const float* c0;
+  int B;
   float* zero; size_t n_zero;     // carried gradients, sync lines, status
   int64_t* counters;
 };
@@ -455,6 +457,12 @@ __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
   const int x = threadIdx.x & 31, y0 = threadIdx.x >> 5, H = P.H;
   for (size_t i = blockIdx.x * 256 + threadIdx.x; i < P.n_zero; i += (size_t)gridDim.x * 256) P.zero[i] = 0.f;
   if (blockIdx.x == 0 && threadIdx.x < 8) P.counters[threadIdx.x] = 0;
+  const size_t bh = (size_t)P.B * H;
+  for (int l = 0; l < P.L; ++l)
+    for (size_t i = blockIdx.x * 256 + threadIdx.x; i < bh; i += (size_t)gridDim.x * 256) {
+      reinterpret_cast<T*>(P.init + l * P.hc)[i] = reinterpret_cast<const T*>(P.h0)[l * bh + i];
+      reinterpret_cast<float*>(P.init + l * P.hc + P.csz_off)[i] = P.c0[l * bh + i];
+    }
   auto tiles = [](int rows, int cols) { return ((rows + 31) / 32) * ((cols + 31) / 32); };
   int total = tiles(P.d.groups_o * 4, P.d.hp);
   for (int l = 0; l < P.L; ++l) total += tiles(4 * H, P.d.kf[l]) + tiles(P.d.groups_h * 4, P.d.kb[l]);
@@ -730,15 +738,15 @@ std::vector<std::shared_ptr<Kept>> g_kept;
 constexpr size_t kKeep = 8, kMaxPinned = (size_t)64 << 20;
 
 bool same_problem(const Layout& a, const Layout& b) {
-  return a.L == b.L && a.I == b.I && a.H == b.H && a.O == b.O && a.B == b.B && a.dtype == b.dtype && a.t == b.t && a.gru == b.gru;
+  return a.L == b.L && a.I == b.I && a.H == b.H && a.O == b.O && a.B == b.B && a.dtype == b.dtype && a.t == b.t && a.gru == b.gru && a.tensor_cores == b.tensor_cores;
 }
 
 std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable) {
   const DeviceFacts f = facts();
   const Config c = choose_config(y, f.sms, f.clusters);
-  const pod::Config pc = pod::choose_config(y, f.sms, f.clusters);
-  if (!c.ok && !pc.ok) return nullptr;
-  const bool use_pod = pc.ok && (!c.ok || pc.cycles <= c.cycles);
+  const pod::Config pc = pod::choose_config(y, y.tensor_cores, f.sms, f.clusters);
+  const bool use_pod = pc.ok && (y.total >> 32) == 0 && (!c.ok || pc.cycles <= c.cycles);
+  if (!c.ok && !use_pod) return nullptr;
   {
     std::lock_guard<std::mutex> lock(g_mu);
     for (size_t i = 0; i < g_kept.size(); ++i) {
@@ -804,6 +812,7 @@ void launch_pack(const Layout& y, const Dims& d, const tc::StepPtrs& io, cudaStr
     P.wb[l] = reinterpret_cast<T*>(io.ws + y.off_wb[l]);
   }
   P.wr = reinterpret_cast<T*>(io.ws + y.off_wr);
+  P.init = io.ws + y.off_init; P.hc = y.hsz + y.csz; P.csz_off = y.hsz; P.h0 = io.h0; P.c0 = io.c0; P.B = y.B;
   P.zero = reinterpret_cast<float*>(io.ws + y.off_dc);
   P.n_zero = (y.off_zero_end - y.off_dc) / 4;
   P.counters = io.counters;
@@ -816,7 +825,10 @@ void fill_products(Products& P, const Layout& y, const tc::StepPtrs& io, bool wa
   const int H = y.H, G = 4 * H, rows = steps * y.B;
   const size_t SB = (size_t)y.S * y.B;
   const float* dz = reinterpret_cast<const float*>(io.ws + y.off_dz);
-  const char *hk = io.ws + y.off_st_h, *hp = io.ws + y.off_st_hp;
+  // a layer's h: row block i is h_{k-1} of the step in block i of dz, block i + 1 its h_k
+  auto h_rows = [&](int l, int block) {
+    return (const void*)(io.ws + y.off_st_h + (((size_t)l * (y.S + 1) + block) * y.B * H) * y.esz);
+  };
   P.n = 0; P.tiles = 0;
   auto add = [&](const float* A, int lda, bool a_mn, const void* B, int ldb, float* C, int ldc, int M, int N, int K, bool acc,
                  int hidden, int skip, int last) {
@@ -826,13 +838,13 @@ void fill_products(Products& P, const Layout& y, const tc::StepPtrs& io, bool wa
   for (int l = 0; l < y.L; ++l) {
     const int I = l ? H : y.I, K = I + H;
     const float* z = dz + (size_t)l * SB * G;
-    const void* in = l ? (const void*)(hk + (size_t)(l - 1) * SB * H * y.esz) : (const void*)(io.x + (size_t)k0 * y.B * I * y.esz);
+    const void* in = l ? h_rows(l - 1, 1) : (const void*)(io.x + (size_t)k0 * y.B * I * y.esz);
     float* dW = io.dW + y.w_layer_offset(l);
     // (GRU: the rows of n meet the input through d n_pre and the state through d q)
     add(z, G, true, in, I, dW, K, G, I, rows, accumulate, H, y.gru ? 3 : -1, 3);
-    add(z, G, true, hp + (size_t)l * SB * H * y.esz, H, dW + I, K, G, H, rows, accumulate, H, y.gru ? 2 : -1, y.gru ? 2 : 3);
+    add(z, G, true, h_rows(l, 0), H, dW + I, K, G, H, rows, accumulate, H, y.gru ? 2 : -1, y.gru ? 2 : 3);
   }
-  add(reinterpret_cast<const float*>(io.ws + y.off_dy), y.O, true, hk + (size_t)(y.L - 1) * SB * H * y.esz, H, io.dW_out, H, y.O, H,
+  add(reinterpret_cast<const float*>(io.ws + y.off_dy), y.O, true, h_rows(y.L - 1, 1), H, io.dW_out, H, y.O, H,
       rows, accumulate, 0, -1, 3);
   if (want_dx) add(dz, G, false, io.W, y.I + H, io.dx + (size_t)k0 * y.B * y.I, y.I, rows, y.I, G, false, H, y.gru ? 3 : -1, 3);
 }
@@ -855,8 +867,20 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     return n;
   }
   const Dims d = dims(y);
-  if (y.dtype == MEBPTT_BF16) launch_pack<__nv_bfloat16>(y, d, io, s);
-  else launch_pack<float>(y, d, io, s);
+  if (kept->pod) {
+    pod::PackArgs q{};
+    q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.c = kept->pc;
+    q.W = io.W; q.W_out = io.W_out; q.h0 = io.h0; q.c0 = io.c0;
+    for (int l = 0; l < y.L; ++l) { q.wf[l] = io.ws + y.off_wf[l]; q.w_off[l] = y.w_layer_offset(l); }
+    q.wr = io.ws + y.off_wr; q.init = io.ws + y.off_init; q.hc = y.hsz + y.csz; q.csz_off = y.hsz;
+    q.zero = reinterpret_cast<float*>(io.ws + y.off_dc); q.n_zero = (y.off_zero_end - y.off_dc) / 4;
+    q.counters = io.counters;
+    pod::launch_pack(y.dtype, y.gru, q, s);
+  } else if (y.dtype == MEBPTT_BF16) {
+    launch_pack<__nv_bfloat16>(y, d, io, s);
+  } else {
+    launch_pack<float>(y, d, io, s);
+  }
 
   Args a{};
   pod::Args pa{};
@@ -864,31 +888,26 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
   pod::Fn pf = nullptr;
   auto common = [&](auto& q) {
     q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.S = y.S;
-    q.d = d;
-    for (int l = 0; l < y.L; ++l) { q.off_wf[l] = y.off_wf[l]; q.off_wb[l] = y.off_wb[l]; }
+    for (int l = 0; l < y.L; ++l) q.off_wf[l] = y.off_wf[l];
     q.off_wr = y.off_wr;
     q.hc = y.hsz + y.csz; q.csz_off = y.hsz; q.plane = y.plane; q.gsz = y.gsz; q.rec_gates = y.rec_gates;
     q.ws = io.ws;
-    q.off_dz = y.off_dz; q.off_hk = y.off_st_h; q.off_hp = y.off_st_hp; q.off_dy = y.off_dy; q.off_carry = y.off_carry; q.off_dc = y.off_dc;
-    q.x = io.x; q.h0 = io.h0; q.c0 = io.c0; q.bias = io.b; q.b_out = io.b_out; q.targets = io.targets;
+    q.off_dz = y.off_dz; q.off_hk = y.off_st_h; q.off_dy = y.off_dy; q.off_carry = y.off_carry; q.off_dc = y.off_dc;
+    q.x = io.x; q.bias = io.b; q.b_out = io.b_out; q.targets = io.targets;
     q.status = reinterpret_cast<int*>(io.ws + y.off_status);
     q.counters = io.counters;
   };
-  auto splits = [&](auto& q, const auto& cfg) {
-    for (int l = 0; l < y.L; ++l) { q.ns_f[l] = cfg.ns_f[l]; q.ns_b[l] = cfg.ns_b[l]; }
-    q.ns_r = cfg.ns_r; q.resident = cfg.resident; q.T = cfg.T;
-  };
   if (kept->pod) {
-    const pod::Config& pc = kept->pc;
     common(pa);
-    splits(pa, pc);
-    pa.slot_floats = pc.slot_floats; pa.red_floats = pc.red_floats;
-    pf = pod::kernel(y.dtype, y.gru, pc.nb);
+    pa.c = kept->pc;
+    pa.rec_in = y.rec_in;
+    pf = pod::kernel(y.dtype, y.gru, pa.c.nb);
     if (allow(reinterpret_cast<const void*>(pf)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
   } else {
     common(a);
-    splits(a, c);
-    a.rows = c.rows; a.cluster = c.cluster ? 1 : 0; a.pool_floats = c.pool_floats;
+    a.d = d; a.T = c.T; a.rows = c.rows; a.cluster = c.cluster ? 1 : 0;
+    for (int l = 0; l < y.L; ++l) { a.ns_f[l] = c.ns_f[l]; a.ns_b[l] = c.ns_b[l]; a.off_wb[l] = y.off_wb[l]; }
+    a.ns_r = c.ns_r; a.resident = c.resident; a.pool_floats = c.pool_floats;
     a.sync = reinterpret_cast<unsigned*>(io.ws + y.off_sync);
     fn = walk_fn(y, c.nb);
     if (allow(reinterpret_cast<const void*>(fn)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
@@ -914,7 +933,7 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
       int rc;
       if (kept->pod) {
         pa.tasks = reinterpret_cast<const pod::Task*>(region + (g.task0 - up_lo));
-        pa.n_tasks = (int)g.ntasks; pa.phases = g.phases;
+        pa.n_tasks = (int)g.ntasks; pa.phases = g.phases; pa.fwd_ops = g.fwd_ops; pa.bwd_ops = g.bwd_ops;
         void* args[1] = {&pa};
         rc = launch(reinterpret_cast<const void*>(pf), kept->pc.pods * kept->pc.T, kept->pc.T, kept->pc.smem, args, s);
       } else {

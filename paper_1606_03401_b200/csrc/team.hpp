@@ -30,7 +30,6 @@ constexpr int kSmemMax = 227 * 1024;
 constexpr int kTaskWindow = 64;        // tasks a CTA fetches at a time; no phase straddles two windows
 constexpr int kMaxPhaseTasks = 8;
 constexpr int kMaxLayers = 16;
-constexpr uint32_t kInit = 0xffffffffu;   // "location" of the caller's initial state
 
 enum TaskKind : uint8_t { NOP = 0, FWD = 1, READ = 2, BWD = 3 };
 enum TaskFlag : uint8_t {
@@ -44,7 +43,7 @@ enum TaskFlag : uint8_t {
 struct Task {
   uint8_t kind, layer, flags, pad0;
   int32_t k;
-  uint32_t src;    // F: input state; R, B: record of step k.  256-byte units from the workspace base, or kInit
+  uint32_t src;    // F: input state; R, B: record of step k.  256-byte units from the workspace base
   uint32_t dst;    // F: record written; B: state k-1 (whole-state block)
   uint32_t sidx;   // row block of step k in the stages
   uint32_t a_off, red_off, pad1;   // this task's share of the phase pool, in floats
@@ -86,6 +85,7 @@ Config choose_config(const Layout& y, int sms, const int* max_clusters);
 struct Launch {          // one launch of the persistent kernel
   size_t task0 = 0, ntasks = 0;   // a whole number of windows
   int phases = 0;
+  int fwd_ops = 0, bwd_ops = 0;   // operations it executes
   int chunk = -1;                 // >= 0: this chunk of S steps is complete afterwards
 };
 struct Schedule {

@@ -138,7 +138,7 @@ bool supported(const mebptt_lstm_desc* d) {
   state_layout(d, y);
   if (y.tensor_path || y.stepwise_tc || y.stepwise_x3 || y.L > kMaxLayers || y.t >= (1 << 30)) return false;
   const int clusters[5] = {148, 74, 36, 16, 7};
-  return pod::choose_config(y, 148, clusters).ok || choose_config(y, 148, clusters).ok;
+  return pod::choose_config(y, y.tensor_cores, 148, clusters).ok || choose_config(y, 148, clusters).ok;
 }
 
 namespace {
@@ -173,7 +173,7 @@ struct Scheduler {
   }
   uint32_t address(int32_t loc) const {
     switch (loc) {
-      case MEBPTT_LOC_INIT: return kInit;
+      case MEBPTT_LOC_INIT: return (uint32_t)(y.off_init >> 8);
       case MEBPTT_LOC_PING: return base_pingpong[0];
       case MEBPTT_LOC_PONG: return base_pingpong[1];
       case MEBPTT_LOC_CORE: return base_core[core];

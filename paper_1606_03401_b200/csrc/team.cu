@@ -13,6 +13,7 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "env.hpp"
@@ -539,72 +540,221 @@ struct Product {
 constexpr int kMaxProducts = 2 * kMaxLayers + 2;
 struct Products { int n, tiles; Product p[kMaxProducts]; };
 
+// Row of the weights that gate row r of a stage belongs to; -1: none.
+__device__ __forceinline__ int gate_row(const Product& p, int r) {
+  if (!p.H) return r;
+  const int q = r & 3;
+  return q == p.skip ? -1 : (q == 3 ? p.last : q) * p.H + (r >> 2);
+}
+
+// A tile of a product is formed by two groups of 128 threads, each over every other slice of the
+// contraction index, so that the loads of one hide behind the arithmetic of the other (a chunk has
+// few tiles: with one group an SM held eight warps that waited for one another); the second group's
+// sums are added to the first's at the end.  Operands come in 16-byte pieces where their rows allow it.
+constexpr int kTileThreads = 256;
+__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); }
+
+// 4 consecutive values p[0..3], of which the first n exist.
+__device__ __forceinline__ float4 load_some(const float* p, int n, bool whole) {
+  if (whole && n >= 4) return *reinterpret_cast<const float4*>(p);
+  return make_float4(n > 0 ? p[0] : 0.f, n > 1 ? p[1] : 0.f, n > 2 ? p[2] : 0.f, n > 3 ? p[3] : 0.f);
+}
+__device__ __forceinline__ uint2 load_some(const __nv_bfloat16* p, int n, bool whole) {
+  if (whole && n >= 4) return *reinterpret_cast<const uint2*>(p);
+  const unsigned short* q = reinterpret_cast<const unsigned short*>(p);
+  uint2 r = make_uint2(0, 0);
+  if (n > 0) r.x = q[0];
+  if (n > 1) r.x |= (uint32_t)q[1] << 16;
+  if (n > 2) r.y = q[2];
+  if (n > 3) r.y |= (uint32_t)q[3] << 16;
+  return r;
+}
+__device__ __forceinline__ float4 widen(float4 v) { return v; }
+__device__ __forceinline__ float4 widen(uint2 v) {
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+}
+
+// The pieces of a slice of TK steps that a thread brings: N = TK / 8 of A and of B.
+template <class T, int TK>
+struct Slice {
+  static constexpr int N = TK / 8;
+  using Piece = typename std::conditional<std::is_same<T, float>::value, float4, uint2>::type;
+  float4 a[N];
+  Piece b[N];
+  // t: thread of the group.  Operands stored [k][*]: piece (t & 15) of step (t >> 4) + 8 e; A stored
+  // [m][k]: piece t % (TK / 4) of row t / (TK / 4) + e * 512 / TK.
+  __device__ __forceinline__ void fetch(const Product& p, int m0, int n0, int k0, int t) {
+    const bool wa = (p.lda & 3) == 0 && (reinterpret_cast<uintptr_t>(p.A) & 15) == 0;
+    const bool wb = (p.ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(p.B) & (4 * sizeof(T) - 1)) == 0;
+    const int c = (t & 15) * 4;
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      const int k = k0 + (t >> 4) + 8 * e;
+      const bool on = k < p.K;
+      if (p.a_mn) {
+        a[e] = load_some(p.A + (size_t)(on ? k : 0) * p.lda + m0 + c, on ? p.M - m0 - c : 0, wa);
+      } else {
+        const int m = m0 + t / (TK / 4) + e * (512 / TK), kk = k0 + (t % (TK / 4)) * 4;
+        a[e] = load_some(p.A + (size_t)(m < p.M ? m : 0) * p.lda + kk, m < p.M ? p.K - kk : 0, wa);
+      }
+      const int row = !on ? -1 : p.a_mn ? k : gate_row(p, k);
+      b[e] = load_some(reinterpret_cast<const T*>(p.B) + (size_t)(row < 0 ? 0 : row) * p.ldb + n0 + c, row < 0 ? 0 : p.N - n0 - c, wb);
+    }
+  }
+};
+
+// FMA, 8 x 4 results a thread.
 template <class T>
-__global__ void __launch_bounds__(256) chunk_products(const __grid_constant__ Products P) {
-  constexpr int TK = 16;
-  __shared__ __align__(16) float As[2][TK][68], Bs[2][TK][68];
+__device__ __forceinline__ void product_fma(const Product& p, int m0, int n0, float* smem) {
+  constexpr int TK = 16, LD = 68;
+  const int g = threadIdx.x >> 7, t = threadIdx.x & 127, tx = t & 15, ty = t >> 4;
+  float (*As)[LD] = reinterpret_cast<float (*)[LD]>(smem + g * 2 * TK * LD);
+  float (*Bs)[LD] = As + TK;
+  Slice<T, TK> s;
+  float acc[8][4] = {};
+  const int its = (p.K + TK - 1) / TK;
+  s.fetch(p, m0, n0, g * TK, t);
+  for (int it = g; it < its; it += 2) {
+#pragma unroll
+    for (int e = 0; e < s.N; ++e) {
+      if (p.a_mn) {
+        *reinterpret_cast<float4*>(&As[(t >> 4) + 8 * e][(t & 15) * 4]) = s.a[e];
+      } else {
+        const int m = t / (TK / 4) + e * (512 / TK), k = (t % (TK / 4)) * 4;
+        As[k][m] = s.a[e].x; As[k + 1][m] = s.a[e].y; As[k + 2][m] = s.a[e].z; As[k + 3][m] = s.a[e].w;
+      }
+      *reinterpret_cast<float4*>(&Bs[(t >> 4) + 8 * e][(t & 15) * 4]) = widen(s.b[e]);
+    }
+    group_sync(g);
+    if (it + 2 < its) s.fetch(p, m0, n0, (it + 2) * TK, t);
+#pragma unroll
+    for (int k = 0; k < TK; ++k) {
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 8]), a1 = *reinterpret_cast<const float4*>(&As[k][ty * 8 + 4]);
+      const float4 b = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
+      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = fmaf(av[r], bv[q], acc[r][q]);
+    }
+    group_sync(g);
+  }
+  __syncthreads();
+  float* const x = smem + t;
+  if (g == 1)
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i * 128] = acc[i >> 2][i & 3];
+  __syncthreads();
+  if (g == 1) return;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    const int m = m0 + ty * 8 + r, row = m < p.M ? (p.a_mn ? gate_row(p, m) : m) : -1;
+    if (row < 0) continue;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int n = n0 + tx * 4 + q;
+      const float v = acc[r][q] + x[(r * 4 + q) * 128];
+      float* o = p.C + (size_t)row * p.ldc + n;
+      if (n < p.N) *o = p.accumulate ? *o + v : v;
+    }
+  }
+}
+
+// Bfloat16 storage: A (float32 gradients) as three bfloat16 planes that add up to it, on mma.sync; a warp
+// has 32 x 32 results.
+__device__ __forceinline__ void product_mma(const Product& p, int m0, int n0, float* smem) {
+  constexpr int TK = 32, LM = 72, LK = 40;   // row lengths of [k][m] and [m][k] tiles: no bank conflicts for ldmatrix
+  constexpr int plane = 64 * LK;
+  const int g = threadIdx.x >> 7, t = threadIdx.x & 127, lane = t & 31, warp = t >> 5, wm = (warp & 1) * 32, wn = (warp >> 1) * 32;
+  __nv_bfloat16* const As = reinterpret_cast<__nv_bfloat16*>(smem) + g * (3 * plane + TK * LM);   // [plane][TK][LM] or [plane][64][LK]
+  __nv_bfloat16* const Bs = As + 3 * plane;                                                      // [TK][LM]
+  Slice<__nv_bfloat16, TK> s;
+  float acc[2][4][4] = {};
+  auto put_tile = [&]() {
+#pragma unroll
+    for (int e = 0; e < s.N; ++e) {
+      __nv_bfloat16* d = As + (p.a_mn ? ((t >> 4) + 8 * e) * LM + (t & 15) * 4 : (t / (TK / 4) + e * (512 / TK)) * LK + (t % (TK / 4)) * 4);
+      float4 v = s.a[e];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(d + q * plane) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        v.x -= __low2float(lo); v.y -= __high2float(lo); v.z -= __low2float(hi); v.w -= __high2float(hi);
+      }
+      *reinterpret_cast<uint2*>(Bs + ((t >> 4) + 8 * e) * LM + (t & 15) * 4) = s.b[e];
+    }
+  };
+  auto ldsm = [](uint32_t (&r)[4], uint32_t addr, bool trans) {
+    if (trans) asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+    else asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+  };
+  s.fetch(p, m0, n0, g * TK, t);
+  const int its = (p.K + TK - 1) / TK;
+  const uint32_t a0 = sm100::smem_u32(As), b0 = sm100::smem_u32(Bs);
+  const int l8 = lane & 7, q8 = lane >> 3;   // row inside an 8 x 8 block, block
+  for (int it = g; it < its; it += 2) {
+    put_tile();
+    group_sync(g);
+    if (it + 2 < its) s.fetch(p, m0, n0, (it + 2) * TK, t);
+#pragma unroll
+    for (int k = 0; k < TK; k += 16) {
+      uint32_t b[2][4];
+#pragma unroll
+      for (int j = 0; j < 2; ++j)   // blocks (k, n), (k + 8, n), (k, n + 8), (k + 8, n + 8)
+        ldsm(b[j], b0 + ((k + (q8 & 1) * 8 + l8) * LM + wn + j * 16 + (q8 >> 1) * 8) * 2, true);
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          uint32_t a[4];             // blocks (m, k), (m + 8, k), (m, k + 8), (m + 8, k + 8)
+          if (p.a_mn) ldsm(a, a0 + (q * plane + (k + (q8 >> 1) * 8 + l8) * LM + wm + i * 16 + (q8 & 1) * 8) * 2, true);
+          else ldsm(a, a0 + (q * plane + (wm + i * 16 + (q8 & 1) * 8 + l8) * LK + k + (q8 >> 1) * 8) * 2, false);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            float (&d)[4] = acc[i][j];
+            asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[j >> 1][(j & 1) * 2]), "r"(b[j >> 1][(j & 1) * 2 + 1]));
+          }
+        }
+    }
+    group_sync(g);
+  }
+  __syncthreads();
+  float* const x = smem + t;
+  if (g == 1)
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i * 128] = acc[i >> 4][(i >> 2) & 3][i & 3];
+  __syncthreads();
+  if (g == 1) return;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int m = m0 + wm + i * 16 + h * 8 + (lane >> 2), row = m < p.M ? (p.a_mn ? gate_row(p, m) : m) : -1;
+      if (row < 0) continue;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int n = n0 + wn + j * 8 + 2 * (lane & 3) + q;
+          float* o = p.C + (size_t)row * p.ldc + n;
+          const float v = acc[i][j][h * 2 + q] + x[(i * 16 + j * 4 + h * 2 + q) * 128];
+          if (n < p.N) *o = p.accumulate ? *o + v : v;
+        }
+    }
+}
+
+// MMA: the caller has not forbidden tensor cores.
+template <class T, bool MMA>
+__global__ void __launch_bounds__(kTileThreads) chunk_products(const __grid_constant__ Products P) {
+  __shared__ __align__(16) float smem[MMA ? 3 * 64 * 40 + 32 * 72 : 4 * 16 * 68];
   int i = P.n - 1;
   while ((int)blockIdx.x < P.p[i].tile0) --i;
   const Product& p = P.p[i];
   const int t = blockIdx.x - p.tile0, nx = (p.N + 63) / 64, m0 = (t / nx) * 64, n0 = (t % nx) * 64;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const T* B = reinterpret_cast<const T*>(p.B);
-  float ra[4], rb[4], acc[4][4] = {};
-  auto fetch_tile = [&](int k0) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int idx = tid + e * 256;
-      const int km = idx >> 6, mm = idx & 63;      // [k][m] order
-      const int mk = idx >> 4, kk = idx & 15;      // [m][k] order
-      const int m = p.a_mn ? mm : mk, k = k0 + (p.a_mn ? km : kk);
-      const bool on = m0 + m < p.M && k < p.K;
-      ra[e] = on ? p.A[p.a_mn ? (size_t)k * p.lda + m0 + m : (size_t)(m0 + m) * p.lda + k] : 0.f;
-      const int kb = k0 + km, row = (p.a_mn || !p.H) ? kb : ((kb & 3) == 3 ? p.last : kb & 3) * p.H + (kb >> 2);
-      rb[e] = (n0 + mm < p.N && kb < p.K && (p.a_mn || (kb & 3) != p.skip)) ? to_f(B[(size_t)row * p.ldb + n0 + mm]) : 0.f;
-    }
-  };
-  auto put_tile = [&](int s) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int idx = tid + e * 256;
-      if (p.a_mn) As[s][idx >> 6][idx & 63] = ra[e]; else As[s][idx & 15][idx >> 4] = ra[e];
-      Bs[s][idx >> 6][idx & 63] = rb[e];
-    }
-  };
-  fetch_tile(0);
-  put_tile(0);
-  __syncthreads();
-  const int its = (p.K + TK - 1) / TK;
-  for (int it = 0; it < its; ++it) {
-    const int s = it & 1;
-    if (it + 1 < its) fetch_tile((it + 1) * TK);
-#pragma unroll
-    for (int k = 0; k < TK; ++k) {
-      const float4 a = *reinterpret_cast<const float4*>(&As[s][k][ty * 4]), b = *reinterpret_cast<const float4*>(&Bs[s][k][tx * 4]);
-      const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(av[r], bv[c], acc[r][c]);
-    }
-    if (it + 1 < its) put_tile(s ^ 1);
-    __syncthreads();
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int m = m0 + ty * 4 + r, n = n0 + tx * 4 + c;
-      if (m < p.M && n < p.N) {
-        int row = m;
-        if (p.a_mn && p.H) {
-          if ((m & 3) == p.skip) continue;
-          row = ((m & 3) == 3 ? p.last : m & 3) * p.H + (m >> 2);
-        }
-        float* q = p.C + (size_t)row * p.ldc + n;
-        *q = p.accumulate ? *q + acc[r][c] : acc[r][c];
-      }
-    }
+  if constexpr (MMA) product_mma(p, m0, n0, smem);
+  else product_fma<T>(p, m0, n0, smem);
 }
 
 // Bias gradients (column sums of a chunk's dz and dy) and the loss terms of its steps.  dy = 2 d / (B O),
@@ -950,8 +1100,9 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
       const int64_t k0 = (int64_t)g.chunk * y.S;
       const int steps = (int)std::min<int64_t>(y.S, y.t - k0);
       fill_products(P, y, io, want_dx, k0, steps, !first);
-      if (y.dtype == MEBPTT_BF16) chunk_products<__nv_bfloat16><<<P.tiles, 256, 0, s>>>(P);
-      else chunk_products<float><<<P.tiles, 256, 0, s>>>(P);
+      if (y.dtype != MEBPTT_BF16) chunk_products<float, false><<<P.tiles, kTileThreads, 0, s>>>(P);
+      else if (y.tensor_cores) chunk_products<__nv_bfloat16, true><<<P.tiles, kTileThreads, 0, s>>>(P);
+      else chunk_products<__nv_bfloat16, false><<<P.tiles, kTileThreads, 0, s>>>(P);
       const Sums q{reinterpret_cast<const float*>(io.ws + y.off_dz), reinterpret_cast<const float*>(io.ws + y.off_dy), io.db, io.db_out,
                    loss_t + k0, y.L, y.NG, y.H, y.O, y.B, y.S, steps, first ? 0 : 1};
       chunk_sums<<<y.L * ((4 * y.H + 31) / 32) + (y.O + 31) / 32 + steps, 1024, 0, s>>>(q);

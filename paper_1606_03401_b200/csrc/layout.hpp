@@ -235,7 +235,7 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
   y.off_dc = take((size_t)y.L * bh4);
   y.off_loss_t = take((size_t)y.t * 4);
   if (y.team) {
-    const size_t G = 4 * (size_t)y.H, hp = align_up(y.H, 8), gp = align_up(G, 8), h4 = align_up(y.H, 4) + 4;
+    const size_t G = 4 * (size_t)y.H, hp = align_up(y.H, 16), gp = align_up(G, 16), h4 = align_up(y.H, 16);
     y.S = 2048 / y.B > 0 ? 2048 / y.B : 1;
     if (y.S > 64) y.S = 64;
     if (y.S > y.t) y.S = (int)y.t;
@@ -246,10 +246,10 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     auto larger = [](size_t u, size_t v) { return u > v ? u : v; };
     for (int l = 0; l < y.L; ++l) {
       const size_t in = l ? y.H + 96 : align_up(y.I, 16);
-      y.off_wf[l] = take(larger(G * (align_up(l ? y.H : y.I, 8) + hp), 4 * ((size_t)y.H + 16) * (in + y.H + 104)) * y.esz);
-      y.off_wb[l] = take(h4 * (gp + (l + 1 < y.L ? gp : align_up(y.O, 8))) * y.esz);
+      y.off_wf[l] = take(larger(4 * h4 * (align_up(l ? y.H : y.I, 16) + hp), 4 * ((size_t)y.H + 16) * (in + y.H + 104)) * y.esz);
+      y.off_wb[l] = take(h4 * (gp + (l + 1 < y.L ? gp : align_up(y.O, 16))) * y.esz);
     }
-    y.off_wr = take(larger(align_up(y.O, 4) * hp, ((size_t)y.O + 64) * (y.H + 104)) * y.esz);
+    y.off_wr = take(larger(align_up(y.O, 16) * hp, ((size_t)y.O + 64) * (y.H + 104)) * y.esz);
     y.off_init = take(y.unit);   // the caller's initial state, laid out like a hidden state
     y.off_st_dz = y.off_dz = take((size_t)y.L * rows * G * 4);
     // h of the chunk's steps and of the one before: row block i holds h_{k-1} of the step in block i of dz

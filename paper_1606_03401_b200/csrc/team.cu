@@ -34,7 +34,7 @@ namespace {
 
 struct Args {
   int L, I, H, O, B, S;
-  int T, rows, cluster;
+  int T, rows;
   Dims d;
   int ns_f[kMaxLayers], ns_b[kMaxLayers], ns_r;
   uint64_t resident;
@@ -81,52 +81,63 @@ __device__ __forceinline__ void four_rows(const float* a, int lda, const T* w, i
   }
 }
 
-// Copies rows [0, nb) of a staged operand segment: src row stride `ld` elements, `len` elements, zeros
-// up to `padded` and for rows past `valid`.
-template <class T>
-__device__ __forceinline__ void stage(float* dst, int lda, const T* src, size_t ld, int len, int padded, int nb, int valid,
-                                      int tid) {
-  const int total = nb * padded;
-  for (int e = tid; e < total; e += kThreads) {
-    const int b = e / padded, k = e - b * padded;
-    float v = 0.f;
-    if (k < len && b < valid) v = to_f(ld_l2(src + (size_t)b * ld + k));
-    dst[(size_t)b * lda + k] = v;
+// Four values as float32.
+__device__ __forceinline__ float4 widen(float4 v) { return v; }
+__device__ __forceinline__ float4 widen(uint2 v) {
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
+}
+
+// ---- operands -------------------------------------------------------------------------------
+
+// Four consecutive elements p[0..3] of which the first n exist, from the L2.
+__device__ __forceinline__ float4 piece(const float* p, int n, bool whole) {
+  if (whole && n >= 4) return __ldcg(reinterpret_cast<const float4*>(p));
+  return make_float4(n > 0 ? __ldcg(p) : 0.f, n > 1 ? __ldcg(p + 1) : 0.f, n > 2 ? __ldcg(p + 2) : 0.f, n > 3 ? __ldcg(p + 3) : 0.f);
+}
+__device__ __forceinline__ uint2 piece(const __nv_bfloat16* p, int n, bool whole) {
+  if (whole && n >= 4) return __ldcg(reinterpret_cast<const uint2*>(p));
+  const unsigned short* q = reinterpret_cast<const unsigned short*>(p);
+  uint2 r = make_uint2(0, 0);
+  if (n > 0) r.x = __ldcg(q);
+  if (n > 1) r.x |= (uint32_t)__ldcg(q + 1) << 16;
+  if (n > 2) r.y = __ldcg(q + 2);
+  if (n > 3) r.y |= (uint32_t)__ldcg(q + 3) << 16;
+  return r;
+}
+// Brings NB rows of `len` elements (`padded` with zeros, ld apart in memory) to wherever put(row, element,
+// piece) wants them.  A warp has one row; its loads are under way together.
+template <int NB, class T, class Put>
+__device__ __forceinline__ void stage(const T* src, size_t ld, int len, int padded, int valid, int warp, int lane, Put put) {
+  const bool whole = ((ld | (size_t)len) & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & (4 * sizeof(T) - 1)) == 0;
+  const int b = warp & (NB - 1), stride = (kWarps / NB) * 32;
+  const T* row = src + (size_t)b * ld;
+  const int lim = b < valid ? len : 0;
+  for (int v = (warp / NB) * 32 + lane; v < padded >> 2; v += 4 * stride) {
+    decltype(piece(row, 0, true)) x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = piece(row + 4 * (v + i * stride), lim - 4 * (v + i * stride), whole);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (v + i * stride < padded >> 2) put(b, 4 * (v + i * stride), x[i]);
   }
 }
-// The same for float32 rows that allow 16-byte accesses.
-__device__ __forceinline__ void stage4(float* dst, int lda, const float* src, size_t ld, int len, int padded, int nb,
-                                       int valid, int tid) {
-  const int q = padded >> 2, total = nb * q;
-  for (int e = tid; e < total; e += kThreads) {
-    const int b = e / q, k = (e - b * q) * 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (k < len && b < valid) v = __ldcg(reinterpret_cast<const float4*>(src + (size_t)b * ld + k));
-    *reinterpret_cast<float4*>(dst + (size_t)b * lda + k) = v;
-  }
-}
-// ... and for bfloat16 rows that allow 8-byte accesses.
-__device__ __forceinline__ void stage4(float* dst, int lda, const __nv_bfloat16* src, size_t ld, int len, int padded, int nb,
-                                       int valid, int tid) {
-  const int q = padded >> 2, total = nb * q;
-  for (int e = tid; e < total; e += kThreads) {
-    const int b = e / q, k = (e - b * q) * 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (k < len && b < valid) {
-      const uint2 u = __ldcg(reinterpret_cast<const uint2*>(src + (size_t)b * ld + k));
-      v = make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
-                      __uint_as_float(u.y & 0xffff0000u));
+
+// A group of 16 weight rows in the order of the tensor cores' fragments against up to 8 operand rows in PL
+// bfloat16 planes, steps [lo, hi) of 16; c[0], c[1]: row lane / 4, batch rows 2 (lane & 3), + 1; c[2], c[3]: row + 8.
+template <int NB, int PL>
+__device__ __forceinline__ void sixteen_rows(uint32_t a, uint32_t pitch, const uint4* w, int lo, int hi, int lane, float (&c)[4]) {
+  const uint32_t at = a + ((lane & 7) % NB) * pitch + ((lane >> 3) & 1) * 16;
+#pragma unroll 4
+  for (int k = lo; k < hi; ++k) {
+    const uint4 f = w[k * 32 + lane];
+#pragma unroll
+    for (int p = 0; p < PL; ++p) {
+      uint32_t b0, b1;
+      asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(b0), "=r"(b1) : "r"(at + p * NB * pitch + k * 32) : "memory");
+      asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                   : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(f.x), "r"(f.y), "r"(f.z), "r"(f.w), "r"(b0), "r"(b1));
     }
-    *reinterpret_cast<float4*>(dst + (size_t)b * lda + k) = v;
   }
-}
-template <class T>
-__device__ __forceinline__ void stage_any(float* dst, int lda, const T* src, size_t ld, int len, int padded, int nb, int valid,
-                                          int tid) {
-  if (((ld | (size_t)len) & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & (4 * sizeof(T) - 1)) == 0)
-    stage4(dst, lda, src, ld, len, padded, nb, valid, tid);
-  else
-    stage(dst, lda, src, ld, len, padded, nb, valid, tid);
 }
 
 // The state of layer l in a block of whole-stack states.
@@ -223,15 +234,8 @@ __device__ __forceinline__ void apply(const Args& A, const Task& t, size_t row, 
 
 // Meeting of the team's CTAs: everything written before it is visible after it.
 __device__ __forceinline__ bool meet(const Args& A, unsigned* line, unsigned target, volatile int* flag) {
-  if (A.T == 1) { __syncthreads(); return true; }
-  if (A.cluster) {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    return true;
-  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(line) : "memory");
     bool ok = false;
     for (uint32_t i = 0; i < sm100::kSpinLimit; ++i) {
@@ -246,8 +250,9 @@ __device__ __forceinline__ bool meet(const Args& A, unsigned* line, unsigned tar
   return *flag == 0;
 }
 
-template <class T, bool GRU, int NB>
+template <class T, bool GRU, int NB, bool MMA>
 __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args A) {
+  constexpr int RPG = MMA ? 16 : 4, UPG = RPG / 4;                    // rows of a group, units of a forward group
   extern __shared__ __align__(128) unsigned char smem[];
   Task* window = reinterpret_cast<Task*>(smem);                       // two windows of tasks
   volatile int& s_flag = *reinterpret_cast<volatile int*>(smem + 2 * kTaskWindow * sizeof(Task));
@@ -258,13 +263,21 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
   const int H = A.H, L = A.L;
   const int row0 = team * A.rows, rows = min(A.rows, A.B - row0);
   if (tid == 0) s_flag = *A.status;   // an earlier launch gave up: do nothing
-  int u0, u1, gh0, gh1, go0, go1;
-  part(H, A.T, rank, u0, u1);
-  part(A.d.groups_h, A.T, rank, gh0, gh1);
-  part(A.d.groups_o, A.T, rank, go0, go1);
+  int f0, f1, b0, b1, r0g, r1g;       // groups of this CTA
+  part(A.d.gf, A.T, rank, f0, f1);
+  part(A.d.gb, A.T, rank, b0, b1);
+  part(A.d.gr, A.T, rank, r0g, r1g);
+  // first column (unit, readout row) and number of columns of the CTA by kind of task
+  auto cols_at = [&](int kind) { return kind == FWD ? f0 * UPG : (kind == READ ? r0g : b0) * RPG; };
+  auto cols_of = [&](int kind) {
+    return max(0, kind == FWD ? min(f1 * UPG, H) - f0 * UPG : kind == READ ? min(r1g * RPG, A.O) - r0g * RPG : min(b1 * RPG, H) - b0 * RPG);
+  };
+  auto groups_of = [&](int kind) { return kind == FWD ? f1 - f0 : kind == READ ? r1g - r0g : b1 - b0; };
+  auto splits_of = [&](const Task& k) { return k.kind == FWD ? A.ns_f[k.layer] : k.kind == READ ? A.ns_r : A.ns_b[k.layer]; };
+  auto width_of = [&](const Task& k) { return k.kind == FWD ? A.d.kf[k.layer] : k.kind == READ ? A.d.hp : A.d.kb[k.layer]; };
 
   // resident weights, in the order of their bits; offsets in elements
-  const int nf = (u1 - u0) * 4, nbk = (gh1 - gh0) * 4, nr = (go1 - go0) * 4;
+  const int nf = (f1 - f0) * RPG, nbk = (b1 - b0) * RPG, nr = (r1g - r0g) * RPG;
   auto f_at = [&](int l) { int o = 0; for (int i = 0; i < l; ++i) if (A.resident >> (2 * i) & 1) o += nf * A.d.kf[i]; return o; };
   auto b_at = [&](int l) {
     int o = f_at(L);
@@ -278,12 +291,12 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
     for (int i = tid; i < q; i += kThreads) d4[i] = __ldcg(s4 + i);
   };
   for (int l = 0; l < L; ++l) {
-    const T* wf = reinterpret_cast<const T*>(A.ws + A.off_wf[l]) + (size_t)u0 * 4 * A.d.kf[l];
-    const T* wb = reinterpret_cast<const T*>(A.ws + A.off_wb[l]) + (size_t)gh0 * 4 * A.d.kb[l];
+    const T* wf = reinterpret_cast<const T*>(A.ws + A.off_wf[l]) + (size_t)f0 * RPG * A.d.kf[l];
+    const T* wb = reinterpret_cast<const T*>(A.ws + A.off_wb[l]) + (size_t)b0 * RPG * A.d.kb[l];
     if (A.resident >> (2 * l) & 1) copy_in(held + f_at(l), wf, (size_t)nf * A.d.kf[l]);
     if (A.resident >> (2 * l + 1) & 1) copy_in(held + b_at(l), wb, (size_t)nbk * A.d.kb[l]);
   }
-  if (A.resident >> 63) copy_in(held + b_at(L), reinterpret_cast<const T*>(A.ws + A.off_wr) + (size_t)go0 * 4 * A.d.hp, (size_t)nr * A.d.hp);
+  if (A.resident >> 63) copy_in(held + b_at(L), reinterpret_cast<const T*>(A.ws + A.off_wr) + (size_t)r0g * RPG * A.d.hp, (size_t)nr * A.d.hp);
 
   auto load_window = [&](int w) {
     if (tid < kTaskWindow * 2)
@@ -316,109 +329,130 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
       // operands of every task of the phase
       for (int i = 0; i < n; ++i) {
         const Task& k = t[i];
-        const int l = k.layer;
-        float* a = pool + k.a_off;
+        const int l = k.layer, width = width_of(k);
+        float* const a = pool + k.a_off;
+        // values as they are stored: float32, or bfloat16 rows width + 8 apart
+        auto plain = [&](const T* src, int len, int padded, int at) {
+          stage<NB>(src + (size_t)r0 * len, (size_t)len, len, padded, valid, warp, lane, [&](int b, int e, auto x) {
+            if constexpr (MMA) *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a) + b * (width + 8) + at + e) = x;
+            else *reinterpret_cast<float4*>(a + b * width + at + e) = widen(x);
+          });
+        };
+        // float32 gradients, on the tensor cores as three bfloat16 planes that add up to them
+        auto gradient = [&](const float* src, int len, int padded, int at) {
+          stage<NB>(src + (size_t)r0 * len, (size_t)len, len, padded, valid, warp, lane, [&](int b, int e, float4 v) {
+            if constexpr (MMA) {
+              __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(a) + b * (width + 8) + at + e;
+#pragma unroll
+              for (int q = 0; q < 3; ++q) {
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+                *reinterpret_cast<uint2*>(d + q * NB * (width + 8)) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+                v.x -= __low2float(lo); v.y -= __high2float(lo); v.z -= __low2float(hi); v.w -= __high2float(hi);
+              }
+            } else {
+              *reinterpret_cast<float4*>(a + b * width + at + e) = v;
+            }
+          });
+        };
         if (k.kind == FWD) {
-          const int lda = A.d.kf[l], I = l ? H : A.I;
-          const T* in = l ? h_at<T>(A, k.dst, l - 1) : reinterpret_cast<const T*>(A.x) + (size_t)(k.k - 1) * A.B * A.I;
-          stage_any(a, lda, in + (size_t)r0 * I, I, I, A.d.ip[l], NB, valid, tid);
-          stage_any(a + A.d.ip[l], lda, h_at<T>(A, k.src, l) + (size_t)r0 * H, H, H, A.d.hp, NB, valid, tid);
-          works += (u1 - u0) * A.ns_f[l];
-          elems += (u1 - u0) * NB;
+          plain(l ? h_at<T>(A, k.dst, l - 1) : reinterpret_cast<const T*>(A.x) + (size_t)(k.k - 1) * A.B * A.I, l ? H : A.I, A.d.ip[l], 0);
+          plain(h_at<T>(A, k.src, l), H, A.d.hp, A.d.ip[l]);
         } else if (k.kind == READ) {
-          stage_any(a, A.d.hp, h_at<T>(A, k.src, l) + (size_t)r0 * H, H, H, A.d.hp, NB, valid, tid);
-          works += (go1 - go0) * A.ns_r;
-          elems += (min(go1 * 4, A.O) - go0 * 4) * NB;
+          plain(h_at<T>(A, k.src, l), H, A.d.hp, 0);
         } else {
-          const int lda = A.d.kb[l], G = 4 * H;
-          const float* dzn = (k.flags & CARRY_IN)
-                                 ? reinterpret_cast<const float*>(A.ws + A.off_carry) + ((size_t)((k.k + 1) & 1) * L + l) * A.B * G
-                                 : reinterpret_cast<const float*>(A.ws + A.off_dz) + ((size_t)l * A.S + k.sidx + 1) * A.B * G;
-          stage_any(a, lda, dzn + (size_t)r0 * G, G, G, A.d.gp, NB, valid, tid);
-          if (l + 1 < L)
-            stage_any(a + A.d.gp, lda,
-                      reinterpret_cast<const float*>(A.ws + A.off_dz) + (((size_t)(l + 1) * A.S + k.sidx) * A.B + r0) * G, G, G,
-                      A.d.gp, NB, valid, tid);
-          else
-            stage_any(a + A.d.gp, lda, reinterpret_cast<const float*>(A.ws + A.off_dy) + ((size_t)k.sidx * A.B + r0) * A.O, A.O,
-                      A.O, lda - A.d.gp, NB, valid, tid);
-          works += (gh1 - gh0) * A.ns_b[l];
-          elems += (min(gh1 * 4, H) - gh0 * 4) * NB;
+          const int G = 4 * H;
+          const float* const dz = reinterpret_cast<const float*>(A.ws + A.off_dz);
+          gradient((k.flags & CARRY_IN) ? reinterpret_cast<const float*>(A.ws + A.off_carry) + ((size_t)((k.k + 1) & 1) * L + l) * A.B * G
+                                        : dz + ((size_t)l * A.S + k.sidx + 1) * A.B * G,
+                   G, A.d.gp, 0);
+          if (l + 1 < L) gradient(dz + ((size_t)(l + 1) * A.S + k.sidx) * A.B * G, G, A.d.gp, A.d.gp);
+          else gradient(reinterpret_cast<const float*>(A.ws + A.off_dy) + (size_t)k.sidx * A.B * A.O, A.O, width - A.d.gp, A.d.gp);
         }
+        works += groups_of(k.kind) * splits_of(k);
+        elems += cols_of(k.kind) * NB;
       }
-      // element f of the phase: its task, batch row and column
-      auto locate = [&](int f, const Task*& k, int& b, int& j, int& j0) {
+      // element f of the phase: its task, batch row (the fast index) and column
+      auto locate = [&](int f, const Task*& k, int& b, int& j) {
         for (int i = 0; i < n; ++i) {
           k = t + i;
-          const int lo = k->kind == FWD ? u0 : k->kind == READ ? go0 * 4 : gh0 * 4;
-          const int hi = k->kind == FWD ? u1 : k->kind == READ ? min(go1 * 4, A.O) : min(gh1 * 4, H);
-          const int m = (hi - lo) * NB;
-          if (f < m) { b = f / (hi - lo); j = lo + f - b * (hi - lo); j0 = lo; return; }
+          const int m = cols_of(k->kind) * NB;
+          if (f < m) { b = f & (NB - 1); j = f / NB; return; }
           f -= m;
         }
       };
       Operands o;
       const Task* ek = nullptr;
-      int eb = 0, ej = 0, ej0 = 0;
+      int eb = 0, ej = 0;
       if (tid < elems) {
-        locate(tid, ek, eb, ej, ej0);
-        if (eb < valid) fetch<T, GRU>(A, *ek, (size_t)(r0 + eb), ej, o);
+        locate(tid, ek, eb, ej);
+        if (eb < valid) fetch<T, GRU>(A, *ek, (size_t)(r0 + eb), cols_at(ek->kind) + ej, o);
       }
       __syncthreads();
       // partial sums
       for (int wk = warp; wk < works; wk += kWarps) {
-        int rem = wk, i = 0, ns = 1, groups = 0;
+        int rem = wk, i = 0, ns = 1;
         for (;; ++i) {
-          const Task& k = t[i];
-          ns = k.kind == FWD ? A.ns_f[k.layer] : k.kind == READ ? A.ns_r : A.ns_b[k.layer];
-          groups = k.kind == FWD ? u1 - u0 : k.kind == READ ? go1 - go0 : gh1 - gh0;
-          if (rem < groups * ns) break;
-          rem -= groups * ns;
+          ns = splits_of(t[i]);
+          const int m = groups_of(t[i].kind) * ns;
+          if (rem < m) break;
+          rem -= m;
         }
         const Task& k = t[i];
-        const int l = k.layer, g = rem / ns, s = rem - g * ns;
-        const int ld = k.kind == FWD ? A.d.kf[l] : k.kind == READ ? A.d.hp : A.d.kb[l];
-        const int nv = ld >> 2, its = (nv + 31) >> 5;
-        const int b0 = its * s / ns, b1 = its * (s + 1) / ns;
-        float acc[NB * 4];
-#pragma unroll
-        for (int q = 0; q < NB * 4; ++q) acc[q] = 0.f;
+        const int l = k.layer, g = rem / ns, s = rem - g * ns, ld = width_of(k);
         const int bit = k.kind == FWD ? 2 * l : k.kind == READ ? 63 : 2 * l + 1;
-        if (A.resident >> bit & 1) {
-          const int off = k.kind == FWD ? f_at(l) : k.kind == READ ? b_at(L) : b_at(l);
-          four_rows<T, NB>(pool + k.a_off, ld, held + off + (size_t)g * 4 * ld, ld, b0, b1, nv, lane, acc);
+        const bool res = A.resident >> bit & 1;
+        const T* wg;
+        if (res) {
+          wg = held + (k.kind == FWD ? f_at(l) : k.kind == READ ? b_at(L) : b_at(l)) + (size_t)g * RPG * ld;
         } else {
           const size_t off = k.kind == FWD ? A.off_wf[l] : k.kind == READ ? A.off_wr : A.off_wb[l];
-          const int first = k.kind == FWD ? u0 : k.kind == READ ? go0 : gh0;
-          four_rows<T, NB>(pool + k.a_off, ld, reinterpret_cast<const T*>(A.ws + off) + (size_t)(first + g) * 4 * ld, ld, b0, b1,
-                           nv, lane, acc);
+          wg = reinterpret_cast<const T*>(A.ws + off) + (size_t)((k.kind == FWD ? f0 : k.kind == READ ? r0g : b0) + g) * RPG * ld;
         }
-        const float v = lane_sums<NB * 4>(acc, lane);
-        constexpr int per = 32 / (NB * 4);
-        if (lane % per == 0) pool[k.red_off + (size_t)(g * ns + s) * NB * 4 + lane / per] = v;
+        float* const red = pool + k.red_off + (size_t)(g * ns + s) * NB * RPG;
+        if constexpr (MMA) {
+          const int steps = ld >> 4, lo = steps * s / ns, hi = steps * (s + 1) / ns;
+          float c[4] = {};
+          const uint32_t a = sm100::smem_u32(pool + k.a_off), pitch = (ld + 8) * 2;
+          if (k.kind == BWD) sixteen_rows<NB, 3>(a, pitch, reinterpret_cast<const uint4*>(wg), lo, hi, lane, c);
+          else sixteen_rows<NB, 1>(a, pitch, reinterpret_cast<const uint4*>(wg), lo, hi, lane, c);
+          const int c0 = 2 * (lane & 3), r = lane >> 2;
+          if (c0 < NB) {   // [batch row][16]
+            red[c0 * 16 + r] = c[0]; red[c0 * 16 + r + 8] = c[2];
+            if (NB > 1) { red[(c0 + 1) * 16 + r] = c[1]; red[(c0 + 1) * 16 + r + 8] = c[3]; }
+          }
+        } else {
+          const int nv = ld >> 2, its = (nv + 31) >> 5;
+          float acc[NB * 4];
+#pragma unroll
+          for (int q = 0; q < NB * 4; ++q) acc[q] = 0.f;
+          four_rows<T, NB>(pool + k.a_off, ld, wg, ld, its * s / ns, its * (s + 1) / ns, nv, lane, acc);
+          const float v = lane_sums<NB * 4>(acc, lane);
+          constexpr int per = 32 / (NB * 4);
+          if (lane % per == 0) red[lane / per] = v;   // [batch row][4]
+        }
       }
       __syncthreads();
       for (int f = tid; f < elems; f += kThreads) {
         if (f != tid) {
-          locate(f, ek, eb, ej, ej0);
-          if (eb < valid) fetch<T, GRU>(A, *ek, (size_t)(r0 + eb), ej, o);
+          locate(f, ek, eb, ej);
+          if (eb < valid) fetch<T, GRU>(A, *ek, (size_t)(r0 + eb), cols_at(ek->kind) + ej, o);
         }
         if (eb >= valid) continue;
         const Task& k = *ek;
-        const int ns = k.kind == FWD ? A.ns_f[k.layer] : k.kind == READ ? A.ns_r : A.ns_b[k.layer];
+        const int ns = splits_of(k), per = k.kind == FWD ? UPG : RPG, g = ej / per, in = ej - g * per;
+        const float* p = pool + k.red_off + (size_t)g * ns * NB * RPG + eb * RPG;
         float z[4] = {0.f, 0.f, 0.f, 0.f};
         if (k.kind == FWD) {
-          const float* p = pool + k.red_off + (size_t)(ej - ej0) * ns * NB * 4 + eb * 4;
-          for (int s = 0; s < ns; ++s, p += NB * 4) {
+          p += in * 4;
+          for (int s = 0; s < ns; ++s, p += NB * RPG) {
             const float4 v = *reinterpret_cast<const float4*>(p);
             z[0] += v.x; z[1] += v.y; z[2] += v.z; z[3] += v.w;
           }
         } else {
-          const int jj = ej - ej0;
-          const float* p = pool + k.red_off + (size_t)(jj >> 2) * ns * NB * 4 + eb * 4 + (jj & 3);
-          for (int s = 0; s < ns; ++s, p += NB * 4) z[0] += *p;
+          p += in;
+          for (int s = 0; s < ns; ++s, p += NB * RPG) z[0] += *p;
         }
-        apply<T, GRU>(A, k, (size_t)(r0 + eb), ej, o, z);
+        apply<T, GRU>(A, k, (size_t)(r0 + eb), cols_at(k.kind) + ej, o, z);
       }
       if ((sub + 1) * NB < rows) __syncthreads();
     }
@@ -452,8 +486,18 @@ struct PackArgs {
   int64_t* counters;
 };
 
-template <class T, bool GRU>
+// Where element (row, column) of a matrix of rows of `width` goes: row after row, or in the order of the
+// tensor cores' fragments, 16 rows a tile: [tile][16 columns][lane][8].
+template <bool MMA>
+__device__ __forceinline__ size_t place(int row, int col, int width) {
+  if (!MMA) return (size_t)row * width + col;
+  const int r = row & 15, c = col & 15, lane = (r & 7) * 4 + ((c & 7) >> 1), reg = (r >> 3) + 2 * (c >> 3);
+  return (((size_t)(row >> 4) * (width >> 4) + (col >> 4)) * 32 + lane) * 8 + reg * 2 + (c & 1);
+}
+
+template <class T, bool GRU, bool MMA>
 __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
+  const int rf = P.d.gf * P.d.rpg, rb = P.d.gb * P.d.rpg, rr = P.d.gr * P.d.rpg;   // rows with the padding
   __shared__ float tile[32][33];
   const int x = threadIdx.x & 31, y0 = threadIdx.x >> 5, H = P.H;
   for (size_t i = blockIdx.x * 256 + threadIdx.x; i < P.n_zero; i += (size_t)gridDim.x * 256) P.zero[i] = 0.f;
@@ -465,15 +509,15 @@ __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
       reinterpret_cast<float*>(P.init + l * P.hc + P.csz_off)[i] = P.c0[l * bh + i];
     }
   auto tiles = [](int rows, int cols) { return ((rows + 31) / 32) * ((cols + 31) / 32); };
-  int total = tiles(P.d.groups_o * 4, P.d.hp);
-  for (int l = 0; l < P.L; ++l) total += tiles(4 * H, P.d.kf[l]) + tiles(P.d.groups_h * 4, P.d.kb[l]);
+  int total = tiles(rr, P.d.hp);
+  for (int l = 0; l < P.L; ++l) total += tiles(rf, P.d.kf[l]) + tiles(rb, P.d.kb[l]);
   for (int b = blockIdx.x; b < total; b += gridDim.x) {
     int t = b, l = 0, what = 0;   // 0: forward rows, 1: transposed, 2: readout
     for (; l < P.L; ++l) {
-      int n = tiles(4 * H, P.d.kf[l]);
+      int n = tiles(rf, P.d.kf[l]);
       if (t < n) { what = 0; break; }
       t -= n;
-      n = tiles(P.d.groups_h * 4, P.d.kb[l]);
+      n = tiles(rb, P.d.kb[l]);
       if (t < n) { what = 1; break; }
       t -= n;
     }
@@ -482,7 +526,7 @@ __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
       const int kf = P.d.kf[l], nx = (kf + 31) / 32, r0 = (t / nx) * 32, c = (t % nx) * 32 + x;
       const int I = l ? H : P.I, K = I + H, ip = P.d.ip[l];
       const T* W = P.W + P.w_off[l];
-      for (int r = r0 + y0; r < r0 + 32 && r < 4 * H; r += 8) {
+      for (int r = r0 + y0; r < r0 + 32 && r < rf; r += 8) {
         if (c >= kf) continue;
         const int j = r >> 2, q = r & 3;
         const bool rec = c >= ip;
@@ -490,12 +534,12 @@ __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
         bool on = rec ? c - ip < H : c < I;
         int row = q * H + j;
         if (GRU && q >= 2) { on = on && (rec == (q == 3)); row = 2 * H + j; }
-        P.wf[l][(size_t)r * kf + c] = on ? W[(size_t)row * K + col] : T(0.f);
+        P.wf[l][place<MMA>(r, c, kf)] = on && j < H ? W[(size_t)row * K + col] : T(0.f);
       }
     } else if (what == 2) {
       const int hp = P.d.hp, nx = (hp + 31) / 32, r0 = (t / nx) * 32, c = (t % nx) * 32 + x;
-      for (int r = r0 + y0; r < r0 + 32 && r < P.d.groups_o * 4; r += 8)
-        if (c < hp) P.wr[(size_t)r * hp + c] = (r < P.O && c < H) ? P.W_out[(size_t)r * H + c] : T(0.f);
+      for (int r = r0 + y0; r < r0 + 32 && r < rr; r += 8)
+        if (c < hp) P.wr[place<MMA>(r, c, hp)] = (r < P.O && c < H) ? P.W_out[(size_t)r * H + c] : T(0.f);
     } else {
       // out[j][g]: tile rows j0.., columns g0..; read with j fastest
       const int kb = P.d.kb[l], nx = (kb + 31) / 32, j0 = (t / nx) * 32, g0 = (t % nx) * 32;
@@ -522,7 +566,7 @@ __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
       __syncthreads();
       for (int yy = y0; yy < 32; yy += 8) {
         const int j = j0 + yy, g = g0 + x;
-        if (j < P.d.groups_h * 4 && g < kb) store(P.wb[l] + (size_t)j * kb + g, tile[x][yy]);
+        if (j < rb && g < kb) store(P.wb[l] + place<MMA>(j, g, kb), tile[x][yy]);
       }
       __syncthreads();
     }
@@ -568,10 +612,6 @@ __device__ __forceinline__ uint2 load_some(const __nv_bfloat16* p, int n, bool w
   if (n > 2) r.y = q[2];
   if (n > 3) r.y |= (uint32_t)q[3] << 16;
   return r;
-}
-__device__ __forceinline__ float4 widen(float4 v) { return v; }
-__device__ __forceinline__ float4 widen(uint2 v) {
-  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
 }
 
 // The pieces of a slice of TK steps that a thread brings: N = TK / 8 of A and of B.
@@ -805,13 +845,14 @@ __global__ void __launch_bounds__(1024) chunk_sums(const Sums q) {
 }
 
 using WalkFn = void (*)(const Args);
-template <class T, bool GRU>
+template <class T, bool GRU, bool MMA>
 WalkFn walk_nb(int nb) {
-  return nb == 1 ? walk<T, GRU, 1> : nb == 2 ? walk<T, GRU, 2> : nb == 4 ? walk<T, GRU, 4> : walk<T, GRU, 8>;
+  return nb == 1 ? walk<T, GRU, 1, MMA> : nb == 2 ? walk<T, GRU, 2, MMA> : nb == 4 ? walk<T, GRU, 4, MMA> : walk<T, GRU, 8, MMA>;
 }
 WalkFn walk_fn(const Layout& y, int nb) {
-  if (y.dtype == MEBPTT_BF16) return y.gru ? walk_nb<__nv_bfloat16, true>(nb) : walk_nb<__nv_bfloat16, false>(nb);
-  return y.gru ? walk_nb<float, true>(nb) : walk_nb<float, false>(nb);
+  if (y.dtype != MEBPTT_BF16) return y.gru ? walk_nb<float, true, false>(nb) : walk_nb<float, false, false>(nb);
+  if (y.tensor_cores) return y.gru ? walk_nb<__nv_bfloat16, true, true>(nb) : walk_nb<__nv_bfloat16, false, true>(nb);
+  return y.gru ? walk_nb<__nv_bfloat16, true, false>(nb) : walk_nb<__nv_bfloat16, false, false>(nb);
 }
 
 }  // namespace
@@ -893,7 +934,7 @@ bool same_problem(const Layout& a, const Layout& b) {
 
 std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable) {
   const DeviceFacts f = facts();
-  const Config c = choose_config(y, f.sms, f.clusters);
+  const Config c = choose_config(y, f.sms);
   const pod::Config pc = pod::choose_config(y, y.tensor_cores, f.sms, f.clusters);
   const bool use_pod = pc.ok && (y.total >> 32) == 0 && (!c.ok || pc.cycles <= c.cycles);
   if (!c.ok && !use_pod) return nullptr;
@@ -901,8 +942,7 @@ std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable
     std::lock_guard<std::mutex> lock(g_mu);
     for (size_t i = 0; i < g_kept.size(); ++i) {
       Kept& k = *g_kept[i];
-      if (k.plan_id == p->id && same_problem(k.y, y) && (k.pageable || !pageable) && k.pod == use_pod && k.c.T == c.T && k.c.teams == c.teams &&
-          k.c.cluster == c.cluster && k.pc.T == pc.T && k.pc.nb == pc.nb) {
+      if (k.plan_id == p->id && same_problem(k.y, y) && (k.pageable || !pageable) && k.pod == use_pod && k.c.T == c.T && k.c.teams == c.teams && k.pc.T == pc.T && k.pc.nb == pc.nb) {
         std::shared_ptr<Kept> hit = g_kept[i];
         g_kept.erase(g_kept.begin() + (long)i);
         g_kept.insert(g_kept.begin(), hit);
@@ -966,8 +1006,12 @@ void launch_pack(const Layout& y, const Dims& d, const tc::StepPtrs& io, cudaStr
   P.zero = reinterpret_cast<float*>(io.ws + y.off_dc);
   P.n_zero = (y.off_zero_end - y.off_dc) / 4;
   P.counters = io.counters;
-  if (y.gru) pack<T, true><<<592, 256, 0, s>>>(P);
-  else pack<T, false><<<592, 256, 0, s>>>(P);
+  constexpr bool half = !std::is_same<T, float>::value;
+  if (half && d.mma) {
+    if (y.gru) pack<T, true, half><<<592, 256, 0, s>>>(P); else pack<T, false, half><<<592, 256, 0, s>>>(P);
+  } else {
+    if (y.gru) pack<T, true, false><<<592, 256, 0, s>>>(P); else pack<T, false, false><<<592, 256, 0, s>>>(P);
+  }
 }
 
 // The products of chunk `chunk` (steps [k0, k0 + steps), 0-based).
@@ -1055,7 +1099,7 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     if (allow(reinterpret_cast<const void*>(pf)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
   } else {
     common(a);
-    a.d = d; a.T = c.T; a.rows = c.rows; a.cluster = c.cluster ? 1 : 0;
+    a.d = d; a.T = c.T; a.rows = c.rows;
     for (int l = 0; l < y.L; ++l) { a.ns_f[l] = c.ns_f[l]; a.ns_b[l] = c.ns_b[l]; a.off_wb[l] = y.off_wb[l]; }
     a.ns_r = c.ns_r; a.resident = c.resident; a.pool_floats = c.pool_floats;
     a.sync = reinterpret_cast<unsigned*>(io.ws + y.off_sync);
@@ -1092,7 +1136,7 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
         a.sync_base = met * (unsigned)c.T;
         met += (unsigned)g.phases;
         void* args[1] = {&a};
-        rc = launch(reinterpret_cast<const void*>(fn), c.teams * c.T, c.cluster ? c.T : 0, c.smem, args, s);
+        rc = launch(reinterpret_cast<const void*>(fn), c.teams * c.T, 0, c.smem, args, s);
       }
       if (rc != MEBPTT_OK) return rc;
     }

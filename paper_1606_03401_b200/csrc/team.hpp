@@ -50,14 +50,17 @@ struct Task {
 };
 static_assert(sizeof(Task) == 32, "Task layout");
 
-// Sizes that follow from the shape alone.
+// Sizes that follow from the shape alone.  A group is what a warp forms at a time: 4 weight rows on FMA
+// (a unit's gates, 4 units of the transposed weights, 4 readout rows), 16 on the tensor cores.
 struct Dims {
+  bool mma;             // bfloat16 storage, tensor cores not forbidden
+  int rpg;              // rows of a group
   int kf[kMaxLayers];   // row length of the packed forward weights (input part and recurrent part padded)
   int ip[kMaxLayers];   // padded input part of it
   int kb[kMaxLayers];   // row length of the transposed weights: 4H (recurrent), then 4H of the layer above or O
   int gp;               // padded 4H
   int hp;               // padded H: row length of the readout weights
-  int groups_o, groups_h;   // groups of 4 readout rows / of 4 units
+  int gf, gb, gr;       // groups of forward rows, of units, of readout rows
 };
 Dims dims(const Layout& y);
 
@@ -65,7 +68,6 @@ struct Config {
   bool ok = false;
   double cycles = 0;                        // estimate for two forward operations and one backward operation
   int T = 1, teams = 1, rows = 1, nb = 1;   // CTAs per team, teams, batch rows per team, rows taken at a time
-  bool cluster = true;                      // the team is a thread-block cluster (T <= 16), else a slice of a cooperative grid
   int ns_f[kMaxLayers] = {}, ns_b[kMaxLayers] = {}, ns_r = 1;   // parts the contraction index is cut into
   int pool_floats = 0;                      // shared memory for a phase's operands and partial sums
   uint64_t resident = 0;                    // bit 2l: F(l) weights in shared memory, 2l+1: B(l), 63: readout
@@ -78,8 +80,8 @@ Need need_f(const Layout& y, const Dims& d, const Config& c, int l);
 Need need_r(const Layout& y, const Dims& d, const Config& c);
 Need need_b(const Layout& y, const Dims& d, const Config& c, int l);
 
-// sms: SMs of the device; max_clusters[i]: clusters of 2^i CTAs that fit the device at once (i = 0..4)
-Config choose_config(const Layout& y, int sms, const int* max_clusters);
+// sms: SMs of the device
+Config choose_config(const Layout& y, int sms);
 // (supported, in layout.hpp: whether some configuration exists; asked for the layout, before a device is known)
 
 struct Launch {          // one launch of the persistent kernel

@@ -10,62 +10,68 @@ namespace mebptt {
 namespace team {
 
 namespace {
-inline int pad8(int v) { return (v + 7) & ~7; }
+inline int pad16(int v) { return (v + 15) & ~15; }
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
-inline int iters(int k) { return ceil_div(k, 128); }   // a warp takes 128 elements of the contraction index at a time
 }  // namespace
 
 Dims dims(const Layout& y) {
   Dims d{};
-  d.gp = pad8(4 * y.H);
-  d.hp = pad8(y.H);
-  for (int l = 0; l < y.L; ++l) {
-    d.ip[l] = pad8(l == 0 ? y.I : y.H);
+  d.mma = y.dtype == MEBPTT_BF16 && y.tensor_cores;
+  d.rpg = d.mma ? 16 : 4;
+  d.gp = pad16(4 * y.H);
+  d.hp = pad16(y.H);
+  for (int l = 0; l < y.L && l < kMaxLayers; ++l) {
+    d.ip[l] = pad16(l == 0 ? y.I : y.H);
     d.kf[l] = d.ip[l] + d.hp;
-    d.kb[l] = d.gp + (l + 1 < y.L ? d.gp : pad8(y.O));
+    d.kb[l] = d.gp + (l + 1 < y.L ? d.gp : pad16(y.O));
   }
-  d.groups_o = ceil_div(y.O, 4);
-  d.groups_h = ceil_div(y.H, 4);
+  d.gf = ceil_div(4 * y.H, d.rpg);
+  d.gb = ceil_div(y.H, d.rpg);
+  d.gr = ceil_div(y.O, d.rpg);
   return d;
 }
 
-Need need_f(const Layout& y, const Dims& d, const Config& c, int l) {
-  return Need{c.nb * d.kf[l], ceil_div(y.H, c.T) * c.ns_f[l] * c.nb * 4};
+namespace {
+// floats of pool: k staged elements a row (gradients on the tensor cores in three planes), partial sums
+Need need(const Dims& d, const Config& c, int groups, int k, int ns, bool planes) {
+  const int row = d.mma ? (planes ? 3 : 1) * (k + 8) / 2 : k;
+  return Need{(c.nb * row + 3) & ~3, ceil_div(groups, c.T) * ns * c.nb * d.rpg};
 }
-Need need_r(const Layout& y, const Dims& d, const Config& c) {
-  (void)y;
-  return Need{c.nb * d.hp, ceil_div(d.groups_o, c.T) * c.ns_r * c.nb * 4};
-}
-Need need_b(const Layout& y, const Dims& d, const Config& c, int l) {
-  (void)y;
-  return Need{c.nb * d.kb[l], ceil_div(d.groups_h, c.T) * c.ns_b[l] * c.nb * 4};
-}
+}  // namespace
+Need need_f(const Layout& y, const Dims& d, const Config& c, int l) { (void)y; return need(d, c, d.gf, d.kf[l], c.ns_f[l], false); }
+Need need_r(const Layout& y, const Dims& d, const Config& c) { (void)y; return need(d, c, d.gr, d.hp, c.ns_r, false); }
+Need need_b(const Layout& y, const Dims& d, const Config& c, int l) { (void)y; return need(d, c, d.gb, d.kb[l], c.ns_b[l], true); }
 
 namespace {
 
-// One task's share of a phase in clock cycles, by what a CTA's shared memory delivers: per group and
-// 128 elements of the contraction, nb operand vectors and 4 weight vectors of 16 bytes a lane.
-double task_cycles(const Config& c, int groups_cta, int k, int ns, int esz, bool resident) {
-  const int nsub = ceil_div(c.rows, c.nb), w = groups_cta * ns;
-  const double through = (double)groups_cta * iters(k) * (4.0 * c.nb + 4.0 * esz);
-  const double chain = (double)ceil_div(w, kWarps) * (ceil_div(iters(k), ns) * 70.0 + 120.0);
-  double t = std::max(through, chain);
+// One task's share of a phase in clock cycles: operands from the L2 into shared memory, then what the
+// arithmetic and the weights take, from shared memory or from the L2.
+double task_cycles(const Config& c, const Dims& d, int groups_cta, int k, int ns, int esz, bool resident, bool planes) {
+  const int nsub = ceil_div(c.rows, c.nb), rounds = ceil_div(groups_cta * ns, kWarps);
+  double t;
+  if (d.mma) {
+    t = rounds * (ceil_div(k / 16, ns) * (planes ? 60.0 : 35.0) + 200.0);
+  } else {
+    const int its = ceil_div(k, 128);
+    t = std::max((double)groups_cta * its * (4.0 * c.nb + 4.0 * esz), rounds * (ceil_div(its, ns) * 80.0 + 300.0));
+  }
   const double ctas = (double)c.teams * c.T;
   if (!resident) {   // weights from the L2, as fast as an SM takes them in or all SMs together get them
-    const double bytes = (double)groups_cta * 4 * k * esz;
-    t = std::max(t, std::max(bytes / 45.0, bytes * ctas / 3000.0));
+    const double bytes = (double)groups_cta * d.rpg * k * esz;
+    t = std::max(t, std::max(bytes / 45.0, bytes * ctas / 4000.0));
   }
-  const double stage = (double)c.nb * k * 4;
-  return nsub * (t + std::max(stage / 40.0, stage * ctas / 3000.0));
+  const double stage = (double)c.nb * k * (planes ? 4 : esz);
+  return nsub * (t + 300.0 + std::max(stage / 30.0, stage * ctas / 4000.0));
 }
 
 // Fills in everything that follows from T, teams and rows; returns the estimated cycles of two
 // forward operations and one backward operation, or a negative value if the shape does not fit.
 double finish(const Layout& y, const Dims& d, Config& c) {
-  const int uf = ceil_div(y.H, c.T), ub = ceil_div(d.groups_h, c.T), ur = ceil_div(d.groups_o, c.T);
+  const int uf = ceil_div(d.gf, c.T), ub = ceil_div(d.gb, c.T), ur = ceil_div(d.gr, c.T);
   c.nb = 1;
   while (c.nb < 8 && c.nb < c.rows) c.nb *= 2;
-  auto parts = [](int groups, int k) { return std::max(1, std::min(iters(k), kWarps / groups)); };
+  const int esz = (int)y.esz, step = d.mma ? 64 : 128;   // least elements of the contraction index worth a piece of their own
+  auto parts = [&](int groups, int k) { return std::max(1, std::min(ceil_div(k, step), kWarps / groups)); };
   c.ns_r = parts(ur, d.hp);
   int most = 0, sum_f = 0, sum_b = 0;
   const Need nr = need_r(y, d, c);
@@ -82,54 +88,48 @@ double finish(const Layout& y, const Dims& d, Config& c) {
   const int fixed = 2 * kTaskWindow * (int)sizeof(Task) + 256;
   const int budget = kSmemMax - fixed;
   if ((int64_t)most * 4 > budget) return -1.0;
-  auto bytes_f = [&](int l) { return (int64_t)uf * 4 * d.kf[l] * (int64_t)y.esz; };
-  auto bytes_b = [&](int l) { return (int64_t)ub * 4 * d.kb[l] * (int64_t)y.esz; };
-  const int64_t bytes_r = (int64_t)ur * 4 * d.hp * (int64_t)y.esz;
+  auto bytes_f = [&](int l) { return (int64_t)uf * d.rpg * d.kf[l] * esz; };
+  auto bytes_b = [&](int l) { return (int64_t)ub * d.rpg * d.kb[l] * esz; };
+  const int64_t bytes_r = (int64_t)ur * d.rpg * d.hp * esz;
   int64_t all = bytes_r;
   for (int l = 0; l < y.L; ++l) all += bytes_f(l) + bytes_b(l);
   // room for a phase of the wavefront over the layers where the weights leave it, at least for one task
   int64_t pool = std::min<int64_t>((int64_t)want * 4, std::max<int64_t>((int64_t)most * 4, budget - all));
-  int64_t left = budget - pool;
+  c.pool_floats = (int)((pool + 15) / 16) * 4;
+  if ((int64_t)c.pool_floats * 4 > budget) c.pool_floats = budget / 16 * 4;
+  int64_t left = budget - (int64_t)c.pool_floats * 4, held = 0;
   c.resident = 0;
-  int64_t held = 0;
   auto keep = [&](int bit, int64_t bytes) {
     if (bytes <= left) { c.resident |= 1ull << bit; left -= bytes; held += bytes; }
   };
   for (int l = 0; l < y.L; ++l) keep(2 * l, bytes_f(l));
   for (int l = 0; l < y.L; ++l) keep(2 * l + 1, bytes_b(l));
   keep(63, bytes_r);
-  c.pool_floats = (int)(pool / 4) & ~3;
-  c.w_floats4 = (int)(held / 16);
   c.smem = fixed + c.pool_floats * 4 + (int)held;
-  const double sync = c.T == 1 ? 100.0 : (c.cluster ? 700.0 : 2600.0);
-  double cyc = 3 * (7000.0 + sync) + task_cycles(c, ur, d.hp, c.ns_r, (int)y.esz, (c.resident >> 63) & 1);
+  double cyc = 3 * 6500.0 + task_cycles(c, d, ur, d.hp, c.ns_r, esz, (c.resident >> 63) & 1, false);
   for (int l = 0; l < y.L; ++l)
-    cyc += 2 * task_cycles(c, uf, d.kf[l], c.ns_f[l], (int)y.esz, (c.resident >> (2 * l)) & 1) +
-           task_cycles(c, ub, d.kb[l], c.ns_b[l], (int)y.esz, (c.resident >> (2 * l + 1)) & 1);
+    cyc += 2 * task_cycles(c, d, uf, d.kf[l], c.ns_f[l], esz, (c.resident >> (2 * l)) & 1, false) +
+           task_cycles(c, d, ub, d.kb[l], c.ns_b[l], esz, (c.resident >> (2 * l + 1)) & 1, true);
   c.ok = true;
   return cyc;
 }
 
 }  // namespace
 
-// The team size with the least estimated time: small problems are bound by the meetings of a team's
-// CTAs (a CTA of its own meets nobody, a cluster meets in hardware, a slice of the grid through a
-// counter in the L2), large ones by the work, the weights an SM can hold and what the L2 delivers.
-Config choose_config(const Layout& y, int sms, const int* max_clusters) {
-  const Dims d = dims(y);
+// The number of teams with the least estimated time: with more of them a team has fewer rows to stage
+// and meets fewer CTAs, with fewer a CTA has fewer weights, which it can then hold.
+Config choose_config(const Layout& y, int sms) {
   Config best;
-  double best_cyc = 0;
-  auto consider = [&](int T, int teams, bool cluster) {
-    if (teams < 1) return;
+  if (y.L > kMaxLayers) return best;
+  const Dims d = dims(y);
+  for (int teams = 1; teams <= sms / 17; ++teams) {
     Config c;
-    c.T = T; c.cluster = cluster;
+    c.T = sms / teams;
     c.rows = ceil_div(y.B, std::min(teams, y.B));
     c.teams = ceil_div(y.B, c.rows);
-    const double cyc = finish(y, d, c);
-    if (cyc >= 0 && (!best.ok || cyc < best_cyc)) { best = c; best_cyc = cyc; best.cycles = cyc; }
-  };
-  for (int i = 0; i <= 4; ++i) consider(1 << i, std::min(max_clusters[i], sms >> i), true);
-  for (int teams = 1; teams <= sms / 17; ++teams) consider(sms / teams, teams, false);
+    c.cycles = finish(y, d, c);
+    if (c.cycles >= 0 && (!best.ok || c.cycles < best.cycles)) best = c;
+  }
   return best;
 }
 
@@ -138,7 +138,7 @@ bool supported(const mebptt_lstm_desc* d) {
   state_layout(d, y);
   if (y.tensor_path || y.stepwise_tc || y.stepwise_x3 || y.L > kMaxLayers || y.t >= (1 << 30)) return false;
   const int clusters[5] = {148, 74, 36, 16, 7};
-  return pod::choose_config(y, y.tensor_cores, 148, clusters).ok || choose_config(y, 148, clusters).ok;
+  return pod::choose_config(y, y.tensor_cores, 148, clusters).ok || choose_config(y, 148).ok;
 }
 
 namespace {

@@ -106,7 +106,7 @@ double finish(const Layout& y, const Dims& d, Config& c) {
   for (int l = 0; l < y.L; ++l) keep(2 * l + 1, bytes_b(l));
   keep(63, bytes_r);
   c.smem = fixed + c.pool_floats * 4 + (int)held;
-  double cyc = 3 * 6500.0 + task_cycles(c, d, ur, d.hp, c.ns_r, esz, (c.resident >> 63) & 1, false);
+  double cyc = 3 * 9500.0 + task_cycles(c, d, ur, d.hp, c.ns_r, esz, (c.resident >> 63) & 1, false);
   for (int l = 0; l < y.L; ++l)
     cyc += 2 * task_cycles(c, d, uf, d.kf[l], c.ns_f[l], esz, (c.resident >> (2 * l)) & 1, false) +
            task_cycles(c, d, ub, d.kb[l], c.ns_b[l], esz, (c.resident >> (2 * l + 1)) & 1, true);

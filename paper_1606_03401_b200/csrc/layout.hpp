@@ -52,7 +52,7 @@ struct Layout {
   size_t rec_gates = 0;  // gates of layer 0
   size_t rec_in = 0;     // input hidden state
   // workspace offsets: states
-  size_t off_arena = 0, off_core = 0, off_core2 = 0, off_ping = 0, off_pong = 0, off_init = 0;
+  size_t off_arena = 0, off_core = 0, off_ping = 0, off_pong = 0, off_init = 0;
   // carried gradients and per-step scratch of the CUDA-core path
   size_t off_dh = 0, off_dc = 0, off_dha = 0, off_dz = 0, off_dy = 0;
   size_t off_loss_part = 0, off_loss_t = 0;
@@ -65,7 +65,11 @@ struct Layout {
   size_t off_sync = 0, off_tape = 0, off_status = 0, off_split_dh = 0;
   size_t off_a3_run = 0, off_zrun = 0, off_hrun = 0, off_dha_run = 0, off_dy_run = 0, split_floats = 0;
   size_t n_sync = 0, tape_bytes = 0;
-  // team path: packed weights per layer, readout weights, dz of the step after a chunk, end of what a step clears
+  // team path: states per group of batch rows, in blocks of one layer's h of the group (a cell state takes
+  // 4 / esz of them): blocks of a location's unit, of a hidden state, of all states; first blocks of the named states
+  int loc_blocks = 0, unit_blocks = 0;
+  int64_t n_blocks = 0, blk_core[2] = {}, blk_ping = 0, blk_pong = 0, blk_init = 0;
+  // packed weights per layer, readout weights, dz of the step after a chunk, end of what a step clears
   size_t off_wf[16] = {}, off_wb[16] = {}, off_wr = 0, off_carry = 0, off_zero_end = 0;
   size_t total = 0;
   int64_t arena_units = 0;
@@ -221,7 +225,8 @@ inline std::vector<WorkItem> work_items(const Plan* p, int S) {
 // packed weights are then done without)
 inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y, bool compact = false) {
   state_layout(d, y);
-  y.team = !compact && team::supported(d);
+  // (plans over byte sizes that are no whole blocks of the team path's states go without it)
+  y.team = !compact && (p->sigma <= 1 || (y.L * (1 + (int)(4 / y.esz))) % p->sigma == 0) && team::supported(d);
   y.arena_units = p->arena_units;
   y.loc_bytes = y.unit / (size_t)(p->sigma > 0 ? p->sigma : 1);
   size_t o = 0;
@@ -240,7 +245,23 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     if (y.S > 64) y.S = 64;
     if (y.S > y.t) y.S = (int)y.t;
     const size_t rows = (size_t)y.S * y.B;
-    y.off_core2 = take(y.rec);   // the working core alternates, so that one leaf's forward operation can pass the last one's backward
+    // States: a group of batch rows walks the tape without waiting for the others, so each has an arena of
+    // its own -- in one arena for all rows what one group writes for a later operation would lie over another
+    // group's rows of an earlier one.  Sizes are those of the common layout but for the rounding of rows to
+    // 16 bytes.  The working core alternates between two buffers, so that one leaf's forward operation can
+    // pass the last one's backward.
+    const int cr = (int)(4 / y.esz);
+    y.unit_blocks = y.L * (1 + cr);
+    const int rec_blocks = 2 * y.unit_blocks + 4 * y.L;
+    y.loc_blocks = y.unit_blocks / (p->sigma > 0 ? p->sigma : 1);
+    int64_t blocks = y.arena_units * y.loc_blocks;
+    auto named = [&](int64_t n) { const int64_t r = blocks; blocks += n; return r; };
+    y.blk_core[0] = named(rec_blocks); y.blk_core[1] = named(rec_blocks);
+    y.blk_ping = named(y.unit_blocks); y.blk_pong = named(y.unit_blocks); y.blk_init = named(y.unit_blocks);
+    y.n_blocks = blocks;
+    const size_t states = (size_t)blocks * y.B * align_up((size_t)y.H * y.esz + 15, 16);
+    if (o < y.off_arena + states) o = align_up(y.off_arena + states, y.granule);
+    y.off_loss_t = take((size_t)y.t * 4);
     // packed weights, in whichever of the two kernels' orders is used (the pod kernel pads rows, and
     // units to its CTAs: at most 16 and 96 more)
     auto larger = [](size_t u, size_t v) { return u > v ? u : v; };
@@ -250,7 +271,6 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
       y.off_wb[l] = take(h4 * (gp + (l + 1 < y.L ? gp : align_up(y.O, 16))) * y.esz);
     }
     y.off_wr = take(larger(align_up(y.O, 16) * hp, ((size_t)y.O + 64) * (y.H + 104)) * y.esz);
-    y.off_init = take(y.unit);   // the caller's initial state, laid out like a hidden state
     y.off_st_dz = y.off_dz = take((size_t)y.L * rows * G * 4);
     // h of the chunk's steps and of the one before: row block i holds h_{k-1} of the step in block i of dz
     y.off_st_h = take((size_t)y.L * (rows + y.B) * y.H * y.esz);

@@ -30,6 +30,7 @@ using team::cell_forward;
 using team::lane_sums;
 using team::load4;
 using team::part;
+using team::States;
 using team::store;
 using team::to_f;
 
@@ -79,7 +80,6 @@ __device__ __forceinline__ void mma(float (&c)[4], const uint32_t (&a)[4], const
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-__device__ __forceinline__ int log2i(int v) { return 31 - __clz(v); }
 
 // ---- products ------------------------------------------------------------------------------
 
@@ -87,8 +87,8 @@ __device__ __forceinline__ int log2i(int v) { return 31 - __clz(v); }
 // Lanes split the contraction index; the sums of unit / row group g, part s go to red[(g ns + s)][NB][4].
 template <int NB>
 __device__ __forceinline__ void rows_fma(const float* in, int pin, int nin, const float* h, int ph, int nh, const float* w, int ldw, int groups,
-                                         int ns, float* red, int wk, int lane) {
-  const int lg = log2i(ns), ia = (nin + 31) >> 5, its = ia + ((nh + 31) >> 5);
+                                         int lg, float* red, int wk, int lane) {
+  const int ns = 1 << lg, ia = (nin + 31) >> 5, its = ia + ((nh + 31) >> 5);
   for (; wk < groups * ns; wk += kWarps) {
     const int g = wk >> lg, s = wk & (ns - 1);
     const int lo = its * s >> lg, hi = its * (s + 1) >> lg;
@@ -131,8 +131,8 @@ __device__ __forceinline__ void rows_fma(const float* in, int pin, int nin, cons
 // another, so that a thread ends with the four gates of its unit for two batch rows.
 template <int NB>
 __device__ __forceinline__ void units_mma(uint32_t in, int nin, uint32_t h, int nh, uint32_t pin, uint32_t ph, uint32_t w, uint32_t ldw, int U,
-                                          int ns, float* red, int wk, int lane) {
-  const int lg = log2i(ns), steps = nin + nh, works = ((U + 7) >> 3) * ns;   // nin, nh: 16-wide steps
+                                          int lg, float* red, int wk, int lane) {
+  const int ns = 1 << lg, steps = nin + nh, works = ((U + 7) >> 3) * ns;   // nin, nh: 16-wide steps
   for (; wk < works; wk += kWarps) {
     const int g = wk >> lg, s = wk & (ns - 1), ng = min(8, U - 8 * g);
     const int lo = steps * s >> lg, hi = steps * (s + 1) >> lg;
@@ -161,9 +161,9 @@ __device__ __forceinline__ void units_mma(uint32_t in, int nin, uint32_t h, int 
 
 // R on the tensor cores: 16 readout rows a tile; red[(tile ns + s)][16][NB].
 template <int NB>
-__device__ __forceinline__ void readout_mma(uint32_t h, uint32_t ph, int steps, uint32_t w, uint32_t ldw, int rows, int ns, float* red, int wk,
+__device__ __forceinline__ void readout_mma(uint32_t h, uint32_t ph, int steps, uint32_t w, uint32_t ldw, int rows, int lg, float* red, int wk,
                                             int lane) {
-  const int lg = log2i(ns), works = ((rows + 15) >> 4) * ns;
+  const int ns = 1 << lg, works = ((rows + 15) >> 4) * ns;
   for (; wk < works; wk += kWarps) {
     const int g = wk >> lg, s = wk & (ns - 1), lo = steps * s >> lg, hi = steps * (s + 1) >> lg;
     const int row = min(16 * g + ((lane >> 3) & 1) * 8 + (lane & 7), rows - 1);
@@ -195,8 +195,7 @@ struct Share {
   int nc;                 // columns of one buffer
 };
 template <int NB>
-__device__ __forceinline__ void shares_fma(const float* d, const float* w, int ldw, int rows, int cols, int ns, int step, const Share& s, int tid) {
-  const int lg = log2i(ns);
+__device__ __forceinline__ void shares_fma(const float* d, const float* w, int ldw, int rows, int cols, int lg, int step, const Share& s, int tid) {
   for (int job = tid; job < cols << lg; job += kThreads) {
     int col = job, q = 0;
     while (col >= cols) { col -= cols; ++q; }
@@ -286,8 +285,6 @@ __device__ __forceinline__ void put_planes(bf16* p, int stride, float v) {
   }
 }
 
-struct Main { float v[7]; };   // what a cell needs from memory: see ahead()
-
 template <class T, bool GRU, int NB, int PL>
 __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ Args A) {
   constexpr bool MMA = std::is_same<T, bf16>::value;
@@ -297,6 +294,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   unsigned char* const ctl = smem + kWindows * kWindow * sizeof(Task);
   uint64_t* const bars = reinterpret_cast<uint64_t*>(ctl);                  // even and odd phases
   uint32_t* const peer = reinterpret_cast<uint32_t*>(ctl + 64);             // where each CTA's shared memory begins
+  volatile int* const dead = reinterpret_cast<volatile int*>(ctl + 128);    // a wait gave up
   unsigned char* const area = ctl + 1024;
   uint2* const to = reinterpret_cast<uint2*>(area + C.at_map);              // Share::to
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -308,6 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   const int u = units_of(rank);
 
   if (tid == 0) {
+    *dead = 0;
     sm100::mbar_init(bars, 1);
     sm100::mbar_init(bars + 1, 1);
     sm100::mbar_fence_init();
@@ -326,13 +325,13 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     const bool on = r < NT && j < units_of(r);
     to[i] = on ? make_uint2(peer[r] + ((rank * C.ns_b) * U + j) * NB * 4, peer[r]) : make_uint2(0, 0);
   }
-  // weights: layer by layer, then the readout.  (Where they lie is worked out again at each use: an array of
-  // pointers would live in local memory, and with this much shared memory taken there is no L1 to hold it.)
+  // weights: layer by layer, then the readout
   const int w0 = 4 * U * C.pitch_w(0), w1 = 4 * U * C.pitch_w(1);
   T* const held = reinterpret_cast<T*>(area + C.at_w);
-  auto weights = [&](int l) -> const T* {     // l == L: readout
-    if (MMA || C.resident) return held + (l ? w0 + (l - 1) * w1 : 0);
-    return reinterpret_cast<const T*>(A.ws + (l == L ? A.off_wr : A.off_wf[l])) + (size_t)rank * (l == L ? C.op * C.pitch_r() : l ? w1 : w0);
+  // weight `at` (counted from the start of the CTA's weights) where they are not held
+  auto slice = [&](int l, uint32_t at) -> const T* {   // l == L: readout
+    return reinterpret_cast<const T*>(A.ws + (l == L ? A.off_wr : A.off_wf[l])) + (size_t)rank * (l == L ? C.op * C.pitch_r() : l ? w1 : w0) +
+           (at - (l ? w0 + (l - 1) * w1 : 0));
   };
   if (C.resident)
     for (int l = 0; l <= L; ++l) {
@@ -349,9 +348,13 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   const bool sends = el < L && (eju & ~3) < u && eb < valid;   // (its group of four has a unit)
   const int row = pod * NB + eb, ej = rank * U + eju, lay = has ? el : 0;
   const size_t e = has ? (size_t)row * H + ej : 0;
-  // offsets into the workspace (under 4 GB here): state, gates, dz and h stages, carried dz, of this element
-  const uint32_t o_h = (uint32_t)(lay * A.hc + e * sizeof(T)), o_c = (uint32_t)(lay * A.hc + A.csz_off + e * 4);
-  const uint32_t o_g = (uint32_t)(A.rec_gates + lay * A.gsz + e * sizeof(T));
+  // offsets (all under 4 GB here) of this element: h, c and gates from the pod's states, dz and h stages and
+  // carried dz from the workspace
+  using St = States<T>;
+  const St S(A.ws + A.off_states, A.n_blocks, pod, NB, A.B, H);
+  const uint32_t le = eb * H + ej, hs_ = S.hs;
+  const uint32_t o_h = lay * (1 + St::CR) * hs_ + le * (uint32_t)sizeof(T), o_c = (lay * (1 + St::CR) + 1) * hs_ + le * 4;
+  const uint32_t o_g = (L * (1 + St::CR) + 4 * lay) * hs_ + le * (uint32_t)sizeof(T), o_in = (L * (1 + St::CR) + 4 * L) * hs_;
   const uint32_t bh = (uint32_t)A.B * H;                         // elements of a row block of the h stage, a quarter of those of dz
   const uint32_t o_dz = (uint32_t)(A.off_dz + (lay * (size_t)A.S * bh + e) * 16);
   const uint32_t o_cy = (uint32_t)(A.off_carry + ((size_t)lay * bh + e) * 16);
@@ -384,54 +387,55 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   for (int r = 0; r < NT; ++r) gh += (units_of(r) + 3) >> 2;
   const uint32_t by_h = valid * gh * 4 * (uint32_t)sizeof(T), by_x = valid * ((A.I + 3) >> 2) * 4 * (uint32_t)sizeof(T);
   const uint32_t by_p = NT * C.ns_b * u * NB * 4;
-  // where F(l) and R leave their partial sums, and the warp that starts with each
-  auto red_f = [&](int l) {
-    int o = 0;
-    for (int i = 0; i < l; ++i) o += (MMA ? (U + 7) / 8 * 8 : U) * C.ns_f[i] * NB * 4;
-    return o;
-  };
-  const int my_red = red_f(lay), red_r = red_f(L);
-  const uint32_t p_area = area0 + C.at_p;
-  auto p_at = [&](int l, int above, int par) { return p_area + (uint32_t)(((l * 2 + above) * 2 + par) * C.p_slot); };
-
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
   // ---- fetched one phase ahead ----
-  Main om;
-  float4 ol = make_float4(0.f, 0.f, 0.f, 0.f), ox = ol, oz = ol;
-  float o_target = 0.f;
-  auto at = [&](uint32_t o, uint32_t loc) { return A.ws + (o + (loc << 8)); };
-  auto task = [&](const uint4* ph, int i) { return reinterpret_cast<const Task*>(ph + 2 * i); };   // i: 1 + index
-  auto ahead = [&](const uint4* ph, const uint4& h0, const uint4& h1) {
-    const uint32_t r_x = h0.y >> 16;   // h0: n cells sums n_h | n_p n_x r d | x pad | main; h1: load carry
-    if (has) {
-      const int im = (h0.w >> (4 * el)) & 15, il = (h1.x >> (4 * el)) & 15, iz = (h1.y >> (4 * el)) & 15;
-      if (im) {
-        const Task& k = *task(ph, im);
-        if (k.kind == FWD) {
-          om.v[4] = GRU ? to_f(*reinterpret_cast<const T*>(at(o_h, k.src))) : *reinterpret_cast<const float*>(at(o_c, k.src));
-          if (!GRU && (k.flags & COPY_IN)) om.v[5] = to_f(*reinterpret_cast<const T*>(at(o_h, k.src)));
-        } else {
-          const char* g = at(o_g, k.src);
+  // Records are read as two 16-byte words; these pick fields of a task out of them.
+  auto rec = [&](int i) { return windows[i]; };               // i: 2 x record (+ 1 for the second half)
+  auto k_of = [](const uint4& a) { return (int)a.y; };
+  auto sidx_of = [](const uint4& b) { return b.x & 0xffff; };
+  auto sa_of = [](const uint4& b) { return (b.x >> 16) * 16; };
+  auto sb_of = [](const uint4& b) { return (b.y & 0xffff) * 16; };
+  auto so_of = [](const uint4& b) { return (b.y >> 16) * 16; };
+  auto red_of = [](const uint4& b) { return (b.w & 0xffff) * 16; };
+  auto flags_of = [](const uint4& a) { return a.x >> 16; };
+  constexpr uint32_t no_slot = (uint32_t)kNone * 16;
+  const int sh = has ? 4 * el : 28;                           // this layer's place in the header's index words (28: never used)
+  const int shs = sends ? 4 * el : 28;
+  float om[7];
+  float ol = 0.f, o_target = 0.f;
+  float4 ox = make_float4(0.f, 0.f, 0.f, 0.f), oz = ox;
+  auto at = [&](uint32_t o, uint32_t loc) { return S.base + (o + loc * hs_); };
+  // h0: n cells sums n_h | n_p n_x r x | products - | main     h1: load carry bwd -
+  auto ahead = [&](int cur, const uint4& h0, const uint4& h1) {
+    const int im = (h0.w >> sh) & 15, il = (h1.x >> sh) & 15, iz = (h1.y >> sh) & 15;
+    if (im) {
+      const uint4 a = rec(cur + 2 * im);
+      if ((h1.z >> sh) & 15) {
+        const char* g = at(o_g, a.z);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) om.v[q] = to_f(*reinterpret_cast<const T*>(g + q * A.plane));
-          om.v[4] = to_f(*reinterpret_cast<const T*>(at(o_h, k.dst)));
-          if (!GRU) {
-            om.v[5] = *reinterpret_cast<const float*>(at(o_c, k.src));
-            om.v[6] = *reinterpret_cast<const float*>(at(o_c, k.dst));
-          }
+        for (int q = 0; q < 4; ++q) om[q] = to_f(*reinterpret_cast<const T*>(g + q * hs_));
+        om[4] = to_f(*reinterpret_cast<const T*>(at(o_h, a.w)));
+        if (!GRU) {
+          om[5] = *reinterpret_cast<const float*>(at(o_c, a.z));
+          om[6] = *reinterpret_cast<const float*>(at(o_c, a.w));
         }
-      }
-      if (il) ol.x = to_f(*reinterpret_cast<const T*>(at(o_h, task(ph, il)->src)));
-      if (iz) {
-        const Task& k = *task(ph, iz);
-        oz = *reinterpret_cast<const float4*>(A.ws + (k.sidx == kNone ? o_cy + ((k.k + 1) & 1) * L * bh * 16 : o_dz + k.sidx * bh * 16));
+      } else {
+        om[4] = GRU ? to_f(*reinterpret_cast<const T*>(at(o_h, a.z))) : *reinterpret_cast<const float*>(at(o_c, a.z));
+        if (!GRU && (flags_of(a) & COPY_IN)) om[5] = to_f(*reinterpret_cast<const T*>(at(o_h, a.z)));
       }
     }
-    if (has_r && (r_x & 0xff)) o_target = __ldg(A.targets + i_r + (size_t)(task(ph, r_x & 0xff)->k - 1) * A.B * A.O);
-    if (has_x && (h0.z & 0xff)) {
-      const T* x = reinterpret_cast<const T*>(A.x) + i_x + (size_t)(task(ph, h0.z & 0xff)->k - 1) * A.B * A.I;
+    if (il) ol = to_f(*reinterpret_cast<const T*>(at(o_h, rec(cur + 2 * il).z)));
+    if (iz) {
+      const int k = k_of(rec(cur + 2 * iz));
+      const uint32_t sidx = sidx_of(rec(cur + 2 * iz + 1));
+      oz = *reinterpret_cast<const float4*>(A.ws + (sidx == kNone ? o_cy + ((k + 1) & 1) * L * bh * 16 : o_dz + sidx * bh * 16));
+    }
+    const uint32_t ir = (h0.y >> 16) & 0xff, ix = h0.y >> 24;
+    if (ir && has_r) o_target = __ldg(A.targets + i_r + (size_t)(k_of(rec(cur + 2 * ir)) - 1) * A.B * A.O);
+    if (ix && has_x) {
+      const T* x = reinterpret_cast<const T*>(A.x) + i_x + (size_t)(k_of(rec(cur + 2 * ix)) - 1) * A.B * A.I;
       ox.x = to_f(x[0]);
       ox.y = x_n > 1 ? to_f(x[1]) : 0.f;
       ox.z = x_n > 2 ? to_f(x[2]) : 0.f;
@@ -453,49 +457,50 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     else push4(to + off, __float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w), to + bar);
   };
 
+  // one phase's operand of F and B per layer: the same for every layer but the first
+  const int ldw0 = C.pitch_w(0), ldw1 = C.pitch_w(1), ldr = C.pitch_r();
+  const int step = U * NB * 4;
   int w = 0, i0 = 0, ph = 0;
   bool entered = true;       // first phase of a window
-  const uint4* cur = windows;
-  uint4 h0 = cur[0], h1 = cur[1];
+  int cur = 0;               // the phase's header: 2 x record
+  uint4 h0 = rec(0), h1 = rec(1);
   ahead(cur, h0, h1);
   for (; ph < A.phases; ++ph) {
     const uint32_t bar = bar0 - base + 8 * (ph & 1);
     const bool cells = (h0.x >> 8) & 0xff, sums = (h0.x >> 16) & 0xff;
-    unsigned char* const dz_buf = area + C.at_dz + (size_t)(ph & 1) * L * C.dz_buf;
-    float* const red = reinterpret_cast<float*>(area + C.at_red + (size_t)(ph & 1) * C.red_bytes);
-    bool ok = true;
-    if (ph > 0) ok = wait_for(bar0 + 8 * ((ph - 1) & 1), ((ph - 1) >> 1) & 1);
+    unsigned char* const dz_buf = area + C.at_dz + (ph & 1) * L * C.dz_buf;
+    const uint32_t red_par = (ph & 1) * C.red_bytes;
+    if (ph > 0 && !wait_for(bar0 + 8 * ((ph - 1) & 1), ((ph - 1) >> 1) & 1)) *dead = 1;
 
-    const int im = has ? (h0.w >> (4 * el)) & 15 : 0;
-    const Task* const mt = task(cur, im);
-    if (cells && has) {
-      const int iz = (h1.y >> (4 * el)) & 15;
-      float d[4];
-      bool on = false;
-      if (im && mt->kind == BWD) {
-        on = true;
-        float s0 = 0.f, s1 = 0.f;
-        const int par = mt->k & 1, n = NT * C.ns_b, step = U * NB;
-        const float* a = reinterpret_cast<const float*>(smem + p_at(el, 0, par)) + eju * NB + eb;
-        const float* b = reinterpret_cast<const float*>(smem + p_at(el, 1, par)) + eju * NB + eb;
-        if (!(mt->flags & FIRST))
+    // ---- gradients of the own units ----
+    if (cells) {
+      const int ib = (h1.z >> sh) & 15, iz = (h1.y >> sh) & 15;
+      if (ib | iz) {
+        float d[4];
+        if (ib) {
+          const uint4 a = rec(cur + 2 * ib), b = rec(cur + 2 * ib + 1);
+          const uint32_t fl = flags_of(a), sidx = sidx_of(b);
+          float s0 = 0.f, s1 = 0.f;
+          const float* p0 = reinterpret_cast<const float*>(area + sa_of(b)) + eju * NB + eb;
+          const float* p1 = reinterpret_cast<const float*>(area + sb_of(b)) + eju * NB + eb;
+          const int n = (fl & FIRST) ? 0 : NT * C.ns_b;
 #pragma unroll 4
-          for (int i = 0; i < n; ++i) s0 += a[i * step];
-#pragma unroll 4
-        for (int i = 0; i < n; ++i) s1 += b[i * step];
-        const float g[4] = {om.v[0], om.v[1], om.v[2], om.v[3]};
-        cell_backward<GRU>(s0 + s1, g, om.v[4], om.v[5], om.v[6], dc, d);
-        const float4 quad = make_float4(d[0], d[1], d[2], d[3]);
-        *reinterpret_cast<float4*>(A.ws + (o_dz + mt->sidx * bh * 16)) = quad;
-        if (mt->flags & CLOSE) *reinterpret_cast<float4*>(A.ws + (o_cy + (mt->k & 1) * L * bh * 16)) = quad;
-        T* const hs = reinterpret_cast<T*>(A.ws + (o_st + mt->sidx * bh * (uint32_t)sizeof(T)));
-        store(hs, om.v[4]);
-        if (mt->flags & OPEN) store(hs + bh, to_f(*reinterpret_cast<const T*>(at(o_h, mt->src))));
-      } else if (iz) {
-        on = true;
-        d[0] = oz.x; d[1] = oz.y; d[2] = oz.z; d[3] = oz.w;
-      }
-      if (on) {
+          for (int i = 0; i < NT * C.ns_b; ++i, p0 += U * NB, p1 += U * NB) {
+            const float v0 = *p0;
+            s1 += *p1;
+            if (i < n) s0 += v0;
+          }
+          const float g[4] = {om[0], om[1], om[2], om[3]};
+          cell_backward<GRU>(s0 + s1, g, om[4], om[5], om[6], dc, d);
+          const float4 quad = make_float4(d[0], d[1], d[2], d[3]);
+          *reinterpret_cast<float4*>(A.ws + (o_dz + sidx * bh * 16)) = quad;
+          T* const hs = reinterpret_cast<T*>(A.ws + (o_st + sidx * bh * (uint32_t)sizeof(T)));
+          store(hs, om[4]);
+          if (fl & CLOSE) *reinterpret_cast<float4*>(A.ws + (o_cy + (k_of(a) & 1) * L * bh * 16)) = quad;
+          if (fl & OPEN) store(hs + bh, to_f(*reinterpret_cast<const T*>(at(o_h, a.z))));
+        } else {
+          d[0] = oz.x; d[1] = oz.y; d[2] = oz.z; d[3] = oz.w;
+        }
         unsigned char* const my = dz_buf + el * C.dz_buf;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -504,137 +509,127 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
         }
       }
     }
-    bool stop = false;
-    if (cells || !sums) stop = __syncthreads_or(!ok);
+    if (cells || !sums) {
+      __syncthreads();
+      if (*dead) break;
+    }
 
     // ---- products ----
-    {
-      Share sh{to, 0, 0, bar, C.kh};
-      int first = 0;           // warp that takes the first piece of the next class
-      const int step = U * NB * 4;
-      auto back = [&](int l, bool input, bool own, int k) {
-        const int ldw = C.pitch_w(l), skip = input ? 0 : l ? C.kh : C.kx, cols = (input ? C.kh : 0) + (own ? C.kh : 0);
-        unsigned char* const d = dz_buf + l * C.dz_buf;
-        sh.dst1 = p_at(l, 0, (k - 1) & 1);
-        sh.dst0 = input ? p_at(l - 1, 1, k & 1) : sh.dst1;
-        if constexpr (MMA) {
-          shares_mma<NB, PL>(sm100::smem_u32(d), C.dz_pitch, sm100::smem_u32(weights(l) + skip), ldw * 2, 4 * U, cols, sh, (warp - first) & (kWarps - 1), lane);
-          first += cols >> 5;
-        } else {
-          shares_fma<NB>(reinterpret_cast<const float*>(d), weights(l) + skip, ldw, 4 * U, cols, C.ns_b, step, sh, tid);
-        }
-      };
 #pragma unroll 1
-      for (int l = 0; l < L; ++l) {
-        const int i = (h0.w >> (4 * l)) & 15, z = (h1.y >> (4 * l)) & 15;
-        if (z) back(l, false, true, task(cur, z)->k + 1);
-        if (!i) continue;
-        const Task& k = *task(cur, i);
-        if (k.kind == BWD) {
-          back(l, l > 0, !(k.flags & CLOSE), k.k);
-        } else {
-          const int wk = (warp - first) & (kWarps - 1), ldw = C.pitch_w(l), nin = l ? C.kh : C.kx, pin = l ? C.pitch_h : C.pitch_x;
-          float* const r = red + red_f(l);
-          unsigned char* const in = area + k.sa * 16;
-          unsigned char* const hs = area + k.sb * 16;
-          if constexpr (MMA) units_mma<NB>(sm100::smem_u32(in), nin / 16, sm100::smem_u32(hs), C.kh / 16, pin, C.pitch_h, sm100::smem_u32(weights(l)), ldw * 2, U, C.ns_f[l], r, wk, lane);
-          else rows_fma<NB>(reinterpret_cast<const float*>(in), pin / 4, nin / 4, reinterpret_cast<const float*>(hs), C.pitch_h / 4, C.kh / 4, weights(l), ldw, U, C.ns_f[l], r, wk, lane);
-          first += (MMA ? (U + 7) / 8 : U) * C.ns_f[l];
-        }
-      }
-      if (const int i = (h0.y >> 16) & 0xff) {       // R
-        const int wk = (warp - first) & (kWarps - 1);
-        unsigned char* const hs = area + task(cur, i)->sb * 16;
-        first += MMA ? ((C.op + 15) >> 4) * C.ns_r : 0;
-        if constexpr (MMA) readout_mma<NB>(sm100::smem_u32(hs), C.pitch_h, C.kh / 16, sm100::smem_u32(weights(L)), C.pitch_r() * 2, C.op, C.ns_r, red + red_r, wk, lane);
-        else rows_fma<NB>(nullptr, 0, 0, reinterpret_cast<const float*>(hs), C.pitch_h / 4, C.kh / 4, weights(L), C.pitch_r(), C.op / 4, C.ns_r, red + red_r, wk, lane);
-      }
-      if (const int i = h0.y >> 24) {                // D
-        const int k = task(cur, i)->k;
-        unsigned char* const d = area + C.at_dy + (k & 1) * C.dy_buf;
-        sh.dst0 = p_at(L - 1, 1, k & 1);
-        if constexpr (MMA) shares_mma<NB, PL>(sm100::smem_u32(d), C.dy_pitch, sm100::smem_u32(weights(L)), C.pitch_r() * 2, C.op, C.kh, sh, (warp - first) & (kWarps - 1), lane);
-        else shares_fma<NB>(reinterpret_cast<const float*>(d), weights(L), C.pitch_r(), C.op, C.kh, C.ns_b, step, sh, tid);
+    for (int i = 1; i <= (int)(h0.z & 0xff); ++i) {
+      const uint4 a = rec(cur + 2 * i), b = rec(cur + 2 * i + 1);
+      const uint32_t kind = a.x & 0xff, l = (a.x >> 8) & 0xff;
+      const int wk = (warp - (int)(a.x >> 24)) & (kWarps - 1);
+      const T* wp = MMA || C.resident ? held + b.z : slice(kind == READ || kind == DHA ? L : (int)l, b.z);
+      if (kind == FWD) {
+        float* const r = reinterpret_cast<float*>(area + red_of(b) + red_par);
+        if constexpr (MMA)
+          units_mma<NB>(sm100::smem_u32(area + sa_of(b)), l ? C.kh / 16 : C.kx / 16, sm100::smem_u32(area + sb_of(b)), C.kh / 16, l ? C.pitch_h : C.pitch_x, C.pitch_h,
+                        sm100::smem_u32(wp), (l ? ldw1 : ldw0) * 2, U, l ? C.lg_f1 : C.lg_f0, r, wk, lane);
+        else
+          rows_fma<NB>(reinterpret_cast<const float*>(area + sa_of(b)), (l ? C.pitch_h : C.pitch_x) / 4, (l ? C.kh : C.kx) / 4, reinterpret_cast<const float*>(area + sb_of(b)),
+                       C.pitch_h / 4, C.kh / 4, wp, l ? ldw1 : ldw0, U, l ? C.lg_f1 : C.lg_f0, r, wk, lane);
+      } else if (kind == READ) {
+        float* const r = reinterpret_cast<float*>(area + red_of(b) + red_par);
+        if constexpr (MMA) readout_mma<NB>(sm100::smem_u32(area + sb_of(b)), C.pitch_h, C.kh / 16, sm100::smem_u32(wp), ldr * 2, C.op, C.lg_r, r, wk, lane);
+        else rows_fma<NB>(nullptr, 0, 0, reinterpret_cast<const float*>(area + sb_of(b)), C.pitch_h / 4, C.kh / 4, wp, ldr, C.op / 4, C.lg_r, r, wk, lane);
+      } else {   // B, Z, D
+        const bool out = kind == DHA;
+        const Share sr{to, area0 + red_of(b), area0 + so_of(b), bar, C.kh};
+        unsigned char* const d = out ? area + sa_of(b) : dz_buf + l * C.dz_buf;
+        const int ld = out ? ldr : l ? ldw1 : ldw0, rows = out ? C.op : 4 * U, cols = b.w >> 16;
+        if constexpr (MMA) shares_mma<NB, PL>(sm100::smem_u32(d), out ? C.dy_pitch : C.dz_pitch, sm100::smem_u32(wp), ld * 2, rows, cols, sr, wk, lane);
+        else shares_fma<NB>(reinterpret_cast<const float*>(d), wp, ld, rows, cols, C.lg_b, step, sr, tid);
       }
     }
-    if (sums) stop |= __syncthreads_or(!ok);
-    if (stop) break;
+    if (sums) {
+      __syncthreads();
+      if (*dead) break;
+    }
     if (warp == kWarps - 1) {   // the operands have been read: a word to everybody, and what to expect oneself
       if (lane < NT) push(peer[lane] + area0 + C.at_dummy + 4 * rank, 0, peer[lane] + bar);
       if (lane == 31) sm100::mbar_arrive_expect_tx(bars + (ph & 1), (h0.x >> 24) * by_h + (h0.y & 0xff) * by_p + ((h0.y >> 8) & 0xff) * by_x + 4 * NT);
     }
 
     // ---- states, readouts, loads ----
-    if (h0.x >> 24 || sums) {
+    const uint32_t fwd = h0.w & ~h1.z;       // index words of the F tasks alone (a layer has an F or a B)
+    if (fwd) {
+      const int f = (fwd >> sh) & 15;
+      uint4 a{}, b{};
       float hv = 0.f;
-      const bool f = im && mt->kind == FWD;
       if (f) {
-        const int ns = C.ns_f[el];
-        const float4* p = reinterpret_cast<const float4*>(red + my_red) + eju * ns * NB + eb;
+        a = rec(cur + 2 * f); b = rec(cur + 2 * f + 1);
+        const int ns = 1 << (el ? C.lg_f1 : C.lg_f0);
+        const float4* p = reinterpret_cast<const float4*>(area + red_of(b) + red_par) + eju * ns * NB + eb;
         float z[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
         for (int q = 0; q < ns; ++q, p += NB) {
           const float4 r = *p;
           z[0] += r.x; z[1] += r.y; z[2] += r.z; z[3] += r.w;
         }
         float g[4], cv;
-        cell_forward<GRU>(z, bias, om.v[4], g, hv, cv);
+        cell_forward<GRU>(z, bias, om[4], g, hv, cv);
         T stored;
         store(&stored, hv);
-        *reinterpret_cast<T*>(at(o_h, mt->dst)) = stored;
+        *reinterpret_cast<T*>(at(o_h, a.w)) = stored;
         hv = to_f(stored);       // the others read what was stored
-        if (!GRU) *reinterpret_cast<float*>(at(o_c, mt->dst)) = cv;
-        if (mt->flags & GATES) {
-          char* gp = at(o_g, mt->dst);
+        if (!GRU) *reinterpret_cast<float*>(at(o_c, a.w)) = cv;
+        if (flags_of(a) & GATES) {
+          char* gp = at(o_g, a.w);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) store(reinterpret_cast<T*>(gp + q * A.plane), g[q]);
+          for (int q = 0; q < 4; ++q) store(reinterpret_cast<T*>(gp + q * hs_), g[q]);
         }
-        if (mt->flags & COPY_IN) {
-          store(reinterpret_cast<T*>(at(o_h, mt->dst) + A.rec_in), GRU ? om.v[4] : om.v[5]);
-          if (!GRU) *reinterpret_cast<float*>(at(o_c, mt->dst) + A.rec_in) = om.v[4];
+        if (flags_of(a) & COPY_IN) {
+          store(reinterpret_cast<T*>(at(o_h, a.w) + o_in), GRU ? om[4] : om[5]);
+          if (!GRU) *reinterpret_cast<float*>(at(o_c, a.w) + o_in) = om[4];
         }
       }
-      auto send = [&](float v, uint32_t so, bool on) {
-        const float4 q = gather4(v);
-        if (on)
-          for (int r = eju & 3; r < NT; r += 4) push_quad(peer[r], area0 + so * 16 + at_push, q, bar);
-      };
-      if (h0.w) {
-        // (a group of four may hold units past the last one: their tasks are those of the group)
-        const int gi = sends ? (h0.w >> (4 * el)) & 15 : 0;
-        const Task* const gt = task(cur, gi);
-        const bool on = gi && gt->kind == FWD && gt->so != kNone;
-        send(hv, on ? gt->so : 0, on);
-      }
-      if (h1.x) {
-        const int gi = sends ? (h1.x >> (4 * el)) & 15 : 0;
-        send(has ? ol.x : 0.f, gi ? task(cur, gi)->so : 0, gi != 0);
+      // (a group of four may hold units past the last one: their lanes send with it all the same)
+      const int gi = (fwd >> shs) & 15;
+      const uint32_t so = gi ? so_of(rec(cur + 2 * gi + 1)) : no_slot;
+      const float4 q = gather4(hv);
+      if (so != no_slot)
+        for (int r = eju & 3; r < NT; r += 4) push_quad(peer[r], area0 + so + at_push, q, bar);
+    }
+    if (h1.x) {
+      const int gi = (h1.x >> shs) & 15;
+      const float4 q = gather4(has ? ol : 0.f);
+      if (gi) {
+        const uint32_t so = so_of(rec(cur + 2 * gi + 1));
+        for (int r = eju & 3; r < NT; r += 4) push_quad(peer[r], area0 + so + at_push, q, bar);
       }
     }
-    if (has_r && ((h0.y >> 16) & 0xff)) {
-      const Task& k = *task(cur, (h0.y >> 16) & 0xff);
-      const float* p = red + red_r + (MMA ? ((rj >> 4) * C.ns_r * 16 + (rj & 15)) * NB + rb : (rj >> 2) * C.ns_r * NB * 4 + rb * 4 + (rj & 3));
+    const uint32_t ir = (h0.y >> 16) & 0xff, ix = h0.y >> 24;
+    if (ir && has_r) {
+      const uint4 b = rec(cur + 2 * ir + 1);
+      const int ns = 1 << C.lg_r;
+      const float* p = reinterpret_cast<const float*>(area + red_of(b) + red_par) +
+                       (MMA ? ((rj >> 4) * ns * 16 + (rj & 15)) * NB + rb : (rj >> 2) * ns * NB * 4 + rb * 4 + (rj & 3));
       float z = 0.f;
-      for (int q = 0; q < C.ns_r; ++q, p += MMA ? 16 * NB : NB * 4) z += *p;
+      for (int q = 0; q < ns; ++q, p += MMA ? 16 * NB : NB * 4) z += *p;
       const float dy = 2.f * (z + r_bias - o_target) * dy_scale;
-      reinterpret_cast<float*>(A.ws + A.off_dy)[i_r + k.sidx * A.B * A.O] = dy;
-      unsigned char* const d = area + C.at_dy + (k.k & 1) * C.dy_buf;
+      reinterpret_cast<float*>(A.ws + A.off_dy)[i_r + sidx_of(b) * A.B * A.O] = dy;
+      unsigned char* const d = area + so_of(b);
       if (MMA) put_planes<PL>(reinterpret_cast<bf16*>(d) + rb * (C.dy_pitch / 2) + rj, NB * (C.dy_pitch / 2), dy);
       else reinterpret_cast<float*>(d)[rj * NB + rb] = dy;
     }
-    if (has_x && (h0.z & 0xff)) {
-      const uint32_t off = area0 + task(cur, h0.z & 0xff)->so * 16 + xb * C.pitch_x + 4 * xg * (uint32_t)sizeof(T);
+    if (ix && has_x) {
+      const uint32_t off = area0 + so_of(rec(cur + 2 * ix + 1)) + xb * C.pitch_x + 4 * xg * (uint32_t)sizeof(T);
       for (int r = 0; r < NT; ++r) push_quad(peer[r], off, ox, bar);
     }
     if (entered && w + 2 < n_windows) load_window(w + 2);
     entered = false;
-    i0 += 1 + (h0.x & 0xff);
     if (ph + 1 < A.phases) {
-      cur = windows + ((w & (kWindows - 1)) * kWindow + i0) * 2;
-      if (i0 >= kWindow || (reinterpret_cast<const uint32_t*>(cur)[0] & 0xff) == 0) {
+      const int nx = i0 + 1 + (h0.x & 0xff);
+      i0 = nx;
+      cur = ((w & (kWindows - 1)) * kWindow + i0) * 2;
+      if (i0 < kWindow) h0 = rec(cur);
+      if (i0 >= kWindow || (h0.x & 0xff) == 0) {
         ++w; i0 = 0; entered = true;
-        cur = windows + (w & (kWindows - 1)) * kWindow * 2;
+        cur = (w & (kWindows - 1)) * kWindow * 2;
+        h0 = rec(cur);
       }
-      h0 = cur[0]; h1 = cur[1];
+      h1 = rec(cur + 1);
       ahead(cur, h0, h1);
     }
   }
@@ -662,8 +657,11 @@ __global__ void __launch_bounds__(256) pod_pack(const __grid_constant__ PackArgs
   const size_t bh = (size_t)P.B * H;
   for (int l = 0; l < L; ++l)
     for (size_t i = first; i < bh; i += all) {
-      reinterpret_cast<T*>(P.init + l * P.hc)[i] = reinterpret_cast<const T*>(P.h0)[l * bh + i];
-      reinterpret_cast<float*>(P.init + l * P.hc + P.csz_off)[i] = P.c0[l * bh + i];
+      const int b = (int)(i / H), g = b / C.nb;
+      const States<T> S(P.states, P.n_blocks, g, C.nb, P.B, H);
+      const size_t le = i - (size_t)g * C.nb * H;
+      S.h((uint32_t)P.init, l)[le] = reinterpret_cast<const T*>(P.h0)[l * bh + i];
+      S.c((uint32_t)P.init, l)[le] = P.c0[l * bh + i];
     }
   const int per = 4 * C.U, rows = C.T * (L * per + C.op);
   const T zero = T(0.f);

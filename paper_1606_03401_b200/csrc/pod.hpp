@@ -39,7 +39,7 @@ namespace pod {
 
 using team::kThreads;
 using team::kWarps;
-constexpr int kMaxLayers = 8;
+constexpr int kMaxLayers = 7;     // (an eighth place in the index words stays free)
 constexpr int kWindow = 64, kWindows = 4;     // records fetched at a time, windows held
 constexpr int kHSlots = 4, kXSlots = 4;       // h of a layer; x
 
@@ -51,23 +51,33 @@ enum Flag : uint8_t {
   CLOSE = 16,               // B: the chunk's first step: dz_k goes to the carry buffer, no share for step k - 1
   COUNT = 32
 };
-// A phase: a header, then its tasks.  At most one F or B, one load and one Z per layer, one R, one D
-// and one LOAD_X in a phase.
+// A phase: a header, then its tasks, those with products first.  At most one F or B, one load and one Z
+// per layer, one R, one D and one LOAD_X in a phase.  Everything that is the same for all CTAs is worked
+// out here: an instruction saved in a phase is saved a thousand times.
 struct Header {
   uint8_t n;                // tasks; 0: nothing but padding up to the next window
-  uint8_t cells;            // has B or Z: dz is formed before the products
+  uint8_t cells;            // has B, Z or D: what other threads left has to be waited for before the products
   uint8_t sums;             // has F or R: partial sums are read after the products
-  uint8_t n_h, n_p, n_x;    // pushes every CTA receives of: h, shares, x
-  uint8_t r, d, x, pad[3];  // 1 + index of the READ, DHA, LOAD_X task; 0: none
+  uint8_t n_h;              // pushes every CTA receives of: h,
+  uint8_t n_p, n_x;         // shares, x
+  uint8_t r, x;             // 1 + index of the READ, LOAD_X task; 0: none
+  uint8_t products;         // tasks with products
+  uint8_t pad[3];
   uint32_t main, load, carry;   // 4 bits per layer: 1 + index of its F or B, of its load, of its Z
-  uint32_t pad2[2];
+  uint32_t bwd;             // 4 bits per layer: 1 + index of its B
+  uint32_t pad2;
 };
 struct Task {
-  uint8_t kind, layer, flags, pad0;
+  uint8_t kind, layer, flags, rot;   // rot: warp that takes the first piece of the products
   int32_t k;
-  uint32_t src, dst;        // F: input state, record written; B: record of step k, state k-1; LOAD_H: the state.  256-byte units
-  uint16_t sidx, sa, sb, so;   // row block of step k in the stages; slots of the operands (input, h) and of the result, 16-byte units
-  uint32_t pad[2];
+  uint32_t src, dst;        // F: input state, record written; B: record of step k, state k-1; LOAD_H: the state.  Blocks from the start of the pod's states
+  // 16-byte units of the operand area:
+  //   F: sa input, sb h slot, so slot of the result (or kNone), red partial sums     R: sb, red; so dy
+  //   B: sa, sb shares received from step k + 1 and from above; so, red where shares for step k - 1 and for below are sent
+  //   Z: so as B    D: sa dy, so    loads: so
+  uint16_t sidx, sa, sb, so;
+  uint32_t w;               // first weight of the products, elements from the start of the CTA's weights
+  uint16_t red, cols;       // cols: B, Z, D: columns of the products
 };
 static_assert(sizeof(Header) == 32 && sizeof(Task) == 32, "records");
 constexpr uint16_t kNone = 0xffff;
@@ -82,6 +92,7 @@ struct Config {
   int rows_o = 0, op = 0;   // readout rows per CTA, the same padded to 4
   int extra = 0;            // elements added to a row of weights against bank conflicts
   int ns_f[kMaxLayers] = {}, ns_r = 1, ns_b = 1;   // parts the contraction index is cut into; shares a CTA sends per unit
+  int lg_f0 = 0, lg_f1 = 0, lg_r = 0, lg_b = 0;    // their logarithms (all layers but the first are alike)
   bool mma = false;         // bfloat16 weights on the tensor cores (else FMA on widened values)
   bool resident = false;    // the weights fit in shared memory
   int planes = 1;           // mma: bfloat16 planes a float32 gradient is split into
@@ -90,6 +101,9 @@ struct Config {
   int at_h = 0, at_p = 0, p_slot = 0, at_dz = 0, dz_buf = 0, dz_pitch = 0, at_dy = 0, dy_buf = 0, dy_pitch = 0;
   int at_red = 0, red_bytes = 0, at_dummy = 0, at_map = 0, at_w = 0;
   int smem = 0;
+  int red_f(int l) const { return (mma ? (U + 7) / 8 * 8 : U) * (l ? ns_f[1] : ns_f[0]) * nb * 16; }   // bytes of F(l)'s partial sums
+  int share_slot(int l, int above, int par) const { return at_p + ((l * 2 + above) * 2 + par) * p_slot; }
+  int w_at(int l) const { return l ? 4 * U * pitch_w(0) + (l - 1) * 4 * U * pitch_w(1) : 0; }   // elements; l = L: readout
   MEBPTT_BOTH int pitch_w(int l) const { return (l ? kh : kx) + kh + extra; }   // elements of a row of layer l's weights
   MEBPTT_BOTH int pitch_r() const { return kh + extra; }
   MEBPTT_BOTH int slot_x(int i) const { return i * x_slot; }

@@ -52,6 +52,8 @@ Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max
         c.ns_f[l] = c.mma ? parts(ng, (kin(c, l) + c.kh) / 16) : parts(c.U, slices(kin(c, l)) + slices(c.kh));
       c.ns_r = c.mma ? parts(ceil_div(c.op, 16), c.kh / 16) : parts(c.op / 4, slices(c.kh));
       c.ns_b = c.mma ? 1 : c.kh <= kThreads / 4 ? 4 : c.kh <= kThreads / 2 ? 2 : 1;
+      auto lg = [](int v) { int n = 0; while (1 << n < v) ++n; return n; };
+      c.lg_f0 = lg(c.ns_f[0]); c.lg_f1 = y.L > 1 ? lg(c.ns_f[1]) : 0; c.lg_r = lg(c.ns_r); c.lg_b = lg(c.ns_b);
       // the operand area
       c.pitch_x = c.mma ? (c.kx + 8) * 2 : c.kx * 4;
       c.pitch_h = c.mma ? (c.kh + 8) * 2 : c.kh * 4;
@@ -69,7 +71,7 @@ Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max
       c.at_dz = take((int64_t)2 * y.L * c.dz_buf);
       c.at_dy = take((int64_t)2 * c.dy_buf);
       int64_t red = c.mma ? (int64_t)ceil_div(c.op, 16) * 16 * c.ns_r * nb * 4 : (int64_t)c.op * c.ns_r * nb * 4;
-      for (int l = 0; l < y.L; ++l) red += (int64_t)(c.mma ? ng * 8 : c.U) * c.ns_f[l] * nb * 16;
+      for (int l = 0; l < y.L; ++l) red += c.red_f(l);
       c.red_bytes = (int)std::min<int64_t>((red + 15) & ~15ll, 1 << 26);
       c.at_red = take((int64_t)2 * c.red_bytes);
       c.at_dummy = take(64);
@@ -84,7 +86,7 @@ Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max
       c.smem = fixed + at + (c.resident ? (int)weights : 0);
       const int waves = ceil_div(c.pods, fit);
       const double active = (double)std::min(c.pods, fit) * c.T;
-      // (fitted to a scan of T and nb over four problems: a phase's fixed part is some 5000 cycles, whatever it does)
+      // (fitted to a scan of T and nb over four problems: a phase's fixed part is some 4000 cycles, whatever it does)
       double cyc_f = 0, cyc_b = 0;
       for (int l = 0; l < y.L; ++l) {
         const int kk = kin(c, l) + c.kh, nc = l ? kk : c.kh;
@@ -103,7 +105,7 @@ Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max
           cyc_f += f; cyc_b += b;
         }
       }
-      c.cycles = waves * (3 * (4500.0 + 20.0 * c.T) + 2 * cyc_f + cyc_b);
+      c.cycles = waves * (3 * (3500.0 + 20.0 * c.T) + 2 * cyc_f + cyc_b);
       c.ok = true;
       if (!best.ok || c.cycles < best.cycles) best = c;
     }
@@ -117,6 +119,7 @@ struct Item {                    // a task before its slots are known
   int64_t in = 0, out = 0;       // versions of the states it reads and writes (0: the caller's, else 1 + index of the operation)
 };
 using Key = int64_t;             // an operand vector: x_k, or h of a layer in some version
+inline bool has_products(const Task& t) { return t.kind == FWD || t.kind == READ || t.kind == BWD || t.kind == DHA || t.kind == CARRY; }
 inline Key key_x(int64_t k) { return k << 8 | 255; }
 inline Key key_h(int l, int64_t version) { return version << 8 | l; }
 
@@ -133,16 +136,11 @@ struct Builder {
   int64_t base = 0, top = -1, n_open = 0;
   std::vector<int64_t> cell, named, state, version, b_phase, d_phase;   // phases of B(l, k) at [l][k & 3], of D(k) at [k & 3]
   int core = 0;
-  uint32_t at_init, at_ping, at_pong, at_core[2], at_arena, loc_step;
 
   Builder(const Layout& y_, const Config& c_, Schedule& s_)
       : y(y_), c(c_), s(s_), cell((size_t)y_.arena_units, -1), named((size_t)4 * y_.L, -1),
         state((size_t)(y_.arena_units + 5) * y_.L, -1), version((size_t)y_.arena_units + 5, 0), b_phase((size_t)4 * y_.L, -1),
         d_phase(4, -1) {
-    at_init = (uint32_t)(y.off_init >> 8);
-    at_ping = (uint32_t)(y.off_ping >> 8); at_pong = (uint32_t)(y.off_pong >> 8);
-    at_core[0] = (uint32_t)(y.off_core >> 8); at_core[1] = (uint32_t)(y.off_core2 >> 8);
-    at_arena = (uint32_t)(y.off_arena >> 8); loc_step = (uint32_t)(y.loc_bytes >> 8);
   }
   size_t slot_of(int32_t loc) const {
     return loc >= 0 ? (size_t)loc + 5
@@ -150,17 +148,17 @@ struct Builder {
   }
   uint32_t address(int32_t loc) const {
     switch (loc) {
-      case MEBPTT_LOC_INIT: return at_init;
-      case MEBPTT_LOC_PING: return at_ping;
-      case MEBPTT_LOC_PONG: return at_pong;
-      case MEBPTT_LOC_CORE: return at_core[core];
-      default: return at_arena + (uint32_t)loc * loc_step;
+      case MEBPTT_LOC_INIT: return (uint32_t)y.blk_init;
+      case MEBPTT_LOC_PING: return (uint32_t)y.blk_ping;
+      case MEBPTT_LOC_PONG: return (uint32_t)y.blk_pong;
+      case MEBPTT_LOC_CORE: return (uint32_t)y.blk_core[core];
+      default: return (uint32_t)loc * (uint32_t)y.loc_blocks;
     }
   }
   int units(int32_t loc, int fmt) const {
     if (loc < 0) return 1;
-    const size_t bytes = fmt == MEBPTT_FMT_HIDDEN ? y.unit : fmt == MEBPTT_FMT_INTERNAL ? y.rec : y.rec_in;
-    return (int)((bytes + y.loc_bytes - 1) / y.loc_bytes);
+    const int blocks = fmt == MEBPTT_FMT_HIDDEN ? y.unit_blocks : y.unit_blocks + 4 * y.L + (fmt == MEBPTT_FMT_INTERNAL ? y.unit_blocks : 0);
+    return (blocks + y.loc_blocks - 1) / y.loc_blocks;
   }
   template <class F> void cells(int32_t loc, int n, int l, F f) {
     if (loc >= 0) { for (int i = 0; i < n && (size_t)(loc + i) < cell.size(); ++i) f(cell[(size_t)(loc + i)]); }
@@ -240,7 +238,7 @@ struct Builder {
       // its shares for the layer below take the place of those of step k + 2
       if (l > 0) after = std::max(after, b_phase[(size_t)(l - 1) * 4 + ((q + 2) & 3)]);
       if (op.dst_fmt == MEBPTT_FMT_INTERNAL) {
-        b.t.dst = b.t.src + (uint32_t)(y.rec_in >> 8);
+        b.t.dst = b.t.src + (uint32_t)(y.unit_blocks + 4 * y.L);
       } else {
         b.t.dst = address(op.aux);
         after = std::max(after, state[slot_of(op.aux) * L + l]);
@@ -413,18 +411,59 @@ struct Builder {
     auto pad = [&] { while (s.tasks.size() % kWindow) s.tasks.push_back(Task{}); };
     for (std::vector<Task>& ph : out) {
       if (ph.empty()) ph.push_back(Task{});                     // keeps its place as an empty phase
+      std::stable_sort(ph.begin(), ph.end(), [](const Task& u, const Task& v) { return has_products(u) > has_products(v); });
       Header h{};
       h.n = (uint8_t)ph.size();
+      int rot = 0;
       for (size_t i = 0; i < ph.size(); ++i) {
-        const Task& t = ph[i];
+        Task& t = ph[i];
         if (t.flags & COUNT) ++(t.kind == FWD ? g.fwd_ops : g.bwd_ops);
-        const uint32_t at = (uint32_t)(i + 1), nib = at << (4 * t.layer);
+        const int l = t.layer, L = y.L;
+        const uint32_t at = (uint32_t)(i + 1), nib = at << (4 * l);
+        h.products += has_products(t);
+        t.rot = (uint8_t)(rot & (kWarps - 1));
         switch (t.kind) {
-          case FWD: h.main |= nib; h.sums = 1; h.n_h += t.so != kNone; break;
-          case BWD: h.main |= nib; h.cells = 1; h.n_p += (t.flags & CLOSE ? 0 : 1) + (t.layer > 0); break;
-          case READ: h.r = (uint8_t)at; h.sums = 1; break;
-          case DHA: h.d = (uint8_t)at; h.cells = 1; ++h.n_p; break;   // (dy was left by other threads: the barrier before the products)
-          case CARRY: h.carry |= nib; h.cells = 1; ++h.n_p; break;
+          case FWD: {
+            h.main |= nib; h.sums = 1; h.n_h += t.so != kNone;
+            int red = c.at_red;
+            for (int j = 0; j < l; ++j) red += c.red_f(j);
+            t.red = u16(red); t.w = (uint32_t)c.w_at(l);
+            rot += (c.mma ? ceil_div(c.U, 8) : c.U) * (l ? c.ns_f[1] : c.ns_f[0]);
+            break;
+          }
+          case READ: {
+            h.r = (uint8_t)at; h.sums = 1;
+            int red = c.at_red;
+            for (int j = 0; j < L; ++j) red += c.red_f(j);
+            t.red = u16(red); t.w = (uint32_t)c.w_at(L); t.so = u16(c.at_dy + (t.k & 1) * c.dy_buf);
+            rot += ceil_div(c.op, c.mma ? 16 : 4) * c.ns_r;
+            break;
+          }
+          case BWD: {
+            const bool own = !(t.flags & CLOSE), below = l > 0;
+            h.main |= nib; h.bwd |= nib; h.cells = 1; h.n_p += own + below;
+            t.sa = u16(c.share_slot(l, 0, t.k & 1)); t.sb = u16(c.share_slot(l, 1, t.k & 1));
+            t.so = u16(c.share_slot(l, 0, (t.k - 1) & 1));
+            t.red = below ? u16(c.share_slot(l - 1, 1, t.k & 1)) : t.so;
+            t.w = (uint32_t)(c.w_at(l) + (below ? 0 : kin(c, l)));
+            t.cols = (uint16_t)((own + below) * c.kh);
+            rot += t.cols / 32;
+            break;
+          }
+          case CARRY:
+            h.carry |= nib; h.cells = 1; ++h.n_p;
+            t.so = t.red = u16(c.share_slot(l, 0, t.k & 1));
+            t.w = (uint32_t)(c.w_at(l) + kin(c, l));
+            t.cols = (uint16_t)c.kh;
+            rot += t.cols / 32;
+            break;
+          case DHA:   // (dy was left by other threads: the barrier before the products)
+            h.cells = 1; ++h.n_p;
+            t.sa = u16(c.at_dy + (t.k & 1) * c.dy_buf); t.so = t.red = u16(c.share_slot(L - 1, 1, t.k & 1));
+            t.w = (uint32_t)c.w_at(L);
+            t.cols = (uint16_t)c.kh;
+            rot += t.cols / 32;
+            break;
           case LOAD_H: h.load |= nib; ++h.n_h; break;
           case LOAD_X: h.x = (uint8_t)at; ++h.n_x; break;
           default: break;

@@ -14,7 +14,8 @@ namespace pod {
 struct Args {
   int L, I, H, O, B, S;
   Config c;
-  size_t hc, csz_off, plane, gsz, rec_gates, rec_in;   // bytes: layer stride of a hidden state, its c part, gate plane, a layer's planes; planes and input state in a record
+  size_t off_states;                   // states, by pod
+  int64_t n_blocks;
   char* ws;
   size_t off_wf[team::kMaxLayers], off_wr;
   size_t off_dz, off_hk, off_dy, off_carry, off_dc;
@@ -36,8 +37,9 @@ struct PackArgs {
   Config c;
   const void *W, *W_out, *h0;
   const float* c0;
-  char *wf[kMaxLayers], *wr, *init;
-  size_t w_off[kMaxLayers], hc, csz_off;
+  char *wf[kMaxLayers], *wr, *states;  // the initial state goes to block `init` of each pod's states
+  int64_t n_blocks, init;
+  size_t w_off[kMaxLayers];
   float* zero;
   size_t n_zero;
   int64_t* counters;

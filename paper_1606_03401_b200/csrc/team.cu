@@ -39,8 +39,8 @@ struct Args {
   int ns_f[kMaxLayers], ns_b[kMaxLayers], ns_r;
   uint64_t resident;
   int pool_floats;
-  size_t hc, csz_off, plane, gsz;      // bytes: layer stride of a hidden state, its c part, gate plane, a layer's planes
-  size_t rec_gates;                    // bytes into a record
+  size_t off_states;                   // states, by team
+  int64_t n_blocks;
   char* ws;
   size_t off_wf[kMaxLayers], off_wb[kMaxLayers], off_wr;
   size_t off_dz, off_hk, off_dy, off_carry, off_dc;
@@ -140,77 +140,58 @@ __device__ __forceinline__ void sixteen_rows(uint32_t a, uint32_t pitch, const u
   }
 }
 
-// The state of layer l in a block of whole-stack states.
-template <class T>
-__device__ __forceinline__ const T* h_at(const Args& A, uint32_t loc, int l) {
-  return reinterpret_cast<const T*>(A.ws + ((size_t)loc << 8) + (size_t)l * A.hc);
-}
-__device__ __forceinline__ const float* c_at(const Args& A, uint32_t loc, int l) {
-  return reinterpret_cast<const float*>(A.ws + ((size_t)loc << 8) + (size_t)l * A.hc + A.csz_off);
-}
-template <class T>
-__device__ __forceinline__ T* gates_at(const Args& A, uint32_t rec, int l) {
-  return reinterpret_cast<T*>(A.ws + ((size_t)rec << 8) + A.rec_gates + (size_t)l * A.gsz);
-}
-
 // What a task's element needs from memory beside its sums; fetched while the operands are staged.
 struct Operands { float v[9]; };
 
 template <class T, bool GRU>
-__device__ __forceinline__ void fetch(const Args& A, const Task& t, size_t row, int j, Operands& o) {
+__device__ __forceinline__ void fetch(const Args& A, const States<T>& S, const Task& t, size_t row, int lr, int j, Operands& o) {
   const int H = A.H, l = t.layer;
-  const size_t e = row * H + j;
+  const size_t e = row * H + j, le = (size_t)lr * H + j;   // among all rows, among the team's
   if (t.kind == FWD) {
     const float* bias = A.bias + (size_t)l * (GRU ? 3 : 4) * H + j;
 #pragma unroll
     for (int q = 0; q < (GRU ? 3 : 4); ++q) o.v[q] = __ldg(bias + (size_t)q * H);
     if (GRU) {
-      o.v[4] = to_f(ld_l2(h_at<T>(A, t.src, l) + e));
+      o.v[4] = to_f(ld_l2(S.h(t.src, l) + le));
     } else {
-      o.v[4] = ld_l2(c_at(A, t.src, l) + e);
-      if (t.flags & COPY_IN) o.v[5] = to_f(ld_l2(h_at<T>(A, t.src, l) + e));
+      o.v[4] = ld_l2(S.c(t.src, l) + le);
+      if (t.flags & COPY_IN) o.v[5] = to_f(ld_l2(S.h(t.src, l) + le));
     }
   } else if (t.kind == READ) {
     o.v[0] = __ldg(A.b_out + j);
     o.v[1] = __ldg(A.targets + ((size_t)(t.k - 1) * A.B + row) * A.O + j);
   } else {
-    const T* g = gates_at<T>(A, t.src, l) + e;
-    const size_t pl = A.plane / sizeof(T);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) o.v[q] = to_f(ld_l2(g + q * pl));
+    for (int q = 0; q < 4; ++q) o.v[q] = to_f(ld_l2(S.gate(t.src, A.L, l, q) + le));
     o.v[4] = ld_l2(reinterpret_cast<const float*>(A.ws + A.off_dc) + (size_t)l * A.B * H + e);
-    o.v[5] = to_f(ld_l2(h_at<T>(A, t.dst, l) + e));   // h_{k-1}
-    if (t.flags & CARRY_IN) o.v[6] = to_f(ld_l2(h_at<T>(A, t.src, l) + e));   // h_k
+    o.v[5] = to_f(ld_l2(S.h(t.dst, l) + le));   // h_{k-1}
+    if (t.flags & CARRY_IN) o.v[6] = to_f(ld_l2(S.h(t.src, l) + le));   // h_k
     if (!GRU) {
-      o.v[7] = ld_l2(c_at(A, t.src, l) + e);
-      o.v[8] = ld_l2(c_at(A, t.dst, l) + e);
+      o.v[7] = ld_l2(S.c(t.src, l) + le);
+      o.v[8] = ld_l2(S.c(t.dst, l) + le);
     }
   }
 }
 
 // z: the element's sums (four gates; one value for R and B).
 template <class T, bool GRU>
-__device__ __forceinline__ void apply(const Args& A, const Task& t, size_t row, int j, const Operands& o, const float (&z)[4]) {
+__device__ __forceinline__ void apply(const Args& A, const States<T>& S, const Task& t, size_t row, int lr, int j, const Operands& o, const float (&z)[4]) {
   const int H = A.H, l = t.layer;
-  const size_t e = row * H + j;
+  const size_t e = row * H + j, le = (size_t)lr * H + j;
   if (t.kind == FWD) {
-    char* dst = A.ws + ((size_t)t.dst << 8);
-    T* h_out = reinterpret_cast<T*>(dst + (size_t)l * A.hc) + e;
-    T* g = gates_at<T>(A, t.dst, l) + e;
-    const size_t pl = A.plane / sizeof(T);
-    char* in = A.ws + ((size_t)t.dst << 8) + A.rec_gates + (size_t)A.L * A.gsz;   // copy of the input state
     const float bias[4] = {o.v[0], o.v[1], o.v[2], o.v[3]}, cp = o.v[4];
     float gv[4], h, cv;
     cell_forward<GRU>(z, bias, cp, gv, h, cv);
-    store(h_out, h);
-    if (!GRU) reinterpret_cast<float*>(dst + (size_t)l * A.hc + A.csz_off)[e] = cv;
+    store(S.h(t.dst, l) + le, h);
+    if (!GRU) S.c(t.dst, l)[le] = cv;
     if (t.flags & GATES) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) store(g + q * pl, gv[q]);
+      for (int q = 0; q < 4; ++q) store(S.gate(t.dst, A.L, l, q) + le, gv[q]);
     }
     if (t.flags & COPY_IN) {
-      store(reinterpret_cast<T*>(in + (size_t)l * A.hc) + e, GRU ? cp : o.v[5]);
-      if (!GRU) reinterpret_cast<float*>(in + (size_t)l * A.hc + A.csz_off)[e] = cp;
+      const uint32_t in = States<T>::input(t.dst, A.L);
+      store(S.h(in, l) + le, GRU ? cp : o.v[5]);
+      if (!GRU) S.c(in, l)[le] = cp;
     }
   } else if (t.kind == READ) {
     const float d = z[0] + o.v[0] - o.v[1];
@@ -262,6 +243,7 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
   const int team = blockIdx.x / A.T, rank = blockIdx.x - team * A.T;
   const int H = A.H, L = A.L;
   const int row0 = team * A.rows, rows = min(A.rows, A.B - row0);
+  const States<T> S(A.ws + A.off_states, A.n_blocks, team, A.rows, A.B, H);
   if (tid == 0) s_flag = *A.status;   // an earlier launch gave up: do nothing
   int f0, f1, b0, b1, r0g, r1g;       // groups of this CTA
   part(A.d.gf, A.T, rank, f0, f1);
@@ -332,8 +314,8 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
         const int l = k.layer, width = width_of(k);
         float* const a = pool + k.a_off;
         // values as they are stored: float32, or bfloat16 rows width + 8 apart
-        auto plain = [&](const T* src, int len, int padded, int at) {
-          stage<NB>(src + (size_t)r0 * len, (size_t)len, len, padded, valid, warp, lane, [&](int b, int e, auto x) {
+        auto plain = [&](const T* src, int first, int len, int padded, int at) {
+          stage<NB>(src + (size_t)first * len, (size_t)len, len, padded, valid, warp, lane, [&](int b, int e, auto x) {
             if constexpr (MMA) *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a) + b * (width + 8) + at + e) = x;
             else *reinterpret_cast<float4*>(a + b * width + at + e) = widen(x);
           });
@@ -355,10 +337,10 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
           });
         };
         if (k.kind == FWD) {
-          plain(l ? h_at<T>(A, k.dst, l - 1) : reinterpret_cast<const T*>(A.x) + (size_t)(k.k - 1) * A.B * A.I, l ? H : A.I, A.d.ip[l], 0);
-          plain(h_at<T>(A, k.src, l), H, A.d.hp, A.d.ip[l]);
+          plain(l ? S.h(k.dst, l - 1) : reinterpret_cast<const T*>(A.x) + (size_t)(k.k - 1) * A.B * A.I, l ? sub * NB : r0, l ? H : A.I, A.d.ip[l], 0);
+          plain(S.h(k.src, l), sub * NB, H, A.d.hp, A.d.ip[l]);
         } else if (k.kind == READ) {
-          plain(h_at<T>(A, k.src, l), H, A.d.hp, 0);
+          plain(S.h(k.src, l), sub * NB, H, A.d.hp, 0);
         } else {
           const int G = 4 * H;
           const float* const dz = reinterpret_cast<const float*>(A.ws + A.off_dz);
@@ -385,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
       int eb = 0, ej = 0;
       if (tid < elems) {
         locate(tid, ek, eb, ej);
-        if (eb < valid) fetch<T, GRU>(A, *ek, (size_t)(r0 + eb), cols_at(ek->kind) + ej, o);
+        if (eb < valid) fetch<T, GRU>(A, S, *ek, (size_t)(r0 + eb), sub * NB + eb, cols_at(ek->kind) + ej, o);
       }
       __syncthreads();
       // partial sums
@@ -435,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
       for (int f = tid; f < elems; f += kThreads) {
         if (f != tid) {
           locate(f, ek, eb, ej);
-          if (eb < valid) fetch<T, GRU>(A, *ek, (size_t)(r0 + eb), cols_at(ek->kind) + ej, o);
+          if (eb < valid) fetch<T, GRU>(A, S, *ek, (size_t)(r0 + eb), sub * NB + eb, cols_at(ek->kind) + ej, o);
         }
         if (eb >= valid) continue;
         const Task& k = *ek;
@@ -452,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
           p += in;
           for (int s = 0; s < ns; ++s, p += NB * RPG) z[0] += *p;
         }
-        apply<T, GRU>(A, k, (size_t)(r0 + eb), cols_at(k.kind) + ej, o, z);
+        apply<T, GRU>(A, S, k, (size_t)(r0 + eb), sub * NB + eb, cols_at(k.kind) + ej, o, z);
       }
       if ((sub + 1) * NB < rows) __syncthreads();
     }
@@ -479,7 +461,7 @@ struct PackArgs {
   const T *W, *W_out;
   size_t w_off[kMaxLayers];
   T *wf[kMaxLayers], *wb[kMaxLayers], *wr;
-  char* init; size_t hc, csz_off;   // the caller's initial state goes to this block of states
+  char* states; int64_t n_blocks, init; int R;   // the caller's initial state goes to block `init` of each group's states
   const void* h0; const float* c0;
   int B;
   float* zero; size_t n_zero;     // carried gradients, sync lines, status
@@ -505,8 +487,11 @@ __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
   const size_t bh = (size_t)P.B * H;
   for (int l = 0; l < P.L; ++l)
     for (size_t i = blockIdx.x * 256 + threadIdx.x; i < bh; i += (size_t)gridDim.x * 256) {
-      reinterpret_cast<T*>(P.init + l * P.hc)[i] = reinterpret_cast<const T*>(P.h0)[l * bh + i];
-      reinterpret_cast<float*>(P.init + l * P.hc + P.csz_off)[i] = P.c0[l * bh + i];
+      const int b = (int)(i / H), g = b / P.R;
+      const States<T> S(P.states, P.n_blocks, g, P.R, P.B, H);
+      const size_t le = i - (size_t)g * P.R * H;
+      S.h((uint32_t)P.init, l)[le] = reinterpret_cast<const T*>(P.h0)[l * bh + i];
+      S.c((uint32_t)P.init, l)[le] = P.c0[l * bh + i];
     }
   auto tiles = [](int rows, int cols) { return ((rows + 31) / 32) * ((cols + 31) / 32); };
   int total = tiles(rr, P.d.hp);
@@ -992,7 +977,7 @@ int launch(const void* fn, int grid, int cluster, int smem, void** args, cudaStr
 }
 
 template <class T>
-void launch_pack(const Layout& y, const Dims& d, const tc::StepPtrs& io, cudaStream_t s) {
+void launch_pack(const Layout& y, const Dims& d, int rows, const tc::StepPtrs& io, cudaStream_t s) {
   PackArgs<T> P{};
   P.L = y.L; P.I = y.I; P.H = y.H; P.O = y.O; P.d = d;
   P.W = reinterpret_cast<const T*>(io.W); P.W_out = reinterpret_cast<const T*>(io.W_out);
@@ -1002,7 +987,7 @@ void launch_pack(const Layout& y, const Dims& d, const tc::StepPtrs& io, cudaStr
     P.wb[l] = reinterpret_cast<T*>(io.ws + y.off_wb[l]);
   }
   P.wr = reinterpret_cast<T*>(io.ws + y.off_wr);
-  P.init = io.ws + y.off_init; P.hc = y.hsz + y.csz; P.csz_off = y.hsz; P.h0 = io.h0; P.c0 = io.c0; P.B = y.B;
+  P.states = io.ws + y.off_arena; P.n_blocks = y.n_blocks; P.init = y.blk_init; P.R = rows; P.h0 = io.h0; P.c0 = io.c0; P.B = y.B;
   P.zero = reinterpret_cast<float*>(io.ws + y.off_dc);
   P.n_zero = (y.off_zero_end - y.off_dc) / 4;
   P.counters = io.counters;
@@ -1066,14 +1051,14 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.c = kept->pc;
     q.W = io.W; q.W_out = io.W_out; q.h0 = io.h0; q.c0 = io.c0;
     for (int l = 0; l < y.L; ++l) { q.wf[l] = io.ws + y.off_wf[l]; q.w_off[l] = y.w_layer_offset(l); }
-    q.wr = io.ws + y.off_wr; q.init = io.ws + y.off_init; q.hc = y.hsz + y.csz; q.csz_off = y.hsz;
+    q.wr = io.ws + y.off_wr; q.states = io.ws + y.off_arena; q.n_blocks = y.n_blocks; q.init = y.blk_init;
     q.zero = reinterpret_cast<float*>(io.ws + y.off_dc); q.n_zero = (y.off_zero_end - y.off_dc) / 4;
     q.counters = io.counters;
     pod::launch_pack(y.dtype, y.gru, q, s);
   } else if (y.dtype == MEBPTT_BF16) {
-    launch_pack<__nv_bfloat16>(y, d, io, s);
+    launch_pack<__nv_bfloat16>(y, d, c.rows, io, s);
   } else {
-    launch_pack<float>(y, d, io, s);
+    launch_pack<float>(y, d, c.rows, io, s);
   }
 
   Args a{};
@@ -1084,7 +1069,7 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.S = y.S;
     for (int l = 0; l < y.L; ++l) q.off_wf[l] = y.off_wf[l];
     q.off_wr = y.off_wr;
-    q.hc = y.hsz + y.csz; q.csz_off = y.hsz; q.plane = y.plane; q.gsz = y.gsz; q.rec_gates = y.rec_gates;
+    q.off_states = y.off_arena; q.n_blocks = y.n_blocks;
     q.ws = io.ws;
     q.off_dz = y.off_dz; q.off_hk = y.off_st_h; q.off_dy = y.off_dy; q.off_carry = y.off_carry; q.off_dc = y.off_dc;
     q.x = io.x; q.bias = io.b; q.b_out = io.b_out; q.targets = io.targets;
@@ -1094,7 +1079,6 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
   if (kept->pod) {
     common(pa);
     pa.c = kept->pc;
-    pa.rec_in = y.rec_in;
     pf = pod::kernel(y.dtype, y.gru, pa.c.nb);
     if (allow(reinterpret_cast<const void*>(pf)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
   } else {

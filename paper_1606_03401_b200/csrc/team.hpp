@@ -43,7 +43,7 @@ enum TaskFlag : uint8_t {
 struct Task {
   uint8_t kind, layer, flags, pad0;
   int32_t k;
-  uint32_t src;    // F: input state; R, B: record of step k.  256-byte units from the workspace base
+  uint32_t src;    // F: input state; R, B: record of step k.  blocks from the start of the team's states
   uint32_t dst;    // F: record written; B: state k-1 (whole-state block)
   uint32_t sidx;   // row block of step k in the stages
   uint32_t a_off, red_off, pad1;   // this task's share of the phase pool, in floats

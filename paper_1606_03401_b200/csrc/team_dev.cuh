@@ -47,6 +47,24 @@ __device__ __forceinline__ float lane_sums(float (&v)[N], int lane) {
   return v[0];
 }
 
+// The states of one group of batch rows (row R i and on, of group i): blocks of `hs` bytes -- one layer's h
+// of the group -- with a cell state in the CR blocks behind its h, layer after layer, then four gate blocks a
+// layer, then the input state.
+template <class T>
+struct States {
+  static constexpr int CR = (int)(4 / sizeof(T));
+  char* base;
+  uint32_t hs;
+  __host__ __device__ static uint32_t block(int rows, int H) { return ((uint32_t)rows * H * (uint32_t)sizeof(T) + 15) & ~15u; }
+  __host__ __device__ States(char* all, int64_t blocks, int group, int R, int B, int H)
+      : base(all + (size_t)group * blocks * block(R, H)), hs(block(R < B - group * R ? R : B - group * R, H)) {}
+  __host__ __device__ char* at(uint32_t block) const { return base + (size_t)block * hs; }
+  __host__ __device__ T* h(uint32_t loc, int l) const { return reinterpret_cast<T*>(at(loc + l * (1 + CR))); }
+  __host__ __device__ float* c(uint32_t loc, int l) const { return reinterpret_cast<float*>(at(loc + l * (1 + CR) + 1)); }
+  __host__ __device__ T* gate(uint32_t loc, int L, int l, int q) const { return reinterpret_cast<T*>(at(loc + L * (1 + CR) + 4 * l + q)); }
+  __host__ __device__ static uint32_t input(uint32_t loc, int L) { return loc + L * (1 + CR) + 4 * L; }
+};
+
 __device__ __forceinline__ void part(int n, int T, int r, int& lo, int& hi) {   // CTA r's share of n things
   lo = (int)((int64_t)n * r / T);
   hi = (int)((int64_t)n * (r + 1) / T);

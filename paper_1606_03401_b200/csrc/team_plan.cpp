@@ -106,7 +106,7 @@ double finish(const Layout& y, const Dims& d, Config& c) {
   for (int l = 0; l < y.L; ++l) keep(2 * l + 1, bytes_b(l));
   keep(63, bytes_r);
   c.smem = fixed + c.pool_floats * 4 + (int)held;
-  double cyc = 3 * 9500.0 + task_cycles(c, d, ur, d.hp, c.ns_r, esz, (c.resident >> 63) & 1, false);
+  double cyc = 3 * 10500.0 + task_cycles(c, d, ur, d.hp, c.ns_r, esz, (c.resident >> 63) & 1, false);
   for (int l = 0; l < y.L; ++l)
     cyc += 2 * task_cycles(c, d, uf, d.kf[l], c.ns_f[l], esz, (c.resident >> (2 * l)) & 1, false) +
            task_cycles(c, d, ub, d.kb[l], c.ns_b[l], esz, (c.resident >> (2 * l + 1)) & 1, true);
@@ -161,23 +161,18 @@ struct Scheduler {
   std::vector<int64_t> state;              // [location slot][L]
   std::vector<int64_t> bwd_prev;           // per layer: phase of the latest B
   int core = 0;                            // the working core alternates between two buffers
-  uint32_t base_pingpong[2], base_core[2], base_arena, loc_step;
 
   Scheduler(const Layout& y_, const Config& c_, Schedule& s_, int64_t arena_units)
       : y(y_), c(c_), d(dims(y_)), s(s_), cell((size_t)arena_units, -1), named((size_t)4 * y_.L, -1), state((size_t)(arena_units + 5) * y_.L, -1),
         bwd_prev((size_t)y_.L, -1) {
-    base_pingpong[0] = (uint32_t)(y.off_ping >> 8); base_pingpong[1] = (uint32_t)(y.off_pong >> 8);
-    base_core[0] = (uint32_t)(y.off_core >> 8); base_core[1] = (uint32_t)(y.off_core2 >> 8);
-    base_arena = (uint32_t)(y.off_arena >> 8);
-    loc_step = (uint32_t)(y.loc_bytes >> 8);
   }
   uint32_t address(int32_t loc) const {
     switch (loc) {
-      case MEBPTT_LOC_INIT: return (uint32_t)(y.off_init >> 8);
-      case MEBPTT_LOC_PING: return base_pingpong[0];
-      case MEBPTT_LOC_PONG: return base_pingpong[1];
-      case MEBPTT_LOC_CORE: return base_core[core];
-      default: return base_arena + (uint32_t)loc * loc_step;
+      case MEBPTT_LOC_INIT: return (uint32_t)y.blk_init;
+      case MEBPTT_LOC_PING: return (uint32_t)y.blk_ping;
+      case MEBPTT_LOC_PONG: return (uint32_t)y.blk_pong;
+      case MEBPTT_LOC_CORE: return (uint32_t)y.blk_core[core];
+      default: return (uint32_t)loc * (uint32_t)y.loc_blocks;
     }
   }
   int64_t* state_of(int32_t loc) {
@@ -187,8 +182,8 @@ struct Scheduler {
   }
   int units(int32_t loc, int fmt) const {   // cells a record takes
     if (loc < 0) return 1;
-    const size_t bytes = fmt == MEBPTT_FMT_HIDDEN ? y.unit : fmt == MEBPTT_FMT_INTERNAL ? y.rec : y.rec_in;
-    return (int)((bytes + y.loc_bytes - 1) / y.loc_bytes);
+    const int blocks = fmt == MEBPTT_FMT_HIDDEN ? y.unit_blocks : y.unit_blocks + 4 * y.L + (fmt == MEBPTT_FMT_INTERNAL ? y.unit_blocks : 0);
+    return (blocks + y.loc_blocks - 1) / y.loc_blocks;
   }
   template <class F> void cells(int32_t loc, int n, int l, F f) {
     if (loc >= 0) { for (int i = 0; i < n && (size_t)(loc + i) < cell.size(); ++i) f(cell[(size_t)(loc + i)]); }
@@ -287,7 +282,7 @@ struct Scheduler {
       b.src = address(op.src);
       int64_t after = std::max(std::max(in[l], above), bwd_prev[(size_t)l]);
       if (op.dst_fmt == MEBPTT_FMT_INTERNAL) {
-        b.dst = b.src + (uint32_t)(y.rec_in >> 8);
+        b.dst = b.src + (uint32_t)(y.unit_blocks + 4 * y.L);
       } else {
         b.dst = address(op.aux);
         after = std::max(after, state_of(op.aux)[l]);

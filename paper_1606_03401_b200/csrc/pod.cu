@@ -53,16 +53,17 @@ __device__ __forceinline__ void push4(uint32_t addr, uint32_t a, uint32_t b, uin
                "r"(c), "r"(d), "r"(bar)
                : "memory");
 }
+// (The hint lets the hardware hold the warp until the barrier turns, for 20 us a time, instead of having it
+// poll: sixteen polling warps take issue slots from the ones that still work.)
 __device__ __forceinline__ bool wait_for(uint32_t bar, uint32_t parity) {
-  for (uint32_t i = 0; i < sm100::kSpinLimit; ++i) {
+  for (uint32_t i = 0; i < (1u << 16); ++i) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
     if (ok) return true;
-    if (i > 1024) __nanosleep(64);
   }
   return false;
 }
@@ -401,6 +402,8 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   auto red_of = [](const uint4& b) { return (b.w & 0xffff) * 16; };
   auto flags_of = [](const uint4& a) { return a.x >> 16; };
   constexpr uint32_t no_slot = (uint32_t)kNone * 16;
+  // whether any thread of the warp has an element of the kind: the others have nothing to do but products
+  const bool warp_s = __any_sync(0xffffffffu, sends), warp_r = __any_sync(0xffffffffu, has_r), warp_x = __any_sync(0xffffffffu, has_x);
   const int sh = has ? 4 * el : 28;                           // this layer's place in the header's index words (28: never used)
   const int shs = sends ? 4 * el : 28;
   float om[7];
@@ -409,6 +412,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   auto at = [&](uint32_t o, uint32_t loc) { return S.base + (o + loc * hs_); };
   // h0: n cells sums n_h | n_p n_x r x | products - | main     h1: load carry bwd -
   auto ahead = [&](int cur, const uint4& h0, const uint4& h1) {
+    if (warp_s) {
     const int im = (h0.w >> sh) & 15, il = (h1.x >> sh) & 15, iz = (h1.y >> sh) & 15;
     if (im) {
       const uint4 a = rec(cur + 2 * im);
@@ -432,9 +436,10 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
       const uint32_t sidx = sidx_of(rec(cur + 2 * iz + 1));
       oz = *reinterpret_cast<const float4*>(A.ws + (sidx == kNone ? o_cy + ((k + 1) & 1) * L * bh * 16 : o_dz + sidx * bh * 16));
     }
+    }
     const uint32_t ir = (h0.y >> 16) & 0xff, ix = h0.y >> 24;
-    if (ir && has_r) o_target = __ldg(A.targets + i_r + (size_t)(k_of(rec(cur + 2 * ir)) - 1) * A.B * A.O);
-    if (ix && has_x) {
+    if (warp_r && ir && has_r) o_target = __ldg(A.targets + i_r + (size_t)(k_of(rec(cur + 2 * ir)) - 1) * A.B * A.O);
+    if (warp_x && ix && has_x) {
       const T* x = reinterpret_cast<const T*>(A.x) + i_x + (size_t)(k_of(rec(cur + 2 * ix)) - 1) * A.B * A.I;
       ox.x = to_f(x[0]);
       ox.y = x_n > 1 ? to_f(x[1]) : 0.f;
@@ -473,7 +478,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     if (ph > 0 && !wait_for(bar0 + 8 * ((ph - 1) & 1), ((ph - 1) >> 1) & 1)) *dead = 1;
 
     // ---- gradients of the own units ----
-    if (cells) {
+    if (cells && warp_s) {
       const int ib = (h1.z >> sh) & 15, iz = (h1.y >> sh) & 15;
       if (ib | iz) {
         float d[4];
@@ -517,9 +522,13 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     // ---- products ----
 #pragma unroll 1
     for (int i = 1; i <= (int)(h0.z & 0xff); ++i) {
-      const uint4 a = rec(cur + 2 * i), b = rec(cur + 2 * i + 1);
+      const uint4 a = rec(cur + 2 * i);
       const uint32_t kind = a.x & 0xff, l = (a.x >> 8) & 0xff;
       const int wk = (warp - (int)(a.x >> 24)) & (kWarps - 1);
+      if (kind == FWD && wk >= (l ? C.works_f1 : C.works_f0)) continue;
+      if (kind == READ && wk >= C.works_r) continue;
+      const uint4 b = rec(cur + 2 * i + 1);
+      if (MMA && wk >= (int)(b.w >> 21) && kind != FWD && kind != READ) continue;   // cols / 32
       const T* wp = MMA || C.resident ? held + b.z : slice(kind == READ || kind == DHA ? L : (int)l, b.z);
       if (kind == FWD) {
         float* const r = reinterpret_cast<float*>(area + red_of(b) + red_par);
@@ -553,7 +562,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
 
     // ---- states, readouts, loads ----
     const uint32_t fwd = h0.w & ~h1.z;       // index words of the F tasks alone (a layer has an F or a B)
-    if (fwd) {
+    if (fwd && warp_s) {
       const int f = (fwd >> sh) & 15;
       uint4 a{}, b{};
       float hv = 0.f;
@@ -591,7 +600,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
       if (so != no_slot)
         for (int r = eju & 3; r < NT; r += 4) push_quad(peer[r], area0 + so + at_push, q, bar);
     }
-    if (h1.x) {
+    if (h1.x && warp_s) {
       const int gi = (h1.x >> shs) & 15;
       const float4 q = gather4(has ? ol : 0.f);
       if (gi) {
@@ -600,7 +609,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
       }
     }
     const uint32_t ir = (h0.y >> 16) & 0xff, ix = h0.y >> 24;
-    if (ir && has_r) {
+    if (warp_r && ir && has_r) {
       const uint4 b = rec(cur + 2 * ir + 1);
       const int ns = 1 << C.lg_r;
       const float* p = reinterpret_cast<const float*>(area + red_of(b) + red_par) +
@@ -613,7 +622,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
       if (MMA) put_planes<PL>(reinterpret_cast<bf16*>(d) + rb * (C.dy_pitch / 2) + rj, NB * (C.dy_pitch / 2), dy);
       else reinterpret_cast<float*>(d)[rj * NB + rb] = dy;
     }
-    if (ix && has_x) {
+    if (warp_x && ix && has_x) {
       const uint32_t off = area0 + so_of(rec(cur + 2 * ix + 1)) + xb * C.pitch_x + 4 * xg * (uint32_t)sizeof(T);
       for (int r = 0; r < NT; ++r) push_quad(peer[r], off, ox, bar);
     }

@@ -92,6 +92,7 @@ struct Config {
   int rows_o = 0, op = 0;   // readout rows per CTA, the same padded to 4
   int extra = 0;            // elements added to a row of weights against bank conflicts
   int ns_f[kMaxLayers] = {}, ns_r = 1, ns_b = 1;   // parts the contraction index is cut into; shares a CTA sends per unit
+  int works_f0 = 0, works_f1 = 0, works_r = 0;     // pieces of work of F and R
   int lg_f0 = 0, lg_f1 = 0, lg_r = 0, lg_b = 0;    // their logarithms (all layers but the first are alike)
   bool mma = false;         // bfloat16 weights on the tensor cores (else FMA on widened values)
   bool resident = false;    // the weights fit in shared memory

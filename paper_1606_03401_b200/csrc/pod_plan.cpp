@@ -54,6 +54,7 @@ Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max
       c.ns_b = c.mma ? 1 : c.kh <= kThreads / 4 ? 4 : c.kh <= kThreads / 2 ? 2 : 1;
       auto lg = [](int v) { int n = 0; while (1 << n < v) ++n; return n; };
       c.lg_f0 = lg(c.ns_f[0]); c.lg_f1 = y.L > 1 ? lg(c.ns_f[1]) : 0; c.lg_r = lg(c.ns_r); c.lg_b = lg(c.ns_b);
+      c.works_f0 = (c.mma ? ng : c.U) << c.lg_f0; c.works_f1 = (c.mma ? ng : c.U) << c.lg_f1; c.works_r = ceil_div(c.op, c.mma ? 16 : 4) << c.lg_r;
       // the operand area
       c.pitch_x = c.mma ? (c.kx + 8) * 2 : c.kx * 4;
       c.pitch_h = c.mma ? (c.kh + 8) * 2 : c.kh * 4;

@@ -227,6 +227,7 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
   state_layout(d, y);
   // (plans over byte sizes that are no whole blocks of the team path's states go without it)
   y.team = !compact && (p->sigma <= 1 || (y.L * (1 + (int)(4 / y.esz))) % p->sigma == 0) && team::supported(d);
+  if (y.team) y.stepwise_tc = y.stepwise_x3 = false;
   y.arena_units = p->arena_units;
   y.loc_bytes = y.unit / (size_t)(p->sigma > 0 ? p->sigma : 1);
   size_t o = 0;

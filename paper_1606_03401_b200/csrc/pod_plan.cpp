@@ -87,7 +87,7 @@ Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max
       c.smem = fixed + at + (c.resident ? (int)weights : 0);
       const int waves = ceil_div(c.pods, fit);
       const double active = (double)std::min(c.pods, fit) * c.T;
-      // (fitted to a scan of T and nb over four problems: a phase's fixed part is some 4000 cycles, whatever it does)
+      // (fitted to a scan of T and nb over four problems: a phase's fixed part is some 4500 cycles, whatever it does)
       double cyc_f = 0, cyc_b = 0;
       for (int l = 0; l < y.L; ++l) {
         const int kk = kin(c, l) + c.kh, nc = l ? kk : c.kh;
@@ -103,10 +103,10 @@ Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max
             f = std::max(f, std::max(bf / 40.0, bf * active / 5000.0));
             b = std::max(b, std::max(bb / 40.0, bb * active / 5000.0));
           }
-          cyc_f += f; cyc_b += b;
+          cyc_f += f * (1.0 + 0.17 * nb); cyc_b += b * (1.0 + 0.17 * nb);
         }
       }
-      c.cycles = waves * (3 * (3500.0 + 20.0 * c.T) + 2 * cyc_f + cyc_b);
+      c.cycles = waves * (3 * (4400.0 + 20.0 * c.T) + 2 * cyc_f + cyc_b);
       c.ok = true;
       if (!best.ok || c.cycles < best.cycles) best = c;
     }

@@ -68,8 +68,6 @@ double task_cycles(const Config& c, const Dims& d, int groups_cta, int k, int ns
 // forward operations and one backward operation, or a negative value if the shape does not fit.
 double finish(const Layout& y, const Dims& d, Config& c) {
   const int uf = ceil_div(d.gf, c.T), ub = ceil_div(d.gb, c.T), ur = ceil_div(d.gr, c.T);
-  c.nb = 1;
-  while (c.nb < 8 && c.nb < c.rows) c.nb *= 2;
   const int esz = (int)y.esz, step = d.mma ? 64 : 128;   // least elements of the contraction index worth a piece of their own
   auto parts = [&](int groups, int k) { return std::max(1, std::min(ceil_div(k, step), kWarps / groups)); };
   c.ns_r = parts(ur, d.hp);
@@ -106,7 +104,7 @@ double finish(const Layout& y, const Dims& d, Config& c) {
   for (int l = 0; l < y.L; ++l) keep(2 * l + 1, bytes_b(l));
   keep(63, bytes_r);
   c.smem = fixed + c.pool_floats * 4 + (int)held;
-  double cyc = 3 * 10500.0 + task_cycles(c, d, ur, d.hp, c.ns_r, esz, (c.resident >> 63) & 1, false);
+  double cyc = 3 * 14000.0 + task_cycles(c, d, ur, d.hp, c.ns_r, esz, (c.resident >> 63) & 1, false);
   for (int l = 0; l < y.L; ++l)
     cyc += 2 * task_cycles(c, d, uf, d.kf[l], c.ns_f[l], esz, (c.resident >> (2 * l)) & 1, false) +
            task_cycles(c, d, ub, d.kb[l], c.ns_b[l], esz, (c.resident >> (2 * l + 1)) & 1, true);
@@ -123,22 +121,33 @@ Config choose_config(const Layout& y, int sms) {
   if (y.L > kMaxLayers) return best;
   const Dims d = dims(y);
   for (int teams = 1; teams <= sms / 17; ++teams) {
-    Config c;
-    c.T = sms / teams;
-    c.rows = ceil_div(y.B, std::min(teams, y.B));
-    c.teams = ceil_div(y.B, c.rows);
-    c.cycles = finish(y, d, c);
-    if (c.cycles >= 0 && (!best.ok || c.cycles < best.cycles)) best = c;
+    const int rows = ceil_div(y.B, std::min(teams, y.B));
+    for (int nb = 1; nb <= 8; nb *= 2) {   // rows taken at a time: as many as there are, if they fit
+      if (nb > 1 && nb >= 2 * rows) break;
+      Config c;
+      c.T = sms / teams; c.rows = rows; c.teams = ceil_div(y.B, rows); c.nb = nb;
+      c.cycles = finish(y, d, c);
+      if (c.cycles >= 0 && (!best.ok || c.cycles < best.cycles)) best = c;
+    }
   }
   return best;
 }
 
+// Shapes the step-by-step tensor-core kernels could take as well go to whichever is estimated faster:
+// they spend some 45 us a layer on two forward operations and a backward one whatever the widths (three
+// or four dependent launches each; measured from 160 to 1024 units), and stay ahead where the
+// recurrent weights are large.  (Asked for the layout, before a device is known: a B200 is assumed.)
 bool supported(const mebptt_lstm_desc* d) {
+  constexpr double kStepwise = 70000.0;   // cycles; a fifth less than measured, to be worth leaving
   Layout y;
   state_layout(d, y);
-  if (y.tensor_path || y.stepwise_tc || y.stepwise_x3 || y.L > kMaxLayers || y.t >= (1 << 30)) return false;
-  const int clusters[5] = {148, 74, 36, 16, 7};
-  return pod::choose_config(y, y.tensor_cores, 148, clusters).ok || choose_config(y, 148).ok;
+  if (y.tensor_path || y.L > kMaxLayers || y.t >= (1 << 30)) return false;
+  const int clusters[5] = {148, 74, 33, 15, 7};
+  const pod::Config pc = pod::choose_config(y, y.tensor_cores, 148, clusters);
+  const Config c = choose_config(y, 148);
+  if (!pc.ok && !c.ok) return false;
+  if (!y.stepwise_tc && !y.stepwise_x3) return true;
+  return (pc.ok && pc.cycles < kStepwise * y.L) || (c.ok && c.cycles < kStepwise * y.L);
 }
 
 namespace {

@@ -162,6 +162,11 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
     x3.a3_run = bf(y.off_a3_run);
     x3.h_run = reinterpret_cast<float*>(ws + y.off_hrun);
   }
+  stepwise3::RunsX3 runs{};
+  if (y.x3_runs) {
+    runs.w_f = bf(y.off_w_f); runs.w_b = bf(y.off_w_b); runs.exch_f = bf(y.off_exch_f); runs.exch_b = bf(y.off_exch_b);
+    runs.sync = reinterpret_cast<uint32_t*>(ws + y.off_sync); runs.n_sync = y.n_sync;
+  }
   const bool staged = y.stepwise_tc || y.stepwise_x3;   // weight gradients per chunk of S steps
   int rc = MEBPTT_OK;
 
@@ -174,7 +179,11 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
   cudaMemsetAsync(io.db_out, 0, (size_t)y.O * 4, s);
   cudaMemsetAsync(io.counters, 0, 8 * sizeof(int64_t), s);
 
-  if (y.stepwise_x3)
+  if (y.x3_runs) {
+    stepwise3::pack_input_weights(x3, desc->want_dx != 0, y.I, y.H, y.O, reinterpret_cast<const float*>(io.W),
+                                  reinterpret_cast<const float*>(io.W_out), s);
+    if (!stepwise3::runs_begin(runs, y.I, y.H, y.B, reinterpret_cast<const float*>(io.W), s)) return MEBPTT_ERR_UNSUPPORTED;
+  } else if (y.stepwise_x3)
     stepwise3::pack_weights(x3, y.L, y.I, y.H, y.O, reinterpret_cast<const float*>(io.W), w_off,
                             reinterpret_cast<const float*>(io.W_out), s);
   auto run_op = [&](const mebptt_op& op) {
@@ -253,7 +262,51 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
   // everything else, and the leaves of the recursion, go operation by operation.  Both give the
   // same bits; MEBPTT_STEPWISE_PER_OP=1 keeps to single operations (the tests compare the two).
   const bool per_op_only = env::stepwise_per_op();
-  if (!(y.stepwise_tc || y.stepwise_x3) || per_op_only) {
+  if (y.x3_runs) {
+    // a persistent launch per run, with what the run can batch before it (input projections; readout
+    // and the gradient entering h_k) and after it (the gradient of x)
+    std::vector<stepwise::FwdRunStep> fst((size_t)y.S);
+    std::vector<stepwise::BwdRunStep> bst((size_t)y.S);
+    std::vector<const float*> h_top((size_t)y.S);
+    float* zrun = reinterpret_cast<float*>(ws + y.off_zrun);
+    auto run = [&](const mebptt_op* ops, int n) {
+      if (ops[0].kind == MEBPTT_OP_FWD) {
+        for (int j = 0; j < n; ++j) {
+          const FwdPtrs q = fwd_ptrs(y, io, ops[j], 0);
+          fst[j] = stepwise::FwdRunStep{q.h_prev, q.c_prev, q.h_out, q.c_out, q.gates, q.h_in_copy, q.c_in_copy};
+        }
+        const float* x = reinterpret_cast<const float*>(io.x) + (size_t)(ops[0].k - 1) * y.B * y.I;
+        rc = stepwise3::project_run(x3, x, n, y.I, y.H, y.B, io.b, zrun, s);
+        if (rc == MEBPTT_OK) rc = stepwise3::forward_run(runs, fst.data(), n, zrun, plane_elems, io.counters, status, s);
+        return;
+      }
+      const int64_t k_lo = ops[n - 1].k;
+      const int s_lo = (int)((k_lo - 1) % y.S);
+      for (int i = 0; i < n; ++i) {
+        const BwdPtrs q = bwd_ptrs(y, io, ops[i], 0);
+        bst[i] = stepwise::BwdRunStep{q.gates, q.c_t, q.c_prev, q.in, q.h_prev};
+        h_top[n - 1 - i] = reinterpret_cast<const float*>(loc_base(y, ws, ops[i].src) + y.h_off(0));
+      }
+      rc = stepwise3::readout_run(h_top.data(), n, s_lo, io.b_out, io.targets + (size_t)(k_lo - 1) * y.B * y.O,
+                                  loss_t + (k_lo - 1), y.B, y.H, y.O, x3, s);
+      const size_t row = (size_t)s_lo * y.B;
+      if (rc == MEBPTT_OK)
+        rc = stepwise3::backward_run(runs, bst.data(), n, x3.dha_run, dh_rec, dc_rec, x3.st_dz3 + row * 12 * y.H,
+                                     x3.st_hp2 + row * 2 * y.H, x3.st_in2 + row * 2 * y.I, plane_elems, io.counters, status, s);
+      if (rc == MEBPTT_OK && desc->want_dx)
+        rc = stepwise3::input_gradient_run(x3, s_lo, n, y.I, y.H, y.B, io.dx + (size_t)(k_lo - 1) * y.B * y.I, s);
+      if (rc == MEBPTT_OK && s_lo == 0) {
+        const int64_t chunk = (k_lo - 1) / y.S;
+        const int steps = (int)((chunk + 1) * y.S <= y.t ? y.S : y.t - chunk * y.S);
+        rc = stepwise3::flush_chunk(x3, steps, 1, y.B, y.I, y.H, y.O, w_off, io.dW, io.dW_out, io.db, io.db_out, s);
+      }
+    };
+    for (const WorkItem& wi : work_items(p, y.S)) {
+      const bool single = wi.kind == WorkItem::LEAF || per_op_only;
+      const int ops = wi.kind == WorkItem::LEAF ? 2 * wi.n : wi.n;
+      for (int j = 0; j < ops && rc == MEBPTT_OK; j += single ? 1 : ops) run(p->tape.data() + wi.i + j, single ? 1 : ops);
+    }
+  } else if (!(y.stepwise_tc || y.stepwise_x3) || per_op_only) {
     for (const mebptt_op& op : p->tape) {
       if (rc != MEBPTT_OK) break;
       run_op(op);
@@ -530,6 +583,15 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
     const int64_t dha = tc::gemm_split_count(false, true, y.B, y.H, 3 * y.O, pf) > 1 ? 2 : 1;
     const int64_t bwd = L + L + to_h * (L - 1) + (desc->want_dx ? to_x : 0);   // dh = dz W_hh: one launch in any case
     const int64_t chunks = (p->t + y.S - 1) / y.S;
+    if (y.x3_runs) {
+      // packing; forward run: split, projection, run; backward run: readout, run, d_in; chunks as below
+      int64_t n = 5 + (desc->want_dx ? 1 : 0) + chunks * 11 + 1;
+      for (const WorkItem& wi : work_items(p, y.S)) {
+        const int64_t f = wi.kind == WorkItem::LEAF ? wi.n : wi.kind == WorkItem::FWD, b = wi.kind == WorkItem::LEAF ? wi.n : wi.kind == WorkItem::BWD;
+        n += 3 * f + (5 + dha + (desc->want_dx ? to_x : 0)) * b;
+      }
+      return n;
+    }
     // the readout of a run of n >= 2 backward operations is taken once for the run (the same
     // launches), and a run of n >= 2 forward operations splits its operands once per layer (then
     // GEMM and cell kernel per step)

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_bf16.h>
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <cstddef>
@@ -190,5 +191,29 @@ int flush_chunk(const Scratch& w, int steps, int L, int B, int I0, int H, int O,
 int forward_run_layer(const stepwise::FwdRunStep* st, int n, const float* in, int64_t in_step_stride, int I,
                       const float* bias, int B, int H, size_t plane_elems, int64_t* counters, const Scratch& w,
                       size_t w_off, float* h_stage, cudaStream_t s);
+// Runs of one layer's operations by persistent kernels (runs_x3.cu), for the shapes x3_runs_supported
+// (layout.hpp) names.  What the kernels need for one training step:
+struct RunsX3 {
+  __nv_bfloat16 *w_f, *w_b;        // W_hh in halves, in the two kernels' orders: [8 H][HP], [256 ceil(H / 32)][HP]
+  __nv_bfloat16 *exch_f, *exch_b;  // the vectors the CTAs exchange: [2][B / 32][64][HP], [2][B / 32][4][64][HP]
+  uint32_t* sync;                  // step counters, two lines of 128 bytes a launch
+  size_t n_sync;
+  int I, H, B, HP, groups;         // (filled in by runs_begin from here on)
+  int launches;
+  CUtensorMap tm_h, tm_w, tm_dz, tm_wt;
+};
+// Packs the weights W ([4H][I + H]) and clears what a step must find clear; false if a tensor map was refused.
+bool runs_begin(RunsX3& r, int I, int H, int B, const float* W, cudaStream_t s);
+// n <= 32 consecutive forward operations; zx: [n][B][4H], x W_ih + b of their steps.
+int forward_run(RunsX3& r, const stepwise::FwdRunStep* st, int n, const float* zx, size_t plane_elems, int64_t* counters,
+                int* status, cudaStream_t s);
+// n <= 32 backward operations, time descending; dha: [n][B][H] in ascending time, the stages likewise
+// from the run's first step in time.
+int backward_run(RunsX3& r, const stepwise::BwdRunStep* st, int n, const float* dha, float* dh, float* dc, __nv_bfloat16* st_dz3,
+                 __nv_bfloat16* st_hp2, __nv_bfloat16* st_in2, size_t plane_elems, int64_t* counters, int* status, cudaStream_t s);
+// The input products of a run on that path.  wih3: [4H][3I] and, for the gradient of the inputs, wmn3: [3 * 4H][I].
+void pack_input_weights(const Scratch& w, bool want_dx, int I, int H, int O, const float* W, const float* W_out, cudaStream_t s);
+int project_run(const Scratch& w, const float* x, int n, int I, int H, int B, const float* bias, float* zx, cudaStream_t s);
+int input_gradient_run(const Scratch& w, int s_lo, int n, int I, int H, int B, float* dx, cudaStream_t s);
 }  // namespace stepwise3
 }  // namespace mebptt

@@ -35,6 +35,7 @@ struct Layout {
   bool tensor_path = false;
   bool stepwise_tc = false;   // step-by-step operations with their contractions on the tensor cores
   bool stepwise_x3 = false;   // likewise for float32 storage, operands split into bfloat16 halves
+  bool x3_runs = false;       // of the latter, one layer whose runs persistent kernels take
   bool tensor_cores = true;   // not forbidden by the caller
   bool gru = false;           // the core is a GRU (CUDA-core kernels)
   bool team = false;          // CUDA-core shapes walked by the persistent kernel of team.cu
@@ -63,6 +64,7 @@ struct Layout {
   size_t off_z = 0, off_split = 0, off_st_dz = 0, off_st_in = 0, off_st_hp = 0, off_st_dy = 0, off_st_h = 0;
   size_t off_zx = 0, off_zleaf = 0, off_hprev = 0, off_hk = 0, off_y = 0;
   size_t off_sync = 0, off_tape = 0, off_status = 0, off_split_dh = 0;
+  size_t off_w_f = 0, off_w_b = 0, off_exch_f = 0, off_exch_b = 0;
   size_t off_a3_run = 0, off_zrun = 0, off_hrun = 0, off_dha_run = 0, off_dy_run = 0, split_floats = 0;
   size_t n_sync = 0, tape_bytes = 0;
   // team path: states per group of batch rows, in blocks of one layer's h of the group (a cell state takes
@@ -130,6 +132,14 @@ inline bool stepwise_x3_supported(const mebptt_lstm_desc* d) {
          (d->batch / 32) * ((d->readout + 31) / 32) <= 4096;
 }
 
+// Of those, the shapes whose runs the persistent kernels of runs_x3.cu take: one layer, 32 batch rows a
+// group of CTAs, a CTA per 8 hidden units (clusters of four share 32) with its halves of the weights in
+// shared memory beside a ring of the exchanged vector, and all groups on the device at once (33
+// clusters of four with a CTA an SM; at 64 rows that ends at 512 units, and wider layers go step by step).
+inline bool x3_runs_supported(const Layout& y) {
+  return y.stepwise_x3 && y.L == 1 && ((y.B == 32 && y.H <= 1024) || (y.B == 64 && y.H <= 512));
+}
+
 inline void state_layout(const mebptt_lstm_desc* d, Layout& y) {
   y.L = d->layers; y.I = d->input; y.H = d->hidden; y.O = d->readout; y.B = d->batch;
   y.dtype = d->dtype; y.t = d->t;
@@ -139,6 +149,7 @@ inline void state_layout(const mebptt_lstm_desc* d, Layout& y) {
   y.tensor_path = tensor_path_supported(d);
   y.stepwise_tc = stepwise_tc_supported(d);
   y.stepwise_x3 = stepwise_x3_supported(d);
+  y.x3_runs = x3_runs_supported(y);
   y.esz = (d->dtype == MEBPTT_BF16) ? 2 : 4;
   const size_t row = (size_t)y.H * y.esz;
   y.granule = 256 / gcd_sz(256, row) * row;  // lcm(256, row bytes)
@@ -227,7 +238,7 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
   state_layout(d, y);
   // (plans over byte sizes that are no whole blocks of the team path's states go without it)
   y.team = !compact && (p->sigma <= 1 || (y.L * (1 + (int)(4 / y.esz))) % p->sigma == 0) && team::supported(d);
-  if (y.team) y.stepwise_tc = y.stepwise_x3 = false;
+  if (y.team) y.stepwise_tc = y.stepwise_x3 = y.x3_runs = false;
   y.arena_units = p->arena_units;
   y.loc_bytes = y.unit / (size_t)(p->sigma > 0 ? p->sigma : 1);
   size_t o = 0;
@@ -321,16 +332,26 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
       const size_t rows = (size_t)y.S * y.B;
       y.off_z = take((size_t)y.B * G * 4);
       // the readout of a run of up to S steps at once; its split-K scratch as on the bfloat16 path
-      y.off_a3_run = take(rows * 3 * Kmax * 2);
+      y.off_a3_run = take(rows * 3 * (y.x3_runs ? (size_t)y.I : Kmax) * 2);
       y.off_hrun = take(y.L > 1 ? rows * y.H * 4 : 0);
+      if (y.x3_runs) {
+        const size_t hp = align_up(y.H, 64), groups = (size_t)y.B / 32;
+        y.off_zrun = take(rows * G * 4);
+        y.off_w_f = take((size_t)8 * y.H * hp * 2);
+        y.off_w_b = take(align_up(y.H, 32) * 8 * hp * 2);
+        y.off_exch_f = take(2 * groups * 64 * hp * 2);
+        y.off_exch_b = take(2 * groups * 256 * hp * 2);
+        y.n_sync = 64 * (p->tape.size() + 1);   // two lines a launch, at most an operation each
+        y.off_sync = take(y.n_sync * 4);
+      }
       y.off_dy_run = take(rows * y.O * 4);
       y.off_dha_run = take(rows * y.H * 4);
       y.split_floats = (size_t)148 * 128 * 128 * ((rows + 127) / 128);
       y.off_split = take(y.split_floats * 4);
-      y.off_split_dh = take((size_t)y.L * 148 * 128 * 128 * 4);
-      y.off_a3 = take((size_t)y.B * 3 * Kmax * 2);
-      y.off_w3 = take(3 * y.w_total_elems() * 2);
-      y.off_wmn3 = take(3 * y.w_total_elems() * 2);
+      y.off_split_dh = take(y.x3_runs ? 0 : (size_t)y.L * 148 * 128 * 128 * 4);
+      y.off_a3 = take(y.x3_runs ? 0 : (size_t)y.B * 3 * Kmax * 2);
+      y.off_w3 = take(y.x3_runs ? 3 * G * y.I * 2 : 3 * y.w_total_elems() * 2);
+      y.off_wmn3 = take(y.x3_runs ? (d->want_dx ? 3 * G * y.I * 2 : 0) : 3 * y.w_total_elems() * 2);
       y.off_wout3 = take((size_t)3 * y.O * y.H * 2);
       y.off_woutmn3 = take((size_t)3 * y.O * y.H * 2);
       y.off_st_dz = take((size_t)y.L * rows * 3 * G * 2);

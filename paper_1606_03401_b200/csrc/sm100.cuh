@@ -275,5 +275,27 @@ __device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
   asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// ---- bounded waits that share a CTA-wide failure flag --------------------------------------
+__device__ __forceinline__ bool wait_or_fail(uint64_t* bar, uint32_t parity, volatile int* failed) {
+  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if (i > 256) {
+      if (*failed) return false;
+      __nanosleep(64);
+    }
+  }
+  *failed = 1;
+  return false;
+}
+__device__ __forceinline__ bool wait_counter(const uint32_t* ctr, uint32_t target, volatile int* failed,
+                                             uint32_t limit = kSpinLimit >> 1) {
+  for (uint32_t i = 0; i < limit; ++i) {
+    if (ld_acquire(ctr) >= target) return true;
+    if (i > 4096 && *failed) return false;
+  }
+  *failed = 1;
+  return false;
+}
+
 }  // namespace sm100
 }  // namespace mebptt

@@ -44,27 +44,27 @@ __device__ __forceinline__ void split2(float v, bf16& hi, bf16& mid) {
 
 inline int ew_blocks(size_t n) { return (int)((n + 255) / 256 > 1184 ? 1184 : (n + 255) / 256); }
 
-// out [R][3C] = [hi | mid | hi] of W [R][C]: the right operand of a contraction over columns.
-__global__ void pack3_cols(const float* W, int R, int C, bf16* out) {
+// out [R][3C] = [hi | mid | hi] of W [R][C] (rows ld apart): the right operand of a contraction over columns.
+__global__ void pack3_cols(const float* W, int ld, int R, int C, bf16* out) {
   sm100::grid_dep_wait();
   sm100::grid_dep_launch();
   const size_t n = (size_t)R * C;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
     const size_t r = e / C, c = e % C;
     bf16 hi, mid;
-    split2(W[e], hi, mid);
+    split2(W[r * ld + c], hi, mid);
     bf16* o = out + r * 3 * (size_t)C + c;
     o[0] = hi; o[C] = mid; o[2 * (size_t)C] = hi;
   }
 }
-// out [3R][C] = [hi ; mid ; hi] of W [R][C]: the right operand of a contraction over rows.
-__global__ void pack3_rows(const float* W, int R, int C, bf16* out) {
+// out [3R][C] = [hi ; mid ; hi] of W [R][C] (rows ld apart): the right operand of a contraction over rows.
+__global__ void pack3_rows(const float* W, int ld, int R, int C, bf16* out) {
   sm100::grid_dep_wait();
   sm100::grid_dep_launch();
   const size_t n = (size_t)R * C;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
     bf16 hi, mid;
-    split2(W[e], hi, mid);
+    split2(W[e / C * ld + e % C], hi, mid);
     out[e] = hi; out[n + e] = mid; out[2 * n + e] = hi;
   }
 }
@@ -276,12 +276,36 @@ void pack_weights(const Scratch& w, int L, int I0, int H, int O, const float* W,
   for (int l = 0; l < L; ++l) {
     const int K = (l == 0 ? I0 : H) + H;
     const size_t n = (size_t)G * K;
-    launch_pdl(pack3_cols, dim3(ew_blocks(n)), dim3(256), 0, s, W + w_off[l], G, K, w.w3 + 3 * w_off[l]);
-    launch_pdl(pack3_rows, dim3(ew_blocks(n)), dim3(256), 0, s, W + w_off[l], G, K, w.wmn3 + 3 * w_off[l]);
+    launch_pdl(pack3_cols, dim3(ew_blocks(n)), dim3(256), 0, s, W + w_off[l], K, G, K, w.w3 + 3 * w_off[l]);
+    launch_pdl(pack3_rows, dim3(ew_blocks(n)), dim3(256), 0, s, W + w_off[l], K, G, K, w.wmn3 + 3 * w_off[l]);
   }
   const size_t no = (size_t)O * H;
-  launch_pdl(pack3_cols, dim3(ew_blocks(no)), dim3(256), 0, s, W_out, O, H, w.wout3);
-  launch_pdl(pack3_rows, dim3(ew_blocks(no)), dim3(256), 0, s, W_out, O, H, w.woutmn3);
+  launch_pdl(pack3_cols, dim3(ew_blocks(no)), dim3(256), 0, s, W_out, H, O, H, w.wout3);
+  launch_pdl(pack3_rows, dim3(ew_blocks(no)), dim3(256), 0, s, W_out, H, O, H, w.woutmn3);
+}
+
+void pack_input_weights(const Scratch& w, bool want_dx, int I, int H, int O, const float* W, const float* W_out, cudaStream_t s) {
+  const int G = 4 * H, K = I + H;
+  launch_pdl(pack3_cols, dim3(ew_blocks((size_t)G * I)), dim3(256), 0, s, W, K, G, I, w.w3);
+  if (want_dx) launch_pdl(pack3_rows, dim3(ew_blocks((size_t)G * I)), dim3(256), 0, s, W, K, G, I, w.wmn3);
+  const size_t no = (size_t)O * H;
+  launch_pdl(pack3_cols, dim3(ew_blocks(no)), dim3(256), 0, s, W_out, H, O, H, w.wout3);
+  launch_pdl(pack3_rows, dim3(ew_blocks(no)), dim3(256), 0, s, W_out, H, O, H, w.woutmn3);
+}
+
+int project_run(const Scratch& w, const float* x, int n, int I, int H, int B, const float* bias, float* zx, cudaStream_t s) {
+  const size_t ni = (size_t)n * B * I;
+  launch_pdl(split_a3, dim3(ew_blocks(ni)), dim3(256), 0, s, x, I, (const float*)nullptr, 0, n * B, w.a3_run);
+  return gemm_bf16(w.a3_run, 3 * I, false, w.w3, 3 * I, false, GemmOut{GemmOut::STORE_F32, zx, 4 * H, bias, 0}, n * B, 4 * H,
+                   3 * I, w.status, s);
+}
+
+// (split along K into the parts one step's product would take, so that all runs sum in one order)
+int input_gradient_run(const Scratch& w, int s_lo, int n, int I, int H, int B, float* dx, cudaStream_t s) {
+  const int G = 4 * H;
+  const int splits = tc::gemm_split_count(false, true, B, I, 3 * G, w.split.partial_floats);
+  return gemm_bf16(w.st_dz3 + (size_t)s_lo * B * 3 * G, 3 * G, false, w.wmn3, I, true, GemmOut{GemmOut::STORE_F32, dx, I, nullptr, 0},
+                   n * B, I, 3 * G, w.status, s, true, &w.split_run, splits);
 }
 
 int forward_step(const generic::FwdArgs& a, const Scratch& w, int l, size_t w_off, cudaStream_t s) {

@@ -75,26 +75,6 @@ __device__ __forceinline__ float tanh_fast(float x) {
   asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ bool wait_or_fail(uint64_t* bar, uint32_t parity, volatile int* failed) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (i > 256) {
-      if (*failed) return false;
-      __nanosleep(64);
-    }
-  }
-  *failed = 1;
-  return false;
-}
-__device__ __forceinline__ bool wait_counter(const uint32_t* ctr, uint32_t target, volatile int* failed,
-                                             uint32_t limit = kSpinLimit >> 1) {
-  for (uint32_t i = 0; i < limit; ++i) {
-    if (ld_acquire(ctr) >= target) return true;
-    if (i > 4096 && *failed) return false;
-  }
-  *failed = 1;
-  return false;
-}
 __device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
 

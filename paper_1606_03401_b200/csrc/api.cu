@@ -154,7 +154,6 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
     x3.st_dz3 = bf(y.off_st_dz); x3.st_in2 = bf(y.off_st_in); x3.st_hp2 = bf(y.off_st_hp);
     x3.st_dy3 = bf(y.off_st_dy); x3.st_h3 = bf(y.off_st_h);
     x3.split_run = tc::SplitWs{reinterpret_cast<float*>(ws + y.off_split), y.split_floats};
-    x3.dy_run = reinterpret_cast<float*>(ws + y.off_dy_run);
     x3.dha_run = reinterpret_cast<float*>(ws + y.off_dha_run);
     x3.loss_part = loss_part;
     x3.split_dh = reinterpret_cast<float*>(ws + y.off_split_dh);
@@ -269,30 +268,21 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
     std::vector<stepwise::BwdRunStep> bst((size_t)y.S);
     std::vector<const float*> h_top((size_t)y.S);
     float* zrun = reinterpret_cast<float*>(ws + y.off_zrun);
-    auto run = [&](const mebptt_op* ops, int n) {
-      if (ops[0].kind == MEBPTT_OP_FWD) {
-        for (int j = 0; j < n; ++j) {
-          const FwdPtrs q = fwd_ptrs(y, io, ops[j], 0);
-          fst[j] = stepwise::FwdRunStep{q.h_prev, q.c_prev, q.h_out, q.c_out, q.gates, q.h_in_copy, q.c_in_copy};
-        }
-        const float* x = reinterpret_cast<const float*>(io.x) + (size_t)(ops[0].k - 1) * y.B * y.I;
-        rc = stepwise3::project_run(x3, x, n, y.I, y.H, y.B, io.b, zrun, s);
-        if (rc == MEBPTT_OK) rc = stepwise3::forward_run(runs, fst.data(), n, zrun, plane_elems, io.counters, status, s);
-        return;
-      }
-      const int64_t k_lo = ops[n - 1].k;
+    float* zleaf = reinterpret_cast<float*>(ws + y.off_zleaf3);
+    float* products = reinterpret_cast<float*>(ws + y.off_leaf);
+    float* leaves = products + (size_t)stepwise3::X3_LEAVES * y.B * 16 * y.H;
+    const float* x = reinterpret_cast<const float*>(io.x);
+    const int parts = (y.B / 32) * ((y.O + 31) / 32);
+    // readout, backward run and what follows it; bst and h_top are filled in
+    auto backward = [&](int64_t k_lo, int n) {
       const int s_lo = (int)((k_lo - 1) % y.S);
-      for (int i = 0; i < n; ++i) {
-        const BwdPtrs q = bwd_ptrs(y, io, ops[i], 0);
-        bst[i] = stepwise::BwdRunStep{q.gates, q.c_t, q.c_prev, q.in, q.h_prev};
-        h_top[n - 1 - i] = reinterpret_cast<const float*>(loc_base(y, ws, ops[i].src) + y.h_off(0));
-      }
-      rc = stepwise3::readout_run(h_top.data(), n, s_lo, io.b_out, io.targets + (size_t)(k_lo - 1) * y.B * y.O,
-                                  loss_t + (k_lo - 1), y.B, y.H, y.O, x3, s);
       const size_t row = (size_t)s_lo * y.B;
+      rc = stepwise3::readout_run(h_top.data(), n, s_lo, io.b_out, io.targets + (size_t)(k_lo - 1) * y.B * y.O, nullptr, y.B, y.H,
+                                  y.O, x3, s);
       if (rc == MEBPTT_OK)
         rc = stepwise3::backward_run(runs, bst.data(), n, x3.dha_run, dh_rec, dc_rec, x3.st_dz3 + row * 12 * y.H,
-                                     x3.st_hp2 + row * 2 * y.H, x3.st_in2 + row * 2 * y.I, plane_elems, io.counters, status, s);
+                                     x3.st_hp2 + row * 2 * y.H, x3.st_in2 + row * 2 * y.I, plane_elems, x3.loss_part, parts,
+                                     loss_t + (k_lo - 1), io.counters, status, s);
       if (rc == MEBPTT_OK && desc->want_dx)
         rc = stepwise3::input_gradient_run(x3, s_lo, n, y.I, y.H, y.B, io.dx + (size_t)(k_lo - 1) * y.B * y.I, s);
       if (rc == MEBPTT_OK && s_lo == 0) {
@@ -301,10 +291,62 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
         rc = stepwise3::flush_chunk(x3, steps, 1, y.B, y.I, y.H, y.O, w_off, io.dW, io.dW_out, io.db, io.db_out, s);
       }
     };
-    for (const WorkItem& wi : work_items(p, y.S)) {
-      const bool single = wi.kind == WorkItem::LEAF || per_op_only;
-      const int ops = wi.kind == WorkItem::LEAF ? 2 * wi.n : wi.n;
-      for (int j = 0; j < ops && rc == MEBPTT_OK; j += single ? 1 : ops) run(p->tape.data() + wi.i + j, single ? 1 : ops);
+    const std::vector<WorkItem> items = work_items(p, y.S);
+    const std::vector<int> windows = projection_windows(items, p, y.S, y.t);
+    int64_t zx_lo = 0;
+    for (size_t item = 0; item < items.size() && rc == MEBPTT_OK; ++item) {
+      const WorkItem& wi = items[item];
+      const mebptt_op* ops = p->tape.data() + wi.i;
+      if (wi.kind == WorkItem::FWD) {
+        const int64_t k0 = ops[0].k;
+        if (windows[item]) {
+          zx_lo = k0;
+          rc = stepwise3::project_run(x3, x + (size_t)(k0 - 1) * y.B * y.I, windows[item] - (int)k0, y.I, y.H, y.B, io.b, zrun, s);
+        }
+        for (int j = 0; j < wi.n; ++j) {
+          const FwdPtrs q = fwd_ptrs(y, io, ops[j], 0);
+          fst[j] = stepwise::FwdRunStep{q.h_prev, q.c_prev, q.h_out, q.c_out, q.gates, q.h_in_copy, q.c_in_copy};
+        }
+        const float* zx = zrun + (size_t)(k0 - zx_lo) * y.B * 4 * y.H;
+        const int step = per_op_only ? 1 : wi.n;
+        for (int j = 0; j < wi.n && rc == MEBPTT_OK; j += step)
+          rc = stepwise3::forward_run(runs, fst.data() + j, step, zx + (size_t)j * y.B * 4 * y.H, plane_elems, io.counters, status, s);
+      } else if (wi.kind == WorkItem::BWD) {
+        const int step = per_op_only ? 1 : wi.n;
+        for (int j = 0; j < wi.n && rc == MEBPTT_OK; j += step) {
+          for (int i = 0; i < step; ++i) {
+            const BwdPtrs q = bwd_ptrs(y, io, ops[j + i], 0);
+            bst[i] = stepwise::BwdRunStep{q.gates, q.c_t, q.c_prev, q.in, q.h_prev};
+            h_top[step - 1 - i] = reinterpret_cast<const float*>(loc_base(y, ws, ops[j + i].src) + y.h_off(0));
+          }
+          backward(ops[j + step - 1].k, step);
+        }
+      } else {
+        // leaves, as many at a time as there is room for: their forward operations all start from memorised states
+        const float *h_prev[stepwise3::X3_LEAVES], *c_prev[stepwise3::X3_LEAVES];
+        const int most = per_op_only ? 1 : stepwise3::X3_LEAVES;
+        for (int done = 0; done < wi.n && rc == MEBPTT_OK;) {
+          const int n = wi.n - done < most ? wi.n - done : most;
+          const int64_t k_lo = ops[2 * (done + n - 1)].k;
+          for (int i = 0; i < n; ++i) {   // leaf i has step k_lo + n - 1 - i
+            const mebptt_op& f = ops[2 * (done + i)];
+            const FwdPtrs q = fwd_ptrs(y, io, f, 0);
+            const int a = n - 1 - i;
+            h_prev[a] = (const float*)q.h_prev; c_prev[a] = q.c_prev;
+            const float* o = leaves + (size_t)a * 6 * plane_elems;
+            bst[i] = stepwise::BwdRunStep{o, o + 4 * plane_elems, q.c_prev, x + (size_t)(f.k - 1) * y.B * y.I, q.h_prev};
+            h_top[a] = o + 5 * plane_elems;
+          }
+          const int s_lo = (int)((k_lo - 1) % y.S);
+          rc = stepwise3::project_run(x3, x + (size_t)(k_lo - 1) * y.B * y.I, n, y.I, y.H, y.B, io.b, zleaf, s);
+          if (rc != MEBPTT_OK) break;
+          stepwise3::split_states(x3, h_prev, n, s_lo, y.H, y.B, s);
+          rc = stepwise3::forward_leaves(runs, x3.st_hp2 + (size_t)s_lo * y.B * 2 * y.H, c_prev, n, zleaf, products, leaves,
+                                         plane_elems, io.counters, status, s);
+          if (rc == MEBPTT_OK) backward(k_lo, n);
+          done += n;
+        }
+      }
     }
   } else if (!(y.stepwise_tc || y.stepwise_x3) || per_op_only) {
     for (const mebptt_op& op : p->tape) {
@@ -574,7 +616,7 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
   }
   if (y.stepwise_x3) {
     // weights: 2 packing kernels per layer and 2 for the readout; forward operation: split, GEMM,
-    // cell per layer; readout: split, GEMM, loss sum, split, dha GEMM; backward operation per
+    // cell per layer; readout: split, GEMM, loss sum, dha GEMM; backward operation per
     // layer: gate kernel, one or two d_in GEMMs; a chunk: 3 GEMMs per product and L + 1 bias sums
     const size_t pf = (size_t)148 * 128 * 128;
     const int G = 4 * y.H;
@@ -584,11 +626,16 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
     const int64_t bwd = L + L + to_h * (L - 1) + (desc->want_dx ? to_x : 0);   // dh = dz W_hh: one launch in any case
     const int64_t chunks = (p->t + y.S - 1) / y.S;
     if (y.x3_runs) {
-      // packing; forward run: split, projection, run; backward run: readout, run, d_in; chunks as below
+      // packing; a window of projections: split and GEMM; forward run: one; backward run: readout of two
+      // and dha, run, d_in; a batch of leaves: split, GEMM, states, two GEMMs, cells before that; chunks as below
       int64_t n = 5 + (desc->want_dx ? 1 : 0) + chunks * 11 + 1;
-      for (const WorkItem& wi : work_items(p, y.S)) {
-        const int64_t f = wi.kind == WorkItem::LEAF ? wi.n : wi.kind == WorkItem::FWD, b = wi.kind == WorkItem::LEAF ? wi.n : wi.kind == WorkItem::BWD;
-        n += 3 * f + (5 + dha + (desc->want_dx ? to_x : 0)) * b;
+      const std::vector<WorkItem> items = work_items(p, y.S);
+      const std::vector<int> windows = projection_windows(items, p, y.S, y.t);
+      const int64_t back = 3 + dha + (desc->want_dx ? to_x : 0);
+      for (size_t i = 0; i < items.size(); ++i) {
+        if (items[i].kind == WorkItem::FWD) n += 1 + (windows[i] ? 2 : 0);
+        else if (items[i].kind == WorkItem::BWD) n += back;
+        else n += (items[i].n + stepwise3::X3_LEAVES - 1) / stepwise3::X3_LEAVES * (6 + back);
       }
       return n;
     }
@@ -597,8 +644,8 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
     // GEMM and cell kernel per step)
     int64_t readouts = 0, forwards = 0;
     for (const WorkItem& wi : work_items(p, y.S)) {
-      if (wi.kind == WorkItem::LEAF) { readouts += wi.n * (4 + dha); forwards += wi.n * 3 * L; }
-      else if (wi.kind == WorkItem::BWD) readouts += 4 + dha;
+      if (wi.kind == WorkItem::LEAF) { readouts += wi.n * (3 + dha); forwards += wi.n * 3 * L; }
+      else if (wi.kind == WorkItem::BWD) readouts += 3 + dha;
       else forwards += wi.n == 1 ? 3 * L : L * (1 + 2 * (int64_t)wi.n);
     }
     return 2 * L + 2 + forwards + readouts + p->t * bwd + chunks * (3 * (2 * L + 1) + L + 1) + 1;

@@ -163,7 +163,6 @@ struct Scratch {
   __nv_bfloat16* st_dy3;     // [S B][3 O]
   __nv_bfloat16* st_h3;      // [S B][3 H]  top layer h_k
   // the readout of a run of up to S backward operations at once
-  float* dy_run;             // [S B][O]
   float* dha_run;            // [S B][H]  gradient entering the top layer at each step of the run
   float* loss_part;          // partial sums of the loss terms, per step
   float* split_dh;           // as on the bfloat16 path: per-layer split-K scratch of dh = dz W_hh,
@@ -180,7 +179,7 @@ int readout(const generic::ReadoutArgs& a, const Scratch& w, int sidx, cudaStrea
 int backward_layer(const generic::BwdArgs& a, const Scratch& w, int l, size_t w_off, int sidx, cudaStream_t s);
 // Readout, loss terms, dy and the gradient entering the top layer (-> w.dha_run, row block a for
 // step s_lo + a) of n steps at once; h_top[a]: the top layer's h of step s_lo + a; target, loss_t:
-// those of the first of the steps.
+// those of the first of the steps; loss_t NULL: the loss terms stay in w.loss_part.
 int readout_run(const float* const* h_top, int n, int s_lo, const float* b_out, const float* target, float* loss_t,
                 int B, int H, int O, const Scratch& w, cudaStream_t s);
 int flush_chunk(const Scratch& w, int steps, int L, int B, int I0, int H, int O, const size_t* w_off, float* dW,
@@ -210,10 +209,19 @@ int forward_run(RunsX3& r, const stepwise::FwdRunStep* st, int n, const float* z
 // n <= 32 backward operations, time descending; dha: [n][B][H] in ascending time, the stages likewise
 // from the run's first step in time.
 int backward_run(RunsX3& r, const stepwise::BwdRunStep* st, int n, const float* dha, float* dh, float* dc, __nv_bfloat16* st_dz3,
-                 __nv_bfloat16* st_hp2, __nv_bfloat16* st_in2, size_t plane_elems, int64_t* counters, int* status, cudaStream_t s);
+                 __nv_bfloat16* st_hp2, __nv_bfloat16* st_in2, size_t plane_elems, const float* loss_part, int loss_parts,
+                 float* loss_t, int64_t* counters, int* status, cudaStream_t s);
+// The forward operations of n <= X3_LEAVES leaves at once (their h_{k-1}, c_{k-1} are all memorised): hp2 [n B][2H]
+// holds the halves of h_{k-1}, zx as above, both in ascending time; z: scratch for 2 n B 8H floats.  State
+// and gates of leaf a go to out + 6 a plane_elems: four gate planes, c, h.
+constexpr int X3_LEAVES = 8;
+int forward_leaves(RunsX3& r, const __nv_bfloat16* hp2, const float* const* c_prev, int n, const float* zx, float* z, float* out,
+                   size_t plane_elems, int64_t* counters, int* status, cudaStream_t s);
 // The input products of a run on that path.  wih3: [4H][3I] and, for the gradient of the inputs, wmn3: [3 * 4H][I].
 void pack_input_weights(const Scratch& w, bool want_dx, int I, int H, int O, const float* W, const float* W_out, cudaStream_t s);
 int project_run(const Scratch& w, const float* x, int n, int I, int H, int B, const float* bias, float* zx, cudaStream_t s);
+// Halves of n states h[a] into the stage of h_{k-1}, from row block s_lo on.
+void split_states(const Scratch& w, const float* const* h, int n, int s_lo, int H, int B, cudaStream_t s);
 int input_gradient_run(const Scratch& w, int s_lo, int n, int I, int H, int B, float* dx, cudaStream_t s);
 }  // namespace stepwise3
 }  // namespace mebptt

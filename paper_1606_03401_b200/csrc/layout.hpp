@@ -65,7 +65,7 @@ struct Layout {
   size_t off_zx = 0, off_zleaf = 0, off_hprev = 0, off_hk = 0, off_y = 0;
   size_t off_sync = 0, off_tape = 0, off_status = 0, off_split_dh = 0;
   size_t off_w_f = 0, off_w_b = 0, off_exch_f = 0, off_exch_b = 0;
-  size_t off_a3_run = 0, off_zrun = 0, off_hrun = 0, off_dha_run = 0, off_dy_run = 0, split_floats = 0;
+  size_t off_a3_run = 0, off_zrun = 0, off_hrun = 0, off_dha_run = 0, off_zleaf3 = 0, off_leaf = 0, split_floats = 0;
   size_t n_sync = 0, tape_bytes = 0;
   // team path: states per group of batch rows, in blocks of one layer's h of the group (a cell state takes
   // 4 / esz of them): blocks of a location's unit, of a hidden state, of all states; first blocks of the named states
@@ -232,6 +232,34 @@ inline std::vector<WorkItem> work_items(const Plan* p, int S) {
   return items;
 }
 
+// Input projections are computed for the S steps from the start of a forward run on, unless the buffer
+// already holds them: recomputation sweeps keep returning to the same stored state, so one projection
+// serves many short runs.  (The values do not depend on how steps are batched.)  The tape is known, so
+// a window ends where the last run that will still find its steps in it ends (the first forward run
+// that does not fit in the S steps from the window's start on replaces it).  Per item: the end of the
+// window that it opens, 0 if it finds its steps in place.
+inline std::vector<int> projection_windows(const std::vector<WorkItem>& items, const Plan* p, int S, int64_t t) {
+  std::vector<int> ends(items.size(), 0);
+  int lo = 0, hi = 0;
+  for (size_t item = 0; item < items.size(); ++item) {
+    const WorkItem& wi = items[item];
+    if (wi.kind != WorkItem::FWD) continue;
+    const int k0 = p->tape[wi.i].k, n = wi.n;
+    if (k0 >= lo && k0 + n <= hi) continue;
+    lo = k0;
+    const int cap = (int)((int64_t)k0 + S <= t + 1 ? k0 + S : t + 1);
+    hi = k0 + n;
+    for (size_t j = item + 1; j < items.size(); ++j) {
+      if (items[j].kind != WorkItem::FWD) continue;
+      const int kj = p->tape[items[j].i].k, ej = kj + items[j].n;
+      if (kj < k0 || ej > cap) break;
+      if (ej > hi) hi = ej;
+    }
+    ends[item] = hi;
+  }
+  return ends;
+}
+
 // compact: the least working memory, for callers that bring a fixed amount (the team path's stages and
 // packed weights are then done without)
 inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y, bool compact = false) {
@@ -337,6 +365,9 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
       if (y.x3_runs) {
         const size_t hp = align_up(y.H, 64), groups = (size_t)y.B / 32;
         y.off_zrun = take(rows * G * 4);
+        // a batch of leaves: input projections, products, states with their gates
+        y.off_zleaf3 = take((size_t)8 * y.B * G * 4);
+        y.off_leaf = take((size_t)8 * y.B * 16 * y.H * 4 + 8 * 6 * y.plane);
         y.off_w_f = take((size_t)8 * y.H * hp * 2);
         y.off_w_b = take(align_up(y.H, 32) * 8 * hp * 2);
         y.off_exch_f = take(2 * groups * 64 * hp * 2);
@@ -344,7 +375,6 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
         y.n_sync = 64 * (p->tape.size() + 1);   // two lines a launch, at most an operation each
         y.off_sync = take(y.n_sync * 4);
       }
-      y.off_dy_run = take(rows * y.O * 4);
       y.off_dha_run = take(rows * y.H * 4);
       y.split_floats = (size_t)148 * 128 * 128 * ((rows + 127) / 128);
       y.off_split = take(y.split_floats * 4);

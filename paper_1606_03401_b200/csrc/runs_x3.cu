@@ -91,6 +91,9 @@ struct BwdX3Args {
   int* status;
   int64_t* counters;
   size_t plane;
+  const float* loss_part; // [n][loss_parts] in ascending time, and where the loss terms go
+  float* loss_t;
+  int loss_parts;
   int n, B, H, HP, I, ncg, groups;
   uint32_t expect, poll_limit;
 };
@@ -415,6 +418,11 @@ __global__ void __launch_bounds__(192, 1) bwd_run_x3(const __grid_constant__ CUt
       }
       named_barrier(1, 128);   // this CTA's derivatives precede the release
       if (tid == 0) red_release_add(sync, 1u);
+      if (i == 0 && blockIdx.x == 0 && tid < a.n) {   // loss terms, their parts in a fixed order
+        float sum = 0.f;
+        for (int p = 0; p < a.loss_parts; ++p) sum += a.loss_part[tid * a.loss_parts + p];
+        a.loss_t[tid] = sum;
+      }
       // off the recurrence: the next operation's inputs, the stages of the weight gradients
       const int blk = a.n - 1 - i;   // row block of the stages, from the run's first step in time
       if (owner) {
@@ -495,6 +503,36 @@ __global__ void pack_runs_bwd(const float* W, int K, int I, int H, int HP, bf16*
   }
 }
 
+// The cells of a batch of leaves from the products of their h_{k-1}: z1 = h_hi W_f, z2 = h_mid W_f over the rows
+// of w_f, summed as the forward kernel sums them.
+struct LeafPtrs { const float* c_prev[X3_LEAVES]; };
+__global__ void leaf_cells(const LeafPtrs src, const float* zx, const float* z1, const float* z2, float* out, size_t plane, int B, int H,
+                           int64_t* counters) {
+  grid_dep_wait();
+  grid_dep_launch();
+  const int leaf = blockIdx.y;
+  const float* cpv = src.c_prev[leaf];
+  float* o = out + (size_t)leaf * 6 * plane;
+  const size_t n = (size_t)B * H;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const int b = (int)(e / H), j = (int)(e % H);
+    const size_t row = (size_t)leaf * B + b;
+    const size_t at = row * 8 * H + (size_t)(j / RU) * 64 + 4 * (j % RU);
+    const float4 hh = *reinterpret_cast<const float4*>(z1 + at), mh = *reinterpret_cast<const float4*>(z1 + at + 32);
+    const float4 hm = *reinterpret_cast<const float4*>(z2 + at);
+    const float* zr = zx + row * 4 * H + j;
+    const float gi = sigmoidf_(zr[0] + ((hh.x + hm.x) + mh.x));
+    const float gf = sigmoidf_(zr[H] + ((hh.y + hm.y) + mh.y));
+    const float gg = tanhf(zr[2 * (size_t)H] + ((hh.z + hm.z) + mh.z));
+    const float go = sigmoidf_(zr[3 * (size_t)H] + ((hh.w + hm.w) + mh.w));
+    const float c = fmaf(gf, cpv[e], gi * gg);
+    o[e] = gi; o[plane + e] = gf; o[2 * plane + e] = gg; o[3 * plane + e] = go;
+    o[4 * plane + e] = c;
+    o[5 * plane + e] = go * tanhf(c);
+  }
+  if (blockIdx.x == 0 && leaf == 0 && threadIdx.x == 0) counters[0] += gridDim.y;
+}
+
 inline int round64(int v) { return (v + 63) / 64 * 64; }
 
 }  // namespace
@@ -534,8 +572,10 @@ int forward_run(RunsX3& r, const stepwise::FwdRunStep* st, int n, const float* z
 }
 
 int backward_run(RunsX3& r, const stepwise::BwdRunStep* st, int n, const float* dha, float* dh, float* dc, __nv_bfloat16* st_dz3,
-                 __nv_bfloat16* st_hp2, __nv_bfloat16* st_in2, size_t plane_elems, int64_t* counters, int* status, cudaStream_t s) {
+                 __nv_bfloat16* st_hp2, __nv_bfloat16* st_in2, size_t plane_elems, const float* loss_part, int loss_parts, float* loss_t,
+                 int64_t* counters, int* status, cudaStream_t s) {
   BwdX3Args a{};
+  a.loss_part = loss_part; a.loss_parts = loss_parts; a.loss_t = loss_t;
   for (int i = 0; i < n; ++i) a.op[i] = st[i];
   const int fault = tc::wait_fault_mask();
   a.dha = dha; a.dh = dh; a.dc = dc; a.exch = r.exch_b; a.st_dz3 = st_dz3; a.st_hp2 = st_hp2; a.st_in2 = st_in2;
@@ -548,6 +588,26 @@ int backward_run(RunsX3& r, const stepwise::BwdRunStep* st, int n, const float* 
   void* args[] = {(void*)&r.tm_dz, (void*)&r.tm_wt, (void*)&a};
   return launch_coop((const void*)bwd_run_x3, r.groups * a.ncg, 192, bwd_smem(r.HP / 64), s, args, CS, false) == cudaSuccess
              ? MEBPTT_OK : MEBPTT_ERR_CUDA;
+}
+
+// A leaf on its own is a launch of a persistent kernel each way, a readout and a projection (H = 1000, B = 32:
+// some 80 us); batched, the forward operations are two products and a cell kernel, and the readout and the
+// backward operations of up to X3_LEAVES leaves are one run (150 steps at full memory: 12.2 -> 4.4 ms).
+int forward_leaves(RunsX3& r, const __nv_bfloat16* hp2, const float* const* c_prev, int n, const float* zx, float* z, float* out,
+                   size_t plane_elems, int64_t* counters, int* status, cudaStream_t s) {
+  const int M = n * r.B, N = 8 * r.H;
+  float* z2 = z + (size_t)M * N;
+  for (int half = 0; half < 2; ++half) {
+    const int rc = gemm_bf16(hp2 + (size_t)half * r.H, 2 * r.H, false, r.w_f, r.HP, false,
+                             GemmOut{GemmOut::STORE_F32, half ? z2 : z, N, nullptr, 0}, M, N, r.H, status, s);
+    if (rc != MEBPTT_OK) return rc;
+  }
+  LeafPtrs ptrs{};
+  for (int a = 0; a < n; ++a) ptrs.c_prev[a] = c_prev[a];
+  const size_t blocks = ((size_t)r.B * r.H + 255) / 256;
+  launch_pdl(leaf_cells, dim3((unsigned)(blocks > 128 ? 128 : blocks), (unsigned)n), dim3(256), 0, s, ptrs, zx, (const float*)z,
+             (const float*)z2, out, plane_elems, r.B, r.H, counters);
+  return MEBPTT_OK;
 }
 
 }  // namespace stepwise3

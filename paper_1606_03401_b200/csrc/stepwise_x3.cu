@@ -12,8 +12,8 @@
 //
 // Operations (per layer), with K = I + H, G = 4H:
 //   forward    a3 = split([in ; h_prev]) ; z = a3 W3^T + b ; gates, c, h from z
-//   readout    h3 = split(h) ; y = h3 Wout3^T + b_out with loss and dy (float32) in the epilogue ;
-//              dy3 = split(dy) ; dha = dy3 WoutMN3
+//   readout    h3 = split(h) ; y = h3 Wout3^T + b_out with loss and the halves of dy in the epilogue ;
+//              dha = dy3 WoutMN3
 //   backward   dz3 from the stored gates ; d_in = dz3 WMN3
 //   per chunk  dW += dz^T [in ; h_prev], dW_out += dy^T h from the staged halves: three GEMMs per
 //              product (hi hi, hi mid, mid hi); db += sum of dz, db_out += sum of dy, as hi + mid
@@ -102,6 +102,23 @@ __global__ void split_blocks3(RunPtrs src, int C, int B, bf16* out) {
     split2(a[e], hi, mid);
     bf16* o = dst + r * 3 * (size_t)C + c;
     o[0] = hi; o[C] = hi; o[2 * (size_t)C] = mid;
+  }
+}
+
+// The halves [hi | mid] of up to 64 row blocks of [B][C] that lie apart.
+__global__ void split_blocks2(RunPtrs src, int C, int B, bf16* out) {
+  sm100::grid_dep_wait();
+  sm100::grid_dep_launch();
+  const float* a = src.p[blockIdx.y];
+  bf16* dst = out + (size_t)blockIdx.y * B * 2 * C;
+  const size_t n = (size_t)B * C;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const size_t r = e / C;
+    const int c = (int)(e % C);
+    bf16 hi, mid;
+    split2(a[e], hi, mid);
+    dst[r * 2 * C + c] = hi;
+    dst[r * 2 * C + C + c] = mid;
   }
 }
 
@@ -300,6 +317,13 @@ int project_run(const Scratch& w, const float* x, int n, int I, int H, int B, co
                    3 * I, w.status, s);
 }
 
+void split_states(const Scratch& w, const float* const* h, int n, int s_lo, int H, int B, cudaStream_t s) {
+  RunPtrs ptrs{};
+  for (int a = 0; a < n; ++a) ptrs.p[a] = h[a];
+  const int blocks = ew_blocks((size_t)B * H);
+  launch_pdl(split_blocks2, dim3(blocks > 64 ? 64 : blocks, n), dim3(256), 0, s, ptrs, H, B, w.st_hp2 + (size_t)s_lo * B * 2 * H);
+}
+
 // (split along K into the parts one step's product would take, so that all runs sum in one order)
 int input_gradient_run(const Scratch& w, int s_lo, int n, int I, int H, int B, float* dx, cudaStream_t s) {
   const int G = 4 * H;
@@ -358,18 +382,17 @@ int forward_run_layer(const stepwise::FwdRunStep* st, int n, const float* in, in
 int readout(const generic::ReadoutArgs& a, const Scratch& w, int sidx, cudaStream_t s) {
   bf16* h3 = w.st_h3 + (size_t)sidx * a.B * 3 * a.H;
   bf16* dy3 = w.st_dy3 + (size_t)sidx * a.B * 3 * a.O;
-  const size_t nh = (size_t)a.B * a.H, no = (size_t)a.B * a.O;
+  const size_t nh = (size_t)a.B * a.H;
   launch_pdl(split_a3, dim3(ew_blocks(nh)), dim3(256), 0, s, (const float*)a.h, a.H, nullptr, 0, a.B, h3);
   GemmOut o{GemmOut::LOSS_DY, nullptr, a.O, a.b_out, 0};
   o.target = a.target;
-  o.dy32 = a.dy;
+  o.dy3 = dy3;
   o.loss_part = a.loss_part;
   o.parts = (a.O + 31) / 32;
   o.scale = 1.f / ((float)a.B * (float)a.O);
   int rc = gemm_bf16(h3, 3 * a.H, false, w.wout3, 3 * a.H, false, o, a.B, a.O, 3 * a.H, w.status, s);
   if (rc != MEBPTT_OK) return rc;
   launch_pdl(sum_parts, dim3(1), dim3(32), 0, s, a.loss_part, (a.B / 32) * o.parts, a.loss_k);
-  launch_pdl(split_a3, dim3(ew_blocks(no)), dim3(256), 0, s, a.dy, a.O, nullptr, 0, a.B, dy3);
   // dha[b][j] = sum_o dy[b][o] W_out[o][j]
   return gemm_bf16(dy3, 3 * a.O, false, w.woutmn3, a.H, true, GemmOut{GemmOut::STORE_F32, a.dha, a.H, nullptr, 0}, a.B,
                    a.H, 3 * a.O, w.status, s, true, &w.split);
@@ -382,21 +405,20 @@ int readout_run(const float* const* h_top, int n, int s_lo, const float* b_out, 
                 int B, int H, int O, const Scratch& w, cudaStream_t s) {
   bf16* h3 = w.st_h3 + (size_t)s_lo * B * 3 * H;
   bf16* dy3 = w.st_dy3 + (size_t)s_lo * B * 3 * O;
-  const size_t nh = (size_t)B * H, no = (size_t)n * B * O;
+  const size_t nh = (size_t)B * H;
   RunPtrs ptrs{};
   for (int a = 0; a < n; ++a) ptrs.p[a] = h_top[a];
   launch_pdl(split_blocks3, dim3(ew_blocks(nh) > 64 ? 64 : ew_blocks(nh), n), dim3(256), 0, s, ptrs, H, B, h3);
   const int parts = (O + 31) / 32, per_step = (B / 32) * parts;
   GemmOut o{GemmOut::LOSS_DY, nullptr, O, b_out, 0};
   o.target = target;
-  o.dy32 = w.dy_run;
+  o.dy3 = dy3;
   o.loss_part = w.loss_part;
   o.parts = parts;
   o.scale = 1.f / ((float)B * (float)O);
   int rc = gemm_bf16(h3, 3 * H, false, w.wout3, 3 * H, false, o, n * B, O, 3 * H, w.status, s);
   if (rc != MEBPTT_OK) return rc;
-  launch_pdl(sum_parts_steps, dim3((n + 31) / 32), dim3(32), 0, s, (const float*)w.loss_part, per_step, n, loss_t);
-  launch_pdl(split_a3, dim3(ew_blocks(no)), dim3(256), 0, s, (const float*)w.dy_run, O, (const float*)nullptr, 0, n * B, dy3);
+  if (loss_t) launch_pdl(sum_parts_steps, dim3((n + 31) / 32), dim3(32), 0, s, (const float*)w.loss_part, per_step, n, loss_t);
   const int splits = tc::gemm_split_count(false, true, B, H, 3 * O, w.split.partial_floats);
   return gemm_bf16(dy3, 3 * O, false, w.woutmn3, H, true, GemmOut{GemmOut::STORE_F32, w.dha_run, H, nullptr, 0}, n * B, H,
                    3 * O, w.status, s, true, &w.split_run, splits);

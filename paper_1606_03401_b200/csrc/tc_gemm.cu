@@ -233,13 +233,13 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ 
           const float* tp = out.target + (size_t)row * out.ld + col0;
           __nv_bfloat16* dp = reinterpret_cast<__nv_bfloat16*>(out.ptr) + (size_t)row * out.ld + col0;
           const float two = 2.f * out.scale;
-          float* d32 = out.dy32 ? out.dy32 + (size_t)row * out.ld + col0 : nullptr;
+          __nv_bfloat16* d3 = out.dy3 ? reinterpret_cast<__nv_bfloat16*>(out.dy3) + (size_t)row * 3 * out.ld + col0 : nullptr;
           if (col0 + 32 <= N && ((reinterpret_cast<uintptr_t>(tp) & 15) == 0) && ((reinterpret_cast<uintptr_t>(dp) & 15) == 0) &&
-              ((reinterpret_cast<uintptr_t>(out.bias) & 15) == 0) && ((reinterpret_cast<uintptr_t>(d32) & 15) == 0)) {
+              ((reinterpret_cast<uintptr_t>(out.bias) & 15) == 0) && ((reinterpret_cast<uintptr_t>(d3) & 15) == 0) && out.ld % 8 == 0) {
             float4 t4[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) t4[j] = *reinterpret_cast<const float4*>(tp + 4 * j);
-            uint32_t packed[16];
+            uint32_t packed[16], rest[16];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -247,11 +247,24 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ 
               const float d0 = (__uint_as_float(r[4 * j]) + bv.x) - t4[j].x;
               const float d1 = (__uint_as_float(r[4 * j + 1]) + bv.y) - t4[j].y;
               const float d2 = (__uint_as_float(r[4 * j + 2]) + bv.z) - t4[j].z;
-              const float d3 = (__uint_as_float(r[4 * j + 3]) + bv.w) - t4[j].w;
-              sq = fmaf(d0, d0, sq); sq = fmaf(d1, d1, sq); sq = fmaf(d2, d2, sq); sq = fmaf(d3, d3, sq);
+              const float dd = (__uint_as_float(r[4 * j + 3]) + bv.w) - t4[j].w;
+              sq = fmaf(d0, d0, sq); sq = fmaf(d1, d1, sq); sq = fmaf(d2, d2, sq); sq = fmaf(dd, dd, sq);
               packed[2 * j] = pack_bf16x2(d0 * two, d1 * two);
-              packed[2 * j + 1] = pack_bf16x2(d2 * two, d3 * two);
-              if (d32) *reinterpret_cast<float4*>(d32 + 4 * j) = make_float4(d0 * two, d1 * two, d2 * two, d3 * two);
+              packed[2 * j + 1] = pack_bf16x2(d2 * two, dd * two);
+              if (d3) {
+                const float2 h0 = unpack_bf16x2(packed[2 * j]), h1 = unpack_bf16x2(packed[2 * j + 1]);
+                rest[2 * j] = pack_bf16x2(d0 * two - h0.x, d1 * two - h0.y);
+                rest[2 * j + 1] = pack_bf16x2(d2 * two - h1.x, dd * two - h1.y);
+              }
+            }
+            if (d3) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const uint4 hi = make_uint4(packed[4 * j], packed[4 * j + 1], packed[4 * j + 2], packed[4 * j + 3]);
+                *reinterpret_cast<uint4*>(d3 + 8 * j) = hi;
+                *reinterpret_cast<uint4*>(d3 + out.ld + 8 * j) = hi;
+                *reinterpret_cast<uint4*>(d3 + 2 * out.ld + 8 * j) = make_uint4(rest[4 * j], rest[4 * j + 1], rest[4 * j + 2], rest[4 * j + 3]);
+              }
             }
             if (out.ptr) {
 #pragma unroll
@@ -265,7 +278,12 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ 
                 const float d = (__uint_as_float(r[j]) + (out.bias ? out.bias[col0 + j] : 0.f)) - tp[j];
                 sq = fmaf(d, d, sq);
                 if (out.ptr) dp[j] = __float2bfloat16_rn(d * two);
-                if (d32) d32[j] = d * two;
+                if (d3) {
+                  const __nv_bfloat16 hi = __float2bfloat16_rn(d * two);
+                  d3[j] = hi;
+                  d3[out.ld + j] = hi;
+                  d3[2 * out.ld + j] = __float2bfloat16_rn(d * two - __bfloat162float(hi));
+                }
               }
           }
         }

@@ -1694,29 +1694,7 @@ void build_host_part(Prepared& P, const Layout& y, const Plan* p, bool allow_pin
   const int S = y.S;
   const size_t nops = p->tape.size();
   P.items = work_items(p, S);
-  // Input projections Zx: computed for the S steps from the start of a forward run on, unless the
-  // buffer already holds them: recomputation sweeps keep returning to the same stored state, so one
-  // projection serves many short runs.  (The values do not depend on how steps are batched.)  The
-  // tape is known, so the window ends where the last run that will still find its steps in it ends
-  // (the first forward run that does not fit in the S steps from the window's start on replaces it).
-  P.zx_hi.assign(P.items.size(), 0);
-  int zx_lo = 0, zx_hi = 0;
-  for (size_t item = 0; item < P.items.size(); ++item) {
-    const WorkItem& wi = P.items[item];
-    if (wi.kind != WorkItem::FWD) continue;
-    const int k0 = p->tape[wi.i].k, n = wi.n;
-    if (k0 >= zx_lo && k0 + n <= zx_hi) continue;
-    zx_lo = k0;
-    const int cap = (int)((int64_t)k0 + S <= y.t + 1 ? k0 + S : y.t + 1);
-    zx_hi = k0 + n;
-    for (size_t j = item + 1; j < P.items.size(); ++j) {
-      if (P.items[j].kind != WorkItem::FWD) continue;
-      const int kj = p->tape[P.items[j].i].k, ej = kj + P.items[j].n;
-      if (kj < k0 || ej > cap) break;
-      if (ej > zx_hi) zx_hi = ej;
-    }
-    P.zx_hi[item] = zx_hi;
-  }
+  P.zx_hi = projection_windows(P.items, p, S, y.t);
   P.zx_next.assign(P.items.size(), -1);
   for (int item = (int)P.items.size() - 1, next = -1; item >= 0; --item)
     if (P.zx_hi[item]) { P.zx_next[item] = next; next = item; }

@@ -133,12 +133,16 @@ Config choose_config(const Layout& y, int sms) {
   return best;
 }
 
-// Shapes the step-by-step tensor-core kernels could take as well go to whichever is estimated faster:
-// they spend some 45 us a layer on two forward operations and a backward one whatever the widths (three
-// or four dependent launches each; measured from 160 to 1024 units), and stay ahead where the
-// recurrent weights are large.  (Asked for the layout, before a device is known: a B200 is assumed.)
+// Shapes other tensor-core kernels could take as well go to whichever is estimated faster, by the clock
+// cycles of two forward operations and a backward one.  Step by step these take some 45 us a layer
+// whatever the widths (three or four dependent launches each; measured from 160 to 1024 units), and stay
+// ahead where the recurrent weights are large.  The persistent kernels for float32 storage take some
+// 20 us and a launch or several a run: at H = 160, B = 32 (estimated 29600) both were within a
+// fifth of each other, at 224 units and 64 rows or 304 and 32 (43700 and up) those were 1.1 to 1.4 times
+// faster under every plan.  (Asked for the layout, before a device is known: a B200 is assumed.)
 bool supported(const mebptt_lstm_desc* d) {
-  constexpr double kStepwise = 70000.0;   // cycles; a fifth less than measured, to be worth leaving
+  constexpr double kStepwise = 70000.0;   // a fifth less than measured, to be worth leaving
+  constexpr double kRuns = 33000.0;
   Layout y;
   state_layout(d, y);
   if (y.tensor_path || y.L > kMaxLayers || y.t >= (1 << 30)) return false;
@@ -147,7 +151,8 @@ bool supported(const mebptt_lstm_desc* d) {
   const Config c = choose_config(y, 148);
   if (!pc.ok && !c.ok) return false;
   if (!y.stepwise_tc && !y.stepwise_x3) return true;
-  return (pc.ok && pc.cycles < kStepwise * y.L) || (c.ok && c.cycles < kStepwise * y.L);
+  const double least = y.x3_runs ? kRuns : kStepwise * y.L;
+  return (pc.ok && pc.cycles < least) || (c.ok && c.cycles < least);
 }
 
 namespace {

@@ -222,13 +222,13 @@ typedef struct {
   int64_t t;        /* sequence length; must equal the plan's         */
 } mebptt_lstm_desc;
 
-/* Run on the CUDA-core kernels even where the tensor-core kernels cover the shape (the two
- * paths round differently; results are deterministic within each). */
+/* Keep every contraction in float32 FMA on the CUDA cores even where the tensor-core kernels cover
+ * the shape (the paths round differently; results are deterministic within each). */
 enum { MEBPTT_FLAG_NO_TENSOR_CORES = 1 };
 /* Measurement aid: bracket every launch of the two persistent kernels of the tensor-core path
  * (forward runs, backward runs) with a pair of CUDA events on the caller's stream, to be
  * collected by mebptt_lstm_run_times.  Each pair costs a few microseconds of stream time, so a
- * step that is timed as a whole should not set it.  Ignored by the CUDA-core path. */
+ * step that is timed as a whole should not set it.  Ignored by the other paths. */
 enum { MEBPTT_FLAG_TIME_RUNS = 2 };
 /* The recurrent core is a GRU instead of an LSTM (Section 1: the method does not depend on the
  * architecture of the core; plans, tape, budgets and every entry point are the same):
@@ -237,7 +237,8 @@ enum { MEBPTT_FLAG_TIME_RUNS = 2 };
  * W is then [3H][I_l + H] per layer (row blocks r, z, n), b [3H], and so are dW, db.  The hidden
  * state is h alone: c0 is not read, and the cell-state part of a memory slot stays unused, so the
  * sizes of slots and the units of m are those of the LSTM layout (alpha = 4: h_t, the planes r, z,
- * n, q, and h_{t-1}).  Runs on the CUDA-core kernels in every precision (MEBPTT_TF32 = MEBPTT_FP32). */
+ * n, q, and h_{t-1}).  Float32 storage is computed in float32 (MEBPTT_TF32 = MEBPTT_FP32); bf16 operands go
+ * through the tensor cores unless they are forbidden. */
 enum { MEBPTT_FLAG_GRU = 4 };
 
 /* Bytes of one hidden-state unit (all layers) for this descriptor; 0 on a bad descriptor. */

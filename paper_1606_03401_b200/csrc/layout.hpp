@@ -37,8 +37,8 @@ struct Layout {
   bool stepwise_x3 = false;   // likewise for float32 storage, operands split into bfloat16 halves
   bool x3_runs = false;       // of the latter, one layer whose runs persistent kernels take
   bool tensor_cores = true;   // not forbidden by the caller
-  bool gru = false;           // the core is a GRU (CUDA-core kernels)
-  bool team = false;          // CUDA-core shapes walked by the persistent kernel of team.cu
+  bool gru = false;           // the core is a GRU
+  bool team = false;          // the tape is walked by the persistent kernels of pod.cu or team.cu
   int NG = 4;                 // row blocks of H rows in a layer's weight matrix and bias: 4 (LSTM) or 3 (GRU)
   size_t esz = 0;        // bytes of one operand element
   size_t granule = 0;
@@ -54,7 +54,7 @@ struct Layout {
   size_t rec_in = 0;     // input hidden state
   // workspace offsets: states
   size_t off_arena = 0, off_core = 0, off_ping = 0, off_pong = 0, off_init = 0;
-  // carried gradients and per-step scratch of the CUDA-core path
+  // carried gradients and per-step scratch of the operation-by-operation paths
   size_t off_dh = 0, off_dc = 0, off_dha = 0, off_dz = 0, off_dy = 0;
   size_t off_loss_part = 0, off_loss_t = 0;
   // tensor-core path: packed weights, staging of S consecutive time steps, control

@@ -37,7 +37,9 @@ constexpr int BN_WIDE = 128, BN_NARROW = 32;   // tile widths; narrow tiles spre
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int gemm_smem(int stages, int bn) { return stages * (A_BYTES + bn * BK * 2) + 1024; }  // + slack to align the ring to 1024 B
 
-template <bool A_MN, bool B_MN, int BN = BN_WIDE>
+// HALVES: an instance whose loss epilogue writes dy in halves (in the one instance all share, bf16 training steps
+// lost 0.4 %; with an instance of its own for the bf16 loss as well, 1 % where every step's readout is batched).
+template <bool A_MN, bool B_MN, int BN = BN_WIDE, bool HALVES = false>
 __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ CUtensorMap tma,
                                                         const __grid_constant__ CUtensorMap tmb, GemmOut out,
                                                         int M, int N, int K, int STAGES, int* status,
@@ -231,15 +233,17 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ 
         float sq = 0.f;
         if (row < M) {
           const float* tp = out.target + (size_t)row * out.ld + col0;
-          __nv_bfloat16* dp = reinterpret_cast<__nv_bfloat16*>(out.ptr) + (size_t)row * out.ld + col0;
+          // halves: a row is [hi | hi | mid], each as wide as C
+          __nv_bfloat16* dp = HALVES ? reinterpret_cast<__nv_bfloat16*>(out.dy3) + (size_t)row * 3 * out.ld + col0
+                                     : reinterpret_cast<__nv_bfloat16*>(out.ptr) + (size_t)row * out.ld + col0;
           const float two = 2.f * out.scale;
-          __nv_bfloat16* d3 = out.dy3 ? reinterpret_cast<__nv_bfloat16*>(out.dy3) + (size_t)row * 3 * out.ld + col0 : nullptr;
           if (col0 + 32 <= N && ((reinterpret_cast<uintptr_t>(tp) & 15) == 0) && ((reinterpret_cast<uintptr_t>(dp) & 15) == 0) &&
-              ((reinterpret_cast<uintptr_t>(out.bias) & 15) == 0) && ((reinterpret_cast<uintptr_t>(d3) & 15) == 0) && out.ld % 8 == 0) {
+              ((reinterpret_cast<uintptr_t>(out.bias) & 15) == 0) && (!HALVES || out.ld % 8 == 0)) {
             float4 t4[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) t4[j] = *reinterpret_cast<const float4*>(tp + 4 * j);
-            uint32_t packed[16], rest[16];
+            uint32_t packed[16];
+            [[maybe_unused]] uint32_t rest[16];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -251,25 +255,20 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ 
               sq = fmaf(d0, d0, sq); sq = fmaf(d1, d1, sq); sq = fmaf(d2, d2, sq); sq = fmaf(dd, dd, sq);
               packed[2 * j] = pack_bf16x2(d0 * two, d1 * two);
               packed[2 * j + 1] = pack_bf16x2(d2 * two, dd * two);
-              if (d3) {
+              if constexpr (HALVES) {
                 const float2 h0 = unpack_bf16x2(packed[2 * j]), h1 = unpack_bf16x2(packed[2 * j + 1]);
                 rest[2 * j] = pack_bf16x2(d0 * two - h0.x, d1 * two - h0.y);
                 rest[2 * j + 1] = pack_bf16x2(d2 * two - h1.x, dd * two - h1.y);
               }
             }
-            if (d3) {
 #pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const uint4 hi = make_uint4(packed[4 * j], packed[4 * j + 1], packed[4 * j + 2], packed[4 * j + 3]);
-                *reinterpret_cast<uint4*>(d3 + 8 * j) = hi;
-                *reinterpret_cast<uint4*>(d3 + out.ld + 8 * j) = hi;
-                *reinterpret_cast<uint4*>(d3 + 2 * out.ld + 8 * j) = make_uint4(rest[4 * j], rest[4 * j + 1], rest[4 * j + 2], rest[4 * j + 3]);
+            for (int j = 0; j < 4; ++j) {
+              const uint4 v = make_uint4(packed[4 * j], packed[4 * j + 1], packed[4 * j + 2], packed[4 * j + 3]);
+              *reinterpret_cast<uint4*>(dp + 8 * j) = v;
+              if constexpr (HALVES) {
+                *reinterpret_cast<uint4*>(dp + out.ld + 8 * j) = v;
+                *reinterpret_cast<uint4*>(dp + 2 * out.ld + 8 * j) = make_uint4(rest[4 * j], rest[4 * j + 1], rest[4 * j + 2], rest[4 * j + 3]);
               }
-            }
-            if (out.ptr) {
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                *reinterpret_cast<uint4*>(dp + 8 * j) = make_uint4(packed[4 * j], packed[4 * j + 1], packed[4 * j + 2], packed[4 * j + 3]);
             }
           } else {
 #pragma unroll
@@ -277,12 +276,11 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ 
               if (col0 + j < N) {
                 const float d = (__uint_as_float(r[j]) + (out.bias ? out.bias[col0 + j] : 0.f)) - tp[j];
                 sq = fmaf(d, d, sq);
-                if (out.ptr) dp[j] = __float2bfloat16_rn(d * two);
-                if (d3) {
-                  const __nv_bfloat16 hi = __float2bfloat16_rn(d * two);
-                  d3[j] = hi;
-                  d3[out.ld + j] = hi;
-                  d3[2 * out.ld + j] = __float2bfloat16_rn(d * two - __bfloat162float(hi));
+                const __nv_bfloat16 hi = __float2bfloat16_rn(d * two);
+                dp[j] = hi;
+                if constexpr (HALVES) {
+                  dp[out.ld + j] = hi;
+                  dp[2 * out.ld + j] = __float2bfloat16_rn(d * two - __bfloat162float(hi));
                 }
               }
           }
@@ -407,6 +405,8 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
               int M, int N, int K, int* status, cudaStream_t s, bool early, const SplitWs* split, int force_splits,
               SplitParts* defer) {
   if (M <= 0 || N <= 0 || K <= 0) return MEBPTT_ERR_ARG;
+  const bool loss = out.kind == GemmOut::LOSS_DY;
+  if (loss && (a_mn || b_mn || !(out.dy3 || out.ptr))) return MEBPTT_ERR_ARG;
   // A short-and-wide product over K-major operands (a few steps' worth of rows against a whole
   // weight matrix) gives few 128-wide tiles, each streaming all of K through one SM: 32-wide tiles
   // put four times as many SMs to work on the same bytes.
@@ -437,6 +437,9 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
     cudaFuncSetAttribute(gemm_bf16_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          gemm_smem(MAX_STAGES, BN_NARROW));
+    cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_WIDE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_NARROW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         gemm_smem(MAX_STAGES, BN_NARROW));
     return true;
   }();
   (void)attrs;
@@ -444,7 +447,8 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
   // loop.  Grids of at most one wave: 6 stages, more loads in flight per CTA to hide their latency.
   const int stages = (grid.x * grid.y * grid.z <= 148) ? MAX_STAGES : 3;
   const int GEMM_SMEM = gemm_smem(stages, BN);
-  auto* fn = narrow ? gemm_bf16_kernel<false, false, BN_NARROW>
+  auto* fn = loss && out.dy3 ? (narrow ? gemm_bf16_kernel<false, false, BN_NARROW, true> : gemm_bf16_kernel<false, false, BN_WIDE, true>)
+             : narrow ? gemm_bf16_kernel<false, false, BN_NARROW>
              : a_mn ? (b_mn ? gemm_bf16_kernel<true, true> : gemm_bf16_kernel<true, false>)
                     : (b_mn ? gemm_bf16_kernel<false, true> : gemm_bf16_kernel<false, false>);
   const cudaError_t e = launch_on(early, fn, grid, dim3(128), (size_t)GEMM_SMEM, s, ta, tb, out, M, N, K, stages, status,

@@ -37,10 +37,14 @@ constexpr int BN_WIDE = 128, BN_NARROW = 32;   // tile widths; narrow tiles spre
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int gemm_smem(int stages, int bn) { return stages * (A_BYTES + bn * BK * 2) + 1024; }  // + slack to align the ring to 1024 B
 
-// HALVES: an instance whose loss epilogue writes dy in halves (in the one instance all share, bf16 training steps
-// lost 0.4 %; with an instance of its own for the bf16 loss as well, 1 % where every step's readout is batched).
+// HALVES: an instance whose loss epilogue writes dy in halves.  (Its registers and instructions in the other
+// instances' epilogue cost bf16 training steps 0.4 %; an instance of its own for the bf16 loss, too, costs 1 %:
+// its loads of the targets are then fewer in flight.)
+// Four CTAs an SM would be more than shared memory holds: the bound lets the compiler keep up to 128 registers,
+// so that more of an epilogue's loads are in flight, and the instances with an MN-major operand (the gradients)
+// have no loss epilogue (H = 1024, full memory with dx: 12.30 -> 12.22 ms; MSM m = 100: 18.13 -> 18.03 ms).
 template <bool A_MN, bool B_MN, int BN = BN_WIDE, bool HALVES = false>
-__global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ CUtensorMap tma,
+__global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant__ CUtensorMap tma,
                                                         const __grid_constant__ CUtensorMap tmb, GemmOut out,
                                                         int M, int N, int K, int STAGES, int* status,
                                                         float* partial, int fault) {
@@ -227,7 +231,7 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(const __grid_constant__ 
       uint32_t r[32];
       load_acc(c, r);
       const int col0 = n0 + c * 32;
-      if (out.kind == GemmOut::LOSS_DY) {
+      if (!A_MN && !B_MN && out.kind == GemmOut::LOSS_DY) {
         // squared-error loss fused into the readout: this lane's row against its targets, columns in
         // ascending order, then the 32 rows of the warp in a fixed butterfly order
         float sq = 0.f;

@@ -469,6 +469,22 @@ int mebptt_gemm_bf16(const void *A, int64_t lda, int a_major, const void *B, int
  */
 int mebptt_test_wait_fault(int mask);
 
+/*
+ * Testing aid: which kernels a step of this problem under this plan runs on, so that a test written for
+ * one of them can tell that it still gets there.  out[0]: MEBPTT_ROUTE_*; out[1]: time steps per staged
+ * chunk (0: none are staged); out[2], out[3]: CTAs and batch rows of a pod or team, else 0.
+ */
+enum {
+  MEBPTT_ROUTE_OPERATIONS = 0,   /* a launch per contraction on the CUDA cores             */
+  MEBPTT_ROUTE_PERSISTENT = 1,   /* persistent tensor-core kernels, one bfloat16 layer     */
+  MEBPTT_ROUTE_STEPWISE = 2,     /* bfloat16 GEMMs, operation by operation                 */
+  MEBPTT_ROUTE_STEPWISE_F32 = 3, /* the same with float32 storage                          */
+  MEBPTT_ROUTE_RUNS_F32 = 4,     /* persistent kernels, one layer of float32 storage       */
+  MEBPTT_ROUTE_PODS = 5,         /* whole tapes, a cluster of CTAs per group of batch rows */
+  MEBPTT_ROUTE_TEAMS = 6         /* whole tapes, a cooperative grid                        */
+};
+int mebptt_test_route(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan, int64_t *out);
+
 const char *mebptt_strerror(int status);
 
 #ifdef __cplusplus

@@ -90,6 +90,7 @@ _SIGS = {
     "mebptt_lstm_prepare": (_i32, [_descp, _vp]),
     "mebptt_lstm_prepare_stats": (_i32, [C.POINTER(_i64)]),
     "mebptt_test_wait_fault": (_i32, [_i32]),
+    "mebptt_test_route": (_i32, [_descp, _vp, C.POINTER(_i64)]),
     "mebptt_slot_copy": (_i32, [_vp, _vp, _sz, _vp]),
     "mebptt_gemm_bf16": (_i32, [_vp, _i64, _i32, _vp, _i64, _i32, _vp, _i64, _i32, _vp, _i64, _i64, _i64, _vp, _vp]),
     "mebptt_strerror": (C.c_char_p, [_i32]),
@@ -315,6 +316,16 @@ def mebptt_lstm_prepare_stats() -> dict:
 
 def mebptt_test_wait_fault(mask: int) -> None:
     _check(lib.mebptt_test_wait_fault(int(mask)), "mebptt_test_wait_fault")
+
+
+ROUTES = ("operations", "persistent", "stepwise", "stepwise_f32", "runs_f32", "pods", "teams")
+
+
+def mebptt_test_route(desc, plan) -> dict:
+    """Which kernels a step runs on: {"route": one of ROUTES, "chunk": steps, "ctas": n, "rows": n}."""
+    out = (_i64 * 4)()
+    _check(lib.mebptt_test_route(C.byref(desc), plan.handle, out), "mebptt_test_route")
+    return {"route": ROUTES[out[0]], "chunk": out[1], "ctas": out[2], "rows": out[3]}
 
 
 def mebptt_lstm_run_times() -> dict:

@@ -12,7 +12,9 @@
 #include "layout.hpp"
 #include "mebptt.h"
 #include "plan.hpp"
+#include "pod.hpp"
 #include "tc.hpp"
+#include "team.hpp"
 #include "team_run.hpp"
 
 using namespace mebptt;
@@ -781,6 +783,24 @@ int mebptt_lstm_prepare(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan)
 int mebptt_test_wait_fault(int mask) {
   if (mask < 0 || mask > 7) return MEBPTT_ERR_ARG;
   tc::set_wait_fault_mask(mask);
+  return MEBPTT_OK;
+}
+
+int mebptt_test_route(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, int64_t* out) {
+  if (!out) return MEBPTT_ERR_ARG;
+  const int rc = check_common(desc, plan);
+  if (rc != MEBPTT_OK) return rc;
+  Layout y;
+  workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
+  out[0] = y.tensor_path ? MEBPTT_ROUTE_PERSISTENT : y.stepwise_tc ? MEBPTT_ROUTE_STEPWISE : y.x3_runs ? MEBPTT_ROUTE_RUNS_F32
+           : y.stepwise_x3 ? MEBPTT_ROUTE_STEPWISE_F32 : MEBPTT_ROUTE_OPERATIONS;
+  out[1] = y.S; out[2] = 0; out[3] = 0;
+  if (y.team) {
+    const team::Route r = team::route(y);
+    out[0] = r.pod ? MEBPTT_ROUTE_PODS : MEBPTT_ROUTE_TEAMS;
+    out[2] = r.pod ? r.pc.T : r.c.T;
+    out[3] = r.pod ? r.pc.nb : r.c.rows;
+  }
   return MEBPTT_OK;
 }
 

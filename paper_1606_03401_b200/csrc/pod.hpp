@@ -112,10 +112,23 @@ struct Config {
 };
 inline int kin(const Config& c, int l) { return l ? c.kh : c.kx; }
 
-Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max_clusters);
+Config choose_config(const Layout& y, const team::DeviceFacts& dev);
 // elements of the packed weights: layer l, readout
 size_t packed_elems(const Config& c, int l);
 size_t packed_readout_elems(const Config& c);
+
+}  // namespace pod
+
+struct team::Route {
+  bool ok = false;
+  bool pod = false;      // the pod kernel with pc, else the walking kernel with c
+  double cycles = 0;
+  Config c;
+  pod::Config pc;
+};
+namespace team { Route route(const Layout& y); }
+
+namespace pod {
 
 struct Schedule {
   std::vector<Task> tasks;   // records

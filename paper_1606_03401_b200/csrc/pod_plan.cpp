@@ -21,15 +21,15 @@ size_t packed_readout_elems(const Config& c) { return (size_t)c.T * c.op * c.pit
 // arithmetic of a phase shows beside its fixed part, CTAs until the pushes to all of them do; pods
 // that do not fit the device at once take turns.  The tensor cores want their weights in shared memory;
 // the FMA path can read them from the L2, which then bounds it.
-Config choose_config(const Layout& y, bool tensor_cores, int sms, const int* max_clusters) {
+Config choose_config(const Layout& y, const team::DeviceFacts& dev) {
   Config best;
   const int esz = (int)y.esz;
-  if (y.L > kMaxLayers || (y.dtype == MEBPTT_BF16 && !tensor_cores)) return best;
+  if (y.L > kMaxLayers || (y.dtype == MEBPTT_BF16 && !y.tensor_cores)) return best;
   for (int lt = 0; lt <= 4; ++lt)
     for (int nb = 1; nb <= 8; nb *= 2) {
       Config c;
       c.T = 1 << lt; c.nb = nb; c.pods = ceil_div(y.B, nb);
-      const int fit = std::min(max_clusters[lt], sms >> lt);
+      const int fit = std::min(dev.clusters[lt], dev.sms >> lt);
       if (fit < 1 || c.T > y.H || (nb > 1 && nb >= 2 * y.B)) continue;
       c.mma = y.dtype == MEBPTT_BF16;
       c.planes = 3;

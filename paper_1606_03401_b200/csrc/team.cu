@@ -847,10 +847,6 @@ WalkFn walk_fn(const Layout& y, int nb) {
 // ------------------------------------------------------------------------------------------
 namespace {
 
-// What a shape's configuration needs to know of a device: SMs, and clusters of 1, 2, .. 16 CTAs of the
-// walking kernel (a whole SM each) that fit at once.  Without a device: the figures of a B200.
-struct DeviceFacts { bool known = false; int sms = 148; int clusters[5] = {148, 74, 36, 16, 7}; };
-
 // The kernels take nearly a whole SM's shared memory and clusters of up to 16 CTAs.
 cudaError_t allow(const void* fn) {
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
@@ -858,21 +854,23 @@ cudaError_t allow(const void* fn) {
   return e;
 }
 
+}  // namespace
+
 DeviceFacts facts() {
   static std::mutex mu;
   static DeviceFacts table[64];
+  static bool known[64];
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return DeviceFacts{}; }
   std::lock_guard<std::mutex> lock(mu);
   DeviceFacts& f = table[dev];
-  if (!f.known) {
-    int sms = 0;
-    pod::Fn fn = pod::kernel(MEBPTT_FP32, false, 1);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || allow(reinterpret_cast<const void*>(fn)) != cudaSuccess) {
-      cudaGetLastError();
-      return DeviceFacts{};
-    }
+  if (known[dev]) return f;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); return DeviceFacts{}; }
+  if (sms < f.sms) {
     f.sms = sms;
+    const pod::Fn fn = pod::kernel(MEBPTT_FP32, false, 1);
+    const bool may = allow(reinterpret_cast<const void*>(fn)) == cudaSuccess;
     for (int i = 0; i <= 4; ++i) {
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
@@ -881,13 +879,16 @@ DeviceFacts facts() {
       cfg.gridDim = dim3((unsigned)(sms >> i) << i); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kSmemMax - 1024;
       cfg.attrs = at; cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      if (!may || cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) n = 0;
       f.clusters[i] = n;
     }
-    f.known = true;
+    cudaGetLastError();
   }
+  known[dev] = true;
   return f;
 }
+
+namespace {
 
 // The schedule of a plan for one problem on one device, kept from step to step (eight of them, most
 // recently used first); its tasks lie in page-locked memory where that can be had.
@@ -895,9 +896,7 @@ struct Kept {
   uint64_t plan_id = 0;
   Layout y;
   bool pageable = false;
-  bool pod = false;            // the pod kernel serves it (pc), else the walking kernel (c)
-  Config c;
-  pod::Config pc;
+  Route route;
   std::vector<Launch> launches;
   char* tasks = nullptr;       // 32 bytes each
   bool pinned = false;
@@ -918,16 +917,14 @@ bool same_problem(const Layout& a, const Layout& b) {
 }
 
 std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable) {
-  const DeviceFacts f = facts();
-  const Config c = choose_config(y, f.sms);
-  const pod::Config pc = pod::choose_config(y, y.tensor_cores, f.sms, f.clusters);
-  const bool use_pod = pc.ok && (y.total >> 32) == 0 && (!c.ok || pc.cycles <= c.cycles);
-  if (!c.ok && !use_pod) return nullptr;
+  Route r = route(y);
+  if (r.pod && y.total >> 32) { r.pod = false; r.ok = r.c.ok; }   // (the pod kernel's offsets have 32 bits)
+  if (!r.ok) return nullptr;
   {
     std::lock_guard<std::mutex> lock(g_mu);
     for (size_t i = 0; i < g_kept.size(); ++i) {
       Kept& k = *g_kept[i];
-      if (k.plan_id == p->id && same_problem(k.y, y) && (k.pageable || !pageable) && k.pod == use_pod && k.c.T == c.T && k.c.teams == c.teams && k.pc.T == pc.T && k.pc.nb == pc.nb) {
+      if (k.plan_id == p->id && same_problem(k.y, y) && (k.pageable || !pageable) && k.route.pod == r.pod && k.route.c.T == r.c.T && k.route.c.teams == r.c.teams && k.route.pc.T == r.pc.T && k.route.pc.nb == r.pc.nb) {
         std::shared_ptr<Kept> hit = g_kept[i];
         g_kept.erase(g_kept.begin() + (long)i);
         g_kept.insert(g_kept.begin(), hit);
@@ -936,14 +933,14 @@ std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable
     }
   }
   std::shared_ptr<Kept> k = std::make_shared<Kept>();
-  k->plan_id = p->id; k->y = y; k->c = c; k->pc = pc; k->pod = use_pod; k->pageable = pageable;
+  k->plan_id = p->id; k->y = y; k->route = r; k->pageable = pageable;
   Schedule ws;
   pod::Schedule ps;
-  if (use_pod) pod::build_schedule(y, p, pc, ps);
-  else build_schedule(y, p, c, ws);
-  k->launches = use_pod ? ps.launches : ws.launches;
-  const void* from = use_pod ? (const void*)ps.tasks.data() : (const void*)ws.tasks.data();
-  const size_t bytes = (use_pod ? ps.tasks.size() : ws.tasks.size()) * sizeof(Task);
+  if (r.pod) pod::build_schedule(y, p, r.pc, ps);
+  else build_schedule(y, p, r.c, ws);
+  k->launches = r.pod ? ps.launches : ws.launches;
+  const void* from = r.pod ? (const void*)ps.tasks.data() : (const void*)ws.tasks.data();
+  const size_t bytes = (r.pod ? ps.tasks.size() : ws.tasks.size()) * sizeof(Task);
   void* mem = nullptr;
   if (!pageable && bytes <= kMaxPinned && cudaHostAlloc(&mem, bytes, cudaHostAllocDefault) == cudaSuccess) {
     k->pinned = true;
@@ -1039,16 +1036,18 @@ void forget_plan(uint64_t plan_id) {
 int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool want_dx, cudaStream_t s, bool dry) {
   const std::shared_ptr<Kept> kept = schedule_for(y, p, io.pageable_tape);
   if (!kept) return dry ? -1 : MEBPTT_ERR_OOM;
-  const Config& c = kept->c;
+  const Config& c = kept->route.c;
+  const pod::Config& pc = kept->route.pc;
+  const bool pods = kept->route.pod;
   if (dry) {
     int64_t n = 2;   // packing, finalisation
     for (const Launch& g : kept->launches) n += g.chunk >= 0 ? 3 : 1;
     return n;
   }
   const Dims d = dims(y);
-  if (kept->pod) {
+  if (pods) {
     pod::PackArgs q{};
-    q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.c = kept->pc;
+    q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.c = pc;
     q.W = io.W; q.W_out = io.W_out; q.h0 = io.h0; q.c0 = io.c0;
     for (int l = 0; l < y.L; ++l) { q.wf[l] = io.ws + y.off_wf[l]; q.w_off[l] = y.w_layer_offset(l); }
     q.wr = io.ws + y.off_wr; q.states = io.ws + y.off_arena; q.n_blocks = y.n_blocks; q.init = y.blk_init;
@@ -1076,9 +1075,9 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     q.status = reinterpret_cast<int*>(io.ws + y.off_status);
     q.counters = io.counters;
   };
-  if (kept->pod) {
+  if (pods) {
     common(pa);
-    pa.c = kept->pc;
+    pa.c = pc;
     pf = pod::kernel(y.dtype, y.gru, pa.c.nb);
     if (allow(reinterpret_cast<const void*>(pf)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
   } else {
@@ -1109,11 +1108,11 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     }
     if (g.ntasks) {
       int rc;
-      if (kept->pod) {
+      if (pods) {
         pa.tasks = reinterpret_cast<const pod::Task*>(region + (g.task0 - up_lo));
         pa.n_tasks = (int)g.ntasks; pa.phases = g.phases; pa.fwd_ops = g.fwd_ops; pa.bwd_ops = g.bwd_ops;
         void* args[1] = {&pa};
-        rc = launch(reinterpret_cast<const void*>(pf), kept->pc.pods * kept->pc.T, kept->pc.T, kept->pc.smem, args, s);
+        rc = launch(reinterpret_cast<const void*>(pf), pc.pods * pc.T, pc.T, pc.smem, args, s);
       } else {
         a.tasks = region + (g.task0 - up_lo);
         a.n_tasks = (int)g.ntasks;

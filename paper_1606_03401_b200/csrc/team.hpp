@@ -71,7 +71,6 @@ struct Config {
   int ns_f[kMaxLayers] = {}, ns_b[kMaxLayers] = {}, ns_r = 1;   // parts the contraction index is cut into
   int pool_floats = 0;                      // shared memory for a phase's operands and partial sums
   uint64_t resident = 0;                    // bit 2l: F(l) weights in shared memory, 2l+1: B(l), 63: readout
-  int w_floats4 = 0;                        // 16-byte units of resident weights
   int smem = 0;
 };
 // What a phase's pool holds for one task, in floats: staged operand rows and partial sums.
@@ -80,9 +79,18 @@ Need need_f(const Layout& y, const Dims& d, const Config& c, int l);
 Need need_r(const Layout& y, const Dims& d, const Config& c);
 Need need_b(const Layout& y, const Dims& d, const Config& c, int l);
 
-// sms: SMs of the device
 Config choose_config(const Layout& y, int sms);
-// (supported, in layout.hpp: whether some configuration exists; asked for the layout, before a device is known)
+
+// What a configuration needs to know of the device: SMs, and clusters of 1, 2, .. 16 CTAs (a whole SM each)
+// that are resident at once.  These are a B200's, and on a device with as many SMs they are not asked for: the
+// same problem then takes the same kernels, with the same bits, on every one of them, and in a count made
+// without a device.  A part of a device (fewer SMs) is asked.
+struct DeviceFacts { int sms = 148; int clusters[5] = {148, 74, 33, 15, 7}; };
+DeviceFacts facts();
+
+// The kernel a problem goes to: the pod kernel (pod.hpp) or the walking kernel, whichever is estimated
+// faster.  It depends on the descriptor alone, not on the plan.
+struct Route;
 
 struct Launch {          // one launch of the persistent kernel
   size_t task0 = 0, ntasks = 0;   // a whole number of windows

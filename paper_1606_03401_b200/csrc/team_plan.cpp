@@ -139,20 +139,26 @@ Config choose_config(const Layout& y, int sms) {
 // ahead where the recurrent weights are large.  The persistent kernels for float32 storage take some
 // 20 us and a launch or several a run: at H = 160, B = 32 (estimated 29600) both were within a
 // fifth of each other, at 224 units and 64 rows or 304 and 32 (43700 and up) those were 1.1 to 1.4 times
-// faster under every plan.  (Asked for the layout, before a device is known: a B200 is assumed.)
+// faster under every plan.
 bool supported(const mebptt_lstm_desc* d) {
   constexpr double kStepwise = 70000.0;   // a fifth less than measured, to be worth leaving
   constexpr double kRuns = 33000.0;
   Layout y;
   state_layout(d, y);
   if (y.tensor_path || y.L > kMaxLayers || y.t >= (1 << 30)) return false;
-  const int clusters[5] = {148, 74, 33, 15, 7};
-  const pod::Config pc = pod::choose_config(y, y.tensor_cores, 148, clusters);
-  const Config c = choose_config(y, 148);
-  if (!pc.ok && !c.ok) return false;
-  if (!y.stepwise_tc && !y.stepwise_x3) return true;
-  const double least = y.x3_runs ? kRuns : kStepwise * y.L;
-  return (pc.ok && pc.cycles < least) || (c.ok && c.cycles < least);
+  const Route r = route(y);
+  return r.ok && ((!y.stepwise_tc && !y.stepwise_x3) || r.cycles < (y.x3_runs ? kRuns : kStepwise * y.L));
+}
+
+Route route(const Layout& y) {
+  const DeviceFacts dev = facts();
+  Route r;
+  r.c = choose_config(y, dev.sms);
+  r.pc = pod::choose_config(y, dev);
+  r.pod = r.pc.ok && (!r.c.ok || r.pc.cycles <= r.c.cycles);
+  r.ok = r.pod || r.c.ok;
+  r.cycles = r.pod ? r.pc.cycles : r.c.cycles;
+  return r;
 }
 
 namespace {

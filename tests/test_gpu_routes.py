@@ -1,0 +1,48 @@
+"""GPU: which kernels serve a problem is settled by its descriptor, not by the device or by there being one."""
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+CHILD = r"""
+import json, sys
+sys.path.insert(0, {root!r})
+from paper_1606_03401_b200 import binding as B
+if {device}:
+    import torch
+    torch.zeros(1, device="cuda:0")
+out = []
+for dtype in ("fp32", "bf16"):
+    for layers in (1, 2, 3):
+        for hidden in (24, 64, 100, 130, 200, 256, 300, 520):
+            for batch in (1, 3, 17, 33, 36, 64, 70, 140):
+                for flags in (0, B.MEBPTT_FLAG_GRU):
+                    desc = B.make_desc(layers, 40, hidden, 24, batch, 12, dtype, flags=flags)
+                    plan = B.mebptt_plan(12, 5, B.MEBPTT_HSM)
+                    r = B.mebptt_test_route(desc, plan)
+                    out.append([r["route"], r["chunk"], r["ctas"], r["rows"], B.mebptt_lstm_launch_count(desc, plan),
+                                B.mebptt_lstm_workspace_bytes(desc, plan)])
+print("ROUTES " + json.dumps(out))
+"""
+
+
+def _routes(device):
+    env = dict(os.environ)
+    if not device:
+        env["CUDA_VISIBLE_DEVICES"] = ""
+    out = subprocess.run([sys.executable, "-c", CHILD.format(root=ROOT, device=device)], env=env, capture_output=True,
+                         text=True, timeout=600)
+    assert out.returncode == 0, out.stderr[-2000:]
+    return json.loads([l for l in out.stdout.splitlines() if l.startswith("ROUTES ")][-1][len("ROUTES "):])
+
+
+def test_a_count_without_a_device_is_that_of_the_device():
+    with_device, without = _routes(True), _routes(False)
+    assert with_device == without
+    assert {r[0] for r in without} >= {"pods", "teams", "persistent"}

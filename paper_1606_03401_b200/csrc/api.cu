@@ -570,9 +570,7 @@ size_t mebptt_lstm_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_pl
   if (check_common(desc, plan) != MEBPTT_OK) return 0;
   Layout y;
   workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
-  // the persistent kernels address the workspace in 16-byte units held in 32 bits
-  if (y.tensor_path && y.total >= ((size_t)1 << 36)) return 0;
-  return y.total;
+  return addressable(y) ? y.total : 0;
 }
 
 size_t mebptt_lstm_working_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
@@ -663,8 +661,7 @@ size_t least_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* 
   if (check_common(desc, plan) != MEBPTT_OK) return 0;
   Layout y;
   workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y, true);
-  if (y.tensor_path && y.total >= ((size_t)1 << 36)) return 0;
-  return y.total;
+  return addressable(y) ? y.total : 0;
 }
 int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, const void* W, const void* b,
                     const void* W_out, const void* b_out, const void* x, const void* targets, const void* h0,
@@ -680,7 +677,7 @@ int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, con
   workspace_layout(desc, p, y);
   // a fixed workspace that is too small for the team path's stages can still serve the kernels without
   if (!side_stream && y.team && y.total > workspace_bytes) workspace_layout(desc, p, y, true);
-  if (y.tensor_path && y.total >= ((size_t)1 << 36)) return MEBPTT_ERR_UNSUPPORTED;   // 16-byte offsets in 32 bits
+  if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < y.total)
     return MEBPTT_ERR_WORKSPACE;
   StepIO io{(const char*)W, (const char*)W_out, (const char*)x, (const char*)h0,
@@ -707,6 +704,7 @@ size_t mebptt_lstm_host_workspace_bytes(const mebptt_lstm_desc* desc, const mebp
   if (check_common(desc, plan) != MEBPTT_OK) return 0;
   Layout y;
   workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
+  if (!addressable(y)) return 0;
   Staging g;
   staging_layout(y, desc->want_dx != 0, y.total, g);
   return g.total;
@@ -725,6 +723,7 @@ int mebptt_lstm_train_step_host(const mebptt_lstm_desc* desc, const mebptt_plan_
   const Plan* p = reinterpret_cast<const Plan*>(plan);
   Layout y;
   workspace_layout(desc, p, y);
+  if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
   Staging g;
   staging_layout(y, desc->want_dx != 0, y.total, g);
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < g.total)

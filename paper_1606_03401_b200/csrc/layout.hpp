@@ -28,6 +28,13 @@ bool supported(const mebptt_lstm_desc* d);
 constexpr size_t kMaxLaunchTasks = 32768;   // 1 MB of tasks per launch at most: what the workspace holds at a time
 }
 
+// Steps per chunk where the tape is walked: 2048 rows of the batched products, at most 64 steps.
+inline int walked_chunk_steps(int B, int64_t t) {
+  int s = 2048 / B > 0 ? 2048 / B : 1;
+  if (s > 64) s = 64;
+  return s > t ? (int)t : s;
+}
+
 struct Layout {
   int L = 0, I = 0, H = 0, O = 0, B = 0;
   int dtype = 0;
@@ -281,9 +288,7 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
   y.off_loss_t = take((size_t)y.t * 4);
   if (y.team) {
     const size_t G = 4 * (size_t)y.H, hp = align_up(y.H, 16), gp = align_up(G, 16), h4 = align_up(y.H, 16);
-    y.S = 2048 / y.B > 0 ? 2048 / y.B : 1;
-    if (y.S > 64) y.S = 64;
-    if (y.S > y.t) y.S = (int)y.t;
+    y.S = walked_chunk_steps(y.B, y.t);
     const size_t rows = (size_t)y.S * y.B;
     // States: a group of batch rows walks the tape without waiting for the others, so each has an arena of
     // its own -- in one arena for all rows what one group writes for a later operation would lie over another
@@ -427,6 +432,13 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     y.off_status = take(256);
   }
   y.total = o;
+}
+
+// Whether the kernels can address the workspace: the persistent ones hold offsets in 16-byte units, those
+// that walk a tape block numbers, both in 32 bits.
+inline bool addressable(const Layout& y) {
+  if (y.tensor_path) return y.total < (size_t)1 << 36;
+  return !y.team || y.n_blocks >> 32 == 0;
 }
 
 }  // namespace mebptt

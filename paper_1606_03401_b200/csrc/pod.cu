@@ -286,7 +286,8 @@ __device__ __forceinline__ void put_planes(bf16* p, int stride, float v) {
   }
 }
 
-template <class T, bool GRU, int NB, int PL>
+// WIDE: a pod's states pass 4 GB.  The sums are the same.
+template <class T, bool GRU, int NB, int PL, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ Args A) {
   constexpr bool MMA = std::is_same<T, bf16>::value;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -349,17 +350,17 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   const bool sends = el < L && (eju & ~3) < u && eb < valid;   // (its group of four has a unit)
   const int row = pod * NB + eb, ej = rank * U + eju, lay = has ? el : 0;
   const size_t e = has ? (size_t)row * H + ej : 0;
-  // offsets (all under 4 GB here) of this element: h, c and gates from the pod's states, dz and h stages and
-  // carried dz from the workspace
+  // offsets of this element: h, c and gates from the pod's states, dz and h stages and carried dz from the start
+  // of the stages (under 4 GB by the rule of choose_config)
   using St = States<T>;
   const St S(A.ws + A.off_states, A.n_blocks, pod, NB, A.B, H);
   const uint32_t le = eb * H + ej, hs_ = S.hs;
   const uint32_t o_h = lay * (1 + St::CR) * hs_ + le * (uint32_t)sizeof(T), o_c = (lay * (1 + St::CR) + 1) * hs_ + le * 4;
   const uint32_t o_g = (L * (1 + St::CR) + 4 * lay) * hs_ + le * (uint32_t)sizeof(T), o_in = (L * (1 + St::CR) + 4 * L) * hs_;
   const uint32_t bh = (uint32_t)A.B * H;                         // elements of a row block of the h stage, a quarter of those of dz
-  const uint32_t o_dz = (uint32_t)(A.off_dz + (lay * (size_t)A.S * bh + e) * 16);
-  const uint32_t o_cy = (uint32_t)(A.off_carry + ((size_t)lay * bh + e) * 16);
-  const uint32_t o_st = (uint32_t)(A.off_hk + (lay * (size_t)(A.S + 1) * bh + e) * sizeof(T));
+  const uint32_t o_dz = (uint32_t)((lay * (size_t)A.S * bh + e) * 16);
+  const uint32_t o_cy = (uint32_t)(A.off_carry - A.off_dz + ((size_t)lay * bh + e) * 16);
+  const uint32_t o_st = (uint32_t)(A.off_hk - A.off_dz + (lay * (size_t)(A.S + 1) * bh + e) * sizeof(T));
   auto dc_at = [&]() { return reinterpret_cast<float*>(A.ws + A.off_dc + ((size_t)lay * bh + e) * 4); };
   float dc = has ? *dc_at() : 0.f;
   float bias[4] = {0.f, 0.f, 0.f, 0.f};
@@ -409,7 +410,10 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   float om[7];
   float ol = 0.f, o_target = 0.f;
   float4 ox = make_float4(0.f, 0.f, 0.f, 0.f), oz = ox;
-  auto at = [&](uint32_t o, uint32_t loc) { return S.base + (o + loc * hs_); };
+  // The states of a generous budget pass 4 GB.  Below that an offset of 32 bits from a base that is the same for
+  // all threads takes no instruction to add; with 64 bits throughout, the two-layer GRU of 256 units took 1 %
+  // longer (2864 -> 2891 us).
+  auto at = [&](uint32_t o, uint32_t loc) { return WIDE ? S.base + (uint64_t)loc * hs_ + o : S.base + (o + loc * hs_); };
   // h0: n cells sums n_h | n_p n_x r x | products - | main     h1: load carry bwd -
   auto ahead = [&](int cur, const uint4& h0, const uint4& h1) {
     if (warp_s) {
@@ -434,7 +438,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     if (iz) {
       const int k = k_of(rec(cur + 2 * iz));
       const uint32_t sidx = sidx_of(rec(cur + 2 * iz + 1));
-      oz = *reinterpret_cast<const float4*>(A.ws + (sidx == kNone ? o_cy + ((k + 1) & 1) * L * bh * 16 : o_dz + sidx * bh * 16));
+      oz = *reinterpret_cast<const float4*>(A.stages + (sidx == kNone ? o_cy + ((k + 1) & 1) * L * bh * 16 : o_dz + sidx * bh * 16));
     }
     }
     const uint32_t ir = (h0.y >> 16) & 0xff, ix = h0.y >> 24;
@@ -498,10 +502,10 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
           const float g[4] = {om[0], om[1], om[2], om[3]};
           cell_backward<GRU>(s0 + s1, g, om[4], om[5], om[6], dc, d);
           const float4 quad = make_float4(d[0], d[1], d[2], d[3]);
-          *reinterpret_cast<float4*>(A.ws + (o_dz + sidx * bh * 16)) = quad;
-          T* const hs = reinterpret_cast<T*>(A.ws + (o_st + sidx * bh * (uint32_t)sizeof(T)));
+          *reinterpret_cast<float4*>(A.stages + (o_dz + sidx * bh * 16)) = quad;
+          T* const hs = reinterpret_cast<T*>(A.stages + (o_st + sidx * bh * (uint32_t)sizeof(T)));
           store(hs, om[4]);
-          if (fl & CLOSE) *reinterpret_cast<float4*>(A.ws + (o_cy + (k_of(a) & 1) * L * bh * 16)) = quad;
+          if (fl & CLOSE) *reinterpret_cast<float4*>(A.stages + (o_cy + (k_of(a) & 1) * L * bh * 16)) = quad;
           if (fl & OPEN) store(hs + bh, to_f(*reinterpret_cast<const T*>(at(o_h, a.z))));
         } else {
           d[0] = oz.x; d[1] = oz.y; d[2] = oz.z; d[3] = oz.w;
@@ -717,16 +721,23 @@ __global__ void __launch_bounds__(256) pod_pack(const __grid_constant__ PackArgs
   }
 }
 
-template <class T, bool GRU, int PL>
+template <class T, bool GRU, int PL, bool WIDE>
 Fn by_rows(int nb) {
-  return nb == 1 ? pod_walk<T, GRU, 1, PL> : nb == 2 ? pod_walk<T, GRU, 2, PL> : nb == 4 ? pod_walk<T, GRU, 4, PL> : pod_walk<T, GRU, 8, PL>;
+  return nb == 1   ? pod_walk<T, GRU, 1, PL, WIDE>
+         : nb == 2 ? pod_walk<T, GRU, 2, PL, WIDE>
+         : nb == 4 ? pod_walk<T, GRU, 4, PL, WIDE>
+                   : pod_walk<T, GRU, 8, PL, WIDE>;
+}
+template <class T, int PL>
+Fn by_core(bool gru, int nb, bool wide) {
+  if (gru) return wide ? by_rows<T, true, PL, true>(nb) : by_rows<T, true, PL, false>(nb);
+  return wide ? by_rows<T, false, PL, true>(nb) : by_rows<T, false, PL, false>(nb);
 }
 
 }  // namespace
 
-Fn kernel(int dtype, bool gru, int nb) {
-  if (dtype == MEBPTT_BF16) return gru ? by_rows<bf16, true, 3>(nb) : by_rows<bf16, false, 3>(nb);
-  return gru ? by_rows<float, true, 1>(nb) : by_rows<float, false, 1>(nb);
+Fn kernel(int dtype, bool gru, int nb, bool wide) {
+  return dtype == MEBPTT_BF16 ? by_core<bf16, 3>(gru, nb, wide) : by_core<float, 1>(gru, nb, wide);
 }
 
 void launch_pack(int dtype, bool gru, const PackArgs& p, cudaStream_t s) {

@@ -25,6 +25,10 @@ Config choose_config(const Layout& y, const team::DeviceFacts& dev) {
   Config best;
   const int esz = (int)y.esz;
   if (y.L > kMaxLayers || (y.dtype == MEBPTT_BF16 && !y.tensor_cores)) return best;
+  // a thread's offsets from the start of the stages (dz, h, dy, carried dz) and of a step of x have 32 bits (a rule on the descriptor:
+  // how much a plan keeps must not choose the kernel, and with it the order of sums)
+  const int64_t bh = (int64_t)y.B * y.H, steps = std::max(walked_chunk_steps(y.B, y.t), 2);
+  if ((y.L * (steps + 4) * bh * 20 + (int64_t)steps * y.B * y.O * 4) >> 32 || ((int64_t)y.B * y.I) >> 31) return best;
   for (int lt = 0; lt <= 4; ++lt)
     for (int nb = 1; nb <= 8; nb *= 2) {
       Config c;

@@ -19,6 +19,7 @@ struct Args {
   char* ws;
   size_t off_wf[team::kMaxLayers], off_wr;
   size_t off_dz, off_hk, off_dy, off_carry, off_dc;
+  char* stages;                        // ws + off_dz
   const void* x;
   const float *bias, *b_out, *targets;
   const Task* tasks;
@@ -28,7 +29,8 @@ struct Args {
 };
 
 using Fn = void (*)(const Args);
-Fn kernel(int dtype, bool gru, int nb);
+// wide: the states of a pod pass 4 GB
+Fn kernel(int dtype, bool gru, int nb, bool wide);
 
 // Packs the weights in the order the kernel keeps them, lays the initial state out, clears what a step
 // starts from at zero.

@@ -869,7 +869,7 @@ DeviceFacts facts() {
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); return DeviceFacts{}; }
   if (sms < f.sms) {
     f.sms = sms;
-    const pod::Fn fn = pod::kernel(MEBPTT_FP32, false, 1);
+    const pod::Fn fn = pod::kernel(MEBPTT_FP32, false, 1, false);
     const bool may = allow(reinterpret_cast<const void*>(fn)) == cudaSuccess;
     for (int i = 0; i <= 4; ++i) {
       cudaLaunchAttribute at[1];
@@ -917,8 +917,7 @@ bool same_problem(const Layout& a, const Layout& b) {
 }
 
 std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable) {
-  Route r = route(y);
-  if (r.pod && y.total >> 32) { r.pod = false; r.ok = r.c.ok; }   // (the pod kernel's offsets have 32 bits)
+  const Route r = route(y);
   if (!r.ok) return nullptr;
   {
     std::lock_guard<std::mutex> lock(g_mu);
@@ -1077,8 +1076,10 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
   };
   if (pods) {
     common(pa);
+    pa.stages = io.ws + y.off_dz;
     pa.c = pc;
-    pf = pod::kernel(y.dtype, y.gru, pa.c.nb);
+    const size_t states = (size_t)y.n_blocks * align_up((size_t)pc.nb * y.H * y.esz, 16);
+    pf = pod::kernel(y.dtype, y.gru, pc.nb, states >> 32 != 0);
     if (allow(reinterpret_cast<const void*>(pf)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
   } else {
     common(a);

@@ -1,10 +1,14 @@
-"""GPU: which kernels serve a problem is settled by its descriptor, not by the device or by there being one."""
+"""GPU: which kernels serve a problem is settled by its descriptor: not by the plan, nor by the
+device or there being one."""
 import json
 import os
 import subprocess
 import sys
 
 import pytest
+
+from paper_1606_03401_b200 import synth
+from tests.util import assert_bit_identical
 
 pytestmark = pytest.mark.gpu
 
@@ -46,3 +50,23 @@ def test_a_count_without_a_device_is_that_of_the_device():
     with_device, without = _routes(True), _routes(False)
     assert with_device == without
     assert {r[0] for r in without} >= {"pods", "teams", "persistent"}
+
+
+@pytest.mark.parametrize("size,alpha", [
+    (dict(input=16, hidden=128, batch=1024, t=1100, readout=8), 4),              # of all pods together
+    (dict(layers=3, input=16, hidden=256, batch=8, t=6000, readout=8), 64),      # of one pod (slots far larger than a state)
+])
+def test_states_past_4_gib_take_the_same_kernels_and_give_the_same_bits(size, alpha):
+    """Full memory keeps more than 4 GiB of states here, which 32-bit offsets do not reach; a tight plan keeps little."""
+    from paper_1606_03401_b200 import binding as B
+    from paper_1606_03401_b200 import harness as H
+    cfg = synth.with_overrides(synth.CONFIGS["c1"], **size)
+    dp = H.DeviceProblem(cfg, want_dx=True)
+    tight, full = dp.plan("hsm", 40), dp.plan("ism", cfg.t, alpha=alpha)
+    assert B.mebptt_lstm_workspace_bytes(dp.desc, full) > (4 << 30) + B.mebptt_lstm_working_bytes(dp.desc, full)
+    assert B.mebptt_test_route(dp.desc, full) == B.mebptt_test_route(dp.desc, tight)
+    assert B.mebptt_test_route(dp.desc, full)["route"] == "pods"
+    want = dp.run(tight)
+    got = dp.run(full)
+    assert got["counters"][0] == cfg.t and got["counters"][3] == 0 and want["counters"][3] == 0
+    assert_bit_identical(got, want, want_dx=True)

@@ -23,8 +23,13 @@ namespace mebptt {
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 inline size_t gcd_sz(size_t a, size_t b) { while (b) { size_t r = a % b; a = b; b = r; } return a; }
 
+struct Layout;
 namespace team {
 bool supported(const mebptt_lstm_desc* d);
+// elements of the packed weights, in the order of the kernel that serves the problem (wb: 0 where one copy
+// serves both directions)
+struct PackedSizes { size_t wf[16], wb[16], wr; };
+PackedSizes packed_sizes(const Layout& y);
 constexpr size_t kMaxLaunchTasks = 32768;   // 1 MB of tasks per launch at most: what the workspace holds at a time
 }
 
@@ -287,7 +292,7 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
   y.off_dc = take((size_t)y.L * bh4);
   y.off_loss_t = take((size_t)y.t * 4);
   if (y.team) {
-    const size_t G = 4 * (size_t)y.H, hp = align_up(y.H, 16), gp = align_up(G, 16), h4 = align_up(y.H, 16);
+    const size_t G = 4 * (size_t)y.H;
     y.S = walked_chunk_steps(y.B, y.t);
     const size_t rows = (size_t)y.S * y.B;
     // States: a group of batch rows walks the tape without waiting for the others, so each has an arena of
@@ -307,15 +312,12 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     const size_t states = (size_t)blocks * y.B * align_up((size_t)y.H * y.esz + 15, 16);
     if (o < y.off_arena + states) o = align_up(y.off_arena + states, y.granule);
     y.off_loss_t = take((size_t)y.t * 4);
-    // packed weights, in whichever of the two kernels' orders is used (the pod kernel pads rows, and
-    // units to its CTAs: at most 16 and 96 more)
-    auto larger = [](size_t u, size_t v) { return u > v ? u : v; };
+    const team::PackedSizes packed = team::packed_sizes(y);
     for (int l = 0; l < y.L; ++l) {
-      const size_t in = l ? y.H + 96 : align_up(y.I, 16);
-      y.off_wf[l] = take(larger(4 * h4 * (align_up(l ? y.H : y.I, 16) + hp), 4 * ((size_t)y.H + 16) * (in + y.H + 104)) * y.esz);
-      y.off_wb[l] = take(h4 * (gp + (l + 1 < y.L ? gp : align_up(y.O, 16))) * y.esz);
+      y.off_wf[l] = take(packed.wf[l] * y.esz);
+      y.off_wb[l] = take(packed.wb[l] * y.esz);
     }
-    y.off_wr = take(larger(align_up(y.O, 16) * hp, ((size_t)y.O + 64) * (y.H + 104)) * y.esz);
+    y.off_wr = take(packed.wr * y.esz);
     y.off_st_dz = y.off_dz = take((size_t)y.L * rows * G * 4);
     // h of the chunk's steps and of the one before: row block i holds h_{k-1} of the step in block i of dz
     y.off_st_h = take((size_t)y.L * (rows + y.B) * y.H * y.esz);

@@ -161,6 +161,23 @@ Route route(const Layout& y) {
   return r;
 }
 
+PackedSizes packed_sizes(const Layout& y) {
+  PackedSizes s{};
+  const Route r = route(y);
+  if (r.pod) {
+    for (int l = 0; l < y.L; ++l) s.wf[l] = pod::packed_elems(r.pc, l);
+    s.wr = pod::packed_readout_elems(r.pc);
+  } else {
+    const Dims d = dims(y);
+    for (int l = 0; l < y.L; ++l) {
+      s.wf[l] = (size_t)d.gf * d.rpg * d.kf[l];
+      s.wb[l] = (size_t)d.gb * d.rpg * d.kb[l];
+    }
+    s.wr = (size_t)d.gr * d.rpg * d.hp;
+  }
+  return s;
+}
+
 namespace {
 
 // Places each task in the earliest phase after everything it depends on.  Tasks come in the order of

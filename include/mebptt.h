@@ -485,6 +485,18 @@ enum {
 };
 int mebptt_test_route(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan, int64_t *out);
 
+/*
+ * Testing aid: the schedule that a whole tape is walked by (MEBPTT_ROUTE_PODS, MEBPTT_ROUTE_TEAMS), as the
+ * records its kernel reads, for a replay on the host.  room > 0: with so many records a launch instead of what
+ * the workspace has room for.  Fills info[0..18] (pods, steps per chunk, room, and where states and operands
+ * lie: csrc/api.cu has the order), up to most_records records of 32 bytes and most_launches launches of four
+ * values (first record, records, phases, chunk that is complete afterwards or -1).  Returns the number of
+ * records, -1 for another route or a launch that does not fit.
+ */
+int64_t mebptt_test_schedule(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan, int64_t room,
+                             int64_t *info, void *records, int64_t most_records, int64_t *launches,
+                             int64_t most_launches);
+
 const char *mebptt_strerror(int status);
 
 #ifdef __cplusplus

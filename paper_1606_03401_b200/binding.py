@@ -90,6 +90,7 @@ _SIGS = {
     "mebptt_lstm_prepare": (_i32, [_descp, _vp]),
     "mebptt_lstm_prepare_stats": (_i32, [C.POINTER(_i64)]),
     "mebptt_test_wait_fault": (_i32, [_i32]),
+    "mebptt_test_schedule": (_i64, [_descp, _vp, _i64, C.POINTER(_i64), _vp, _i64, C.POINTER(_i64), _i64]),
     "mebptt_test_route": (_i32, [_descp, _vp, C.POINTER(_i64)]),
     "mebptt_slot_copy": (_i32, [_vp, _vp, _sz, _vp]),
     "mebptt_gemm_bf16": (_i32, [_vp, _i64, _i32, _vp, _i64, _i32, _vp, _i64, _i32, _vp, _i64, _i64, _i64, _vp, _vp]),
@@ -326,6 +327,23 @@ def mebptt_test_route(desc, plan) -> dict:
     out = (_i64 * 4)()
     _check(lib.mebptt_test_route(C.byref(desc), plan.handle, out), "mebptt_test_route")
     return {"route": ROUTES[out[0]], "chunk": out[1], "ctas": out[2], "rows": out[3]}
+
+
+SCHEDULE_INFO = ("pods", "chunk", "room", "unit_blocks", "loc_blocks", "n_blocks", "core0", "core1", "ping", "pong", "init",
+                 "x_slot", "h_slot", "at_h", "at_p", "p_slot", "at_dy", "dy_buf", "launches")
+
+
+def mebptt_test_schedule(desc, plan, room: int = 0):
+    """(info, records [n, 32] of bytes, launches [n, 4]) of a walked tape."""
+    info = (_i64 * 19)()
+    n = lib.mebptt_test_schedule(C.byref(desc), plan.handle, room, info, None, 0, None, 0)
+    if n < 0:
+        raise MebpttError(MEBPTT_ERR_UNSUPPORTED, "mebptt_test_schedule")
+    d = dict(zip(SCHEDULE_INFO, info))
+    records, launches = np.zeros((n, 32), np.uint8), np.zeros((d["launches"], 4), np.int64)
+    lib.mebptt_test_schedule(C.byref(desc), plan.handle, room, info, records.ctypes.data, n,
+                             launches.ctypes.data_as(C.POINTER(_i64)), d["launches"])
+    return d, records, launches
 
 
 def mebptt_lstm_run_times() -> dict:

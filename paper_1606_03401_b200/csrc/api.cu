@@ -803,6 +803,31 @@ int mebptt_test_route(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, i
   return MEBPTT_OK;
 }
 
+int64_t mebptt_test_schedule(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, int64_t room, int64_t* info, void* records,
+                             int64_t most_records, int64_t* launches, int64_t most_launches) {
+  if (!info || check_common(desc, plan) != MEBPTT_OK) return -1;
+  const Plan* p = reinterpret_cast<const Plan*>(plan);
+  Layout y;
+  workspace_layout(desc, p, y);
+  if (!y.team) return -1;
+  const team::Route r = team::route(y);
+  team::Records rec;
+  if (!team::build_records(y, p, r, room > 0 ? (size_t)room : y.tape_bytes / 32, rec)) return -1;
+  const int64_t v[16] = {r.pod, y.S, (int64_t)y.tape_bytes / 32, y.unit_blocks, y.loc_blocks, y.n_blocks, y.blk_core[0], y.blk_core[1], y.blk_ping, y.blk_pong,
+                         y.blk_init, r.pc.x_slot, r.pc.h_slot, r.pc.at_h, r.pc.at_p, r.pc.p_slot};
+  memcpy(info, v, sizeof v);
+  info[16] = r.pc.at_dy; info[17] = r.pc.dy_buf;
+  const int64_t n = (int64_t)rec.bytes.size() / 32;
+  if (records) memcpy(records, rec.bytes.data(), (size_t)(n < most_records ? n : most_records) * 32);
+  info[18] = (int64_t)rec.launches.size();
+  for (int64_t i = 0; launches && i < info[18] && i < most_launches; ++i) {
+    const team::Launch& g = rec.launches[(size_t)i];
+    const int64_t q[4] = {(int64_t)g.task0, (int64_t)g.ntasks, g.phases, g.chunk};
+    memcpy(launches + 4 * i, q, sizeof q);
+  }
+  return n;
+}
+
 int mebptt_lstm_prepare_stats(int64_t* out) {
   if (!out) return MEBPTT_ERR_ARG;
   tc::prepare_stats(out);

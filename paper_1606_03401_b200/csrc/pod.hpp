@@ -126,7 +126,13 @@ struct team::Route {
   Config c;
   pod::Config pc;
 };
-namespace team { Route route(const Layout& y); }
+namespace team {
+Route route(const Layout& y);
+// The schedule of a plan for the kernel that serves it, as the 32-byte records that kernel reads; false if a
+// launch does not fit the room there is for one.
+struct Records { std::vector<unsigned char> bytes; std::vector<Launch> launches; };
+bool build_records(const Layout& y, const Plan* p, const Route& r, size_t room, Records& out);
+}  // namespace team
 
 namespace pod {
 
@@ -134,7 +140,9 @@ struct Schedule {
   std::vector<Task> tasks;   // records
   std::vector<team::Launch> launches;
 };
-void build_schedule(const Layout& y, const Plan* p, const Config& c, Schedule& s);
+// room: records a launch may have (a whole number of windows; at least kLeastRoom)
+constexpr size_t kLeastRoom = 4 * kWindow;
+void build_schedule(const Layout& y, const Plan* p, const Config& c, size_t room, Schedule& s);
 
 }  // namespace pod
 }  // namespace mebptt

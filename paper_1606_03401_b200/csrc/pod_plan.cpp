@@ -494,18 +494,27 @@ struct Builder {
 
 }  // namespace
 
-void build_schedule(const Layout& y, const Plan* p, const Config& c, Schedule& s) {
-  Builder w(y, c, s);
-  int64_t index = 0;
-  for (const mebptt_op& op : p->tape) {
-    if (op.kind == MEBPTT_OP_FWD) {
-      w.forward(op, index);
-    } else {
-      w.backward(op);
-      if ((op.k - 1) % y.S == 0) w.close((int)((op.k - 1) / y.S));
+// A launch ends with its chunk, or when as many tasks are open as leave room for the records they become:
+// with headers, loads and padding up to seven times as many (0.99 of that over some thousand problems), and
+// where it is more, launches of fewer tasks.
+void build_schedule(const Layout& y, const Plan* p, const Config& c, size_t room, Schedule& s) {
+  for (int64_t most = (int64_t)team::kMaxLaunchTasks / 7;; most = std::min<int64_t>(most / 2, (int64_t)room / 8)) {
+    s = Schedule{};
+    Builder w(y, c, s);
+    int64_t index = 0;
+    for (const mebptt_op& op : p->tape) {
+      if (op.kind == MEBPTT_OP_FWD) {
+        w.forward(op, index);
+      } else {
+        w.backward(op);
+        if ((op.k - 1) % y.S == 0) w.close((int)((op.k - 1) / y.S));
+      }
+      ++index;
+      if (w.n_open > most) w.close(-1);
     }
-    ++index;
-    if (w.n_open > (int64_t)team::kMaxLaunchTasks / 7) w.close(-1);
+    size_t largest = 0;
+    for (const team::Launch& g : s.launches) largest = std::max(largest, g.ntasks);
+    if (largest <= room || most == 0) return;
   }
 }
 

@@ -916,8 +916,10 @@ bool same_problem(const Layout& a, const Layout& b) {
   return a.L == b.L && a.I == b.I && a.H == b.H && a.O == b.O && a.B == b.B && a.dtype == b.dtype && a.t == b.t && a.gru == b.gru && a.tensor_cores == b.tensor_cores;
 }
 
-std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable) {
+// Null, and a status, where there is none.
+std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable, int& status) {
   const Route r = route(y);
+  status = MEBPTT_ERR_UNSUPPORTED;
   if (!r.ok) return nullptr;
   {
     std::lock_guard<std::mutex> lock(g_mu);
@@ -933,23 +935,20 @@ std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable
   }
   std::shared_ptr<Kept> k = std::make_shared<Kept>();
   k->plan_id = p->id; k->y = y; k->route = r; k->pageable = pageable;
-  Schedule ws;
-  pod::Schedule ps;
-  if (r.pod) pod::build_schedule(y, p, r.pc, ps);
-  else build_schedule(y, p, r.c, ws);
-  k->launches = r.pod ? ps.launches : ws.launches;
-  const void* from = r.pod ? (const void*)ps.tasks.data() : (const void*)ws.tasks.data();
-  const size_t bytes = (r.pod ? ps.tasks.size() : ws.tasks.size()) * sizeof(Task);
+  Records rec;
+  if (!build_records(y, p, r, y.tape_bytes / sizeof(Task), rec)) return nullptr;
+  k->launches = rec.launches;
   void* mem = nullptr;
-  if (!pageable && bytes <= kMaxPinned && cudaHostAlloc(&mem, bytes, cudaHostAllocDefault) == cudaSuccess) {
+  if (!pageable && rec.bytes.size() <= kMaxPinned && cudaHostAlloc(&mem, rec.bytes.size(), cudaHostAllocDefault) == cudaSuccess) {
     k->pinned = true;
   } else {
     cudaGetLastError();
-    mem = malloc(bytes);
+    mem = malloc(rec.bytes.size());
+    status = MEBPTT_ERR_OOM;
     if (!mem) return nullptr;
   }
   k->tasks = static_cast<char*>(mem);
-  memcpy(mem, from, bytes);
+  memcpy(k->tasks, rec.bytes.data(), rec.bytes.size());
   std::lock_guard<std::mutex> lock(g_mu);
   g_kept.insert(g_kept.begin(), k);
   if (g_kept.size() > kKeep) g_kept.pop_back();
@@ -1033,8 +1032,9 @@ void forget_plan(uint64_t plan_id) {
 }
 
 int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool want_dx, cudaStream_t s, bool dry) {
-  const std::shared_ptr<Kept> kept = schedule_for(y, p, io.pageable_tape);
-  if (!kept) return dry ? -1 : MEBPTT_ERR_OOM;
+  int status = MEBPTT_OK;
+  const std::shared_ptr<Kept> kept = schedule_for(y, p, io.pageable_tape, status);
+  if (!kept) return dry ? -1 : status;
   const Config& c = kept->route.c;
   const pod::Config& pc = kept->route.pc;
   const bool pods = kept->route.pod;

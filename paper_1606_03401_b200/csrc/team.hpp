@@ -103,7 +103,8 @@ struct Schedule {
   std::vector<Launch> launches;
   int64_t phases = 0;
 };
-void build_schedule(const Layout& y, const Plan* p, const Config& c, Schedule& s);
+// room: records a launch may have (a whole number of windows)
+void build_schedule(const Layout& y, const Plan* p, const Config& c, size_t room, Schedule& s);
 
 }  // namespace team
 }  // namespace mebptt

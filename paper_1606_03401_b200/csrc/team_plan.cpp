@@ -189,6 +189,7 @@ struct Scheduler {
   Schedule& s;
   std::vector<std::vector<Task>> open;     // tasks by phase, from phase `base` on
   std::vector<int> used;                   // floats of the pool taken, likewise
+  const size_t room;                       // records of a launch
   int64_t base = 0;                        // phases before this one belong to earlier launches
   int64_t top = -1;                        // last phase used
   // when the cells (units) of the arena were last touched; the same for ping, pong and the two cores,
@@ -199,8 +200,8 @@ struct Scheduler {
   std::vector<int64_t> bwd_prev;           // per layer: phase of the latest B
   int core = 0;                            // the working core alternates between two buffers
 
-  Scheduler(const Layout& y_, const Config& c_, Schedule& s_, int64_t arena_units)
-      : y(y_), c(c_), d(dims(y_)), s(s_), cell((size_t)arena_units, -1), named((size_t)4 * y_.L, -1), state((size_t)(arena_units + 5) * y_.L, -1),
+  Scheduler(const Layout& y_, const Config& c_, Schedule& s_, int64_t arena_units, size_t room_)
+      : y(y_), c(c_), d(dims(y_)), s(s_), room(room_), cell((size_t)arena_units, -1), named((size_t)4 * y_.L, -1), state((size_t)(arena_units + 5) * y_.L, -1),
         bwd_prev((size_t)y_.L, -1) {
   }
   uint32_t address(int32_t loc) const {
@@ -268,7 +269,7 @@ struct Scheduler {
     for (auto& ph : open) {
       if (ph.empty()) continue;
       if (s.tasks.size() % kTaskWindow + ph.size() > (size_t)kTaskWindow) pad();
-      if (s.tasks.size() - cur.task0 + kTaskWindow > kMaxLaunchTasks) end(-1);
+      if (s.tasks.size() > cur.task0 && s.tasks.size() - cur.task0 + kTaskWindow > room) end(-1);
       ph.back().flags |= LAST;
       s.tasks.insert(s.tasks.end(), ph.begin(), ph.end());
       ++cur.phases;
@@ -341,8 +342,8 @@ struct Scheduler {
 
 }  // namespace
 
-void build_schedule(const Layout& y, const Plan* p, const Config& c, Schedule& s) {
-  Scheduler w(y, c, s, y.arena_units);
+void build_schedule(const Layout& y, const Plan* p, const Config& c, size_t room, Schedule& s) {
+  Scheduler w(y, c, s, y.arena_units, room);
   for (const mebptt_op& op : p->tape) {
     if (op.kind == MEBPTT_OP_FWD) {
       w.forward(op);
@@ -353,6 +354,28 @@ void build_schedule(const Layout& y, const Plan* p, const Config& c, Schedule& s
     // a tape with very many recomputations between two backward operations: do not hold it all open
     if (w.open.size() > 4 * kMaxLaunchTasks) w.close(-1);
   }
+}
+
+bool build_records(const Layout& y, const Plan* p, const Route& r, size_t room, Records& out) {
+  if (room < (r.pod ? pod::kLeastRoom : (size_t)kTaskWindow)) return false;
+  auto keep = [&](const auto& s) {
+    out.bytes.resize(s.tasks.size() * sizeof(Task));
+    memcpy(out.bytes.data(), s.tasks.data(), out.bytes.size());
+    out.launches = s.launches;
+  };
+  if (r.pod) {
+    pod::Schedule s;
+    pod::build_schedule(y, p, r.pc, room, s);
+    keep(s);
+  } else {
+    Schedule s;
+    build_schedule(y, p, r.c, room, s);
+    keep(s);
+  }
+  // (the launches copy their records to the room and read them there: one that did not fit would read what lies behind)
+  for (const Launch& g : out.launches)
+    if (g.ntasks > room) return false;
+  return true;
 }
 
 }  // namespace team

@@ -34,3 +34,20 @@ def test_weights_are_packed_in_the_order_of_the_kernel_that_runs_and_no_other(si
     weights = (L * 4 * H * (2 * H + 120) + 4 * H * max(0, I - H) + (O + 64) * (H + 104)) * e
     weights = 1.25 * weights * (1 if route["route"] == "pods" else 2)
     assert B.mebptt_lstm_working_bytes(desc, plan) <= stages + carried + states + tape + weights + 64 * 1024
+
+
+@pytest.mark.parametrize("size", WALKED)
+@pytest.mark.parametrize("mode,m", [(B.MEBPTT_HSM, 2), (B.MEBPTT_MSM, 9), (B.MEBPTT_ISM, 10 ** 6)])
+def test_no_launch_has_more_records_than_there_is_room_for(size, mode, m):
+    """A launch reads its records from a region of the workspace; whatever the region's size, they fit, and
+    every operation is still there once."""
+    desc, plan = _problem(size), B.mebptt_plan(size[5], m, mode)
+    layers = size[0]
+    for room in (0, 256, 1024, 32768):
+        info, records, launches = B.mebptt_test_schedule(desc, plan, room)
+        assert launches[:, 1].max() <= (room or info["room"])
+        assert (launches[:, 0] + launches[:, 1]).max() <= len(records) and (launches[:, 1] % 64 == 0).all()
+        assert (launches[:, 3] >= 0).sum() == -(-size[5] // info["chunk"])
+        if not info["pods"]:      # (a pod's headers are records of another kind: replayed elsewhere)
+            kinds = records[:, 0]
+            assert (kinds == 1).sum() == plan.cost * layers and (kinds == 3).sum() == size[5] * layers

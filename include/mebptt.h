@@ -488,7 +488,7 @@ int mebptt_test_route(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan, i
 /*
  * Testing aid: the schedule that a whole tape is walked by (MEBPTT_ROUTE_PODS, MEBPTT_ROUTE_TEAMS), as the
  * records its kernel reads, for a replay on the host.  room > 0: with so many records a launch instead of what
- * the workspace has room for.  Fills info[0..18] (pods, steps per chunk, room, and where states and operands
+ * the workspace has room for.  Fills info[0..19] (pods, steps per chunk, room, and where states and operands
  * lie: csrc/api.cu has the order), up to most_records records of 32 bytes and most_launches launches of four
  * values (first record, records, phases, chunk that is complete afterwards or -1).  Returns the number of
  * records, -1 for another route or a launch that does not fit.

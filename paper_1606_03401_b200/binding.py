@@ -330,12 +330,12 @@ def mebptt_test_route(desc, plan) -> dict:
 
 
 SCHEDULE_INFO = ("pods", "chunk", "room", "unit_blocks", "loc_blocks", "n_blocks", "core0", "core1", "ping", "pong", "init",
-                 "x_slot", "h_slot", "at_h", "at_p", "p_slot", "at_dy", "dy_buf", "launches")
+                 "x_slot", "h_slot", "at_h", "at_p", "p_slot", "at_dy", "dy_buf", "launches", "parts")
 
 
 def mebptt_test_schedule(desc, plan, room: int = 0):
     """(info, records [n, 32] of bytes, launches [n, 4]) of a walked tape."""
-    info = (_i64 * 19)()
+    info = (_i64 * 20)()
     n = lib.mebptt_test_schedule(C.byref(desc), plan.handle, room, info, None, 0, None, 0)
     if n < 0:
         raise MebpttError(MEBPTT_ERR_UNSUPPORTED, "mebptt_test_schedule")

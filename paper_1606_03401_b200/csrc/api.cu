@@ -816,7 +816,7 @@ int64_t mebptt_test_schedule(const mebptt_lstm_desc* desc, const mebptt_plan_t* 
   const int64_t v[16] = {r.pod, y.S, (int64_t)y.tape_bytes / 32, y.unit_blocks, y.loc_blocks, y.n_blocks, y.blk_core[0], y.blk_core[1], y.blk_ping, y.blk_pong,
                          y.blk_init, r.pc.x_slot, r.pc.h_slot, r.pc.at_h, r.pc.at_p, r.pc.p_slot};
   memcpy(info, v, sizeof v);
-  info[16] = r.pc.at_dy; info[17] = r.pc.dy_buf;
+  info[16] = r.pc.at_dy; info[17] = r.pc.dy_buf; info[19] = y.parts;
   const int64_t n = (int64_t)rec.bytes.size() / 32;
   if (records) memcpy(records, rec.bytes.data(), (size_t)(n < most_records ? n : most_records) * 32);
   info[18] = (int64_t)rec.launches.size();

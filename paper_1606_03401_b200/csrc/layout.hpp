@@ -26,10 +26,15 @@ inline size_t gcd_sz(size_t a, size_t b) { while (b) { size_t r = a % b; a = b; 
 struct Layout;
 namespace team {
 bool supported(const mebptt_lstm_desc* d);
-// elements of the packed weights, in the order of the kernel that serves the problem (wb: 0 where one copy
-// serves both directions)
-struct PackedSizes { size_t wf[16], wb[16], wr; };
-PackedSizes packed_sizes(const Layout& y);
+// what the kernel that serves the problem wants: elements of the packed weights in its order (wb: 0 where one
+// copy serves both directions), batch rows of a group
+struct Wants { size_t wf[16], wb[16], wr; int rows; };
+Wants wants(const Layout& y);
+// bytes of a block of a group of `rows` batch rows: its parts start at multiples of 16 bytes
+inline size_t block_bytes(int rows, int H, size_t esz, int parts) {
+  const size_t a = (size_t)16 * parts;
+  return ((size_t)rows * H * esz + a - 1) / a * a;
+}
 constexpr size_t kMaxLaunchTasks = 32768;   // 1 MB of tasks per launch at most: what the workspace holds at a time
 }
 
@@ -80,8 +85,10 @@ struct Layout {
   size_t off_a3_run = 0, off_zrun = 0, off_hrun = 0, off_dha_run = 0, off_zleaf3 = 0, off_leaf = 0, split_floats = 0;
   size_t n_sync = 0, tape_bytes = 0;
   // team path: states per group of batch rows, in blocks of one layer's h of the group (a cell state takes
-  // 4 / esz of them): blocks of a location's unit, of a hidden state, of all states; first blocks of the named states
-  int loc_blocks = 0, unit_blocks = 0;
+  // 4 / esz of them).  Where a plan's unit is no whole number of blocks, addresses count parts of a block
+  // (`parts` to a block): parts of a location's unit, blocks of a hidden state; parts of all states; first parts
+  // of the named states
+  int loc_blocks = 0, unit_blocks = 0, parts = 1;
   int64_t n_blocks = 0, blk_core[2] = {}, blk_ping = 0, blk_pong = 0, blk_init = 0;
   // packed weights per layer, readout weights, dz of the step after a chunk, end of what a step clears
   size_t off_wf[16] = {}, off_wb[16] = {}, off_wr = 0, off_carry = 0, off_zero_end = 0;
@@ -276,8 +283,7 @@ inline std::vector<int> projection_windows(const std::vector<WorkItem>& items, c
 // packed weights are then done without)
 inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y, bool compact = false) {
   state_layout(d, y);
-  // (plans over byte sizes that are no whole blocks of the team path's states go without it)
-  y.team = !compact && (p->sigma <= 1 || (y.L * (1 + (int)(4 / y.esz))) % p->sigma == 0) && team::supported(d);
+  y.team = !compact && team::supported(d);
   if (y.team) y.stepwise_tc = y.stepwise_x3 = y.x3_runs = false;
   y.arena_units = p->arena_units;
   y.loc_bytes = y.unit / (size_t)(p->sigma > 0 ? p->sigma : 1);
@@ -297,27 +303,28 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     const size_t rows = (size_t)y.S * y.B;
     // States: a group of batch rows walks the tape without waiting for the others, so each has an arena of
     // its own -- in one arena for all rows what one group writes for a later operation would lie over another
-    // group's rows of an earlier one.  Sizes are those of the common layout but for the rounding of rows to
-    // 16 bytes.  The working core alternates between two buffers, so that one leaf's forward operation can
+    // group's rows of an earlier one.  Sizes are those of the common layout without its rounding to granules.  The working core alternates between two buffers, so that one leaf's forward operation can
     // pass the last one's backward.
     const int cr = (int)(4 / y.esz);
     y.unit_blocks = y.L * (1 + cr);
-    const int rec_blocks = 2 * y.unit_blocks + 4 * y.L;
-    y.loc_blocks = y.unit_blocks / (p->sigma > 0 ? p->sigma : 1);
+    const int rec_blocks = 2 * y.unit_blocks + 4 * y.L, sigma = p->sigma > 0 ? p->sigma : 1;
+    y.parts = sigma / (int)gcd_sz((size_t)sigma, (size_t)y.unit_blocks);
+    y.loc_blocks = y.unit_blocks * y.parts / sigma;
     int64_t blocks = y.arena_units * y.loc_blocks;
-    auto named = [&](int64_t n) { const int64_t r = blocks; blocks += n; return r; };
+    auto named = [&](int64_t n) { const int64_t r = blocks; blocks += n * y.parts; return r; };
     y.blk_core[0] = named(rec_blocks); y.blk_core[1] = named(rec_blocks);
     y.blk_ping = named(y.unit_blocks); y.blk_pong = named(y.unit_blocks); y.blk_init = named(y.unit_blocks);
     y.n_blocks = blocks;
-    const size_t states = (size_t)blocks * y.B * align_up((size_t)y.H * y.esz + 15, 16);
+    const team::Wants want = team::wants(y);
+    const size_t part = team::block_bytes(want.rows, y.H, y.esz, y.parts) / y.parts;
+    const size_t states = (size_t)blocks * part * (((size_t)y.B + want.rows - 1) / want.rows);
     if (o < y.off_arena + states) o = align_up(y.off_arena + states, y.granule);
     y.off_loss_t = take((size_t)y.t * 4);
-    const team::PackedSizes packed = team::packed_sizes(y);
     for (int l = 0; l < y.L; ++l) {
-      y.off_wf[l] = take(packed.wf[l] * y.esz);
-      y.off_wb[l] = take(packed.wb[l] * y.esz);
+      y.off_wf[l] = take(want.wf[l] * y.esz);
+      y.off_wb[l] = take(want.wb[l] * y.esz);
     }
-    y.off_wr = take(packed.wr * y.esz);
+    y.off_wr = take(want.wr * y.esz);
     y.off_st_dz = y.off_dz = take((size_t)y.L * rows * G * 4);
     // h of the chunk's steps and of the one before: row block i holds h_{k-1} of the step in block i of dz
     y.off_st_h = take((size_t)y.L * (rows + y.B) * y.H * y.esz);

@@ -286,7 +286,7 @@ __device__ __forceinline__ void put_planes(bf16* p, int stride, float v) {
   }
 }
 
-// WIDE: a pod's states pass 4 GB.  The sums are the same.
+// WIDE: a pod's states pass 4 GB, or locations count parts of a block.  The sums are the same.
 template <class T, bool GRU, int NB, int PL, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ Args A) {
   constexpr bool MMA = std::is_same<T, bf16>::value;
@@ -353,8 +353,8 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   // offsets of this element: h, c and gates from the pod's states, dz and h stages and carried dz from the start
   // of the stages (under 4 GB by the rule of choose_config)
   using St = States<T>;
-  const St S(A.ws + A.off_states, A.n_blocks, pod, NB, A.B, H);
-  const uint32_t le = eb * H + ej, hs_ = S.hs;
+  const St S(A.ws + A.off_states, A.n_blocks, WIDE ? A.parts : 1, pod, NB, A.B, H);
+  const uint32_t le = eb * H + ej, hs_ = S.hs, part_ = S.part;
   const uint32_t o_h = lay * (1 + St::CR) * hs_ + le * (uint32_t)sizeof(T), o_c = (lay * (1 + St::CR) + 1) * hs_ + le * 4;
   const uint32_t o_g = (L * (1 + St::CR) + 4 * lay) * hs_ + le * (uint32_t)sizeof(T), o_in = (L * (1 + St::CR) + 4 * L) * hs_;
   const uint32_t bh = (uint32_t)A.B * H;                         // elements of a row block of the h stage, a quarter of those of dz
@@ -410,10 +410,11 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   float om[7];
   float ol = 0.f, o_target = 0.f;
   float4 ox = make_float4(0.f, 0.f, 0.f, 0.f), oz = ox;
-  // The states of a generous budget pass 4 GB.  Below that an offset of 32 bits from a base that is the same for
-  // all threads takes no instruction to add; with 64 bits throughout, the two-layer GRU of 256 units took 1 %
-  // longer (2864 -> 2891 us).
-  auto at = [&](uint32_t o, uint32_t loc) { return WIDE ? S.base + (uint64_t)loc * hs_ + o : S.base + (o + loc * hs_); };
+  // The states of a generous budget pass 4 GB, and a plan over byte sizes counts in parts of a block.  Where
+  // neither is so, an offset of 32 bits from a base that is the same for all threads takes no instruction to
+  // add; with 64 bits throughout, the two-layer GRU of 256 units took 1 % longer (2864 -> 2891 us), with parts
+  // 0.4 % more.
+  auto at = [&](uint32_t o, uint32_t loc) { return WIDE ? S.base + (uint64_t)loc * part_ + o : S.base + (o + loc * part_); };
   // h0: n cells sums n_h | n_p n_x r x | products - | main     h1: load carry bwd -
   auto ahead = [&](int cur, const uint4& h0, const uint4& h1) {
     if (warp_s) {
@@ -671,7 +672,7 @@ __global__ void __launch_bounds__(256) pod_pack(const __grid_constant__ PackArgs
   for (int l = 0; l < L; ++l)
     for (size_t i = first; i < bh; i += all) {
       const int b = (int)(i / H), g = b / C.nb;
-      const States<T> S(P.states, P.n_blocks, g, C.nb, P.B, H);
+      const States<T> S(P.states, P.n_blocks, P.parts, g, C.nb, P.B, H);
       const size_t le = i - (size_t)g * C.nb * H;
       S.h((uint32_t)P.init, l)[le] = reinterpret_cast<const T*>(P.h0)[l * bh + i];
       S.c((uint32_t)P.init, l)[le] = P.c0[l * bh + i];

@@ -163,7 +163,7 @@ struct Builder {
   int units(int32_t loc, int fmt) const {
     if (loc < 0) return 1;
     const int blocks = fmt == MEBPTT_FMT_HIDDEN ? y.unit_blocks : y.unit_blocks + 4 * y.L + (fmt == MEBPTT_FMT_INTERNAL ? y.unit_blocks : 0);
-    return (blocks + y.loc_blocks - 1) / y.loc_blocks;
+    return (blocks * y.parts + y.loc_blocks - 1) / y.loc_blocks;
   }
   template <class F> void cells(int32_t loc, int n, int l, F f) {
     if (loc >= 0) { for (int i = 0; i < n && (size_t)(loc + i) < cell.size(); ++i) f(cell[(size_t)(loc + i)]); }
@@ -243,7 +243,7 @@ struct Builder {
       // its shares for the layer below take the place of those of step k + 2
       if (l > 0) after = std::max(after, b_phase[(size_t)(l - 1) * 4 + ((q + 2) & 3)]);
       if (op.dst_fmt == MEBPTT_FMT_INTERNAL) {
-        b.t.dst = b.t.src + (uint32_t)(y.unit_blocks + 4 * y.L);
+        b.t.dst = b.t.src + (uint32_t)((y.unit_blocks + 4 * y.L) * y.parts);
       } else {
         b.t.dst = address(op.aux);
         after = std::max(after, state[slot_of(op.aux) * L + l]);

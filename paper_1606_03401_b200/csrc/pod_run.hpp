@@ -16,6 +16,7 @@ struct Args {
   Config c;
   size_t off_states;                   // states, by pod
   int64_t n_blocks;
+  int parts;
   char* ws;
   size_t off_wf[team::kMaxLayers], off_wr;
   size_t off_dz, off_hk, off_dy, off_carry, off_dc;
@@ -29,7 +30,7 @@ struct Args {
 };
 
 using Fn = void (*)(const Args);
-// wide: the states of a pod pass 4 GB
+// wide: the states of a pod pass 4 GB, or locations count parts of a block
 Fn kernel(int dtype, bool gru, int nb, bool wide);
 
 // Packs the weights in the order the kernel keeps them, lays the initial state out, clears what a step
@@ -41,6 +42,7 @@ struct PackArgs {
   const float* c0;
   char *wf[kMaxLayers], *wr, *states;  // the initial state goes to block `init` of each pod's states
   int64_t n_blocks, init;
+  int parts;
   size_t w_off[kMaxLayers];
   float* zero;
   size_t n_zero;

@@ -41,6 +41,7 @@ struct Args {
   int pool_floats;
   size_t off_states;                   // states, by team
   int64_t n_blocks;
+  int parts;
   char* ws;
   size_t off_wf[kMaxLayers], off_wb[kMaxLayers], off_wr;
   size_t off_dz, off_hk, off_dy, off_carry, off_dc;
@@ -189,7 +190,7 @@ __device__ __forceinline__ void apply(const Args& A, const States<T>& S, const T
       for (int q = 0; q < 4; ++q) store(S.gate(t.dst, A.L, l, q) + le, gv[q]);
     }
     if (t.flags & COPY_IN) {
-      const uint32_t in = States<T>::input(t.dst, A.L);
+      const uint32_t in = S.input(t.dst, A.L);
       store(S.h(in, l) + le, GRU ? cp : o.v[5]);
       if (!GRU) S.c(in, l)[le] = cp;
     }
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1) walk(const __grid_constant__ Args
   const int team = blockIdx.x / A.T, rank = blockIdx.x - team * A.T;
   const int H = A.H, L = A.L;
   const int row0 = team * A.rows, rows = min(A.rows, A.B - row0);
-  const States<T> S(A.ws + A.off_states, A.n_blocks, team, A.rows, A.B, H);
+  const States<T> S(A.ws + A.off_states, A.n_blocks, A.parts, team, A.rows, A.B, H);
   if (tid == 0) s_flag = *A.status;   // an earlier launch gave up: do nothing
   int f0, f1, b0, b1, r0g, r1g;       // groups of this CTA
   part(A.d.gf, A.T, rank, f0, f1);
@@ -461,7 +462,7 @@ struct PackArgs {
   const T *W, *W_out;
   size_t w_off[kMaxLayers];
   T *wf[kMaxLayers], *wb[kMaxLayers], *wr;
-  char* states; int64_t n_blocks, init; int R;   // the caller's initial state goes to block `init` of each group's states
+  char* states; int64_t n_blocks, init; int parts, R;   // the caller's initial state goes to block `init` of each group's states
   const void* h0; const float* c0;
   int B;
   float* zero; size_t n_zero;     // carried gradients, sync lines, status
@@ -488,7 +489,7 @@ __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
   for (int l = 0; l < P.L; ++l)
     for (size_t i = blockIdx.x * 256 + threadIdx.x; i < bh; i += (size_t)gridDim.x * 256) {
       const int b = (int)(i / H), g = b / P.R;
-      const States<T> S(P.states, P.n_blocks, g, P.R, P.B, H);
+      const States<T> S(P.states, P.n_blocks, P.parts, g, P.R, P.B, H);
       const size_t le = i - (size_t)g * P.R * H;
       S.h((uint32_t)P.init, l)[le] = reinterpret_cast<const T*>(P.h0)[l * bh + i];
       S.c((uint32_t)P.init, l)[le] = P.c0[l * bh + i];
@@ -982,7 +983,7 @@ void launch_pack(const Layout& y, const Dims& d, int rows, const tc::StepPtrs& i
     P.wb[l] = reinterpret_cast<T*>(io.ws + y.off_wb[l]);
   }
   P.wr = reinterpret_cast<T*>(io.ws + y.off_wr);
-  P.states = io.ws + y.off_arena; P.n_blocks = y.n_blocks; P.init = y.blk_init; P.R = rows; P.h0 = io.h0; P.c0 = io.c0; P.B = y.B;
+  P.states = io.ws + y.off_arena; P.n_blocks = y.n_blocks; P.parts = y.parts; P.init = y.blk_init; P.R = rows; P.h0 = io.h0; P.c0 = io.c0; P.B = y.B;
   P.zero = reinterpret_cast<float*>(io.ws + y.off_dc);
   P.n_zero = (y.off_zero_end - y.off_dc) / 4;
   P.counters = io.counters;
@@ -1049,7 +1050,7 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.c = pc;
     q.W = io.W; q.W_out = io.W_out; q.h0 = io.h0; q.c0 = io.c0;
     for (int l = 0; l < y.L; ++l) { q.wf[l] = io.ws + y.off_wf[l]; q.w_off[l] = y.w_layer_offset(l); }
-    q.wr = io.ws + y.off_wr; q.states = io.ws + y.off_arena; q.n_blocks = y.n_blocks; q.init = y.blk_init;
+    q.wr = io.ws + y.off_wr; q.states = io.ws + y.off_arena; q.n_blocks = y.n_blocks; q.parts = y.parts; q.init = y.blk_init;
     q.zero = reinterpret_cast<float*>(io.ws + y.off_dc); q.n_zero = (y.off_zero_end - y.off_dc) / 4;
     q.counters = io.counters;
     pod::launch_pack(y.dtype, y.gru, q, s);
@@ -1067,7 +1068,7 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     q.L = y.L; q.I = y.I; q.H = y.H; q.O = y.O; q.B = y.B; q.S = y.S;
     for (int l = 0; l < y.L; ++l) q.off_wf[l] = y.off_wf[l];
     q.off_wr = y.off_wr;
-    q.off_states = y.off_arena; q.n_blocks = y.n_blocks;
+    q.off_states = y.off_arena; q.n_blocks = y.n_blocks; q.parts = y.parts;
     q.ws = io.ws;
     q.off_dz = y.off_dz; q.off_hk = y.off_st_h; q.off_dy = y.off_dy; q.off_carry = y.off_carry; q.off_dc = y.off_dc;
     q.x = io.x; q.bias = io.b; q.b_out = io.b_out; q.targets = io.targets;
@@ -1078,8 +1079,8 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     common(pa);
     pa.stages = io.ws + y.off_dz;
     pa.c = pc;
-    const size_t states = (size_t)y.n_blocks * align_up((size_t)pc.nb * y.H * y.esz, 16);
-    pf = pod::kernel(y.dtype, y.gru, pc.nb, states >> 32 != 0);
+    const size_t states = (size_t)y.n_blocks * (block_bytes(pc.nb, y.H, y.esz, y.parts) / y.parts);
+    pf = pod::kernel(y.dtype, y.gru, pc.nb, states >> 32 != 0 || y.parts > 1);
     if (allow(reinterpret_cast<const void*>(pf)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
   } else {
     common(a);

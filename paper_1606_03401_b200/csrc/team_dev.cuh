@@ -49,20 +49,26 @@ __device__ __forceinline__ float lane_sums(float (&v)[N], int lane) {
 
 // The states of one group of batch rows (row R i and on, of group i): blocks of `hs` bytes -- one layer's h
 // of the group -- with a cell state in the CR blocks behind its h, layer after layer, then four gate blocks a
-// layer, then the input state.
+// layer, then the input state.  Locations count parts of a block, `parts` to a block.
 template <class T>
 struct States {
   static constexpr int CR = (int)(4 / sizeof(T));
   char* base;
-  uint32_t hs;
-  __host__ __device__ static uint32_t block(int rows, int H) { return ((uint32_t)rows * H * (uint32_t)sizeof(T) + 15) & ~15u; }
-  __host__ __device__ States(char* all, int64_t blocks, int group, int R, int B, int H)
-      : base(all + (size_t)group * blocks * block(R, H)), hs(block(R < B - group * R ? R : B - group * R, H)) {}
-  __host__ __device__ char* at(uint32_t block) const { return base + (size_t)block * hs; }
-  __host__ __device__ T* h(uint32_t loc, int l) const { return reinterpret_cast<T*>(at(loc + l * (1 + CR))); }
-  __host__ __device__ float* c(uint32_t loc, int l) const { return reinterpret_cast<float*>(at(loc + l * (1 + CR) + 1)); }
-  __host__ __device__ T* gate(uint32_t loc, int L, int l, int q) const { return reinterpret_cast<T*>(at(loc + L * (1 + CR) + 4 * l + q)); }
-  __host__ __device__ static uint32_t input(uint32_t loc, int L) { return loc + L * (1 + CR) + 4 * L; }
+  uint32_t hs, part;
+  int parts;
+  __host__ __device__ static uint32_t block(int rows, int H, int parts) {
+    const uint32_t a = 16 * (uint32_t)parts;
+    return ((uint32_t)rows * H * (uint32_t)sizeof(T) + a - 1) / a * a;
+  }
+  // n: parts of a group's states
+  __host__ __device__ States(char* all, int64_t n, int parts_, int group, int R, int B, int H)
+      : base(all + (size_t)group * n * (block(R, H, parts_) / parts_)), hs(block(R < B - group * R ? R : B - group * R, H, parts_)), part(hs / parts_),
+        parts(parts_) {}
+  __host__ __device__ char* at(uint32_t loc, int blocks) const { return base + (size_t)loc * part + (size_t)blocks * hs; }
+  __host__ __device__ T* h(uint32_t loc, int l) const { return reinterpret_cast<T*>(at(loc, l * (1 + CR))); }
+  __host__ __device__ float* c(uint32_t loc, int l) const { return reinterpret_cast<float*>(at(loc, l * (1 + CR) + 1)); }
+  __host__ __device__ T* gate(uint32_t loc, int L, int l, int q) const { return reinterpret_cast<T*>(at(loc, L * (1 + CR) + 4 * l + q)); }
+  __host__ __device__ uint32_t input(uint32_t loc, int L) const { return loc + (L * (1 + CR) + 4 * L) * parts; }
 };
 
 __device__ __forceinline__ void part(int n, int T, int r, int& lo, int& hi) {   // CTA r's share of n things

@@ -161,12 +161,13 @@ Route route(const Layout& y) {
   return r;
 }
 
-PackedSizes packed_sizes(const Layout& y) {
-  PackedSizes s{};
+Wants wants(const Layout& y) {
+  Wants s{};
   const Route r = route(y);
   if (r.pod) {
     for (int l = 0; l < y.L; ++l) s.wf[l] = pod::packed_elems(r.pc, l);
     s.wr = pod::packed_readout_elems(r.pc);
+    s.rows = r.pc.nb;
   } else {
     const Dims d = dims(y);
     for (int l = 0; l < y.L; ++l) {
@@ -174,6 +175,7 @@ PackedSizes packed_sizes(const Layout& y) {
       s.wb[l] = (size_t)d.gb * d.rpg * d.kb[l];
     }
     s.wr = (size_t)d.gr * d.rpg * d.hp;
+    s.rows = r.c.rows;
   }
   return s;
 }
@@ -221,7 +223,7 @@ struct Scheduler {
   int units(int32_t loc, int fmt) const {   // cells a record takes
     if (loc < 0) return 1;
     const int blocks = fmt == MEBPTT_FMT_HIDDEN ? y.unit_blocks : y.unit_blocks + 4 * y.L + (fmt == MEBPTT_FMT_INTERNAL ? y.unit_blocks : 0);
-    return (blocks + y.loc_blocks - 1) / y.loc_blocks;
+    return (blocks * y.parts + y.loc_blocks - 1) / y.loc_blocks;
   }
   template <class F> void cells(int32_t loc, int n, int l, F f) {
     if (loc >= 0) { for (int i = 0; i < n && (size_t)(loc + i) < cell.size(); ++i) f(cell[(size_t)(loc + i)]); }
@@ -320,7 +322,7 @@ struct Scheduler {
       b.src = address(op.src);
       int64_t after = std::max(std::max(in[l], above), bwd_prev[(size_t)l]);
       if (op.dst_fmt == MEBPTT_FMT_INTERNAL) {
-        b.dst = b.src + (uint32_t)(y.unit_blocks + 4 * y.L);
+        b.dst = b.src + (uint32_t)((y.unit_blocks + 4 * y.L) * y.parts);
       } else {
         b.dst = address(op.aux);
         after = std::max(after, state_of(op.aux)[l]);

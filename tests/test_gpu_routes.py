@@ -70,3 +70,26 @@ def test_states_past_4_gib_take_the_same_kernels_and_give_the_same_bits(size, al
     got = dp.run(full)
     assert got["counters"][0] == cfg.t and got["counters"][3] == 0 and want["counters"][3] == 0
     assert_bit_identical(got, want, want_dx=True)
+
+
+@pytest.mark.parametrize("size,gru,sigma,route", [
+    (dict(layers=2, input=161, hidden=300, batch=40, t=24, readout=29), False, 5, "teams"),
+    (dict(layers=1, input=16, hidden=200, batch=40, t=30, readout=8), True, 2, "pods"),
+    (dict(layers=2, input=16, hidden=100, batch=40, t=30, readout=8), True, 5, "pods"),
+    (dict(layers=3, input=16, hidden=64, batch=9, t=40, readout=8), False, 7, "pods"),
+    (dict(layers=3, input=16, hidden=200, batch=40, t=20, readout=8), True, 2, "teams"),
+])
+def test_plans_in_fractions_of_a_hidden_state_give_the_bits_of_other_plans(size, gru, sigma, route):
+    """Locations of such a plan are no whole blocks of a group's states."""
+    from paper_1606_03401_b200 import binding as B
+    from paper_1606_03401_b200 import harness as H
+    cfg = synth.with_overrides(synth.CONFIGS["c1"], dtype="bf16", **size, **({"cell": "gru"} if gru else {}))
+    dp = H.DeviceProblem(cfg, want_dx=True)
+    full = dp.run(dp.full_memory_plan())
+    for units in (4, 11):
+        for use_beta in (False, True):
+            plan = B.mebptt_plan_bytes_exact(dp.desc, units * B.mebptt_lstm_unit_bytes(dp.desc), use_beta)
+            assert plan.sigma == sigma and B.mebptt_test_route(dp.desc, plan)["route"] == route
+            res = dp.run(plan)
+            assert res["counters"][0] == plan.cost and res["counters"][1] == cfg.t and res["counters"][3] == 0
+            assert_bit_identical(res, full, want_dx=True)

@@ -51,3 +51,19 @@ def test_no_launch_has_more_records_than_there_is_room_for(size, mode, m):
         if not info["pods"]:      # (a pod's headers are records of another kind: replayed elsewhere)
             kinds = records[:, 0]
             assert (kinds == 1).sum() == plan.cost * layers and (kinds == 3).sum() == size[5] * layers
+
+
+@pytest.mark.parametrize("dtype,gru", [("fp32", False), ("bf16", False), ("bf16", True)])
+def test_plans_over_byte_sizes_take_the_kernels_of_other_plans(dtype, gru):
+    """The unit of such a plan is any fraction of a hidden state (seventh parts among these)."""
+    sigmas = set()
+    plan = B.mebptt_plan(20, 5, B.MEBPTT_HSM)
+    for layers in (1, 2, 3):
+        for hidden in (20, 64, 100, 200, 300):
+            for batch in (1, 5, 9, 20, 40, 48):
+                desc = _problem((layers, 16, hidden, 8, batch, 20, dtype, gru))
+                exact = B.mebptt_plan_bytes_exact(desc, 12 * B.mebptt_lstm_unit_bytes(desc))
+                want, got = B.mebptt_test_route(desc, plan), B.mebptt_test_route(desc, exact)
+                assert got == want and want["route"] in ("pods", "teams", "persistent"), (layers, hidden, batch)
+                sigmas.add(exact.sigma)
+    assert dtype == "fp32" or {2, 3, 5, 7} <= sigmas

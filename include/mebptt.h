@@ -258,7 +258,14 @@ int64_t mebptt_budget_bytes_to_units(const mebptt_lstm_desc *desc, size_t bytes)
  *                        m is taken for which mebptt_lstm_workspace_bytes of the resulting plan
  *                        still fits.  (Appendix C notes that the working memory has to be part
  *                        of the allowance once it is not negligible; here it is not: staging for
- *                        a chunk of time steps, packed weights.)
+ *                        a chunk of time steps, packed weights.)  Where a whole tape is walked by
+ *                        one kernel (float32, GRU and ragged problems) the plan carries how much of
+ *                        it a step takes: chunks are made shorter until the working memory is half
+ *                        of the budget, with the same kernels and bits; and where the shortest leave
+ *                        less than an eighth of the budget for the states, the plan is marked to do
+ *                        without stages and packed weights: its step runs operation by operation
+ *                        (some 15 times slower), and its results agree with those of other plans to
+ *                        rounding only, not to the bit.
  * MEBPTT_ERR_BUDGET if not even m = 1 fits.  *out as for mebptt_plan.
  */
 int mebptt_plan_for_bytes(const mebptt_lstm_desc *desc, size_t budget_bytes, int mode, int include_working,
@@ -311,7 +318,9 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc *desc, const mebptt_plan
  *   [4..7] reserved.  counters[0] equals mebptt_plan_cost(plan) after a successful step.
  * Determinism: no atomics; for a fixed descriptor and inputs every plan yields bit-identical
  *   outputs (each backward step sees bit-identical internal states whether they were stored
- *   or recomputed, and all accumulations run in the order t .. 1).
+ *   or recomputed, and all accumulations run in the order t .. 1).  One exception, on request: a plan
+ *   made for a whole-device budget too small for the staging (mebptt_plan_for_bytes) runs on other
+ *   kernels; all such plans of a problem again agree to the bit among themselves.
  * Returns MEBPTT_OK once everything is enqueued, or an error with nothing enqueued.
  */
 int mebptt_lstm_train_step(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan,
@@ -352,7 +361,8 @@ int mebptt_lstm_train_step_host(const mebptt_lstm_desc *desc, const mebptt_plan_
  *   mebptt_plan_bytes_exact(desc, bytes, use_beta, include_working)  takes as the unit the
  *       greatest common divisor of the byte sizes of the three kinds of state in desc's layout
  *       (config 5: 1 MiB, sizes 3 : 10 : 7), converts the byte budget and plans as above; with
- *       include_working the budget covers the whole device workspace, as in mebptt_plan_for_bytes.
+ *       include_working the budget covers the whole device workspace, as in mebptt_plan_for_bytes
+ *       (what is said there of small budgets holds here too).
  *   mebptt_plan_sigma  the sigma of a plan (1 for every other constructor).
  *
  * A plan can be executed with a descriptor whose layout fits its sizes (checked; else
@@ -395,7 +405,10 @@ int mebptt_lstm_prepare_stats(int64_t *out);
  * no stream or event.
  *
  *   - Problems whose workspace (mebptt_lstm_workspace_bytes) exceeds the array are refused with
- *     MEBPTT_ERR_WORKSPACE and nothing is enqueued; use mebptt_lstm_train_step for those.
+ *     MEBPTT_ERR_WORKSPACE and nothing is enqueued; use mebptt_lstm_train_step for those.  Where a
+ *     whole tape is walked by one kernel, smaller workspaces are tried first: shorter chunks, with
+ *     the bits of the ordinary entry point, and at last the operation-by-operation kernels of
+ *     mebptt_plan_for_bytes, whose results agree with it to rounding only.
  *   - The first call on each device is a set-up call: it looks up the array's device address
  *     (with that device current).  With CUDA's default lazy module loading that look-up is also
  *     the moment the driver places the array -- and, at their first launch, the code of the

@@ -494,6 +494,52 @@ void staging_layout(const Layout& y, bool want_dx, size_t base, Staging& g) {
   g.total = o;
 }
 
+// The plan with the largest m, in units of `unit` bytes and at least `least`, that a budget holds: the states alone,
+// or the whole workspace.  For the latter the footprint is settled first: the longest chunks whose working memory
+// takes no more than half of the budget, else the shortest, and without any if an eighth is not left for the
+// states (a policy with next to none recomputes so much that the slower kernels are ahead).
+template <class Make>
+int plan_in(const mebptt_lstm_desc* desc, size_t budget, size_t unit, int64_t least, bool whole, Make make, mebptt_plan_t** out) {
+  const int64_t most = (int64_t)(budget / unit);
+  if (most < least) return MEBPTT_ERR_BUDGET;
+  Plan* plan = nullptr;
+  int rc = make(most, &plan);
+  if (rc != MEBPTT_OK) return rc;
+  mebptt_plan_t* const handle = reinterpret_cast<mebptt_plan_t*>(plan);
+  if (!whole) { *out = handle; return MEBPTT_OK; }
+  const std::vector<Footprint> all = footprints(desc, Footprint{});
+  size_t first = 0;
+  for (; first + 1 < all.size(); ++first) {
+    plan->footprint = all[first];
+    const size_t working = mebptt_lstm_working_bytes(desc, handle);
+    if (working <= (first + 2 < all.size() ? budget / 2 : budget - budget / 8)) break;
+  }
+  for (size_t i = first; i < all.size(); ++i) {
+    int64_t m = most;
+    for (int round = 0; round < 64 && m >= least; ++round) {
+      if (!plan) {
+        rc = make(m, &plan);
+        if (rc == MEBPTT_ERR_BUDGET) break;
+        if (rc != MEBPTT_OK) return rc;
+      }
+      plan->footprint = all[i];
+      const size_t need = mebptt_lstm_workspace_bytes(desc, reinterpret_cast<mebptt_plan_t*>(plan));
+      if (need != 0 && need <= budget) { *out = reinterpret_cast<mebptt_plan_t*>(plan); return MEBPTT_OK; }
+      // too large by `need - budget`: give up that many units (the working memory changes little with m,
+      // so this lands on or just above the answer; the loop settles the rest).  A budget above the
+      // mode's saturation point was clamped by the planner: go on from there.
+      const int64_t m_used = plan->m;
+      mebptt_plan_free(reinterpret_cast<mebptt_plan_t*>(plan));
+      plan = nullptr;
+      if (need == 0) return MEBPTT_ERR_UNSUPPORTED;
+      const int64_t drop = (int64_t)((need - budget + unit - 1) / unit);
+      m = (m_used < m ? m_used : m) - (drop > 0 ? drop : 1);
+    }
+  }
+  if (plan) mebptt_plan_free(reinterpret_cast<mebptt_plan_t*>(plan));
+  return MEBPTT_ERR_BUDGET;
+}
+
 }  // namespace
 
 extern "C" {
@@ -517,24 +563,8 @@ int mebptt_plan_for_bytes(const mebptt_lstm_desc* desc, size_t budget_bytes, int
   const size_t unit = mebptt_lstm_unit_bytes(desc);
   if (!unit) return MEBPTT_ERR_ARG;
   const size_t per_m = (mode == MEBPTT_ISM) ? 4 * unit : unit;   // what one more of the mode's units costs
-  int64_t m = (int64_t)(budget_bytes / per_m);
-  for (int round = 0; round < 64 && m >= 1; ++round) {
-    mebptt_plan_t* plan = nullptr;
-    const int rc = mebptt_plan(desc->t, m, mode, &plan);
-    if (rc != MEBPTT_OK) return rc;
-    if (!include_working) { *out = plan; return MEBPTT_OK; }
-    const size_t need = mebptt_lstm_workspace_bytes(desc, plan);
-    if (need == 0) { mebptt_plan_free(plan); return MEBPTT_ERR_UNSUPPORTED; }
-    if (need <= budget_bytes) { *out = plan; return MEBPTT_OK; }
-    // too large by `need - budget_bytes`: give up that many units (the working memory changes
-    // little with m, so this lands on or just above the answer; the loop settles the rest).
-    // A budget above the mode's saturation point was clamped by the planner: go on from there.
-    const int64_t m_used = mebptt_plan_m(plan);
-    mebptt_plan_free(plan);
-    const int64_t drop = (int64_t)((need - budget_bytes + per_m - 1) / per_m);
-    m = (m_used < m ? m_used : m) - (drop > 0 ? drop : 1);
-  }
-  return MEBPTT_ERR_BUDGET;
+  return plan_in(desc, budget_bytes, per_m, 1, include_working != 0,
+                 [&](int64_t m, Plan** plan) { return build_plan(desc->t, m, mode, 4, 0, plan); }, out);
 }
 
 int mebptt_plan_bytes_exact(const mebptt_lstm_desc* desc, size_t budget_bytes, int use_beta, int include_working,
@@ -549,21 +579,8 @@ int mebptt_plan_bytes_exact(const mebptt_lstm_desc* desc, size_t budget_bytes, i
   const size_t f = gcd_sz(gcd_sz(y.unit, y.rec), rec_short);
   const int sigma = (int)(y.unit / f), alpha = (int)(y.rec / f), beta = use_beta ? (int)(rec_short / f) : 0;
   if (sigma > 64) return MEBPTT_ERR_UNSUPPORTED;
-  int64_t m = (int64_t)(budget_bytes / f);
-  for (int round = 0; round < 64 && m >= sigma; ++round) {
-    mebptt_plan_t* plan = nullptr;
-    const int rc = mebptt_plan_sized(desc->t, m, sigma, alpha, beta, &plan);
-    if (rc != MEBPTT_OK) return rc;
-    if (!include_working) { *out = plan; return MEBPTT_OK; }
-    const size_t need = mebptt_lstm_workspace_bytes(desc, plan);
-    if (need == 0) { mebptt_plan_free(plan); return MEBPTT_ERR_UNSUPPORTED; }
-    if (need <= budget_bytes) { *out = plan; return MEBPTT_OK; }
-    const int64_t m_used = mebptt_plan_m(plan);
-    mebptt_plan_free(plan);
-    const int64_t drop = (int64_t)((need - budget_bytes + f - 1) / f);
-    m = (m_used < m ? m_used : m) - (drop > 0 ? drop : 1);
-  }
-  return MEBPTT_ERR_BUDGET;
+  return plan_in(desc, budget_bytes, f, sigma, include_working != 0,
+                 [&](int64_t m, Plan** plan) { return build_plan(desc->t, m, MEBPTT_MSM, alpha, beta, plan, sigma); }, out);
 }
 
 size_t mebptt_lstm_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
@@ -657,11 +674,21 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
 }  // extern "C"
 
 namespace mebptt {
-size_t least_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
+// The plan's layout, or, in a fixed workspace that is too small for it, the largest of the smaller ones that fits.
+// 0 on a bad descriptor or plan, else what the chosen one (or the least, if none fits) takes.
+size_t fitted_layout(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, size_t bytes, Layout& y) {
   if (check_common(desc, plan) != MEBPTT_OK) return 0;
+  const Plan* p = reinterpret_cast<const Plan*>(plan);
+  for (const Footprint& s : footprints(desc, p->footprint)) {
+    workspace_layout(desc, p, y, s);
+    if (!addressable(y)) return 0;
+    if (y.total <= bytes) break;
+  }
+  return y.total;
+}
+size_t fitted_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, size_t bytes) {
   Layout y;
-  workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y, true);
-  return addressable(y) ? y.total : 0;
+  return fitted_layout(desc, plan, bytes, y);
 }
 int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, const void* W, const void* b,
                     const void* W_out, const void* b_out, const void* x, const void* targets, const void* h0,
@@ -674,9 +701,8 @@ int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, con
   if (desc->want_dx && !dx) return MEBPTT_ERR_ARG;
   const Plan* p = reinterpret_cast<const Plan*>(plan);
   Layout y;
-  workspace_layout(desc, p, y);
-  // a fixed workspace that is too small for the team path's stages can still serve the kernels without
-  if (!side_stream && y.team && y.total > workspace_bytes) workspace_layout(desc, p, y, true);
+  if (side_stream) workspace_layout(desc, p, y);
+  else fitted_layout(desc, plan, workspace_bytes, y);   // (the entry point with a fixed workspace)
   if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < y.total)
     return MEBPTT_ERR_WORKSPACE;

@@ -8,6 +8,13 @@
 
 namespace mebptt {
 
+// What a plan for a whole-device budget gives up to fit it (where a tape is walked; the other paths have one
+// size of working memory).
+struct Footprint {
+  int chunk_steps = 0;      // steps per staged chunk at most (0: as many as pay); the sums are the same
+  bool compact = false;     // no stages and no packed weights: the operation-by-operation kernels
+};
+
 struct Plan {
   uint64_t id = 0;          // unique per plan object of the process (what cached per-plan data is keyed by)
   int64_t t = 0, m = 0;
@@ -16,6 +23,7 @@ struct Plan {
   int64_t cost = 0;         // C(t, m)
   int64_t peak_units = 0;   // paper's accounting
   int64_t arena_units = 0;  // physical hidden-state units the arena must hold
+  Footprint footprint;          // how much working memory a step takes beside the arena
   // row-major [t + 1][m + 1]
   std::vector<int64_t> C;
   std::vector<int32_t> D, D2;

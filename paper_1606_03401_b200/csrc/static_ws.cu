@@ -26,8 +26,9 @@ int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, con
                     const void* W_out, const void* b_out, const void* x, const void* targets, const void* h0,
                     const void* c0, void* workspace, size_t workspace_bytes, void* stream, float* loss, float* dW,
                     float* db, float* dW_out, float* db_out, float* dx, int64_t* counters, bool side_stream);
-// The least workspace the step can run in (api.cu); 0 on a bad descriptor or plan.
-size_t least_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan);
+// What the step takes of a workspace of so many bytes (api.cu; more than that: it does not fit); 0 on a bad
+// descriptor or plan.
+size_t fitted_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, size_t bytes);
 }
 
 namespace {
@@ -66,7 +67,7 @@ extern "C" int mebptt_lstm_train_step_static(const mebptt_lstm_desc* desc, const
                                              float* db_out, float* dx, int64_t* counters) {
   // per-launch timing records CUDA events, created on demand: not here
   if (desc && (desc->flags & MEBPTT_FLAG_TIME_RUNS)) return MEBPTT_ERR_ARG;
-  const size_t need = mebptt::least_workspace_bytes(desc, plan);
+  const size_t need = mebptt::fitted_workspace_bytes(desc, plan, (size_t)MEBPTT_STATIC_WORKSPACE_BYTES);
   if (need == 0) return MEBPTT_ERR_ARG;                                   // bad descriptor or plan
   if (need > (size_t)MEBPTT_STATIC_WORKSPACE_BYTES) return MEBPTT_ERR_WORKSPACE;  // does not fit the fixed array
   void* ws = nullptr;

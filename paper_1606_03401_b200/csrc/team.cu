@@ -560,10 +560,12 @@ __global__ void __launch_bounds__(256) pack(const PackArgs<T> P) {
 }
 
 // The contractions of a finished chunk: weight gradients and dx, all in one launch, 64 x 64 tiles.
-// C[m][n] (+)= sum_k A(m, k) B[k][n]; A is stored [k][m] (a_mn) or [m][k].
+// C[m][n] (+)= sum_k A(m, k) B[k][n]; A is stored [k][m] (a_mn) or [m][k].  The contraction index is summed in
+// blocks, each by itself, and the blocks are added to C from the last to the first: with blocks of a fixed
+// number of time steps the result does not depend on how many steps a chunk has.
 struct Product {
   const float* A; const void* B; float* C;
-  int lda, ldb, ldc, M, N, K, a_mn, accumulate, tile0;
+  int lda, ldb, ldc, M, N, K, block, a_mn, accumulate, tile0;
   int H, skip, last;   // H > 0: gate rows 4 u + q of A (a_mn) or of the contraction belong to rows q H + u of the weights;
                        // rows with q == skip to none, and those with q == 3 to block `last`
 };
@@ -577,10 +579,10 @@ __device__ __forceinline__ int gate_row(const Product& p, int r) {
   return q == p.skip ? -1 : (q == 3 ? p.last : q) * p.H + (r >> 2);
 }
 
-// A tile of a product is formed by two groups of 128 threads, each over every other slice of the
+// A tile of a product is formed by two groups of 128 threads, each over every other block of the
 // contraction index, so that the loads of one hide behind the arithmetic of the other (a chunk has
-// few tiles: with one group an SM held eight warps that waited for one another); the second group's
-// sums are added to the first's at the end.  Operands come in 16-byte pieces where their rows allow it.
+// few tiles: with one group an SM held eight warps that waited for one another); the first group
+// adds up both groups' blocks.  Operands come in 16-byte pieces where their rows allow it.
 constexpr int kTileThreads = 256;
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); }
 
@@ -609,25 +611,46 @@ struct Slice {
   Piece b[N];
   // t: thread of the group.  Operands stored [k][*]: piece (t & 15) of step (t >> 4) + 8 e; A stored
   // [m][k]: piece t % (TK / 4) of row t / (TK / 4) + e * 512 / TK.
-  __device__ __forceinline__ void fetch(const Product& p, int m0, int n0, int k0, int t) {
+  // Steps from k1 on count as zero.
+  __device__ __forceinline__ void fetch(const Product& p, int m0, int n0, int k0, int k1, int t) {
     const bool wa = (p.lda & 3) == 0 && (reinterpret_cast<uintptr_t>(p.A) & 15) == 0;
     const bool wb = (p.ldb & 3) == 0 && (reinterpret_cast<uintptr_t>(p.B) & (4 * sizeof(T) - 1)) == 0;
     const int c = (t & 15) * 4;
 #pragma unroll
     for (int e = 0; e < N; ++e) {
       const int k = k0 + (t >> 4) + 8 * e;
-      const bool on = k < p.K;
+      const bool on = k < k1;
       if (p.a_mn) {
         a[e] = load_some(p.A + (size_t)(on ? k : 0) * p.lda + m0 + c, on ? p.M - m0 - c : 0, wa);
       } else {
         const int m = m0 + t / (TK / 4) + e * (512 / TK), kk = k0 + (t % (TK / 4)) * 4;
-        a[e] = load_some(p.A + (size_t)(m < p.M ? m : 0) * p.lda + kk, m < p.M ? p.K - kk : 0, wa);
+        a[e] = load_some(p.A + (size_t)(m < p.M ? m : 0) * p.lda + kk, m < p.M ? k1 - kk : 0, wa);
       }
       const int row = !on ? -1 : p.a_mn ? k : gate_row(p, k);
       b[e] = load_some(reinterpret_cast<const T*>(p.B) + (size_t)(row < 0 ? 0 : row) * p.ldb + n0 + c, row < 0 ? 0 : p.N - n0 - c, wb);
     }
   }
 };
+
+// The blocks of a product, two at a time: group g forms block `last - g`.  slice(k0, k1, next0, next1) takes the
+// fetched steps from k0 on and fetches those from next0 on (none if next0 < 0); done(g, two) adds the sums up,
+// two: of both groups.
+template <int TK, class First, class Take, class Done>
+__device__ __forceinline__ void blocks_of(const Product& p, int g, First first, Take take, Done done) {
+  const int blocks = (p.K + p.block - 1) / p.block;
+  auto end = [&](int b) { return min(p.K, (b + 1) * p.block); };
+  if (blocks - 1 - g >= 0) first((blocks - 1 - g) * p.block, end(blocks - 1 - g));
+  for (int last = blocks - 1; last >= 0; last -= 2) {
+    const int b = last - g;
+    if (b >= 0)
+      for (int k = b * p.block; k < end(b); k += TK) {
+        if (k + TK < end(b)) take(k + TK, end(b));
+        else if (b >= 2) take((b - 2) * p.block, end(b - 2));
+        else take(-1, 0);
+      }
+    done(last > 0);
+  }
+}
 
 // FMA, 8 x 4 results a thread.
 template <class T>
@@ -636,54 +659,65 @@ __device__ __forceinline__ void product_fma(const Product& p, int m0, int n0, fl
   const int g = threadIdx.x >> 7, t = threadIdx.x & 127, tx = t & 15, ty = t >> 4;
   float (*As)[LD] = reinterpret_cast<float (*)[LD]>(smem + g * 2 * TK * LD);
   float (*Bs)[LD] = As + TK;
+  float* const x = smem + 4 * TK * LD + t;     // the second group's sums
   Slice<T, TK> s;
-  float acc[8][4] = {};
-  const int its = (p.K + TK - 1) / TK;
-  s.fetch(p, m0, n0, g * TK, t);
-  for (int it = g; it < its; it += 2) {
+  float acc[8][4] = {}, sum[8][4];
+  auto at = [&](int r, int q) -> float* {      // null: no element of C
+    const int m = m0 + ty * 8 + r, n = n0 + tx * 4 + q, row = m < p.M ? (p.a_mn ? gate_row(p, m) : m) : -1;
+    return row < 0 || n >= p.N ? nullptr : p.C + (size_t)row * p.ldc + n;
+  };
+  bool any = p.accumulate;
+  if (g == 0 && any)
 #pragma unroll
-    for (int e = 0; e < s.N; ++e) {
-      if (p.a_mn) {
-        *reinterpret_cast<float4*>(&As[(t >> 4) + 8 * e][(t & 15) * 4]) = s.a[e];
-      } else {
-        const int m = t / (TK / 4) + e * (512 / TK), k = (t % (TK / 4)) * 4;
-        As[k][m] = s.a[e].x; As[k + 1][m] = s.a[e].y; As[k + 2][m] = s.a[e].z; As[k + 3][m] = s.a[e].w;
-      }
-      *reinterpret_cast<float4*>(&Bs[(t >> 4) + 8 * e][(t & 15) * 4]) = widen(s.b[e]);
-    }
-    group_sync(g);
-    if (it + 2 < its) s.fetch(p, m0, n0, (it + 2) * TK, t);
+    for (int i = 0; i < 32; ++i) { const float* o = at(i >> 2, i & 3); sum[i >> 2][i & 3] = o ? *o : 0.f; }
+  blocks_of<TK>(
+      p, g, [&](int k0, int k1) { s.fetch(p, m0, n0, k0, k1, t); },
+      [&](int next0, int next1) {
 #pragma unroll
-    for (int k = 0; k < TK; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 8]), a1 = *reinterpret_cast<const float4*>(&As[k][ty * 8 + 4]);
-      const float4 b = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-      const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {b.x, b.y, b.z, b.w};
+        for (int e = 0; e < s.N; ++e) {
+          if (p.a_mn) {
+            *reinterpret_cast<float4*>(&As[(t >> 4) + 8 * e][(t & 15) * 4]) = s.a[e];
+          } else {
+            const int m = t / (TK / 4) + e * (512 / TK), k = (t % (TK / 4)) * 4;
+            As[k][m] = s.a[e].x; As[k + 1][m] = s.a[e].y; As[k + 2][m] = s.a[e].z; As[k + 3][m] = s.a[e].w;
+          }
+          *reinterpret_cast<float4*>(&Bs[(t >> 4) + 8 * e][(t & 15) * 4]) = widen(s.b[e]);
+        }
+        group_sync(g);
+        if (next0 >= 0) s.fetch(p, m0, n0, next0, next1, t);
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
+        for (int k = 0; k < TK; ++k) {
+          const float4 a0 = *reinterpret_cast<const float4*>(&As[k][ty * 8]), a1 = *reinterpret_cast<const float4*>(&As[k][ty * 8 + 4]);
+          const float4 b = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
+          const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[r][q] = fmaf(av[r], bv[q], acc[r][q]);
-    }
-    group_sync(g);
-  }
-  __syncthreads();
-  float* const x = smem + t;
-  if (g == 1)
+          for (int r = 0; r < 8; ++r)
 #pragma unroll
-    for (int i = 0; i < 32; ++i) x[i * 128] = acc[i >> 2][i & 3];
-  __syncthreads();
+            for (int q = 0; q < 4; ++q) acc[r][q] = fmaf(av[r], bv[q], acc[r][q]);
+        }
+        group_sync(g);
+      },
+      [&](bool two) {
+        if (g == 1)
+#pragma unroll
+          for (int i = 0; i < 32; ++i) x[i * 128] = acc[i >> 2][i & 3];
+        __syncthreads();
+        if (g == 0)
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            float& v = sum[i >> 2][i & 3];
+            v = any ? v + acc[i >> 2][i & 3] : acc[i >> 2][i & 3];
+            if (two) v += x[i * 128];
+          }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[i >> 2][i & 3] = 0.f;
+        any = true;
+        __syncthreads();
+      });
   if (g == 1) return;
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int m = m0 + ty * 8 + r, row = m < p.M ? (p.a_mn ? gate_row(p, m) : m) : -1;
-    if (row < 0) continue;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int n = n0 + tx * 4 + q;
-      const float v = acc[r][q] + x[(r * 4 + q) * 128];
-      float* o = p.C + (size_t)row * p.ldc + n;
-      if (n < p.N) *o = p.accumulate ? *o + v : v;
-    }
-  }
+  for (int i = 0; i < 32; ++i)
+    if (float* o = at(i >> 2, i & 3)) *o = sum[i >> 2][i & 3];
 }
 
 // Bfloat16 storage: A (float32 gradients) as three bfloat16 planes that add up to it, on mma.sync; a warp
@@ -714,67 +748,77 @@ __device__ __forceinline__ void product_mma(const Product& p, int m0, int n0, fl
     if (trans) asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
     else asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
   };
-  s.fetch(p, m0, n0, g * TK, t);
-  const int its = (p.K + TK - 1) / TK;
   const uint32_t a0 = sm100::smem_u32(As), b0 = sm100::smem_u32(Bs);
   const int l8 = lane & 7, q8 = lane >> 3;   // row inside an 8 x 8 block, block
-  for (int it = g; it < its; it += 2) {
-    put_tile();
-    group_sync(g);
-    if (it + 2 < its) s.fetch(p, m0, n0, (it + 2) * TK, t);
+  // the second group's sums, over its tiles (read before: the barrier behind each slice)
+  float* const x = reinterpret_cast<float*>(reinterpret_cast<__nv_bfloat16*>(smem) + 3 * plane + TK * LM) + t;
+  float sum[32];
+  auto at = [&](int i) -> float* {           // i: fragment of 16 rows, 8 columns, half of the rows, column; null: no element of C
+    const int m = m0 + wm + (i >> 4) * 16 + ((i >> 1) & 1) * 8 + (lane >> 2), n = n0 + wn + ((i >> 2) & 3) * 8 + 2 * (lane & 3) + (i & 1);
+    const int row = m < p.M ? (p.a_mn ? gate_row(p, m) : m) : -1;
+    return row < 0 || n >= p.N ? nullptr : p.C + (size_t)row * p.ldc + n;
+  };
+  bool any = p.accumulate;
+  if (g == 0 && any)
 #pragma unroll
-    for (int k = 0; k < TK; k += 16) {
-      uint32_t b[2][4];
+    for (int i = 0; i < 32; ++i) { const float* o = at(i); sum[i] = o ? *o : 0.f; }
+  blocks_of<TK>(
+      p, g, [&](int k0, int k1) { s.fetch(p, m0, n0, k0, k1, t); },
+      [&](int next0, int next1) {
+        put_tile();
+        group_sync(g);
+        if (next0 >= 0) s.fetch(p, m0, n0, next0, next1, t);
 #pragma unroll
-      for (int j = 0; j < 2; ++j)   // blocks (k, n), (k + 8, n), (k, n + 8), (k + 8, n + 8)
-        ldsm(b[j], b0 + ((k + (q8 & 1) * 8 + l8) * LM + wn + j * 16 + (q8 >> 1) * 8) * 2, true);
+        for (int k = 0; k < TK; k += 16) {
+          uint32_t b[2][4];
 #pragma unroll
-      for (int q = 0; q < 3; ++q)
+          for (int j = 0; j < 2; ++j)   // blocks (k, n), (k + 8, n), (k, n + 8), (k + 8, n + 8)
+            ldsm(b[j], b0 + ((k + (q8 & 1) * 8 + l8) * LM + wn + j * 16 + (q8 >> 1) * 8) * 2, true);
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          uint32_t a[4];             // blocks (m, k), (m + 8, k), (m, k + 8), (m + 8, k + 8)
-          if (p.a_mn) ldsm(a, a0 + (q * plane + (k + (q8 >> 1) * 8 + l8) * LM + wm + i * 16 + (q8 & 1) * 8) * 2, true);
-          else ldsm(a, a0 + (q * plane + (wm + i * 16 + (q8 & 1) * 8 + l8) * LK + k + (q8 >> 1) * 8) * 2, false);
+          for (int q = 0; q < 3; ++q)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            float (&d)[4] = acc[i][j];
-            asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[j >> 1][(j & 1) * 2]), "r"(b[j >> 1][(j & 1) * 2 + 1]));
-          }
+            for (int i = 0; i < 2; ++i) {
+              uint32_t a[4];             // blocks (m, k), (m + 8, k), (m, k + 8), (m + 8, k + 8)
+              if (p.a_mn) ldsm(a, a0 + (q * plane + (k + (q8 >> 1) * 8 + l8) * LM + wm + i * 16 + (q8 & 1) * 8) * 2, true);
+              else ldsm(a, a0 + (q * plane + (wm + i * 16 + (q8 & 1) * 8 + l8) * LK + k + (q8 >> 1) * 8) * 2, false);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                float (&d)[4] = acc[i][j];
+                asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                             : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                             : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[j >> 1][(j & 1) * 2]), "r"(b[j >> 1][(j & 1) * 2 + 1]));
+              }
+            }
         }
-    }
-    group_sync(g);
-  }
-  __syncthreads();
-  float* const x = smem + t;
-  if (g == 1)
+        group_sync(g);
+      },
+      [&](bool two) {
+        if (g == 1)
 #pragma unroll
-    for (int i = 0; i < 32; ++i) x[i * 128] = acc[i >> 4][(i >> 2) & 3][i & 3];
-  __syncthreads();
+          for (int i = 0; i < 32; ++i) x[i * 128] = acc[i >> 4][(i >> 2) & 3][i & 3];
+        __syncthreads();
+        if (g == 0)
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const float v = acc[i >> 4][(i >> 2) & 3][i & 3];
+            sum[i] = any ? sum[i] + v : v;
+            if (two) sum[i] += x[i * 128];
+          }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[i >> 4][(i >> 2) & 3][i & 3] = 0.f;
+        any = true;
+        __syncthreads();
+      });
   if (g == 1) return;
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int m = m0 + wm + i * 16 + h * 8 + (lane >> 2), row = m < p.M ? (p.a_mn ? gate_row(p, m) : m) : -1;
-      if (row < 0) continue;
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int n = n0 + wn + j * 8 + 2 * (lane & 3) + q;
-          float* o = p.C + (size_t)row * p.ldc + n;
-          const float v = acc[i][j][h * 2 + q] + x[(i * 16 + j * 4 + h * 2 + q) * 128];
-          if (n < p.N) *o = p.accumulate ? *o + v : v;
-        }
-    }
+  for (int i = 0; i < 32; ++i)
+    if (float* o = at(i)) *o = sum[i];
 }
 
 // MMA: the caller has not forbidden tensor cores.
 template <class T, bool MMA>
 __global__ void __launch_bounds__(kTileThreads) chunk_products(const __grid_constant__ Products P) {
-  __shared__ __align__(16) float smem[MMA ? 3 * 64 * 40 + 32 * 72 : 4 * 16 * 68];
+  __shared__ __align__(16) float smem[MMA ? 3 * 64 * 40 + 32 * 72 : 4 * 16 * 68 + 32 * 128];
   int i = P.n - 1;
   while ((int)blockIdx.x < P.p[i].tile0) --i;
   const Product& p = P.p[i];
@@ -787,10 +831,10 @@ __global__ void __launch_bounds__(kTileThreads) chunk_products(const __grid_cons
 // so the mean of d * d over a step is the sum of dy * dy times B O / 4.
 struct Sums {
   const float *dz, *dy; float *db, *db_out, *loss_t;
-  int L, NG, H, O, B, S, steps, accumulate;
+  int L, NG, H, O, B, S, steps, block, accumulate;   // block: rows summed by themselves, as in Product
 };
 __global__ void __launch_bounds__(1024) chunk_sums(const Sums q) {
-  __shared__ float part_s[32][33];
+  __shared__ float part_s[2][32][33];
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5, G = 4 * q.H, nh = (G + 31) / 32, no = (q.O + 31) / 32;
   const int rows = q.steps * q.B;
   int b = blockIdx.x;
@@ -798,32 +842,40 @@ __global__ void __launch_bounds__(1024) chunk_sums(const Sums q) {
     const bool out = b >= q.L * nh;
     const int l = b / nh, n = (out ? b - q.L * nh : b - l * nh) * 32 + x, N = out ? q.O : G, ld = out ? q.O : G;
     const float* v = out ? q.dy : q.dz + (size_t)l * q.S * q.B * G;
-    float a0 = 0.f, a1 = 0.f;
-    if (n < N) {
-      int r = y;
-      for (; r + 32 < rows; r += 64) { a0 += v[(size_t)r * ld + n]; a1 += v[(size_t)(r + 32) * ld + n]; }
-      if (r < rows) a0 += v[(size_t)r * ld + n];
-    }
-    part_s[y][x] = a0 + a1;
-    __syncthreads();
-    if (y == 0 && n < N) {
-      float s = 0.f;
+    float* const o = out ? q.db_out + n : q.db + (size_t)l * q.NG * q.H + (size_t)(n & 3) * q.H + (n >> 2);
+    const bool mine = y == 0 && n < N && (out || (n & 3) < q.NG);   // (a GRU's d q belongs to no bias)
+    bool any = q.accumulate;
+    float sum = mine && any ? *o : 0.f;
+    for (int blk = (rows - 1) / q.block; blk >= 0; --blk) {
+      float (*part)[33] = part_s[blk & 1];
+      const int end = min(rows, (blk + 1) * q.block);
+      float a0 = 0.f, a1 = 0.f;
+      if (n < N) {
+        int r = blk * q.block + y;
+        for (; r + 32 < end; r += 64) { a0 += v[(size_t)r * ld + n]; a1 += v[(size_t)(r + 32) * ld + n]; }
+        if (r < end) a0 += v[(size_t)r * ld + n];
+      }
+      part[y][x] = a0 + a1;
+      __syncthreads();
+      if (mine) {
+        float s = 0.f;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) s += part_s[i][x];
-      if (!out && (n & 3) >= q.NG) return;   // (a GRU's d q belongs to no bias)
-      float* o = out ? q.db_out + n : q.db + (size_t)l * q.NG * q.H + (size_t)(n & 3) * q.H + (n >> 2);
-      *o = q.accumulate ? *o + s : s;
+        for (int i = 0; i < 32; ++i) s += part[i][x];
+        sum = any ? sum + s : s;
+        any = true;
+      }
     }
+    if (mine) *o = sum;
   } else {
     const int k = b - q.L * nh - no;
     const float* v = q.dy + (size_t)k * q.B * q.O;
     float a = 0.f;
     for (int e = threadIdx.x; e < q.B * q.O; e += 1024) a = fmaf(v[e], v[e], a);
     for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-    if (x == 0) part_s[0][y] = a;
+    if (x == 0) part_s[0][0][y] = a;
     __syncthreads();
     if (y == 0) {
-      a = part_s[0][x];
+      a = part_s[0][0][x];
       for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
       if (x == 0) q.loss_t[k] = a * ((float)q.B * (float)q.O * 0.25f);
     }
@@ -914,7 +966,8 @@ std::vector<std::shared_ptr<Kept>> g_kept;
 constexpr size_t kKeep = 8, kMaxPinned = (size_t)64 << 20;
 
 bool same_problem(const Layout& a, const Layout& b) {
-  return a.L == b.L && a.I == b.I && a.H == b.H && a.O == b.O && a.B == b.B && a.dtype == b.dtype && a.t == b.t && a.gru == b.gru && a.tensor_cores == b.tensor_cores;
+  return a.L == b.L && a.I == b.I && a.H == b.H && a.O == b.O && a.B == b.B && a.dtype == b.dtype && a.t == b.t && a.gru == b.gru && a.tensor_cores == b.tensor_cores &&
+         a.S == b.S && a.tape_bytes == b.tape_bytes;
 }
 
 // Null, and a status, where there is none.
@@ -1007,7 +1060,9 @@ void fill_products(Products& P, const Layout& y, const tc::StepPtrs& io, bool wa
   P.n = 0; P.tiles = 0;
   auto add = [&](const float* A, int lda, bool a_mn, const void* B, int ldb, float* C, int ldc, int M, int N, int K, bool acc,
                  int hidden, int skip, int last) {
-    P.p[P.n++] = Product{A, B, C, lda, ldb, ldc, M, N, K, a_mn ? 1 : 0, acc ? 1 : 0, P.tiles, hidden, skip, last};
+    // (dx is summed over the gates: halves, one for each group)
+    const int block = a_mn ? sum_steps(y.B) * y.B : (int)align_up(((size_t)K + 1) / 2, 32);
+    P.p[P.n++] = Product{A, B, C, lda, ldb, ldc, M, N, K, block, a_mn ? 1 : 0, acc ? 1 : 0, P.tiles, hidden, skip, last};
     P.tiles += ((M + 63) / 64) * ((N + 63) / 64);
   };
   for (int l = 0; l < y.L; ++l) {
@@ -1133,7 +1188,7 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
       else if (y.tensor_cores) chunk_products<__nv_bfloat16, true><<<P.tiles, kTileThreads, 0, s>>>(P);
       else chunk_products<__nv_bfloat16, false><<<P.tiles, kTileThreads, 0, s>>>(P);
       const Sums q{reinterpret_cast<const float*>(io.ws + y.off_dz), reinterpret_cast<const float*>(io.ws + y.off_dy), io.db, io.db_out,
-                   loss_t + k0, y.L, y.NG, y.H, y.O, y.B, y.S, steps, first ? 0 : 1};
+                   loss_t + k0, y.L, y.NG, y.H, y.O, y.B, y.S, steps, sum_steps(y.B) * y.B, first ? 0 : 1};
       chunk_sums<<<y.L * ((4 * y.H + 31) / 32) + (y.O + 31) / 32 + steps, 1024, 0, s>>>(q);
       first = false;
     }

@@ -8,7 +8,7 @@ import sys
 import pytest
 
 from paper_1606_03401_b200 import synth
-from tests.util import assert_bit_identical
+from tests.util import assert_bit_identical, assert_close_to_oracle, oracle_run
 
 pytestmark = pytest.mark.gpu
 
@@ -93,3 +93,45 @@ def test_plans_in_fractions_of_a_hidden_state_give_the_bits_of_other_plans(size,
             res = dp.run(plan)
             assert res["counters"][0] == plan.cost and res["counters"][1] == cfg.t and res["counters"][3] == 0
             assert_bit_identical(res, full, want_dx=True)
+
+
+@pytest.mark.parametrize("dtype,gru,size", [
+    ("fp32", False, dict(layers=2, input=33, hidden=96, batch=13, t=150, readout=20)),     # pods, a ragged last chunk
+    ("bf16", True, dict(layers=2, input=64, hidden=256, batch=32, t=90, readout=40)),      # pods, tensor cores
+    ("bf16", False, dict(layers=2, input=40, hidden=300, batch=40, t=70, readout=29)),     # teams, 2048 rows no whole chunk
+    ("fp32", False, dict(layers=2, input=24, hidden=520, batch=300, t=14, readout=16)),    # teams, a step a block
+])
+def test_whole_device_budgets_shorten_chunks_without_a_change_in_a_bit(dtype, gru, size):
+    """A budget that counts the working memory cuts the staged chunks short, and at last the kernels that need
+    any: every length of chunk gives the bits of the ordinary plan, the operations those of one another and
+    both the oracle's gradients."""
+    from paper_1606_03401_b200 import binding as B
+    from paper_1606_03401_b200 import harness as H
+    cfg = synth.with_overrides(synth.CONFIGS["c1"], dtype=dtype, **size, **({"cell": "gru"} if gru else {}))
+    dp = H.DeviceProblem(cfg, want_dx=True)
+    ref = oracle_run(dp.prob)
+    ordinary = dp.plan("msm", 12)
+    full = dp.run(ordinary)
+    assert_close_to_oracle(full, ref, dtype, want_dx=True)
+    route, nbytes = B.mebptt_test_route(dp.desc, ordinary), 4 * B.mebptt_lstm_workspace_bytes(dp.desc, ordinary)
+    seen, alone = {}, []
+    while True:
+        try:
+            plan = B.mebptt_plan_for_bytes(dp.desc, nbytes, B.MEBPTT_MSM, include_working=True)
+        except B.MebpttError:
+            break
+        r = B.mebptt_test_route(dp.desc, plan)
+        if seen.setdefault((r["route"], r["chunk"]), 0) < 2:
+            seen[r["route"], r["chunk"]] += 1
+            dp._ws = None                       # exactly the workspace that was asked for
+            res = dp.run(plan)
+            assert dp._ws.numel() <= nbytes
+            assert res["counters"][0] == plan.cost and res["counters"][1] == cfg.t and res["counters"][3] == 0
+            if r["route"] == route["route"]:
+                assert_bit_identical(res, full, want_dx=True)
+            else:
+                alone.append(res)
+                assert_close_to_oracle(res, ref, dtype, want_dx=True)
+                assert_bit_identical(res, alone[0], want_dx=True)
+        nbytes = nbytes * 4 // 5
+    assert len(alone) == 2 and (route["route"], route["chunk"]) in seen and len(seen) >= 3, seen

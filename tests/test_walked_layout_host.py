@@ -67,3 +67,61 @@ def test_plans_over_byte_sizes_take_the_kernels_of_other_plans(dtype, gru):
                 assert got == want and want["route"] in ("pods", "teams", "persistent"), (layers, hidden, batch)
                 sigmas.add(exact.sigma)
     assert dtype == "fp32" or {2, 3, 5, 7} <= sigmas
+
+
+def _refused(desc, nbytes, mode):
+    try:
+        return B.mebptt_plan_for_bytes(desc, nbytes, mode, include_working=True)
+    except B.MebpttError as e:
+        assert e.status == B.MEBPTT_ERR_BUDGET
+        return None
+
+
+@pytest.mark.parametrize("size,least", [
+    ((2, 161, 300, 29, 20, 160, "bf16", False), 1_000_000),     # teams
+    ((2, 161, 300, 29, 40, 160, "bf16", False), 1_750_000),     # teams
+    ((1, 77, 200, 61, 13, 120, "fp32", False), 300_000),        # pods
+    ((2, 128, 256, 128, 32, 128, "bf16", True), 1_000_000),     # pods
+    ((1, 32, 64, 32, 4, 64, "fp32", False), 25_000),            # pods, one length of chunk
+])
+@pytest.mark.parametrize("mode", [B.MEBPTT_HSM, B.MEBPTT_MSM])
+def test_a_whole_device_budget_is_met_from_a_few_states_on(size, least, mode):
+    """What the operation-by-operation kernels hold beside the states was always enough for a plan; more memory
+    never makes one more expensive on the same kernels, and the kernels that walk the tape come in with it."""
+    desc = _problem(size)
+    assert _refused(desc, least // 4, mode) is None
+    seen, cheapest, nbytes = [], {}, least
+    while nbytes < 200_000_000:
+        plan = _refused(desc, nbytes, mode)
+        assert plan is not None, nbytes
+        assert B.mebptt_lstm_workspace_bytes(desc, plan) <= nbytes
+        r = B.mebptt_test_route(desc, plan)
+        if r["route"] != "operations":
+            # room for the states, and for one more at most
+            assert B.mebptt_lstm_workspace_bytes(desc, plan) - B.mebptt_lstm_working_bytes(desc, plan) > 0
+        key = (r["route"], r["chunk"])
+        assert plan.cost <= cheapest.get(key, plan.cost)
+        cheapest[key] = plan.cost
+        seen.append(r["chunk"])
+        nbytes = nbytes * 7 // 6
+    assert seen[0] == 0 and seen == sorted(seen) and seen[-1] == B.mebptt_test_route(desc, B.mebptt_plan(size[5], 8, mode))["chunk"]
+
+
+@pytest.mark.parametrize("use_beta", [False, True])
+def test_a_whole_device_budget_in_exact_sizes_is_met_too(use_beta):
+    desc = _problem((2, 161, 300, 29, 40, 160, "bf16", False))
+    for nbytes in (2_000_000, 5_000_000, 20_000_000, 60_000_000):
+        plan = B.mebptt_plan_bytes_exact(desc, nbytes, use_beta, include_working=True)
+        assert plan.sigma == 5 and B.mebptt_lstm_workspace_bytes(desc, plan) <= nbytes
+    assert B.mebptt_test_route(desc, plan)["route"] == "teams"
+
+
+def test_chunks_are_whole_blocks_of_sums():
+    """The weight gradients are summed in blocks of a fixed number of steps: a chunk that cut one would change bits."""
+    for batch in (1, 5, 13, 32, 33, 48, 100, 129, 3000):
+        desc = _problem((2, 20, 40, 10, batch, 400, "fp32", False))
+        blocks = next(s for s in (1, 2, 4, 8, 16, 32, 64) if s * batch >= 256 or s == 64)
+        for nbytes in (10 ** 6 * k * k for k in range(1, 24, 2)):
+            plan = _refused(desc, nbytes * (1 + batch // 40), B.MEBPTT_HSM)
+            if plan is not None:
+                assert B.mebptt_test_route(desc, plan)["chunk"] % blocks == 0

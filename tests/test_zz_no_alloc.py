@@ -63,6 +63,29 @@ def test_static_workspace_step_matches_ordinary_step_twice(base, kw, mode, m):
         assert_bit_identical(_static_run(dp, other), want, want_dx=True)
 
 
+@pytest.mark.parametrize("kw,chunk", [
+    (dict(layers=3, input=40, hidden=256, batch=32, t=150, readout=40), True),     # shorter chunks
+    (dict(layers=3, input=40, hidden=520, batch=20, t=30, readout=40), False),     # not even those: operations
+])
+def test_static_workspace_step_in_less_memory_than_the_ordinary_step_takes(kw, chunk):
+    """Where only the staging keeps a walked tape out of the array, chunks are cut short, with the same bits;
+    where the packed weights alone do, the operations run one by one, within the type's rounding."""
+    from paper_1606_03401_b200 import binding as B
+    from paper_1606_03401_b200 import harness
+    from tests.util import assert_close_to_oracle, oracle_run
+    cfg = synth.with_overrides(synth.CONFIGS["c1"], **kw)
+    dp = harness.DeviceProblem(cfg, want_dx=True)
+    plan = dp.plan("msm", 30)
+    assert B.mebptt_test_route(dp.desc, plan)["route"] in ("pods", "teams")
+    assert B.mebptt_lstm_workspace_bytes(dp.desc, plan) > B.MEBPTT_STATIC_WORKSPACE_BYTES
+    got = _static_run(dp, plan)
+    assert got["counters"][0] == plan.cost and got["counters"][1] == cfg.t and got["counters"][3] == 0
+    assert_close_to_oracle(got, oracle_run(dp.prob), cfg.dtype, want_dx=True)
+    if chunk:
+        assert_bit_identical(got, dp.run(plan), want_dx=True)
+        assert_bit_identical(_static_run(dp, plan), got, want_dx=True)
+
+
 def test_static_workspace_step_refuses_per_launch_timing():
     """Timing every launch creates CUDA events on demand, which the allocation-free call must not."""
     from paper_1606_03401_b200 import binding as B

@@ -375,16 +375,17 @@ int mebptt_plan_sigma(const mebptt_plan_t *plan);
 
 /*
  * What a training step derives from (descriptor, plan, workspace address, device) alone -- the
- * runs the tape of Algorithm 2 is cut into, the tape in the form the kernels read, the kernel
- * variants the device can keep resident, the TMA tensor maps -- is prepared once and kept in a
- * small cache inside the library (eight sets, least recently used out first); mebptt_plan_free
- * drops the sets of its plan.  The first mebptt_lstm_train_step of a combination therefore costs
+ * runs the tape of Algorithm 2 is cut into, or the schedule it is walked by; the tape in the form
+ * the kernels read; on the persistent bfloat16 path the kernel variants the device can keep
+ * resident and the TMA tensor maps -- is prepared once and kept in a small cache inside the library
+ * (eight sets of each kind, least recently used out first); mebptt_plan_free drops the sets of its
+ * plan.  The first mebptt_lstm_train_step of a combination therefore costs
  * some host time (page-locked memory is allocated for the tape); later ones only look the set up,
  * copy the tape asynchronously and enqueue.  (The paper has no counterpart: its Algorithm 2
  * walks the policy tables on the host at every step.)
  *
  * mebptt_lstm_prepare makes the host part of a set ahead of time, or finds it; it needs no GPU
- * and returns a status.  mebptt_lstm_prepare_stats fills out[0..3] (host array) with: sets built
+ * and returns a status.  (Operation by operation on the CUDA cores there is nothing to prepare.)  mebptt_lstm_prepare_stats fills out[0..3] (host array) with: sets built
  * since the library was loaded, look-ups served from the cache, sets whose tape lies in
  * page-locked memory, sets held now.
  */

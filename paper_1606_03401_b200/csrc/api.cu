@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cstdlib>
 #include <cstring>
+#include <memory>
+#include <mutex>
 #include <vector>
 
 #include "env.hpp"
@@ -22,6 +24,41 @@ using namespace mebptt;
 namespace {
 
 using StepIO = tc::StepPtrs;
+
+// The work items a plan's tape is cut into, and the projection windows of its runs: kept from step to step for
+// the paths that have nothing else to prepare (eight, most recently used first).
+struct Cut {
+  uint64_t plan_id = 0;
+  int S = 0;
+  std::vector<WorkItem> items;
+  std::vector<int> windows;
+};
+std::mutex g_cut_mu;
+std::vector<std::shared_ptr<const Cut>> g_cuts;
+int64_t g_cuts_built = 0, g_cuts_reused = 0;
+
+std::shared_ptr<const Cut> cut_for(const Layout& y, const Plan* p) {
+  {
+    std::lock_guard<std::mutex> lock(g_cut_mu);
+    for (size_t i = 0; i < g_cuts.size(); ++i)
+      if (g_cuts[i]->plan_id == p->id && g_cuts[i]->S == y.S) {
+        const std::shared_ptr<const Cut> hit = g_cuts[i];
+        g_cuts.erase(g_cuts.begin() + (long)i);
+        g_cuts.insert(g_cuts.begin(), hit);
+        ++g_cuts_reused;
+        return hit;
+      }
+  }
+  std::shared_ptr<Cut> c = std::make_shared<Cut>();
+  c->plan_id = p->id; c->S = y.S;
+  c->items = work_items(p, y.S);
+  c->windows = projection_windows(c->items, p, y.S, y.t);
+  std::lock_guard<std::mutex> lock(g_cut_mu);
+  ++g_cuts_built;
+  g_cuts.insert(g_cuts.begin(), c);
+  if (g_cuts.size() > 8) g_cuts.pop_back();
+  return c;
+}
 
 // Base address of the hidden block (or record) at a tape location; LOC_INIT has none.
 inline char* loc_base(const Layout& y, char* ws, int32_t loc) {
@@ -293,8 +330,9 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
         rc = stepwise3::flush_chunk(x3, steps, 1, y.B, y.I, y.H, y.O, w_off, io.dW, io.dW_out, io.db, io.db_out, s);
       }
     };
-    const std::vector<WorkItem> items = work_items(p, y.S);
-    const std::vector<int> windows = projection_windows(items, p, y.S, y.t);
+    const std::shared_ptr<const Cut> cut = cut_for(y, p);
+    const std::vector<WorkItem>& items = cut->items;
+    const std::vector<int>& windows = cut->windows;
     int64_t zx_lo = 0;
     for (size_t item = 0; item < items.size() && rc == MEBPTT_OK; ++item) {
       const WorkItem& wi = items[item];
@@ -356,7 +394,8 @@ int run_step(const mebptt_lstm_desc* desc, const Plan* p, const Layout& y, const
       run_op(op);
     }
   } else {
-    const std::vector<WorkItem> items = work_items(p, y.S);
+    const std::shared_ptr<const Cut> cut = cut_for(y, p);
+    const std::vector<WorkItem>& items = cut->items;
     std::vector<stepwise::FwdRunStep> fst((size_t)y.S);
     std::vector<stepwise::BwdRunStep> bst((size_t)y.S);
     std::vector<const void*> h_top((size_t)y.S);
@@ -623,7 +662,8 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
     // readout once per run (stage, GEMM with loss, loss terms, dha), the gradient handed down
     // once per layer and run
     int64_t n_launch = chunks * (3 * L + 2) + 1;
-    for (const WorkItem& wi : work_items(p, y.S)) {
+    const std::shared_ptr<const Cut> cut = cut_for(y, p);
+    for (const WorkItem& wi : cut->items) {
       if (wi.kind == WorkItem::LEAF) n_launch += wi.n * (3 * L + 2 + dha + bwd);
       else if (wi.kind == WorkItem::FWD) n_launch += wi.n == 1 ? 3 * L : L * (1 + 2 * (int64_t)wi.n);
       else if (wi.n == 1) n_launch += 2 + dha + bwd;
@@ -646,8 +686,9 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
       // packing; a window of projections: split and GEMM; forward run: one; backward run: readout of two
       // and dha, run, d_in; a batch of leaves: split, GEMM, states, two GEMMs, cells before that; chunks as below
       int64_t n = 5 + (desc->want_dx ? 1 : 0) + chunks * 11 + 1;
-      const std::vector<WorkItem> items = work_items(p, y.S);
-      const std::vector<int> windows = projection_windows(items, p, y.S, y.t);
+      const std::shared_ptr<const Cut> cut = cut_for(y, p);
+      const std::vector<WorkItem>& items = cut->items;
+      const std::vector<int>& windows = cut->windows;
       const int64_t back = 3 + dha + (desc->want_dx ? to_x : 0);
       for (size_t i = 0; i < items.size(); ++i) {
         if (items[i].kind == WorkItem::FWD) n += 1 + (windows[i] ? 2 : 0);
@@ -660,7 +701,8 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
     // launches), and a run of n >= 2 forward operations splits its operands once per layer (then
     // GEMM and cell kernel per step)
     int64_t readouts = 0, forwards = 0;
-    for (const WorkItem& wi : work_items(p, y.S)) {
+    const std::shared_ptr<const Cut> cut = cut_for(y, p);
+    for (const WorkItem& wi : cut->items) {
       if (wi.kind == WorkItem::LEAF) { readouts += wi.n * (3 + dha); forwards += wi.n * 3 * L; }
       else if (wi.kind == WorkItem::BWD) readouts += 3 + dha;
       else forwards += wi.n == 1 ? 3 * L : L * (1 + 2 * (int64_t)wi.n);
@@ -674,6 +716,11 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
 }  // extern "C"
 
 namespace mebptt {
+void forget_cuts(uint64_t plan_id) {
+  std::lock_guard<std::mutex> lock(g_cut_mu);
+  for (size_t i = g_cuts.size(); i-- > 0;)
+    if (g_cuts[i]->plan_id == plan_id) g_cuts.erase(g_cuts.begin() + (long)i);
+}
 // The plan's layout, or, in a fixed workspace that is too small for it, the largest of the smaller ones that fits.
 // 0 on a bad descriptor or plan, else what the chosen one (or the least, if none fits) takes.
 size_t fitted_layout(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, size_t bytes, Layout& y) {
@@ -801,8 +848,11 @@ int mebptt_lstm_prepare(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan)
   const Plan* p = reinterpret_cast<const Plan*>(plan);
   Layout y;
   workspace_layout(desc, p, y);
-  if (!y.tensor_path) return MEBPTT_OK;   // the other paths walk the plan's tape as it is
-  return tc::prepare_host(y, p, desc->want_dx != 0);
+  if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
+  if (y.tensor_path) return tc::prepare_host(y, p, desc->want_dx != 0);
+  if (y.team) return team::prepare_host(y, p);
+  if (y.stepwise_tc || y.stepwise_x3) cut_for(y, p);
+  return MEBPTT_OK;   // operation by operation the plan's tape is walked as it is
 }
 
 int mebptt_test_wait_fault(int mask) {
@@ -856,7 +906,11 @@ int64_t mebptt_test_schedule(const mebptt_lstm_desc* desc, const mebptt_plan_t* 
 
 int mebptt_lstm_prepare_stats(int64_t* out) {
   if (!out) return MEBPTT_ERR_ARG;
+  for (int i = 0; i < 4; ++i) out[i] = 0;
   tc::prepare_stats(out);
+  team::prepare_stats(out);
+  std::lock_guard<std::mutex> lock(g_cut_mu);
+  out[0] += g_cuts_built; out[1] += g_cuts_reused; out[3] += (int64_t)g_cuts.size();
   return MEBPTT_OK;
 }
 

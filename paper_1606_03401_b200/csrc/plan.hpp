@@ -35,5 +35,6 @@ int build_plan(int64_t t, int64_t m, int mode, int alpha, int beta, Plan** out, 
 int build_chen_plan(int64_t t, int alpha, int beta, Plan** out);
 int build_chen_recursive_plan(int64_t t, int k, int alpha, int beta, Plan** out);
 int validate_plan(const Plan& p);
+void forget_cuts(uint64_t plan_id);   // api.cu: the work items kept for a plan that is being freed
 
 }  // namespace mebptt

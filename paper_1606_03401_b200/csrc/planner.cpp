@@ -736,6 +736,7 @@ void mebptt_plan_free(mebptt_plan_t* plan) {
   if (!plan) return;
   mebptt::tc::forget_plan(reinterpret_cast<Plan*>(plan)->id);   // what the executor prepared for this plan goes with it
   mebptt::team::forget_plan(reinterpret_cast<Plan*>(plan)->id);
+  mebptt::forget_cuts(reinterpret_cast<Plan*>(plan)->id);
   delete reinterpret_cast<Plan*>(plan);
 }
 

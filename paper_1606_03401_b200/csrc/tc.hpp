@@ -126,8 +126,8 @@ constexpr uint32_t fault_poll_limit = 1u << 14;
 
 // The prepared sets (work items, device tape, kernel variants, tensor maps) that run_step keeps per
 // (problem, plan, workspace, device).  forget_plan drops those of a plan that is being freed;
-// prepare_host makes (or finds) the host part only and returns its status; prepare_stats fills
-// out[0..3] with sets built, sets reused, sets with a page-locked tape, sets held.
+// prepare_host makes (or finds) the host part only and returns its status; prepare_stats adds to
+// out[0..3] sets built, sets reused, sets with a page-locked tape, sets held.
 void forget_plan(uint64_t plan_id);
 int prepare_host(const Layout& y, const Plan* p, bool want_dx);
 void prepare_stats(int64_t* out);

@@ -1901,9 +1901,9 @@ void forget_plan(uint64_t plan_id) {
 }
 
 void prepare_stats(int64_t* out) {
-  for (int i = 0; i < 3; ++i) out[i] = g_prep_stats[i].load();
+  for (int i = 0; i < 3; ++i) out[i] += g_prep_stats[i].load();
   std::lock_guard<std::mutex> lock(g_prep_mu);
-  out[3] = (int64_t)g_prep.size();
+  out[3] += (int64_t)g_prep.size();
 }
 
 int prepare_host(const Layout& y, const Plan* p, bool want_dx) { return prepare(y, p, want_dx, nullptr, false)->rc; }

@@ -964,6 +964,7 @@ struct Kept {
 std::mutex g_mu;
 std::vector<std::shared_ptr<Kept>> g_kept;
 constexpr size_t kKeep = 8, kMaxPinned = (size_t)64 << 20;
+int64_t g_built = 0, g_reused = 0, g_pinned = 0;   // (under g_mu)
 
 bool same_problem(const Layout& a, const Layout& b) {
   return a.L == b.L && a.I == b.I && a.H == b.H && a.O == b.O && a.B == b.B && a.dtype == b.dtype && a.t == b.t && a.gru == b.gru && a.tensor_cores == b.tensor_cores &&
@@ -983,6 +984,7 @@ std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable
         std::shared_ptr<Kept> hit = g_kept[i];
         g_kept.erase(g_kept.begin() + (long)i);
         g_kept.insert(g_kept.begin(), hit);
+        ++g_reused;
         return hit;
       }
     }
@@ -1004,6 +1006,8 @@ std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable
   k->tasks = static_cast<char*>(mem);
   memcpy(k->tasks, rec.bytes.data(), rec.bytes.size());
   std::lock_guard<std::mutex> lock(g_mu);
+  ++g_built;
+  g_pinned += k->pinned;
   g_kept.insert(g_kept.begin(), k);
   if (g_kept.size() > kKeep) g_kept.pop_back();
   return k;
@@ -1085,6 +1089,16 @@ void forget_plan(uint64_t plan_id) {
   std::lock_guard<std::mutex> lock(g_mu);
   for (size_t i = g_kept.size(); i-- > 0;)
     if (g_kept[i]->plan_id == plan_id) g_kept.erase(g_kept.begin() + (long)i);
+}
+
+int prepare_host(const Layout& y, const Plan* p) {
+  int status = MEBPTT_OK;
+  return schedule_for(y, p, false, status) ? MEBPTT_OK : status;
+}
+
+void prepare_stats(int64_t* out) {
+  std::lock_guard<std::mutex> lock(g_mu);
+  out[0] += g_built; out[1] += g_reused; out[2] += g_pinned; out[3] += (int64_t)g_kept.size();
 }
 
 int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool want_dx, cudaStream_t s, bool dry) {

@@ -6,6 +6,8 @@ looked up afterwards; freeing a plan drops what was made for it.
 """
 import gc
 
+import pytest
+
 from paper_1606_03401_b200 import binding as B
 
 
@@ -70,8 +72,32 @@ def test_the_cache_holds_eight_sets_and_evicts_the_least_recently_used():
 
 
 def test_paths_without_a_device_tape_need_no_preparation():
-    desc = B.make_desc(1, 32, 64, 32, 4, 64, "fp32")
+    desc = B.make_desc(1, 60000, 64, 32, 4, 64, "fp32")      # a row of inputs that no CTA has room for
     plan = B.mebptt_plan(64, 8, B.MEBPTT_HSM)
+    assert B.mebptt_test_route(desc, plan)["route"] == "operations"
     s0 = _stats()
     B.mebptt_lstm_prepare(desc, plan)
     assert _stats() == s0
+
+
+@pytest.mark.parametrize("route,desc", [
+    ("pods", B.make_desc(1, 32, 64, 32, 4, 64, "fp32")),
+    ("teams", B.make_desc(2, 161, 300, 29, 20, 64, "bf16", want_dx=1)),
+    ("stepwise", B.make_desc(2, 64, 1024, 64, 32, 64, "bf16")),
+    ("stepwise_f32", B.make_desc(2, 64, 1024, 64, 32, 64, "tf32")),
+    ("runs_f32", B.make_desc(1, 64, 1024, 64, 32, 64, "tf32")),
+])
+def test_every_other_path_has_its_set_built_ahead_of_the_step(route, desc):
+    plan = B.mebptt_plan(64, 8, B.MEBPTT_MSM)
+    assert B.mebptt_test_route(desc, plan)["route"] == route
+    s0 = _stats()
+    B.mebptt_lstm_prepare(desc, plan)
+    s1 = _stats()
+    assert s1["built"] == s0["built"] + 1 and s1["held"] == s0["held"] + 1
+    B.mebptt_lstm_prepare(desc, plan)
+    assert B.mebptt_lstm_launch_count(desc, plan) > 0       # goes through the same set
+    s2 = _stats()
+    assert s2["built"] == s1["built"] and s2["reused"] == s1["reused"] + 2 and s2["held"] == s1["held"]
+    del plan
+    gc.collect()
+    assert _stats()["held"] == s0["held"]

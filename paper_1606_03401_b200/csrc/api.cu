@@ -7,6 +7,7 @@
 #include <cstring>
 #include <memory>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "env.hpp"
@@ -24,6 +25,16 @@ using namespace mebptt;
 namespace {
 
 using StepIO = tc::StepPtrs;
+
+// What a C entry point does, with a failed host allocation as a status instead of an exception.
+template <class F>
+auto guarded(F f, decltype(f()) failed) -> decltype(f()) {
+  try {
+    return f();
+  } catch (const std::bad_alloc&) {
+    return failed;
+  }
+}
 
 // The work items a plan's tape is cut into, and the projection windows of its runs: kept from step to step for
 // the paths that have nothing else to prepare (eight, most recently used first).
@@ -602,8 +613,8 @@ int mebptt_plan_for_bytes(const mebptt_lstm_desc* desc, size_t budget_bytes, int
   const size_t unit = mebptt_lstm_unit_bytes(desc);
   if (!unit) return MEBPTT_ERR_ARG;
   const size_t per_m = (mode == MEBPTT_ISM) ? 4 * unit : unit;   // what one more of the mode's units costs
-  return plan_in(desc, budget_bytes, per_m, 1, include_working != 0,
-                 [&](int64_t m, Plan** plan) { return build_plan(desc->t, m, mode, 4, 0, plan); }, out);
+  auto make = [&](int64_t m, Plan** plan) { return build_plan(desc->t, m, mode, 4, 0, plan); };
+  return guarded([&] { return plan_in(desc, budget_bytes, per_m, 1, include_working != 0, make, out); }, MEBPTT_ERR_OOM);
 }
 
 int mebptt_plan_bytes_exact(const mebptt_lstm_desc* desc, size_t budget_bytes, int use_beta, int include_working,
@@ -618,26 +629,31 @@ int mebptt_plan_bytes_exact(const mebptt_lstm_desc* desc, size_t budget_bytes, i
   const size_t f = gcd_sz(gcd_sz(y.unit, y.rec), rec_short);
   const int sigma = (int)(y.unit / f), alpha = (int)(y.rec / f), beta = use_beta ? (int)(rec_short / f) : 0;
   if (sigma > 64) return MEBPTT_ERR_UNSUPPORTED;
-  return plan_in(desc, budget_bytes, f, sigma, include_working != 0,
-                 [&](int64_t m, Plan** plan) { return build_plan(desc->t, m, MEBPTT_MSM, alpha, beta, plan, sigma); }, out);
+  auto make = [&](int64_t m, Plan** plan) { return build_plan(desc->t, m, MEBPTT_MSM, alpha, beta, plan, sigma); };
+  return guarded([&] { return plan_in(desc, budget_bytes, f, sigma, include_working != 0, make, out); }, MEBPTT_ERR_OOM);
 }
 
 size_t mebptt_lstm_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
   if (check_common(desc, plan) != MEBPTT_OK) return 0;
-  Layout y;
-  workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
-  return addressable(y) ? y.total : 0;
+  return guarded([&]() -> size_t {
+    Layout y;
+    workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
+    return addressable(y) ? y.total : 0;
+  }, 0);
 }
 
 size_t mebptt_lstm_working_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
   if (check_common(desc, plan) != MEBPTT_OK) return 0;
-  Layout y;
-  workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
-  return y.total - y.off_core;
+  return guarded([&]() -> size_t {
+    Layout y;
+    workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
+    return y.total - y.off_core;
+  }, 0);
 }
 
 int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
   if (check_common(desc, plan) != MEBPTT_OK) return -1;
+  return guarded([&]() -> int64_t {
   const Plan* p = reinterpret_cast<const Plan*>(plan);
   Layout y;
   workspace_layout(desc, p, y);
@@ -711,6 +727,7 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
   }
   // (a GRU layer's backward operation takes two launches more: its weight gradient comes in three blocks)
   return p->cost * L + p->t * (5 + (y.gru ? 6 : 4) * L) + 1;
+  }, -1);
 }
 
 }  // extern "C"
@@ -734,8 +751,10 @@ size_t fitted_layout(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, si
   return y.total;
 }
 size_t fitted_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, size_t bytes) {
-  Layout y;
-  return fitted_layout(desc, plan, bytes, y);
+  return guarded([&]() -> size_t {
+    Layout y;
+    return fitted_layout(desc, plan, bytes, y);
+  }, 0);
 }
 int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, const void* W, const void* b,
                     const void* W_out, const void* b_out, const void* x, const void* targets, const void* h0,
@@ -746,6 +765,7 @@ int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, con
   if (!W || !b || !W_out || !b_out || !x || !targets || !h0 || !c0) return MEBPTT_ERR_ARG;
   if (!loss || !dW || !db || !dW_out || !db_out || !counters) return MEBPTT_ERR_ARG;
   if (desc->want_dx && !dx) return MEBPTT_ERR_ARG;
+  return guarded([&]() -> int {
   const Plan* p = reinterpret_cast<const Plan*>(plan);
   Layout y;
   if (side_stream) workspace_layout(desc, p, y);
@@ -759,6 +779,7 @@ int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, con
   io.time_runs = (desc->flags & MEBPTT_FLAG_TIME_RUNS) != 0;
   io.pageable_tape = !side_stream;   // the allocation-free entry point (the only caller without side stream) locks no pages
   return run_step(desc, p, y, io, (cudaStream_t)stream, side_stream);
+  }, MEBPTT_ERR_OOM);
 }
 }  // namespace mebptt
 
@@ -775,12 +796,14 @@ int mebptt_lstm_train_step(const mebptt_lstm_desc* desc, const mebptt_plan_t* pl
 
 size_t mebptt_lstm_host_workspace_bytes(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
   if (check_common(desc, plan) != MEBPTT_OK) return 0;
-  Layout y;
-  workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
-  if (!addressable(y)) return 0;
-  Staging g;
-  staging_layout(y, desc->want_dx != 0, y.total, g);
-  return g.total;
+  return guarded([&]() -> size_t {
+    Layout y;
+    workspace_layout(desc, reinterpret_cast<const Plan*>(plan), y);
+    if (!addressable(y)) return 0;
+    Staging g;
+    staging_layout(y, desc->want_dx != 0, y.total, g);
+    return g.total;
+  }, 0);
 }
 
 int mebptt_lstm_train_step_host(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, const void* W,
@@ -793,6 +816,7 @@ int mebptt_lstm_train_step_host(const mebptt_lstm_desc* desc, const mebptt_plan_
   if (!W || !b || !W_out || !b_out || !x || !targets || !h0 || !c0) return MEBPTT_ERR_ARG;
   if (!loss || !dW || !db || !dW_out || !db_out || !counters) return MEBPTT_ERR_ARG;
   if (desc->want_dx && !dx) return MEBPTT_ERR_ARG;
+  return guarded([&]() -> int {
   const Plan* p = reinterpret_cast<const Plan*>(plan);
   Layout y;
   workspace_layout(desc, p, y);
@@ -838,6 +862,7 @@ int mebptt_lstm_train_step_host(const mebptt_lstm_desc* desc, const mebptt_plan_
   if (desc->want_dx) cudaMemcpyAsync(dx, ws + g.dx, g.ndx, cudaMemcpyDeviceToHost, s);
   cudaMemcpyAsync(counters, ws + g.counters, 8 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
   return cudaGetLastError() == cudaSuccess ? MEBPTT_OK : MEBPTT_ERR_CUDA;
+  }, MEBPTT_ERR_OOM);
 }
 
 int mebptt_lstm_run_times(double* ms, int64_t* launches, int64_t* ops) { return tc::run_times(ms, launches, ops); }
@@ -845,14 +870,16 @@ int mebptt_lstm_run_times(double* ms, int64_t* launches, int64_t* ops) { return 
 int mebptt_lstm_prepare(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
   const int rc = check_common(desc, plan);
   if (rc != MEBPTT_OK) return rc;
-  const Plan* p = reinterpret_cast<const Plan*>(plan);
-  Layout y;
-  workspace_layout(desc, p, y);
-  if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
-  if (y.tensor_path) return tc::prepare_host(y, p, desc->want_dx != 0);
-  if (y.team) return team::prepare_host(y, p);
-  if (y.stepwise_tc || y.stepwise_x3) cut_for(y, p);
-  return MEBPTT_OK;   // operation by operation the plan's tape is walked as it is
+  return guarded([&]() -> int {
+    const Plan* p = reinterpret_cast<const Plan*>(plan);
+    Layout y;
+    workspace_layout(desc, p, y);
+    if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
+    if (y.tensor_path) return tc::prepare_host(y, p, desc->want_dx != 0);
+    if (y.team) return team::prepare_host(y, p);
+    if (y.stepwise_tc || y.stepwise_x3) cut_for(y, p);
+    return MEBPTT_OK;   // operation by operation the plan's tape is walked as it is
+  }, MEBPTT_ERR_OOM);
 }
 
 int mebptt_test_wait_fault(int mask) {

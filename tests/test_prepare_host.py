@@ -101,3 +101,34 @@ def test_every_other_path_has_its_set_built_ahead_of_the_step(route, desc):
     del plan
     gc.collect()
     assert _stats()["held"] == s0["held"]
+
+
+CHILD = r"""
+import resource, sys
+sys.path.insert(0, {root!r})
+from paper_1606_03401_b200 import binding as B
+desc = B.make_desc({desc}, flags={flags})
+plan = B.mebptt_plan(desc.t, 150, B.MEBPTT_HSM)
+held = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (held + (1 << 20), resource.RLIM_INFINITY))
+try:
+    B.mebptt_lstm_prepare(desc, plan)
+    print("STATUS", 0)
+except B.MebpttError as e:
+    print("STATUS", e.status)
+"""
+
+
+@pytest.mark.parametrize("desc,flags", [
+    ('1, 32, 64, 32, 4, 20000, "fp32"', 0),                  # pods
+    ('1, 65, 520, 29, 20, 20000, "bf16"', 4),                # teams
+])
+def test_host_memory_that_runs_out_is_a_status(desc, flags):
+    """No C++ exception leaves the library: a schedule there is no memory for is MEBPTT_ERR_OOM."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", CHILD.format(root=root, desc=desc, flags=flags)], capture_output=True, text=True,
+                         timeout=300)
+    assert out.returncode == 0 and "STATUS %d" % B.MEBPTT_ERR_OOM in out.stdout, (out.returncode, out.stdout, out.stderr[-800:])

@@ -883,7 +883,7 @@ int mebptt_lstm_prepare(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan)
 }
 
 int mebptt_test_wait_fault(int mask) {
-  if (mask < 0 || mask > 7) return MEBPTT_ERR_ARG;
+  if (mask < 0 || mask > 31) return MEBPTT_ERR_ARG;
   tc::set_wait_fault_mask(mask);
   return MEBPTT_OK;
 }

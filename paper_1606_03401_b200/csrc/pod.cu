@@ -55,8 +55,8 @@ __device__ __forceinline__ void push4(uint32_t addr, uint32_t a, uint32_t b, uin
 }
 // (The hint lets the hardware hold the warp until the barrier turns, for 20 us a time, instead of having it
 // poll: sixteen polling warps take issue slots from the ones that still work.)
-__device__ __forceinline__ bool wait_for(uint32_t bar, uint32_t parity) {
-  for (uint32_t i = 0; i < (1u << 16); ++i) {
+__device__ __forceinline__ bool wait_for(uint32_t bar, uint32_t parity, uint32_t polls) {
+  for (uint32_t i = 0; i < polls; ++i) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -296,7 +296,8 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   unsigned char* const ctl = smem + kWindows * kWindow * sizeof(Task);
   uint64_t* const bars = reinterpret_cast<uint64_t*>(ctl);                  // even and odd phases
   uint32_t* const peer = reinterpret_cast<uint32_t*>(ctl + 64);             // where each CTA's shared memory begins
-  volatile int* const dead = reinterpret_cast<volatile int*>(ctl + 128);    // a wait gave up
+  // a wait of an even or odd phase gave up (a thread may be a phase ahead of one that has yet to look)
+  volatile int* const dead = reinterpret_cast<volatile int*>(ctl + 128);
   unsigned char* const area = ctl + 1024;
   uint2* const to = reinterpret_cast<uint2*>(area + C.at_map);              // Share::to
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
   const int u = units_of(rank);
 
   if (tid == 0) {
-    *dead = 0;
+    dead[0] = dead[1] = 0;
     sm100::mbar_init(bars, 1);
     sm100::mbar_init(bars + 1, 1);
     sm100::mbar_fence_init();
@@ -480,7 +481,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     const bool cells = (h0.x >> 8) & 0xff, sums = (h0.x >> 16) & 0xff;
     unsigned char* const dz_buf = area + C.at_dz + (ph & 1) * L * C.dz_buf;
     const uint32_t red_par = (ph & 1) * C.red_bytes;
-    if (ph > 0 && !wait_for(bar0 + 8 * ((ph - 1) & 1), ((ph - 1) >> 1) & 1)) *dead = 1;
+    if (ph > 0 && !wait_for(bar0 + 8 * ((ph - 1) & 1), ((ph - 1) >> 1) & 1, A.polls)) dead[ph & 1] = 1;
 
     // ---- gradients of the own units ----
     if (cells && warp_s) {
@@ -521,7 +522,7 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     }
     if (cells || !sums) {
       __syncthreads();
-      if (*dead) break;
+      if (dead[ph & 1]) break;
     }
 
     // ---- products ----
@@ -558,11 +559,11 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     }
     if (sums) {
       __syncthreads();
-      if (*dead) break;
+      if (dead[ph & 1]) break;
     }
     if (warp == kWarps - 1) {   // the operands have been read: a word to everybody, and what to expect oneself
       if (lane < NT) push(peer[lane] + area0 + C.at_dummy + 4 * rank, 0, peer[lane] + bar);
-      if (lane == 31) sm100::mbar_arrive_expect_tx(bars + (ph & 1), (h0.x >> 24) * by_h + (h0.y & 0xff) * by_p + ((h0.y >> 8) & 0xff) * by_x + 4 * NT);
+      if (lane == 31) sm100::mbar_arrive_expect_tx(bars + (ph & 1), (h0.x >> 24) * by_h + (h0.y & 0xff) * by_p + ((h0.y >> 8) & 0xff) * by_x + 4 * NT + A.extra_bytes);
     }
 
     // ---- states, readouts, loads ----
@@ -648,12 +649,15 @@ __global__ void __launch_bounds__(kThreads, 1) pod_walk(const __grid_constant__ 
     }
   }
   bool ok = ph == A.phases;
-  if (ok && ph > 0) ok = wait_for(bar0 + 8 * ((ph - 1) & 1), ((ph - 1) >> 1) & 1);
+  if (ok && ph > 0) ok = wait_for(bar0 + 8 * ((ph - 1) & 1), ((ph - 1) >> 1) & 1, A.polls);
   if (!ok) *A.status = MEBPTT_ERR_TIMEOUT;
   if (has) *dc_at() = dc;
-  // nobody leaves while pushes to its shared memory may be under way
+  // nobody leaves while pushes to its shared memory may be under way: all of them have arrived, or the wait for
+  // them gave up; then nobody pushes any more behind this barrier, and what is still under way gets time to land
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (!ok)
+    for (int i = 0; i < 1024; ++i) __nanosleep(200);
   if (tid == 0 && blockIdx.x == 0 && ok) {
     A.counters[0] += A.fwd_ops;
     A.counters[1] += A.bwd_ops;

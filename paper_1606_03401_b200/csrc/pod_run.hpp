@@ -25,6 +25,7 @@ struct Args {
   const float *bias, *b_out, *targets;
   const Task* tasks;
   int n_tasks, phases, fwd_ops, bwd_ops;
+  uint32_t polls, extra_bytes;         // a wait gives up after so many polls of 20 us; bytes a phase expects and nobody sends (testing aid)
   int* status;
   int64_t* counters;
 };

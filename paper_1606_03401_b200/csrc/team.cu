@@ -51,6 +51,7 @@ struct Args {
   int n_tasks;
   unsigned* sync;                      // one 128-byte line per team
   unsigned sync_base;                  // arrivals before this launch, per team
+  unsigned polls;                      // a wait gives up after so many polls
   int* status;
   int64_t* counters;
 };
@@ -224,7 +225,10 @@ __device__ __forceinline__ bool meet(const Args& A, unsigned* line, unsigned tar
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(line) : "memory");
       if ((int)(v - target) >= 0) { ok = true; break; }
-      if (i > 256) __nanosleep(32);
+      if (i > 256) {
+        if (i >= A.polls) break;
+        __nanosleep(32);
+      }
     }
     if (!ok) { *A.status = MEBPTT_ERR_TIMEOUT; *flag = 1; }
   }
@@ -1130,6 +1134,7 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
   }
 
   Args a{};
+  unsigned met = 0;            // arrivals of a team before a launch
   pod::Args pa{};
   WalkFn fn = nullptr;
   pod::Fn pf = nullptr;
@@ -1147,6 +1152,9 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
   if (pods) {
     common(pa);
     pa.stages = io.ws + y.off_dz;
+    const bool fault = tc::wait_fault_mask() & 8;
+    pa.polls = fault ? 64 : 1u << 16;
+    pa.extra_bytes = fault ? 16 : 0;
     pa.c = pc;
     const size_t states = (size_t)y.n_blocks * (block_bytes(pc.nb, y.H, y.esz, y.parts) / y.parts);
     pf = pod::kernel(y.dtype, y.gru, pc.nb, states >> 32 != 0 || y.parts > 1);
@@ -1157,6 +1165,9 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
     for (int l = 0; l < y.L; ++l) { a.ns_f[l] = c.ns_f[l]; a.ns_b[l] = c.ns_b[l]; a.off_wb[l] = y.off_wb[l]; }
     a.ns_r = c.ns_r; a.resident = c.resident; a.pool_floats = c.pool_floats;
     a.sync = reinterpret_cast<unsigned*>(io.ws + y.off_sync);
+    const bool fault = tc::wait_fault_mask() & 16;
+    a.polls = fault ? tc::fault_poll_limit : sm100::kSpinLimit;
+    met = fault ? 1 : 0;   // (arrivals that nobody makes)
     fn = walk_fn(y, c.nb);
     if (allow(reinterpret_cast<const void*>(fn)) != cudaSuccess) { cudaGetLastError(); return MEBPTT_ERR_CUDA; }
   }
@@ -1167,7 +1178,6 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
   const size_t room = y.tape_bytes / sizeof(Task);
   size_t up_lo = 0, up_hi = 0;   // tasks that lie in the region
   bool first = true;
-  unsigned met = 0;
   Products P;
   for (size_t i = 0; i < ls.size(); ++i) {
     const Launch& g = ls[i];
@@ -1187,8 +1197,8 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
       } else {
         a.tasks = region + (g.task0 - up_lo);
         a.n_tasks = (int)g.ntasks;
-        a.sync_base = met * (unsigned)c.T;
-        met += (unsigned)g.phases;
+        a.sync_base = met;
+        met += (unsigned)g.phases * (unsigned)c.T;
         void* args[1] = {&a};
         rc = launch(reinterpret_cast<const void*>(fn), c.teams * c.T, 0, c.smem, args, s);
       }

@@ -228,9 +228,10 @@ def test_run_times_count_every_backward_operation_and_change_no_result(H):
                                    dict(layers=1, input=128, hidden=1152, batch=64, t=9, readout=64),
                                    dict(layers=1, input=64, hidden=128, batch=128, t=17, readout=72)])
 def test_stepwise_tensor_core_path_matches_oracle_and_cuda_core_path(H, shape):
-    """bf16 shapes outside the persistent kernels' range (several layers, H > 1024, B > 64): every
-    operation is a sequence of launches whose contractions run on the tensor cores.  Oracle
-    parity, bit identity across plans, agreement with the CUDA-core kernels."""
+    """bf16 shapes outside the persistent kernels' range (several layers, H > 1024, B > 64), on the
+    tensor cores: the wide one as a sequence of launches per operation, the narrow ones as walked
+    tapes (test_gpu_stepwise.py has more of the former).  Oracle parity, bit identity across plans,
+    agreement with the CUDA-core kernels."""
     from paper_1606_03401_b200 import binding as B
     from tests.util import rel_l2
     cfg = _cfg("c2", **shape)
@@ -259,8 +260,8 @@ def test_stepwise_tensor_core_path_matches_oracle_and_cuda_core_path(H, shape):
                                    dict(layers=3, input=24, hidden=64, batch=96, t=23, readout=8),
                                    dict(layers=2, input=128, hidden=2048, batch=128, t=19, readout=128)])
 def test_stepwise_runs_give_the_bits_of_single_operations(H, shape, monkeypatch):
-    """The step-by-step tensor-core path takes runs of consecutive operations one layer at a time,
-    with the input products, the readout and the gradients handed down batched over the run (at
+    """The step-by-step tensor-core path (the widest shape here; the narrow ones are walked as tapes,
+    and test_gpu_stepwise.py has others) takes runs of consecutive operations one layer at a time, with the input products, the readout and the gradients handed down batched over the run (at
     config 5's widths some of those contractions are split along K).  Operation by operation
     (MEBPTT_STEPWISE_PER_OP=1) every sum must come out the same, bit for bit, under long runs and
     short ones, with and without dx."""
@@ -281,7 +282,8 @@ def test_stepwise_runs_give_the_bits_of_single_operations(H, shape, monkeypatch)
                                    dict(layers=1, input=256, hidden=1024, batch=32, t=70, readout=256)])
 def test_float32_storage_run_readout_gives_the_bits_of_single_operations(H, shape, monkeypatch):
     """With float32 storage the readout of a run of backward operations is taken for the whole run
-    at once; operation by operation (MEBPTT_STEPWISE_PER_OP=1) the bits must be the same."""
+    at once; operation by operation (MEBPTT_STEPWISE_PER_OP=1) the bits must be the same.  (The wide
+    shape; the narrow one is walked as a tape, and test_gpu_stepwise.py has networks of several layers.)"""
     cfg = _cfg("c4", **shape)
     dp = H.DeviceProblem(cfg, want_dx=True)
     plans = [dp.full_memory_plan(), dp.plan("msm", 11), dp.plan("ism", 3), dp.plan("hsm", 2)]
@@ -300,7 +302,8 @@ def test_float32_storage_run_readout_gives_the_bits_of_single_operations(H, shap
 def test_float32_storage_on_tensor_cores_matches_oracle_within_1e_4(H, shape):
     """The tf32 data type: float32 storage, contractions on the tensor cores as three bfloat16
     products per float32 product.  Oracle parity at the float32 tolerance, bit identity across
-    plans, agreement with the float32 FMA kernels."""
+    plans, agreement with the float32 FMA kernels.  (The narrow shapes are walked as tapes, in FMA
+    arithmetic; test_gpu_stepwise.py has more of the others.)"""
     from paper_1606_03401_b200 import binding as B
     from tests.util import rel_l2
     cfg = _cfg("c4", **shape)
@@ -424,15 +427,15 @@ def test_c5_full_size_properties(H):
 
 
 GENERAL_CASES = [
-    # CUDA-core path (float32)
+    # a tape walked in pods (float32)
     ("c1", dict(t=24)),
     # persistent tensor path, config 2's widths, more than two staged chunks of S = 32 steps
     ("c2", dict(t=70)),
     # persistent tensor path, batch below the tile height and a hidden size that is no multiple of 64
     ("c2", dict(input=72, hidden=200, batch=24, t=37, readout=40)),
-    # step-by-step bf16 path, two layers, more than two chunks of S = 32 steps
+    # a tape walked in pods, bf16, two layers, more than one chunk
     ("c5", dict(layers=2, input=64, hidden=72, batch=32, t=70, readout=40)),
-    # step-by-step path for float32 storage, more than two chunks
+    # tapes walked in pods, float32 storage
     ("c4", dict(layers=1, input=64, hidden=128, batch=32, t=70, readout=40)),
     ("c4", dict(layers=2, input=40, hidden=72, batch=32, t=37, readout=24)),
 ]
@@ -443,7 +446,7 @@ def test_general_biases_and_initial_state_match_oracle_on_every_path(H, base, kw
     """Every bias entry, the readout bias and the initial state drawn at random (the benchmark
     recipe leaves them at constants, which cannot expose a misplaced bias entry, a dropped readout
     bias or a mishandled caller's (h0, c0)): oracle parity per tensor and per block with dx, under
-    full memory and one plan of each kind, on each of the four kernel paths."""
+    full memory and one plan of each kind, (the step-by-step paths: test_gpu_stepwise.py)."""
     cfg = _cfg(base, **kw)
     prob = synth.make_problem(cfg, general=True)
     assert np.abs(prob["b_out"]).min() > 0 and np.abs(prob["h0"]).max() > 0.5 and np.abs(prob["c0"]).max() > 0.5
@@ -498,11 +501,11 @@ def test_c5_shape_across_chunks_against_oracle_with_byte_budget(H):
 
 
 @pytest.mark.parametrize("base,kw,plans", [
-    ("c1", dict(t=20), [("hsm", 4), ("msm", 9)]),                                                   # CUDA-core path
-    ("c1", dict(t=20, layers=2, cell="gru"), [("msm", 9)]),                                          # CUDA-core path, GRU core
+    ("c1", dict(t=20), [("hsm", 4), ("msm", 9)]),                                                   # pods
+    ("c1", dict(t=20, layers=2, cell="gru"), [("msm", 9)]),                                          # pods, GRU core
     ("c2", dict(input=128, hidden=256, batch=64, t=70, readout=128), [("hsm", 5), ("msm", 13), ("ism", 70)]),  # persistent tensor path
-    ("c5", dict(layers=2, input=64, hidden=72, batch=32, t=45, readout=40), [("msm", 11), ("ism", 45)]),      # step by step, bf16
-    ("c4", dict(layers=1, input=64, hidden=128, batch=32, t=45, readout=40), [("msm", 11), ("ism", 45)]),     # step by step, float32 storage
+    ("c5", dict(layers=2, input=64, hidden=72, batch=32, t=45, readout=40), [("msm", 11), ("ism", 45)]),      # pods, bf16
+    ("c4", dict(layers=1, input=64, hidden=128, batch=32, t=45, readout=40), [("msm", 11), ("ism", 45)]),     # pods, float32 storage
 ])
 def test_launch_count_is_what_the_profiler_sees(H, base, kw, plans):
     """mebptt_lstm_launch_count (the benchmark's gpu_launches) against the kernels CUPTI records for
@@ -569,7 +572,7 @@ def test_prepared_set_is_reused_per_workspace_and_the_enqueue_is_cheap(H):
 
 @pytest.mark.parametrize("base,kw", [
     ("c2", dict(input=128, hidden=256, batch=64, t=70, readout=128)),                  # persistent tensor path
-    ("c5", dict(layers=2, input=64, hidden=128, batch=32, t=45, readout=40)),           # step by step, bf16, two layers
+    ("c5", dict(layers=2, input=64, hidden=128, batch=32, t=45, readout=40)),           # pods, bf16, two layers
     ("c1", dict(t=24)),                                                                 # float32: sizes 1 : 4 : 3
 ])
 def test_plans_over_the_layouts_byte_sizes_give_the_same_gradients(H, base, kw):

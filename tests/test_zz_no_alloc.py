@@ -34,7 +34,7 @@ def _static_run(dp, plan):
 
 
 @pytest.mark.parametrize("base,kw,mode,m", [
-    ("c1", dict(), "hsm", 8),                                                      # fp32, CUDA-core kernels
+    ("c1", dict(), "hsm", 8),                                                      # fp32, a walked tape
     ("c2", dict(input=64, hidden=128, batch=32, t=40, readout=64), "msm", 9),      # bf16, tensor-core kernels
 ])
 def test_static_workspace_step_matches_ordinary_step_twice(base, kw, mode, m):

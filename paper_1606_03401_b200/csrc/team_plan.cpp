@@ -137,9 +137,13 @@ Config choose_config(const Layout& y, int sms) {
 // cycles of two forward operations and a backward one.  Step by step these take some 45 us a layer
 // whatever the widths (three or four dependent launches each; measured from 160 to 1024 units), and stay
 // ahead where the recurrent weights are large.  The persistent kernels for float32 storage take some
-// 20 us and a launch or several a run: at H = 160, B = 32 (estimated 29600) both were within a
-// fifth of each other, at 224 units and 64 rows or 304 and 32 (43700 and up) those were 1.1 to 1.4 times
-// faster under every plan.
+// 20 us and a launch or several a run.  Measured on both sides of the line (150 steps, input and readout as
+// wide, us under HSM 20, ISM 20, MSM 30 and full memory; walked, then runs):
+//   H = 192, B = 32 (estimated 29200)  3478 2606 2874 1907   3655 2712 3559 1804
+//   H = 160, B = 64 (31000)            4137 3139 3413 2378   3988 2997 3841 2099
+//   H = 208, B = 32 (32000)            3613 2764 2988 2079   3884 2840 3791 1850
+//   H = 224, B = 32 (33200)            3787 2932 3155 2200   3759 2756 3634 1827
+//   H = 176, B = 64 (34700)            4599 3505 3797 2665   4238 3142 4114 2141
 bool supported(const mebptt_lstm_desc* d) {
   constexpr double kStepwise = 70000.0;   // a fifth less than measured, to be worth leaving
   constexpr double kRuns = 33000.0;

@@ -64,7 +64,7 @@ struct States {
   __host__ __device__ States(char* all, int64_t n, int parts_, int group, int R, int B, int H)
       : base(all + (size_t)group * n * (block(R, H, parts_) / parts_)), hs(block(R < B - group * R ? R : B - group * R, H, parts_)), part(hs / parts_),
         parts(parts_) {}
-  __host__ __device__ char* at(uint32_t loc, int blocks) const { return base + (size_t)loc * part + (size_t)blocks * hs; }
+  __host__ __device__ char* at(uint32_t loc, int blocks) const { return base + (size_t)(loc + (uint32_t)(blocks * parts)) * part; }
   __host__ __device__ T* h(uint32_t loc, int l) const { return reinterpret_cast<T*>(at(loc, l * (1 + CR))); }
   __host__ __device__ float* c(uint32_t loc, int l) const { return reinterpret_cast<float*>(at(loc, l * (1 + CR) + 1)); }
   __host__ __device__ T* gate(uint32_t loc, int L, int l, int q) const { return reinterpret_cast<T*>(at(loc, L * (1 + CR) + 4 * l + q)); }

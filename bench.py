@@ -348,7 +348,7 @@ def main():
         dp.desc.flags &= ~B.MEBPTT_FLAG_TIME_RUNS
         runs = B.mebptt_lstm_run_times()
         if runs["forward"][1] == 0:
-            runs = None     # the shape runs on the CUDA-core path
+            runs = None     # another path serves the shape
     if runs:
         f_ms, f_n, f_ops = runs["forward"]
         b_ms, b_n, b_ops = runs["backward"]
@@ -379,9 +379,13 @@ def main():
         achieved = flops_fwd_op / (fwd_op_ms * 1e-3) / 1e12 if fwd_op_ms else None
         roofline = {"bound": "tensor", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": (achieved / peak_tf) if achieved else None, "traffic": None,
-                    "kernel": ("forward operation, step by step (per layer: two tensor-core GEMMs and a cell kernel)"
-                               if cfg.dtype == "bf16" and not (cfg.batch % 32) else
-                               "forward operation on the CUDA-core path (gate contraction + cell update in one launch per layer)"),
+                    "kernel": "forward operation " + {
+                        "pods": "inside pod_walk (whole tapes, a cluster of CTAs per group of batch rows)",
+                        "teams": "inside walk (whole tapes, a cooperative grid)",
+                        "runs_f32": "inside fwd_run_x3 (a run of forward operations, float32 storage)",
+                        "stepwise": "step by step (per layer: two tensor-core GEMMs and a cell kernel)",
+                        "stepwise_f32": "step by step (per layer: split operands, a tensor-core GEMM and a cell kernel)",
+                    }.get(B.mebptt_test_route(dp.desc, plan)["route"], "on the CUDA cores (a launch per layer)"),
                     "how": "(T(m) - T(full memory)) / (C(t,m) - t) = duration of one forward operation; "
                            f"{flops_fwd_op} flops per operation; peak = bf16 sustained ({pk['source']})"
                            + ("" if cfg.dtype == "bf16" else " / 2: float32 storage takes three bf16 MMAs per product, so the "

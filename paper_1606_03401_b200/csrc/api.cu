@@ -654,79 +654,79 @@ size_t mebptt_lstm_working_bytes(const mebptt_lstm_desc* desc, const mebptt_plan
 int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan) {
   if (check_common(desc, plan) != MEBPTT_OK) return -1;
   return guarded([&]() -> int64_t {
-  const Plan* p = reinterpret_cast<const Plan*>(plan);
-  Layout y;
-  workspace_layout(desc, p, y);
-  if (y.tensor_path) return tc::run_step(y, p, StepIO{}, desc->want_dx != 0, nullptr, true, false);
-  if (y.team) return team::run_step(y, p, StepIO{}, desc->want_dx != 0, nullptr, true);
-  // forward operation: one kernel per layer; backward operation: 5 for the readout and
-  // 4 per layer; one to finalise
-  const int64_t L = desc->layers;
-  if (y.stepwise_tc) {
-    // forward operation: two GEMMs and the cell kernel per layer; readout: GEMM with loss, loss
-    // term and stage, dha GEMM; backward operation per layer: gate kernel and one or two d_in GEMMs
-    // (a contraction that is split along K takes a second launch to add its parts)
-    const size_t pf = (size_t)148 * 128 * 128;
-    const int G = 4 * y.H;
-    const int64_t to_h = tc::gemm_split_count(false, true, y.B, y.H, G, pf) > 1 ? 2 : 1;   // dz W -> [B][H]
-    const int64_t to_x = tc::gemm_split_count(false, true, y.B, y.I, G, pf) > 1 ? 2 : 1;   // dz W -> [B][I]
-    const int64_t dha = tc::gemm_split_count(false, true, y.B, y.H, y.O, pf) > 1 ? 2 : 1;
-    // (the recurrent dh = dz W_hh is one launch in any case: its parts are added by the next gate kernel)
-    const int64_t bwd = L + L + to_h * (L - 1) + (desc->want_dx ? to_x : 0);
-    const int64_t chunks = (p->t + y.S - 1) / y.S;   // each flushed by 2 L + 1 GEMMs and L + 1 bias sums
-    // runs of n >= 2 operations go layer by layer: one input product per layer and run, the
-    // readout once per run (stage, GEMM with loss, loss terms, dha), the gradient handed down
-    // once per layer and run
-    int64_t n_launch = chunks * (3 * L + 2) + 1;
-    const std::shared_ptr<const Cut> cut = cut_for(y, p);
-    for (const WorkItem& wi : cut->items) {
-      if (wi.kind == WorkItem::LEAF) n_launch += wi.n * (3 * L + 2 + dha + bwd);
-      else if (wi.kind == WorkItem::FWD) n_launch += wi.n == 1 ? 3 * L : L * (1 + 2 * (int64_t)wi.n);
-      else if (wi.n == 1) n_launch += 2 + dha + bwd;
-      else n_launch += 3 + dha + L * wi.n * 2 + (L - 1) * to_h + (desc->want_dx ? to_x : 0);
-    }
-    return n_launch;
-  }
-  if (y.stepwise_x3) {
-    // weights: 2 packing kernels per layer and 2 for the readout; forward operation: split, GEMM,
-    // cell per layer; readout: split, GEMM, loss sum, dha GEMM; backward operation per
-    // layer: gate kernel, one or two d_in GEMMs; a chunk: 3 GEMMs per product and L + 1 bias sums
-    const size_t pf = (size_t)148 * 128 * 128;
-    const int G = 4 * y.H;
-    const int64_t to_h = tc::gemm_split_count(false, true, y.B, y.H, 3 * G, pf) > 1 ? 2 : 1;
-    const int64_t to_x = tc::gemm_split_count(false, true, y.B, y.I, 3 * G, pf) > 1 ? 2 : 1;
-    const int64_t dha = tc::gemm_split_count(false, true, y.B, y.H, 3 * y.O, pf) > 1 ? 2 : 1;
-    const int64_t bwd = L + L + to_h * (L - 1) + (desc->want_dx ? to_x : 0);   // dh = dz W_hh: one launch in any case
-    const int64_t chunks = (p->t + y.S - 1) / y.S;
-    if (y.x3_runs) {
-      // packing; a window of projections: split and GEMM; forward run: one; backward run: readout of two
-      // and dha, run, d_in; a batch of leaves: split, GEMM, states, two GEMMs, cells before that; chunks as below
-      int64_t n = 5 + (desc->want_dx ? 1 : 0) + chunks * 11 + 1;
+    const Plan* p = reinterpret_cast<const Plan*>(plan);
+    Layout y;
+    workspace_layout(desc, p, y);
+    if (y.tensor_path) return tc::run_step(y, p, StepIO{}, desc->want_dx != 0, nullptr, true, false);
+    if (y.team) return team::run_step(y, p, StepIO{}, desc->want_dx != 0, nullptr, true);
+    // forward operation: one kernel per layer; backward operation: 5 for the readout and
+    // 4 per layer; one to finalise
+    const int64_t L = desc->layers;
+    if (y.stepwise_tc) {
+      // forward operation: two GEMMs and the cell kernel per layer; readout: GEMM with loss, loss
+      // term and stage, dha GEMM; backward operation per layer: gate kernel and one or two d_in GEMMs
+      // (a contraction that is split along K takes a second launch to add its parts)
+      const size_t pf = (size_t)148 * 128 * 128;
+      const int G = 4 * y.H;
+      const int64_t to_h = tc::gemm_split_count(false, true, y.B, y.H, G, pf) > 1 ? 2 : 1;   // dz W -> [B][H]
+      const int64_t to_x = tc::gemm_split_count(false, true, y.B, y.I, G, pf) > 1 ? 2 : 1;   // dz W -> [B][I]
+      const int64_t dha = tc::gemm_split_count(false, true, y.B, y.H, y.O, pf) > 1 ? 2 : 1;
+      // (the recurrent dh = dz W_hh is one launch in any case: its parts are added by the next gate kernel)
+      const int64_t bwd = L + L + to_h * (L - 1) + (desc->want_dx ? to_x : 0);
+      const int64_t chunks = (p->t + y.S - 1) / y.S;   // each flushed by 2 L + 1 GEMMs and L + 1 bias sums
+      // runs of n >= 2 operations go layer by layer: one input product per layer and run, the
+      // readout once per run (stage, GEMM with loss, loss terms, dha), the gradient handed down
+      // once per layer and run
+      int64_t n_launch = chunks * (3 * L + 2) + 1;
       const std::shared_ptr<const Cut> cut = cut_for(y, p);
-      const std::vector<WorkItem>& items = cut->items;
-      const std::vector<int>& windows = cut->windows;
-      const int64_t back = 3 + dha + (desc->want_dx ? to_x : 0);
-      for (size_t i = 0; i < items.size(); ++i) {
-        if (items[i].kind == WorkItem::FWD) n += 1 + (windows[i] ? 2 : 0);
-        else if (items[i].kind == WorkItem::BWD) n += back;
-        else n += (items[i].n + stepwise3::X3_LEAVES - 1) / stepwise3::X3_LEAVES * (6 + back);
+      for (const WorkItem& wi : cut->items) {
+        if (wi.kind == WorkItem::LEAF) n_launch += wi.n * (3 * L + 2 + dha + bwd);
+        else if (wi.kind == WorkItem::FWD) n_launch += wi.n == 1 ? 3 * L : L * (1 + 2 * (int64_t)wi.n);
+        else if (wi.n == 1) n_launch += 2 + dha + bwd;
+        else n_launch += 3 + dha + L * wi.n * 2 + (L - 1) * to_h + (desc->want_dx ? to_x : 0);
       }
-      return n;
+      return n_launch;
     }
-    // the readout of a run of n >= 2 backward operations is taken once for the run (the same
-    // launches), and a run of n >= 2 forward operations splits its operands once per layer (then
-    // GEMM and cell kernel per step)
-    int64_t readouts = 0, forwards = 0;
-    const std::shared_ptr<const Cut> cut = cut_for(y, p);
-    for (const WorkItem& wi : cut->items) {
-      if (wi.kind == WorkItem::LEAF) { readouts += wi.n * (3 + dha); forwards += wi.n * 3 * L; }
-      else if (wi.kind == WorkItem::BWD) readouts += 3 + dha;
-      else forwards += wi.n == 1 ? 3 * L : L * (1 + 2 * (int64_t)wi.n);
+    if (y.stepwise_x3) {
+      // weights: 2 packing kernels per layer and 2 for the readout; forward operation: split, GEMM,
+      // cell per layer; readout: split, GEMM, loss sum, dha GEMM; backward operation per
+      // layer: gate kernel, one or two d_in GEMMs; a chunk: 3 GEMMs per product and L + 1 bias sums
+      const size_t pf = (size_t)148 * 128 * 128;
+      const int G = 4 * y.H;
+      const int64_t to_h = tc::gemm_split_count(false, true, y.B, y.H, 3 * G, pf) > 1 ? 2 : 1;
+      const int64_t to_x = tc::gemm_split_count(false, true, y.B, y.I, 3 * G, pf) > 1 ? 2 : 1;
+      const int64_t dha = tc::gemm_split_count(false, true, y.B, y.H, 3 * y.O, pf) > 1 ? 2 : 1;
+      const int64_t bwd = L + L + to_h * (L - 1) + (desc->want_dx ? to_x : 0);   // dh = dz W_hh: one launch in any case
+      const int64_t chunks = (p->t + y.S - 1) / y.S;
+      if (y.x3_runs) {
+        // packing; a window of projections: split and GEMM; forward run: one; backward run: readout of two
+        // and dha, run, d_in; a batch of leaves: split, GEMM, states, two GEMMs, cells before that; chunks as below
+        int64_t n = 5 + (desc->want_dx ? 1 : 0) + chunks * 11 + 1;
+        const std::shared_ptr<const Cut> cut = cut_for(y, p);
+        const std::vector<WorkItem>& items = cut->items;
+        const std::vector<int>& windows = cut->windows;
+        const int64_t back = 3 + dha + (desc->want_dx ? to_x : 0);
+        for (size_t i = 0; i < items.size(); ++i) {
+          if (items[i].kind == WorkItem::FWD) n += 1 + (windows[i] ? 2 : 0);
+          else if (items[i].kind == WorkItem::BWD) n += back;
+          else n += (items[i].n + stepwise3::X3_LEAVES - 1) / stepwise3::X3_LEAVES * (6 + back);
+        }
+        return n;
+      }
+      // the readout of a run of n >= 2 backward operations is taken once for the run (the same
+      // launches), and a run of n >= 2 forward operations splits its operands once per layer (then
+      // GEMM and cell kernel per step)
+      int64_t readouts = 0, forwards = 0;
+      const std::shared_ptr<const Cut> cut = cut_for(y, p);
+      for (const WorkItem& wi : cut->items) {
+        if (wi.kind == WorkItem::LEAF) { readouts += wi.n * (3 + dha); forwards += wi.n * 3 * L; }
+        else if (wi.kind == WorkItem::BWD) readouts += 3 + dha;
+        else forwards += wi.n == 1 ? 3 * L : L * (1 + 2 * (int64_t)wi.n);
+      }
+      return 2 * L + 2 + forwards + readouts + p->t * bwd + chunks * (3 * (2 * L + 1) + L + 1) + 1;
     }
-    return 2 * L + 2 + forwards + readouts + p->t * bwd + chunks * (3 * (2 * L + 1) + L + 1) + 1;
-  }
-  // (a GRU layer's backward operation takes two launches more: its weight gradient comes in three blocks)
-  return p->cost * L + p->t * (5 + (y.gru ? 6 : 4) * L) + 1;
+    // (a GRU layer's backward operation takes two launches more: its weight gradient comes in three blocks)
+    return p->cost * L + p->t * (5 + (y.gru ? 6 : 4) * L) + 1;
   }, -1);
 }
 
@@ -766,19 +766,19 @@ int train_step_impl(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, con
   if (!loss || !dW || !db || !dW_out || !db_out || !counters) return MEBPTT_ERR_ARG;
   if (desc->want_dx && !dx) return MEBPTT_ERR_ARG;
   return guarded([&]() -> int {
-  const Plan* p = reinterpret_cast<const Plan*>(plan);
-  Layout y;
-  if (side_stream) workspace_layout(desc, p, y);
-  else fitted_layout(desc, plan, workspace_bytes, y);   // (the entry point with a fixed workspace)
-  if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
-  if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < y.total)
-    return MEBPTT_ERR_WORKSPACE;
-  StepIO io{(const char*)W, (const char*)W_out, (const char*)x, (const char*)h0,
-            (const float*)b, (const float*)b_out, (const float*)targets, (const float*)c0,
-            (char*)workspace, loss, dW, db, dW_out, db_out, dx, counters};
-  io.time_runs = (desc->flags & MEBPTT_FLAG_TIME_RUNS) != 0;
-  io.pageable_tape = !side_stream;   // the allocation-free entry point (the only caller without side stream) locks no pages
-  return run_step(desc, p, y, io, (cudaStream_t)stream, side_stream);
+    const Plan* p = reinterpret_cast<const Plan*>(plan);
+    Layout y;
+    if (side_stream) workspace_layout(desc, p, y);
+    else fitted_layout(desc, plan, workspace_bytes, y);   // (the entry point with a fixed workspace)
+    if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
+    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < y.total)
+      return MEBPTT_ERR_WORKSPACE;
+    StepIO io{(const char*)W, (const char*)W_out, (const char*)x, (const char*)h0,
+              (const float*)b, (const float*)b_out, (const float*)targets, (const float*)c0,
+              (char*)workspace, loss, dW, db, dW_out, db_out, dx, counters};
+    io.time_runs = (desc->flags & MEBPTT_FLAG_TIME_RUNS) != 0;
+    io.pageable_tape = !side_stream;   // the allocation-free entry point (the only caller without side stream) locks no pages
+    return run_step(desc, p, y, io, (cudaStream_t)stream, side_stream);
   }, MEBPTT_ERR_OOM);
 }
 }  // namespace mebptt
@@ -817,51 +817,51 @@ int mebptt_lstm_train_step_host(const mebptt_lstm_desc* desc, const mebptt_plan_
   if (!loss || !dW || !db || !dW_out || !db_out || !counters) return MEBPTT_ERR_ARG;
   if (desc->want_dx && !dx) return MEBPTT_ERR_ARG;
   return guarded([&]() -> int {
-  const Plan* p = reinterpret_cast<const Plan*>(plan);
-  Layout y;
-  workspace_layout(desc, p, y);
-  if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
-  Staging g;
-  staging_layout(y, desc->want_dx != 0, y.total, g);
-  if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < g.total)
-    return MEBPTT_ERR_WORKSPACE;
-  char* ws = (char*)workspace;
-  cudaStream_t s = (cudaStream_t)stream;
-  cudaMemcpyAsync(ws + g.W, W, g.nW, cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(ws + g.b, b, g.nb, cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(ws + g.W_out, W_out, g.nW_out, cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(ws + g.b_out, b_out, g.nb_out, cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(ws + g.h0, h0, g.nh0, cudaMemcpyHostToDevice, s);
-  cudaMemcpyAsync(ws + g.c0, c0, g.nc0, cudaMemcpyHostToDevice, s);
-  // x is read progressively by the forward pass and the targets not before the first backward
-  // operation: the tensor-core path copies both beside the forward pass
-  const bool late_targets = y.tensor_path && !env::no_overlap();
-  if (!late_targets) {
-    cudaMemcpyAsync(ws + g.x, x, g.nx, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(ws + g.targets, targets, g.ntargets, cudaMemcpyHostToDevice, s);
-  }
-  if (cudaGetLastError() != cudaSuccess) return MEBPTT_ERR_CUDA;
-  StepIO io{ws + g.W, ws + g.W_out, ws + g.x, ws + g.h0,
-            (const float*)(ws + g.b), (const float*)(ws + g.b_out), (const float*)(ws + g.targets),
-            (const float*)(ws + g.c0), ws,
-            (float*)(ws + g.loss), (float*)(ws + g.dW), (float*)(ws + g.db), (float*)(ws + g.dW_out),
-            (float*)(ws + g.db_out), desc->want_dx ? (float*)(ws + g.dx) : nullptr,
-            (int64_t*)(ws + g.counters)};
-  if (late_targets) {
-    io.targets_host = targets; io.targets_bytes = g.ntargets;
-    io.x_host = x; io.x_bytes = g.nx;
-  }
-  io.time_runs = (desc->flags & MEBPTT_FLAG_TIME_RUNS) != 0;
-  rc = run_step(desc, p, y, io, s);
-  if (rc != MEBPTT_OK) return rc;
-  cudaMemcpyAsync(loss, ws + g.loss, 4, cudaMemcpyDeviceToHost, s);
-  cudaMemcpyAsync(dW, ws + g.dW, y.w_total_elems() * 4, cudaMemcpyDeviceToHost, s);
-  cudaMemcpyAsync(db, ws + g.db, g.nb, cudaMemcpyDeviceToHost, s);
-  cudaMemcpyAsync(dW_out, ws + g.dW_out, (size_t)y.O * y.H * 4, cudaMemcpyDeviceToHost, s);
-  cudaMemcpyAsync(db_out, ws + g.db_out, g.nb_out, cudaMemcpyDeviceToHost, s);
-  if (desc->want_dx) cudaMemcpyAsync(dx, ws + g.dx, g.ndx, cudaMemcpyDeviceToHost, s);
-  cudaMemcpyAsync(counters, ws + g.counters, 8 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-  return cudaGetLastError() == cudaSuccess ? MEBPTT_OK : MEBPTT_ERR_CUDA;
+    const Plan* p = reinterpret_cast<const Plan*>(plan);
+    Layout y;
+    workspace_layout(desc, p, y);
+    if (!addressable(y)) return MEBPTT_ERR_UNSUPPORTED;
+    Staging g;
+    staging_layout(y, desc->want_dx != 0, y.total, g);
+    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) || workspace_bytes < g.total)
+      return MEBPTT_ERR_WORKSPACE;
+    char* ws = (char*)workspace;
+    cudaStream_t s = (cudaStream_t)stream;
+    cudaMemcpyAsync(ws + g.W, W, g.nW, cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(ws + g.b, b, g.nb, cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(ws + g.W_out, W_out, g.nW_out, cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(ws + g.b_out, b_out, g.nb_out, cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(ws + g.h0, h0, g.nh0, cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(ws + g.c0, c0, g.nc0, cudaMemcpyHostToDevice, s);
+    // x is read progressively by the forward pass and the targets not before the first backward
+    // operation: the tensor-core path copies both beside the forward pass
+    const bool late_targets = y.tensor_path && !env::no_overlap();
+    if (!late_targets) {
+      cudaMemcpyAsync(ws + g.x, x, g.nx, cudaMemcpyHostToDevice, s);
+      cudaMemcpyAsync(ws + g.targets, targets, g.ntargets, cudaMemcpyHostToDevice, s);
+    }
+    if (cudaGetLastError() != cudaSuccess) return MEBPTT_ERR_CUDA;
+    StepIO io{ws + g.W, ws + g.W_out, ws + g.x, ws + g.h0,
+              (const float*)(ws + g.b), (const float*)(ws + g.b_out), (const float*)(ws + g.targets),
+              (const float*)(ws + g.c0), ws,
+              (float*)(ws + g.loss), (float*)(ws + g.dW), (float*)(ws + g.db), (float*)(ws + g.dW_out),
+              (float*)(ws + g.db_out), desc->want_dx ? (float*)(ws + g.dx) : nullptr,
+              (int64_t*)(ws + g.counters)};
+    if (late_targets) {
+      io.targets_host = targets; io.targets_bytes = g.ntargets;
+      io.x_host = x; io.x_bytes = g.nx;
+    }
+    io.time_runs = (desc->flags & MEBPTT_FLAG_TIME_RUNS) != 0;
+    rc = run_step(desc, p, y, io, s);
+    if (rc != MEBPTT_OK) return rc;
+    cudaMemcpyAsync(loss, ws + g.loss, 4, cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(dW, ws + g.dW, y.w_total_elems() * 4, cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(db, ws + g.db, g.nb, cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(dW_out, ws + g.dW_out, (size_t)y.O * y.H * 4, cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(db_out, ws + g.db_out, g.nb_out, cudaMemcpyDeviceToHost, s);
+    if (desc->want_dx) cudaMemcpyAsync(dx, ws + g.dx, g.ndx, cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(counters, ws + g.counters, 8 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+    return cudaGetLastError() == cudaSuccess ? MEBPTT_OK : MEBPTT_ERR_CUDA;
   }, MEBPTT_ERR_OOM);
 }
 

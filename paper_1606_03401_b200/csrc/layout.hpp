@@ -315,7 +315,8 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     const size_t rows = (size_t)y.S * y.B;
     // States: a group of batch rows walks the tape without waiting for the others, so each has an arena of
     // its own -- in one arena for all rows what one group writes for a later operation would lie over another
-    // group's rows of an earlier one.  Sizes are those of the common layout without its rounding to granules.  The working core alternates between two buffers, so that one leaf's forward operation can
+    // group's rows of an earlier one.  Sizes are those of the common layout without its rounding to granules.
+    // The working core alternates between two buffers, so that one leaf's forward operation can
     // pass the last one's backward.
     const int cr = (int)(4 / y.esz);
     y.unit_blocks = y.L * (1 + cr);

@@ -40,7 +40,7 @@ constexpr size_t kMaxLaunchTasks = 32768;   // 1 MB of tasks per launch at most:
 
 // Where the tape is walked, the weight gradients of so many time steps (at least 256 rows) are summed by
 // themselves and then added to those of later steps, however many steps a chunk has: chunks can be cut short
-// where memory is, without a change in a bit.  (128 rows: GRU 2 x 256 2867 -> 2882 us, 2 x 300 4962 -> 4979.)
+// where memory is, without a change in a bit.  (128 rows: GRU 2 x 256 2860 -> 2881 us, 2 x 300 4951 -> 4976.)
 inline int sum_steps(int B) {
   int s = 1;
   while (s < 64 && s * B < 256) s *= 2;

@@ -583,10 +583,12 @@ __device__ __forceinline__ int gate_row(const Product& p, int r) {
   return q == p.skip ? -1 : (q == 3 ? p.last : q) * p.H + (r >> 2);
 }
 
-// A tile of a product is formed by two groups of 128 threads, each over every other block of the
-// contraction index, so that the loads of one hide behind the arithmetic of the other (a chunk has
-// few tiles: with one group an SM held eight warps that waited for one another); the first group
-// adds up both groups' blocks.  Operands come in 16-byte pieces where their rows allow it.
+// A tile of a product is formed by two groups of 128 threads, each over every other slice of a block
+// of the contraction index, so that the loads of one hide behind the arithmetic of the other (a chunk
+// has few tiles: with one group an SM held eight warps that waited for one another); the second group's
+// sums are added to the first's at the end of a block.  (Whole blocks to each group, an exchange for two
+// of them: the second group is idle where a short sequence has one, up to 5 % of a step.)  Operands come
+// in 16-byte pieces where their rows allow it.
 constexpr int kTileThreads = 256;
 __device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); }
 
@@ -636,23 +638,25 @@ struct Slice {
   }
 };
 
-// The blocks of a product, two at a time: group g forms block `last - g`.  slice(k0, k1, next0, next1) takes the
-// fetched steps from k0 on and fetches those from next0 on (none if next0 < 0); done(g, two) adds the sums up,
-// two: of both groups.
+// The slices of TK steps that group g takes of a product, block by block from the last: take(next, end) uses the
+// fetched slice and fetches the one at `next` (of the block that ends at `end`; none if next < 0); done() adds a
+// block up.
 template <int TK, class First, class Take, class Done>
 __device__ __forceinline__ void blocks_of(const Product& p, int g, First first, Take take, Done done) {
   const int blocks = (p.K + p.block - 1) / p.block;
   auto end = [&](int b) { return min(p.K, (b + 1) * p.block); };
-  if (blocks - 1 - g >= 0) first((blocks - 1 - g) * p.block, end(blocks - 1 - g));
-  for (int last = blocks - 1; last >= 0; last -= 2) {
-    const int b = last - g;
-    if (b >= 0)
-      for (int k = b * p.block; k < end(b); k += TK) {
-        if (k + TK < end(b)) take(k + TK, end(b));
-        else if (b >= 2) take((b - 2) * p.block, end(b - 2));
-        else take(-1, 0);
-      }
-    done(last > 0);
+  auto fetch = [&](int b, auto f) {   // the group's first slice of block b or of the next one that has one
+    for (; b >= 0; --b)
+      if (b * p.block + g * TK < end(b)) { f(b * p.block + g * TK, end(b)); return; }
+    f(-1, 0);
+  };
+  fetch(blocks - 1, [&](int k, int e) { if (k >= 0) first(k, e); });
+  for (int b = blocks - 1; b >= 0; --b) {
+    for (int k = b * p.block + g * TK; k < end(b); k += 2 * TK) {
+      if (k + 2 * TK < end(b)) take(k + 2 * TK, end(b));
+      else fetch(b - 1, take);
+    }
+    done();
   }
 }
 
@@ -701,7 +705,7 @@ __device__ __forceinline__ void product_fma(const Product& p, int m0, int n0, fl
         }
         group_sync(g);
       },
-      [&](bool two) {
+      [&]() {
         if (g == 1)
 #pragma unroll
           for (int i = 0; i < 32; ++i) x[i * 128] = acc[i >> 2][i & 3];
@@ -709,9 +713,8 @@ __device__ __forceinline__ void product_fma(const Product& p, int m0, int n0, fl
         if (g == 0)
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
-            float& v = sum[i >> 2][i & 3];
-            v = any ? v + acc[i >> 2][i & 3] : acc[i >> 2][i & 3];
-            if (two) v += x[i * 128];
+            const float v = acc[i >> 2][i & 3] + x[i * 128];
+            sum[i >> 2][i & 3] = any ? sum[i >> 2][i & 3] + v : v;
           }
 #pragma unroll
         for (int i = 0; i < 32; ++i) acc[i >> 2][i & 3] = 0.f;
@@ -796,7 +799,7 @@ __device__ __forceinline__ void product_mma(const Product& p, int m0, int n0, fl
         }
         group_sync(g);
       },
-      [&](bool two) {
+      [&]() {
         if (g == 1)
 #pragma unroll
           for (int i = 0; i < 32; ++i) x[i * 128] = acc[i >> 4][(i >> 2) & 3][i & 3];
@@ -804,9 +807,8 @@ __device__ __forceinline__ void product_mma(const Product& p, int m0, int n0, fl
         if (g == 0)
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
-            const float v = acc[i >> 4][(i >> 2) & 3][i & 3];
+            const float v = acc[i >> 4][(i >> 2) & 3][i & 3] + x[i * 128];
             sum[i] = any ? sum[i] + v : v;
-            if (two) sum[i] += x[i * 128];
           }
 #pragma unroll
         for (int i = 0; i < 32; ++i) acc[i >> 4][(i >> 2) & 3][i & 3] = 0.f;
@@ -1068,8 +1070,7 @@ void fill_products(Products& P, const Layout& y, const tc::StepPtrs& io, bool wa
   P.n = 0; P.tiles = 0;
   auto add = [&](const float* A, int lda, bool a_mn, const void* B, int ldb, float* C, int ldc, int M, int N, int K, bool acc,
                  int hidden, int skip, int last) {
-    // (dx is summed over the gates: halves, one for each group)
-    const int block = a_mn ? sum_steps(y.B) * y.B : (int)align_up(((size_t)K + 1) / 2, 32);
+    const int block = a_mn ? sum_steps(y.B) * y.B : K;   // (dx is summed over the gates)
     P.p[P.n++] = Product{A, B, C, lda, ldb, ldc, M, N, K, block, a_mn ? 1 : 0, acc ? 1 : 0, P.tiles, hidden, skip, last};
     P.tiles += ((M + 63) / 64) * ((N + 63) / 64);
   };

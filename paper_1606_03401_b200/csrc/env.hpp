@@ -9,7 +9,7 @@
 //                             of the caller's stream itself
 //   MEBPTT_NO_ZX_AHEAD=1      input projections in the step's stream, when a run needs them, instead of a
 //                             window ahead on a stream of their own
-//   MEBPTT_BWD_CLUSTER=0|4|8  backward run kernel: unclustered (what a profiler that cannot launch
+//   MEBPTT_BWD_CLUSTER=0|4|8  backward run kernel of layers of more than 512 units: unclustered (what a profiler that cannot launch
 //                             clustered cooperative grids can capture), or the cluster size
 //   MEBPTT_NO_BWD_GROUPS=1    backward run kernel without groups of batch rows (same bits)
 //   MEBPTT_NO_SPLITK=1        no contraction is split along K (other rounding on the step-by-step paths)

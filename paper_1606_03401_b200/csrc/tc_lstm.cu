@@ -40,8 +40,10 @@
 #include <mutex>
 #include <vector>
 
+#include "cluster_runs.hpp"
 #include "launch.hpp"
 #include "layout.hpp"
+#include "lstm_dev.cuh"
 #include "sm100.cuh"
 #include "tc.hpp"
 #include "tmap.hpp"
@@ -57,26 +59,6 @@ constexpr int NU = 8;            // hidden units per CTA
 constexpr int NG = 4 * NU;       // gate columns per CTA
 constexpr int NST = 8;           // ring stages of 64 contraction indices
 constexpr int LOSS_PARTS = 64;   // partial sums per step of the loss
-
-// Tape entry as the kernels see it.  Offsets are in units of 16 bytes from the workspace base.
-struct DevOp {
-  int32_t k;
-  int32_t fmt;
-  uint32_t h_src, c_src;   // FWD: state k-1.            BWD: h_{k-1}, c_{k-1}
-  uint32_t h_dst, c_dst;   // FWD: where h_k, c_k go.    BWD: h_k, c_k of the stored internal state
-  uint32_t gates;          // FWD: gate planes to write, 0 = none.   BWD: gate planes to read
-  uint32_t in_copy;        // FWD: hidden block receiving the copy of state k-1, 0 = none
-};
-static_assert(sizeof(DevOp) == 32, "DevOp layout");
-
-__device__ __forceinline__ float sigmoid_fast(float x) { return __fdividef(1.f, 1.f + __expf(-x)); }
-__device__ __forceinline__ float tanh_fast(float x) {
-  float y;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
 
 // ------------------------------------------------------------------------------------------
 // forward run
@@ -1664,6 +1646,9 @@ struct Prepared {
   CUtensorMap tm_dz_g[2], tm_wt_g;
   int fwd_ncg = 0, fwd_smem = 0, fwd_bb = 0;
   bool fwd_slab = false;
+  int cluster_rows = 0;            // batch rows of its clusters
+  bool cluster = false;            // both run kernels of cluster_runs.cu instead of those above
+  CUtensorMap tm_w_cl, tm_wt_cl;
   int rc = MEBPTT_OK;
 
   Prepared() = default;
@@ -1752,6 +1737,14 @@ void build_device_part(Prepared& P, const Layout& y, char* ws) {
   __nv_bfloat16* dz = reinterpret_cast<__nv_bfloat16*>(ws + y.off_dz);
   __nv_bfloat16* wp_hh = reinterpret_cast<__nv_bfloat16*>(ws + y.off_wp_hh);
   __nv_bfloat16* wpT_hh = reinterpret_cast<__nv_bfloat16*>(ws + y.off_wpT_hh);
+  // Up to 512 hidden units a layer's recurrence fits a cluster; the grid-wide kernels are for what is wider (and for a
+  // device that cannot hold such a cluster).  A forward and a backward operation in runs of 32: 2.8 -> 0.78 and 3.9 ->
+  // 0.90 us at H = 256, 3.1 -> 1.32 and 4.0 -> 1.73 us at H = 512; a launch with its set-up takes as long as before.
+  if (cluster_runs_supported(H) && (P.cluster_rows = cluster_rows(B, H)) > 0) {
+    P.cluster = cluster_maps(&P.tm_w_cl, &P.tm_wt_cl, wp_hh, wpT_hh, H);
+    if (!P.cluster) P.rc = MEBPTT_ERR_UNSUPPORTED;
+    return;
+  }
   const int KBh = (H + 63) / 64;
   const int KB0 = fwd_first_part_blocks(H);       // 64-wide blocks of the recurrent contraction in its first part
   const int fwd_groups = B > FB ? 2 : 1;          // groups of CTAs that each own FB batch rows
@@ -2080,7 +2073,13 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
         }
       }
       ++launches;
-      if (!dry && rc == MEBPTT_OK) {
+      if (!dry && rc == MEBPTT_OK && P.cluster) {
+        const ClusterFwdArgs a{dops + i, n, ws, zx_cur + (size_t)(k0 - zx_lo) * B * G, status, io.counters, B, H, off16(y.plane),
+                               off16(y.hsz), (fault & 1) ? 16u : 0u, (fault & 1) ? fault_poll_limit : kSpinLimit};
+        const int span = span_begin(timer, 0, n, s);
+        if (!cuda_ok(cluster_forward(P.tm_w_cl, a, P.cluster_rows, s), "forward run launch (clusters)")) rc = MEBPTT_ERR_CUDA;
+        span_end(timer, span, s);
+      } else if (!dry && rc == MEBPTT_OK) {
         FwdRunArgs a{dops + i, n, ws, zx_cur + (size_t)(k0 - zx_lo) * B * G, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status,
                      io.counters, B, H, fwd_ncg, fwd_bb, fwd_slab ? 1 : 0,
                      (uint32_t)fwd_ncg + ((fault & 1) ? 1u : 0u), (fault & 1) ? fault_poll_limit : (kSpinLimit >> 1),
@@ -2160,7 +2159,13 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
       }
       gemm(dy_c + (size_t)s_lo * B * O, O, false, woutT, O, false,
            GemmOut{GemmOut::STORE_F32, dha + (size_t)s_lo * B * H, H, nullptr, 0}, n * B, H, O);
-      if (!dry && rc == MEBPTT_OK) {
+      if (!dry && rc == MEBPTT_OK && P.cluster) {
+        const ClusterBwdArgs a{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, status, io.counters, B, H, S, off16(y.plane),
+                               leaf ? zleaf : nullptr, parts, (fault & 2) ? 16u : 0u, (fault & 2) ? fault_poll_limit : kSpinLimit};
+        const int span = span_begin(timer, 1, n, s);
+        if (!cuda_ok(cluster_backward(P.tm_wt_cl, a, P.cluster_rows, s), "backward run launch (clusters)")) rc = MEBPTT_ERR_CUDA;
+        span_end(timer, span, s);
+      } else if (!dry && rc == MEBPTT_OK) {
         const bool grouped = P.bwd_grp;
         BwdRunArgs a{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status,
                      io.counters, B, H, S, off16(y.plane), off16(y.hsz), leaf ? zleaf : nullptr, parts,

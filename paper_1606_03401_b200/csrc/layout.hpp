@@ -17,6 +17,7 @@
 
 #include "mebptt.h"
 #include "plan.hpp"
+#include "ring_runs.hpp"
 
 namespace mebptt {
 
@@ -94,7 +95,7 @@ struct Layout {
   size_t off_sync = 0, off_tape = 0, off_status = 0, off_split_dh = 0;
   size_t off_w_f = 0, off_w_b = 0, off_exch_f = 0, off_exch_b = 0;
   size_t off_a3_run = 0, off_zrun = 0, off_hrun = 0, off_dha_run = 0, off_zleaf3 = 0, off_leaf = 0, split_floats = 0;
-  size_t n_sync = 0, tape_bytes = 0;
+  size_t n_sync = 0, tape_bytes = 0, off_ring = 0, ring_bytes = 0;
   // team path: states per group of batch rows, in blocks of one layer's h of the group (a cell state takes
   // 4 / esz of them).  Where a plan's unit is no whole number of blocks, addresses count parts of a block
   // (`parts` to a block): parts of a location's unit, blocks of a hidden state; parts of all states; first parts
@@ -450,6 +451,8 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     y.off_loss_part = take((size_t)y.S * loss_parts_per_step(y.B, y.O) * 4);
     y.n_sync = 64 * (work_items(p, y.S).size() + 1);   // two 128-byte lines per persistent launch (one per group of CTAs)
     y.off_sync = take(y.n_sync * 4);
+    y.ring_bytes = tc::ring_runs_supported(y.H, y.B) ? tc::ring_bytes(y.H, y.B) : 0;   // the exchange of wide layers
+    y.off_ring = take(y.ring_bytes);
     y.tape_bytes = (size_t)p->tape.size() * 32 * 2;   // the tape, and the compacted entries of leaf batches
     y.off_tape = take(y.tape_bytes);
     y.off_status = take(256);

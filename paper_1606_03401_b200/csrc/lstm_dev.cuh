@@ -35,5 +35,12 @@ __device__ __forceinline__ float tanh_fast(float x) {
 __device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
 
+// The contraction with W_hh is summed in two parts from 513 units on, z = (Zx + part 0) + part 1, and the batched
+// products of a leaf batch add them in that order, so that both give the same bits.  64-wide blocks in the first part:
+__host__ __device__ inline int fwd_first_part_blocks(int H) {
+  const int KB = (H + 63) / 64;
+  return KB > 8 ? (KB + 1) / 2 : KB;
+}
+
 }  // namespace tc
 }  // namespace mebptt

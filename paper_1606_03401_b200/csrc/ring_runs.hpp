@@ -1,0 +1,38 @@
+// Runs of the bfloat16 recurrence for 513 to 1024 hidden units, whose exchange goes through a ring in the L2.
+#pragma once
+
+#include "cluster_runs.hpp"
+
+namespace mebptt {
+namespace tc {
+
+constexpr int RING_SLOTS = 4;    // steps a ring holds
+constexpr int RING_CLUSTER = 4;  // CTAs that share the contraction index of a backward step
+
+inline bool ring_runs_supported(int H, int B) { return H % 8 == 0 && H > 16 * CU && H <= 32 * CU && B <= 64; }
+// CTAs of a group of batch rows: 32 units each, whole clusters (the last ones may have no unit)
+inline int ring_ctas(int H) { return (H + RING_CLUSTER * CU - 1) / (RING_CLUSTER * CU) * RING_CLUSTER; }
+// bytes of both rings, two sets each: launches alternate between them
+inline size_t ring_bytes(int H, int B) {
+  const size_t rows = (size_t)(B + 15) / 16 * 16, row = (size_t)ring_ctas(H) * CU * 2;
+  return 2 * RING_SLOTS * rows * (row + 4 * row) + 256;
+}
+
+struct RingArgs {
+  char* ring;            // slots of this launch's set: words of ones wherever nothing has been written
+  char* other;           // the other set, which the launch before used and this one clears
+  const char* never;     // 16 bytes of ones that nobody writes
+  uint32_t fault;        // testing aid: wait for those as well
+  uint32_t poll_limit;
+};
+// The sets of launch number `id` of its direction.
+RingArgs ring_args(char* rings, int H, int B, bool backward, int id, bool fault, uint32_t poll_limit);
+
+// Tensor maps: boxes of 64 columns by 128 rows, as for the cluster kernels.
+// Batch rows of a group (8 or 16); 0 where the device cannot keep the kernels' CTAs resident.
+int ring_rows(int B, int H);
+cudaError_t ring_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, const RingArgs& r, int rows, cudaStream_t s);
+cudaError_t ring_backward(const CUtensorMap& tm_wt, const ClusterBwdArgs& a, const RingArgs& r, int rows, cudaStream_t s);
+
+}  // namespace tc
+}  // namespace mebptt

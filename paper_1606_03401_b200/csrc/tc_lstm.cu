@@ -3,27 +3,16 @@
 //
 // What sits on the recurrence, and therefore cannot be batched over time, is only the
 // product with the recurrent weights: z_t = Zx_t + h_{t-1} W_hh^T going forward and
-// dh_{t-1} = dz_t W_hh going backward.  Both run in persistent kernels that walk a run of
-// consecutive tape operations with W_hh resident in shared memory:
+// dh_{t-1} = dz_t W_hh going backward.  Both run in persistent kernels that walk a run of consecutive tape
+// operations with the weights resident: cluster_runs.cu for at most 512 hidden units, ring_runs.cu for more, and for
+// short runs of wide layers those of this file,
 //
-//   fwd_run_kernel   CTA c owns hidden units 8c .. 8c+7, i.e. the 32 gate rows {i,f,g,o} x 8 of
-//                    W_hh, permuted so that the four gates of a unit are adjacent columns.  Per
-//                    step: TMA streams h_{t-1} ([B][H], 64 columns at a time) through a ring,
-//                    one thread issues tcgen05.mma (M = 64 or 128 batch rows, N = 32, K = 16)
-//                    into TMEM, then each thread owning a batch row reads its 32 accumulators,
-//                    adds the batched input projection Zx_t (bias included), applies the gates
-//                    and updates c_t, h_t for its 8 units -- c_t and h_t stay in registers from
-//                    step to step -- and writes the state where the tape says (scratch, a slot
-//                    of the arena, or a whole internal state).
-//   bwd_run_kernel   same ownership.  Per step each thread forms dz for its 8 units x 4 gates
-//                    from dh (read back from TMEM), dc (registers), the stored gates and cell
-//                    states, writes dz (bfloat16) to the staging chunk, and the CTA then
-//                    contracts the whole dz_t ([B][4H]) against its 8 rows of W_hh^T
-//                    (M = batch, N = 8, K = 16) to get its slice of dh_{t-1}.
+//   fwd_run_kernel         weights in shared memory, h_{k-1} fetched by TMA once a step counter says that it is there
+//   bwd_run_group_kernel   likewise with dz_k, the contraction split over the four CTAs of a cluster
 //
-// Between steps every CTA needs all of h_t (or dz_t): a grid-wide counter in global memory is
-// bumped by each CTA after its stores (release) and polled by the one thread that issues the
-// next step's TMA loads (acquire), with a proxy fence on both sides because the loads go
+// whose set-up is shorter.  Between their steps every CTA needs all of h_t (or dz_t): a grid-wide counter in global
+// memory is bumped by each CTA after its stores (release) and polled by the one thread that issues the
+// next step's TMA loads (acquire), with a proxy fence because the loads go
 // through the async proxy.  The kernels are launched cooperatively, so all CTAs are resident
 // and the wait cannot deadlock; it is bounded all the same.
 //
@@ -44,6 +33,7 @@
 #include "launch.hpp"
 #include "layout.hpp"
 #include "lstm_dev.cuh"
+#include "ring_runs.hpp"
 #include "sm100.cuh"
 #include "tc.hpp"
 #include "tmap.hpp"
@@ -55,9 +45,6 @@ namespace {
 
 using namespace sm100;
 
-constexpr int NU = 8;            // hidden units per CTA
-constexpr int NG = 4 * NU;       // gate columns per CTA
-constexpr int NST = 8;           // ring stages of 64 contraction indices
 constexpr int LOSS_PARTS = 64;   // partial sums per step of the loss
 
 // ------------------------------------------------------------------------------------------
@@ -120,21 +107,11 @@ struct FwdRunArgs {
   int64_t* counters;
   int B, H;
   int ncg;               // CTAs per group
-  int bb;                // K tiles (64 contraction indices each) per barrier and, in slab mode, per copy
-  int slab;              // 1: tm_h is a blocked 3-D map and one copy brings bb tiles; 0: one 2-D copy per tile
   uint32_t expect;       // signals a step is complete with: ncg (a testing aid may ask for one too many)
   uint32_t poll_limit;   // polls of the step counter before the wait gives up
   uint32_t plane16;      // distance between gate planes, in 16-byte units
   uint32_t hsz16;        // distance from h to c inside a hidden block, in 16-byte units
 };
-
-// 64-wide blocks of the contraction index in the first part of the split (all of them if there is
-// one part only: below 640 columns the second accumulator and its hand-over cost more than starting
-// the MMAs half a fetch earlier saves)
-__host__ __device__ inline int fwd_first_part_blocks(int H) {
-  const int KB = (H + 63) / 64;
-  return KB >= 10 ? (KB + 1) / 2 : KB;
-}
 
 // State update of one thread: batch row b, hidden units j0 .. j0 + 3.  z[u] holds the four
 // pre-activations (i, f, g, o) of unit j0 + u; writes h_k at once and the rest of the state after
@@ -280,17 +257,10 @@ __global__ void __launch_bounds__(192, 1) fwd_run_kernel(const __grid_constant__
       if (!go) continue;
       // the acquire of lane 0 reaches the other lanes through the shuffle; the proxy fence then orders
       // a lane's TMA read after the h_k written by the other CTAs
-      if (a.slab) {
-        if (lane < NQ) {
-          fence_proxy_async_global();
-          mbar_arrive_expect_tx(&full[lane], (uint32_t)KB0 * H_TILE);   // a box counts in full, also where it is filled with zeros
-          tma_load_3d(tiles + lane * KB0 * H_TILE, &tm_h, 0, row, lane * KB0, &full[lane]);
-        }
-      } else if (lane < KB) {
+      if (lane < NQ) {
         fence_proxy_async_global();
-        const int q = lane >= KB0 ? 1 : 0;
-        if (lane == q * KB0) mbar_arrive_expect_tx(&full[q], (uint32_t)(q ? KB - KB0 : KB0) * H_TILE);
-        tma_load_2d(tiles + lane * H_TILE, &tm_h, lane * 64, row, &full[q]);
+        mbar_arrive_expect_tx(&full[lane], (uint32_t)KB0 * H_TILE);   // a box counts in full, also where it is filled with zeros
+        tma_load_3d(tiles + lane * KB0 * H_TILE, &tm_h, 0, row, lane * KB0, &full[lane]);
       }
       armed = i;
       if (i == a.n - 1 && lane == 0) grid_dep_launch();   // last step under way: the next kernel may set itself up
@@ -400,515 +370,26 @@ struct BwdRunArgs {
   int* status;
   int64_t* counters;
   int B, H, S;
-  uint32_t plane16, hsz16;
+  uint32_t plane16;
   const float* zleaf;      // leaf batch: [S][B][4H] pre-activations z_k (gate columns permuted); NULL otherwise
   int loss_parts;          // partial sums of the loss per step
-  int tb;                  // clustered kernel: K tiles per barrier and, in slab mode, per copy
-  int slab;                // clustered kernel: 1: tm_dz is a blocked 3-D map and one copy brings tb tiles
+  int tb;                  // K tiles per barrier and per copy
   uint32_t expect;         // signals a step is complete with: the grid size (a testing aid may ask for one too many)
   uint32_t poll_limit;     // polls of the step counter before the wait gives up
 };
 
-// What the gate derivatives of one batch row and 8 hidden units read from memory at one step: the
-// stored gates and cell states and the readout gradient.  None of it depends on the recurrence,
-// so it can be fetched while the exchange of the previous step is still in flight.
-struct GateInputs {
-  uint4 qi, qf, qg, qo;
-  float4 t0, t1, p0, p1, d0, d1;
-};
-__device__ __forceinline__ GateInputs load_gate_inputs(const BwdRunArgs& a, const DevOp& op, int sidx, int b, int cta,
-                                                       size_t e0, size_t pl) {
-  GateInputs in;
-  const char* ws = a.ws;
-  const float* dha = a.dha + ((size_t)sidx * a.B) * a.H + e0;
-  in.d0 = *reinterpret_cast<const float4*>(dha);
-  in.d1 = *reinterpret_cast<const float4*>(dha + 4);
-  const float* cpp = reinterpret_cast<const float*>(ws + (size_t)op.c_src * 16) + e0;
-  in.p0 = *reinterpret_cast<const float4*>(cpp);
-  in.p1 = *reinterpret_cast<const float4*>(cpp + 4);
-  if (a.zleaf) {
-    // A leaf of the recursion: no internal state was stored.  Its forward operation is redone
-    // here from the pre-activations, with exactly the arithmetic of the forward kernel (gates
-    // rounded to bfloat16 as they would have been stored, c_k from the unrounded gates).
-    const float4* zp = reinterpret_cast<const float4*>(a.zleaf + ((size_t)sidx * a.B + b) * 4 * a.H + (size_t)cta * NG);
-    const float cp[NU] = {in.p0.x, in.p0.y, in.p0.z, in.p0.w, in.p1.x, in.p1.y, in.p1.z, in.p1.w};
-    float ct[NU];
-    uint32_t gi[4], gf[4], gg[4], go[4];
-#pragma unroll
-    for (int u = 0; u < NU; u += 2) {
-      float iv[2], fv[2], gv[2], ov[2];
-#pragma unroll
-      for (int d = 0; d < 2; ++d) {
-        const float4 z = zp[u + d];
-        iv[d] = sigmoid_fast(z.x);
-        fv[d] = sigmoid_fast(z.y);
-        gv[d] = tanh_fast(z.z);
-        ov[d] = sigmoid_fast(z.w);
-        ct[u + d] = fmaf(fv[d], cp[u + d], iv[d] * gv[d]);
-      }
-      gi[u / 2] = pack_bf16x2(iv[0], iv[1]);
-      gf[u / 2] = pack_bf16x2(fv[0], fv[1]);
-      gg[u / 2] = pack_bf16x2(gv[0], gv[1]);
-      go[u / 2] = pack_bf16x2(ov[0], ov[1]);
-    }
-    in.qi = make_uint4(gi[0], gi[1], gi[2], gi[3]);
-    in.qf = make_uint4(gf[0], gf[1], gf[2], gf[3]);
-    in.qg = make_uint4(gg[0], gg[1], gg[2], gg[3]);
-    in.qo = make_uint4(go[0], go[1], go[2], go[3]);
-    in.t0 = make_float4(ct[0], ct[1], ct[2], ct[3]);
-    in.t1 = make_float4(ct[4], ct[5], ct[6], ct[7]);
-    return in;
-  }
-  const __nv_bfloat16* g = reinterpret_cast<const __nv_bfloat16*>(ws + (size_t)op.gates * 16) + e0;
-  in.qi = *reinterpret_cast<const uint4*>(g);
-  in.qf = *reinterpret_cast<const uint4*>(g + pl);
-  in.qg = *reinterpret_cast<const uint4*>(g + 2 * pl);
-  in.qo = *reinterpret_cast<const uint4*>(g + 3 * pl);
-  const float* ctp = reinterpret_cast<const float*>(ws + (size_t)op.c_dst * 16) + e0;
-  in.t0 = *reinterpret_cast<const float4*>(ctp);
-  in.t1 = *reinterpret_cast<const float4*>(ctp + 4);
-  return in;
-}
-
-// Gate derivatives from the fetched inputs and the carried (dh, dc); writes dz (bfloat16, columns
-// 4 u + q) to the staging chunk and leaves dc = dc_t * f for the next (earlier) step.
-__device__ __forceinline__ void compute_gates(const BwdRunArgs& a, const GateInputs& in, int sidx, int b, int cta,
-                                              const float (&dh)[NU], float (&dc)[NU]) {
-  const int G = 4 * a.H;
-  const float dhav[NU] = {in.d0.x, in.d0.y, in.d0.z, in.d0.w, in.d1.x, in.d1.y, in.d1.z, in.d1.w};
-  const uint32_t wi[4] = {in.qi.x, in.qi.y, in.qi.z, in.qi.w}, wf[4] = {in.qf.x, in.qf.y, in.qf.z, in.qf.w};
-  const uint32_t wg[4] = {in.qg.x, in.qg.y, in.qg.z, in.qg.w}, wo[4] = {in.qo.x, in.qo.y, in.qo.z, in.qo.w};
-  const float ct[NU] = {in.t0.x, in.t0.y, in.t0.z, in.t0.w, in.t1.x, in.t1.y, in.t1.z, in.t1.w};
-  const float cp[NU] = {in.p0.x, in.p0.y, in.p0.z, in.p0.w, in.p1.x, in.p1.y, in.p1.z, in.p1.w};
-  uint32_t out[NG / 2];
-#pragma unroll
-  for (int u = 0; u < NU; ++u) {
-    const int w = u >> 1;
-    const bool hi = (u & 1) != 0;
-    const float gi = hi ? bf16_hi(wi[w]) : bf16_lo(wi[w]);
-    const float gf = hi ? bf16_hi(wf[w]) : bf16_lo(wf[w]);
-    const float gg = hi ? bf16_hi(wg[w]) : bf16_lo(wg[w]);
-    const float go = hi ? bf16_hi(wo[w]) : bf16_lo(wo[w]);
-    const float dht = dhav[u] + dh[u];
-    const float th = tanh_fast(ct[u]);
-    const float d_o = dht * th;
-    const float dct = fmaf(dht * go, 1.f - th * th, dc[u]);
-    const float zi = dct * gg * gi * (1.f - gi);
-    const float zf = dct * cp[u] * gf * (1.f - gf);
-    const float zg = dct * gi * (1.f - gg * gg);
-    const float zo = d_o * go * (1.f - go);
-    dc[u] = dct * gf;
-    out[2 * u] = pack_bf16x2(zi, zf);
-    out[2 * u + 1] = pack_bf16x2(zg, zo);
-  }
-  uint4* dzp = reinterpret_cast<uint4*>(a.dz + ((size_t)sidx * a.B + b) * G + (size_t)cta * NG);
-#pragma unroll
-  for (int v = 0; v < NG / 8; ++v) dzp[v] = make_uint4(out[4 * v], out[4 * v + 1], out[4 * v + 2], out[4 * v + 3]);
-}
-
-__device__ __forceinline__ void backward_gates(const BwdRunArgs& a, const DevOp& op, int sidx, int b, int cta,
-                                               size_t e0, size_t pl, const float (&dh)[NU], float (&dc)[NU]) {
-  const GateInputs in = load_gate_inputs(a, op, sidx, b, cta, e0, pl);
-  compute_gates(a, in, sidx, b, cta, dh, dc);
-}
-
-template <int BM>
-__global__ void __launch_bounds__(128, 1) bwd_run_kernel(const __grid_constant__ CUtensorMap tm_dz,
-                                                         const __grid_constant__ CUtensorMap tm_wt,
-                                                         const BwdRunArgs a) {
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t wfull, full[NST], empty[NST], acc;
-  __shared__ uint32_t tmem_slot;
-  __shared__ int failed;
-
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int KB = (4 * a.H + 63) / 64;
-  uint8_t* sW = sm;                    // KB tiles of [8 rows][128 B]: rows 8c .. 8c+7 of W_hh^T
-  uint8_t* ring = sm + KB * 1024;
-  constexpr uint32_t A_TILE = BM * 128;
-
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int cta = blockIdx.x, ncta = gridDim.x;
-  const bool is_p = (tid == 0), is_mma = (tid == 32);
-
-  if (tid == 0) {
-    mbar_init(&wfull, 1);
-    for (int s = 0; s < NST; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    mbar_init(&acc, 1);
-    failed = 0;
-    mbar_fence_init();
-    tma_prefetch_desc(&tm_dz);
-    tma_prefetch_desc(&tm_wt);
-  }
-  if (warp == 1) tmem_alloc(&tmem_slot, 32);
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = tmem_slot;
-  grid_dep_wait();
-  if (tid == 0) grid_dep_launch();
-
-  if (is_p) {
-    mbar_arrive_expect_tx(&wfull, (uint32_t)KB * 1024u);
-    for (int kb = 0; kb < KB; ++kb) tma_load_2d(sW + kb * 1024, &tm_wt, kb * 64, cta * NU, &wfull);
-  }
-
-  const int b = (BM == 64) ? (16 * warp + lane) : (32 * warp + lane);
-  const bool owner = ((BM == 64) ? (lane < 16) : true) && b < a.B;
-  const int j0 = cta * NU;
-  const size_t e0 = (size_t)b * a.H + j0;
-  const size_t pl = (size_t)a.plane16 * 8;
-  float dh[NU], dc[NU];
-  if (owner) {
-    const float4 a0 = *reinterpret_cast<const float4*>(a.dh + e0), a1 = *reinterpret_cast<const float4*>(a.dh + e0 + 4);
-    const float4 c0 = *reinterpret_cast<const float4*>(a.dc + e0), c1 = *reinterpret_cast<const float4*>(a.dc + e0 + 4);
-    dh[0] = a0.x; dh[1] = a0.y; dh[2] = a0.z; dh[3] = a0.w; dh[4] = a1.x; dh[5] = a1.y; dh[6] = a1.z; dh[7] = a1.w;
-    dc[0] = c0.x; dc[1] = c0.y; dc[2] = c0.z; dc[3] = c0.w; dc[4] = c1.x; dc[5] = c1.y; dc[6] = c1.z; dc[7] = c1.w;
-  } else {
-#pragma unroll
-    for (int u = 0; u < NU; ++u) { dh[u] = 0.f; dc[u] = 0.f; }
-  }
-
-  uint32_t issued = 0, consumed = 0;
-  constexpr uint32_t idesc = make_idesc(1, BM, NU, false, false);
-
-  for (int i = 0; i < a.n; ++i) {
-    const DevOp op = a.ops[i];
-    const int sidx = (op.k - 1) % a.S;
-    if (i > 0) {
-      // dh for this step = the slice of dz_{k+1} W_hh this CTA computed in the previous iteration
-      const bool got = wait_or_fail(&acc, (uint32_t)(i - 1) & 1, &failed);
-      tc_fence_after_sync();
-      uint32_t r[NU];
-      tmem_ld_32x8(tmem + ((uint32_t)(32 * warp) << 16), r);
-      tmem_ld_wait();
-      if (got) {
-#pragma unroll
-        for (int u = 0; u < NU; ++u) dh[u] = __uint_as_float(r[u]);
-      }
-    }
-    if (owner && !failed) backward_gates(a, op, sidx, b, cta, e0, pl, dh, dc);
-    if (cta == 0 && tid == 0) {
-      // loss term of this step: its partial sums in a fixed order
-      float s = 0.f;
-      for (int p = 0; p < a.loss_parts; ++p) s += a.loss_part[sidx * a.loss_parts + p];
-      a.loss_t[op.k - 1] = s;
-    }
-    fence_proxy_async();
-    tc_fence_before_sync();
-    __syncthreads();
-    if (tid == 0) red_release_add(a.sync, 1u);
-    if (failed) break;
-
-    if (is_p) {
-      // ---- producer: all of dz_k through the ring -----------------------------------------
-      bool ok = wait_counter(a.sync, (uint32_t)(i + 1) * a.expect, &failed, a.poll_limit);
-      if (ok) {
-        fence_proxy_async();
-        const int32_t row = sidx * a.B;
-        for (int kb = 0; kb < KB && ok; ++kb, ++issued) {
-          const uint32_t s = issued % NST, it = issued / NST;
-          if (it > 0) ok = wait_or_fail(&empty[s], (it - 1) & 1, &failed);
-          if (!ok) break;
-          mbar_arrive_expect_tx(&full[s], A_TILE);
-          tma_load_2d(ring + s * A_TILE, &tm_dz, kb * 64, row, &full[s]);
-        }
-      }
-    } else if (is_mma) {
-      bool ok = true;
-      if (i == 0) ok = wait_or_fail(&wfull, 0, &failed);
-      for (int kb = 0; kb < KB && ok; ++kb, ++consumed) {
-        const uint32_t s = consumed % NST, it = consumed / NST;
-        ok = wait_or_fail(&full[s], it & 1, &failed);
-        if (!ok) break;
-        tc_fence_after_sync();
-        const uint32_t a0 = smem_u32(ring + s * A_TILE), b0 = smem_u32(sW + kb * 1024);
-#pragma unroll
-        for (int k4 = 0; k4 < 4; ++k4)
-          mma_f16(tmem, make_desc_sw128(a0 + k4 * 32, 16, 1024), make_desc_sw128(b0 + k4 * 32, 16, 1024), idesc,
-                  (kb > 0 || k4 > 0) ? 1u : 0u);
-        mma_commit(&empty[s]);
-      }
-      mma_commit(&acc);
-    }
-    __syncwarp();
-  }
-
-  if (!failed) {
-    // the gradient that leaves the run: dh from the last product, dc from registers
-    const bool got = wait_or_fail(&acc, (uint32_t)(a.n - 1) & 1, &failed);
-    tc_fence_after_sync();
-    uint32_t r[NU];
-    tmem_ld_32x8(tmem + ((uint32_t)(32 * warp) << 16), r);
-    tmem_ld_wait();
-    if (got && owner) {
-      *reinterpret_cast<float4*>(a.dh + e0) = make_float4(__uint_as_float(r[0]), __uint_as_float(r[1]),
-                                                           __uint_as_float(r[2]), __uint_as_float(r[3]));
-      *reinterpret_cast<float4*>(a.dh + e0 + 4) = make_float4(__uint_as_float(r[4]), __uint_as_float(r[5]),
-                                                               __uint_as_float(r[6]), __uint_as_float(r[7]));
-      *reinterpret_cast<float4*>(a.dc + e0) = make_float4(dc[0], dc[1], dc[2], dc[3]);
-      *reinterpret_cast<float4*>(a.dc + e0 + 4) = make_float4(dc[4], dc[5], dc[6], dc[7]);
-    }
-  }
-  tc_fence_before_sync();
-  __syncthreads();
-  if (failed) {
-    if (tid == 0) *a.status = MEBPTT_ERR_TIMEOUT;
-    if (is_p) {
-      for (uint32_t q = (issued > NST ? issued - NST : 0); q < issued; ++q)
-        (void)mbar_wait(&full[q % NST], (q / NST) & 1);
-      (void)mbar_wait(&wfull, 0);
-    }
-    __syncthreads();
-  } else if (cta == 0 && tid == 0) {
-    a.counters[1] += a.n;
-  }
-  if (warp == 1) tmem_dealloc(tmem, 32);
-}
-
-// ------------------------------------------------------------------------------------------
-// backward run, split over thread-block clusters
-// ------------------------------------------------------------------------------------------
-// The product dh_{k-1} = dz_k W_hh has K = 4H: a CTA that wants its 8 columns on its own must
-// pull all of dz_k (B x 4H) through shared memory every step.  Here CS neighbouring CTAs (one
-// cluster, 8 CS hidden units) share the work along K instead: CTA r multiplies the K-slice
-// [r G/CS, (r+1) G/CS) of dz_k by the matching [8 CS x G/CS] block of W_hh^T, resident in its
-// shared memory, into a partial [B x 8 CS] tile; the partial tiles go to shared memory, the
-// cluster synchronises, and each owner thread adds the CS partial values of its 8 columns in the
-// order r = 0 .. CS-1, reading its peers' tiles through distributed shared memory.
-template <int CS>
-__global__ void __launch_bounds__(192, 1) bwd_run_cluster_kernel(const __grid_constant__ CUtensorMap tm_dz,
-                                                                 const __grid_constant__ CUtensorMap tm_wt,
-                                                                 const BwdRunArgs a) {
-  constexpr int BM = 64;
-  constexpr int NC = NU * CS;              // columns of dh the cluster produces
-  constexpr uint32_t A_TILE = BM * 128;
-  constexpr uint32_t W_TILE = NC * 128;
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t wfull, full[4], acc, pready[2];
-  __shared__ uint32_t tmem_slot;
-  __shared__ int failed;
-
-  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int G = 4 * a.H;
-  const int KBS = (G / 64) / CS;           // 64-wide K blocks in this CTA's slice (<= 16)
-  const int TB = a.tb;                     // K tiles per barrier
-  const int NQ = (KBS + TB - 1) / TB;      // <= 4
-  uint8_t* sW = sm;                        // KBS tiles [NC rows][128 B]
-  uint8_t* ring = sW + KBS * W_TILE;       // KBS tiles [64 rows][128 B], all of the slice at once
-  // partial sums received from the cluster: [2 buffers][CS senders][64 rows][8 columns]
-  float* recv = reinterpret_cast<float*>(ring + NQ * TB * A_TILE);
-
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int cta = blockIdx.x, ncta = gridDim.x;
-  const uint32_t rank = cluster_ctarank();
-  const int cl = cta / CS;
-
-  if (tid == 0) {
-    mbar_init(&wfull, 1);
-    for (int s = 0; s < 4; ++s) mbar_init(&full[s], 1);
-    mbar_init(&acc, 1);
-    mbar_init(&pready[0], CS);
-    mbar_init(&pready[1], CS);
-    failed = 0;
-    mbar_fence_init();
-    tma_prefetch_desc(&tm_dz);
-    tma_prefetch_desc(&tm_wt);
-  }
-  if (warp == 4) tmem_alloc(&tmem_slot, 64);
-  tc_fence_before_sync();
-  cluster_sync();                          // peers arrive on each other's barriers: all must be initialised
-  tc_fence_after_sync();
-  const uint32_t tmem = tmem_slot;
-  grid_dep_wait();
-
-  if (warp == 4) {
-    // ---- producer: this CTA's K-slice of dz_k, all of it in flight at once; lane 0 watches the
-    // step counter, lanes 0 .. NQ-1 each request one block of four K tiles -------------------------
-    if (lane == 0) {
-      mbar_arrive_expect_tx(&wfull, (uint32_t)KBS * W_TILE);
-      for (int kb = 0; kb < KBS; ++kb)
-        tma_load_2d(sW + kb * W_TILE, &tm_wt, ((int)rank * KBS + kb) * 64, cl * NC, &wfull);
-    }
-    int armed = -1;
-    for (int i = 0; i < a.n; ++i) {
-      const int sidx = (a.ops[i].k - 1) % a.S;
-      if (cta == 0 && lane == 31) {
-        // loss term of this step: its partial sums in a fixed order (on a lane that is off the
-        // critical path of the recurrence)
-        float sum = 0.f;
-        for (int p = 0; p < a.loss_parts; ++p) sum += a.loss_part[sidx * a.loss_parts + p];
-        a.loss_t[a.ops[i].k - 1] = sum;
-      }
-      int go = 1;
-      if (lane == 0) go = !failed && wait_counter(a.sync, (uint32_t)(i + 1) * a.expect, &failed, a.poll_limit) && !failed;
-      go = __shfl_sync(0xffffffffu, go, 0);
-      if (!go) continue;
-      if (lane < NQ) {
-        // (the TMA unit takes its copy requests one at a time, ~100 ns each: in slab mode one copy over
-        // a map that sees a row as blocks of 64 columns brings the TB tiles of a barrier)
-        fence_proxy_async_global();
-        const int32_t row = sidx * a.B;
-        const int q = lane;
-        const int kb0 = TB * q, kb1 = (kb0 + TB < KBS) ? kb0 + TB : KBS;
-        if (a.slab) {
-          mbar_arrive_expect_tx(&full[q], (uint32_t)TB * A_TILE);   // a box counts in full
-          tma_load_3d(ring + kb0 * A_TILE, &tm_dz, 0, row, (int)rank * KBS + kb0, &full[q]);
-        } else {
-          mbar_arrive_expect_tx(&full[q], (uint32_t)(kb1 - kb0) * A_TILE);
-          for (int kb = kb0; kb < kb1; ++kb)
-            tma_load_2d(ring + kb * A_TILE, &tm_dz, ((int)rank * KBS + kb) * 64, row, &full[q]);
-        }
-      }
-      armed = i;
-      if (i == a.n - 1 && lane == 0) grid_dep_launch();
-      __syncwarp();
-    }
-    if (failed && lane == 0) {
-      (void)mbar_wait(&wfull, 0);
-      if (armed >= 0)
-        for (int q = 0; q < NQ; ++q) (void)mbar_wait(&full[q], (uint32_t)armed & 1);
-    }
-  } else if (warp == 5) {
-    // ---- MMA issuer: the whole warp walks the loop, one elected lane issues --------------------
-    constexpr uint32_t idesc = make_idesc(1, BM, NC, false, false);
-    bool ok = wait_or_fail(&wfull, 0, &failed);
-    const uint64_t a_desc0 = make_desc_sw128(smem_u32(ring), 16, 1024);
-    const uint64_t b_desc0 = make_desc_sw128(smem_u32(sW), 16, 1024);
-    for (int i = 0; i < a.n; ++i) {
-      uint64_t da = a_desc0, db = b_desc0;
-      for (int q = 0; q < NQ && ok; ++q) {
-        ok = wait_or_fail(&full[q], (uint32_t)i & 1, &failed);
-        if (!ok) break;
-        tc_fence_after_sync();
-        const int nkb = (TB * q + TB < KBS) ? TB : KBS - TB * q;
-        if (elect_one()) {
-          for (int kb = 0; kb < nkb; ++kb)
-            mma_f16_x4(tmem, da + (uint64_t)(kb * (A_TILE >> 4)), db + (uint64_t)(kb * (W_TILE >> 4)), idesc,
-                       (q > 0 || kb > 0) ? 1u : 0u);
-        }
-        __syncwarp();
-        da += (uint64_t)TB * (A_TILE >> 4);
-        db += (uint64_t)TB * (W_TILE >> 4);
-      }
-      if (elect_one()) mma_commit(&acc);   // always: the epilogue counts on one arrival per step
-      __syncwarp();
-    }
-  } else {
-    // ---- gate derivatives: warp w owns tile rows 16w .. 16w+15 ----------------------------------
-    const int b = 16 * warp + lane;
-    const bool row_thread = lane < 16;             // holds an accumulator row in TMEM
-    const bool owner = row_thread && b < a.B;
-    const int j0 = cta * NU;
-    const size_t e0 = (size_t)b * a.H + j0;
-    const size_t pl = (size_t)a.plane16 * 8;
-    float dh[NU], dc[NU];
-    if (owner) {
-      const float4 a0 = *reinterpret_cast<const float4*>(a.dh + e0), a1 = *reinterpret_cast<const float4*>(a.dh + e0 + 4);
-      const float4 c0 = *reinterpret_cast<const float4*>(a.dc + e0), c1 = *reinterpret_cast<const float4*>(a.dc + e0 + 4);
-      dh[0] = a0.x; dh[1] = a0.y; dh[2] = a0.z; dh[3] = a0.w; dh[4] = a1.x; dh[5] = a1.y; dh[6] = a1.z; dh[7] = a1.w;
-      dc[0] = c0.x; dc[1] = c0.y; dc[2] = c0.z; dc[3] = c0.w; dc[4] = c1.x; dc[5] = c1.y; dc[6] = c1.z; dc[7] = c1.w;
-    } else {
-#pragma unroll
-      for (int u = 0; u < NU; ++u) { dh[u] = 0.f; dc[u] = 0.f; }
-    }
-
-    // Reduces the partial tiles of product number `it` into this thread's dh.  Each row thread
-    // reads its row of this CTA's partial tile from TMEM and sends the 8 columns that belong to
-    // CTA p straight into p's shared memory; once all CS senders have signalled, the owner adds
-    // the CS partial values of its columns in the order of the ranks.
-    auto reduce_partials = [&](int it) {
-      float* buf = recv + (size_t)(it & 1) * CS * BM * NU;
-      const bool got = wait_or_fail(&acc, (uint32_t)it & 1, &failed);
-      tc_fence_after_sync();
-#pragma unroll
-      for (int c0 = 0; c0 < NC; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld_32x32(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c0, r);
-        tmem_ld_wait();
-        if (row_thread) {
-#pragma unroll
-          for (int pp = 0; pp < 4; ++pp) {   // 32 columns = the columns of four CTAs
-            float* dst = buf + ((size_t)rank * BM + b) * NU;      // slot of sender `rank`, row b
-            const uint32_t peer = (uint32_t)(c0 / NU + pp);
-            st_peer_f4(dst, peer, make_float4(__uint_as_float(r[8 * pp]), __uint_as_float(r[8 * pp + 1]),
-                                              __uint_as_float(r[8 * pp + 2]), __uint_as_float(r[8 * pp + 3])));
-            st_peer_f4(dst + 4, peer, make_float4(__uint_as_float(r[8 * pp + 4]), __uint_as_float(r[8 * pp + 5]),
-                                                  __uint_as_float(r[8 * pp + 6]), __uint_as_float(r[8 * pp + 7])));
-          }
-        }
-      }
-      tc_fence_before_sync();
-      named_barrier(1, 128);
-      if (tid < CS) mbar_arrive_peer(&pready[it & 1], (uint32_t)tid);   // release: the stores above are visible
-      bool all = false;
-      for (uint32_t spin = 0; spin < kSpinLimit; ++spin) {
-        if (mbar_try_wait_cluster(&pready[it & 1], (uint32_t)(it >> 1) & 1)) { all = true; break; }
-        if (spin > 256) {
-          if (failed) break;
-          __nanosleep(64);
-        }
-      }
-      if (!all) failed = 1;
-      if (got && all && owner) {
-        float sum[NU];
-#pragma unroll
-        for (int u = 0; u < NU; ++u) sum[u] = 0.f;
-#pragma unroll
-        for (int p = 0; p < CS; ++p) {
-          const float4* src = reinterpret_cast<const float4*>(buf + ((size_t)p * BM + b) * NU);
-          const float4 v0 = src[0], v1 = src[1];
-          sum[0] += v0.x; sum[1] += v0.y; sum[2] += v0.z; sum[3] += v0.w;
-          sum[4] += v1.x; sum[5] += v1.y; sum[6] += v1.z; sum[7] += v1.w;
-        }
-#pragma unroll
-        for (int u = 0; u < NU; ++u) dh[u] = sum[u];
-      }
-    };
-
-    GateInputs gin;
-    if (owner) gin = load_gate_inputs(a, a.ops[0], (a.ops[0].k - 1) % a.S, b, cta, e0, pl);
-    for (int i = 0; i < a.n; ++i) {
-      const DevOp op = a.ops[i];
-      const int sidx = (op.k - 1) % a.S;
-      if (i > 0) reduce_partials(i - 1);
-      if (owner && !failed) compute_gates(a, gin, sidx, b, cta, dh, dc);
-      named_barrier(1, 128);   // all of this CTA's dz stores precede the release below
-      if (tid == 0) red_release_add(a.sync, 1u);
-      // the inputs of the next (earlier) step do not depend on the recurrence: fetch them while the
-      // exchange of this step is in flight
-      if (owner && i + 1 < a.n) gin = load_gate_inputs(a, a.ops[i + 1], (a.ops[i + 1].k - 1) % a.S, b, cta, e0, pl);
-    }
-    reduce_partials(a.n - 1);
-    if (owner && !failed) {
-      *reinterpret_cast<float4*>(a.dh + e0) = make_float4(dh[0], dh[1], dh[2], dh[3]);
-      *reinterpret_cast<float4*>(a.dh + e0 + 4) = make_float4(dh[4], dh[5], dh[6], dh[7]);
-      *reinterpret_cast<float4*>(a.dc + e0) = make_float4(dc[0], dc[1], dc[2], dc[3]);
-      *reinterpret_cast<float4*>(a.dc + e0 + 4) = make_float4(dc[4], dc[5], dc[6], dc[7]);
-    }
-  }
-
-  tc_fence_before_sync();
-  cluster_sync();   // no CTA leaves while a peer may still read its partial tiles or signal it
-  if (tid == 0) {
-    if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (cta == 0) a.counters[1] += a.n;
-  }
-  if (warp == 4) tmem_dealloc(tmem, 64);
-}
-
 // ------------------------------------------------------------------------------------------
 // backward run, clusters inside groups of batch rows
 // ------------------------------------------------------------------------------------------
-// The same split along K as above (clusters of four CTAs, partial tiles reduced in rank order), with
-// what the forward kernel does about latency: the grid is cut into groups of CTAs that each own
-// FB = 32 batch rows and have a step counter of their own, so that a CTA pulls half the bytes of
-// dz_k and a step is signalled by half the CTAs; the product is taken transposed (the cluster's 64
+// The product dh_{k-1} = dz_k W_hh has K = 4H: a CTA that wants its columns on its own must pull all of dz_k through
+// shared memory every step.  Here the four CTAs of a cluster share the work along K instead: CTA r multiplies the K-slice
+// [r G/4, (r+1) G/4) of dz_k by the matching [64 x G/4] block of W_hh^T, resident in its shared memory, into a partial
+// tile that goes through distributed shared memory to the CTAs that own the columns, where the partial values are added
+// in the order of the ranks.  As in the forward kernel the grid is cut into groups of CTAs that each own
+// FB = 32 batch rows and have a step counter of their own; the product is taken transposed (the cluster's 64
 // columns of dh, as rows of W_hh^T resident in shared memory, are the M side of the MMA, the 32
 // batch rows the N side); and all 128 epilogue threads take part in the gate derivatives, each with
-// four hidden units of one batch row.  CTA c of a group owns hidden units 16 c .. 16 c + 15; the
-// partial sums of a column are added in the order of the ranks as above, so both kernels give the
-// same bits.
+// four hidden units of one batch row.  CTA c of a group owns hidden units 16 c .. 16 c + 15.
 struct GateInputs4 {
   uint2 qi, qf, qg, qo;
   float4 t, p, d;
@@ -1637,17 +1118,10 @@ struct Prepared {
   size_t tape_entries = 0;
   bool pinned = false;
   // device part
-  CUtensorMap tm_h, tm_w, tm_dz[2], tm_wt, tm_dz_b[2], tm_wt_c;
-  int bwd_cs = 0, bwdc_smem = 0;   // cluster size of the backward kernel (0: one CTA per 8 columns, unclustered)
-  int bwd_tb = 4;                  // its K tiles per barrier
-  bool bwd_slab = false;           // its slice of dz by one copy per barrier instead of one per K tile
-  bool bwd_grp = false;            // the backward kernel with groups of batch rows (then bwd_cs is its cluster size)
-  int bwdg_smem = 0, bwdg_tb = 8, bwdg_ncg = 0;
-  CUtensorMap tm_dz_g[2], tm_wt_g;
-  int fwd_ncg = 0, fwd_smem = 0, fwd_bb = 0;
-  bool fwd_slab = false;
-  int cluster_rows = 0;            // batch rows of its clusters
-  bool cluster = false;            // both run kernels of cluster_runs.cu instead of those above
+  bool short_runs = false;         // the kernels of this file take short runs of a layer whose longer ones go through the ring
+  CUtensorMap tm_h, tm_w, tm_dz[2], tm_wt;
+  int fwd_ncg = 0, fwd_smem = 0, bwd_smem = 0, bwd_tb = 8;
+  int run_rows = 0;                // batch rows of a cluster (cluster_runs.cu) or of a group of CTAs (ring_runs.cu)
   CUtensorMap tm_w_cl, tm_wt_cl;
   int rc = MEBPTT_OK;
 
@@ -1732,118 +1206,46 @@ void build_host_part(Prepared& P, const Layout& y, const Plan* p, bool allow_pin
 // Kernel variants and tensor maps for the workspace at `ws` on the current device.
 void build_device_part(Prepared& P, const Layout& y, char* ws) {
   const int B = y.B, H = y.H, S = y.S, G = 4 * H;
-  const int BM = 64;  // batch rows per MMA tile (B <= 64)
-  const int ncta = H / NU;
   __nv_bfloat16* dz = reinterpret_cast<__nv_bfloat16*>(ws + y.off_dz);
   __nv_bfloat16* wp_hh = reinterpret_cast<__nv_bfloat16*>(ws + y.off_wp_hh);
   __nv_bfloat16* wpT_hh = reinterpret_cast<__nv_bfloat16*>(ws + y.off_wpT_hh);
-  // Up to 512 hidden units a layer's recurrence fits a cluster; the grid-wide kernels are for what is wider (and for a
-  // device that cannot hold such a cluster).  A forward and a backward operation in runs of 32: 2.8 -> 0.78 and 3.9 ->
-  // 0.90 us at H = 256, 3.1 -> 1.32 and 4.0 -> 1.73 us at H = 512; a launch with its set-up takes as long as before.
-  if (cluster_runs_supported(H) && (P.cluster_rows = cluster_rows(B, H)) > 0) {
-    P.cluster = cluster_maps(&P.tm_w_cl, &P.tm_wt_cl, wp_hh, wpT_hh, H);
-    if (!P.cluster) P.rc = MEBPTT_ERR_UNSUPPORTED;
-    return;
-  }
-  const int KBh = (H + 63) / 64;
-  const int KB0 = fwd_first_part_blocks(H);       // 64-wide blocks of the recurrent contraction in its first part
-  const int fwd_groups = B > FB ? 2 : 1;          // groups of CTAs that each own FB batch rows
-  const int fwd_parts = KB0 < KBh ? 2 : 1;
-  P.fwd_ncg = (H + FU - 1) / FU;                  // CTAs per group
-  P.fwd_smem = (KBh * FG + fwd_parts * KB0 * FB) * 128 + 2 * FB * PART_LD * 4 + 1024;
-  P.fwd_slab = false;                             // h_{k-1} by one copy per part instead of one per K tile
-  P.fwd_bb = KB0;                                 // K tiles per barrier
-  P.bwd_cs = 0; P.bwdc_smem = 0;
-  {
-    // function attributes belong to the device that is current
-    const int big = 220 * 1024;  // the kernels also hold a few static barriers
-    cudaFuncSetAttribute(fwd_run_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-    cudaFuncSetAttribute(bwd_run_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-  }
+  // Up to 512 hidden units a layer's recurrence fits a cluster; a wider one's exchange goes through a ring in the L2.
+  // A forward and a backward operation in runs of 32, against the kernels of this file: 2.8 -> 0.78 and 3.9 -> 0.90 us at
+  // H = 256, 3.1 -> 1.32 and 4.0 -> 1.73 us at H = 512, 4.1 -> 2.8 and 4.6 -> 3.1 us at H = 1024.
+  if (!cluster_maps(&P.tm_w_cl, &P.tm_wt_cl, wp_hh, wpT_hh, H)) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
+  P.run_rows = cluster_runs_supported(H) ? cluster_rows(B, H) : ring_rows(B, H);
+  if (P.run_rows <= 0) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
+  if (cluster_runs_supported(H) || B <= FB || B > 2 * FB || H % 128 != 0) return;
+  // Short runs (below).  Widths in whole blocks of 128: both kinds of kernels then add the same parts in the same order.
+  const int KBh = (H + 63) / 64, KB0 = fwd_first_part_blocks(H), kbs = (G / 64) / GCS;
+  P.fwd_ncg = H / FU;
+  P.fwd_smem = (KBh * FG + 2 * KB0 * FB) * 128 + 2 * FB * PART_LD * 4 + 1024;
+  P.bwd_tb = kbs > 8 ? 8 : 4;
+  P.bwd_smem = kbs * (FU * GCS * 128) + (kbs + P.bwd_tb - 1) / P.bwd_tb * P.bwd_tb * FB * 128 + 2 * GCS * FU * RECV_LD * 4 + 1024;
+  const void* fn = (const void*)bwd_run_group_kernel;
+  bool ok = cudaFuncSetAttribute(fwd_run_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) == cudaSuccess &&
+            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) == cudaSuccess;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * P.fwd_ncg); cfg.blockDim = dim3(192); cfg.dynamicSmemBytes = P.bwd_smem;
+  cudaLaunchAttribute at1[1];
+  at1[0].id = cudaLaunchAttributeClusterDimension;
+  at1[0].val.clusterDim.x = GCS; at1[0].val.clusterDim.y = 1; at1[0].val.clusterDim.z = 1;
+  cfg.attrs = at1; cfg.numAttrs = 1;
+  int nclusters = 0;
+  ok = ok && cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters * GCS >= 2 * P.fwd_ncg;
+  if (!ok) { cudaGetLastError(); return; }
   // the whole workspace as rows of H bfloat16: any h block starts at a whole row
-  const uint64_t rows = y.total / ((size_t)H * 2);
-  bool ok = make_tmap_2d(&P.tm_h, ws, 2, (uint64_t)H, rows, (uint64_t)H * 2, 64, FB);
-  ok = ok && make_tmap_2d(&P.tm_w, wp_hh, 2, (uint64_t)H, (uint64_t)G, (uint64_t)H * 2, 64, FG);
-  if (ok && H % 64 == 0) {
-    CUtensorMap blocked;
-    if (make_tmap_blocks64(&blocked, ws, (uint64_t)H, rows, (uint64_t)H * 2, FB, (uint32_t)P.fwd_bb)) {
-      P.tm_h = blocked;
-      P.fwd_slab = true;
-    }
-  }
+  ok = make_tmap_blocks64(&P.tm_h, ws, (uint64_t)H, y.total / ((size_t)H * 2), (uint64_t)H * 2, FB, (uint32_t)KB0) &&
+       make_tmap_2d(&P.tm_w, wp_hh, 2, (uint64_t)H, (uint64_t)G, (uint64_t)H * 2, 64, FG) &&
+       make_tmap_2d(&P.tm_wt, wpT_hh, 2, (uint64_t)G, (uint64_t)H, (uint64_t)G * 2, 64, FU * GCS);
   for (int pb = 0; pb < 2; ++pb)
-    ok = ok && make_tmap_2d(&P.tm_dz[pb], dz + (size_t)pb * S * B * G, 2, (uint64_t)G, (uint64_t)S * B, (uint64_t)G * 2, 64,
-                            (uint32_t)BM);
-  ok = ok && make_tmap_2d(&P.tm_wt, wpT_hh, 2, (uint64_t)G, (uint64_t)H, (uint64_t)G * 2, 64, NU);
-  if (!ok) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
-  // the clustered backward kernel, if the device can keep enough clusters resident
-  // (a switch in the environment can override the choice: env.hpp)
-  const int force = env::bwd_cluster();
-  for (int cs : {8, 4}) {
-    if (force >= 0 && force != cs) continue;
-    if (G % 64 != 0 || (G / 64) % cs != 0 || ncta % cs != 0 || (G / 64) / cs > 16) continue;
-    const int kbs = (G / 64) / cs;
-    const int tb = kbs > 8 ? 8 : 4;   // K tiles per barrier: at most four barriers, two where the slice is long
-    const int smem = kbs * (NU * cs * 128) + ((kbs + tb - 1) / tb) * tb * BM * 128 + 2 * cs * BM * NU * 4 + 1024;
-    if (smem > 220 * 1024) continue;
-    const void* fn = cs == 8 ? (const void*)bwd_run_cluster_kernel<8> : (const void*)bwd_run_cluster_kernel<4>;
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ncta); cfg.blockDim = dim3(192); cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at1[1];
-    at1[0].id = cudaLaunchAttributeClusterDimension;
-    at1[0].val.clusterDim.x = cs; at1[0].val.clusterDim.y = 1; at1[0].val.clusterDim.z = 1;
-    cfg.attrs = at1; cfg.numAttrs = 1;
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
-    if (nclusters * cs < ncta) continue;
-    P.bwd_cs = cs; P.bwdc_smem = smem; P.bwd_tb = tb;
-    break;
-  }
-  // the kernel with groups of batch rows, where the batch fills two groups and the driver takes a
-  // map that sees the staging chunk as [columns / 64][rows][64]
-  if (P.bwd_cs && force < 0 && !env::no_bwd_groups() && B > FB && B <= 2 * FB && H % (FU * GCS) == 0 &&
-      (G / 64) % GCS == 0 && (G / 64) / GCS <= 16) {
-    const int kbs = (G / 64) / GCS;
-    const int tb = kbs > 8 ? 8 : 4;
-    const int nq = (kbs + tb - 1) / tb;
-    const int smem = kbs * (FU * GCS * 128) + nq * tb * FB * 128 + 2 * GCS * FU * RECV_LD * 4 + 1024;
-    const int ncg = H / FU;
-    bool g_ok = smem <= 220 * 1024;
-    const void* fn = (const void*)bwd_run_group_kernel;
-    if (g_ok) {
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(2 * ncg); cfg.blockDim = dim3(192); cfg.dynamicSmemBytes = smem;
-      cudaLaunchAttribute at1[1];
-      at1[0].id = cudaLaunchAttributeClusterDimension;
-      at1[0].val.clusterDim.x = GCS; at1[0].val.clusterDim.y = 1; at1[0].val.clusterDim.z = 1;
-      cfg.attrs = at1; cfg.numAttrs = 1;
-      int nclusters = 0;
-      if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess) { cudaGetLastError(); g_ok = false; }
-      else g_ok = nclusters * GCS >= 2 * ncg;
-    }
-    for (int pb = 0; pb < 2 && g_ok; ++pb)
-      g_ok = make_tmap_blocks64(&P.tm_dz_g[pb], dz + (size_t)pb * S * B * G, (uint64_t)G, (uint64_t)S * B, (uint64_t)G * 2, FB,
-                                (uint32_t)tb);
-    g_ok = g_ok && make_tmap_2d(&P.tm_wt_g, wpT_hh, 2, (uint64_t)G, (uint64_t)H, (uint64_t)G * 2, 64, FU * GCS);
-    if (g_ok) { P.bwd_grp = true; P.bwdg_smem = smem; P.bwdg_tb = tb; P.bwdg_ncg = ncg; }
-  }
-  if (P.bwd_cs) {
-    // the staging chunk as [columns / 64][rows][64] if the driver takes such a map, else tile by tile
-    P.bwd_slab = true;
-    for (int pb = 0; pb < 2; ++pb)
-      P.bwd_slab = P.bwd_slab && make_tmap_blocks64(&P.tm_dz_b[pb], dz + (size_t)pb * S * B * G, (uint64_t)G, (uint64_t)S * B,
-                                                   (uint64_t)G * 2, 64, (uint32_t)P.bwd_tb);
-    if (!P.bwd_slab)
-      for (int pb = 0; pb < 2; ++pb)
-        ok = ok && make_tmap_2d(&P.tm_dz_b[pb], dz + (size_t)pb * S * B * G, 2, (uint64_t)G, (uint64_t)S * B,
-                                (uint64_t)G * 2, 64, 64);
-    ok = ok && make_tmap_2d(&P.tm_wt_c, wpT_hh, 2, (uint64_t)G, (uint64_t)H, (uint64_t)G * 2, 64, (uint32_t)(NU * P.bwd_cs));
-    if (!ok) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
-  }
-
+    ok = ok && make_tmap_blocks64(&P.tm_dz[pb], dz + (size_t)pb * S * B * G, (uint64_t)G, (uint64_t)S * B, (uint64_t)G * 2, FB, (uint32_t)P.bwd_tb);
+  P.short_runs = ok;
 }
+// Runs of fewer operations than these are short: the kernels of this file load half the weights at the start of a launch,
+// and take longer for an operation.  At H = 1024, B = 64, in us: forward some 1 + 4.1 n against 8 + 2.6 n, backward
+// 4.7 + 4.6 n against 9.1 + 2.8 n.
+constexpr int SHORT_FWD = 5, SHORT_BWD = 3;
 
 // The set for (problem, plan, workspace, device): from the cache, or built and put there.  ws may
 // be null: then only the host part is made (what counting launches needs, or a machine without a GPU).
@@ -1904,8 +1306,6 @@ int prepare_host(const Layout& y, const Plan* p, bool want_dx) { return prepare(
 int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_dx, cudaStream_t caller, bool dry,
                  bool side_stream) {
   const int B = y.B, H = y.H, I = y.I, O = y.O, S = y.S, G = 4 * H, K = I + H;
-  const int BM = 64;  // batch rows per MMA tile (B <= 64)
-  const int ncta = H / NU;
   int64_t launches = 0;
   char* ws = io.ws;
   auto at = [&](size_t off) { return ws + off; };
@@ -1939,13 +1339,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
 
   const int KBh = (H + 63) / 64;
   const int KB0 = fwd_first_part_blocks(H);       // 64-wide blocks of the recurrent contraction in its first part
-  const int fwd_groups = B > FB ? 2 : 1;          // groups of CTAs that each own FB batch rows
-  const int bwd_smem = ((G + 63) / 64) * 1024 + NST * BM * 128 + 1024;
-  const CUtensorMap &tm_h = P.tm_h, &tm_w = P.tm_w, &tm_wt = P.tm_wt, &tm_wt_c = P.tm_wt_c;
-  const CUtensorMap* tm_dz = P.tm_dz;
-  const CUtensorMap* tm_dz_b = P.tm_dz_b;
-  const int bwd_cs = P.bwd_cs, bwdc_smem = P.bwdc_smem, fwd_ncg = P.fwd_ncg, fwd_smem = P.fwd_smem, fwd_bb = P.fwd_bb;
-  const bool fwd_slab = P.fwd_slab;
+  const bool clusters = cluster_runs_supported(H);   // (else the ring, and for short runs perhaps the kernels of this file)
   // On request (a switch in the environment) the step runs on a stream of the library's, of the most
   // urgent priority, ordered after what the caller's stream holds and joined to it at the end: the
   // caller's stream is of the least urgent priority as a rule, like the stream of the weight-gradient
@@ -1969,6 +1363,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
     cudaMemsetAsync(io.counters, 0, 8 * sizeof(int64_t), s);
     cudaMemsetAsync(sync, 0, y.n_sync * 4, s);
     cudaMemsetAsync(status, 0, 256, s);
+    if (y.ring_bytes) cudaMemsetAsync(at(y.off_ring), 0xff, y.ring_bytes, s);   // nothing has been written there yet
     // (from page-locked memory: an asynchronous copy proper; from pageable memory, which only the
     // allocation-free entry point uses, the call may wait for the stream to reach the copy)
     cudaMemcpyAsync(at(y.off_tape), P.tape, P.tape_entries * sizeof(DevOp), cudaMemcpyHostToDevice, s);
@@ -2009,7 +1404,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
     }
   };
 
-  int launch_id = 0;
+  int launch_id = 0, fwd_launches = 0, bwd_launches = 0;
   int rc = MEBPTT_OK;
   const int fault = wait_fault_mask();   // testing aid, 0 outside the tests of the bounded waits
   if (!dry && !cuda_ok(cudaGetLastError(), "set-up (memsets, tape upload, weight packing)")) rc = MEBPTT_ERR_CUDA;
@@ -2073,22 +1468,23 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
         }
       }
       ++launches;
-      if (!dry && rc == MEBPTT_OK && P.cluster) {
-        const ClusterFwdArgs a{dops + i, n, ws, zx_cur + (size_t)(k0 - zx_lo) * B * G, status, io.counters, B, H, off16(y.plane),
-                               off16(y.hsz), (fault & 1) ? 16u : 0u, (fault & 1) ? fault_poll_limit : kSpinLimit};
+      if (!dry && rc == MEBPTT_OK) {
+        const float* zx_run = zx_cur + (size_t)(k0 - zx_lo) * B * G;
+        const uint32_t polls = (fault & 1) ? fault_poll_limit : kSpinLimit;
+        const ClusterFwdArgs a{dops + i, n, ws, zx_run, status, io.counters, B, H, off16(y.plane), off16(y.hsz), (fault & 1) ? 16u : 0u, polls};
         const int span = span_begin(timer, 0, n, s);
-        if (!cuda_ok(cluster_forward(P.tm_w_cl, a, P.cluster_rows, s), "forward run launch (clusters)")) rc = MEBPTT_ERR_CUDA;
-        span_end(timer, span, s);
-      } else if (!dry && rc == MEBPTT_OK) {
-        FwdRunArgs a{dops + i, n, ws, zx_cur + (size_t)(k0 - zx_lo) * B * G, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status,
-                     io.counters, B, H, fwd_ncg, fwd_bb, fwd_slab ? 1 : 0,
-                     (uint32_t)fwd_ncg + ((fault & 1) ? 1u : 0u), (fault & 1) ? fault_poll_limit : (kSpinLimit >> 1),
-                     off16(y.plane), off16(y.hsz)};
-        void* args[] = {(void*)&tm_h, (void*)&tm_w, (void*)&a};
-        const void* fn = (const void*)fwd_run_kernel;
-        const int span = span_begin(timer, 0, n, s);
-        if (!cuda_ok(launch_coop(fn, fwd_groups * fwd_ncg, 192, fwd_smem, s, args, 1), "forward run launch"))
-          rc = MEBPTT_ERR_CUDA;
+        cudaError_t e;
+        if (clusters) {
+          e = cluster_forward(P.tm_w_cl, a, P.run_rows, s);
+        } else if (P.short_runs && n < SHORT_FWD) {
+          FwdRunArgs sa{dops + i, n, ws, zx_run, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status, io.counters, B, H, P.fwd_ncg,
+                        (uint32_t)P.fwd_ncg + ((fault & 1) ? 1u : 0u), (fault & 1) ? fault_poll_limit : (kSpinLimit >> 1), off16(y.plane), off16(y.hsz)};
+          void* args[] = {(void*)&P.tm_h, (void*)&P.tm_w, (void*)&sa};
+          e = launch_coop((const void*)fwd_run_kernel, 2 * P.fwd_ncg, 192, P.fwd_smem, s, args, 1);
+        } else {
+          e = ring_forward(P.tm_w_cl, a, ring_args(at(y.off_ring), H, B, false, fwd_launches++, fault & 1, polls), P.run_rows, s);
+        }
+        if (!cuda_ok(e, "forward run launch")) rc = MEBPTT_ERR_CUDA;
         span_end(timer, span, s);
       }
       ++launch_id;
@@ -2159,35 +1555,25 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
       }
       gemm(dy_c + (size_t)s_lo * B * O, O, false, woutT, O, false,
            GemmOut{GemmOut::STORE_F32, dha + (size_t)s_lo * B * H, H, nullptr, 0}, n * B, H, O);
-      if (!dry && rc == MEBPTT_OK && P.cluster) {
+      if (!dry && rc == MEBPTT_OK) {
+        const uint32_t polls = (fault & 2) ? fault_poll_limit : kSpinLimit;
         const ClusterBwdArgs a{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, status, io.counters, B, H, S, off16(y.plane),
-                               leaf ? zleaf : nullptr, parts, (fault & 2) ? 16u : 0u, (fault & 2) ? fault_poll_limit : kSpinLimit};
+                               leaf ? zleaf : nullptr, parts, (fault & 2) ? 16u : 0u, polls};
         const int span = span_begin(timer, 1, n, s);
-        if (!cuda_ok(cluster_backward(P.tm_wt_cl, a, P.cluster_rows, s), "backward run launch (clusters)")) rc = MEBPTT_ERR_CUDA;
-        span_end(timer, span, s);
-      } else if (!dry && rc == MEBPTT_OK) {
-        const bool grouped = P.bwd_grp;
-        BwdRunArgs a{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status,
-                     io.counters, B, H, S, off16(y.plane), off16(y.hsz), leaf ? zleaf : nullptr, parts,
-                     grouped ? P.bwdg_tb : P.bwd_tb, (grouped || P.bwd_slab) ? 1 : 0,
-                     (uint32_t)(grouped ? P.bwdg_ncg : ncta) + ((fault & 2) ? 1u : 0u),
-                     (fault & 2) ? fault_poll_limit : (kSpinLimit >> 1)};
-        void* args[] = {(void*)(grouped ? &P.tm_dz_g[pb] : bwd_cs ? &tm_dz_b[pb] : &tm_dz[pb]),
-                        (void*)(grouped ? &P.tm_wt_g : bwd_cs ? &tm_wt_c : &tm_wt), (void*)&a};
-        const int span = span_begin(timer, 1, n, s);
-        if (grouped) {
-          if (!cuda_ok(launch_coop((const void*)bwd_run_group_kernel, 2 * P.bwdg_ncg, 192, P.bwdg_smem, s, args, GCS, false),
-                       "backward run launch (groups of batch rows)"))
-            rc = MEBPTT_ERR_CUDA;
-        } else if (bwd_cs) {
-          const void* fn = bwd_cs == 8 ? (const void*)bwd_run_cluster_kernel<8> : (const void*)bwd_run_cluster_kernel<4>;
-          // launched in plain stream order: early residency of a clustered grid measured no gain
-          if (!cuda_ok(launch_coop(fn, ncta, 192, bwdc_smem, s, args, bwd_cs, false), "backward run launch (clusters)"))
-            rc = MEBPTT_ERR_CUDA;
+        cudaError_t e;
+        if (clusters) {
+          e = cluster_backward(P.tm_wt_cl, a, P.run_rows, s);
+        } else if (P.short_runs && n < SHORT_BWD) {
+          BwdRunArgs sa{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status,
+                        io.counters, B, H, S, off16(y.plane), leaf ? zleaf : nullptr, parts, P.bwd_tb,
+                        (uint32_t)P.fwd_ncg + ((fault & 2) ? 1u : 0u), (fault & 2) ? fault_poll_limit : (kSpinLimit >> 1)};
+          void* args[] = {(void*)&P.tm_dz[pb], (void*)&P.tm_wt, (void*)&sa};
+          // (in plain stream order: early residency of a clustered cooperative grid measured no gain)
+          e = launch_coop((const void*)bwd_run_group_kernel, 2 * P.fwd_ncg, 192, P.bwd_smem, s, args, GCS, false);
         } else {
-          const void* fn = (const void*)bwd_run_kernel<64>;
-          if (!cuda_ok(launch_coop(fn, ncta, 128, bwd_smem, s, args, 1), "backward run launch")) rc = MEBPTT_ERR_CUDA;
+          e = ring_backward(P.tm_wt_cl, a, ring_args(at(y.off_ring), H, B, true, bwd_launches++, fault & 2, polls), P.run_rows, s);
         }
+        if (!cuda_ok(e, "backward run launch")) rc = MEBPTT_ERR_CUDA;
         span_end(timer, span, s);
       }
       ++launch_id;

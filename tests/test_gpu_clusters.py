@@ -1,15 +1,9 @@
-"""GPU: runs of the bfloat16 recurrence inside a thread-block cluster (one layer of at most 512 units), at the edges
-of what a cluster, a CTA and an MMA tile hold; and the grid-wide kernels that wider layers keep.
+"""GPU: runs of the bfloat16 recurrence of one layer -- inside a thread-block cluster up to 512 units, through a ring in
+the L2 and, for short runs, by the grid-wide kernels beyond -- at the edges of what a cluster, a CTA and an MMA tile hold.
 """
-import json
-import os
-import subprocess
-import sys
-
 import pytest
 
 from paper_1606_03401_b200 import synth
-from tests.test_gpu_variants import CHILD, ROOT
 from tests.util import assert_bit_identical, assert_close_to_oracle, oracle_run
 
 pytestmark = pytest.mark.gpu
@@ -31,6 +25,9 @@ def _problem(**size):
     (264, 33), (312, 46),       # 9 and 10 CTAs
     (496, 24), (504, 64),       # 16 CTAs, the last with half and with three quarters of its units
     (512, 64), (512, 48),
+    # wider: 17 CTAs forward and 24 backward, a part of the contraction of 32 columns; 24 and 24; 25 and 32
+    (520, 9), (640, 64), (768, 16), (776, 33),
+    (1000, 20), (1024, 64), (1024, 1),
 ])
 def test_clusters_match_the_oracle_and_every_plan_gives_the_same_bits(hidden, batch):
     cfg, dp = _problem(input=40, hidden=hidden, batch=batch, readout=24, t=41)
@@ -46,10 +43,10 @@ def test_clusters_match_the_oracle_and_every_plan_gives_the_same_bits(hidden, ba
 
 
 @pytest.mark.parametrize("bit", [1, 2])
-@pytest.mark.parametrize("hidden,batch", [(72, 9), (640, 64), (640, 20)])
-def test_waits_of_both_kinds_of_runs_run_out_and_report_timeout(bit, hidden, batch):
+@pytest.mark.parametrize("hidden,batch,t", [(72, 9, 12), (640, 64, 12), (640, 20, 12), (640, 64, 2)])   # clusters, ring, short runs
+def test_waits_of_all_kinds_of_runs_run_out_and_report_timeout(bit, hidden, batch, t):
     from paper_1606_03401_b200 import binding as B
-    cfg, dp = _problem(input=40, hidden=hidden, batch=batch, readout=24, t=12)
+    cfg, dp = _problem(input=40, hidden=hidden, batch=batch, readout=24, t=t)
     plan = dp.full_memory_plan()
     clean = dp.run(plan)
     assert clean["counters"][3] == 0
@@ -63,17 +60,12 @@ def test_waits_of_both_kinds_of_runs_run_out_and_report_timeout(bit, hidden, bat
     assert_bit_identical(again, clean, want_dx=True)
 
 
-def test_backward_kernels_of_wide_layers_give_the_same_bits():
-    child = CHILD.replace("hidden=256", "hidden=640")
-    assert child != CHILD
-
-    def digest(env_extra):
-        env = {k: v for k, v in os.environ.items() if not k.startswith("MEBPTT_")}
-        env.update(env_extra)
-        out = subprocess.run([sys.executable, "-c", child.format(root=ROOT)], env=env, capture_output=True, text=True, timeout=600)
-        assert out.returncode == 0, out.stderr[-2000:]
-        return json.loads([l for l in out.stdout.splitlines() if l.startswith("DIGEST ")][-1][len("DIGEST "):])
-
-    base = digest({})
-    assert base["msm"] == base["full"]
-    assert digest({"MEBPTT_BWD_CLUSTER": "4"}) == base
+def test_short_and_long_runs_of_wide_layers_give_the_same_bits():
+    """Runs of few operations take other kernels: plans whose runs are all short, all long and mixed."""
+    for size in (dict(hidden=640, batch=64), dict(hidden=1024, batch=37)):
+        cfg, dp = _problem(input=40, readout=24, t=36, **size)
+        full = dp.run(dp.full_memory_plan())
+        for plan in (dp.plan("hsm", 1), dp.plan("ism", 2), dp.plan("ism", 4), dp.plan("msm", 13)):
+            res = dp.run(plan)
+            assert res["counters"][0] == plan.cost and res["counters"][3] == 0
+            assert_bit_identical(res, full, want_dx=True)

@@ -241,7 +241,10 @@ __global__ void __launch_bounds__(THREADS, 1) fwd_run_cluster(const __grid_const
       }
       // the rest of the state, off the critical path
       if (got) {
-        if (pvalid && lane < RB) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.ws + (size_t)op.h_dst * 16) + ep) = hnew;
+        if (pvalid && lane < RB) {
+          *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.ws + (size_t)op.h_dst * 16) + ep) = hnew;
+          if (op.stage) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.ws + (size_t)op.stage * 16) + ep) = hnew;
+        }
         if (op.gates) {
 #pragma unroll
           for (int v = 0; v < NV; ++v)
@@ -538,7 +541,10 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_run_cluster(const __grid_c
   cluster_sync();
   if (tid == 0) {
     if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (blockIdx.x == 0) a.counters[1] += a.n;
+    else if (blockIdx.x == 0) {
+      a.counters[0] += a.fwd_ops;
+      a.counters[1] += a.n;
+    }
   }
   if (warp == 4) tmem_dealloc(tmem, tmem_cols((64 + CB) * MT));
 }

@@ -91,7 +91,7 @@ struct Layout {
   size_t off_wp_ih = 0, off_wp_hh = 0, off_wpT_hh = 0, off_wpT_ih = 0, off_bias_p = 0, off_woutT = 0;
   size_t off_a3 = 0, off_w3 = 0, off_wmn3 = 0, off_wout3 = 0, off_woutmn3 = 0;
   size_t off_z = 0, off_split = 0, off_st_dz = 0, off_st_in = 0, off_st_hp = 0, off_st_dy = 0, off_st_h = 0;
-  size_t off_zx = 0, off_zleaf = 0, off_hprev = 0, off_hk = 0, off_y = 0;
+  size_t off_zx = 0, off_zleaf = 0, off_hk = 0, off_y = 0;
   size_t off_sync = 0, off_tape = 0, off_status = 0, off_split_dh = 0;
   size_t off_w_f = 0, off_w_b = 0, off_exch_f = 0, off_exch_b = 0;
   size_t off_a3_run = 0, off_zrun = 0, off_hrun = 0, off_dha_run = 0, off_zleaf3 = 0, off_leaf = 0, split_floats = 0;
@@ -442,8 +442,8 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     // two copies of what the weight-gradient GEMMs read: they may still be running (on the
     // library's side stream) while the backward pass fills the stages of the next chunk
     y.off_dz = take(2 * SB * G * 2);
-    y.off_hprev = take(2 * SB * y.H * 2);
-    y.off_hk = take(2 * SB * y.H * 2);
+    // h of the chunk's steps and of the one before: row block i holds h_{k-1} of the step with row block i in dz
+    y.off_hk = take(2 * (SB + y.B) * y.H * 2);
     y.off_y = take(SB * y.O * 4);
     y.off_dy = take(2 * SB * y.O * 2);
     y.off_dha = take(SB * y.H * 4);

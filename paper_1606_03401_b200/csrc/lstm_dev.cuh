@@ -11,7 +11,7 @@ namespace tc {
 // Tape entry as the kernels see it.  Offsets are in units of 16 bytes from the workspace base.
 struct DevOp {
   int32_t k;
-  int32_t fmt;
+  uint32_t stage;          // FWD: where h_k goes besides, for the chunk that is backpropagated next, 0 = nowhere
   uint32_t h_src, c_src;   // FWD: state k-1.            BWD: h_{k-1}, c_{k-1}
   uint32_t h_dst, c_dst;   // FWD: where h_k, c_k go.    BWD: h_k, c_k of the stored internal state
   uint32_t gates;          // FWD: gate planes to write, 0 = none.   BWD: gate planes to read

@@ -361,7 +361,10 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
       }
       // the rest of the state, off the critical path
       if (got) {
-        if (pvalid && lane < 8) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.ws + (size_t)op.h_dst * 16) + ep) = hnew;
+        if (pvalid && lane < 8) {
+          *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.ws + (size_t)op.h_dst * 16) + ep) = hnew;
+          if (op.stage) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(a.ws + (size_t)op.stage * 16) + ep) = hnew;
+        }
         if (op.gates) {
 #pragma unroll
           for (int v = 0; v < 2; ++v)
@@ -674,7 +677,10 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
   cluster_sync();     // no CTA leaves while a peer may still push to it
   if (tid == 0) {
     if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (blockIdx.x == 0) a.counters[1] += a.n;
+    else if (blockIdx.x == 0) {
+      a.counters[0] += a.fwd_ops;
+      a.counters[1] += a.n;
+    }
   }
   if (warp == GATES) tmem_dealloc(tmem, 512);
 }

@@ -21,6 +21,7 @@
 // the backward pass has completed a chunk of S steps aligned to absolute time -- the weight
 // gradients.  Chunks are tied to time indices, not to run boundaries, and backward steps always
 // come in the order t .. 1, so every sum runs in the same order under every plan.
+#include <algorithm>
 #include <atomic>
 #include <cstdio>
 #include <cstdlib>
@@ -162,6 +163,7 @@ __device__ __forceinline__ void fwd_cell_rest(FwdCell& st, const FwdRunArgs& a, 
                                               int i, int b, int j0, size_t e0) {
   char* ws = a.ws;
   *(reinterpret_cast<float4*>(ws + (size_t)op.c_dst * 16) + e0 / 4) = make_float4(st.c[0], st.c[1], st.c[2], st.c[3]);
+  if (op.stage) *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(ws + (size_t)op.stage * 16) + e0) = o.hnew;
   if (op.gates) {
     __nv_bfloat16* gp = reinterpret_cast<__nv_bfloat16*>(ws + (size_t)op.gates * 16) + e0;
     const size_t pl = (size_t)a.plane16 * 8;   // elements
@@ -373,6 +375,7 @@ struct BwdRunArgs {
   uint32_t plane16;
   const float* zleaf;      // leaf batch: [S][B][4H] pre-activations z_k (gate columns permuted); NULL otherwise
   int loss_parts;          // partial sums of the loss per step
+  int fwd_ops;             // forward operations that were done without a kernel that counts them
   int tb;                  // K tiles per barrier and per copy
   uint32_t expect;         // signals a step is complete with: the grid size (a testing aid may ask for one too many)
   uint32_t poll_limit;     // polls of the step counter before the wait gives up
@@ -665,7 +668,10 @@ __global__ void __launch_bounds__(192, 1) bwd_run_group_kernel(const __grid_cons
   cluster_sync();   // no CTA leaves while a peer may still read its partial tiles or signal it
   if (tid == 0) {
     if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (blockIdx.x == 0) a.counters[1] += a.n;
+    else if (blockIdx.x == 0) {
+      a.counters[0] += a.fwd_ops;
+      a.counters[1] += a.n;
+    }
   }
   if (warp == 4) tmem_dealloc(tmem, 32);
 }
@@ -778,9 +784,10 @@ __global__ void __launch_bounds__(256) pack_weights(const __nv_bfloat16* W, cons
   }
 }
 
-// Copies h_k and h_{k-1} of each step of a backward run from wherever the internal state lies
-// into the staging chunk (row block (k-1) % S), 16 bytes per thread per access.
-__global__ void gather_states(const DevOp* ops, int n, const char* ws, uint4* hk, uint4* hprev, int S,
+// Copies h_k of each step of a backward run, and h_{k-1} of the earliest, from wherever the internal state lies into the
+// chunk's stage (h_k in row block (k-1) % S + 1), 16 bytes per thread per access; of a batch of leaves, whose h_k
+// leaf_forward makes, h_{k-1} of each.
+__global__ void gather_states(const DevOp* ops, int n, const char* ws, uint4* stage, bool leaf, int S,
                               size_t block16) {  // block16: B*H*2/16
   grid_dep_wait();
   grid_dep_launch();
@@ -788,11 +795,12 @@ __global__ void gather_states(const DevOp* ops, int n, const char* ws, uint4* hk
   const int sidx = (op.k - 1) % S;
   const uint4* src_k = reinterpret_cast<const uint4*>(ws + (size_t)op.h_dst * 16);
   const uint4* src_p = reinterpret_cast<const uint4*>(ws + (size_t)op.h_src * 16);
-  uint4* dk = hk + (size_t)sidx * block16;
-  uint4* dp = hprev + (size_t)sidx * block16;
+  uint4* dk = stage + (size_t)(sidx + 1) * block16;
+  uint4* dp = stage + (size_t)sidx * block16;
+  const bool prev = leaf || (int)blockIdx.y == n - 1;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < block16; e += (size_t)gridDim.x * blockDim.x) {
-    if (hk) dk[e] = src_k[e];   // leaf batches have no stored h_k: leaf_forward writes it
-    dp[e] = src_p[e];
+    if (!leaf) dk[e] = src_k[e];
+    if (prev) dp[e] = src_p[e];
   }
 }
 
@@ -821,18 +829,17 @@ __global__ void leaf_forward(const DevOp* ops, int n, const char* ws, const floa
 
 // y (float32, readout with bias) -> dy = 2 (y - target) / (B O) in bfloat16, and LOSS_PARTS
 // partial sums of the squared error per step (each a fixed-order sum over a fixed slice).
-__global__ void loss_dy(const DevOp* ops, const float* y, const float* targets, __nv_bfloat16* dy, float* loss_part,
-                        int S, int B, int O) {
+// step0: index of the first step (0-based), s0: its row block.
+__global__ void loss_dy(const float* y, const float* targets, __nv_bfloat16* dy, float* loss_part, int step0, int s0, int B, int O) {
   __shared__ float red[256];
   grid_dep_wait();
   grid_dep_launch();
-  const DevOp op = ops[blockIdx.y];
-  const int sidx = (op.k - 1) % S;
+  const int sidx = s0 + (int)blockIdx.y;
   const size_t n = (size_t)B * O;
   const size_t per = (n + LOSS_PARTS - 1) / LOSS_PARTS;
   const size_t lo = blockIdx.x * per, hi = (lo + per < n) ? lo + per : n;
   const float* yp = y + (size_t)sidx * n;
-  const float* tp = targets + (size_t)(op.k - 1) * n;
+  const float* tp = targets + (size_t)(step0 + (int)blockIdx.y) * n;
   __nv_bfloat16* dp = dy + (size_t)sidx * n;
   const float inv = 1.f / ((float)B * (float)O);
   float s = 0.f;
@@ -1113,6 +1120,7 @@ struct Prepared {
   // host part
   std::vector<WorkItem> items;
   std::vector<int> zx_next;  // per item that opens a window: the item that opens the next one (-1: none)
+  std::vector<int> next_chunk;  // per item: the chunk of the next item that backpropagates (itself included; -1: none)
   std::vector<int> zx_hi;  // per item: a forward run that projects its inputs anew does so up to this step (exclusive); 0: the window in place serves it
   DevOp* tape = nullptr;   // [2 nops]: the tape, then the compacted leaves of leaf batches
   size_t tape_entries = 0;
@@ -1157,6 +1165,14 @@ void build_host_part(Prepared& P, const Layout& y, const Plan* p, bool allow_pin
   P.zx_next.assign(P.items.size(), -1);
   for (int item = (int)P.items.size() - 1, next = -1; item >= 0; --item)
     if (P.zx_hi[item]) { P.zx_next[item] = next; next = item; }
+  P.next_chunk.assign(P.items.size(), -1);
+  std::vector<int> op_chunk(nops, -1);   // of a forward run's operations: that chunk
+  for (int item = (int)P.items.size() - 1, next = -1; item >= 0; --item) {
+    const WorkItem& wi = P.items[item];
+    if (wi.kind != WorkItem::FWD) next = (p->tape[wi.i].k - 1) / S;
+    else for (int j = 0; j < wi.n; ++j) op_chunk[wi.i + (size_t)j] = next;
+    P.next_chunk[item] = next;
+  }
   // the tape as the kernels read it
   P.tape_entries = 2 * nops;
   const size_t bytes = (P.tape_entries ? P.tape_entries : 1) * sizeof(DevOp);
@@ -1174,8 +1190,11 @@ void build_host_part(Prepared& P, const Layout& y, const Plan* p, bool allow_pin
     const mebptt_op& op = p->tape[i];
     DevOp d{};
     d.k = op.k;
-    d.fmt = op.dst_fmt;
     if (op.kind == MEBPTT_OP_FWD) {
+      // A forward operation leaves its h in the stage of the chunk that is backpropagated next, if it is one of the chunk's
+      // steps or the one before them: readouts and weight gradients read it there.
+      const int c = op_chunk[i], block = c < 0 ? -1 : op.k - c * S;
+      if (block >= 0 && block <= S) d.stage = off16(y.off_hk + ((size_t)(c & 1) * (S + 1) + block) * (size_t)y.B * y.H * 2);
       const size_t src = block_off(op.src), dst = block_off(op.dst);
       d.h_src = off16(src); d.c_src = off16(src + y.hsz);
       d.h_dst = off16(dst); d.c_dst = off16(dst + y.hsz);
@@ -1324,7 +1343,6 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
   float* dc = reinterpret_cast<float*>(at(y.off_dc));
   float* zx = reinterpret_cast<float*>(at(y.off_zx));
   __nv_bfloat16* dz = reinterpret_cast<__nv_bfloat16*>(at(y.off_dz));
-  __nv_bfloat16* hprev = reinterpret_cast<__nv_bfloat16*>(at(y.off_hprev));
   __nv_bfloat16* hk = reinterpret_cast<__nv_bfloat16*>(at(y.off_hk));
   float* yv = reinterpret_cast<float*>(at(y.off_y));
   __nv_bfloat16* dyv = reinterpret_cast<__nv_bfloat16*>(at(y.off_dy));
@@ -1437,6 +1455,22 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
             GemmOut{GemmOut::STORE_F32, zx + (size_t)(w & 1) * S * B * G, G, bias_p, 0}, (hi - k0) * B, G, I);
     cudaEventRecord(side->zx_ready[w & 1], side->zx);
   };
+  // The stage of the chunk that is being backpropagated, or will be next: which row blocks of h it has, and of which steps
+  // the readout is done (loss, dy and the gradient entering h, for all that follows in the chunk).
+  int cur = -1;
+  std::vector<char> has_h((size_t)S + 1, 0), is_read((size_t)S, 0);
+  auto enter_chunk = [&](int c) {
+    if (c != cur) {
+      cur = c;
+      std::fill(has_h.begin(), has_h.end(), 0);
+      std::fill(is_read.begin(), is_read.end(), 0);
+    }
+    if (side && side_busy[c & 1]) {
+      // these stages were last read by GEMMs on the side stream (two chunks ago): wait for them
+      cudaStreamWaitEvent(s, side->done[c & 1], 0);
+      side_busy[c & 1] = false;
+    }
+  };
   for (size_t item = 0; item < items.size() && rc == MEBPTT_OK; ++item) {
     const WorkItem& wi = items[item];
     const size_t i = wi.i;
@@ -1466,6 +1500,11 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
           if (P.zx_next[item] >= 0) project_window((size_t)P.zx_next[item], zx_w + 1);
           zx_cur = zx + (size_t)(zx_w & 1) * S * B * G;
         }
+      }
+      if (const int c = P.next_chunk[item]; c >= 0 && k0 + n > c * S && k0 <= (c + 1) * S) {
+        enter_chunk(c);
+        for (int k = k0; k < k0 + n; ++k)
+          if (k >= c * S && k <= (c + 1) * S) has_h[(size_t)(k - c * S)] = 1;
       }
       ++launches;
       if (!dry && rc == MEBPTT_OK) {
@@ -1501,24 +1540,27 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
       const int pb = chunk & 1;   // which copy of the stages this chunk uses
       const int n = wi.n;
       const int k_hi = first.k, k_lo = k_hi - n + 1;
-      const int s_lo = (k_lo - 1) % S;
-      need_targets(k_lo);   // the targets of steps k_lo .. t (backward steps come in descending order)
+      const int s_lo = (k_lo - 1) % S, s_hi = s_lo + n - 1;
       const size_t SB = (size_t)S * B;
       __nv_bfloat16* dz_c = dz + (size_t)pb * SB * G;
-      __nv_bfloat16* hprev_c = hprev + (size_t)pb * SB * H;
-      __nv_bfloat16* hk_c = hk + (size_t)pb * SB * H;
+      __nv_bfloat16* hprev_c = hk + (size_t)pb * (SB + B) * H;   // row block i: h_{k-1} of the step in row block i of dz
+      __nv_bfloat16* hk_c = hprev_c + (size_t)B * H;             // the same seen from h_k
       __nv_bfloat16* dy_c = dyv + (size_t)pb * SB * O;
-      if (side && side_busy[pb]) {
-        // these stages were last read by GEMMs on the side stream (two chunks ago): wait for them
-        cudaStreamWaitEvent(s, side->done[pb], 0);
-        side_busy[pb] = false;
+      enter_chunk(chunk);
+      ++launches;      // the backward run itself
+      // what the forward runs did not leave in the stage comes from the stored states
+      const size_t last_block = (size_t)s_hi + (leaf ? 0 : 1);
+      bool staged = true;
+      for (size_t i2 = (size_t)s_lo; i2 <= last_block; ++i2) staged = staged && has_h[i2];
+      if (!staged) {
+        ++launches;
+        if (!dry && rc == MEBPTT_OK)
+          launch_pdl(gather_states, dim3(16, n), dim3(256), 0, s, bops, n, ws, reinterpret_cast<uint4*>(hprev_c), leaf, S,
+                     (size_t)B * H * 2 / 16);
+        for (size_t i2 = (size_t)s_lo; i2 <= last_block; ++i2) has_h[i2] = 1;
       }
-      launches += 2;   // gather_states and the backward run itself
-      if (!dry && rc == MEBPTT_OK) {
-        const size_t block16 = (size_t)B * H * 2 / 16;
-        launch_pdl(gather_states, dim3(16, n), dim3(256), 0, s, bops, n, ws,
-                   leaf ? nullptr : reinterpret_cast<uint4*>(hk_c), reinterpret_cast<uint4*>(hprev_c), S, block16);
-      }
+      bool all_read = true;
+      for (int q = s_lo; q <= s_hi; ++q) all_read = all_read && is_read[(size_t)q];
       if (leaf) {
         // z_k = W_ih x_k + b + W_hh h_{k-1} for the n leaves at once (their h_{k-1} are all
         // memorised), then h_k; the gates are redone inside the backward kernel
@@ -1532,40 +1574,54 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
         if (k_first < H)
           gemm(hprev_c + (size_t)s_lo * B * H + k_first, H, false, wp_hh + k_first, H, false,
                GemmOut{GemmOut::ACCUM_F32, zleaf + (size_t)s_lo * B * G, G, nullptr, 0}, n * B, G, H - k_first);
-        ++launches;
-        if (!dry && rc == MEBPTT_OK)
-          launch_pdl(leaf_forward, dim3(32, n), dim3(256), 0, s, bops, n, ws, zleaf, hk_c, S, B, H, io.counters);
+        if (!all_read) {
+          ++launches;
+          if (!dry && rc == MEBPTT_OK)
+            launch_pdl(leaf_forward, dim3(32, n), dim3(256), 0, s, bops, n, ws, zleaf, hk_c, S, B, H, io.counters);
+          for (int q = s_lo; q <= s_hi; ++q) has_h[(size_t)q + 1] = 1;
+        }
       }
-      // readout of the n steps at once, loss terms and dy, then the gradient entering h_k
+      // Readout of the run's steps as far as it is not done, together with all steps before them whose h is there already
+      // (as a rule all of the chunk that the last sweep passed): loss terms and dy, then the gradient entering h_k.  A run
+      // at a time it was a gather and two products, 20 us at H = 1024, in front of every one of 630 short runs.
       const bool fused_loss = loss_fused(B, O);
       const int parts = loss_parts_per_step(B, O);
-      if (fused_loss) {
-        GemmOut o{GemmOut::LOSS_DY, dy_c + (size_t)s_lo * B * O, O, io.b_out, 0};
-        o.target = io.targets + (size_t)(k_lo - 1) * B * O;
-        o.loss_part = loss_part + (size_t)s_lo * parts;
-        o.parts = (O + 31) / 32;
-        o.scale = 1.f / ((float)B * (float)O);
-        gemm(hk_c + (size_t)s_lo * B * H, H, false, io.W_out, H, false, o, n * B, O, H);
-      } else {
-        gemm(hk_c + (size_t)s_lo * B * H, H, false, io.W_out, H, false,
-             GemmOut{GemmOut::STORE_F32, yv + (size_t)s_lo * B * O, O, io.b_out, 0}, n * B, O, H);
-        ++launches;
-        if (!dry && rc == MEBPTT_OK)
-          launch_pdl(loss_dy, dim3(LOSS_PARTS, n), dim3(256), 0, s, bops, yv, io.targets, dy_c, loss_part, S, B, O);
+      for (int hi = s_hi; hi >= s_lo;) {
+        if (is_read[(size_t)hi]) { --hi; continue; }
+        int lo = hi;
+        while (lo > 0 && !is_read[(size_t)lo - 1] && has_h[(size_t)lo]) --lo;
+        const int steps = hi - lo + 1;
+        need_targets(chunk * S + lo + 1);   // of these steps and all after them (backward steps come in descending order)
+        if (fused_loss) {
+          GemmOut o{GemmOut::LOSS_DY, dy_c + (size_t)lo * B * O, O, io.b_out, 0};
+          o.target = io.targets + (size_t)(chunk * S + lo) * B * O;
+          o.loss_part = loss_part + (size_t)lo * parts;
+          o.parts = (O + 31) / 32;
+          o.scale = 1.f / ((float)B * (float)O);
+          gemm(hk_c + (size_t)lo * B * H, H, false, io.W_out, H, false, o, steps * B, O, H);
+        } else {
+          gemm(hk_c + (size_t)lo * B * H, H, false, io.W_out, H, false,
+               GemmOut{GemmOut::STORE_F32, yv + (size_t)lo * B * O, O, io.b_out, 0}, steps * B, O, H);
+          ++launches;
+          if (!dry && rc == MEBPTT_OK)
+            launch_pdl(loss_dy, dim3(LOSS_PARTS, steps), dim3(256), 0, s, yv, io.targets, dy_c, loss_part, chunk * S + lo, lo, B, O);
+        }
+        gemm(dy_c + (size_t)lo * B * O, O, false, woutT, O, false,
+             GemmOut{GemmOut::STORE_F32, dha + (size_t)lo * B * H, H, nullptr, 0}, steps * B, H, O);
+        for (int q = lo; q <= hi; ++q) is_read[(size_t)q] = 1;
+        hi = lo - 1;
       }
-      gemm(dy_c + (size_t)s_lo * B * O, O, false, woutT, O, false,
-           GemmOut{GemmOut::STORE_F32, dha + (size_t)s_lo * B * H, H, nullptr, 0}, n * B, H, O);
       if (!dry && rc == MEBPTT_OK) {
         const uint32_t polls = (fault & 2) ? fault_poll_limit : kSpinLimit;
         const ClusterBwdArgs a{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, status, io.counters, B, H, S, off16(y.plane),
-                               leaf ? zleaf : nullptr, parts, (fault & 2) ? 16u : 0u, polls};
+                               leaf ? zleaf : nullptr, parts, leaf && all_read ? n : 0, (fault & 2) ? 16u : 0u, polls};
         const int span = span_begin(timer, 1, n, s);
         cudaError_t e;
         if (clusters) {
           e = cluster_backward(P.tm_wt_cl, a, P.run_rows, s);
         } else if (P.short_runs && n < SHORT_BWD) {
           BwdRunArgs sa{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status,
-                        io.counters, B, H, S, off16(y.plane), leaf ? zleaf : nullptr, parts, P.bwd_tb,
+                        io.counters, B, H, S, off16(y.plane), leaf ? zleaf : nullptr, parts, leaf && all_read ? n : 0, P.bwd_tb,
                         (uint32_t)P.fwd_ncg + ((fault & 2) ? 1u : 0u), (fault & 2) ? fault_poll_limit : (kSpinLimit >> 1)};
           void* args[] = {(void*)&P.tm_dz[pb], (void*)&P.tm_wt, (void*)&sa};
           // (in plain stream order: early residency of a clustered cooperative grid measured no gain)

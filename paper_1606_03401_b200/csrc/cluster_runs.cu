@@ -541,10 +541,7 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_run_cluster(const __grid_c
   cluster_sync();
   if (tid == 0) {
     if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (blockIdx.x == 0) {
-      a.counters[0] += a.fwd_ops;
-      a.counters[1] += a.n;
-    }
+    else if (blockIdx.x == 0) a.counters[1] += a.n;
   }
   if (warp == 4) tmem_dealloc(tmem, tmem_cols((64 + CB) * MT));
 }

@@ -46,7 +46,6 @@ struct ClusterBwdArgs {
   uint32_t plane16;
   const float* zleaf;      // leaf batch: [S][B][4H] pre-activations z_k (gate columns permuted); NULL otherwise
   int loss_parts;          // partial sums of the loss per step
-  int fwd_ops;             // forward operations that were done without a kernel that counts them
   uint32_t extra, poll_limit;
 };
 

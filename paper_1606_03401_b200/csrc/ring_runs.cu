@@ -677,10 +677,7 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
   cluster_sync();     // no CTA leaves while a peer may still push to it
   if (tid == 0) {
     if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (blockIdx.x == 0) {
-      a.counters[0] += a.fwd_ops;
-      a.counters[1] += a.n;
-    }
+    else if (blockIdx.x == 0) a.counters[1] += a.n;
   }
   if (warp == GATES) tmem_dealloc(tmem, 512);
 }

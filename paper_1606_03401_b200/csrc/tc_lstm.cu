@@ -33,6 +33,7 @@
 #include "cluster_runs.hpp"
 #include "launch.hpp"
 #include "layout.hpp"
+#include "leaf_products.hpp"
 #include "lstm_dev.cuh"
 #include "ring_runs.hpp"
 #include "sm100.cuh"
@@ -375,7 +376,6 @@ struct BwdRunArgs {
   uint32_t plane16;
   const float* zleaf;      // leaf batch: [S][B][4H] pre-activations z_k (gate columns permuted); NULL otherwise
   int loss_parts;          // partial sums of the loss per step
-  int fwd_ops;             // forward operations that were done without a kernel that counts them
   int tb;                  // K tiles per barrier and per copy
   uint32_t expect;         // signals a step is complete with: the grid size (a testing aid may ask for one too many)
   uint32_t poll_limit;     // polls of the step counter before the wait gives up
@@ -668,10 +668,7 @@ __global__ void __launch_bounds__(192, 1) bwd_run_group_kernel(const __grid_cons
   cluster_sync();   // no CTA leaves while a peer may still read its partial tiles or signal it
   if (tid == 0) {
     if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (blockIdx.x == 0) {
-      a.counters[0] += a.fwd_ops;
-      a.counters[1] += a.n;
-    }
+    else if (blockIdx.x == 0) a.counters[1] += a.n;
   }
   if (warp == 4) tmem_dealloc(tmem, 32);
 }
@@ -786,7 +783,7 @@ __global__ void __launch_bounds__(256) pack_weights(const __nv_bfloat16* W, cons
 
 // Copies h_k of each step of a backward run, and h_{k-1} of the earliest, from wherever the internal state lies into the
 // chunk's stage (h_k in row block (k-1) % S + 1), 16 bytes per thread per access; of a batch of leaves, whose h_k
-// leaf_forward makes, h_{k-1} of each.
+// leaf_products makes, h_{k-1} of each.
 __global__ void gather_states(const DevOp* ops, int n, const char* ws, uint4* stage, bool leaf, int S,
                               size_t block16) {  // block16: B*H*2/16
   grid_dep_wait();
@@ -802,29 +799,6 @@ __global__ void gather_states(const DevOp* ops, int n, const char* ws, uint4* st
     if (!leaf) dk[e] = src_k[e];
     if (prev) dp[e] = src_p[e];
   }
-}
-
-// The forward operations of a batch of leaves, after the batched GEMMs have produced their
-// pre-activations z (row block (k-1) % S, gate columns 4 u + q): h_k = o tanh(f c_{k-1} + i g),
-// written to the staging chunk for the readout and the weight gradients.  Same arithmetic as the
-// epilogue of the forward run kernel; the gates themselves are redone by the backward kernel.
-__global__ void leaf_forward(const DevOp* ops, int n, const char* ws, const float* z, __nv_bfloat16* hk, int S, int B,
-                             int H, int64_t* counters) {
-  grid_dep_wait();
-  grid_dep_launch();
-  const DevOp op = ops[blockIdx.y];
-  const int sidx = (op.k - 1) % S;
-  const size_t bh = (size_t)B * H;
-  const float* cprev = reinterpret_cast<const float*>(ws + (size_t)op.c_src * 16);
-  const float4* zs = reinterpret_cast<const float4*>(z + (size_t)sidx * bh * 4);
-  __nv_bfloat16* out = hk + (size_t)sidx * bh;
-  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < bh; e += (size_t)gridDim.x * blockDim.x) {
-    const float4 zz = zs[e];   // (b, u): columns 4 u .. 4 u + 3 of row b
-    const float iv = sigmoid_fast(zz.x), fv = sigmoid_fast(zz.y), gv = tanh_fast(zz.z), ov = sigmoid_fast(zz.w);
-    const float c = fmaf(fv, cprev[e], iv * gv);
-    out[e] = __float2bfloat16_rn(ov * tanh_fast(c));
-  }
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) counters[0] += n;
 }
 
 // y (float32, readout with bias) -> dy = 2 (y - target) / (B O) in bfloat16, and LOSS_PARTS
@@ -1355,8 +1329,6 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
   float* bias_p = reinterpret_cast<float*>(at(y.off_bias_p));
   __nv_bfloat16* woutT = reinterpret_cast<__nv_bfloat16*>(at(y.off_woutT));
 
-  const int KBh = (H + 63) / 64;
-  const int KB0 = fwd_first_part_blocks(H);       // 64-wide blocks of the recurrent contraction in its first part
   const bool clusters = cluster_runs_supported(H);   // (else the ring, and for short runs perhaps the kernels of this file)
   // On request (a switch in the environment) the step runs on a stream of the library's, of the most
   // urgent priority, ordered after what the caller's stream holds and joined to it at the end: the
@@ -1559,27 +1531,15 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
                      (size_t)B * H * 2 / 16);
         for (size_t i2 = (size_t)s_lo; i2 <= last_block; ++i2) has_h[i2] = 1;
       }
-      bool all_read = true;
-      for (int q = s_lo; q <= s_hi; ++q) all_read = all_read && is_read[(size_t)q];
       if (leaf) {
-        // z_k = W_ih x_k + b + W_hh h_{k-1} for the n leaves at once (their h_{k-1} are all
-        // memorised), then h_k; the gates are redone inside the backward kernel
-        const __nv_bfloat16* xk = reinterpret_cast<const __nv_bfloat16*>(io.x) + (size_t)(k_lo - 1) * B * I;
-        gemm(xk, I, false, wp_ih, I, false,
-             GemmOut{GemmOut::STORE_F32, zleaf + (size_t)s_lo * B * G, G, bias_p, 0}, n * B, G, I);
-        // the recurrent part in the two parts the forward kernels sum it in, in their order
-        const int k_first = KB0 < KBh ? 64 * KB0 : H;
-        gemm(hprev_c + (size_t)s_lo * B * H, H, false, wp_hh, H, false,
-             GemmOut{GemmOut::ACCUM_F32, zleaf + (size_t)s_lo * B * G, G, nullptr, 0}, n * B, G, k_first);
-        if (k_first < H)
-          gemm(hprev_c + (size_t)s_lo * B * H + k_first, H, false, wp_hh + k_first, H, false,
-               GemmOut{GemmOut::ACCUM_F32, zleaf + (size_t)s_lo * B * G, G, nullptr, 0}, n * B, G, H - k_first);
-        if (!all_read) {
-          ++launches;
-          if (!dry && rc == MEBPTT_OK)
-            launch_pdl(leaf_forward, dim3(32, n), dim3(256), 0, s, bops, n, ws, zleaf, hk_c, S, B, H, io.counters);
-          for (int q = s_lo; q <= s_hi; ++q) has_h[(size_t)q + 1] = 1;
-        }
+        // z_k = W_ih x_k + b + W_hh h_{k-1} and h_k of the n leaves at once (their h_{k-1} are all memorised); the gates are
+        // redone inside the backward kernel
+        ++launches;
+        if (!dry && rc == MEBPTT_OK)
+          rc = leaf_products(LeafArgs{bops, n, ws, bias_p, zleaf + (size_t)s_lo * B * G, has_h[(size_t)s_hi + 1] ? nullptr : hk_c + (size_t)s_hi * B * H,
+                                      io.counters, status, B, I, H},
+                             reinterpret_cast<const __nv_bfloat16*>(io.x) + (size_t)(k_lo - 1) * B * I, wp_ih, hprev_c + (size_t)s_lo * B * H, wp_hh, s);
+        has_h[(size_t)s_hi + 1] = 1;
       }
       // Readout of the run's steps as far as it is not done, together with all steps before them whose h is there already
       // (as a rule all of the chunk that the last sweep passed): loss terms and dy, then the gradient entering h_k.  A run
@@ -1614,14 +1574,14 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
       if (!dry && rc == MEBPTT_OK) {
         const uint32_t polls = (fault & 2) ? fault_poll_limit : kSpinLimit;
         const ClusterBwdArgs a{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, status, io.counters, B, H, S, off16(y.plane),
-                               leaf ? zleaf : nullptr, parts, leaf && all_read ? n : 0, (fault & 2) ? 16u : 0u, polls};
+                               leaf ? zleaf : nullptr, parts, (fault & 2) ? 16u : 0u, polls};
         const int span = span_begin(timer, 1, n, s);
         cudaError_t e;
         if (clusters) {
           e = cluster_backward(P.tm_wt_cl, a, P.run_rows, s);
         } else if (P.short_runs && n < SHORT_BWD) {
           BwdRunArgs sa{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status,
-                        io.counters, B, H, S, off16(y.plane), leaf ? zleaf : nullptr, parts, leaf && all_read ? n : 0, P.bwd_tb,
+                        io.counters, B, H, S, off16(y.plane), leaf ? zleaf : nullptr, parts, P.bwd_tb,
                         (uint32_t)P.fwd_ncg + ((fault & 2) ? 1u : 0u), (fault & 2) ? fault_poll_limit : (kSpinLimit >> 1)};
           void* args[] = {(void*)&P.tm_dz[pb], (void*)&P.tm_wt, (void*)&sa};
           // (in plain stream order: early residency of a clustered cooperative grid measured no gain)

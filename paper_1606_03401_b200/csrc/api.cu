@@ -701,7 +701,7 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
       if (y.x3_runs) {
         // packing; a window of projections: split and GEMM; forward run: one; backward run: readout of two
         // and dha, run, d_in; a batch of leaves: split, GEMM, states, two GEMMs, cells before that; chunks as below
-        int64_t n = 5 + (desc->want_dx ? 1 : 0) + chunks * 11 + 1;
+        int64_t n = 5 + (desc->want_dx ? 1 : 0) + chunks * 5 + 1;
         const std::shared_ptr<const Cut> cut = cut_for(y, p);
         const std::vector<WorkItem>& items = cut->items;
         const std::vector<int>& windows = cut->windows;
@@ -723,7 +723,7 @@ int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc* desc, const mebptt_plan
         else if (wi.kind == WorkItem::BWD) readouts += 3 + dha;
         else forwards += wi.n == 1 ? 3 * L : L * (1 + 2 * (int64_t)wi.n);
       }
-      return 2 * L + 2 + forwards + readouts + p->t * bwd + chunks * (3 * (2 * L + 1) + L + 1) + 1;
+      return 2 * L + 2 + forwards + readouts + p->t * bwd + chunks * (3 * L + 2) + 1;
     }
     // (a GRU layer's backward operation takes two launches more: its weight gradient comes in three blocks)
     return p->cost * L + p->t * (5 + (y.gru ? 6 : 4) * L) + 1;

@@ -15,8 +15,8 @@
 //   readout    h3 = split(h) ; y = h3 Wout3^T + b_out with loss and the halves of dy in the epilogue ;
 //              dha = dy3 WoutMN3
 //   backward   dz3 from the stored gates ; d_in = dz3 WMN3
-//   per chunk  dW += dz^T [in ; h_prev], dW_out += dy^T h from the staged halves: three GEMMs per
-//              product (hi hi, hi mid, mid hi); db += sum of dz, db_out += sum of dy, as hi + mid
+//   per chunk  dW += dz^T [in ; h_prev], dW_out += dy^T h from the staged halves: one GEMM per
+//              product (mid hi + hi mid + hi hi); db += sum of dz, db_out += sum of dy, as hi + mid
 // All sums run in a fixed order and nothing depends on the plan: results are bit-identical across
 // plans.
 #include "kernels.hpp"
@@ -446,21 +446,14 @@ int backward_layer(const generic::BwdArgs& a, const Scratch& w, int l, size_t w_
 }
 
 namespace {
-// C[m][n] += sum_r (a_hi a_mid)[r][m] (b_hi b_mid)[r][n] as hi hi + hi mid + mid hi; a3 rows are
+// C[m][n] += sum_r (a_hi a_mid)[r][m] (b_hi b_mid)[r][n] as mid hi + hi mid + hi hi; a3 rows are
 // [hi | hi | mid] of width Ma, b2 rows [hi | mid] of width Nb.
 int accum3(const bf16* a3, int Ma, const bf16* b2, int Nb, bool b_is_a3, float* C, int64_t ldc, int R, int* status,
            cudaStream_t s) {
   const int64_t lda = 3 * (int64_t)Ma, ldb = (b_is_a3 ? 3 : 2) * (int64_t)Nb;
-  const bf16* a_hi = a3;
-  const bf16* a_mid = a3 + 2 * (size_t)Ma;
-  const bf16* b_hi = b2;
-  const bf16* b_mid = b2 + (b_is_a3 ? 2 : 1) * (size_t)Nb;
-  const GemmOut o{GemmOut::ACCUM_F32, C, ldc, nullptr, 0};
-  int rc = gemm_bf16(a_hi, lda, true, b_hi, ldb, true, o, Ma, Nb, R, status, s);
-  if (rc != MEBPTT_OK) return rc;
-  rc = gemm_bf16(a_hi, lda, true, b_mid, ldb, true, o, Ma, Nb, R, status, s);
-  if (rc != MEBPTT_OK) return rc;
-  return gemm_bf16(a_mid, lda, true, b_hi, ldb, true, o, Ma, Nb, R, status, s);
+  const tc::GemmHalves halves{2 * Ma, (b_is_a3 ? 2 : 1) * Nb};
+  return gemm_bf16(a3, lda, true, b2, ldb, true, GemmOut{GemmOut::ACCUM_F32, C, ldc, nullptr, 0}, Ma, Nb, R, status, s,
+                   true, nullptr, 0, nullptr, &halves);
 }
 }  // namespace
 

@@ -29,6 +29,12 @@ struct GemmOut {
   float scale = 0.f;
 };
 
+// Operands in bfloat16 halves, hi and mid side by side in each row: the columns from hi to mid of A and of B.
+// The product is then A_mid B_hi + A_hi B_mid + A_hi B_hi, in one accumulator and in that order.
+struct GemmHalves {
+  int a = 0, b = 0;
+};
+
 // Caller buffers of one training step (device pointers).
 struct StepPtrs {
   const char *W, *W_out, *x, *h0;
@@ -98,9 +104,10 @@ int gemm_split_count_deferred(int M, int N, int K);
 // next kernel and *defer says where they are (C is then not touched, not even when accumulating:
 // the consumer adds the parts to it); if it is not, *defer says so (splits = 0).  With defer and
 // force_splits > 1 the tiles are 128 wide whatever the shape.
+// halves (optional): only with a_mn, b_mn and an accumulating output.
 int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb, bool b_mn, const GemmOut& out,
               int M, int N, int K, int* status, cudaStream_t s, bool early = true, const SplitWs* split = nullptr,
-              int force_splits = 0, SplitParts* defer = nullptr);
+              int force_splits = 0, SplitParts* defer = nullptr, const GemmHalves* halves = nullptr);
 
 }  // namespace tc
 

@@ -37,17 +37,23 @@ constexpr int BN_WIDE = 128, BN_NARROW = 32;   // tile widths; narrow tiles spre
 constexpr int A_BYTES = BM * BK * 2;
 constexpr int gemm_smem(int stages, int bn) { return stages * (A_BYTES + bn * BK * 2) + 1024; }  // + slack to align the ring to 1024 B
 
-// HALVES: an instance whose loss epilogue writes dy in halves.  (Its registers and instructions in the other
+// HALVES with K-major operands: an instance whose loss epilogue writes dy in halves.  (Its registers and instructions in the other
 // instances' epilogue cost bf16 training steps 0.4 %; an instance of its own for the bf16 loss, too, costs 1 %:
 // its loads of the targets are then fewer in flight.)
 // Four CTAs an SM would be more than shared memory holds: the bound lets the compiler keep up to 128 registers,
 // so that more of an epilogue's loads are in flight, and the instances with an MN-major operand (the gradients)
 // have no loss epilogue (H = 1024, full memory with dx: 12.30 -> 12.22 ms; MSM m = 100: 18.13 -> 18.03 ms).
+// HALVES with MN-major operands: both lie in halves, and the contraction is walked three times, mid hi, hi mid,
+// hi hi, each a shift of the columns that the copies start at.  What bounds a weight gradient of few rows is not
+// the products but a launch's filling of its ring and its pass over C, of which there were three
+// (H = 1024, t = 4000, ISM m = 50: 122.9 -> 119.6 ms).  The small products come first, so that the
+// accumulator holds no more than before while hi hi is added up.
 template <bool A_MN, bool B_MN, int BN = BN_WIDE, bool HALVES = false>
 __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant__ CUtensorMap tma,
                                                         const __grid_constant__ CUtensorMap tmb, GemmOut out,
                                                         int M, int N, int K, int STAGES, int* status,
-                                                        float* partial, int fault) {
+                                                        float* partial, int fault, GemmHalves halves) {
+  constexpr bool SEGMENTS = HALVES && A_MN && B_MN;
   constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
   static_assert(BN == BN_WIDE || (!A_MN && !B_MN), "narrow tiles exist for K-major operands only");
   extern __shared__ uint8_t smem_raw[];
@@ -60,7 +66,7 @@ __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   // this CTA's part of the contraction index: blocks [kb_lo, kb_lo + nk) of 64
   const int splits = gridDim.z;
-  const int nk_all = (K + BK - 1) / BK;
+  const int nk_one = (K + BK - 1) / BK, nk_all = SEGMENTS ? 3 * nk_one : nk_one;
   const int kb_lo = (int)((int64_t)nk_all * blockIdx.z / splits);
   const int nk = (int)((int64_t)nk_all * (blockIdx.z + 1) / splits) - kb_lo;
   const int tile = blockIdx.y * gridDim.x + blockIdx.x;
@@ -93,6 +99,15 @@ __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant
       // issuer's bounded wait runs out and the kernel leaves through its failure path)
       mbar_arrive_expect_tx(&full[s], STAGE_BYTES + ((fault && kb == 0) ? 16u : 0u));
       ++armed;
+      if constexpr (SEGMENTS) {
+        const int seg = kb / nk_one, k0 = (kb - seg * nk_one) * BK;
+        const int ma = m0 + (seg == 0 ? halves.a : 0), nb = n0 + (seg == 1 ? halves.b : 0);
+        tma_load_2d(sA, &tma, ma, k0, &full[s]);
+        tma_load_2d(sA + 8192, &tma, ma + 64, k0, &full[s]);
+        tma_load_2d(sB, &tmb, nb, k0, &full[s]);
+        tma_load_2d(sB + 8192, &tmb, nb + 64, k0, &full[s]);
+        continue;
+      }
       if (A_MN) {
         tma_load_2d(sA, &tma, m0, (kb_lo + kb) * BK, &full[s]);
         tma_load_2d(sA + 8192, &tma, m0 + 64, (kb_lo + kb) * BK, &full[s]);
@@ -407,8 +422,10 @@ int gemm_split_count_deferred(int M, int N, int K) {
 
 int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb, bool b_mn, const GemmOut& out,
               int M, int N, int K, int* status, cudaStream_t s, bool early, const SplitWs* split, int force_splits,
-              SplitParts* defer) {
+              SplitParts* defer, const GemmHalves* halves) {
   if (M <= 0 || N <= 0 || K <= 0) return MEBPTT_ERR_ARG;
+  if (halves && !(a_mn && b_mn && out.kind == GemmOut::ACCUM_F32 && !split && halves->a % 8 == 0 && halves->b % 8 == 0))
+    return MEBPTT_ERR_ARG;
   const bool loss = out.kind == GemmOut::LOSS_DY;
   if (loss && (a_mn || b_mn || !(out.dy3 || out.ptr))) return MEBPTT_ERR_ARG;
   // A short-and-wide product over K-major operands (a few steps' worth of rows against a whole
@@ -419,9 +436,11 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
   const int BN = narrow ? BN_NARROW : BN_WIDE;
   CUtensorMap ta, tb;
   // K-major: tensor is [M][K], box 64 (k) x tile rows.  MN-major: tensor is [K][M], box 64 (m) x 64 rows.
-  bool ok = a_mn ? make_tmap_2d(&ta, A, 2, (uint64_t)M, (uint64_t)K, (uint64_t)lda * 2, 64, 64)
+  // In halves the map spans the whole row; what a tile at the edge takes from the neighbouring half goes only into
+  // rows and columns that are not written.
+  bool ok = a_mn ? make_tmap_2d(&ta, A, 2, (uint64_t)(halves ? M + halves->a : M), (uint64_t)K, (uint64_t)lda * 2, 64, 64)
                  : make_tmap_2d(&ta, A, 2, (uint64_t)K, (uint64_t)M, (uint64_t)lda * 2, 64, 128);
-  ok = ok && (b_mn ? make_tmap_2d(&tb, B, 2, (uint64_t)N, (uint64_t)K, (uint64_t)ldb * 2, 64, 64)
+  ok = ok && (b_mn ? make_tmap_2d(&tb, B, 2, (uint64_t)(halves ? N + halves->b : N), (uint64_t)K, (uint64_t)ldb * 2, 64, 64)
                    : make_tmap_2d(&tb, B, 2, (uint64_t)K, (uint64_t)N, (uint64_t)ldb * 2, 64, (uint32_t)BN));
   if (!ok) return MEBPTT_ERR_UNSUPPORTED;
   dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
@@ -436,6 +455,7 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
   static const bool attrs = [] {
     const int most = gemm_smem(MAX_STAGES, BN_WIDE);
     cudaFuncSetAttribute(gemm_bf16_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(gemm_bf16_kernel<true, true, BN_WIDE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     cudaFuncSetAttribute(gemm_bf16_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     cudaFuncSetAttribute(gemm_bf16_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     cudaFuncSetAttribute(gemm_bf16_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
@@ -451,12 +471,14 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
   // loop.  Grids of at most one wave: 6 stages, more loads in flight per CTA to hide their latency.
   const int stages = (grid.x * grid.y * grid.z <= 148) ? MAX_STAGES : 3;
   const int GEMM_SMEM = gemm_smem(stages, BN);
-  auto* fn = loss && out.dy3 ? (narrow ? gemm_bf16_kernel<false, false, BN_NARROW, true> : gemm_bf16_kernel<false, false, BN_WIDE, true>)
+  auto* fn = halves ? gemm_bf16_kernel<true, true, BN_WIDE, true>
+             : loss && out.dy3 ? (narrow ? gemm_bf16_kernel<false, false, BN_NARROW, true> : gemm_bf16_kernel<false, false, BN_WIDE, true>)
              : narrow ? gemm_bf16_kernel<false, false, BN_NARROW>
              : a_mn ? (b_mn ? gemm_bf16_kernel<true, true> : gemm_bf16_kernel<true, false>)
                     : (b_mn ? gemm_bf16_kernel<false, true> : gemm_bf16_kernel<false, false>);
   const cudaError_t e = launch_on(early, fn, grid, dim3(128), (size_t)GEMM_SMEM, s, ta, tb, out, M, N, K, stages, status,
-                                  splits > 1 ? split->partial : nullptr, (wait_fault_mask() & 4) ? 1 : 0);
+                                  splits > 1 ? split->partial : nullptr, (wait_fault_mask() & 4) ? 1 : 0,
+                                  halves ? *halves : GemmHalves{});
   if (e != cudaSuccess) {
     cudaGetLastError();
     return MEBPTT_ERR_CUDA;

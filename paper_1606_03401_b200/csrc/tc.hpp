@@ -122,8 +122,8 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
                  bool side_stream);
 
 
-// Testing aid: which bounded waits are made to run out on purpose (0: none).  Bit 0: the step
-// counter of the forward run kernel is told to expect one CTA too many; bit 1: likewise for the
+// Testing aid: which bounded waits are made to run out on purpose (0: none).  Bit 0: a step of the forward run
+// kernels waits for more than comes (one CTA, 16 pushed bytes, a piece of a ring that nobody writes); bit 1: likewise for the
 // backward run kernels; bit 2: the first stage of a GEMM expects 16 bytes more than its copies
 // bring; bit 3: a phase of a pod expects 16 bytes more than are pushed; bit 4: the meeting of a
 // team expects one arrival too many.  The waits then give up after `fault_poll_limit` polls instead of the usual limit, the

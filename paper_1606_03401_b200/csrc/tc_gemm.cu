@@ -11,14 +11,15 @@
 // is stored [k][m] (rows are contraction indices), which is how dz and the layer inputs lie in
 // memory for the weight gradient, so no transposed copies are made.
 //
-// One CTA computes one 128 x 128 tile (128 x 32 where C is short and wide: see gemm_bf16).  A single thread feeds a 3- or 6-stage ring of 128-byte
-// swizzled shared-memory tiles by TMA (64 contraction indices per stage); a single thread issues
+// One CTA computes one 128 x 128 tile (128 x 32 where C is short and wide: see gemm_bf16).  A single thread feeds a ring of
+// 128-byte swizzled shared-memory tiles by TMA (64 contraction indices per tile, one or three tiles per stage); a single thread issues
 // tcgen05.mma (M = 128, N = 128, K = 16, four per stage) into a 128-column TMEM accumulator and
 // releases ring slots with tcgen05.commit; then all four warps read the accumulator with
 // tcgen05.ld (warp w owns TMEM lanes 32w .. 32w+31 = tile rows) and write the tile.
 // Out-of-range parts of a tile are zero-filled by TMA on the way in and masked on the way out.
 // The sum over k runs in one fixed order, so results do not depend on how callers batch steps.
 #include <cstdlib>
+#include <type_traits>
 
 #include "launch.hpp"
 #include "sm100.cuh"
@@ -33,28 +34,38 @@ namespace {
 using namespace sm100;
 
 constexpr int BM = 128, BK = 64, MAX_STAGES = 6;
+constexpr int DEEP_TILES = 3;                  // tiles of a stage of the deep rings
 constexpr int BN_WIDE = 128, BN_NARROW = 32;   // tile widths; narrow tiles spread a short-and-wide C over more SMs
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int gemm_smem(int stages, int bn) { return stages * (A_BYTES + bn * BK * 2) + 1024; }  // + slack to align the ring to 1024 B
+constexpr int gemm_smem(int stages, int bn, int tps) { return stages * tps * (A_BYTES + bn * BK * 2) + 1024; }  // + slack to align the ring to 1024 B
 
-// HALVES with K-major operands: an instance whose loss epilogue writes dy in halves.  (Its registers and instructions in the other
-// instances' epilogue cost bf16 training steps 0.4 %; an instance of its own for the bf16 loss, too, costs 1 %:
+// HALVES with K-major operands: an instance whose loss epilogue writes dy in halves.  (Its registers and instructions in the
+// other instances' epilogue cost bf16 training steps 0.4 %; an instance of its own for the bf16 loss, too, costs 1 %:
 // its loads of the targets are then fewer in flight.)
 // Four CTAs an SM would be more than shared memory holds: the bound lets the compiler keep up to 128 registers,
 // so that more of an epilogue's loads are in flight, and the instances with an MN-major operand (the gradients)
 // have no loss epilogue (H = 1024, full memory with dx: 12.30 -> 12.22 ms; MSM m = 100: 18.13 -> 18.03 ms).
 // HALVES with MN-major operands: both lie in halves, and the contraction is walked three times, mid hi, hi mid,
 // hi hi, each a shift of the columns that the copies start at.  What bounds a weight gradient of few rows is not
-// the products but a launch's filling of its ring and its pass over C, of which there were three
-// (H = 1024, t = 4000, ISM m = 50: 122.9 -> 119.6 ms).  The small products come first, so that the
-// accumulator holds no more than before while hi hi is added up.
-template <bool A_MN, bool B_MN, int BN = BN_WIDE, bool HALVES = false>
+// the products but a launch's filling of its ring and its pass over C, of which there were three (H = 1024, t = 4000,
+// ISM m = 50: 122.9 -> 119.6 ms).  The small products come first, so that the accumulator holds no more than before
+// while hi hi is added up.
+// TPS: tiles of 64 contraction indices per stage.  A grid of at most one wave has an SM for each tile of C, and one tile a
+// stage then passes at 60 to 100 GB/s an SM, however many stages there are: what takes the time is a stage's way
+// through its two barriers and the requests of its copies.  Three tiles a stage, requested together, come near what an
+// SM takes in (120 GB/s); us, one, two and three tiles a stage in 192 KB (narrow tiles of C: 120): 288 x 256, K = 3072
+// 16.7, 12.0, 10.1; 128 x 8192, K = 2048 14.7, 12.1, 11.2; 4096 x 256, MN-major, K = 2048 17.4, 13.4, 12.5.  (Two
+// threads that request: no change.)  More tiles of C than SMs: one a stage, so that two CTAs share an SM and one's epilogue overlaps the other's products (2048 x 4096, K = 256: 13.4
+// against 20.7; 8192 x 8192, K = 4096: 489 against 629).
+// `blocks`: bit 0 (1): the map of A (B) sees 64 columns as a block of its own (make_tmap_blocks64), and one copy brings
+// all tiles of a stage; without it, where the columns are no whole number of blocks, one copy each.
+template <bool A_MN, bool B_MN, int BN = BN_WIDE, bool HALVES = false, int TPS = 1>
 __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant__ CUtensorMap tma,
                                                         const __grid_constant__ CUtensorMap tmb, GemmOut out,
                                                         int M, int N, int K, int STAGES, int* status,
-                                                        float* partial, int fault, GemmHalves halves) {
+                                                        float* partial, int fault, int blocks, GemmHalves halves) {
   constexpr bool SEGMENTS = HALVES && A_MN && B_MN;
-  constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
+  constexpr int B_BYTES = BN * BK * 2, STAGE_BYTES = TPS * (A_BYTES + B_BYTES);
   static_assert(BN == BN_WIDE || (!A_MN && !B_MN), "narrow tiles exist for K-major operands only");
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES], done;
@@ -64,11 +75,12 @@ __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  // this CTA's part of the contraction index: blocks [kb_lo, kb_lo + nk) of 64
+  // this CTA's part of the contraction index: blocks [kb_lo, kb_lo + nk) of 64 (in halves: all of them, three times)
   const int splits = gridDim.z;
-  const int nk_one = (K + BK - 1) / BK, nk_all = SEGMENTS ? 3 * nk_one : nk_one;
+  const int nk_all = (K + BK - 1) / BK;
   const int kb_lo = (int)((int64_t)nk_all * blockIdx.z / splits);
   const int nk = (int)((int64_t)nk_all * (blockIdx.z + 1) / splits) - kb_lo;
+  const int n_one = (nk + TPS - 1) / TPS, n_st = SEGMENTS ? 3 * n_one : n_one;   // stages: of one walk, in all
   const int tile = blockIdx.y * gridDim.x + blockIdx.x;
 
   if (threadIdx.x == 0) {
@@ -90,35 +102,33 @@ __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant
   if (warp == 0 && lane == 0) {
     // ---- producer -----------------------------------------------------------------------
     int armed = 0;  // stages whose full barrier still awaits bytes (for the failure path)
-    for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES;
-      if (kb >= STAGES && !mbar_wait(&empty[s], ((kb / STAGES) - 1) & 1)) { failed = 1; break; }
+    for (int st = 0; st < n_st; ++st) {
+      const int s = st % STAGES;
+      if (st >= STAGES && !mbar_wait(&empty[s], ((st / STAGES) - 1) & 1)) { failed = 1; break; }
       uint8_t* sA = ring + s * STAGE_BYTES;
-      uint8_t* sB = sA + A_BYTES;
+      uint8_t* sB = sA + TPS * A_BYTES;
       // (fault: a testing aid -- the first stage is told to expect 16 bytes that never come, so the
       // issuer's bounded wait runs out and the kernel leaves through its failure path)
-      mbar_arrive_expect_tx(&full[s], STAGE_BYTES + ((fault && kb == 0) ? 16u : 0u));
+      mbar_arrive_expect_tx(&full[s], STAGE_BYTES + ((fault && st == 0) ? 16u : 0u));
       ++armed;
-      if constexpr (SEGMENTS) {
-        const int seg = kb / nk_one, k0 = (kb - seg * nk_one) * BK;
-        const int ma = m0 + (seg == 0 ? halves.a : 0), nb = n0 + (seg == 1 ? halves.b : 0);
-        tma_load_2d(sA, &tma, ma, k0, &full[s]);
-        tma_load_2d(sA + 8192, &tma, ma + 64, k0, &full[s]);
-        tma_load_2d(sB, &tmb, nb, k0, &full[s]);
-        tma_load_2d(sB + 8192, &tmb, nb + 64, k0, &full[s]);
-        continue;
-      }
+      const int seg = SEGMENTS ? st / n_one : 2;
+      const int k0 = kb_lo + (st - (SEGMENTS ? seg * n_one : 0)) * TPS;       // first tile of the stage
+      const int ma = m0 + (seg == 0 ? halves.a : 0), nb = n0 + (seg == 1 ? halves.b : 0);
       if (A_MN) {
-        tma_load_2d(sA, &tma, m0, (kb_lo + kb) * BK, &full[s]);
-        tma_load_2d(sA + 8192, &tma, m0 + 64, (kb_lo + kb) * BK, &full[s]);
+        if (blocks & 1) tma_load_3d(sA, &tma, 0, k0 * BK, ma / 64, &full[s]);
+        else for (int q = 0; q < 2; ++q) tma_load_2d(sA + q * TPS * 8192, &tma, ma + 64 * q, k0 * BK, &full[s]);
+      } else if (blocks & 1) {
+        tma_load_3d(sA, &tma, 0, m0, k0, &full[s]);
       } else {
-        tma_load_2d(sA, &tma, (kb_lo + kb) * BK, m0, &full[s]);
+        for (int t = 0; t < TPS; ++t) tma_load_2d(sA + t * A_BYTES, &tma, (k0 + t) * BK, m0, &full[s]);
       }
       if (B_MN) {
-        tma_load_2d(sB, &tmb, n0, (kb_lo + kb) * BK, &full[s]);
-        tma_load_2d(sB + 8192, &tmb, n0 + 64, (kb_lo + kb) * BK, &full[s]);
+        if (blocks & 2) tma_load_3d(sB, &tmb, 0, k0 * BK, nb / 64, &full[s]);
+        else for (int q = 0; q < 2; ++q) tma_load_2d(sB + q * TPS * 8192, &tmb, nb + 64 * q, k0 * BK, &full[s]);
+      } else if (blocks & 2) {
+        tma_load_3d(sB, &tmb, 0, n0, k0, &full[s]);
       } else {
-        tma_load_2d(sB, &tmb, (kb_lo + kb) * BK, n0, &full[s]);
+        for (int t = 0; t < TPS; ++t) tma_load_2d(sB + t * B_BYTES, &tmb, (k0 + t) * BK, n0, &full[s]);
       }
     }
     (void)armed;
@@ -128,19 +138,27 @@ __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant
     constexpr uint32_t idesc = make_idesc(1, BM, BN, A_MN, B_MN);
     // K-major: 16 contraction indices = 32 B along the row; MN-major: 16 rows of 128 B
     constexpr uint32_t A_STEP = A_MN ? (2048 >> 4) : (32 >> 4), B_STEP = B_MN ? (2048 >> 4) : (32 >> 4);
+    // tiles of a stage: K-major side by side, MN-major 64 rows apart
+    constexpr uint32_t A_TILE = (A_MN ? 8192 : A_BYTES) >> 4, B_TILE = (B_MN ? 8192 : B_BYTES) >> 4;
     const uint32_t ring0 = smem_u32(ring);
-    const uint64_t a_desc0 = A_MN ? make_desc_sw128(ring0, 8192, 1024) : make_desc_sw128(ring0, 16, 1024);
-    const uint64_t b_desc0 = B_MN ? make_desc_sw128(ring0 + A_BYTES, 8192, 1024) : make_desc_sw128(ring0 + A_BYTES, 16, 1024);
+    const uint64_t a_desc0 = A_MN ? make_desc_sw128(ring0, TPS * 8192, 1024) : make_desc_sw128(ring0, 16, 1024);
+    const uint64_t b_desc0 = B_MN ? make_desc_sw128(ring0 + TPS * A_BYTES, TPS * 8192, 1024) : make_desc_sw128(ring0 + TPS * A_BYTES, 16, 1024);
     bool ok = true;
-    for (int kb = 0; kb < nk && ok; ++kb) {
-      const int s = kb % STAGES;
-      if (!mbar_wait(&full[s], (kb / STAGES) & 1)) { failed = 1; ok = false; break; }
+    for (int st = 0; st < n_st && ok; ++st) {
+      const int s = st % STAGES;
+      if (!mbar_wait(&full[s], (st / STAGES) & 1)) { failed = 1; ok = false; break; }
       tc_fence_after_sync();
+      const int live = nk - (SEGMENTS ? st % n_one : st) * TPS;     // tiles from this stage's first on (the last stage may have fewer than TPS)
       if (elect_one()) {
         const uint64_t da = a_desc0 + (uint64_t)(s * (STAGE_BYTES >> 4)), db = b_desc0 + (uint64_t)(s * (STAGE_BYTES >> 4));
 #pragma unroll
-        for (int k4 = 0; k4 < BK / 16; ++k4)
-          mma_f16(tmem, da + (uint64_t)(k4 * A_STEP), db + (uint64_t)(k4 * B_STEP), idesc, (kb > 0 || k4 > 0) ? 1u : 0u);
+        for (int t = 0; t < TPS; ++t) {
+          if (TPS > 1 && t >= live) break;
+#pragma unroll
+          for (int k4 = 0; k4 < BK / 16; ++k4)
+            mma_f16(tmem, da + (uint64_t)(t * A_TILE + k4 * A_STEP), db + (uint64_t)(t * B_TILE + k4 * B_STEP), idesc,
+                    (st > 0 || t > 0 || k4 > 0) ? 1u : 0u);
+        }
         mma_commit(&empty[s]);  // the slot may be refilled once these MMAs have read it
       }
       __syncwarp();
@@ -434,15 +452,6 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
   const int wide_tiles = ((N + BN_WIDE - 1) / BN_WIDE) * ((M + BM - 1) / BM);
   const bool narrow = !a_mn && !b_mn && wide_tiles <= 37 && N >= 2 * BN_NARROW && !(defer && force_splits > 1);
   const int BN = narrow ? BN_NARROW : BN_WIDE;
-  CUtensorMap ta, tb;
-  // K-major: tensor is [M][K], box 64 (k) x tile rows.  MN-major: tensor is [K][M], box 64 (m) x 64 rows.
-  // In halves the map spans the whole row; what a tile at the edge takes from the neighbouring half goes only into
-  // rows and columns that are not written.
-  bool ok = a_mn ? make_tmap_2d(&ta, A, 2, (uint64_t)(halves ? M + halves->a : M), (uint64_t)K, (uint64_t)lda * 2, 64, 64)
-                 : make_tmap_2d(&ta, A, 2, (uint64_t)K, (uint64_t)M, (uint64_t)lda * 2, 64, 128);
-  ok = ok && (b_mn ? make_tmap_2d(&tb, B, 2, (uint64_t)(halves ? N + halves->b : N), (uint64_t)K, (uint64_t)ldb * 2, 64, 64)
-                   : make_tmap_2d(&tb, B, 2, (uint64_t)K, (uint64_t)N, (uint64_t)ldb * 2, 64, (uint32_t)BN));
-  if (!ok) return MEBPTT_ERR_UNSUPPORTED;
   dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM);
   int splits = 1;
   if (split && split->partial && (out.kind == GemmOut::STORE_F32 || (defer && out.kind == GemmOut::ACCUM_F32)) &&
@@ -452,32 +461,60 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
     return MEBPTT_ERR_ARG;
   if (splits > 1 && (size_t)grid.x * grid.y * splits * BM * BN > split->partial_floats) return MEBPTT_ERR_WORKSPACE;
   grid.z = splits;
+  // Grids of at most one wave: two stages of three tiles (a contraction that is longer than both) or six of one, one CTA
+  // an SM.  Larger ones: three stages of one tile, two CTAs per SM, so that one's epilogue overlaps the other's main loop.
+  const bool one_wave = grid.x * grid.y * grid.z <= 148;
+  const int nk = (halves ? 3 : 1) * (((K + BK - 1) / BK + splits - 1) / splits);
+  const int tps = one_wave && nk > MAX_STAGES ? DEEP_TILES : 1;
+  const int stages = tps > 1 ? MAX_STAGES / DEEP_TILES : one_wave ? MAX_STAGES : 3;
+  CUtensorMap ta, tb;
+  int blocks = 0;
+  // K-major: tensor is [M][K], box 64 (k) x tile rows, `tps` of them.  MN-major: tensor is [K][M], box 64 (m) x 64 tps rows, two of
+  // them.  In halves the map spans the whole row; what a tile at the edge takes from the neighbouring half goes only
+  // into rows and columns that are not written.
+  auto encode = [&](CUtensorMap* t, const void* p, bool mn, int rows, int off, int64_t ld, int tile, int bit) {
+    const uint64_t cols = mn ? (uint64_t)(rows + off) : (uint64_t)K, n = mn ? (uint64_t)K : (uint64_t)rows;
+    const uint32_t high = (uint32_t)(mn ? BK * tps : tile);
+    if ((mn || tps > 1) && cols % 64 == 0 && off % 64 == 0) {
+      blocks |= bit;
+      return make_tmap_blocks64(t, p, cols, n, (uint64_t)ld * 2, high, mn ? 2u : (uint32_t)tps);
+    }
+    return make_tmap_2d(t, p, 2, cols, n, (uint64_t)ld * 2, 64, high);
+  };
+  if (!encode(&ta, A, a_mn, M, halves ? halves->a : 0, lda, BM, 1) || !encode(&tb, B, b_mn, N, halves ? halves->b : 0, ldb, BN, 2))
+    return MEBPTT_ERR_UNSUPPORTED;
+  const int smem = gemm_smem(stages, BN, tps);
+  const bool loss3 = loss && out.dy3;
+  auto pick = [&](auto t) {
+    constexpr int T = decltype(t)::value;
+    return halves ? gemm_bf16_kernel<true, true, BN_WIDE, true, T>
+           : loss3 ? (narrow ? gemm_bf16_kernel<false, false, BN_NARROW, true, T> : gemm_bf16_kernel<false, false, BN_WIDE, true, T>)
+           : narrow ? gemm_bf16_kernel<false, false, BN_NARROW, false, T>
+           : a_mn ? (b_mn ? gemm_bf16_kernel<true, true, BN_WIDE, false, T> : gemm_bf16_kernel<true, false, BN_WIDE, false, T>)
+                  : (b_mn ? gemm_bf16_kernel<false, true, BN_WIDE, false, T> : gemm_bf16_kernel<false, false, BN_WIDE, false, T>);
+  };
+  auto* fn = tps > 1 ? pick(std::integral_constant<int, DEEP_TILES>()) : pick(std::integral_constant<int, 1>());
   static const bool attrs = [] {
-    const int most = gemm_smem(MAX_STAGES, BN_WIDE);
-    cudaFuncSetAttribute(gemm_bf16_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(gemm_bf16_kernel<true, true, BN_WIDE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(gemm_bf16_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(gemm_bf16_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(gemm_bf16_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_NARROW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         gemm_smem(MAX_STAGES, BN_NARROW));
-    cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_WIDE, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_NARROW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         gemm_smem(MAX_STAGES, BN_NARROW));
+    auto set = [](auto t) {
+      constexpr int T = decltype(t)::value;
+      const int wide = gemm_smem(MAX_STAGES, BN_WIDE, 1), narrow = gemm_smem(MAX_STAGES, BN_NARROW, 1);
+      const cudaFuncAttribute most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+      cudaFuncSetAttribute(gemm_bf16_kernel<true, true, BN_WIDE, false, T>, most, wide);
+      cudaFuncSetAttribute(gemm_bf16_kernel<true, true, BN_WIDE, true, T>, most, wide);
+      cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_WIDE, false, T>, most, wide);
+      cudaFuncSetAttribute(gemm_bf16_kernel<true, false, BN_WIDE, false, T>, most, wide);
+      cudaFuncSetAttribute(gemm_bf16_kernel<false, true, BN_WIDE, false, T>, most, wide);
+      cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_NARROW, false, T>, most, narrow);
+      cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_WIDE, true, T>, most, wide);
+      cudaFuncSetAttribute(gemm_bf16_kernel<false, false, BN_NARROW, true, T>, most, narrow);
+    };
+    set(std::integral_constant<int, 1>());
+    set(std::integral_constant<int, DEEP_TILES>());
     return true;
   }();
   (void)attrs;
-  // Large grids: 3 stages, two CTAs per SM, so that one CTA's epilogue overlaps the other's main
-  // loop.  Grids of at most one wave: 6 stages, more loads in flight per CTA to hide their latency.
-  const int stages = (grid.x * grid.y * grid.z <= 148) ? MAX_STAGES : 3;
-  const int GEMM_SMEM = gemm_smem(stages, BN);
-  auto* fn = halves ? gemm_bf16_kernel<true, true, BN_WIDE, true>
-             : loss && out.dy3 ? (narrow ? gemm_bf16_kernel<false, false, BN_NARROW, true> : gemm_bf16_kernel<false, false, BN_WIDE, true>)
-             : narrow ? gemm_bf16_kernel<false, false, BN_NARROW>
-             : a_mn ? (b_mn ? gemm_bf16_kernel<true, true> : gemm_bf16_kernel<true, false>)
-                    : (b_mn ? gemm_bf16_kernel<false, true> : gemm_bf16_kernel<false, false>);
-  const cudaError_t e = launch_on(early, fn, grid, dim3(128), (size_t)GEMM_SMEM, s, ta, tb, out, M, N, K, stages, status,
-                                  splits > 1 ? split->partial : nullptr, (wait_fault_mask() & 4) ? 1 : 0,
+  const cudaError_t e = launch_on(early, fn, grid, dim3(128), (size_t)smem, s, ta, tb, out, M, N, K, stages, status,
+                                  splits > 1 ? split->partial : nullptr, (wait_fault_mask() & 4) ? 1 : 0, blocks,
                                   halves ? *halves : GemmHalves{});
   if (e != cudaSuccess) {
     cudaGetLastError();

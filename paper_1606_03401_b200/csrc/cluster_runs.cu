@@ -1,12 +1,12 @@
 // Runs of the bfloat16 recurrence for at most 512 hidden units: a thread-block cluster holds all of W_hh and
-// walks a run for 16 batch rows; what a step produces travels between shared memories, never through the L2.
+// walks a run for 8 or 12 batch rows; what a step produces travels between shared memories, never through the L2.
 //
 // What bounds a step is the trip of the new state to everyone who needs it.  Through global memory (the
 // kernels of tc_lstm.cu, which wider layers need) that trip is a store, a release that waits for it, a counter, a
 // poll and a fetch: 2.8 us an operation at H = 256 and 3.2 at H = 512, of which the products are a fifth.
-// Here the batch rows of an LSTM, which never mix, are cut into groups of 16, and each group is one cluster of
-// ceil(H / 32) CTAs, a CTA with 32 hidden units: its 128 gate rows are a full MMA tile, 16 rows the N.  (Groups of
-// 32 would halve the SMs at work and double what a thread does in an epilogue; 8 is below the N an M of 128 allows.)
+// Here the batch rows of an LSTM, which never mix, are cut into groups of 8 or 12 (cluster_rows), and each group is one
+// cluster of ceil(H / 32) CTAs, a CTA with 32 hidden units: its 128 gate rows are a full MMA tile, the N is 16, the least
+// that an M of 128 allows.
 //
 //   forward    z[128 gate rows][16] = W_hh[rows of this CTA][H] h_{k-1}, both operands in shared memory; the gates;
 //              h_k goes to every CTA of the cluster, straight into the swizzled tile its next MMA reads, by
@@ -292,20 +292,14 @@ __global__ void __launch_bounds__(THREADS, 1) fwd_run_cluster(const __grid_const
 // ------------------------------------------------------------------------------------------
 constexpr int BWD_THREADS = 224;   // warps 0-3: gates; 4: MMAs; 5: what is read and dz, in and out; 6: loss terms
 
-// Shared memory behind the alignment: weights, dz, partial sums received, two stages of inputs.  With 16 rows all of it is
-// too much, and the stages lie over the weights, which are in tensor memory by then.
+// Shared memory behind the alignment: weights, dz, partial sums received, two stages of inputs.
 template <int RB>
 struct BwdSmem {
-  static constexpr bool over = RB == 16;
   static __host__ __device__ uint32_t weights(int H) { return (uint32_t)((H + 127) / 128 * 2) * W_TILE; }
   static __host__ __device__ uint32_t dz(int H) { return weights(H); }                     // [2][2] tiles [16 batch rows][64 gate columns]
   static __host__ __device__ uint32_t recv(int H) { return dz(H) + 4 * H_TILE; }           // [2][CTAs] partial sums
-  static __host__ __device__ uint32_t stages(int H) { return over ? 0 : recv(H) + 2 * (uint32_t)((H + CU - 1) / CU) * recv_slot(RB); }
-  static __host__ __device__ uint32_t total(int H) {
-    const uint32_t end = recv(H) + 2 * (uint32_t)((H + CU - 1) / CU) * recv_slot(RB);
-    const uint32_t in = 2 * (uint32_t)sizeof(GateStage<RB>);
-    return 1024 + (over ? (end > in ? end : in) : end + in);
-  }
+  static __host__ __device__ uint32_t stages(int H) { return recv(H) + 2 * (uint32_t)((H + CU - 1) / CU) * recv_slot(RB); }
+  static __host__ __device__ uint32_t total(int H) { return 1024 + stages(H) + 2 * (uint32_t)sizeof(GateStage<RB>); }
 };
 
 template <int RB>
@@ -388,7 +382,6 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_run_cluster(const __grid_c
       asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&inready[i & 1])) : "memory");
     };
     DevOp next = a.ops[0];
-    if (Smem::over) named_barrier(2, 160);    // the weights have left the room of the stages
     for (int i = 0; i < 2 && i < a.n; ++i) {
       const DevOp op = next;
       if (i + 1 < a.n) next = a.ops[i + 1];
@@ -475,7 +468,6 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_run_cluster(const __grid_c
     };
 
     weights_to_tmem(sW, 2 * MT, wfull, tmem, warp, lane, &failed);
-    if (Smem::over) asm volatile("bar.arrive 2, 160;" ::: "memory");
     GateIn<NV> in;
     (void)wait_or_fail(&inready[0], 0, &failed);
     pick_out<NV, RB>(leaf, sI[0], u, rp, in);
@@ -548,10 +540,10 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_run_cluster(const __grid_c
 
 int cluster_ctas(int H) { return (H + CU - 1) / CU; }
 int fwd_smem(int H) { return (H + 63) / 64 * (int)(W_TILE + 2 * 8 * PIECE) + 1024; }
-int bwd_smem(int H, int RB) { return (int)(RB == 8 ? BwdSmem<8>::total(H) : RB == 12 ? BwdSmem<12>::total(H) : BwdSmem<16>::total(H)); }
+int bwd_smem(int H, int RB) { return (int)(RB == 8 ? BwdSmem<8>::total(H) : BwdSmem<12>::total(H)); }
 const void* kernel(int dir, int RB) {
-  if (dir) return RB == 8 ? (const void*)bwd_run_cluster<8> : RB == 12 ? (const void*)bwd_run_cluster<12> : (const void*)bwd_run_cluster<16>;
-  return RB == 8 ? (const void*)fwd_run_cluster<8> : RB == 12 ? (const void*)fwd_run_cluster<12> : (const void*)fwd_run_cluster<16>;
+  if (dir) return RB == 8 ? (const void*)bwd_run_cluster<8> : (const void*)bwd_run_cluster<12>;
+  return RB == 8 ? (const void*)fwd_run_cluster<8> : (const void*)fwd_run_cluster<12>;
 }
 
 cudaError_t launch_cluster(const void* fn, int threads, int groups, int cs, int smem, void** args, cudaStream_t s) {
@@ -576,7 +568,7 @@ bool cluster_maps(CUtensorMap* tm_w, CUtensorMap* tm_wt, const void* wp_hh, cons
 int cluster_rows(int B, int H) {
   const int cs = cluster_ctas(H);
   int fit = 1 << 30;
-  for (int RB : {8, 12, 16})
+  for (int RB : {8, 12})
     for (int dir = 0; dir < 2; ++dir) {
       const void* fn = kernel(dir, RB);
       cudaLaunchConfig_t cfg = {};
@@ -598,8 +590,8 @@ int cluster_rows(int B, int H) {
   // Fewer rows make a step shorter (all that is sent and most of what a thread does is in proportion to them), as long
   // as the clusters need not take turns.  Forward and backward operation, B = 64, 8, 12 and 16 rows, in us: H = 256 0.78,
   // 1.02, 1.22 and 0.90, 1.21, 1.29; H = 512, where seven clusters fit, 2.1 (in turns), 1.32, 1.57 and 2.5, 1.73, 1.91.
-  if ((B + 7) / 8 <= fit) return 8;
-  return (B + 11) / 12 <= fit ? 12 : 16;
+  // (So 16 rows are never taken: 64 are six clusters of 12.)
+  return (B + 7) / 8 <= fit ? 8 : 12;
 }
 
 cudaError_t cluster_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, int rows, cudaStream_t s) {

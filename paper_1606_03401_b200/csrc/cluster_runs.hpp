@@ -12,7 +12,7 @@ namespace tc {
 struct DevOp;
 
 constexpr int CU = 32;   // hidden units per CTA
-constexpr int CB = 16;   // batch rows of a cluster at most: the least N of an MMA with M = 128
+constexpr int CB = 16;   // rows of a tile of states: the least N of an MMA with M = 128
 
 // A cluster holds all hidden units of a layer: 32 a CTA, 16 CTAs at most.
 inline bool cluster_runs_supported(int H) { return H % 8 == 0 && H >= 64 && H <= 16 * CU; }
@@ -51,7 +51,7 @@ struct ClusterBwdArgs {
 
 // Tensor maps of the two kernels: W_hh with permuted gate rows and its transpose (boxes of 64 columns, 128 rows).
 bool cluster_maps(CUtensorMap* tm_w, CUtensorMap* tm_wt, const void* wp_hh, const void* wpT_hh, int H);
-// Batch rows a cluster takes (8, 12 or 16), so that all clusters are on the device at once where that can be; 0 where
+// Batch rows a cluster takes (8 or 12), so that all clusters are on the device at once where that can be; 0 where
 // the device cannot run clusters of this size.  Sets the kernels' attributes as well.
 int cluster_rows(int B, int H);
 cudaError_t cluster_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, int rows, cudaStream_t s);

@@ -156,24 +156,6 @@ def kernel_breakdown(dp, plans):
             print(f"| {k} | {n} | {v:.1f} | {v / n:.2f} | {100 * v / tot:.1f}% |", file=sys.stderr)
 
 
-def profiled_traffic(kernel_source: str, summary: str):
-    """DRAM bytes per forward operation from the committed ncu summary of the dominant kernel, or
-    None if the kernel's source has changed since the counters were taken (the summary records the
-    hash of the source file it was taken from)."""
-    import hashlib
-    import re
-    try:
-        text = open(os.path.join(ROOT, summary)).read()
-        sha = hashlib.sha256(open(os.path.join(ROOT, kernel_source), "rb").read()).hexdigest()[:16]
-    except OSError:
-        return None
-    m_sha = re.search(r"kernel source sha256\[:16\]:\s*([0-9a-f]{16})", text)
-    m_b = re.search(r"DRAM bytes per forward operation:\s*([0-9.eE+]+)", text)
-    if not m_sha or not m_b or m_sha.group(1) != sha:
-        return None
-    return float(m_b.group(1))
-
-
 def max_over_ranks(v: float, world: int, device) -> float:
     """Slowest rank's time: the job is done when the last replica is."""
     if world == 1:
@@ -353,22 +335,21 @@ def main():
         f_ms, f_n, f_ops = runs["forward"]
         b_ms, b_n, b_ops = runs["backward"]
         flops_rec = 2 * cfg.batch * cfg.hidden * 4 * cfg.hidden      # the recurrent contraction of one operation
-        per_op_traffic = (profiled_traffic("paper_1606_03401_b200/csrc/tc_lstm.cu",
-                                           "profiles/ncu_full_fwd_run_kernel_c3_shapes_t64.md")
-                          if (cfg.name == "c3" and cfg.input == 1024) else None)
+        # (widths the library serves in a cluster, through a ring in the L2; the ring's short runs by grid-wide kernels)
+        kind = ("fwd_run_cluster", "bwd_run_cluster") if cfg.hidden <= 512 else (
+            "fwd_run_ring (runs of fewer than 5: fwd_run_kernel)", "bwd_run_ring (runs of fewer than 3: bwd_run_group_kernel)")
         achieved = f_ops * flops_rec / (f_ms * 1e-3) / 1e12
         roofline = {"bound": "tensor", "achieved": achieved, "peak": peak_tf, "unit": "TFLOP/s",
                     "frac": achieved / peak_tf,
-                    "traffic": (per_op_traffic * (f_ops / f_n)) if per_op_traffic else None,
-                    "kernel": "fwd_run_kernel (a run of forward operations: recurrent gate contraction + cell update)",
+                    "traffic": None,
+                    "kernel": f"{kind[0]}: a run of forward operations, recurrent gate contraction + cell update",
                     "launches": f_n // 3, "ops_per_launch": f_ops / f_n, "us_per_launch": f_ms * 1e3 / f_n,
                     "us_per_op": f_ms * 1e3 / f_ops,
                     "share_of_step": (f_ms / 3) / ms,
-                    "backward_runs": {"kernel": "bwd_run_group_kernel (bwd_run_cluster_kernel where B <= 32)", "launches": b_n // 3,
+                    "backward_runs": {"kernel": kind[1], "launches": b_n // 3,
                                       "us_per_op": b_ms * 1e3 / max(1, b_ops), "share_of_step": (b_ms / 3) / ms},
-                    "traffic_note": ("DRAM bytes per launch = bytes per operation (ncu capture of a 32-operation launch, "
-                                     "config 3's layer sizes) x mean operations per launch; null when the kernel's "
-                                     "source has changed since the capture"),
+                    "traffic_note": "not measured: the backward kernel of this path, a cooperative launch of clusters, does not "
+                                    "start under ncu",
                     "how": f"CUDA events around each launch, 3 steps; {flops_rec} flops per operation x operations per launch / mean "
                            f"launch duration; peak = bf16 sustained ({pk['source']})"}
     else:

@@ -89,7 +89,8 @@ constexpr int LOSS_PARTS = 64;   // partial sums per step of the loss
 // bit pattern until h_k is written with strong stores, polled with strong 16-byte loads into
 // registers and staged into the swizzled tiles by the epilogue warps, the step counter kept off
 // the critical path for the reuse of slots only -- which removes the 1.5 us signalling round but
-// loses as much to the staging and to waiting for the slowest producer (5.3).
+// loses as much to the staging and to waiting for the slowest producer (5.3; with half as many CTAs to a
+// group, their weights in tensor memory, it takes 2.8: ring_runs.cu).
 //
 // Warps 0-3: epilogue; warp 4: TMA producer; warp 5: MMA issuer.  All of h_{k-1} a CTA needs is
 // resident in shared memory for the step (H <= 1024), so the producer never waits for a free slot.

@@ -502,6 +502,13 @@ enum {
 int mebptt_test_route(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan, int64_t *out);
 
 /*
+ * Testing aid: dynamic shared memory, in bytes, of a CTA of the kernels whose CTAs wait for one another while they
+ * hold tensor memory, for `rows` batch rows a cluster or group (MEBPTT_ROUTE_PERSISTENT; shorter: of its runs of few
+ * operations; MEBPTT_ROUTE_RUNS_F32).  -1 for another route.
+ */
+int64_t mebptt_test_run_smem(int route, int shorter, int backward, int hidden, int rows);
+
+/*
  * Testing aid: the schedule that a whole tape is walked by (MEBPTT_ROUTE_PODS, MEBPTT_ROUTE_TEAMS), as the
  * records its kernel reads, for a replay on the host.  room > 0: with so many records a launch instead of what
  * the workspace has room for.  Fills info[0..19] (pods, steps per chunk, room, and where states and operands

@@ -92,6 +92,7 @@ _SIGS = {
     "mebptt_test_wait_fault": (_i32, [_i32]),
     "mebptt_test_schedule": (_i64, [_descp, _vp, _i64, C.POINTER(_i64), _vp, _i64, C.POINTER(_i64), _i64]),
     "mebptt_test_route": (_i32, [_descp, _vp, C.POINTER(_i64)]),
+    "mebptt_test_run_smem": (_i64, [_i32, _i32, _i32, _i32, _i32]),
     "mebptt_slot_copy": (_i32, [_vp, _vp, _sz, _vp]),
     "mebptt_gemm_bf16": (_i32, [_vp, _i64, _i32, _vp, _i64, _i32, _vp, _i64, _i32, _vp, _i64, _i64, _i64, _vp, _vp]),
     "mebptt_strerror": (C.c_char_p, [_i32]),
@@ -327,6 +328,10 @@ def mebptt_test_route(desc, plan) -> dict:
     out = (_i64 * 4)()
     _check(lib.mebptt_test_route(C.byref(desc), plan.handle, out), "mebptt_test_route")
     return {"route": ROUTES[out[0]], "chunk": out[1], "ctas": out[2], "rows": out[3]}
+
+
+def mebptt_test_run_smem(route: str, hidden: int, rows: int, backward: bool, shorter: bool = False) -> int:
+    return lib.mebptt_test_run_smem(ROUTES.index(route), int(shorter), int(backward), hidden, rows)
 
 
 SCHEDULE_INFO = ("pods", "chunk", "room", "unit_blocks", "loc_blocks", "n_blocks", "core0", "core1", "ping", "pong", "init",

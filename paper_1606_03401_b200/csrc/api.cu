@@ -906,6 +906,15 @@ int mebptt_test_route(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, i
   return MEBPTT_OK;
 }
 
+int64_t mebptt_test_run_smem(int route, int shorter, int backward, int hidden, int rows) {
+  if (hidden < 8 || hidden > 1024 || hidden % 8 || (backward != 0 && backward != 1)) return -1;
+  const bool bwd = backward != 0;
+  if (route == MEBPTT_ROUTE_RUNS_F32) return stepwise3::runs_smem(bwd, hidden);
+  if (route != MEBPTT_ROUTE_PERSISTENT) return -1;
+  if (shorter) return tc::short_runs_smem(bwd, hidden);
+  return tc::cluster_runs_supported(hidden) ? tc::cluster_smem(bwd, hidden, rows) : tc::ring_smem(bwd, hidden, rows);
+}
+
 int64_t mebptt_test_schedule(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, int64_t room, int64_t* info, void* records,
                              int64_t most_records, int64_t* launches, int64_t most_launches) {
   if (!info || check_common(desc, plan) != MEBPTT_OK) return -1;

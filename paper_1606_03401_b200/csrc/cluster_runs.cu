@@ -539,8 +539,8 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_run_cluster(const __grid_c
 }
 
 int cluster_ctas(int H) { return (H + CU - 1) / CU; }
-int fwd_smem(int H) { return (H + 63) / 64 * (int)(W_TILE + 2 * 8 * PIECE) + 1024; }
-int bwd_smem(int H, int RB) { return (int)(RB == 8 ? BwdSmem<8>::total(H) : BwdSmem<12>::total(H)); }
+int fwd_smem(int H) { return lone_smem((H + 63) / 64 * (int)(W_TILE + 2 * 8 * PIECE) + 1024); }
+int bwd_smem(int H, int RB) { return lone_smem((int)(RB == 8 ? BwdSmem<8>::total(H) : BwdSmem<12>::total(H))); }
 const void* kernel(int dir, int RB) {
   if (dir) return RB == 8 ? (const void*)bwd_run_cluster<8> : (const void*)bwd_run_cluster<12>;
   return RB == 8 ? (const void*)fwd_run_cluster<8> : (const void*)fwd_run_cluster<12>;
@@ -593,6 +593,8 @@ int cluster_rows(int B, int H) {
   // (So 16 rows are never taken: 64 are six clusters of 12.)
   return (B + 7) / 8 <= fit ? 8 : 12;
 }
+
+int cluster_smem(bool backward, int H, int rows) { return backward ? bwd_smem(H, rows) : fwd_smem(H); }
 
 cudaError_t cluster_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, int rows, cudaStream_t s) {
   void* args[] = {(void*)&tm_w, (void*)&a};

@@ -54,6 +54,7 @@ bool cluster_maps(CUtensorMap* tm_w, CUtensorMap* tm_wt, const void* wp_hh, cons
 // Batch rows a cluster takes (8 or 12), so that all clusters are on the device at once where that can be; 0 where
 // the device cannot run clusters of this size.  Sets the kernels' attributes as well.
 int cluster_rows(int B, int H);
+int cluster_smem(bool backward, int H, int rows);   // dynamic shared memory of a CTA
 cudaError_t cluster_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, int rows, cudaStream_t s);
 cudaError_t cluster_backward(const CUtensorMap& tm_wt, const ClusterBwdArgs& a, int rows, cudaStream_t s);
 

@@ -203,6 +203,7 @@ struct RunsX3 {
 };
 // Packs the weights W ([4H][I + H]) and clears what a step must find clear; false if a tensor map was refused.
 bool runs_begin(RunsX3& r, int I, int H, int B, const float* W, cudaStream_t s);
+int runs_smem(bool backward, int H);   // dynamic shared memory of a CTA
 // n <= 32 consecutive forward operations; zx: [n][B][4H], x W_ih + b of their steps.
 int forward_run(RunsX3& r, const stepwise::FwdRunStep* st, int n, const float* zx, size_t plane_elems, int64_t* counters,
                 int* status, cudaStream_t s);

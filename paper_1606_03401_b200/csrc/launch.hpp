@@ -15,6 +15,16 @@ namespace mebptt {
 
 inline bool pdl_enabled() { return !env::no_pdl(); }
 
+// Dynamic shared memory of a kernel whose CTAs wait for one another while they hold tensor memory: more than half of an
+// SM's 228 KB (a CTA takes 1 KB beside what it asks for), so that no SM ever has two such CTAs, of one kernel or of
+// steps on different streams.  tcgen05.alloc blocks until its columns are free, and the scheduler, which places CTAs by
+// shared memory, registers and threads, knows nothing of them: a CTA of kernel A could hold an SM where one of kernel B
+// waits for columns, and one of B another where A waits, each kernel waiting for its own CTA for good.  CTAs that hold
+// tensor memory and wait for nobody (the contractions) end by themselves, whatever they share an SM with.
+// What it costs is that such CTAs no longer share SMs: with one layer up to 320 units wide, two steps on two streams.
+constexpr int LONE_SMEM = 228 * 1024 / 2 - 1024 + 16;
+inline int lone_smem(int bytes) { return bytes > LONE_SMEM ? bytes : LONE_SMEM; }
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_on(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                              Args&&... args) {

@@ -692,8 +692,8 @@ int threads(bool bwd, int RB) {
 }
 int smem_bytes(bool bwd, int RB, int H) {
   const int KT = bwd ? 2 * ring_ctas(H) / RING_CLUSTER : (H + 63) / 64;
-  if (bwd) return (int)(RB == 8 ? BwdShape<8>::total(KT) : BwdShape<16>::total(KT));
-  return (int)(RB == 8 ? FwdShape<8>::total(KT) : FwdShape<16>::total(KT));
+  if (bwd) return lone_smem((int)(RB == 8 ? BwdShape<8>::total(KT) : BwdShape<16>::total(KT)));
+  return lone_smem((int)(RB == 8 ? FwdShape<8>::total(KT) : FwdShape<16>::total(KT)));
 }
 int fwd_ctas(int H) { return (H + CU - 1) / CU; }
 
@@ -732,6 +732,8 @@ int ring_rows(int B, int H) {
   }
   return 0;
 }
+
+int ring_smem(bool backward, int H, int rows) { return smem_bytes(backward, rows, H); }
 
 cudaError_t ring_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, const RingArgs& r, int rows, cudaStream_t s) {
   int ncta = fwd_ctas(a.H), KT0 = fwd_first_part_blocks(a.H);

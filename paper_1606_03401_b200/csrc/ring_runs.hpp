@@ -31,6 +31,7 @@ RingArgs ring_args(char* rings, int H, int B, bool backward, int id, bool fault,
 // Tensor maps: boxes of 64 columns by 128 rows, as for the cluster kernels.
 // Batch rows of a group (8 or 16); 0 where the device cannot keep the kernels' CTAs resident.
 int ring_rows(int B, int H);
+int ring_smem(bool backward, int H, int rows);   // dynamic shared memory of a CTA
 cudaError_t ring_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, const RingArgs& r, int rows, cudaStream_t s);
 cudaError_t ring_backward(const CUtensorMap& tm_wt, const ClusterBwdArgs& a, const RingArgs& r, int rows, cudaStream_t s);
 

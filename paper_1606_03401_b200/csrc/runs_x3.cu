@@ -52,8 +52,8 @@ constexpr int SYNC_STRIDE = 32;          // words between the step counters of t
 constexpr int TMEM_COLS = 64;
 
 inline __host__ __device__ int whole_boxes(int KB) { return (KB + 3) / 4 * 4; }   // weights come in boxes of four tiles
-inline int fwd_smem(int KB) { return (whole_boxes(KB) + RING * SLAB) * (int)TILE + 2 * RB * PART_LD * 4 + 1024; }
-inline int bwd_smem(int KB) { return (whole_boxes(KB) + RING * SLAB) * (int)TILE + 2 * CS * 2 * RU * RECV_LD * 4 + 1024; }
+inline int fwd_smem(int KB) { return lone_smem((whole_boxes(KB) + RING * SLAB) * (int)TILE + 2 * RB * PART_LD * 4 + 1024); }
+inline int bwd_smem(int KB) { return lone_smem((whole_boxes(KB) + RING * SLAB) * (int)TILE + 2 * CS * 2 * RU * RECV_LD * 4 + 1024); }
 
 __device__ __forceinline__ float sigmoidf_(float a) { return 1.0f / (1.0f + expf(-a)); }
 __device__ __forceinline__ void split2(float v, bf16& hi, bf16& mid) {
@@ -555,6 +555,8 @@ bool runs_begin(RunsX3& r, int I, int H, int B, const float* W, cudaStream_t s) 
          make_tmap_blocks64(&r.tm_dz, r.exch_b, HP, (uint64_t)2 * r.groups * CS * 64, (uint64_t)HP * 2, 64, SLAB) &&
          make_tmap_blocks64(&r.tm_wt, r.w_b, HP, (uint64_t)ncl * CS * 64, (uint64_t)HP * 2, 64, 4);
 }
+
+int runs_smem(bool backward, int H) { return backward ? bwd_smem(round64(H) / 64) : fwd_smem(round64(H) / 64); }
 
 int forward_run(RunsX3& r, const stepwise::FwdRunStep* st, int n, const float* zx, size_t plane_elems, int64_t* counters,
                 int* status, cudaStream_t s) {

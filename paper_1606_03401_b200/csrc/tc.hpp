@@ -128,6 +128,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
 // bring; bit 3: a phase of a pod expects 16 bytes more than are pushed; bit 4: the meeting of a
 // team expects one arrival too many.  The waits then give up after `fault_poll_limit` polls instead of the usual limit, the
 // kernels leave through their ordinary exit path, and the status word receives MEBPTT_ERR_TIMEOUT.
+int short_runs_smem(bool backward, int H);   // dynamic shared memory of a CTA of the kernels for short runs of wide layers
 int wait_fault_mask();
 void set_wait_fault_mask(int mask);
 constexpr uint32_t fault_poll_limit = 1u << 14;

@@ -1197,6 +1197,16 @@ void build_host_part(Prepared& P, const Layout& y, const Plan* p, bool allow_pin
   }
 }
 
+// Dynamic shared memory of the kernels of this file.
+int short_fwd_smem(int H) {
+  const int KB = (H + 63) / 64, KB0 = fwd_first_part_blocks(H);
+  return lone_smem((KB * FG + 2 * KB0 * FB) * 128 + 2 * FB * PART_LD * 4 + 1024);
+}
+int short_bwd_smem(int H) {
+  const int kbs = (4 * H / 64) / GCS, tb = kbs > 8 ? 8 : 4;
+  return lone_smem(kbs * (FU * GCS * 128) + (kbs + tb - 1) / tb * tb * FB * 128 + 2 * GCS * FU * RECV_LD * 4 + 1024);
+}
+
 // Kernel variants and tensor maps for the workspace at `ws` on the current device.
 void build_device_part(Prepared& P, const Layout& y, char* ws) {
   const int B = y.B, H = y.H, S = y.S, G = 4 * H;
@@ -1211,11 +1221,11 @@ void build_device_part(Prepared& P, const Layout& y, char* ws) {
   if (P.run_rows <= 0) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
   if (cluster_runs_supported(H) || B <= FB || B > 2 * FB || H % 128 != 0) return;
   // Short runs (below).  Widths in whole blocks of 128: both kinds of kernels then add the same parts in the same order.
-  const int KBh = (H + 63) / 64, KB0 = fwd_first_part_blocks(H), kbs = (G / 64) / GCS;
+  const int KB0 = fwd_first_part_blocks(H), kbs = (G / 64) / GCS;
   P.fwd_ncg = H / FU;
-  P.fwd_smem = (KBh * FG + 2 * KB0 * FB) * 128 + 2 * FB * PART_LD * 4 + 1024;
+  P.fwd_smem = short_fwd_smem(H);
   P.bwd_tb = kbs > 8 ? 8 : 4;
-  P.bwd_smem = kbs * (FU * GCS * 128) + (kbs + P.bwd_tb - 1) / P.bwd_tb * P.bwd_tb * FB * 128 + 2 * GCS * FU * RECV_LD * 4 + 1024;
+  P.bwd_smem = short_bwd_smem(H);
   const void* fn = (const void*)bwd_run_group_kernel;
   bool ok = cudaFuncSetAttribute(fwd_run_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) == cudaSuccess &&
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) == cudaSuccess;
@@ -1282,6 +1292,8 @@ std::atomic<int> g_wait_fault{0};
 }
 int wait_fault_mask() { return g_wait_fault.load(); }
 void set_wait_fault_mask(int mask) { g_wait_fault.store(mask); }
+
+int short_runs_smem(bool backward, int H) { return backward ? short_bwd_smem(H) : short_fwd_smem(H); }
 
 void forget_plan(uint64_t plan_id) {
   std::lock_guard<std::mutex> lock(g_prep_mu);

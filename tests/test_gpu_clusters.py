@@ -69,3 +69,24 @@ def test_short_and_long_runs_of_wide_layers_give_the_same_bits():
             res = dp.run(plan)
             assert res["counters"][0] == plan.cost and res["counters"][3] == 0
             assert_bit_identical(res, full, want_dx=True)
+
+
+@pytest.mark.parametrize("sizes", [(520, 256), (512, 64), (256, 1024)])
+def test_steps_of_two_widths_on_two_streams_do_not_wait_for_one_another(sizes):
+    """Kernels that hold tensor memory while their CTAs wait for one another, of two steps at a time."""
+    import torch
+    problems = [_problem(input=40, hidden=h, batch=64, readout=24, t=90)[1] for h in sizes]
+    plans = [dp.full_memory_plan() for dp in problems]
+    alone = [dp.run(p) for dp, p in zip(problems, plans)]
+    streams = [torch.cuda.Stream() for _ in problems]
+    torch.cuda.synchronize()
+    for turn in range(6):
+        for i in (0, 1) if turn % 2 else (1, 0):
+            with torch.cuda.stream(streams[i]):
+                problems[i].enqueue(plans[i])
+    torch.cuda.synchronize()
+    for dp, want in zip(problems, alone):
+        res = {k: v.cpu().numpy() for k, v in dp.out.items()}
+        res["loss"] = float(res["loss"][0])
+        assert res["counters"][3] == 0
+        assert_bit_identical(res, want, want_dx=True)

@@ -509,6 +509,12 @@ int mebptt_test_route(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan, i
 int64_t mebptt_test_run_smem(int route, int shorter, int backward, int hidden, int rows);
 
 /*
+ * Testing aid: hidden units, those past the last one included, whose values a step of a run of one bfloat16 layer waits
+ * for.  -1 where nobody waits for units (backward runs inside a cluster wait for every CTA's partial sums).
+ */
+int mebptt_test_run_units(int backward, int hidden);
+
+/*
  * Testing aid: the schedule that a whole tape is walked by (MEBPTT_ROUTE_PODS, MEBPTT_ROUTE_TEAMS), as the
  * records its kernel reads, for a replay on the host.  room > 0: with so many records a launch instead of what
  * the workspace has room for.  Fills info[0..19] (pods, steps per chunk, room, and where states and operands

@@ -915,6 +915,11 @@ int64_t mebptt_test_run_smem(int route, int shorter, int backward, int hidden, i
   return tc::cluster_runs_supported(hidden) ? tc::cluster_smem(bwd, hidden, rows) : tc::ring_smem(bwd, hidden, rows);
 }
 
+int mebptt_test_run_units(int backward, int hidden) {
+  if (hidden < 64 || hidden > 1024 || hidden % 8 || (backward && tc::cluster_runs_supported(hidden))) return -1;
+  return backward ? tc::bwd_waited_units(hidden) : tc::fwd_waited_units(hidden);
+}
+
 int64_t mebptt_test_schedule(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, int64_t room, int64_t* info, void* records,
                              int64_t most_records, int64_t* launches, int64_t most_launches) {
   if (!info || check_common(desc, plan) != MEBPTT_OK) return -1;

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(THREADS, 1) fwd_run_cluster(const __grid_const
     mbar_fence_init();
     tma_prefetch_desc(&tm_w);
   }
-  // units past H and rows past RB are never pushed
+  // pieces past the CTAs' units and rows past RB are never pushed
   for (uint32_t e = tid; e < 2 * h_buf / 16; e += THREADS) reinterpret_cast<uint4*>(sH)[e] = make_uint4(0, 0, 0, 0);
   fence_proxy_async_shared();
   const uint32_t acc_col = 32 * (uint32_t)KT;   // the accumulators, behind the weights
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(THREADS, 1) fwd_run_cluster(const __grid_const
 
   if (warp == 4) {
     constexpr uint32_t idesc = make_idesc(1, 128, CB, false, false);
-    const uint32_t bytes = (uint32_t)(RB * a.H * 2) + a.extra;
+    const uint32_t bytes = (uint32_t)(RB * fwd_waited_units(a.H) * 2) + a.extra;
     if (lane == 0) {
       for (int kb = 0; kb < KT; ++kb) {
         mbar_arrive_expect_tx(&wfull[kb], W_TILE);
@@ -229,8 +229,9 @@ __global__ void __launch_bounds__(THREADS, 1) fwd_run_cluster(const __grid_const
         gate[v][0] = iv; gate[v][1] = fv; gate[v][2] = gv; gate[v][3] = ov;
       }
       __syncwarp();
-      const uint4 hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);
-      if (got && wvalid && prow < RB && i + 1 < a.n) {
+      uint4 hnew = make_uint4(0, 0, 0, 0);                   // (past the last unit)
+      if (wvalid) hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);
+      if (got && prow < RB && i + 1 < a.n) {
         // h_k to every CTA, the next in rank first
         const uint32_t dst = piece + (((uint32_t)i + 1) & 1) * h_buf, bar = (i & 1) ? bar0 : bar1;
         for (uint32_t p = lane / ROWS; p < cs; p += PEERS) {

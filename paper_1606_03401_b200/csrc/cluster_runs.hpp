@@ -17,6 +17,11 @@ constexpr int CB = 16;   // rows of a tile of states: the least N of an MMA with
 // A cluster holds all hidden units of a layer: 32 a CTA, 16 CTAs at most.
 inline bool cluster_runs_supported(int H) { return H % 8 == 0 && H >= 64 && H <= 16 * CU; }
 
+// Units whose h a step of a forward run waits for, those past the last unit included (zeros): every warp of the gates sends
+// its eight, so that nobody is a step behind what the MMAs have begun.  (A barrier can be waited for by its parity only
+// while the phase after that is not over; a warp that sent nothing would be kept in step by timing alone.)
+__host__ __device__ inline int fwd_waited_units(int H) { return (H + CU - 1) / CU * CU; }
+
 struct ClusterFwdArgs {
   const DevOp* ops;      // this launch's operations (consecutive forward operations)
   int n;

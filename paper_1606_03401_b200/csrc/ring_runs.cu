@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
     constexpr int ROWS = RB, PER = 32 / ROWS;                       // pieces of 8 units a warp has in hand at a time
     constexpr int N = 64 / (PER * POLLERS / 2);                     // 64 pieces a part at most
     const int pw = warp - GATES - 1, q = pw / (POLLERS / 2), wl = pw % (POLLERS / 2);
-    const int row = lane % ROWS, p0 = (q ? 8 * KT0 : 0) + wl * PER + lane / ROWS, p_end = q ? a.H / 8 : (8 * KT0 < a.H / 8 ? 8 * KT0 : a.H / 8);
+    const int row = lane % ROWS, p0 = (q ? 8 * KT0 : 0) + wl * PER + lane / ROWS, p_end = q ? fwd_waited_units(a.H) / 8 : 8 * KT0;
     constexpr int STEP = PER * POLLERS / 2;
     uint32_t want = 0;
 #pragma unroll
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
 #pragma unroll
       for (int x = 0; x < N; ++x) {
         v[x] = make_uint4(0, 0, 0, 0);
-        if ((want >> x & 1) && brow + row < a.B) v[x] = *reinterpret_cast<const uint4*>(h0 + ((size_t)(brow + row) * a.H + 8 * (p0 + x * STEP)) * 2);
+        if ((want >> x & 1) && brow + row < a.B && p0 + x * STEP < a.H / 8) v[x] = *reinterpret_cast<const uint4*>(h0 + ((size_t)(brow + row) * a.H + 8 * (p0 + x * STEP)) * 2);
       }
 #pragma unroll
       for (int x = 0; x < N; ++x)
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
     if (pvalid) hprev = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.ws + (size_t)op0.h_src * 16) + ep);
     // this lane's piece in a slot: [8 units][RB rows][16 bytes]
     const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)(jw / 8) * (RB * 16) + (uint32_t)(8 * half + prow) * 16;
-    if (wvalid && lane < 8)
+    if (lane < 8)
       for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
     weights_move(wt, KT, sm + Shape::stages(KT), tmem, warp, lane, Shape::G, &failed);
     __syncwarp();
@@ -354,8 +354,9 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
         gate[v][0] = iv; gate[v][1] = fv; gate[v][2] = gv; gate[v][3] = ov;
       }
       __syncwarp();
-      const uint4 hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);
-      if (got && wvalid && lane < 8) {
+      uint4 hnew = make_uint4(0, 0, 0, 0);                   // (past the last unit)
+      if (wvalid) hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);
+      if (got && lane < 8) {
         if (i + 1 < a.n) store_piece(g.ring + (size_t)((i + 1) & (RING_SLOTS - 1)) * slot_bytes + mine, hnew);
         if (i >= 1) store_piece(g.ring + (size_t)((i - 1) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
       }
@@ -442,20 +443,14 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = blockIdx.x / ncta, cta = blockIdx.x % ncta, groups = gridDim.x / ncta;
   const int rank = cta % RING_CLUSTER, cl = cta / RING_CLUSTER;
-  // pieces of two units in the CTA's quarter (there is more than a CTA of them), in each half, and warps that poll some of
-  // the second
-  const int pieces = min(16 * per, (a.H - rank * per * CU) / 2);
-  const int half0 = 8 * (KT / 2), half1 = max(0, pieces - half0);      // (the first half of them is whole)
-  const int active = min(POLLERS / 2, (half1 + 32 / RB - 1) / (32 / RB));
+  const int half0 = 8 * (KT / 2);                  // pieces of two units in a half of the CTA's quarter
   const uint32_t cta_bytes = 4 * CU * RB * 2, group_bytes = (uint32_t)ncta * cta_bytes, slot_bytes = group_bytes * groups;
 
   if (tid == 0) {
     weights_init(wt);
     mbar_init(&ready, GATES);
     for (int b = 0; b < 2; ++b) {
-      // (a warp of the pollers without pieces takes no part: it would run ahead of the others)
-      mbar_init(&zfull[b][0], (uint32_t)min(POLLERS / 2, (min(half0, pieces) + 32 / RB - 1) / (32 / RB)));
-      mbar_init(&zfull[b][1], (uint32_t)max(active, 1));
+      for (int q = 0; q < 2; ++q) mbar_init(&zfull[b][q], POLLERS / 2);
       mbar_init(&acc[b], 1);
       mbar_init(&full[b], 1);
       mbar_init(&inready[b], 32);
@@ -496,7 +491,7 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
       const int b = i & 1;
       const uint64_t z_desc = make_desc_plain(smem_u32(sZ + b * z_buf), PIECE, 128);
       for (int q = 0; q < 2; ++q) {
-        if (ok && (q == 0 || active)) ok = __all_sync(0xffffffffu, wait_or_fail(&zfull[b][q], (uint32_t)(i >> 1) & 1, &failed));
+        if (ok) ok = __all_sync(0xffffffffu, wait_or_fail(&zfull[b][q], (uint32_t)(i >> 1) & 1, &failed));
         if (!ok) break;
         tc_fence_after_sync();
         if (elect_one()) {
@@ -554,11 +549,11 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
     uint32_t want = 0;
 #pragma unroll
     for (int x = 0; x < N; ++x) {
-      if (p0 + x * STEP < (q ? pieces : min(half0, pieces))) want |= 1u << x;
+      if (p0 + x * STEP < (q + 1) * half0) want |= 1u << x;
     }
     uint8_t* const to = sZ + p0 * PIECE + row * 16;
     const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)(rank * per) * cta_bytes + (size_t)p0 * (RB * 16) + row * 16;
-    for (int i = 0; i < a.n && p0 - lane / RB < (q ? pieces : min(half0, pieces)); ++i) {
+    for (int i = 0; i < a.n; ++i) {
       if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * RB * 16, to + (i & 1) * z_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
       if (g.fault && pw == 0 && !poll_pieces<1>(g.never, 0, to, 0, 1u, &failed, g.poll_limit)) break;
       fence_proxy_async_shared();
@@ -584,13 +579,11 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
     }
     // dz leaves in pieces of two units: an even lane takes them from its neighbour for its first row, an odd one for its second
     const int odd = lane & 1, prow = r0 + odd;
-    const bool has = u < units;                     // (units is a multiple of 8)
     const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)cta * cta_bytes + (uint32_t)(u >> 1) * (RB * 16) + (uint32_t)prow * 16;
-    const bool store_ok = has && prow < rows;
+    const bool store_ok = u < units && prow < rows;   // (units is a multiple of 8)
     __nv_bfloat16* dzp = reinterpret_cast<__nv_bfloat16*>(a.dz) + 4 * ((size_t)s_hi * a.B * a.H + (size_t)(brow + prow) * a.H + unit0 + (u & ~1));
     const size_t dz_step = (size_t)4 * a.B * a.H;
-    if (has)
-      for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
+    for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
     // partial sums: lane l holds column 32 wq + l of the cluster's, which CTA wq owns
     const uint32_t to = map_rank(smem_u32(sR) + (uint32_t)rank * SLOT + (uint32_t)(2 * half) * (CU * 16) + (uint32_t)lane * 16, (uint32_t)wq);
     const uint32_t tb = map_rank(smem_u32(&full[0]), (uint32_t)wq);
@@ -635,13 +628,13 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
       const uint2 get = make_uint2(__shfl_xor_sync(0xffffffffu, send.x, 1), __shfl_xor_sync(0xffffffffu, send.y, 1));
       const uint4 piece = odd ? make_uint4(get.x, get.y, keep.x, keep.y) : make_uint4(keep.x, keep.y, get.x, get.y);
       const bool live = !*(volatile int*)&failed;
-      if (live && has) store_piece(g.ring + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes + mine, piece);
+      if (live) store_piece(g.ring + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes + mine, piece);
       __syncwarp();
       if (lane == 0) mbar_arrive(&used[i & 1]);
       // beside the exchange: dz to its stage, the piece of two steps ago cleared, the inputs of the next (earlier) step
       if (live) {
         if (store_ok) *reinterpret_cast<uint4*>(dzp) = piece;
-        if (has && i >= 2) store_piece(g.ring + (size_t)((i - 2) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
+        if (i >= 2) store_piece(g.ring + (size_t)((i - 2) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
       }
       if (i + 1 < a.n) {
         (void)wait_or_fail(&inready[(i + 1) & 1], (uint32_t)((i + 1) >> 1) & 1, &failed);

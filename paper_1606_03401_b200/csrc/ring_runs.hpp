@@ -12,6 +12,8 @@ constexpr int RING_CLUSTER = 4;  // CTAs that share the contraction index of a b
 inline bool ring_runs_supported(int H, int B) { return H % 8 == 0 && H > 16 * CU && H <= 32 * CU && B <= 64; }
 // CTAs of a group of batch rows: 32 units each, whole clusters (the last ones may have no unit)
 inline int ring_ctas(int H) { return (H + RING_CLUSTER * CU - 1) / (RING_CLUSTER * CU) * RING_CLUSTER; }
+// Units whose dz a step of a backward run waits for, likewise (fwd_waited_units).
+__host__ __device__ inline int bwd_waited_units(int H) { return (H + RING_CLUSTER * CU - 1) / (RING_CLUSTER * CU) * RING_CLUSTER * CU; }
 // bytes of both rings, two sets each: launches alternate between them
 inline size_t ring_bytes(int H, int B) {
   const size_t rows = (size_t)(B + 15) / 16 * 16, row = (size_t)ring_ctas(H) * CU * 2;

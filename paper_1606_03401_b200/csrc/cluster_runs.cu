@@ -17,7 +17,9 @@
 //
 // Two buffers of what is received: a CTA that pushes for step i + 2 has received every peer's push for step i + 1,
 // made after that peer had consumed step i.  Clusters wait for no one outside, so the launch is not cooperative.
-// All waits are bounded; a CTA that gives up stops pushing, and all meet at the barrier of the cluster at the end.
+// All waits are bounded; a CTA that gives up stops pushing, and all meet at the barrier of the cluster at the end.  (The
+// barrier that dz crosses, bar.sync 1, has no limit of its own: it ends because every warp comes to it once a step, at
+// most one step apart, whatever has run out.)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -61,6 +63,17 @@ __device__ __forceinline__ void weights_to_tmem(const uint8_t* tiles, int n, uin
   }
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   tc_fence_before_sync();
+}
+// Bounded wait for MMAs that are committed in every step, whatever has run out: not over early.  What may pass before they
+// are issued is two waits of the others (a step's inputs, then what peers push), each at most kSpinLimit polls.
+__device__ __forceinline__ bool wait_committed(uint64_t* bar, uint32_t parity, volatile int* failed) {
+  for (int turn = 0; turn < 4; ++turn)
+    for (uint32_t i = 0; i < kSpinLimit; ++i) {
+      if (mbar_try_wait(bar, parity)) return true;
+      if (i > 256 || turn) __nanosleep(64);
+    }
+  *failed = 1;
+  return false;
 }
 __host__ __device__ inline uint32_t tmem_cols(int used) { return used <= 64 ? 64u : used <= 128 ? 128u : used <= 256 ? 256u : 512u; }
 // ------------------------------------------------------------------------------------------
@@ -497,7 +510,9 @@ __global__ void __launch_bounds__(BWD_THREADS, 1) bwd_run_cluster(const __grid_c
         (void)wait_or_fail(&inready[(i + 1) & 1], (uint32_t)((i + 1) >> 1) & 1, &failed);
         pick_out<NV, RB>(leaf, sI[(i + 1) & 1], u, rp, in);
       }
-      const bool got = wait_or_fail(&acc, (uint32_t)i & 1, &failed) && !*(volatile int*)&failed;
+      // (not over because another wait ran out: barrier 1 has no limit and counts warps, not which, so no warp may come
+      // to it for a step before all have for the one before)
+      const bool got = wait_committed(&acc, (uint32_t)i & 1, &failed) && !*(volatile int*)&failed;
       tc_fence_after_sync();
       constexpr int COLS = RB == 8 ? 8 : 16;
       uint32_t r[4][COLS];

@@ -198,3 +198,49 @@ def test_the_replay_notices_warps_that_nobody_waits_for(backward, hidden, stuck)
     without units as well."""
     gates = [k for k in _agents(backward, hidden, hidden) if k[0] == "gates"]
     assert [k[1:] for k in gates if not _replay(_agents(backward, hidden, hidden), k)] == stuck
+
+
+# ---- the barrier that dz crosses in backward runs inside a cluster, when a wait has run out ------------------------------
+# bar.sync and bar.arrive count warps, not which, and have no limit: a warp that comes twice takes another's place, and
+# whoever is left waits for good.
+
+def _one_cta(n, failure, over_early):
+    """Warps of bwd_run_cluster in one CTA: at step `failure` what peers push never comes.  over_early: the wait for the MMAs ends
+    when another wait has run out (the model notices what that does); otherwise with the MMAs alone."""
+    state = {"failed": False, "here": 0, "crossed": 0, "mma": 0}
+    COUNT = 6
+
+    def cross(name):
+        state["here"] += 1
+        if state["here"] == COUNT:
+            state["here"], state["crossed"] = 0, state["crossed"] + 1
+
+    def gates(w):
+        for i in range(n):
+            if i > 0 and i - 1 >= failure:
+                yield lambda: True                       # (polls: others may go first)
+                state["failed"] = True
+            cross(w)
+            yield lambda: state["mma"] > i or (over_early and state["failed"])
+
+    def syncs(name):
+        for i in range(n):
+            cross(name)
+            turn = state["crossed"] if state["here"] else state["crossed"] - 1
+            yield lambda: state["crossed"] > turn
+            if name == "mma":
+                state["mma"] += 1
+
+    agents = {("gates", w): gates(w) for w in range(4)}
+    agents["mma"], agents["io"] = syncs("mma"), syncs("io")
+    return agents
+
+
+@pytest.mark.parametrize("failure", [0, 1, 2])
+def test_warps_cross_the_barrier_of_a_failed_backward_run_together(failure):
+    for late in list(_one_cta(5, failure, False)):
+        assert _replay(_one_cta(5, failure, False), late), late
+
+
+def test_a_wait_for_products_that_ends_early_would_leave_warps_in_the_barrier():
+    assert not all(_replay(_one_cta(5, 0, True), late) for late in list(_one_cta(5, 0, True)))

@@ -196,7 +196,9 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = blockIdx.x / ncta, cta = blockIdx.x % ncta, groups = gridDim.x / ncta;
-  const uint32_t group_bytes = (uint32_t)ncta * CU * RB * 2, slot_bytes = group_bytes * groups;
+  // a slot: the groups one after the other, [8 units][R rows][16 bytes] each (the last group's R may be less than RB)
+  const int R = grp == groups - 1 ? ring_last_rows(a.B, RB) : RB;
+  const uint32_t row_bytes = (uint32_t)ncta * CU * 2, group_bytes = row_bytes * RB, slot_bytes = group_bytes * (groups - 1) + row_bytes * ring_last_rows(a.B, RB);
 
   if (tid == 0) {
     weights_init(wt);
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
     uint32_t want = 0;
 #pragma unroll
     for (int x = 0; x < N; ++x)
-      if (p0 + x * STEP < p_end) want |= 1u << x;
+      if (row < R && p0 + x * STEP < p_end) want |= 1u << x;
     uint8_t* const to = sH + p0 * PIECE + row * 16;
     {
       // the state the run starts from, rows past the batch as zeros
@@ -275,10 +277,10 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
       for (int x = 0; x < N; ++x)
         if (want >> x & 1) *reinterpret_cast<uint4*>(to + x * STEP * PIECE) = v[x];
     }
-    const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)p0 * (RB * 16) + row * 16;
+    const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)p0 * (R * 16) + row * 16;
     for (int i = 0; i < a.n; ++i) {
       if (i > 0) {
-        if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * RB * 16, to + (i & 1) * h_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
+        if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * R * 16, to + (i & 1) * h_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
         if (g.fault && pw == 0 && !poll_pieces<1>(g.never, 0, to, 0, 1u, &failed, g.poll_limit)) break;
       }
       fence_proxy_async_shared();
@@ -317,9 +319,10 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
       }
     }
     if (pvalid) hprev = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.ws + (size_t)op0.h_src * 16) + ep);
-    // this lane's piece in a slot: [8 units][RB rows][16 bytes]
-    const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)(jw / 8) * (RB * 16) + (uint32_t)(8 * half + prow) * 16;
-    if (lane < 8)
+    // this lane's piece in a slot
+    const bool sends = lane < 8 && 8 * half + prow < R;
+    const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)(jw / 8) * (R * 16) + (uint32_t)(8 * half + prow) * 16;
+    if (sends)
       for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
     weights_move(wt, KT, sm + Shape::stages(KT), tmem, warp, lane, Shape::G, &failed);
     __syncwarp();
@@ -356,7 +359,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
       __syncwarp();
       uint4 hnew = make_uint4(0, 0, 0, 0);                   // (past the last unit)
       if (wvalid) hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);
-      if (got && lane < 8) {
+      if (got && sends) {
         if (i + 1 < a.n) store_piece(g.ring + (size_t)((i + 1) & (RING_SLOTS - 1)) * slot_bytes + mine, hnew);
         if (i >= 1) store_piece(g.ring + (size_t)((i - 1) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
       }
@@ -444,7 +447,10 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
   const int grp = blockIdx.x / ncta, cta = blockIdx.x % ncta, groups = gridDim.x / ncta;
   const int rank = cta % RING_CLUSTER, cl = cta / RING_CLUSTER;
   const int half0 = 8 * (KT / 2);                  // pieces of two units in a half of the CTA's quarter
-  const uint32_t cta_bytes = 4 * CU * RB * 2, group_bytes = (uint32_t)ncta * cta_bytes, slot_bytes = group_bytes * groups;
+  // a slot: the groups one after the other, [2 units][R rows][16 bytes] each (the last group's R may be less than RB)
+  const int R = grp == groups - 1 ? ring_last_rows(a.B, RB) : RB;
+  const uint32_t row_bytes = (uint32_t)ncta * 4 * CU * 2, group_bytes = row_bytes * RB, slot_bytes = group_bytes * (groups - 1) + row_bytes * ring_last_rows(a.B, RB);
+  const uint32_t cta_bytes = 4 * CU * 2 * (uint32_t)R;
 
   if (tid == 0) {
     weights_init(wt);
@@ -549,12 +555,12 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
     uint32_t want = 0;
 #pragma unroll
     for (int x = 0; x < N; ++x) {
-      if (p0 + x * STEP < (q + 1) * half0) want |= 1u << x;
+      if (row < R && p0 + x * STEP < (q + 1) * half0) want |= 1u << x;
     }
     uint8_t* const to = sZ + p0 * PIECE + row * 16;
-    const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)(rank * per) * cta_bytes + (size_t)p0 * (RB * 16) + row * 16;
+    const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)(rank * per) * cta_bytes + (size_t)p0 * (R * 16) + row * 16;
     for (int i = 0; i < a.n; ++i) {
-      if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * RB * 16, to + (i & 1) * z_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
+      if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * R * 16, to + (i & 1) * z_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
       if (g.fault && pw == 0 && !poll_pieces<1>(g.never, 0, to, 0, 1u, &failed, g.poll_limit)) break;
       fence_proxy_async_shared();
       __syncwarp();
@@ -579,11 +585,12 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
     }
     // dz leaves in pieces of two units: an even lane takes them from its neighbour for its first row, an odd one for its second
     const int odd = lane & 1, prow = r0 + odd;
-    const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)cta * cta_bytes + (uint32_t)(u >> 1) * (RB * 16) + (uint32_t)prow * 16;
-    const bool store_ok = u < units && prow < rows;   // (units is a multiple of 8)
+    const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)cta * cta_bytes + (uint32_t)(u >> 1) * (R * 16) + (uint32_t)prow * 16;
+    const bool store_ok = u < units && prow < rows, sends = prow < R;   // (units is a multiple of 8)
     __nv_bfloat16* dzp = reinterpret_cast<__nv_bfloat16*>(a.dz) + 4 * ((size_t)s_hi * a.B * a.H + (size_t)(brow + prow) * a.H + unit0 + (u & ~1));
     const size_t dz_step = (size_t)4 * a.B * a.H;
-    for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
+    if (sends)
+      for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
     // partial sums: lane l holds column 32 wq + l of the cluster's, which CTA wq owns
     const uint32_t to = map_rank(smem_u32(sR) + (uint32_t)rank * SLOT + (uint32_t)(2 * half) * (CU * 16) + (uint32_t)lane * 16, (uint32_t)wq);
     const uint32_t tb = map_rank(smem_u32(&full[0]), (uint32_t)wq);
@@ -628,13 +635,13 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
       const uint2 get = make_uint2(__shfl_xor_sync(0xffffffffu, send.x, 1), __shfl_xor_sync(0xffffffffu, send.y, 1));
       const uint4 piece = odd ? make_uint4(get.x, get.y, keep.x, keep.y) : make_uint4(keep.x, keep.y, get.x, get.y);
       const bool live = !*(volatile int*)&failed;
-      if (live) store_piece(g.ring + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes + mine, piece);
+      if (live && sends) store_piece(g.ring + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes + mine, piece);
       __syncwarp();
       if (lane == 0) mbar_arrive(&used[i & 1]);
       // beside the exchange: dz to its stage, the piece of two steps ago cleared, the inputs of the next (earlier) step
       if (live) {
         if (store_ok) *reinterpret_cast<uint4*>(dzp) = piece;
-        if (i >= 2) store_piece(g.ring + (size_t)((i - 2) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
+        if (sends && i >= 2) store_piece(g.ring + (size_t)((i - 2) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
       }
       if (i + 1 < a.n) {
         (void)wait_or_fail(&inready[(i + 1) & 1], (uint32_t)((i + 1) >> 1) & 1, &failed);
@@ -693,7 +700,7 @@ int fwd_ctas(int H) { return (H + CU - 1) / CU; }
 }  // namespace
 
 RingArgs ring_args(char* rings, int H, int B, bool backward, int id, bool fault, uint32_t poll_limit) {
-  const size_t rows = (size_t)(B + 15) / 16 * 16, row = (size_t)ring_ctas(H) * CU * 2;
+  const size_t rows = (size_t)ring_slot_rows(B), row = (size_t)ring_ctas(H) * CU * 2;
   const size_t fwd = RING_SLOTS * rows * row, bwd = 4 * fwd;      // bytes of a set
   char* const first = rings + (backward ? 2 * fwd : 0);
   const size_t set = backward ? bwd : fwd;

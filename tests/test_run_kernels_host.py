@@ -26,6 +26,18 @@ def test_an_sm_has_room_for_one_cta_that_holds_tensor_memory_and_waits_for_other
             assert dynamic <= CTA_MOST, hidden
 
 
+
+@pytest.mark.parametrize("hidden,batch,t,most", [
+    (520, 1, 7, 8053760), (520, 1, 100, 8120320), (520, 17, 100, 49853440), (640, 2, 7, 13720320), (776, 64, 7, 136625664),
+    (1024, 1, 100, 23150592), (1024, 3, 100, 33357824), (1024, 64, 100, 184231936),
+])
+def test_the_ring_takes_no_more_than_its_place_in_the_workspace(hidden, batch, t, most):
+    """`most`: the workspace with a stage for h_{k-1} and one for h_k, which the ring and one stage for both replace.  (So
+    small a batch as 3 rows at H = 1024 fits the 32 MB of the step without allocations.)"""
+    desc = B.make_desc(1, 128, hidden, 64, batch, t, "bf16")
+    assert B.mebptt_lstm_workspace_bytes(desc, B.mebptt_plan(t, 8, B.MEBPTT_HSM)) <= most
+
+
 # ---- the waits inside a run, replayed with one warp as late as can be ---------------------------------------------------
 # Barriers are waited for by the parity of a phase: whoever comes when the phase after that is over as well waits for good,
 # or (two phases on) takes the accumulators of another step.

@@ -36,6 +36,7 @@ def _static_run(dp, plan):
 @pytest.mark.parametrize("base,kw,mode,m", [
     ("c1", dict(), "hsm", 8),                                                      # fp32, a walked tape
     ("c2", dict(input=64, hidden=128, batch=32, t=40, readout=64), "msm", 9),      # bf16, tensor-core kernels
+    ("c2", dict(input=72, hidden=1024, batch=3, t=100, readout=64), "hsm", 7),     # the same, through a ring
 ])
 def test_static_workspace_step_matches_ordinary_step_twice(base, kw, mode, m):
     from paper_1606_03401_b200 import binding as B

@@ -26,12 +26,10 @@ __device__ __forceinline__ void push16(uint32_t addr, uint4 v, uint32_t bar) {
                "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
                : "memory");
 }
-// Bounded wait for bytes that peers push, over at once where this CTA has given up.  (The barrier and what it counts lie
-// in this CTA's memory.  An acquire at the scope of the cluster would also wait for this thread's own stores to global
-// memory: 260 cycles without any, 500 to 760 with some.)
+// Bounded wait for bytes that peers push, over at once where this CTA has given up.
 __device__ __forceinline__ bool wait_pushed(uint64_t* bar, uint32_t parity, volatile int* failed, uint32_t limit) {
   for (uint32_t i = 0; i < limit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_try_wait_pushed(smem_u32(bar), parity)) return true;
     if (i > 256) {
       if (*failed) return false;
       __nanosleep(64);

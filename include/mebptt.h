@@ -278,7 +278,8 @@ size_t mebptt_lstm_workspace_bytes(const mebptt_lstm_desc *desc, const mebptt_pl
 size_t mebptt_lstm_working_bytes(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan);
 
 /* Number of kernel launches one mebptt_lstm_train_step enqueues for this descriptor and plan
- * (memsets not counted); -1 on error. */
+ * (memsets not counted); -1 on error.  (On a whole device: where a run of one bfloat16 layer finds room for some of its
+ * groups of batch rows only, they take turns, a launch each.) */
 int64_t mebptt_lstm_launch_count(const mebptt_lstm_desc *desc, const mebptt_plan_t *plan);
 
 /*
@@ -513,6 +514,8 @@ int64_t mebptt_test_run_smem(int route, int shorter, int backward, int hidden, i
  * for.  -1 where nobody waits for units (backward runs inside a cluster wait for every CTA's partial sums).
  */
 int mebptt_test_run_units(int backward, int hidden);
+/* Testing aid: of those of a forward run through the ring, how many the first part of the contraction holds. */
+int mebptt_test_ring_first_part(int hidden);
 
 /*
  * Testing aid: the schedule that a whole tape is walked by (MEBPTT_ROUTE_PODS, MEBPTT_ROUTE_TEAMS), as the

@@ -13,6 +13,7 @@
 #include "env.hpp"
 #include "kernels.hpp"
 #include "layout.hpp"
+#include "lstm_dev.cuh"
 #include "mebptt.h"
 #include "plan.hpp"
 #include "pod.hpp"
@@ -919,6 +920,8 @@ int mebptt_test_run_units(int backward, int hidden) {
   if (hidden < 64 || hidden > 1024 || hidden % 8 || (backward && tc::cluster_runs_supported(hidden))) return -1;
   return backward ? tc::bwd_waited_units(hidden) : tc::fwd_waited_units(hidden);
 }
+
+int mebptt_test_ring_first_part(int hidden) { return 64 * tc::ring_first_part_blocks(hidden); }
 
 int64_t mebptt_test_schedule(const mebptt_lstm_desc* desc, const mebptt_plan_t* plan, int64_t room, int64_t* info, void* records,
                              int64_t most_records, int64_t* launches, int64_t most_launches) {

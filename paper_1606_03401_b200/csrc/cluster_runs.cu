@@ -24,6 +24,7 @@
 #include <cuda_runtime.h>
 
 #include "cluster_runs.hpp"
+#include "env.hpp"
 #include "launch.hpp"
 #include "lstm_dev.cuh"
 #include "mebptt.h"
@@ -583,7 +584,8 @@ bool cluster_maps(CUtensorMap* tm_w, CUtensorMap* tm_wt, const void* wp_hh, cons
 
 int cluster_rows(int B, int H) {
   const int cs = cluster_ctas(H);
-  int fit = 1 << 30;
+  if (env::run_cluster() > 0 && cs > env::run_cluster()) return 0;
+  int fit = run_sms() / cs;
   for (int RB : {8, 12})
     for (int dir = 0; dir < 2; ++dir) {
       const void* fn = kernel(dir, RB);

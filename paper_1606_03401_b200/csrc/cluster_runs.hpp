@@ -57,7 +57,8 @@ struct ClusterBwdArgs {
 // Tensor maps of the two kernels: W_hh with permuted gate rows and its transpose (boxes of 64 columns, 128 rows).
 bool cluster_maps(CUtensorMap* tm_w, CUtensorMap* tm_wt, const void* wp_hh, const void* wpT_hh, int H);
 // Batch rows a cluster takes (8 or 12), so that all clusters are on the device at once where that can be; 0 where
-// the device cannot run clusters of this size.  Sets the kernels' attributes as well.
+// the device cannot run clusters of this size (those of more than eight CTAs, which more than 256 units take, need not
+// fit a partition of a device).  Sets the kernels' attributes as well.
 int cluster_rows(int B, int H);
 int cluster_smem(bool backward, int H, int rows);   // dynamic shared memory of a CTA
 cudaError_t cluster_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, int rows, cudaStream_t s);

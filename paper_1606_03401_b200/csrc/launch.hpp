@@ -25,6 +25,16 @@ inline bool pdl_enabled() { return !env::no_pdl(); }
 constexpr int LONE_SMEM = 228 * 1024 / 2 - 1024 + 16;
 inline int lone_smem(int bytes) { return bytes > LONE_SMEM ? bytes : LONE_SMEM; }
 
+// CTAs that wait for one another the current device keeps resident (one an SM, as above); 0 if it cannot be asked.
+inline int run_sms() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return env::run_sms() > 0 && env::run_sms() < sms ? env::run_sms() : sms;
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_on(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                              Args&&... args) {

@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(128, 2) leaf_products_kernel(const __grid_cons
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   const int M = a.n * a.B, G = 4 * a.H;
   // tiles of the contraction: the input's, then those of h, the first nk1 of them in part 1
-  const int nk0 = (a.I + BK - 1) / BK, KB = (a.H + BK - 1) / BK, nk1 = fwd_first_part_blocks(a.H), nk = nk0 + KB;
+  const int nk0 = (a.I + BK - 1) / BK, KB = (a.H + BK - 1) / BK, nk1 = a.first, nk = nk0 + KB;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(128, 2) leaf_products_kernel(const __grid_cons
 }  // namespace
 
 int leaf_products(const LeafArgs& a, const void* x, const void* wp_ih, const void* hprev, const void* wp_hh, cudaStream_t s) {
-  const int M = a.n * a.B, G = 4 * a.H, parts = fwd_first_part_blocks(a.H) < (a.H + BK - 1) / BK ? 3 : 2;
+  const int M = a.n * a.B, G = 4 * a.H, parts = a.first < (a.H + BK - 1) / BK ? 3 : 2;
   const int wide_tiles = (G + 127) / 128 * ((M + BM - 1) / BM);
   const bool narrow = wide_tiles <= 74;   // tiles of 128 columns would occupy half the SMs at most
   const int BN = narrow ? 32 : 128;

@@ -21,6 +21,7 @@ struct LeafArgs {
   int64_t* counters;
   int* status;
   int B, I, H;
+  int first;              // 64-wide blocks of h in the first part of its contraction (lstm_dev.cuh)
 };
 // x [n][B][I], hprev [n][B][H]: row-major operands; wp_ih [4H][I], wp_hh [4H][H].  Returns a status.
 int leaf_products(const LeafArgs& a, const void* x, const void* wp_ih, const void* hprev, const void* wp_hh, cudaStream_t s);

@@ -37,10 +37,10 @@ __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v 
 
 // The contraction with W_hh is summed in two parts from 513 units on, z = (Zx + part 0) + part 1, and the batched
 // products of a leaf batch add them in that order, so that both give the same bits.  64-wide blocks in the first part:
-__host__ __device__ inline int fwd_first_part_blocks(int H) {
-  const int KB = (H + 63) / 64;
-  return KB > 8 ? (KB + 1) / 2 : KB;
-}
+// (Through the ring in two parts at any width: each leaves something to poll for all of the four warps that poll it, which
+// below 289 units the larger of the halves first would not.)
+__host__ __device__ inline int ring_first_part_blocks(int H) { return ((H + 63) / 64 + (H > 512 ? 1 : 0)) / 2; }
+__host__ __device__ inline int fwd_first_part_blocks(int H) { return H > 512 ? ring_first_part_blocks(H) : (H + 63) / 64; }
 
 }  // namespace tc
 }  // namespace mebptt

@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
   const uint32_t h_buf = (uint32_t)KT * 8 * PIECE;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int grp = blockIdx.x / ncta, cta = blockIdx.x % ncta, groups = gridDim.x / ncta;
+  const int grp = g.first + (int)blockIdx.x / ncta, cta = (int)blockIdx.x % ncta, groups = (a.B + RB - 1) / RB;
   // a slot: the groups one after the other, [8 units][R rows][16 bytes] each (the last group's R may be less than RB)
   const int R = grp == groups - 1 ? ring_last_rows(a.B, RB) : RB;
   const uint32_t row_bytes = (uint32_t)ncta * CU * 2, group_bytes = row_bytes * RB, slot_bytes = group_bytes * (groups - 1) + row_bytes * ring_last_rows(a.B, RB);
@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
   __syncthreads();
   if (tid == 0) {
     if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (blockIdx.x == 0) a.counters[0] += a.n;
+    else if (grp == 0 && cta == 0) a.counters[0] += a.n;
   }
   if (warp == GATES) tmem_dealloc(tmem, 512);
 }
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
   const uint32_t z_buf = (uint32_t)KT * 8 * PIECE;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int grp = blockIdx.x / ncta, cta = blockIdx.x % ncta, groups = gridDim.x / ncta;
+  const int grp = g.first + (int)blockIdx.x / ncta, cta = (int)blockIdx.x % ncta, groups = (a.B + RB - 1) / RB;
   const int rank = cta % RING_CLUSTER, cl = cta / RING_CLUSTER;
   const int half0 = 8 * (KT / 2);                  // pieces of two units in a half of the CTA's quarter
   // a slot: the groups one after the other, [2 units][R rows][16 bytes] each (the last group's R may be less than RB)
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
     asm volatile("cp.async.wait_all;" ::: "memory");
   } else if (warp == GATES + 2) {
     // loss terms of the run: the partial sums of a step in a fixed order
-    if (blockIdx.x == 0)
+    if (grp == 0 && cta == 0)
       for (int i = lane; i < a.n; i += 32) {
         float sum = 0.f;
         for (int p = 0; p < a.loss_parts; ++p) sum += a.loss_part[(s_hi - i) * a.loss_parts + p];
@@ -677,7 +677,7 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
   cluster_sync();     // no CTA leaves while a peer may still push to it
   if (tid == 0) {
     if (failed) *a.status = MEBPTT_ERR_TIMEOUT;
-    else if (blockIdx.x == 0) a.counters[1] += a.n;
+    else if (grp == 0 && cta == 0) a.counters[1] += a.n;
   }
   if (warp == GATES) tmem_dealloc(tmem, 512);
 }
@@ -704,47 +704,61 @@ RingArgs ring_args(char* rings, int H, int B, bool backward, int id, bool fault,
   const size_t fwd = RING_SLOTS * rows * row, bwd = 4 * fwd;      // bytes of a set
   char* const first = rings + (backward ? 2 * fwd : 0);
   const size_t set = backward ? bwd : fwd;
-  return RingArgs{first + (size_t)(id & 1) * set, first + (size_t)(~id & 1) * set, rings + 2 * fwd + 2 * bwd, fault ? 1u : 0u, poll_limit};
+  return RingArgs{first + (size_t)(id & 1) * set, first + (size_t)(~id & 1) * set, rings + 2 * fwd + 2 * bwd, fault ? 1u : 0u, poll_limit, 0};
 }
 
-int ring_rows(int B, int H) {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); return 0; }
+RingFit ring_fit(int B, int H) {
+  const int sms = run_sms();
+  RingFit best{0, 0};
   for (int RB : {8, 16}) {
     const int groups = (B + RB - 1) / RB;
-    bool fits = true;
-    for (int dir = 0; dir < 2 && fits; ++dir) {
+    int at_once = sms / fwd_ctas(H);
+    for (int dir = 0; dir < 2; ++dir) {
       const void* fn = kernel(dir != 0, RB);
-      const int smem = smem_bytes(dir != 0, RB, H), ctas = groups * (dir ? ring_ctas(H) : fwd_ctas(H));
-      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(dir != 0, RB, 32 * CU)) != cudaSuccess) { cudaGetLastError(); return 0; }
-      if (!dir) { fits = ctas <= sms; continue; }
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)ctas); cfg.blockDim = dim3((unsigned)threads(true, RB)); cfg.dynamicSmemBytes = (size_t)smem;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = RING_CLUSTER; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-      cfg.attrs = at; cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
-      fits = n * RING_CLUSTER >= ctas;
+      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(dir != 0, RB, 32 * CU)) != cudaSuccess) { cudaGetLastError(); return RingFit{0, 0}; }
     }
-    if (fits) return RB;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ring_ctas(H)); cfg.blockDim = dim3((unsigned)threads(true, RB)); cfg.dynamicSmemBytes = (size_t)smem_bytes(true, RB, H);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = RING_CLUSTER; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel(true, RB), &cfg) != cudaSuccess) { cudaGetLastError(); return RingFit{0, 0}; }
+    if (n * RING_CLUSTER > sms) n = sms / RING_CLUSTER;
+    if (n * RING_CLUSTER / ring_ctas(H) < at_once) at_once = n * RING_CLUSTER / ring_ctas(H);
+    if (at_once >= groups) return RingFit{RB, groups};
+    if (at_once > 0) best = RingFit{RB, at_once};   // in turns: of more rows, fewer
   }
-  return 0;
+  return best;
 }
 
 int ring_smem(bool backward, int H, int rows) { return smem_bytes(backward, rows, H); }
 
-cudaError_t ring_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, const RingArgs& r, int rows, cudaStream_t s) {
-  int ncta = fwd_ctas(a.H), KT0 = fwd_first_part_blocks(a.H);
-  void* args[] = {(void*)&tm_w, (void*)&a, (void*)&r, (void*)&ncta, (void*)&KT0};
-  return launch_coop(kernel(false, rows), (a.B + rows - 1) / rows * ncta, threads(false, rows), (size_t)smem_bytes(false, rows, a.H), s, args, 1);
+cudaError_t ring_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, const RingArgs& r, RingFit fit, cudaStream_t s) {
+  int ncta = fwd_ctas(a.H), KT0 = ring_first_part_blocks(a.H);
+  const int groups = (a.B + fit.rows - 1) / fit.rows;
+  cudaError_t e = cudaSuccess;
+  RingArgs g = r;
+  for (g.first = 0; g.first < groups && e == cudaSuccess; g.first += fit.groups) {
+    const int n = groups - g.first < fit.groups ? groups - g.first : fit.groups;
+    void* args[] = {(void*)&tm_w, (void*)&a, (void*)&g, (void*)&ncta, (void*)&KT0};
+    e = launch_coop(kernel(false, fit.rows), n * ncta, threads(false, fit.rows), (size_t)smem_bytes(false, fit.rows, a.H), s, args, 1);
+  }
+  return e;
 }
 
-cudaError_t ring_backward(const CUtensorMap& tm_wt, const ClusterBwdArgs& a, const RingArgs& r, int rows, cudaStream_t s) {
+cudaError_t ring_backward(const CUtensorMap& tm_wt, const ClusterBwdArgs& a, const RingArgs& r, RingFit fit, cudaStream_t s) {
   int ncta = ring_ctas(a.H);
-  void* args[] = {(void*)&tm_wt, (void*)&a, (void*)&r, (void*)&ncta};
-  return launch_coop(kernel(true, rows), (a.B + rows - 1) / rows * ncta, threads(true, rows), (size_t)smem_bytes(true, rows, a.H), s, args, RING_CLUSTER, false);
+  const int groups = (a.B + fit.rows - 1) / fit.rows;
+  cudaError_t e = cudaSuccess;
+  RingArgs g = r;
+  for (g.first = 0; g.first < groups && e == cudaSuccess; g.first += fit.groups) {
+    const int n = groups - g.first < fit.groups ? groups - g.first : fit.groups;
+    void* args[] = {(void*)&tm_wt, (void*)&a, (void*)&g, (void*)&ncta};
+    e = launch_coop(kernel(true, fit.rows), n * ncta, threads(true, fit.rows), (size_t)smem_bytes(true, fit.rows, a.H), s, args, RING_CLUSTER, false);
+  }
+  return e;
 }
 
 }  // namespace tc

@@ -9,6 +9,7 @@ namespace tc {
 constexpr int RING_SLOTS = 4;    // steps a ring holds
 constexpr int RING_CLUSTER = 4;  // CTAs that share the contraction index of a backward step
 
+// Widths that nothing else serves.  (A device without clusters of more than eight CTAs has 257 to 512 units here as well.)
 inline bool ring_runs_supported(int H, int B) { return H % 8 == 0 && H > 16 * CU && H <= 32 * CU && B <= 64; }
 // CTAs of a group of batch rows: 32 units each, whole clusters (the last ones may have no unit)
 inline int ring_ctas(int H) { return (H + RING_CLUSTER * CU - 1) / (RING_CLUSTER * CU) * RING_CLUSTER; }
@@ -37,16 +38,19 @@ struct RingArgs {
   const char* never;     // 16 bytes of ones that nobody writes
   uint32_t fault;        // testing aid: wait for those as well
   uint32_t poll_limit;
+  int first;             // the launch's first group of batch rows
 };
 // The sets of launch number `id` of its direction.
 RingArgs ring_args(char* rings, int H, int B, bool backward, int id, bool fault, uint32_t poll_limit);
 
 // Tensor maps: boxes of 64 columns by 128 rows, as for the cluster kernels.
-// Batch rows of a group (8 or 16); 0 where the device cannot keep the kernels' CTAs resident.
-int ring_rows(int B, int H);
+// Batch rows of a group (8 or 16) and groups a launch takes, all of them where the device keeps their CTAs resident at once;
+// otherwise they take turns (batch rows never mix), and where it has no room for one, rows = 0.
+struct RingFit { int rows, groups; };
+RingFit ring_fit(int B, int H);
 int ring_smem(bool backward, int H, int rows);   // dynamic shared memory of a CTA
-cudaError_t ring_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, const RingArgs& r, int rows, cudaStream_t s);
-cudaError_t ring_backward(const CUtensorMap& tm_wt, const ClusterBwdArgs& a, const RingArgs& r, int rows, cudaStream_t s);
+cudaError_t ring_forward(const CUtensorMap& tm_w, const ClusterFwdArgs& a, const RingArgs& r, RingFit fit, cudaStream_t s);
+cudaError_t ring_backward(const CUtensorMap& tm_wt, const ClusterBwdArgs& a, const RingArgs& r, RingFit fit, cudaStream_t s);
 
 }  // namespace tc
 }  // namespace mebptt

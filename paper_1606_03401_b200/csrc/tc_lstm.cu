@@ -1104,7 +1104,8 @@ struct Prepared {
   bool short_runs = false;         // the kernels of this file take short runs of a layer whose longer ones go through the ring
   CUtensorMap tm_h, tm_w, tm_dz[2], tm_wt;
   int fwd_ncg = 0, fwd_smem = 0, bwd_smem = 0, bwd_tb = 8;
-  int run_rows = 0;                // batch rows of a cluster (cluster_runs.cu) or of a group of CTAs (ring_runs.cu)
+  int run_rows = 0;                // batch rows of a cluster (cluster_runs.cu); 0: the ring takes the runs (ring_runs.cu)
+  RingFit ring{0, 0};
   CUtensorMap tm_w_cl, tm_wt_cl;
   int rc = MEBPTT_OK;
 
@@ -1217,8 +1218,11 @@ void build_device_part(Prepared& P, const Layout& y, char* ws) {
   // A forward and a backward operation in runs of 32, against the kernels of this file: 2.8 -> 0.78 and 3.9 -> 0.90 us at
   // H = 256, 3.1 -> 1.32 and 4.0 -> 1.73 us at H = 512, 4.1 -> 2.8 and 4.6 -> 3.1 us at H = 1024.
   if (!cluster_maps(&P.tm_w_cl, &P.tm_wt_cl, wp_hh, wpT_hh, H)) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
-  P.run_rows = cluster_runs_supported(H) ? cluster_rows(B, H) : ring_rows(B, H);
-  if (P.run_rows <= 0) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
+  // A device without the clusters of nine to sixteen CTAs that 257 to 512 units take (a partition of one, a context that
+  // may use a part of the SMs) has the ring for those as well.
+  P.run_rows = cluster_runs_supported(H) ? cluster_rows(B, H) : 0;
+  if (P.run_rows <= 0 && H > 8 * CU) P.ring = ring_fit(B, H);
+  if (P.run_rows <= 0 && P.ring.rows <= 0) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
   if (cluster_runs_supported(H) || B <= FB || B > 2 * FB || H % 128 != 0) return;
   // Short runs (below).  Widths in whole blocks of 128: both kinds of kernels then add the same parts in the same order.
   const int KB0 = fwd_first_part_blocks(H), kbs = (G / 64) / GCS;
@@ -1236,7 +1240,7 @@ void build_device_part(Prepared& P, const Layout& y, char* ws) {
   at1[0].val.clusterDim.x = GCS; at1[0].val.clusterDim.y = 1; at1[0].val.clusterDim.z = 1;
   cfg.attrs = at1; cfg.numAttrs = 1;
   int nclusters = 0;
-  ok = ok && cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters * GCS >= 2 * P.fwd_ncg;
+  ok = ok && cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters * GCS >= 2 * P.fwd_ncg && run_sms() >= 2 * P.fwd_ncg;
   if (!ok) { cudaGetLastError(); return; }
   // the whole workspace as rows of H bfloat16: any h block starts at a whole row
   ok = make_tmap_blocks64(&P.tm_h, ws, (uint64_t)H, y.total / ((size_t)H * 2), (uint64_t)H * 2, FB, (uint32_t)KB0) &&
@@ -1342,7 +1346,11 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
   float* bias_p = reinterpret_cast<float*>(at(y.off_bias_p));
   __nv_bfloat16* woutT = reinterpret_cast<__nv_bfloat16*>(at(y.off_woutT));
 
-  const bool clusters = cluster_runs_supported(H);   // (else the ring, and for short runs perhaps the kernels of this file)
+  const bool clusters = P.run_rows > 0;   // (else the ring, and for short runs perhaps the kernels of this file)
+  // Where the layout has no place for the ring because clusters were to take the runs, it lies in the second copy of the
+  // input projections (16 S >= 512 bytes a unit and row; the ring takes 120), which then are not computed ahead.
+  const bool no_room = P.ring.rows > 0 && !y.ring_bytes;
+  char* const ring = no_room ? reinterpret_cast<char*>(zx + (size_t)S * B * G) : at(y.off_ring);
   // On request (a switch in the environment) the step runs on a stream of the library's, of the most
   // urgent priority, ordered after what the caller's stream holds and joined to it at the end: the
   // caller's stream is of the least urgent priority as a rule, like the stream of the weight-gradient
@@ -1366,7 +1374,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
     cudaMemsetAsync(io.counters, 0, 8 * sizeof(int64_t), s);
     cudaMemsetAsync(sync, 0, y.n_sync * 4, s);
     cudaMemsetAsync(status, 0, 256, s);
-    if (y.ring_bytes) cudaMemsetAsync(at(y.off_ring), 0xff, y.ring_bytes, s);   // nothing has been written there yet
+    if (P.ring.rows > 0) cudaMemsetAsync(ring, 0xff, ring_bytes(H, B), s);   // nothing has been written there yet
     // (from page-locked memory: an asynchronous copy proper; from pageable memory, which only the
     // allocation-free entry point uses, the call may wait for the stream to reach the copy)
     cudaMemcpyAsync(at(y.off_tape), P.tape, P.tape_entries * sizeof(DevOp), cudaMemcpyHostToDevice, s);
@@ -1427,7 +1435,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
   bool targets_waited = false;
   int zx_lo = 0, zx_hi = 0;   // time steps [zx_lo, zx_hi) whose input projections the Zx buffer holds
   float* zleaf = reinterpret_cast<float*>(at(y.off_zleaf));
-  const bool zx_ahead = side && !env::no_zx_ahead();
+  const bool zx_ahead = side && !env::no_zx_ahead() && !no_room;
   int zx_w = -1;          // windows opened so far, less one
   float* zx_cur = zx;     // the copy of the buffer that holds the window in use
   auto project_window = [&](size_t it, int w) {
@@ -1506,7 +1514,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
           void* args[] = {(void*)&P.tm_h, (void*)&P.tm_w, (void*)&sa};
           e = launch_coop((const void*)fwd_run_kernel, 2 * P.fwd_ncg, 192, P.fwd_smem, s, args, 1);
         } else {
-          e = ring_forward(P.tm_w_cl, a, ring_args(at(y.off_ring), H, B, false, fwd_launches++, fault & 1, polls), P.run_rows, s);
+          e = ring_forward(P.tm_w_cl, a, ring_args(ring, H, B, false, fwd_launches++, fault & 1, polls), P.ring, s);
         }
         if (!cuda_ok(e, "forward run launch")) rc = MEBPTT_ERR_CUDA;
         span_end(timer, span, s);
@@ -1550,7 +1558,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
         ++launches;
         if (!dry && rc == MEBPTT_OK)
           rc = leaf_products(LeafArgs{bops, n, ws, bias_p, zleaf + (size_t)s_lo * B * G, has_h[(size_t)s_hi + 1] ? nullptr : hk_c + (size_t)s_hi * B * H,
-                                      io.counters, status, B, I, H},
+                                      io.counters, status, B, I, H, clusters ? (H + 63) / 64 : ring_first_part_blocks(H)},
                              reinterpret_cast<const __nv_bfloat16*>(io.x) + (size_t)(k_lo - 1) * B * I, wp_ih, hprev_c + (size_t)s_lo * B * H, wp_hh, s);
         has_h[(size_t)s_hi + 1] = 1;
       }
@@ -1600,7 +1608,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
           // (in plain stream order: early residency of a clustered cooperative grid measured no gain)
           e = launch_coop((const void*)bwd_run_group_kernel, 2 * P.fwd_ncg, 192, P.bwd_smem, s, args, GCS, false);
         } else {
-          e = ring_backward(P.tm_wt_cl, a, ring_args(at(y.off_ring), H, B, true, bwd_launches++, fault & 2, polls), P.run_rows, s);
+          e = ring_backward(P.tm_wt_cl, a, ring_args(ring, H, B, true, bwd_launches++, fault & 2, polls), P.ring, s);
         }
         if (!cuda_ok(e, "backward run launch")) rc = MEBPTT_ERR_CUDA;
         span_end(timer, span, s);

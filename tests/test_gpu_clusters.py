@@ -1,6 +1,11 @@
 """GPU: runs of the bfloat16 recurrence of one layer -- inside a thread-block cluster up to 512 units, through a ring in
 the L2 and, for short runs, by the grid-wide kernels beyond -- at the edges of what a cluster, a CTA and an MMA tile hold.
 """
+import hashlib
+import os
+import subprocess
+import sys
+
 import pytest
 
 from paper_1606_03401_b200 import synth
@@ -91,3 +96,50 @@ def test_steps_of_two_widths_on_two_streams_do_not_wait_for_one_another(sizes):
         res["loss"] = float(res["loss"][0])
         assert res["counters"][3] == 0
         assert_bit_identical(res, want, want_dx=True)
+
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+CHILD = r"""
+import sys
+sys.path.insert(0, {root!r})
+from tests import test_gpu_clusters as T
+T.smaller_device({hidden}, {batch})
+"""
+
+
+def smaller_device(hidden, batch):
+    """In a process of its own, whose environment says what the device has room for."""
+    cfg, dp = _problem(input=40, hidden=hidden, batch=batch, readout=24, t=41)
+    full = dp.run(dp.full_memory_plan())
+    assert full["counters"][1] == cfg.t and full["counters"][3] == 0
+    assert_close_to_oracle(full, oracle_run(dp.prob), "bf16", want_dx=True)
+    for mode, m in [("hsm", 1), ("hsm", 5), ("ism", 2), ("msm", 9)]:
+        plan = dp.plan(mode, m)
+        res = dp.run(plan)
+        assert res["counters"][0] == plan.cost and res["counters"][1] == cfg.t and res["counters"][3] == 0
+        assert_bit_identical(res, full, want_dx=True)
+    print("BITS", _bits(full))
+
+
+def _bits(res):
+    return hashlib.sha256(b"".join(res[k].tobytes() for k in ("dW", "db", "dW_out", "db_out", "dx"))).hexdigest()
+
+
+@pytest.mark.parametrize("hidden,batch,env,same", [
+    # no clusters of more than eight CTAs: the ring, without a place of its own, in two parts of 2 and 3, 3 and 4, 4 and 4 blocks
+    (264, 33, {"MEBPTT_RUN_CLUSTER": "8"}, False),
+    (392, 9, {"MEBPTT_RUN_CLUSTER": "8"}, False),
+    (512, 64, {"MEBPTT_RUN_CLUSTER": "8"}, False),
+    # fewer SMs than the groups of a batch take: the groups, or the clusters, take turns
+    (640, 64, {"MEBPTT_RUN_SMS": "40"}, True),
+    (1024, 41, {"MEBPTT_RUN_SMS": "70"}, True),
+    (512, 64, {"MEBPTT_RUN_CLUSTER": "8", "MEBPTT_RUN_SMS": "20"}, False),
+])
+def test_a_device_with_room_for_less_takes_other_kernels_or_turns(hidden, batch, env, same):
+    out = subprocess.run([sys.executable, "-c", CHILD.format(root=ROOT, hidden=hidden, batch=batch)], env={**os.environ, **env},
+                         capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    if same:
+        _, dp = _problem(input=40, hidden=hidden, batch=batch, readout=24, t=41)
+        assert out.stdout.split()[-1] == _bits(dp.run(dp.full_memory_plan()))

@@ -212,6 +212,18 @@ def test_the_replay_notices_warps_that_nobody_waits_for(backward, hidden, stuck)
     assert [k[1:] for k in gates if not _replay(_agents(backward, hidden, hidden), k)] == stuck
 
 
+def test_every_warp_that_polls_a_part_of_a_step_has_something_to_wait_for():
+    """Four warps poll each part in turns of pieces of eight units: a warp without any would run ahead of the others."""
+    for hidden in range(264, 1025, 8):               # (up to 512 where a device has no clusters for them)
+        first, waited = B.mebptt_test_ring_first_part(hidden), B.mebptt_test_run_units(False, hidden)
+        for pieces in (first // 8, (waited - first) // 8):
+            for in_hand in (2, 4):                   # pieces a warp has at a time: 16 rows, 8 rows
+                assert 3 * in_hand < pieces <= 64, hidden
+        quarter = -(-hidden // 128) * 16             # backward, pieces of two units: in halves
+        for in_hand in (2, 4):
+            assert 3 * in_hand < quarter // 2 <= 64, hidden
+
+
 # ---- the barrier that dz crosses in backward runs inside a cluster, when a wait has run out ------------------------------
 # bar.sync and bar.arrive count warps, not which, and have no limit: a warp that comes twice takes another's place, and
 # whoever is left waits for good.

@@ -514,6 +514,8 @@ int64_t mebptt_test_run_smem(int route, int shorter, int backward, int hidden, i
  * for.  -1 where nobody waits for units (backward runs inside a cluster wait for every CTA's partial sums).
  */
 int mebptt_test_run_units(int backward, int hidden);
+/* Testing aid: kernels the library has launched in this process so far. */
+int64_t mebptt_test_launches(void);
 /* Testing aid: of those of a forward run through the ring, how many the first part of the contraction holds. */
 int mebptt_test_ring_first_part(int hidden);
 

@@ -95,6 +95,7 @@ _SIGS = {
     "mebptt_test_run_smem": (_i64, [_i32, _i32, _i32, _i32, _i32]),
     "mebptt_test_run_units": (_i32, [_i32, _i32]),
     "mebptt_test_ring_first_part": (_i32, [_i32]),
+    "mebptt_test_launches": (_i64, []),
     "mebptt_slot_copy": (_i32, [_vp, _vp, _sz, _vp]),
     "mebptt_gemm_bf16": (_i32, [_vp, _i64, _i32, _vp, _i64, _i32, _vp, _i64, _i32, _vp, _i64, _i64, _i64, _vp, _vp]),
     "mebptt_strerror": (C.c_char_p, [_i32]),
@@ -338,6 +339,10 @@ def mebptt_test_run_smem(route: str, hidden: int, rows: int, backward: bool, sho
 
 def mebptt_test_run_units(backward: bool, hidden: int) -> int:
     return lib.mebptt_test_run_units(int(backward), hidden)
+
+
+def mebptt_test_launches() -> int:
+    return lib.mebptt_test_launches()
 
 
 def mebptt_test_ring_first_part(hidden: int) -> int:

@@ -12,6 +12,7 @@
 
 #include "env.hpp"
 #include "kernels.hpp"
+#include "launch.hpp"
 #include "layout.hpp"
 #include "lstm_dev.cuh"
 #include "mebptt.h"
@@ -920,6 +921,8 @@ int mebptt_test_run_units(int backward, int hidden) {
   if (hidden < 64 || hidden > 1024 || hidden % 8 || (backward && tc::cluster_runs_supported(hidden))) return -1;
   return backward ? tc::bwd_waited_units(hidden) : tc::fwd_waited_units(hidden);
 }
+
+int64_t mebptt_test_launches(void) { return g_launches.load(); }
 
 int mebptt_test_ring_first_part(int hidden) { return 64 * tc::ring_first_part_blocks(hidden); }
 

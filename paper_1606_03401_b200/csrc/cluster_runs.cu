@@ -570,7 +570,7 @@ cudaError_t launch_cluster(const void* fn, int threads, int groups, int cs, int 
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(groups * cs)); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = s;
+  cfg.gridDim = dim3((unsigned)(groups * cs)); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = counted(s);
   cfg.attrs = at; cfg.numAttrs = pdl_enabled() ? 2u : 1u;
   return cudaLaunchKernelExC(&cfg, fn, args);
 }

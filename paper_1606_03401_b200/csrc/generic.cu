@@ -17,6 +17,7 @@
 //   dW        dW[g][c]    += sum_b dz[b][g] [in ; h_prev][b][c]
 //   dW_out    dW_out[o][j]+= sum_b dy[b][o] h[b][j]
 #include "kernels.hpp"
+#include "launch.hpp"
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -413,7 +414,7 @@ void gru_forward_step_t(const FwdArgs& a, cudaStream_t s) {
   GruFwdB<T> fb{(const T*)a.W, a.H, K, a.I};
   GruFwdEpi<T> epi{a.bias, (const T*)a.h_prev, (T*)a.h_out, (T*)a.gates, (T*)a.h_in_copy, a.B, a.H, a.plane_elems,
                    a.counters};
-  gemm_tiled<true, true, false><<<tiles(a.B, 4 * a.H), 256, 0, s>>>(a.B, 4 * a.H, K, fa, fb, epi);
+  gemm_tiled<true, true, false><<<tiles(a.B, 4 * a.H), 256, 0, counted(s)>>>(a.B, 4 * a.H, K, fa, fb, epi);
 }
 
 template <class T>
@@ -422,26 +423,26 @@ void gru_backward_layer_t(const BwdArgs& a, cudaStream_t s) {
   const size_t n = (size_t)a.B * a.H;
   const int blocks = (int)((n + 255) / 256 > 1184 ? 1184 : (n + 255) / 256);
   float* dhz = a.dc_rec;   // a GRU carries no cell-state gradient: the buffer holds dh z for this step
-  gru_gate_bwd<T><<<blocks, 256, 0, s>>>(a.dha, a.dh_rec, dhz, (const T*)a.gates, a.plane_elems, (const T*)a.h_prev,
+  gru_gate_bwd<T><<<blocks, 256, 0, counted(s)>>>(a.dha, a.dh_rec, dhz, (const T*)a.gates, a.plane_elems, (const T*)a.h_prev,
                                           a.dz, a.B, a.H, a.counters);
   // dW: the rows of r and z against [in ; h_prev]; the rows of n against in (d n_pre) and h_prev (d q)
-  gemm_tiled<false, false, false><<<tiles(2 * H, K), 256, 0, s>>>(2 * H, K, a.B, DzTA{a.dz, G4},
+  gemm_tiled<false, false, false><<<tiles(2 * H, K), 256, 0, counted(s)>>>(2 * H, K, a.B, DzTA{a.dz, G4},
                                                                    InB<T>{(const T*)a.in, (const T*)a.h_prev, a.I, a.H},
                                                                    AccumEpi{a.dW, K});
-  gemm_tiled<false, false, false><<<tiles(H, a.I), 256, 0, s>>>(H, a.I, a.B, DzTA{a.dz + 2 * H, G4},
+  gemm_tiled<false, false, false><<<tiles(H, a.I), 256, 0, counted(s)>>>(H, a.I, a.B, DzTA{a.dz + 2 * H, G4},
                                                                  HB<T>{(const T*)a.in, a.I},
                                                                  AccumEpi{a.dW + (size_t)2 * H * K, K});
-  gemm_tiled<false, false, false><<<tiles(H, H), 256, 0, s>>>(H, H, a.B, DzTA{a.dz + 3 * H, G4},
+  gemm_tiled<false, false, false><<<tiles(H, H), 256, 0, counted(s)>>>(H, H, a.B, DzTA{a.dz + 3 * H, G4},
                                                                HB<T>{(const T*)a.h_prev, a.H},
                                                                AccumEpi{a.dW + (size_t)2 * H * K + a.I, K});
-  colsum_accum_ld<<<(3 * H + 127) / 128, 128, 0, s>>>(a.dz, a.B, 3 * H, G4, a.db);
+  colsum_accum_ld<<<(3 * H + 127) / 128, 128, 0, counted(s)>>>(a.dz, a.B, 3 * H, G4, a.db);
   // d_in = dz4 against the expanded weights, plus dh z on the recurrent columns
   if (a.d_lo) {
-    gemm_tiled<true, false, false><<<tiles(a.B, K), 256, 0, s>>>(a.B, K, G4, DzA{a.dz, G4},
+    gemm_tiled<true, false, false><<<tiles(a.B, K), 256, 0, counted(s)>>>(a.B, K, G4, DzA{a.dz, G4},
                                                                   GruWB<T>{(const T*)a.W, H, K, a.I, 0},
                                                                   GruDinEpi{a.d_lo, a.I, a.dh_rec, a.H, dhz});
   } else {
-    gemm_tiled<true, false, false><<<tiles(a.B, H), 256, 0, s>>>(a.B, H, G4, DzA{a.dz, G4},
+    gemm_tiled<true, false, false><<<tiles(a.B, H), 256, 0, counted(s)>>>(a.B, H, G4, DzA{a.dz, G4},
                                                                   GruWB<T>{(const T*)a.W, H, K, a.I, a.I},
                                                                   GruDinEpi{nullptr, 0, a.dh_rec, a.H, dhz});
   }
@@ -454,7 +455,7 @@ void forward_step_t(const FwdArgs& a, cudaStream_t s) {
   FwdB<T> fb{(const T*)a.W, a.H, K};
   FwdEpi<T> epi{a.bias, a.c_prev, (const T*)a.h_prev, (T*)a.h_out, a.c_out, (T*)a.gates,
                 (T*)a.h_in_copy, a.c_in_copy, a.B, a.H, a.plane_elems, a.counters};
-  gemm_tiled<true, true, false><<<tiles(a.B, 4 * a.H), 256, 0, s>>>(a.B, 4 * a.H, K, fa, fb, epi);
+  gemm_tiled<true, true, false><<<tiles(a.B, 4 * a.H), 256, 0, counted(s)>>>(a.B, 4 * a.H, K, fa, fb, epi);
 }
 
 template <class T>
@@ -462,17 +463,17 @@ void readout_t(const ReadoutArgs& a, cudaStream_t s) {
   RoA<T> fa{(const T*)a.h, a.H};
   RoB<T> fb{(const T*)a.W_out, a.H};
   RoEpi epi{a.b_out, a.target, a.dy, a.loss_part, a.B, a.O, 1.f / ((float)a.B * (float)a.O)};
-  gemm_tiled<true, true, true><<<tiles(a.B, a.O), 256, 0, s>>>(a.B, a.O, a.H, fa, fb, epi);
-  sum_partials<<<1, 32, 0, s>>>(a.loss_part, a.n_loss_part, 1.f / ((float)a.B * (float)a.O), a.loss_k);
+  gemm_tiled<true, true, true><<<tiles(a.B, a.O), 256, 0, counted(s)>>>(a.B, a.O, a.H, fa, fb, epi);
+  sum_partials<<<1, 32, 0, counted(s)>>>(a.loss_part, a.n_loss_part, 1.f / ((float)a.B * (float)a.O), a.loss_k);
   // dha = dy W_out
-  gemm_tiled<true, false, false><<<tiles(a.B, a.H), 256, 0, s>>>(a.B, a.H, a.O, DyA{a.dy, a.O},
+  gemm_tiled<true, false, false><<<tiles(a.B, a.H), 256, 0, counted(s)>>>(a.B, a.H, a.O, DyA{a.dy, a.O},
                                                                   WoutB<T>{(const T*)a.W_out, a.H},
                                                                   StoreEpi{a.dha, a.H});
   // dW_out += dy^T h ; db_out += sum_b dy
-  gemm_tiled<false, false, false><<<tiles(a.O, a.H), 256, 0, s>>>(a.O, a.H, a.B, DyTA{a.dy, a.O},
+  gemm_tiled<false, false, false><<<tiles(a.O, a.H), 256, 0, counted(s)>>>(a.O, a.H, a.B, DyTA{a.dy, a.O},
                                                                    HB<T>{(const T*)a.h, a.H},
                                                                    AccumEpi{a.dW_out, a.H});
-  colsum_accum<<<(a.O + 127) / 128, 128, 0, s>>>(a.dy, a.B, a.O, a.db_out);
+  colsum_accum<<<(a.O + 127) / 128, 128, 0, counted(s)>>>(a.dy, a.B, a.O, a.db_out);
 }
 
 template <class T>
@@ -480,20 +481,20 @@ void backward_layer_t(const BwdArgs& a, cudaStream_t s) {
   const int K = a.I + a.H, G = 4 * a.H;
   const size_t n = (size_t)a.B * a.H;
   const int blocks = (int)((n + 255) / 256 > 1184 ? 1184 : (n + 255) / 256);
-  gate_bwd<T><<<blocks, 256, 0, s>>>(a.dha, a.dh_rec, a.dc_rec, (const T*)a.gates, a.plane_elems, a.c_t,
+  gate_bwd<T><<<blocks, 256, 0, counted(s)>>>(a.dha, a.dh_rec, a.dc_rec, (const T*)a.gates, a.plane_elems, a.c_t,
                                       a.c_prev, a.dz, a.B, a.H, a.counters);
   // dW += dz^T [in ; h_prev] ; db += sum_b dz     (uses h_prev before dh_rec is replaced)
-  gemm_tiled<false, false, false><<<tiles(G, K), 256, 0, s>>>(G, K, a.B, DzTA{a.dz, G},
+  gemm_tiled<false, false, false><<<tiles(G, K), 256, 0, counted(s)>>>(G, K, a.B, DzTA{a.dz, G},
                                                                InB<T>{(const T*)a.in, (const T*)a.h_prev, a.I, a.H},
                                                                AccumEpi{a.dW, K});
-  colsum_accum<<<(G + 127) / 128, 128, 0, s>>>(a.dz, a.B, G, a.db);
+  colsum_accum<<<(G + 127) / 128, 128, 0, counted(s)>>>(a.dz, a.B, G, a.db);
   // d_in = dz W : columns < I feed dx or the layer below, the rest is the new dh_rec
   if (a.d_lo) {
-    gemm_tiled<true, false, false><<<tiles(a.B, K), 256, 0, s>>>(a.B, K, G, DzA{a.dz, G}, WB<T>{(const T*)a.W, K},
+    gemm_tiled<true, false, false><<<tiles(a.B, K), 256, 0, counted(s)>>>(a.B, K, G, DzA{a.dz, G}, WB<T>{(const T*)a.W, K},
                                                                   DinEpi{a.d_lo, a.I, a.dh_rec, a.H});
   } else {
     // only the recurrent columns are needed: contract against W[:, I:]
-    gemm_tiled<true, false, false><<<tiles(a.B, a.H), 256, 0, s>>>(a.B, a.H, G, DzA{a.dz, G},
+    gemm_tiled<true, false, false><<<tiles(a.B, a.H), 256, 0, counted(s)>>>(a.B, a.H, G, DzA{a.dz, G},
                                                                     WB<T>{(const T*)a.W + a.I, K},
                                                                     DinEpi{nullptr, 0, a.dh_rec, a.H});
   }
@@ -523,7 +524,7 @@ void gru_backward_layer(int dtype, const BwdArgs& a, cudaStream_t s) {
 }
 void finalize_step(const float* loss_t, int64_t t, float* loss, int64_t* counters, int64_t peak_units,
                    const int* status, cudaStream_t s) {
-  finalize<<<1, 32, 0, s>>>(loss_t, t, loss, counters, peak_units, status);
+  finalize<<<1, 32, 0, counted(s)>>>(loss_t, t, loss, counters, peak_units, status);
 }
 }  // namespace generic
 }  // namespace mebptt

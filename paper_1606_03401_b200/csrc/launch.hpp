@@ -13,6 +13,13 @@
 
 namespace mebptt {
 
+// Kernels launched by the process, counted where they are (a testing aid: what launch counts are compared with).
+inline std::atomic<int64_t> g_launches{0};
+inline cudaStream_t counted(cudaStream_t s) {
+  g_launches.fetch_add(1, std::memory_order_relaxed);
+  return s;
+}
+
 inline bool pdl_enabled() { return !env::no_pdl(); }
 
 // Dynamic shared memory of a kernel whose CTAs wait for one another while they hold tensor memory: more than half of an
@@ -39,7 +46,7 @@ template <typename... KArgs, typename... Args>
 inline cudaError_t launch_on(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                              Args&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = counted(s);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -82,6 +89,7 @@ inline cudaError_t launch_coop(const void* fn, int grid, int block, size_t smem,
     cfg.attrs = at; cfg.numAttrs = (unsigned)n;
     const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
     if (e == cudaSuccess) {
+      (void)counted(s);
       if (pdl) pdl_state.store(1);
       return e;
     }

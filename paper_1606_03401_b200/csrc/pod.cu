@@ -15,6 +15,7 @@
 
 #include <type_traits>
 
+#include "launch.hpp"
 #include "layout.hpp"
 #include "pod.hpp"
 #include "pod_run.hpp"
@@ -747,9 +748,9 @@ Fn kernel(int dtype, bool gru, int nb, bool wide) {
 
 void launch_pack(int dtype, bool gru, const PackArgs& p, cudaStream_t s) {
   if (dtype == MEBPTT_BF16) {
-    if (gru) pod_pack<bf16, true><<<592, 256, 0, s>>>(p); else pod_pack<bf16, false><<<592, 256, 0, s>>>(p);
+    if (gru) pod_pack<bf16, true><<<592, 256, 0, counted(s)>>>(p); else pod_pack<bf16, false><<<592, 256, 0, counted(s)>>>(p);
   } else {
-    if (gru) pod_pack<float, true><<<592, 256, 0, s>>>(p); else pod_pack<float, false><<<592, 256, 0, s>>>(p);
+    if (gru) pod_pack<float, true><<<592, 256, 0, counted(s)>>>(p); else pod_pack<float, false><<<592, 256, 0, counted(s)>>>(p);
   }
 }
 

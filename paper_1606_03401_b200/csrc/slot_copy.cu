@@ -13,6 +13,7 @@
 #include <cstdint>
 
 #include "kernels.hpp"
+#include "launch.hpp"
 #include "sm100.cuh"
 
 namespace mebptt {
@@ -92,7 +93,7 @@ void copy_bytes(void* dst, const void* src, size_t bytes, cudaStream_t s) {
     const size_t n = bytes / 16;
     size_t blocks = (n + 255) / 256;
     if (blocks > 148 * 8) blocks = 148 * 8;
-    copy16_small<<<(unsigned)blocks, 256, 0, s>>>((uint4*)dst, (const uint4*)src, n);
+    copy16_small<<<(unsigned)blocks, 256, 0, counted(s)>>>((uint4*)dst, (const uint4*)src, n);
     return;
   }
   // per call: function attributes belong to the current device
@@ -102,7 +103,7 @@ void copy_bytes(void* dst, const void* src, size_t bytes, cudaStream_t s) {
   cudaFuncSetAttribute(slot_copy_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, STAGES * CHUNK + 128);
   const size_t nchunks = (bytes + CHUNK - 1) / CHUNK;
   const unsigned grid = (unsigned)(nchunks < (size_t)sms ? nchunks : (size_t)sms);
-  slot_copy_bulk<<<grid, 32, STAGES * CHUNK + 128, s>>>((char*)dst, (const char*)src, bytes);
+  slot_copy_bulk<<<grid, 32, STAGES * CHUNK + 128, counted(s)>>>((char*)dst, (const char*)src, bytes);
 }
 
 }  // namespace generic

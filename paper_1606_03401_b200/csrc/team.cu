@@ -18,6 +18,7 @@
 
 #include "env.hpp"
 #include "kernels.hpp"
+#include "launch.hpp"
 #include "layout.hpp"
 #include "plan.hpp"
 #include "sm100.cuh"
@@ -1022,7 +1023,7 @@ std::shared_ptr<Kept> schedule_for(const Layout& y, const Plan* p, bool pageable
 // cluster: CTAs per cluster, or 0 for a cooperative grid
 int launch(const void* fn, int grid, int cluster, int smem, void** args, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = s;
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = (size_t)smem; cfg.stream = counted(s);
   cudaLaunchAttribute at[1];
   if (cluster) {
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1052,9 +1053,9 @@ void launch_pack(const Layout& y, const Dims& d, int rows, const tc::StepPtrs& i
   P.counters = io.counters;
   constexpr bool half = !std::is_same<T, float>::value;
   if (half && d.mma) {
-    if (y.gru) pack<T, true, half><<<592, 256, 0, s>>>(P); else pack<T, false, half><<<592, 256, 0, s>>>(P);
+    if (y.gru) pack<T, true, half><<<592, 256, 0, counted(s)>>>(P); else pack<T, false, half><<<592, 256, 0, counted(s)>>>(P);
   } else {
-    if (y.gru) pack<T, true, false><<<592, 256, 0, s>>>(P); else pack<T, false, false><<<592, 256, 0, s>>>(P);
+    if (y.gru) pack<T, true, false><<<592, 256, 0, counted(s)>>>(P); else pack<T, false, false><<<592, 256, 0, counted(s)>>>(P);
   }
 }
 
@@ -1209,12 +1210,12 @@ int64_t run_step(const Layout& y, const Plan* p, const tc::StepPtrs& io, bool wa
       const int64_t k0 = (int64_t)g.chunk * y.S;
       const int steps = (int)std::min<int64_t>(y.S, y.t - k0);
       fill_products(P, y, io, want_dx, k0, steps, !first);
-      if (y.dtype != MEBPTT_BF16) chunk_products<float, false><<<P.tiles, kTileThreads, 0, s>>>(P);
-      else if (y.tensor_cores) chunk_products<__nv_bfloat16, true><<<P.tiles, kTileThreads, 0, s>>>(P);
-      else chunk_products<__nv_bfloat16, false><<<P.tiles, kTileThreads, 0, s>>>(P);
+      if (y.dtype != MEBPTT_BF16) chunk_products<float, false><<<P.tiles, kTileThreads, 0, counted(s)>>>(P);
+      else if (y.tensor_cores) chunk_products<__nv_bfloat16, true><<<P.tiles, kTileThreads, 0, counted(s)>>>(P);
+      else chunk_products<__nv_bfloat16, false><<<P.tiles, kTileThreads, 0, counted(s)>>>(P);
       const Sums q{reinterpret_cast<const float*>(io.ws + y.off_dz), reinterpret_cast<const float*>(io.ws + y.off_dy), io.db, io.db_out,
                    loss_t + k0, y.L, y.NG, y.H, y.O, y.B, y.S, steps, sum_steps(y.B) * y.B, first ? 0 : 1};
-      chunk_sums<<<y.L * ((4 * y.H + 31) / 32) + (y.O + 31) / 32 + steps, 1024, 0, s>>>(q);
+      chunk_sums<<<y.L * ((4 * y.H + 31) / 32) + (y.O + 31) / 32 + steps, 1024, 0, counted(s)>>>(q);
       first = false;
     }
   }

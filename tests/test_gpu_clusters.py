@@ -6,6 +6,7 @@ import os
 import subprocess
 import sys
 
+import numpy as np
 import pytest
 
 from paper_1606_03401_b200 import synth
@@ -65,6 +66,32 @@ def test_waits_of_all_kinds_of_runs_run_out_and_report_timeout(bit, hidden, batc
     assert again["counters"][3] == 0 and again["counters"][1] == cfg.t
     assert_bit_identical(again, clean, want_dx=True)
 
+
+@pytest.mark.parametrize("hidden", [256, 640])
+@pytest.mark.parametrize("where,value", [("x", np.nan), ("x", np.inf), ("targets", np.inf), ("targets", np.nan), ("h0", None), ("c0", np.inf)])
+def test_values_that_are_not_finite_pass_through_runs(hidden, where, value):
+    """A ring's words of ones mean that nothing is there: no NaN that a step makes may look like that, or its wait runs out.
+    One place of one batch row has the value (h0: the NaN whose bits are ones); of the others nothing changes."""
+    import torch
+    cfg, dp = _problem(input=40, hidden=hidden, batch=64, readout=24, t=41)
+    clean = dp.run(dp.full_memory_plan())
+    row, v = 11, dp.dev[where]
+    at = v.view(cfg.t, cfg.batch, -1)[20, row] if where in ("x", "targets") else v.view(cfg.batch, -1)[row]
+    if value is None:
+        at.view(torch.int16)[2:4] = -1
+    else:
+        at[3] = value
+    others = np.arange(cfg.batch) != row
+    first = None
+    for plan in (dp.full_memory_plan(), dp.plan("msm", 9), dp.plan("hsm", 1)):
+        res = dp.run(plan)
+        assert res["counters"][0] == plan.cost and res["counters"][1] == cfg.t and res["counters"][3] == 0
+        assert not np.isfinite(res["dW"]).all()
+        dx, want = (r["dx"].reshape(cfg.t, cfg.batch, -1) for r in (res, clean))
+        assert np.array_equal(dx[:, others], want[:, others])
+        first = first or res
+        for k in ("loss", "dW", "db", "dW_out", "db_out", "dx"):
+            assert np.array_equal(res[k], first[k], equal_nan=True), k
 
 def test_short_and_long_runs_of_wide_layers_give_the_same_bits():
     """Runs of few operations take other kernels: plans whose runs are all short, all long and mixed."""

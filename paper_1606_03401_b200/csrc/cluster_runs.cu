@@ -8,9 +8,9 @@
 // cluster of ceil(H / 32) CTAs, a CTA with 32 hidden units: its 128 gate rows are a full MMA tile, the N is 16, the least
 // that an M of 128 allows.
 //
-//   forward    z[128 gate rows][16] = W_hh[rows of this CTA][H] h_{k-1}, both operands in shared memory; the gates;
-//              h_k goes to every CTA of the cluster, straight into the swizzled tile its next MMA reads, by
-//              asynchronous stores that count their bytes on the receiver's barrier.
+//   forward    z[128 gate rows][16] = W_hh[rows of this CTA][H] h_{k-1}, the weights in tensor memory, h_{k-1} in shared
+//              memory; the gates; h_k goes to every CTA of the cluster, straight into the operand its next MMA reads (without
+//              swizzle: below), by asynchronous stores that count their bytes on the receiver's barrier.
 //   backward   dz of the CTA's 32 units (128 gate columns) never leaves the CTA for the recurrence: it is multiplied
 //              by all H columns of W_hh it meets (K = 128), and the partial sums of dh go to the CTAs that own the
 //              columns, which add them in the order of the ranks.  (Gathering dz instead would send four times h.)

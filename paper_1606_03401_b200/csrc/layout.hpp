@@ -131,9 +131,9 @@ inline bool valid_desc(const mebptt_lstm_desc* d) {
   return true;
 }
 
-// Shapes the tensor-core kernels cover: one layer, bfloat16 operands, a batch that fits one MMA
-// tile, sizes that keep every TMA stride a multiple of 16 bytes, and a recurrent weight slice per
-// CTA (8 hidden units x 4 gates x H) that fits in shared memory with one CTA per SM.
+// Shapes the kernels that walk runs of one layer cover: bfloat16 operands, sizes that keep every TMA stride a multiple of
+// 16 bytes, a CTA's part of the recurrent weights (32 hidden units x 4 gates x H) in tensor and shared memory, and
+// a batch whose groups of rows (of 16 at the widest) are on the device at once.
 inline bool tensor_path_supported(const mebptt_lstm_desc* d) {
   return !(d->flags & (MEBPTT_FLAG_NO_TENSOR_CORES | MEBPTT_FLAG_GRU)) && d->dtype == MEBPTT_BF16 && d->layers == 1 && d->batch <= 64 && d->hidden % 8 == 0 &&
          d->input % 8 == 0 && d->readout % 8 == 0 && d->hidden >= 64 &&

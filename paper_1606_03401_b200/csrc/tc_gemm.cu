@@ -13,7 +13,7 @@
 //
 // One CTA computes one 128 x 128 tile (128 x 32 where C is short and wide: see gemm_bf16).  A single thread feeds a ring of
 // 128-byte swizzled shared-memory tiles by TMA (64 contraction indices per tile, one or three tiles per stage); a single thread issues
-// tcgen05.mma (M = 128, N = 128, K = 16, four per stage) into a 128-column TMEM accumulator and
+// tcgen05.mma (M = 128, N = 128, K = 16, four per tile) into a 128-column TMEM accumulator and
 // releases ring slots with tcgen05.commit; then all four warps read the accumulator with
 // tcgen05.ld (warp w owns TMEM lanes 32w .. 32w+31 = tile rows) and write the tile.
 // Out-of-range parts of a tile are zero-filled by TMA on the way in and masked on the way out.

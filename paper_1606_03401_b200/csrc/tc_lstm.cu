@@ -193,10 +193,8 @@ __device__ __forceinline__ void fwd_cell_sum(const FwdCell& st, const float* p0,
   for (int u = 0; u < 4; ++u) {
     const float4 x = *reinterpret_cast<const float4*>(p0 + 4 * u);
     z[u] = make_float4(st.zx[u].x + x.x, st.zx[u].y + x.y, st.zx[u].z + x.z, st.zx[u].w + x.w);
-    if (p1) {
-      const float4 y = *reinterpret_cast<const float4*>(p1 + 4 * u);
-      z[u].x += y.x; z[u].y += y.y; z[u].z += y.z; z[u].w += y.w;
-    }
+    const float4 y = *reinterpret_cast<const float4*>(p1 + 4 * u);
+    z[u].x += y.x; z[u].y += y.y; z[u].z += y.z; z[u].w += y.w;
   }
 }
 
@@ -207,7 +205,7 @@ __global__ void __launch_bounds__(192, 1) fwd_run_kernel(const __grid_constant__
   constexpr uint32_t W_TILE = FG * 128;   // [64 gate rows][64 contraction indices]
   constexpr uint32_t H_TILE = FB * 128;   // [32 batch rows][64 contraction indices]
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t wfull, full[4], acc;
+  __shared__ uint64_t wfull, full[2], acc;
   __shared__ uint32_t tmem_slot;
   __shared__ int failed;
 
@@ -216,7 +214,7 @@ __global__ void __launch_bounds__(192, 1) fwd_run_kernel(const __grid_constant__
   const int KB0 = fwd_first_part_blocks(a.H);
   uint8_t* sW = sm;                    // KB tiles: this CTA's rows of W_hh
   uint8_t* tiles = sm + KB * W_TILE;   // KB tiles: the group's rows of h_{k-1}
-  const int NQ = KB0 < KB ? 2 : 1;     // parts of the contraction: one barrier, one copy (slab mode), one accumulator each
+  constexpr int NQ = 2;                // parts of the contraction: one barrier, one copy, one accumulator each
   float* part = reinterpret_cast<float*>(tiles + NQ * KB0 * H_TILE);   // [2][FB][PART_LD]
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -243,8 +241,8 @@ __global__ void __launch_bounds__(192, 1) fwd_run_kernel(const __grid_constant__
   if (warp == 4) {
     // ---- producer: lane 0 watches the group's step counter, then h_{k-1} is requested.  A copy
     // instruction takes the TMA unit ~80-120 ns to accept whatever its size, and the unit takes one
-    // at a time: 16 tiles requested one by one are a microsecond.  In slab mode one copy (a 3-D box
-    // over a map that sees the row as blocks of 64 columns) brings a whole part of the split. ------
+    // at a time: 16 tiles requested one by one are a microsecond.  One copy (a 3-D box over a map that
+    // sees the row as blocks of 64 columns) brings a whole part of the split. ------------------------
     if (lane == 0) {
       mbar_arrive_expect_tx(&wfull, (uint32_t)KB * W_TILE);
       for (int kb = 0; kb < KB; ++kb) tma_load_2d(sW + kb * W_TILE, &tm_w, kb * 64, cta * FG, &wfull);
@@ -314,14 +312,13 @@ __global__ void __launch_bounds__(192, 1) fwd_run_kernel(const __grid_constant__
     const int j0 = cta * FU + u0;                       // first hidden unit
     const bool owner = b < a.B && j0 < a.H;
     const size_t e0 = (size_t)b * a.H + j0;             // element index of (b, j0) in a [B][H] array
-    const bool two = KB0 < KB;
     FwdCell st;
     fwd_cell_init(st, a, owner, b, j0, e0);
     for (int i = 0; i < a.n; ++i) {
       const DevOp op = a.ops[i];
       const bool got = wait_or_fail(&acc, (uint32_t)i & 1, &failed);
       tc_fence_after_sync();
-      for (int h = 0; h < (two ? 2 : 1); ++h) {
+      for (int h = 0; h < NQ; ++h) {
         uint32_t r[32];
         tmem_ld_32x32(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(h * FB), r);
         tmem_ld_wait();
@@ -337,7 +334,7 @@ __global__ void __launch_bounds__(192, 1) fwd_run_kernel(const __grid_constant__
       if (got && owner) {
         float4 z[4];
         const float* p0 = part + (size_t)bl * PART_LD + 4 * u0;
-        fwd_cell_sum(st, p0, two ? p0 + FB * PART_LD : nullptr, z);
+        fwd_cell_sum(st, p0, p0 + FB * PART_LD, z);
         fwd_cell_gates(st, z, out);
         // h_k first: it is what the other CTAs wait for
         *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.ws + (size_t)op.h_dst * 16) + e0) = out.hnew;
@@ -377,7 +374,6 @@ struct BwdRunArgs {
   uint32_t plane16;
   const float* zleaf;      // leaf batch: [S][B][4H] pre-activations z_k (gate columns permuted); NULL otherwise
   int loss_parts;          // partial sums of the loss per step
-  int tb;                  // K tiles per barrier and per copy
   uint32_t expect;         // signals a step is complete with: the grid size (a testing aid may ask for one too many)
   uint32_t poll_limit;     // polls of the step counter before the wait gives up
 };
@@ -435,7 +431,7 @@ __device__ __forceinline__ GateInputs4 load_gate_inputs4(const BwdRunArgs& a, co
   return in;
 }
 
-// The arithmetic of compute_gates for four hidden units.
+// The gate derivatives of four hidden units, with the arithmetic of the other kernels (bwd_run_ring): same bits.
 __device__ __forceinline__ void compute_gates4(const BwdRunArgs& a, const GateInputs4& in, int sidx, int b, int j0,
                                                const float (&dh)[4], float (&dc)[4]) {
   const int G = 4 * a.H;
@@ -470,6 +466,7 @@ __device__ __forceinline__ void compute_gates4(const BwdRunArgs& a, const GateIn
 }
 
 constexpr int GCS = 4;           // CTAs per cluster
+constexpr int TB = 8;            // K tiles per barrier and per copy: two of each, for 10 to 16 tiles
 constexpr int RECV_LD = FB + 4;  // row stride of a received partial tile, [dh column][batch row] (floats)
 
 __global__ void __launch_bounds__(192, 1) bwd_run_group_kernel(const __grid_constant__ CUtensorMap tm_dz,
@@ -479,22 +476,21 @@ __global__ void __launch_bounds__(192, 1) bwd_run_group_kernel(const __grid_cons
   constexpr uint32_t W_TILE = NC * 128;    // [64 columns of dh][64 contraction indices]
   constexpr uint32_t A_TILE = FB * 128;    // [32 batch rows][64 contraction indices]
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t wfull, full[4], acc, pready[2];
+  __shared__ uint64_t wfull, full[2], acc, pready[2];
   __shared__ uint32_t tmem_slot;
   __shared__ int failed;
 
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int G = 4 * a.H;
-  const int KBS = (G / 64) / GCS;          // 64-wide K blocks in this CTA's slice (<= 16)
-  const int TB = a.tb;                     // K tiles per barrier and per copy
-  const int NQ = (KBS + TB - 1) / TB;      // <= 4
+  const int KBS = (G / 64) / GCS;          // 64-wide K blocks in this CTA's slice (10 to 16)
+  constexpr int NQ = 2;
   uint8_t* sW = sm;                        // KBS tiles of W_hh^T
   uint8_t* ring = sW + KBS * W_TILE;       // KBS tiles of dz_k, all of the slice at once
   // partial sums received from the cluster: [2 buffers][GCS senders][16 columns][RECV_LD]
   float* recv = reinterpret_cast<float*>(ring + NQ * TB * A_TILE);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int ncg = (int)gridDim.x / ((a.B > FB) ? 2 : 1);   // CTAs per group
+  const int ncg = (int)gridDim.x / 2;      // CTAs per group, of which there are two
   const int grp = blockIdx.x / ncg, cta = blockIdx.x % ncg;
   const uint32_t rank = cluster_ctarank();
   const int cl = cta / GCS;
@@ -1103,7 +1099,7 @@ struct Prepared {
   // device part
   bool short_runs = false;         // the kernels of this file take short runs of a layer whose longer ones go through the ring
   CUtensorMap tm_h, tm_w, tm_dz[2], tm_wt;
-  int fwd_ncg = 0, fwd_smem = 0, bwd_smem = 0, bwd_tb = 8;
+  int fwd_ncg = 0, fwd_smem = 0, bwd_smem = 0;
   int run_rows = 0;                // batch rows of a cluster (cluster_runs.cu); 0: the ring takes the runs (ring_runs.cu)
   RingFit ring{0, 0};
   CUtensorMap tm_w_cl, tm_wt_cl;
@@ -1204,8 +1200,7 @@ int short_fwd_smem(int H) {
   return lone_smem((KB * FG + 2 * KB0 * FB) * 128 + 2 * FB * PART_LD * 4 + 1024);
 }
 int short_bwd_smem(int H) {
-  const int kbs = (4 * H / 64) / GCS, tb = kbs > 8 ? 8 : 4;
-  return lone_smem(kbs * (FU * GCS * 128) + (kbs + tb - 1) / tb * tb * FB * 128 + 2 * GCS * FU * RECV_LD * 4 + 1024);
+  return lone_smem((4 * H / 64) / GCS * (FU * GCS * 128) + 2 * TB * FB * 128 + 2 * GCS * FU * RECV_LD * 4 + 1024);
 }
 
 // Kernel variants and tensor maps for the workspace at `ws` on the current device.
@@ -1224,11 +1219,12 @@ void build_device_part(Prepared& P, const Layout& y, char* ws) {
   if (P.run_rows <= 0 && H > 8 * CU) P.ring = ring_fit(B, H);
   if (P.run_rows <= 0 && P.ring.rows <= 0) { P.rc = MEBPTT_ERR_UNSUPPORTED; return; }
   if (cluster_runs_supported(H) || B <= FB || B > 2 * FB || H % 128 != 0) return;
-  // Short runs (below).  Widths in whole blocks of 128: both kinds of kernels then add the same parts in the same order.
-  const int KB0 = fwd_first_part_blocks(H), kbs = (G / 64) / GCS;
+  // Short runs (below).  The kernels for them take the batch in two groups of 32 rows, so more than 32 and at most 64; one group
+  // was not measured against the ring's of 8 rows.  Widths in whole blocks of 128: both kinds of kernels then add the same
+  // parts in the same order.
+  const int KB0 = fwd_first_part_blocks(H);
   P.fwd_ncg = H / FU;
   P.fwd_smem = short_fwd_smem(H);
-  P.bwd_tb = kbs > 8 ? 8 : 4;
   P.bwd_smem = short_bwd_smem(H);
   const void* fn = (const void*)bwd_run_group_kernel;
   bool ok = cudaFuncSetAttribute(fwd_run_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) == cudaSuccess &&
@@ -1247,12 +1243,13 @@ void build_device_part(Prepared& P, const Layout& y, char* ws) {
        make_tmap_2d(&P.tm_w, wp_hh, 2, (uint64_t)H, (uint64_t)G, (uint64_t)H * 2, 64, FG) &&
        make_tmap_2d(&P.tm_wt, wpT_hh, 2, (uint64_t)G, (uint64_t)H, (uint64_t)G * 2, 64, FU * GCS);
   for (int pb = 0; pb < 2; ++pb)
-    ok = ok && make_tmap_blocks64(&P.tm_dz[pb], dz + (size_t)pb * S * B * G, (uint64_t)G, (uint64_t)S * B, (uint64_t)G * 2, FB, (uint32_t)P.bwd_tb);
+    ok = ok && make_tmap_blocks64(&P.tm_dz[pb], dz + (size_t)pb * S * B * G, (uint64_t)G, (uint64_t)S * B, (uint64_t)G * 2, FB, (uint32_t)TB);
   P.short_runs = ok;
 }
 // Runs of fewer operations than these are short: the kernels of this file load half the weights at the start of a launch,
 // and take longer for an operation.  At H = 1024, B = 64, in us: forward some 1 + 4.1 n against 8 + 2.6 n, backward
-// 4.7 + 4.6 n against 9.1 + 2.8 n.
+// 4.7 + 4.6 n against 9.1 + 2.8 n.  The line holds for narrower layers: t = 400, HSM m = 4, ms a step at H = 640, 768 and 1024
+// with these, 14.23, 14.64, 15.95; with (3, 2) 14.25, 14.76, 15.97; (8, 5) 14.33, 14.75, 16.08; none short 15.12, 15.65, 17.22.
 constexpr int SHORT_FWD = 5, SHORT_BWD = 3;
 
 // The set for (problem, plan, workspace, device): from the cache, or built and put there.  ws may
@@ -1602,7 +1599,7 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
           e = cluster_backward(P.tm_wt_cl, a, P.run_rows, s);
         } else if (P.short_runs && n < SHORT_BWD) {
           BwdRunArgs sa{bops, n, ws, dha, dz_c, dh, dc, loss_part, loss_t, sync + (size_t)launch_id * 2 * SYNC_STRIDE, status,
-                        io.counters, B, H, S, off16(y.plane), leaf ? zleaf : nullptr, parts, P.bwd_tb,
+                        io.counters, B, H, S, off16(y.plane), leaf ? zleaf : nullptr, parts,
                         (uint32_t)P.fwd_ncg + ((fault & 2) ? 1u : 0u), (fault & 2) ? fault_poll_limit : (kSpinLimit >> 1)};
           void* args[] = {(void*)&P.tm_dz[pb], (void*)&P.tm_wt, (void*)&sa};
           // (in plain stream order: early residency of a clustered cooperative grid measured no gain)

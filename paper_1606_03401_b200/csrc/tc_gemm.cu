@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant
       if (A_MN) {
         if (blocks & 1) tma_load_3d(sA, &tma, 0, k0 * BK, ma / 64, &full[s]);
         else for (int q = 0; q < 2; ++q) tma_load_2d(sA + q * TPS * 8192, &tma, ma + 64 * q, k0 * BK, &full[s]);
-      } else if (blocks & 1) {
+      } else if (TPS > 1 && (blocks & 1)) {
         tma_load_3d(sA, &tma, 0, m0, k0, &full[s]);
       } else {
         for (int t = 0; t < TPS; ++t) tma_load_2d(sA + t * A_BYTES, &tma, (k0 + t) * BK, m0, &full[s]);
@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(128, 4) gemm_bf16_kernel(const __grid_constant
       if (B_MN) {
         if (blocks & 2) tma_load_3d(sB, &tmb, 0, k0 * BK, nb / 64, &full[s]);
         else for (int q = 0; q < 2; ++q) tma_load_2d(sB + q * TPS * 8192, &tmb, nb + 64 * q, k0 * BK, &full[s]);
-      } else if (blocks & 2) {
+      } else if (TPS > 1 && (blocks & 2)) {
         tma_load_3d(sB, &tmb, 0, n0, k0, &full[s]);
       } else {
         for (int t = 0; t < TPS; ++t) tma_load_2d(sB + t * B_BYTES, &tmb, (k0 + t) * BK, n0, &full[s]);
@@ -462,10 +462,14 @@ int gemm_bf16(const void* A, int64_t lda, bool a_mn, const void* B, int64_t ldb,
   if (splits > 1 && (size_t)grid.x * grid.y * splits * BM * BN > split->partial_floats) return MEBPTT_ERR_WORKSPACE;
   grid.z = splits;
   // Grids of at most one wave: two stages of three tiles (a contraction that is longer than both) or six of one, one CTA
-  // an SM.  Larger ones: three stages of one tile, two CTAs per SM, so that one's epilogue overlaps the other's main loop.
+  // an SM.  Six as well where both operands are K-major rows of no whole blocks of 64 and the tiles wide: three tiles then take a
+  // copy each, six in a row, and nothing is gained (us, one and three a stage: 1024 x 1024, K = 456 8.8, 9.0; 520 x 2080,
+  // K = 600 9.8, 10.1 and K = 1992 18.2, 18.5; narrow tiles, 288 x 256, K = 1992 14.1, 12.3).  Larger grids: three stages of
+  // one tile, two CTAs per SM, so that one's epilogue overlaps the other's main loop.
   const bool one_wave = grid.x * grid.y * grid.z <= 148;
   const int nk = (halves ? 3 : 1) * (((K + BK - 1) / BK + splits - 1) / splits);
-  const int tps = one_wave && nk > MAX_STAGES ? DEEP_TILES : 1;
+  const bool copy_each = !a_mn && !b_mn && K % 64 != 0;
+  const int tps = one_wave && nk > MAX_STAGES && (narrow || !copy_each) ? DEEP_TILES : 1;
   const int stages = tps > 1 ? MAX_STAGES / DEEP_TILES : one_wave ? MAX_STAGES : 3;
   CUtensorMap ta, tb;
   int blocks = 0;

@@ -243,8 +243,9 @@ __global__ void __launch_bounds__(THREADS, 1) fwd_run_cluster(const __grid_const
         gate[v][0] = iv; gate[v][1] = fv; gate[v][2] = gv; gate[v][3] = ov;
       }
       __syncwarp();
-      uint4 hnew = make_uint4(0, 0, 0, 0);                   // (past the last unit)
-      if (wvalid) hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);
+      // (Past the last unit these are zeros: its weights and Zx are.  A row with a NaN has one there as well, beside NaNs in
+      // all of its units.)
+      const uint4 hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);
       if (got && prow < RB && i + 1 < a.n) {
         // h_k to every CTA, the next in rank first
         const uint32_t dst = piece + (((uint32_t)i + 1) & 1) * h_buf, bar = (i & 1) ? bar0 : bar1;

@@ -357,8 +357,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
         gate[v][0] = iv; gate[v][1] = fv; gate[v][2] = gv; gate[v][3] = ov;
       }
       __syncwarp();
-      uint4 hnew = make_uint4(0, 0, 0, 0);                   // (past the last unit)
-      if (wvalid) hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);
+      const uint4 hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);   // (past the last unit: as in fwd_run_cluster)
       if (got && sends) {
         if (i + 1 < a.n) store_piece(g.ring + (size_t)((i + 1) & (RING_SLOTS - 1)) * slot_bytes + mine, hnew);
         if (i >= 1) store_piece(g.ring + (size_t)((i - 1) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());

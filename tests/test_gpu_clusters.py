@@ -67,7 +67,7 @@ def test_waits_of_all_kinds_of_runs_run_out_and_report_timeout(bit, hidden, batc
     assert_bit_identical(again, clean, want_dx=True)
 
 
-@pytest.mark.parametrize("hidden", [256, 640])
+@pytest.mark.parametrize("hidden", [256, 264, 520, 640])
 @pytest.mark.parametrize("where,value", [("x", np.nan), ("x", np.inf), ("targets", np.inf), ("targets", np.nan), ("h0", None), ("c0", np.inf)])
 def test_values_that_are_not_finite_pass_through_runs(hidden, where, value):
     """A ring's words of ones mean that nothing is there: no NaN that a step makes may look like that, or its wait runs out.

@@ -451,7 +451,7 @@ inline void workspace_layout(const mebptt_lstm_desc* d, const Plan* p, Layout& y
     y.off_loss_part = take((size_t)y.S * loss_parts_per_step(y.B, y.O) * 4);
     y.n_sync = 64 * (work_items(p, y.S).size() + 1);   // two 128-byte lines per persistent launch (one per group of CTAs)
     y.off_sync = take(y.n_sync * 4);
-    y.ring_bytes = tc::ring_runs_supported(y.H, y.B) ? tc::ring_bytes(y.H, y.B) : 0;   // the exchange of wide layers
+    y.ring_bytes = tc::ring_runs_supported(y.H, y.B) ? tc::ring_place(y.H, y.B) : 0;   // the exchange of wide layers
     y.off_ring = take(y.ring_bytes);
     y.tape_bytes = (size_t)p->tape.size() * 32 * 2;   // the tape, and the compacted entries of leaf batches
     y.off_tape = take(y.tape_bytes);

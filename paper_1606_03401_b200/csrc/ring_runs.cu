@@ -196,9 +196,8 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = g.first + (int)blockIdx.x / ncta, cta = (int)blockIdx.x % ncta, groups = (a.B + RB - 1) / RB;
-  // a slot: the groups one after the other, [8 units][R rows][16 bytes] each (the last group's R may be less than RB)
-  const int R = grp == groups - 1 ? ring_last_rows(a.B, RB) : RB;
-  const uint32_t row_bytes = (uint32_t)ncta * CU * 2, group_bytes = row_bytes * RB, slot_bytes = group_bytes * (groups - 1) + row_bytes * ring_last_rows(a.B, RB);
+  // (a slot: the groups one after the other, [8 units][RB rows][16 bytes] each)
+  const uint32_t group_bytes = (uint32_t)ncta * CU * RB * 2, slot_bytes = group_bytes * groups;
 
   if (tid == 0) {
     weights_init(wt);
@@ -262,7 +261,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
     uint32_t want = 0;
 #pragma unroll
     for (int x = 0; x < N; ++x)
-      if (row < R && p0 + x * STEP < p_end) want |= 1u << x;
+      if (p0 + x * STEP < p_end) want |= 1u << x;
     uint8_t* const to = sH + p0 * PIECE + row * 16;
     {
       // the state the run starts from, rows past the batch as zeros
@@ -277,10 +276,10 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
       for (int x = 0; x < N; ++x)
         if (want >> x & 1) *reinterpret_cast<uint4*>(to + x * STEP * PIECE) = v[x];
     }
-    const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)p0 * (R * 16) + row * 16;
+    const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)p0 * (RB * 16) + row * 16;
     for (int i = 0; i < a.n; ++i) {
       if (i > 0) {
-        if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * R * 16, to + (i & 1) * h_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
+        if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * RB * 16, to + (i & 1) * h_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
         if (g.fault && pw == 0 && !poll_pieces<1>(g.never, 0, to, 0, 1u, &failed, g.poll_limit)) break;
       }
       fence_proxy_async_shared();
@@ -320,9 +319,8 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
     }
     if (pvalid) hprev = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(a.ws + (size_t)op0.h_src * 16) + ep);
     // this lane's piece in a slot
-    const bool sends = lane < 8 && 8 * half + prow < R;
-    const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)(jw / 8) * (R * 16) + (uint32_t)(8 * half + prow) * 16;
-    if (sends)
+    const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)(jw / 8) * (RB * 16) + (uint32_t)(8 * half + prow) * 16;
+    if (lane < 8)
       for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
     weights_move(wt, KT, sm + Shape::stages(KT), tmem, warp, lane, Shape::G, &failed);
     __syncwarp();
@@ -358,7 +356,7 @@ __global__ void __launch_bounds__(FwdShape<RB>::THREADS, 1) fwd_run_ring(const _
       }
       __syncwarp();
       const uint4 hnew = *reinterpret_cast<const uint4*>(&st.v[0][prow][0]);   // (past the last unit: as in fwd_run_cluster)
-      if (got && sends) {
+      if (got && lane < 8) {
         if (i + 1 < a.n) store_piece(g.ring + (size_t)((i + 1) & (RING_SLOTS - 1)) * slot_bytes + mine, hnew);
         if (i >= 1) store_piece(g.ring + (size_t)((i - 1) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
       }
@@ -446,10 +444,8 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
   const int grp = g.first + (int)blockIdx.x / ncta, cta = (int)blockIdx.x % ncta, groups = (a.B + RB - 1) / RB;
   const int rank = cta % RING_CLUSTER, cl = cta / RING_CLUSTER;
   const int half0 = 8 * (KT / 2);                  // pieces of two units in a half of the CTA's quarter
-  // a slot: the groups one after the other, [2 units][R rows][16 bytes] each (the last group's R may be less than RB)
-  const int R = grp == groups - 1 ? ring_last_rows(a.B, RB) : RB;
-  const uint32_t row_bytes = (uint32_t)ncta * 4 * CU * 2, group_bytes = row_bytes * RB, slot_bytes = group_bytes * (groups - 1) + row_bytes * ring_last_rows(a.B, RB);
-  const uint32_t cta_bytes = 4 * CU * 2 * (uint32_t)R;
+  // a slot: the groups one after the other, [2 units][RB rows][16 bytes] each
+  const uint32_t cta_bytes = 4 * CU * RB * 2, group_bytes = (uint32_t)ncta * cta_bytes, slot_bytes = group_bytes * groups;
 
   if (tid == 0) {
     weights_init(wt);
@@ -554,12 +550,12 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
     uint32_t want = 0;
 #pragma unroll
     for (int x = 0; x < N; ++x) {
-      if (row < R && p0 + x * STEP < (q + 1) * half0) want |= 1u << x;
+      if (p0 + x * STEP < (q + 1) * half0) want |= 1u << x;
     }
     uint8_t* const to = sZ + p0 * PIECE + row * 16;
-    const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)(rank * per) * cta_bytes + (size_t)p0 * (R * 16) + row * 16;
+    const char* const from = g.ring + (size_t)grp * group_bytes + (size_t)(rank * per) * cta_bytes + (size_t)p0 * (RB * 16) + row * 16;
     for (int i = 0; i < a.n; ++i) {
-      if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * R * 16, to + (i & 1) * z_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
+      if (!poll_pieces<N>(from + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes, STEP * RB * 16, to + (i & 1) * z_buf, STEP * PIECE, want, &failed, g.poll_limit)) break;
       if (g.fault && pw == 0 && !poll_pieces<1>(g.never, 0, to, 0, 1u, &failed, g.poll_limit)) break;
       fence_proxy_async_shared();
       __syncwarp();
@@ -584,12 +580,11 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
     }
     // dz leaves in pieces of two units: an even lane takes them from its neighbour for its first row, an odd one for its second
     const int odd = lane & 1, prow = r0 + odd;
-    const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)cta * cta_bytes + (uint32_t)(u >> 1) * (R * 16) + (uint32_t)prow * 16;
-    const bool store_ok = u < units && prow < rows, sends = prow < R;   // (units is a multiple of 8)
+    const uint32_t mine = (uint32_t)grp * group_bytes + (uint32_t)cta * cta_bytes + (uint32_t)(u >> 1) * (RB * 16) + (uint32_t)prow * 16;
+    const bool store_ok = u < units && prow < rows;   // (units is a multiple of 8)
     __nv_bfloat16* dzp = reinterpret_cast<__nv_bfloat16*>(a.dz) + 4 * ((size_t)s_hi * a.B * a.H + (size_t)(brow + prow) * a.H + unit0 + (u & ~1));
     const size_t dz_step = (size_t)4 * a.B * a.H;
-    if (sends)
-      for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
+    for (int s = 0; s < RING_SLOTS; ++s) store_piece(g.other + (size_t)s * slot_bytes + mine, ones());
     // partial sums: lane l holds column 32 wq + l of the cluster's, which CTA wq owns
     const uint32_t to = map_rank(smem_u32(sR) + (uint32_t)rank * SLOT + (uint32_t)(2 * half) * (CU * 16) + (uint32_t)lane * 16, (uint32_t)wq);
     const uint32_t tb = map_rank(smem_u32(&full[0]), (uint32_t)wq);
@@ -634,13 +629,13 @@ __global__ void __launch_bounds__(BwdShape<RB>::THREADS, 1) bwd_run_ring(const _
       const uint2 get = make_uint2(__shfl_xor_sync(0xffffffffu, send.x, 1), __shfl_xor_sync(0xffffffffu, send.y, 1));
       const uint4 piece = odd ? make_uint4(get.x, get.y, keep.x, keep.y) : make_uint4(keep.x, keep.y, get.x, get.y);
       const bool live = !*(volatile int*)&failed;
-      if (live && sends) store_piece(g.ring + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes + mine, piece);
+      if (live) store_piece(g.ring + (size_t)(i & (RING_SLOTS - 1)) * slot_bytes + mine, piece);
       __syncwarp();
       if (lane == 0) mbar_arrive(&used[i & 1]);
       // beside the exchange: dz to its stage, the piece of two steps ago cleared, the inputs of the next (earlier) step
       if (live) {
         if (store_ok) *reinterpret_cast<uint4*>(dzp) = piece;
-        if (sends && i >= 2) store_piece(g.ring + (size_t)((i - 2) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
+        if (i >= 2) store_piece(g.ring + (size_t)((i - 2) & (RING_SLOTS - 1)) * slot_bytes + mine, ones());
       }
       if (i + 1 < a.n) {
         (void)wait_or_fail(&inready[(i + 1) & 1], (uint32_t)((i + 1) >> 1) & 1, &failed);

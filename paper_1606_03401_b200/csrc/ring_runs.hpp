@@ -15,22 +15,20 @@ inline bool ring_runs_supported(int H, int B) { return H % 8 == 0 && H > 16 * CU
 inline int ring_ctas(int H) { return (H + RING_CLUSTER * CU - 1) / (RING_CLUSTER * CU) * RING_CLUSTER; }
 // Units whose dz a step of a backward run waits for, likewise (fwd_waited_units).
 __host__ __device__ inline int bwd_waited_units(int H) { return (H + RING_CLUSTER * CU - 1) / (RING_CLUSTER * CU) * RING_CLUSTER * CU; }
-// Batch rows of the last group, of RB each, as its slots hold them: no more than there are, but where two sets of warps share
-// the rows of a CTA (RB = 16, eight each) at least one row of the second, which would otherwise send nothing (fwd_waited_units).
-__host__ __device__ inline int ring_last_rows(int B, int RB) {
-  const int rows = B - (B - 1) / RB * RB;
-  return rows < RB - 7 ? RB - 7 : rows;
-}
-// Rows of a slot, in groups of 8 or of 16, whichever the device gets.  (Up to 8 rows are one group either way, which fits
-// with 8 if it does with 16.)
-inline int ring_slot_rows(int B) { return B <= 8 ? B : (B - 1) / 16 * 16 + ring_last_rows(B, 16); }
-// bytes of both rings, two sets each: launches alternate between them.  Less than what the workspace gained when one stage of
-// h took the place of two, of h_{k-1} and of h_k: 4 (S - 1) bytes a unit and row, S >= 32, against 80, or 99 where H is no
-// multiple of 128 -- so that no budget holds fewer states for it.
+// Rows of a slot: whole groups of 8 or of 16, whichever the device gets, whether they exist or not.  A piece of eight units is
+// then a line of 128 bytes that one warp writes.  (With as many rows as there are, lines of several writers: 9 rows at
+// H = 608 16 % slower, 36 at H = 800 17 %.)  Up to 8 rows are one group either way, which fits with 8 if it does with 16.
+inline int ring_slot_rows(int B) { return B <= 8 ? 8 : (B + 15) / 16 * 16; }
+// bytes of both rings, two sets each: launches alternate between them
 inline size_t ring_bytes(int H, int B) {
   const size_t rows = (size_t)ring_slot_rows(B), row = (size_t)ring_ctas(H) * CU * 2;
   return 2 * RING_SLOTS * rows * (row + 4 * row) + 256;
 }
+// Those of them that the workspace has a place for.  One stage of h in place of two, of h_{k-1} and of h_k, has made room for
+// 4 (S - 1) bytes a unit and row, S >= 32, and budgets are to hold no fewer states than with both: a ring takes 80 bytes a
+// unit and row of a slot (99 where H is no multiple of 128), more than that below four rows.  The ring of so few lies in the
+// second copy of the input projections, which then are not computed ahead.
+inline size_t ring_place(int H, int B) { return B > 3 ? ring_bytes(H, B) : 0; }
 
 struct RingArgs {
   char* ring;            // slots of this launch's set: words of ones wherever nothing has been written

@@ -1344,8 +1344,8 @@ int64_t run_step(const Layout& y, const Plan* p, const StepPtrs& io, bool want_d
   __nv_bfloat16* woutT = reinterpret_cast<__nv_bfloat16*>(at(y.off_woutT));
 
   const bool clusters = P.run_rows > 0;   // (else the ring, and for short runs perhaps the kernels of this file)
-  // Where the layout has no place for the ring because clusters were to take the runs, it lies in the second copy of the
-  // input projections (16 S >= 512 bytes a unit and row; the ring takes 120), which then are not computed ahead.
+  // Where the layout has no place for the ring (few rows: ring_place; or clusters were to take the runs), it lies in the second
+  // copy of the input projections, 16 S B H bytes, which then are not computed ahead.
   const bool no_room = P.ring.rows > 0 && !y.ring_bytes;
   char* const ring = no_room ? reinterpret_cast<char*>(zx + (size_t)S * B * G) : at(y.off_ring);
   // On request (a switch in the environment) the step runs on a stream of the library's, of the most

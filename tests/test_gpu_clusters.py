@@ -34,7 +34,8 @@ def _problem(**size):
     # wider: 17 CTAs forward and 24 backward, a part of the contraction of 32 columns; 24 and 24; 25 and 32
     (520, 9), (640, 64), (768, 16), (776, 33),
     (1000, 20), (1024, 64), (1024, 1),
-    (1024, 40), (1024, 41),     # the last group of 16 rows has 8 (a ninth is sent along) and 9
+    (1024, 40), (1024, 41),     # the last group of 16 rows has 8, and 9
+    (520, 1), (776, 3), (640, 4),              # up to three rows the ring lies beside the input projections
 ])
 def test_clusters_match_the_oracle_and_every_plan_gives_the_same_bits(hidden, batch):
     cfg, dp = _problem(input=40, hidden=hidden, batch=batch, readout=24, t=41)
